@@ -186,8 +186,9 @@ typedef struct {
     const char* least_text;         /* fully parenthesised infix, e.g. "(j+(i*8))", "(i<<2)"; min and max as calls, "min(a,b)" */
     uint64_t evals_executed;        /* candidate-point evaluations that ran for this hole: filter_tests plus the exact
                                        evaluations of stage 2 (a hit at a probe point) and stage 3 (a survivor at a
-                                       domain point).  Candidates decided without a test are not in here. */
-    uint64_t filter_survivors;      /* candidates that passed the first probe point */
+                                       domain point).  Candidates decided without a test of their own are not in here. */
+    uint64_t filter_survivors;      /* what the filter passed on: candidates that passed the first probe point, and operands
+                                       for which the leaf join left some leaf open */
     uint64_t probe_survivors;       /* candidates that passed every probe point */
     uint64_t nominal_ops;           /* 32-bit integer operations the filter stage's candidate-point evaluations
                                        that were carried out amount to under the library's cost model: one operation and one
@@ -196,10 +197,12 @@ typedef struct {
     double kernel_ms;               /* device time of the whole call's kernels (CUDA events) */
     double total_ms;                /* host wall time of the whole call */
     int32_t n_launches;             /* kernels the call launched */
-    uint64_t filter_tests;          /* filter-stage tests at the first probe point that ran: pairs of operand subtrees
-                                       both defined there, times the operators whose test loop was entered */
-    uint64_t candidates_skipped;    /* candidates of the operand tiles visited that were decided without a test: an
-                                       operand undefined at the probe (a zero divisor inside it), a remainder whose
+    uint64_t filter_tests;          /* filter-stage tests that ran: pairs of operand subtrees both defined at the first probe
+                                       point, times the operators whose test loop was entered; where one operand is a leaf,
+                                       operands defined at the probes times (leaves tested one by one, plus one condition that
+                                       decides all constants together) times the operators */
+    uint64_t candidates_skipped;    /* candidates of the operand tiles and joins visited that were decided without a test of
+                                       their own: a constant leaf decided together with the others, an operand undefined at the probe (a zero divisor inside it), a remainder whose
                                        divisor cannot exceed the target's magnitude, a quotient or remainder of 32-bit
                                        operands against a target outside 32 bits.  With a rank window the tiles also
                                        cover some ranks outside it; those count here or in filter_tests as well. */
@@ -294,8 +297,9 @@ void xp_result_free(xp_result* r);
  *  - Inputs and outputs stay the caller's: the sketch (loaded earlier with xp_sketch_load,
  *    which does allocate) and `out`, an array of at least n_holes summaries, filled in place.
  *  - opts->workspace is ignored; size / rank windows, flags and stream work as in xp_repair;
- *    cancel is read once, before the launch; timeout_ms is ignored.  The call copies from
- *    pageable host memory and returns after the stream has been synchronised.
+ *    cancel is read once, before the launch; timeout_ms is ignored.  The call copies through
+ *    page-locked host memory that the library keeps from call to call and returns after the stream has been
+ *    synchronised.
  *  - A call whose plan needs more than the fixed array, or a sketch with more than 64 holes,
  *    fails with XP_ERR_TOO_LARGE and a message giving the limit; nothing is launched.
  *  - The first call on a device looks up the array's device address (cudaGetSymbolAddress) and

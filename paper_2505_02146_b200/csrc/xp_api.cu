@@ -154,6 +154,77 @@ struct PinnedArena {
     }
 };
 PinnedArena g_pinned;
+
+// Page-locked blocks for what a search sends and reads back, and pairs of events that time it: kept from call to
+// call in lists that any thread may use (a copy from ordinary memory goes through the driver's staging buffer and
+// makes the host wait; creating a pair of events takes longer than recording it).  A block that would take the list past
+// kStageKeep bytes is freed when it comes back.
+constexpr size_t kStageKeep = 64ull << 20, kStageLeast = 16ull << 10;
+struct StagePool {
+    std::mutex mu;
+    std::multimap<size_t, char*> blocks;
+    size_t kept = 0;
+};
+StagePool g_stage;
+struct StageBlock {                   // returned to the pool when it goes out of scope; nothing may be copying then
+    char* p = nullptr;
+    size_t bytes = 0;
+    bool locked = false;
+    StageBlock(size_t want) {
+        size_t need = kStageLeast;
+        while (need < want) need <<= 1;
+        {
+            std::lock_guard<std::mutex> lock(g_stage.mu);
+            auto it = g_stage.blocks.lower_bound(need);
+            if (it != g_stage.blocks.end() && it->first <= 4 * need) {
+                p = it->second; bytes = it->first; locked = true;
+                g_stage.kept -= bytes;
+                g_stage.blocks.erase(it);
+                return;
+            }
+        }
+        bytes = need;
+        void* q = nullptr;
+        if (cudaHostAlloc(&q, need, cudaHostAllocPortable) == cudaSuccess) { p = (char*)q; locked = true; return; }
+        (void)cudaGetLastError();
+        p = (char*)malloc(need);      // (ordinary memory serves too, more slowly)
+    }
+    ~StageBlock() {
+        if (!p) return;
+        if (!locked) { free(p); return; }
+        std::lock_guard<std::mutex> lock(g_stage.mu);
+        if (g_stage.kept + bytes > kStageKeep) { cudaFreeHost(p); return; }
+        g_stage.blocks.insert({bytes, p});
+        g_stage.kept += bytes;
+    }
+    StageBlock(const StageBlock&) = delete;
+    StageBlock& operator=(const StageBlock&) = delete;
+};
+
+struct EventPool { std::mutex mu; std::map<int, std::vector<std::pair<cudaEvent_t, cudaEvent_t>>> free_pairs; };
+EventPool g_events;
+struct EventPair {                    // events belong to the device that was current when they were made
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    int dev = -1;
+    cudaError_t open() {
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        {
+            std::lock_guard<std::mutex> lock(g_events.mu);
+            auto& v = g_events.free_pairs[dev];
+            if (!v.empty()) { e0 = v.back().first; e1 = v.back().second; v.pop_back(); return cudaSuccess; }
+        }
+        if ((e = cudaEventCreate(&e0)) != cudaSuccess) return e;
+        return cudaEventCreate(&e1);
+    }
+    ~EventPair() {
+        if (!e0 || !e1) { if (e0) cudaEventDestroy(e0); return; }
+        std::lock_guard<std::mutex> lock(g_events.mu);
+        auto& v = g_events.free_pairs[dev];
+        if (v.size() >= 64) { cudaEventDestroy(e0); cudaEventDestroy(e1); return; }
+        v.push_back({e0, e1});
+    }
+};
 }  // namespace
 
 static const char* const kOpText[] = {"+", "-", "*", "/", "%", "<", "<=", "==", "!=", "min", "max", "&&", "||", "<<", ">>"};
@@ -169,6 +240,8 @@ struct xp_grammar {
     std::vector<xp_production> prods;
     std::vector<LeafDev> leaves;
     std::vector<BinDev> bins;
+    std::vector<ConstDev> consts;    // per nonterminal: its constants ascending, then its variables (see GrammarDev::consts)
+    int const_begin[kMaxNt + 1] = {0}, var_begin[kMaxNt] = {0};
     int leaf_begin[kMaxNt + 1] = {0};
     int bin_begin[kMaxNt + 1] = {0};
     u64 cnt[kMaxNt][kMaxSize + 1] = {{0}};
@@ -253,6 +326,16 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
     }
     g->leaf_begin[g->n_nt] = (int)g->leaves.size();
     g->bin_begin[g->n_nt] = (int)g->bins.size();
+    for (int nt = 0; nt < g->n_nt; ++nt) {
+        const int lb = g->leaf_begin[nt], le = g->leaf_begin[nt + 1];
+        g->const_begin[nt] = (int)g->consts.size();
+        for (int i = lb; i < le; ++i) if (g->leaves[i].var < 0) g->consts.push_back(ConstDev{g->leaves[i].value, i - lb, 0});
+        std::sort(g->consts.begin() + g->const_begin[nt], g->consts.end(), [](const ConstDev& a, const ConstDev& b) {
+            return a.value != b.value ? a.value < b.value : a.pos < b.pos; });
+        g->var_begin[nt] = (int)g->consts.size();
+        for (int i = lb; i < le; ++i) if (g->leaves[i].var >= 0) g->consts.push_back(ConstDev{g->leaves[i].var, i - lb, 0});
+    }
+    g->const_begin[g->n_nt] = (int)g->consts.size();
     build_counts(g);
     *out = g;
     return XP_OK;
@@ -347,16 +430,20 @@ static xp_status grammar_to_device(xp_grammar* g, size_t* copied, PinnedArena* s
     memcpy(h.leaf_begin, g->leaf_begin, sizeof(h.leaf_begin));
     memcpy(h.bin_begin, g->bin_begin, sizeof(h.bin_begin));
     memcpy(h.cnt, g->cnt, sizeof(h.cnt));
-    // one device block and one copy: header | leaves | binary productions
+    memcpy(h.const_begin, g->const_begin, sizeof(h.const_begin));
+    memcpy(h.var_begin, g->var_begin, sizeof(h.var_begin));
+    // one device block and one copy: header | leaves | binary productions | constants
     const size_t off_leaves = (sizeof(GrammarDev) + 255) & ~(size_t)255;
     const size_t off_bins = off_leaves + ((sizeof(LeafDev) * (g->leaves.size() + 1) + 255) & ~(size_t)255);
-    const size_t total = off_bins + sizeof(BinDev) * (g->bins.size() + 1);
+    const size_t off_consts = off_bins + ((sizeof(BinDev) * (g->bins.size() + 1) + 255) & ~(size_t)255);
+    const size_t total = off_consts + sizeof(ConstDev) * (g->consts.size() + 1);
     char* block = nullptr;
     size_t granted = 0;
     XP_CUDA(pool_alloc((void**)&block, total, &g->d_device, &granted));
     g->d_bytes = granted;
     h.leaves = (const LeafDev*)(block + off_leaves);
     h.bins = (const BinDev*)(block + off_bins);
+    h.consts = (const ConstDev*)(block + off_consts);
     std::vector<char> stage_own;
     char* stage = staging ? staging->take(total) : nullptr;
     const bool queued = stage != nullptr;
@@ -365,6 +452,7 @@ static xp_status grammar_to_device(xp_grammar* g, size_t* copied, PinnedArena* s
     memcpy(stage, &h, sizeof(h));
     if (!g->leaves.empty()) memcpy(stage + off_leaves, g->leaves.data(), sizeof(LeafDev) * g->leaves.size());
     if (!g->bins.empty()) memcpy(stage + off_bins, g->bins.data(), sizeof(BinDev) * g->bins.size());
+    if (!g->consts.empty()) memcpy(stage + off_consts, g->consts.data(), sizeof(ConstDev) * g->consts.size());
     cudaError_t e = queued ? cudaMemcpyAsync(block, stage, total, cudaMemcpyHostToDevice, nullptr)
                            : cudaMemcpy(block, stage, total, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { pool_release(block, g->d_bytes, g->d_device); return fail(XP_ERR_CUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e)); }
@@ -379,8 +467,9 @@ static xp_status grammar_to_device(xp_grammar* g, size_t* copied, PinnedArena* s
 
 struct HoleHost {
     int start_nt = 0, max_size = 0;
-    bool filter_ok = false;          // the probe filter applies (probe 0 exists, context affine there)
+    bool filter_ok = false;          // the probe filter applies (probe 0 exists, context affine or a comparison there, subtree tables)
     bool never = false;              // the spec is undefined at some point: no candidate can match
+    bool exact = false;              // the leaf join's conditions do not apply (a context factor of 2^31 or more, or 0)
     bool compares = false;           // the filter works on an interval of hole values (the context compares)
     bool second = false;             // filter hits are looked at once more at probe 1 from the start (hits are frequent)
 };
@@ -404,7 +493,6 @@ struct xp_sketch {
     size_t off_holes = 0;
     int tab_size_cap = 0, tab_probes_cap = 0;        // most sizes / probes that the subtree tables of a hole cover
     u64 entries_at[kMaxSize + 1] = {0};              // subtree-table entries per size (all nonterminals)
-    u64 big_entries = 0;                             // most entries of a hole's first-probe table of the next size
     // The sketch's part of a launch plan under default options (every size, no rank window, no flag), as
     // if it were the only sketch of the call: built on the first such call and copied, with ticket, sketch
     // and accumulator numbers shifted, into the plan of every later one (a batch of thousands of small
@@ -412,6 +500,8 @@ struct xp_sketch {
     mutable std::mutex plan_mu;
     mutable bool plan_cached = false;
     mutable std::vector<SegDev> plan_segs;
+    mutable std::vector<JoinSeg> plan_jsegs;
+    mutable std::vector<JoinGroup> plan_jgroups;
     mutable std::vector<u64> plan_ops;
     mutable u64 plan_tickets = 0;
 };
@@ -449,12 +539,12 @@ extern "C" void xp_sketch_destroy(xp_sketch* s) {
 }
 
 // Entries of the subtree-value tables of a hole with size bound max_size: sizes 1, 2, ... while
-// every nonterminal has at most kTabMaxEntries trees of that size, and never the sizes that only
-// occur as whole candidates (operands have at most max_size - 2 nodes).
+// every nonterminal has at most kTabMaxEntries trees of that size; apart from the leaves never the sizes
+// that only occur as whole candidates (operands have at most max_size - 2 nodes).
 static u64 table_entries(const xp_grammar* g, int max_size, u64 (*off)[kMaxSize + 1], int* tmax_out) {
     u64 total = 0;
     int tmax = 0;
-    for (int k = 1; k <= max_size - 2; ++k) {
+    for (int k = 1; k == 1 || k <= max_size - 2; ++k) {
         bool fits = true;
         for (int nt = 0; nt < g->n_nt; ++nt) fits = fits && g->cnt[nt][k] <= kTabMaxEntries;
         if (!fits) break;
@@ -478,7 +568,6 @@ struct LoadState {
     i64 table_points = 0;            // rows of a table domain (0 for a box)
     u64 entries_at[kMaxSize + 1] = {0};      // subtree-table entries per size (all nonterminals)
     int size_cap = 0, probes_cap = 0;        // over the holes
-    u64 big_entries = 0;                     // most entries of a hole's first-probe table of the next size
 };
 
 // First half of a load: checks the description, lays out and allocates the sketch's device
@@ -545,7 +634,7 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     const size_t off_holes = off;   off += al(sizeof(HoleDev) * nh + sizeof(u32) * nh);       // holes, then one flag each
     const size_t off_bad = off_holes + sizeof(HoleDev) * nh;
     size_t off_coords = 0;
-    std::vector<size_t> off_spec(nh, 0), off_tabv(nh, 0), off_tabk(nh, 0), off_tabm(nh, 0), off_bigv(nh, 0), off_bigk(nh, 0);
+    std::vector<size_t> off_spec(nh, 0), off_tabv(nh, 0), off_tabk(nh, 0), off_tabm(nh, 0), off_pair(nh, 0), off_sets(nh, 0);
     if (copy_coords && coords_bytes <= kPackMax) { off_coords = off; off += al(coords_bytes); }
     for (int h = 0; h < nh; ++h)
         if (d->holes[h].spec_kind == XP_SPEC_TABLE && np > 0 && !d->holes[h].spec_table_on_device && spec_bytes <= kPackMax) {
@@ -574,27 +663,9 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             off_tabv[h] = off; off += al(sizeof(i64) * entries * probes);
             off_tabk[h] = off; off += al(entries * probes);
             off_tabm[h] = off; off += al(entries);
+            off_pair[h] = off; off += al(2 * sizeof(i32) * entries);
         }
-        // one size further at the first probe only (see HoleDev::big_size): the register-side operands of the largest candidates
-        int big = o.tab_size_cap + 1;                     // the next size that has trees at all
-        while (big <= hd.max_size - 2) {
-            bool any = false;
-            for (int nt = 0; nt < g->n_nt; ++nt) any = any || g->cnt[nt][big] > 0;
-            if (any) break;
-            ++big;
-        }
-        if (entries > 0 && o.tab_size_cap >= 1 && big <= hd.max_size - 2) {
-            u64 total = 0;
-            for (int nt = 0; nt < g->n_nt; ++nt) { o.big_off[nt] = total; total += (g->cnt[nt][big] + 7) & ~7ull; }     // (ranges start at multiples of 8: bigvalue_kernel)
-            size_t free_b = 0, total_b = 0;
-            const bool room = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && (u64)free_b > 3 * total * 9;
-            if (total > 0 && total <= kBigMaxEntries && total * 9 <= kBigBudgetBytes && room) {
-                o.big_size = big; o.big_total = total;
-                off_bigv[h] = off; off += al(sizeof(i64) * total);
-                off_bigk[h] = off; off += al(total);
-                if (total > L->big_entries) L->big_entries = total;
-            }
-        }
+        off_sets[h] = off; off += al(sizeof(JoinSet) * (size_t)g->n_nt);
     }
     size_t arena_granted = 0;
     if (pool_alloc((void**)&s->arena, off, &s->arena_device, &arena_granted) != cudaSuccess) {
@@ -648,14 +719,11 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
         }
     }
     hs.n_samples = ns;
-    u64 most = 0;                                         // small searches get a cheaper probe choice: the load
-    for (int h = 0; h < nh; ++h) {                        // should not outweigh the search
+    for (int h = 0; h < nh; ++h) {
         u64 c = 0;
         for (int k = 1; k <= d->holes[h].max_size; ++k) c += g->cnt[d->holes[h].start_nt][k];
-        most = c > most ? c : most;
         hh[h].small_search = c <= 100000000ull ? 1 : 0;
     }
-    hs.prep_cands = most <= 100000000ull ? 256 : 1024;
 
     for (int h = 0; h < nh; ++h) {
         const xp_hole_desc& hd = d->holes[h];
@@ -673,11 +741,9 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             o.tab_val = (i64*)(base + off_tabv[h]);
             o.tab_ok = (unsigned char*)(base + off_tabk[h]);
             o.tab_vars = (unsigned char*)(base + off_tabm[h]);
+            o.tab_pair = (i32*)(base + off_pair[h]);
         }
-        if (o.big_size > 0) {
-            o.big_val = (i64*)(base + off_bigv[h]);
-            o.big_ok = (unsigned char*)(base + off_bigk[h]);
-        }
+        o.join_sets = (JoinSet*)(base + off_sets[h]);
         // variables the context and the spec mention (a caller's spec table may depend on all)
         u32 fv = hd.spec_kind == XP_SPEC_EXPR ? 0u : 0xffffffffu;
         for (int i = 0; i < hd.ctx_len; ++i) if (hd.ctx[i].kind == XP_I_VAR) fv |= 1u << hd.ctx[i].arg;
@@ -737,7 +803,7 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     }
     for (int k = 1; k <= kMaxSize; ++k)
         for (int nt = 0; nt < g->n_nt; ++nt) L->entries_at[k] += g->cnt[nt][k];
-    s->tab_size_cap = L->size_cap; s->tab_probes_cap = L->probes_cap; s->big_entries = L->big_entries;
+    s->tab_size_cap = L->size_cap; s->tab_probes_cap = L->probes_cap;
     memcpy(s->entries_at, L->entries_at, sizeof(s->entries_at));
 #undef XP_CUDA_S
     return XP_OK;
@@ -808,7 +874,10 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             }
         }
     }
-    XP_CUDA_B(pool_alloc((void**)&jobs_dev, stage.size(), &jobs_device, &jobs_bytes));
+    // (the prepare kernels' scratch follows the lists)
+    constexpr size_t kPiece = 32768;
+    const size_t scratch_at = (stage.size() + 255) & ~(size_t)255;
+    XP_CUDA_B(pool_alloc((void**)&jobs_dev, scratch_at + prepare_scratch_bytes((int)(n_jobs < kPiece ? n_jobs : kPiece)), &jobs_device, &jobs_bytes));
     XP_CUDA_B(cudaMemcpyAsync(jobs_dev, stage.data(), stage.size(), cudaMemcpyHostToDevice, nullptr));
     SketchDev* const* d_list = (SketchDev* const*)jobs_dev;
     const LoadJob* d_jobs = (const LoadJob*)(jobs_dev + list_bytes);
@@ -816,7 +885,6 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     // the probe choice; the subtree tables, bottom-up, for as many sizes and probes as there can be
     // (blocks beyond what the probe choice settled on for their hole return at once).  Grids are
     // cut into pieces of at most kPiece jobs (a grid dimension holds 65 535).
-    constexpr size_t kPiece = 32768;
     i64 most_points = 0;
     int size_cap = 0, probes_cap = 0;
     u64 most_entries[kMaxSize + 1] = {0};
@@ -829,16 +897,10 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     for (size_t at = 0; at < n; at += kPiece)
         XP_CUDA_B(launch_coord_bounds(d_list + at, (int)(n - at < kPiece ? n - at : kPiece), most_points, nullptr));
     for (size_t at = 0; at < n_jobs; at += kPiece)
-        XP_CUDA_B(launch_prepare(d_jobs + at, (int)(n_jobs - at < kPiece ? n_jobs - at : kPiece), nullptr));
+        XP_CUDA_B(launch_prepare(d_jobs + at, (int)(n_jobs - at < kPiece ? n_jobs - at : kPiece), jobs_dev + scratch_at, nullptr));
     for (int k = 1; k <= size_cap; ++k)
         for (size_t at = 0; at < n_jobs; at += kPiece)
             XP_CUDA_B(launch_subvalues(d_jobs + at, (int)(n_jobs - at < kPiece ? n_jobs - at : kPiece), k, probes_cap, most_entries[k], nullptr));
-    {
-        u64 big = 0;
-        for (size_t i = 0; i < n; ++i) big = st[i].big_entries > big ? st[i].big_entries : big;
-        for (size_t at = 0; at < n_jobs && big > 0; at += 32768)
-            XP_CUDA_B(launch_bigvalues(d_jobs + at, (int)(n_jobs - at < 32768 ? n_jobs - at : 32768), big, nullptr));
-    }
     // what the kernels decided, per hole
     for (size_t i = 0; i < n; ++i) {
         const int nh = st[i].s->n_holes;
@@ -861,8 +923,9 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             u32 bad = 0;
             memcpy(&bad, &st[i].back[sizeof(HoleDev) * nh + sizeof(u32) * h], sizeof(bad));
             // the filter applies where the context at probe 0 is affine in the hole, or a comparison
-            s->holes[h].filter_ok = o.filter_ok != 0;
+            s->holes[h].filter_ok = o.filter_ok != 0 && o.tab_probes > 0;
             s->holes[h].compares = o.filter_ok != 0 && o.aff_ok == 0;
+            s->holes[h].exact = o.aff_ok != 0 && o.join_on == 0;
             s->holes[h].never = bad != 0;                 // the spec is undefined at some point
             s->holes[h].second = o.second != 0;
             s->n_probes.push_back(o.n_probe);
@@ -970,15 +1033,15 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         if (e == cudaSuccess) e = launch_reprobe((const LoadJob*)jobs_dev, (int)jobs.size(), nullptr);
         for (int k = 1; k <= s->tab_size_cap && e == cudaSuccess; ++k)
             e = launch_subvalues((const LoadJob*)jobs_dev, (int)jobs.size(), k, s->tab_probes_cap, s->entries_at[k], nullptr);
-        if (e == cudaSuccess) e = launch_bigvalues((const LoadJob*)jobs_dev, (int)jobs.size(), s->big_entries, nullptr);
         if (e == cudaSuccess) e = cudaMemcpyAsync(hh.data(), s->arena + s->off_holes, sizeof(HoleDev) * nh, cudaMemcpyDeviceToHost, nullptr);
         const cudaError_t e2 = cudaStreamSynchronize(nullptr);
         pool_release(jobs_dev, jobs_bytes, jobs_device);
         if (e != cudaSuccess || e2 != cudaSuccess)
             return fail(XP_ERR_CUDA, std::string("xp_sketch_refine: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
         for (int h = 0; h < nh; ++h) {
-            s->holes[h].filter_ok = hh[h].filter_ok != 0;
+            s->holes[h].filter_ok = hh[h].filter_ok != 0 && hh[h].tab_probes > 0;
             s->holes[h].compares = hh[h].filter_ok != 0 && hh[h].aff_ok == 0;
+            s->holes[h].exact = hh[h].aff_ok != 0 && hh[h].join_on == 0;
             s->holes[h].second = hh[h].second != 0;
             s->n_probes[h] = hh[h].n_probe;
         }
@@ -1016,9 +1079,12 @@ struct xp_result {
 
 struct Plan {
     std::vector<SegDev> segs;
+    std::vector<JoinSeg> jsegs;
+    std::vector<JoinGroup> jgroups;
     std::vector<AccDev> acc;
     std::vector<u64> nominal_ops;    // per accumulator: cost-model operations of the filter stage
-    u64 n_tickets = 0;
+    u64 n_tickets = 0, n_join = 0;
+    bool join_wide = false;          // several operands per lane and step
 };
 
 // Scratch of calls that bring no workspace: one block per process, reused while no other call
@@ -1057,6 +1123,7 @@ static void add_tiles(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
             if (block == 0) continue;
             const u64 this_base = base;
             base += block;
+            if (a == 1 || a == k - 2) continue;              // (a leaf at the root: add_joins)
             if (this_base + block <= lo || this_base >= hi) continue;
             const u64 wlo = lo > this_base ? lo - this_base : 0;
             const u64 whi = hi - this_base < block ? hi - this_base : block;
@@ -1149,6 +1216,115 @@ static void add_tiles(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
     }
 }
 
+static int slot_of_op(int op) { return op <= XP_OP_MOD ? op : op <= XP_OP_MAX ? op - XP_OP_MIN + 5 : op - XP_OP_SHL + 7; }
+
+static JoinSeg new_join_seg(int sketch, int hole, int acc, int k, u64 lo, u64 hi) {
+    JoinSeg sg;
+    memset(&sg, 0, sizeof(sg));
+    sg.rank_begin = lo; sg.rank_end = hi;
+    sg.sketch = sketch; sg.hole = hole; sg.size = k; sg.acc = acc;
+    return sg;
+}
+
+// Leaf-join segments of (start nonterminal, size k >= 3) restricted to ranks [lo, hi): one per operand nonterminal, with
+// a group per leaf nonterminal, for every operator with a leaf of it on either side of such an operand.  Copies of one
+// production open segments of their own; so do shifts, which only the exact form knows.
+static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool exact) {
+    struct Open { JoinSeg seg; std::vector<JoinGroup> groups; };
+    std::vector<Open> open;
+    for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
+        const BinDev& bd = g->bins[b];
+        u64 base = bd.off[k];
+        for (int a = 1; a <= k - 2; ++a) {
+            const u64 cl = g->cnt[bd.lnt][a], cr = g->cnt[bd.rnt][k - 1 - a];
+            const u64 block = cl * cr;
+            const u64 this_base = base;
+            base += block;
+            if (block == 0 || (a != 1 && a != k - 2)) continue;
+            if (this_base + block <= lo || this_base >= hi) continue;
+            const u64 wlo = lo > this_base ? lo - this_base : 0, whi = hi - this_base < block ? hi - this_base : block;
+            const int swap = a == k - 2 ? 0 : 1;             // (k == 3: both operands are leaves; the left one is the operand)
+            const int ent = swap ? bd.rnt : bd.lnt, lnt = swap ? bd.lnt : bd.rnt;
+            u64 e0 = 0, e1 = swap ? cr : cl;                 // operands that the window covers
+            if (!swap) { e0 = wlo / cr; e1 = (whi + cr - 1) / cr; }
+            else if (wlo / cr == (whi - 1) / cr) { e0 = wlo % cr; e1 = (whi - 1) % cr + 1; }
+            const int slot = slot_of_op(bd.op);
+            const bool ex = exact || slot >= 7;
+            Open* at = nullptr;
+            JoinGroup* grp = nullptr;
+            for (size_t i = 0; i < open.size() && !at; ++i) {
+                Open& c = open[i];
+                if (c.seg.nt != ent || (c.seg.exact != 0) != ex) continue;
+                grp = nullptr;
+                for (JoinGroup& q : c.groups) if (q.leaf_nt == lnt) grp = &q;
+                if (grp ? !(((swap ? grp->smask : grp->fmask) >> slot) & 1u) : c.groups.size() < (size_t)kJoinGroups) at = &c;
+            }
+            if (!at) {
+                Open c;
+                c.seg = new_join_seg(sketch, hole, acc, k, lo, hi);
+                c.seg.kind = kJoinLeaf; c.seg.nt = ent; c.seg.esize = k - 2; c.seg.exact = ex ? 1 : 0;
+                c.seg.e_begin = e0; c.seg.e_count = e1 - e0;
+                open.push_back(c);
+                at = &open.back();
+                grp = nullptr;
+            }
+            if (!grp) {
+                JoinGroup q;
+                memset(&q, 0, sizeof(q));
+                q.leaf_nt = lnt;
+                at->groups.push_back(q);
+                grp = &at->groups.back();
+            }
+            JoinSeg& sg = at->seg;
+            const u64 end = sg.e_begin + sg.e_count;
+            if (e0 < sg.e_begin) sg.e_begin = e0;
+            sg.e_count = (e1 > end ? e1 : end) - sg.e_begin;
+            (swap ? grp->smask : grp->fmask) |= 1u << slot;
+            grp->base[swap][slot] = this_base;
+        }
+    }
+    for (Open& c : open) {
+        c.seg.first_group = (i32)plan->jgroups.size();
+        c.seg.n_groups = (i32)c.groups.size();
+        plan->jgroups.insert(plan->jgroups.end(), c.groups.begin(), c.groups.end());
+        JoinSeg sg = c.seg;
+        u64 left = sg.e_count;
+        const u64 most = 1ull << 31;                         // (a suspect's number inside its segment takes 32 bits)
+        while (left > 0) {
+            sg.e_count = left < most ? left : most;
+            plan->jsegs.push_back(sg);
+            sg.e_begin += sg.e_count; left -= sg.e_count;
+        }
+    }
+}
+
+// Every candidate of the window on its own, from the subtree tables.
+static void add_direct(Plan* plan, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi) {
+    JoinSeg sg = new_join_seg(sketch, hole, acc, k, lo, hi);
+    sg.kind = kJoinDirect; sg.nt = nt; sg.esize = k;
+    sg.e_begin = lo; sg.e_count = hi - lo;
+    plan->jsegs.push_back(sg);
+}
+
+// Tickets of the leaf join.  A step is 32 operands (one per lane); in the exact form one operand.  A ticket takes so
+// many steps that every warp of the device gets about four: fewer and the last wave is uneven, more and the
+// warps spend their time taking tickets.  64 steps at most.
+static void number_joins(Plan* plan) {
+    if (plan->jsegs.empty()) return;
+    u64 steps = 0;
+    for (const JoinSeg& c : plan->jsegs) steps += c.exact ? c.e_count : (c.e_count + 31) / 32;
+    u64 per = steps / ((u64)search_warps() * 4);
+    if (per < 1) per = 1;
+    if (per > 64) per = 64;
+    if (per >= 4) per &= ~3ull;
+    plan->join_wide = per >= 4;
+    for (JoinSeg& c : plan->jsegs) {
+        c.first_ticket = plan->n_join;
+        c.chunk = (u32)(c.exact ? per : per * 32);
+        plan->n_join += (c.e_count + c.chunk - 1) / c.chunk;
+    }
+}
+
 constexpr u64 kTileMinRanks = 4096;          // smaller windows are searched rank by rank
 
 static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, Plan* plan);
@@ -1178,6 +1354,8 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
                 Plan own;
                 plan_sketch(s, 0, o, &own);
                 s->plan_segs = std::move(own.segs);
+                s->plan_jsegs = std::move(own.jsegs);
+                s->plan_jgroups = std::move(own.jgroups);
                 s->plan_ops = std::move(own.nominal_ops);
                 s->plan_tickets = own.n_tickets;
                 s->plan_cached = true;
@@ -1197,7 +1375,15 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
             c.acc += acc_base;
         }
         plan->n_tickets += s->plan_tickets;
+        const size_t jat = plan->jsegs.size();
+        plan->jsegs.insert(plan->jsegs.end(), s->plan_jsegs.begin(), s->plan_jsegs.end());
+        const i32 group_base = (i32)plan->jgroups.size();
+        plan->jgroups.insert(plan->jgroups.end(), s->plan_jgroups.begin(), s->plan_jgroups.end());
+        for (size_t j = jat; j < plan->jsegs.size(); ++j) {
+            plan->jsegs[j].sketch = (i32)i; plan->jsegs[j].acc += acc_base; plan->jsegs[j].first_group += group_base;
+        }
     }
+    number_joins(plan);
     return XP_OK;
 }
 
@@ -1226,10 +1412,10 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 }
                 if (lo >= hi) continue;
                 const bool forced = (o->flags & XP_FLAG_ALWAYS_FILTER) != 0;
-                const bool tiles = k >= 3 && ho.filter_ok && !(o->flags & XP_FLAG_NO_FILTER) &&
-                                   (forced || hi - lo >= kTileMinRanks);
-                if (tiles) add_tiles(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile);
-                else add_linear(plan, (int)i, h, acc, k, lo, hi);
+                if (!ho.filter_ok || (o->flags & XP_FLAG_NO_FILTER)) { add_linear(plan, (int)i, h, acc, k, lo, hi); continue; }
+                if (k < 3 || (!forced && hi - lo < kTileMinRanks)) { add_direct(plan, ho.start_nt, (int)i, h, acc, k, lo, hi); continue; }
+                add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact);
+                add_tiles(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile);
             }
         }
     }
@@ -1244,10 +1430,13 @@ static u32 surv_cap_for(size_t n_sketches) {
 }
 constexpr u32 kSurvCapStatic = 8192;         // ... of a call on the library's fixed scratch
 
-static SearchLayout ws_layout(size_t n_segs, size_t n_sketches, size_t n_acc, u32 surv_cap) {
+static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size_t n_sketches, u32 surv_cap) {
     SearchLayout w;
+    const size_t n_acc = plan.acc.size();
     w.segs = 256;
-    w.sketches = w.segs + align256(sizeof(SegDev) * (n_segs + 1));
+    w.jsegs = w.segs + align256(sizeof(SegDev) * plan.segs.size());
+    w.jgroups = w.jsegs + align256(sizeof(JoinSeg) * plan.jsegs.size());
+    w.sketches = w.jgroups + align256(sizeof(JoinGroup) * plan.jgroups.size());
     w.acc = w.sketches + align256(sizeof(SketchDev*) * (n_sketches + 1));
     w.hist = w.acc + align256(sizeof(AccDev) * (n_acc + 1));
     w.head = w.hist + align256(sizeof(u32) * (n_acc + 1));
@@ -1256,31 +1445,42 @@ static SearchLayout ws_layout(size_t n_segs, size_t n_sketches, size_t n_acc, u3
     w.sorted = w.sort_off + align256(sizeof(u32) * (n_acc + 2));
     w.longs = w.sorted + align256(sizeof(u32) * (size_t)surv_cap);
     w.total = w.longs + align256(sizeof(u32) * (size_t)surv_cap);
-    w.n_acc = (int)n_acc;
-    w.dense = 0;
+    w.n_acc = (int)n_acc; w.n_segs = (int)plan.segs.size(); w.n_jsegs = (int)plan.jsegs.size(); w.n_sketches = (int)n_sketches;
     w.surv_cap = surv_cap;
+    w.join_wide = plan.join_wide ? 1 : 0;
+    i64 most = 0;
+    w.dense = w.empty_domain = 0;
+    for (size_t i = 0; i < n_sketches; ++i) {
+        most = sk[i]->n_points > most ? sk[i]->n_points : most;
+        if (sk[i]->n_points == 0) w.empty_domain = 1;
+        for (const HoleHost& h : sk[i]->holes) if (h.second) w.dense = 1;      // (frequent filter hits)
+    }
+    w.max_chunks = (u32)((most + kVerifyChunk - 1) / kVerifyChunk);
     return w;
 }
 
-// Does some hole among the sketches take the second look (frequent filter hits)?
-static int any_dense(const xp_sketch* const* sk, size_t n) {
-    for (size_t i = 0; i < n; ++i)
-        for (const HoleHost& h : sk[i]->holes) if (h.second) return 1;
+// The smallest size with a match (0: none).
+static int least_size(const AccDev& a, int max_size) {
+    for (int k = 1; k <= max_size; ++k) if (a.match_count[k] > 0) return k;
     return 0;
 }
 
-// Chunks of the whole-domain check that the largest domain among the sketches needs.
-static u32 max_chunks_of(const xp_sketch* const* sk, size_t n) {
-    i64 most = 0;
-    for (size_t i = 0; i < n; ++i) most = sk[i]->n_points > most ? sk[i]->n_points : most;
-    return (u32)((most + kVerifyChunk - 1) / kVerifyChunk);
+// What a call sends to the device in one copy: counters at zero, segments, sketches, accumulators in their start state.
+static void stage_plan(char* stage, const SearchLayout& w, const Plan& plan, const xp_sketch* const* sketches) {
+    memset(stage, 0, 256);
+    if (!plan.segs.empty()) memcpy(stage + w.segs, plan.segs.data(), sizeof(SegDev) * plan.segs.size());
+    if (!plan.jsegs.empty()) memcpy(stage + w.jsegs, plan.jsegs.data(), sizeof(JoinSeg) * plan.jsegs.size());
+    if (!plan.jgroups.empty()) memcpy(stage + w.jgroups, plan.jgroups.data(), sizeof(JoinGroup) * plan.jgroups.size());
+    for (int i = 0; i < w.n_sketches; ++i) ((const SketchDev**)(stage + w.sketches))[i] = sketches[i]->d_s;
+    memcpy(stage + w.acc, plan.acc.data(), sizeof(AccDev) * plan.acc.size());
+    memset(stage + w.hist, 0, w.head - w.hist);
 }
 
 extern "C" size_t xp_workspace_bytes(const xp_sketch* const* sketches, size_t n, const xp_repair_opts* opts) {
     if (!sketches || n == 0) return 0;
     Plan plan;
     if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, &plan) != XP_OK) return 0;
-    return ws_layout(plan.segs.size(), n, plan.acc.size(), surv_cap_for(n)).total;
+    return ws_layout(plan, sketches, n, surv_cap_for(n)).total;
 }
 
 extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n, const xp_repair_opts* opts,
@@ -1297,8 +1497,7 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     if (st != XP_OK) return st;
     cudaStream_t stream = (cudaStream_t)o->stream;
 
-    SearchLayout w = ws_layout(plan.segs.size(), n, plan.acc.size(), surv_cap_for(n));
-    w.dense = any_dense(sketches, n);
+    const SearchLayout w = ws_layout(plan, sketches, n, surv_cap_for(n));
     char* ws = (char*)o->workspace;
     bool own_ws = false, cached_ws = false;
     if (ws) {
@@ -1321,58 +1520,58 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
         XP_CUDA(cudaMalloc((void**)&ws, w.total));
         own_ws = true;
     }
-    std::vector<char> stage(w.head, 0);
-    if (!plan.segs.empty()) memcpy(&stage[w.segs], plan.segs.data(), sizeof(SegDev) * plan.segs.size());
-    for (size_t i = 0; i < n; ++i) ((const SketchDev**)&stage[w.sketches])[i] = sketches[i]->d_s;
-    memcpy(&stage[w.acc], plan.acc.data(), sizeof(AccDev) * plan.acc.size());
-
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
     float ms = 0.f;
     int launches = 0;
-    std::vector<AccDev> acc(plan.acc.size());
-    u32 check_word = 0;
-#define XP_CUDA_R(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { if (own_ws) cudaFree(ws); if (cached_ws) g_ws_mu.unlock(); \
-        if (e0) cudaEventDestroy(e0); if (e1) cudaEventDestroy(e1); \
+    const size_t n_acc = plan.acc.size(), acc_bytes = sizeof(AccDev) * n_acc;
+    StageBlock stage(w.head + acc_bytes + 256);
+    EventPair ev;
+    auto give_back = [&]() { if (own_ws) cudaFree(ws); if (cached_ws) g_ws_mu.unlock(); };
+#define XP_CUDA_R(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { cudaStreamSynchronize(stream); give_back(); \
         return fail(e_ == cudaErrorMemoryAllocation ? XP_ERR_NOMEM : XP_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); } } while (0)
-    XP_CUDA_R(cudaEventCreate(&e0));
-    XP_CUDA_R(cudaEventCreate(&e1));
-    XP_CUDA_R(cudaMemcpyAsync(ws, stage.data(), w.head, cudaMemcpyHostToDevice, stream));
-    XP_CUDA_R(cudaEventRecord(e0, stream));
-    const int n_segs = (int)plan.segs.size(), n_acc = (int)plan.acc.size();
-    const u32 max_chunks = max_chunks_of(sketches, n);
+    if (!stage.p) { give_back(); return fail(XP_ERR_NOMEM, "out of host memory"); }
+    stage_plan(stage.p, w, plan, sketches);
+    const AccDev* acc = (const AccDev*)(stage.p + w.head);
+    u32* check_word = (u32*)(stage.p + w.head + acc_bytes);
+    *check_word = 0;
+    XP_CUDA_R(ev.open());
+    XP_CUDA_R(cudaMemcpyAsync(ws, stage.p, w.head, cudaMemcpyHostToDevice, stream));
+    XP_CUDA_R(cudaEventRecord(ev.e0, stream));
     xp_status stopped = XP_OK;
     if (!o->cancel && o->timeout_ms <= 0) {
-        XP_CUDA_R(launch_search_part(ws, w, 0, plan.n_tickets, false, n_segs, (int)n, max_chunks, stream, &launches));
+        XP_CUDA_R(launch_search_part(ws, w, true, 0, plan.n_join, false, stream, &launches));
+        XP_CUDA_R(launch_search_part(ws, w, false, 0, plan.n_tickets, false, stream, &launches));
     } else {
         // Bounded launches: the host waits for each and then looks at the cancel word and the clock.
         // Nothing on the device waits for either, and when the call gives up no kernel is in flight.
-        const u64 n_items = plan.n_tickets;
-        for (u64 t = 0; t < n_items && stopped == XP_OK; t += (u64)XP_CANCEL_TICKETS) {
-            const u64 t_end = t + (u64)XP_CANCEL_TICKETS < n_items ? t + (u64)XP_CANCEL_TICKETS : n_items;
-            XP_CUDA_R(launch_search_part(ws, w, t, t_end, t > 0, n_segs, (int)n, max_chunks, stream, &launches));
-            XP_CUDA_R(cudaStreamSynchronize(stream));
-            if (o->cancel && *o->cancel) stopped = XP_ERR_CANCELLED;
-            else if (o->timeout_ms > 0 && t_end < n_items &&
-                     std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count() >= (double)o->timeout_ms)
-                stopped = XP_ERR_TIMEOUT;
+        for (int kind = 0; kind < 2 && stopped == XP_OK; ++kind) {
+            const u64 n_items = kind == 0 ? plan.n_join : plan.n_tickets;
+            for (u64 t = 0; t < n_items && stopped == XP_OK; t += (u64)XP_CANCEL_TICKETS) {
+                const u64 t_end = t + (u64)XP_CANCEL_TICKETS < n_items ? t + (u64)XP_CANCEL_TICKETS : n_items;
+                XP_CUDA_R(launch_search_part(ws, w, kind == 0, t, t_end, t > 0, stream, &launches));
+                XP_CUDA_R(cudaStreamSynchronize(stream));
+                const bool more = t_end < n_items || (kind == 0 && plan.n_tickets > 0);
+                if (o->cancel && *o->cancel) stopped = XP_ERR_CANCELLED;
+                else if (o->timeout_ms > 0 && more &&
+                         std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count() >= (double)o->timeout_ms)
+                    stopped = XP_ERR_TIMEOUT;
+            }
         }
     }
     if (stopped == XP_OK) {
-        XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets > 0, n_segs, (int)n, n_acc, max_chunks, stream, &launches));
-        XP_CUDA_R(cudaEventRecord(e1, stream));
-        XP_CUDA_R(cudaMemcpyAsync(acc.data(), ws + w.acc, sizeof(AccDev) * acc.size(), cudaMemcpyDeviceToHost, stream));
-        XP_CUDA_R(cudaMemcpyAsync(&check_word, ws + 20, sizeof(check_word), cudaMemcpyDeviceToHost, stream));
+        XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets + plan.n_join > 0, stream, &launches));
+        XP_CUDA_R(cudaEventRecord(ev.e1, stream));
+        XP_CUDA_R(cudaMemcpyAsync(stage.p + w.head, ws + w.acc, acc_bytes, cudaMemcpyDeviceToHost, stream));
+#ifdef XP_CHECKS
+        XP_CUDA_R(cudaMemcpyAsync(check_word, ws + 20, sizeof(*check_word), cudaMemcpyDeviceToHost, stream));
+#endif
         XP_CUDA_R(cudaStreamSynchronize(stream));
-        XP_CUDA_R(cudaEventElapsedTime(&ms, e0, e1));
+        XP_CUDA_R(cudaEventElapsedTime(&ms, ev.e0, ev.e1));
     }
 #undef XP_CUDA_R
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (own_ws) cudaFree(ws);
-    if (cached_ws) g_ws_mu.unlock();
+    give_back();
     if (stopped == XP_ERR_CANCELLED) return fail(stopped, "cancelled between launches (" + std::to_string(launches) + " done)");
     if (stopped == XP_ERR_TIMEOUT) return fail(stopped, "time limit of " + std::to_string((long long)o->timeout_ms) + " ms reached between launches (" + std::to_string(launches) + " done)");
-    if (check_word != 0) return fail(XP_ERR_CUDA, "an index check of the checked build failed (code " + std::to_string(check_word) + ")");
+    if (*check_word != 0) return fail(XP_ERR_CUDA, "an index check of the checked build failed (code " + std::to_string(*check_word) + ")");
 
     size_t ai = 0;
     for (size_t i = 0; i < n; ++i) {
@@ -1394,9 +1593,9 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
             hr.evals = a.evals + a.filter_tests; hr.filter_survivors = a.filter_survivors; hr.probe_survivors = a.probe_survivors;
             hr.filter_tests = a.filter_tests;
             hr.skipped = a.tile_cands > a.filter_tests ? a.tile_cands - a.filter_tests : 0;
-            hr.nominal_ops = plan.nominal_ops[ai] - (a.ops_skipped < plan.nominal_ops[ai] ? a.ops_skipped : plan.nominal_ops[ai]);
-            const int ls = (int)a.pad;
-            if (ls >= 1 && ls <= hr.max_size && a.match_count[ls] > 0) {
+            hr.nominal_ops = plan.nominal_ops[ai] - (a.ops_skipped < plan.nominal_ops[ai] ? a.ops_skipped : plan.nominal_ops[ai]) + 2 * a.join_tests;
+            const int ls = least_size(a, hr.max_size);
+            if (ls >= 1) {
                 hr.solved = 1; hr.least_size = ls; hr.least_rank = a.min_rank[ls];
                 host_unrank(s->g, s->holes[h].start_nt, ls, hr.least_rank, &hr.code, &hr.text);
             }
@@ -1404,7 +1603,7 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
         r->kernel_ms = ms;
         r->n_launches = launches;
         r->h2d_bytes = w.head;
-        r->d2h_bytes = sizeof(AccDev) * acc.size() + sizeof(check_word);
+        r->d2h_bytes = acc_bytes;
         outs[i] = r;
     }
     const double total = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -1430,24 +1629,22 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
     xp_status st = build_plan(&sketch, 1, o, &plan);
     if (st == XP_OK) st = check_device(&sketch, 1);
     if (st != XP_OK) return st;
-    SearchLayout w = ws_layout(plan.segs.size(), 1, plan.acc.size(), kSurvCapStatic);
-    w.dense = any_dense(&sketch, 1);
+    const SearchLayout w = ws_layout(plan, &sketch, 1, kSurvCapStatic);
     if (plan.acc.size() > 64)
         return fail(XP_ERR_TOO_LARGE, "xp_repair_static: the sketch has more than 64 holes; use xp_repair with a workspace");
     if (w.total > kStaticScratchBytes)
         return fail(XP_ERR_TOO_LARGE, "xp_repair_static: the call needs " + std::to_string(w.total) +
                     " bytes of scratch, the fixed array holds " + std::to_string(kStaticScratchBytes) +
                     "; use xp_repair with a workspace");
-    static thread_local char stage[kStaticScratchBytes];          // no heap use that grows with the call
-    memset(stage, 0, w.head);
-    if (!plan.segs.empty()) memcpy(&stage[w.segs], plan.segs.data(), sizeof(SegDev) * plan.segs.size());
-    ((const SketchDev**)&stage[w.sketches])[0] = sketch->d_s;
-    memcpy(&stage[w.acc], plan.acc.data(), sizeof(AccDev) * plan.acc.size());
-    AccDev acc[64];
+    StageBlock stage(w.head + sizeof(AccDev) * plan.acc.size());       // (page-locked host memory that the library keeps)
+    if (!stage.p) return fail(XP_ERR_NOMEM, "out of host memory");
+    stage_plan(stage.p, w, plan, &sketch);
+    const AccDev* acc = (const AccDev*)(stage.p + w.head);
     cudaStream_t stream = (cudaStream_t)o->stream;
-    XP_CUDA(launch_search_static(stage, w, plan.n_tickets, (int)plan.segs.size(), (int)plan.acc.size(),
-                                 max_chunks_of(&sketch, 1), acc, stream));
-    XP_CUDA(cudaStreamSynchronize(stream));
+    cudaError_t e = launch_search_static(stage.p, w, plan.n_tickets, plan.n_join, (AccDev*)(stage.p + w.head), stream);
+    const cudaError_t e2 = cudaStreamSynchronize(stream);         // (before the staging block goes back, whatever happened)
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess) return fail(XP_ERR_CUDA, std::string("xp_repair_static: ") + cudaGetErrorString(e));
     for (int h = 0; h < sketch->n_holes; ++h) {
         xp_hole_summary& r = out[h];
         memset(&r, 0, sizeof(r));
@@ -1458,8 +1655,8 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
             r.match_count[k] = a.match_count[k];
         }
         r.evals_executed = a.evals + a.filter_tests;
-        const int ls = (int)a.pad;
-        if (ls >= 1 && ls <= r.max_size && a.match_count[ls] > 0) {
+        const int ls = least_size(a, r.max_size);
+        if (ls >= 1) {
             r.solved = 1; r.least_size = ls; r.least_rank = a.min_rank[ls];
             std::vector<xp_instr> code;
             std::string text;

@@ -31,8 +31,6 @@ constexpr u64 kStageMaxPoints = 1ull << 26;  // largest box whose points and spe
 constexpr int kProgMax = 64;          // candidate substituted into its context: longest staged program
 constexpr u64 kTabBudgetBytes = 64ull << 20;   // subtree-value tables of one hole, all probes together
 constexpr u64 kTabMaxEntries = 1ull << 22;   // largest (nonterminal, size) subtree-value table per hole
-constexpr u64 kBigMaxEntries = 1ull << 30;   // ... of the one further size that is tabulated at the first probe only
-constexpr u64 kBigBudgetBytes = 12ull << 30; // ... and its bytes (9 per entry), per hole
 constexpr u32 kOpBit = 0x80000000u;  // candidate code word: operator (low bits = XP_OP_*) or leaf index
 constexpr int kMaxFamily = 8;         // tile segments that may share one fill of the register-side operands (a hit's
                                       // queue entry names its member in 3 bits)
@@ -44,14 +42,46 @@ struct LeafDev { i32 var; i32 pad; i64 value; };
 // precede its first tree (off[s]), i.e. the rank offset of the production at that size.
 struct BinDev { i32 op, lnt, rnt, pad; u64 off[kMaxSize + 2]; };
 
+struct ConstDev;
 struct GrammarDev {
     i32 n_vars, n_nt, n_leaves, n_bins;
     i32 leaf_begin[kMaxNt + 1];      // leaves of nonterminal nt: leaves[leaf_begin[nt] .. leaf_begin[nt+1])
     i32 bin_begin[kMaxNt + 1];       // binary productions of nt: bins[bin_begin[nt] .. bin_begin[nt+1])
     u64 cnt[kMaxNt][kMaxSize + 1];   // trees of nt with exactly s nodes
+    i32 const_begin[kMaxNt + 1];     // constants of nt, ascending: consts[const_begin[nt] .. var_begin[nt]); then its
+    i32 var_begin[kMaxNt];           // variables: consts[var_begin[nt] .. const_begin[nt+1]), value = variable
     const LeafDev* leaves;           // device
     const BinDev* bins;              // device
+    const ConstDev* consts;          // device
 };
+
+// ---- the leaf join (csrc/xp_join.cuh) ----
+//
+// Candidates  E op leaf  and  leaf op E  are not tested one by one: a thread holds the operand E's values at two
+// probes (a0, a1) and asks, per operator, for which leaves the result can be the target at both.  Constants have the
+// same value at both probes, so one condition on (a0, a1) decides all of them at once; the variables, and constants
+// when there are only a few, are entries that are tested one by one.
+constexpr int kOpSlots = 9;           // + - * / % min max << >> (in this order; the last two only in the exact form)
+constexpr int kJoinEntries = 12;      // most leaves of a nonterminal that are tested one by one
+constexpr int kJoinFewConsts = 4;     // constants up to this many are entries too
+struct __align__(16) JoinEntry {
+    u32 v0, v1, u0, u1;               // value at the two probes, and its magnitude
+    u32 low0, low1, cm0, cm1;         // as divisor: |target| * |v| (0x80000000: never); floor((2^32-1) / |v|), 0 when the remainder is impossible
+    u32 inv0, inv1, k0k1, pos;        // inverse of |v|'s odd part, trailing zero bits (k0 | k1 << 8); position among the nonterminal's leaves
+};
+struct JoinSet {                      // the leaves of one nonterminal, for one hole
+    i32 ok;                           // every value is below 2^31 in magnitude and the entries fit
+    i32 n_entries, n_const;           // n_const: constants decided as a set (0 when they are entries)
+    i32 cmin, cmax;                   // ... their range
+    u32 cabs;                         // ... and largest magnitude
+    u32 lim;                          // operands of this magnitude or more are left to the exact form
+    u32 mm;                           // bit 0 / 1: the target at probe 0 / 1 is one of the constants (min and max)
+    i32 const_begin;                  // into GrammarDev::consts (ascending)
+    i32 pad[3];
+    JoinEntry e[kJoinEntries];
+};
+
+struct ConstDev { i64 value; i32 pos, pad; };    // a constant leaf of a nonterminal (position among its leaves)
 
 struct HoleDev {
     i32 start_nt, max_size, ctx_len, spec_len;   // spec_len == 0: the spec is a table
@@ -88,9 +118,8 @@ struct HoleDev {
     // probes without tables need the candidate unranked in full.
     // second: filter hits are also checked exactly at probe 1 before they are queued (needs tables, a
     // defined spec and an affine context at probe 1); sample_pass0: how many of the sample_n small
-    // candidates sampled at load satisfied probe 0, sample_big: how many of the kPrepBigSamples random
-    // candidates of the largest size did (a high rate of either makes the second look worth its cost).
-    i32 second, sample_pass0, sample_n, sample_big;
+    // candidates sampled at load satisfied probe 0 (a high rate makes the second look worth its cost).
+    i32 second, sample_pass0, sample_n, pad4;
     i32 second_ok;                                // the second look is possible (tables, spec and context at probe 1): a
                                                   // CTA that sees many filter hits for this hole turns it on for itself
     // Set by the host before the load's kernels run: the largest subtree size and the number of
@@ -100,17 +129,6 @@ struct HoleDev {
     i32 tab_size_cap, tab_probes_cap, small_search;
     i32 filter_ok;                                // the probe filter applies: probe 0 exists, its context is affine or compares
     i32 tab_max_size, tab_probes;
-    // One size further (big_size = the next size above tab_size_cap that has trees, when operands of that size occur and its trees fit
-    // kBigMaxEntries / kBigBudgetBytes) the values are tabulated at probe 0 ONLY: these are the register-side
-    // operands of the largest candidates (config 4: 5.9e8 subtrees of size 7, 5.3 GB), which every search
-    // would otherwise rebuild from the smaller tables tile by tile -- a third of such a search's time.
-    // The memory of a B200 has room for them; they stay resident with the sketch.  big_on is set by the
-    // load's kernels once the smaller tables exist at probe 0.
-    i32 big_size, big_on;
-    u64 big_off[kMaxNt];                          // first entry of each nonterminal
-    u64 big_total;
-    i64* big_val;                                 // device
-    unsigned char* big_ok;                        // device
     u64 tab_total;
     u64 tab_off[kMaxNt][kMaxSize + 1];
     i64* tab_val;                                 // device
@@ -120,6 +138,17 @@ struct HoleDev {
     // caller's table).  On a box domain a candidate is checked on the sub-box of these and its
     // own variables only: no other variable can change either side of the constraint.
     u32 fixed_vars, pad2;
+    // The leaf join: values (a0, a1) at its two probes of every tabulated subtree, 8 bytes each (same index as
+    // tab_val; a0 = kPairNone: undefined at one of them (a1 = 0) or not below 2^31 in magnitude (a1 = 1)); the leaf sets
+    // of the nonterminals; the targets.  join_on: the context is affine at both probes with a factor that 32 bits hold.
+    i32 join_on, join_p1;                         // second probe (0 when there is only one that serves)
+    i32 join_none, n_exact;                       // no value below the operand limit can be the target; probes checked from the tables
+    i64 join_t0, join_t1;                         // hole values that satisfy the constraint at the two probes
+    u64 join_tmod;                                // largest |target| over the probes: a remainder's divisor must exceed it
+    float join_rt0, join_rt1, join_rl0, join_rl1; // 1 / |target| (0 for 0), 1 / (|target| + 1)
+    float join_h0, join_h1;                       // a huge number where the target is 0, else 0
+    JoinSet* join_sets;                           // device, one per nonterminal
+    i32* tab_pair;                                // device
     // Points that ended a survivor's whole-domain check (a candidate that passed every probe and then
     // failed somewhere): a small open-addressed table of point ids (-1: free) with the number of
     // survivors each has ended.  Written by verify_kernel, read and cleared by xp_sketch_refine, which
@@ -132,7 +161,7 @@ constexpr int kKillSlots = 64;
 struct SketchDev {
     const GrammarDev* g;                          // device
     i32 n_vars, n_holes, domain_kind, n_samples;
-    i32 prep_cands, project;                      // project: box domain with staged points (see HoleDev::fixed_vars)                         // sampled candidates the probe choice is based on (<= 1024)
+    i32 pad, project;                             // project: box domain with staged points (see HoleDev::fixed_vars)
     i64 n_points;
     const i32* coords;                            // device: the points of a table domain, or the staged
                                                   // points of a box (null: derive them from the point id)
@@ -154,9 +183,33 @@ struct AccDev {
     u64 filter_survivors, probe_survivors, pad;
     u64 ops_skipped;                 // cost-model operations that the filter did not have to carry out (remainders
                                      // of a tile none of whose divisors exceeds the target's magnitude)
-    u64 filter_tests;                // filter-stage tests at probe 0 that ran: (register operand defined there) x
-                                     // (broadcast operand defined there) x (operators whose loop was entered)
-    u64 tile_cands;                  // candidates of the tiles visited, tested or not
+    u64 filter_tests;                // filter-stage tests that ran.  Tiles: (register operand defined at probe 0) x (broadcast
+                                     // operand defined there) x (operators whose loop was entered); leaf join: operands
+                                     // defined at the probes x (entries tested one by one + one for a set of constants) x operators
+    u64 tile_cands;                  // candidates of the tiles and joins visited, tested or not
+    u64 join_tests;                  // ... filter_tests that the leaf join ran
+};
+constexpr i32 kPairNone = (i32)0x80000000u;
+
+// A piece of the leaf join's work: operands e_begin .. e_begin + e_count of (nt, esize), each against the leaves of
+// n_groups nonterminals.  kJoinDirect: candidates of (nt, esize) themselves, e_begin .. , checked on the probes one by one.
+enum { kJoinLeaf = 0, kJoinDirect = 1 };
+constexpr int kJoinGroups = 8;        // most groups of a segment
+struct JoinGroup {
+    i32 leaf_nt, pad;
+    u32 fmask, smask;                // operator slots of  E op leaf  and  leaf op E
+    u64 base[2][kOpSlots];           // rank of (E 0, leaf 0) per operator: forward, swapped
+};
+struct JoinSeg {
+    u64 first_ticket;
+    u64 rank_begin, rank_end;        // window of ranks searched at this size
+    i32 sketch, hole, size, kind;
+    i32 acc, nt, esize, n_groups;
+    i32 first_group;
+    i32 exact;                       // the operators have no condition (shifts): every candidate is evaluated on its own
+    u32 chunk;                       // operands per ticket
+    i32 pad;
+    u64 e_begin, e_count;
 };
 
 // One contiguous piece of work.  kind 0 (linear): ranks [rank_begin, rank_end) of `size`,
@@ -205,6 +258,11 @@ struct PlanDev {
     u64 n_tickets;
     i32 n_segs, n_sketches;
     const SegDev* segs;              // device
+    const JoinSeg* jsegs;            // device
+    const JoinGroup* jgroups;        // device
+    i32 n_jsegs, pad0;
+    u64 join_base, n_join;           // tickets of the leaf join that belong to this launch
+    u64* join_ticket;                // device counter, zero at launch
     const SketchDev* const* sketches;  // device table of device pointers
     AccDev* acc;                     // device
     u64* ticket;                     // device counter, zero at launch

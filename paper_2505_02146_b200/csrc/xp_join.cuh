@@ -1,0 +1,1033 @@
+// The leaf join: candidates  E op leaf  and  leaf op E, decided from the operand's side.
+//
+// Nearly all candidates of a search have a leaf as one operand of their root (a free grammar of 136 leaves at size 7:
+// four in five; the typed grammar with 257 multipliers and 128 divisors at size 9: 97 %).  Testing them one by one costs
+// operands x leaves x operators.  Here a thread computes an operand's values (a0, a1) at two probes and asks per operator
+// for which leaves the result can be the target (t0, t1) at both:
+//   constants c have ONE value at both probes, so
+//     a + c = t   needs  a0 - a1 = t0 - t1, and c = t0 - a0 in the constants' range       (a - c and c - a likewise);
+//     a * c = t   needs  a0 * t1 = a1 * t0;
+//     a / c = t   needs  an integer |c| in (|a|/(|t|+1), |a|/|t|] at both probes          (single precision, widened);
+//     c / a = t   needs  |c| in [|t||a|, (|t|+1)|a|) at both;
+//     a % c = t   needs  |c| to divide |a| - |t| at both and to exceed the target at EVERY probe (a greatest common divisor);
+//     c % a = t   needs  |c| = |t| mod |a| at both (stepping through the few such |c|);
+//     min, max    need   c = t0 or c = t1, or a itself to be the target at both;
+//   variables (and constants when a nonterminal has four or fewer) are entries tested one by one, at both probes.
+// These are necessary conditions in 32-bit arithmetic for operands below JoinSet::lim in magnitude.  An operand that passes
+// one (a suspect) waits in the warp's first queue until 32 have gathered; then every lane takes one, finds the leaves its
+// conditions leave open (binary search among the sorted constants) and holds each against both probes.  What is left
+// goes to a second queue, and 32 at a time (a lane each, none idle) are checked exactly, in 64 bits, at the other probes.
+// A context that compares asks for an interval of values at every probe: sums and differences with a constant
+// are decided by intersecting the intervals over all probes, the other operators leaf by leaf with an early exit.
+// Operands of JoinSet::lim or more and shifts take the exact form: one operand at a time, lanes over the leaves.
+// Warps work on their own; nothing here waits for another warp.
+#pragma once
+
+namespace xp {
+
+constexpr int kJoinThreads = 256;
+constexpr int kJoinWarps = kJoinThreads / 32;
+constexpr int kJoinP = 4;                                 // operands per lane and step
+constexpr u32 kJoinQueue = 32 + 32 * kJoinP;              // suspects: fewer than 32 wait when a step adds up to 32 per operand of a lane
+
+// What the conditions need of one group (leaf set) of the segment at hand.
+struct GroupCtx {
+    u32 cf, cs, ef, es;                                   // operators whose condition can hold: constants, entries; forward, swapped
+    i32 cmin, cmax;
+    u32 cabs, mm;
+    float fc;
+    i32 n_entries, tests;                                 // tests: what an operand counts for in filter_tests
+    const JoinSet* set;
+};
+
+struct JoinWarp {
+    u32 q_off[kJoinQueue];                                // suspects: operand number relative to the segment's first,
+    i32 q_a0[kJoinQueue], q_a1[kJoinQueue];               //   its values at the two probes
+    u32 c_off[64], c_pos[64], c_code[64];                 // candidates: operand, leaf position, group << 8 | slot << 1 | swapped
+    u32 nc;                                               // candidates waiting
+    GroupCtx grp[kJoinGroups];
+    CandShared cand;                                      // candidate of a whole-domain check that the warp does itself
+};
+
+// What a warp has counted for the accumulator it works on (the sums over lanes are taken when it moves on).
+struct JoinCount { u64 evals; u64 tests, cands; u32 suspects, passes; };
+
+// An operand subtree by reference: a table entry, an operation on two table entries, or (mode 2) its rank.
+struct OperandRef { i32 mode, op; u64 a, b; };
+
+__device__ __forceinline__ OperandRef operand_ref(const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank) {
+    OperandRef r;
+    r.op = 0; r.b = 0;
+    const int tmax = hole->tab_max_size;
+    if (size <= tmax) { r.mode = 0; r.a = hole->tab_off[nt][size] + rank; return r; }
+    if (tmax >= 1 && size >= 3) {
+        int lnt, rnt, a;
+        u64 l, q;
+        unrank_root(g, nt, size, rank, r.op, lnt, rnt, a, l, q);
+        if (a <= tmax && size - 1 - a <= tmax) {
+            r.mode = 1; r.a = hole->tab_off[lnt][a] + l; r.b = hole->tab_off[rnt][size - 1 - a] + q;
+            return r;
+        }
+    }
+    r.mode = 2; r.a = rank;
+    return r;
+}
+
+__device__ __noinline__ bool ref_value_full(const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank, int j, i64& v) {
+    u32 code[kMaxSize];
+    const int n = unrank(g, nt, size, rank, code);
+    return eval_cand(code, n, g->leaves, hole->probe_pt[j], v);
+}
+
+__device__ __forceinline__ bool ref_value(const GrammarDev* g, const HoleDev* hole, const OperandRef& r, int nt, int size, int j, i64& v) {
+    if (r.mode == 2) return ref_value_full(g, hole, nt, size, r.a, j, v);
+    const u64 base = (u64)j * hole->tab_total;
+    if (!XP_CHECKED(j < hole->tab_probes && r.a < hole->tab_total && r.b < hole->tab_total, kChkTable)) return false;
+    if (!hole->tab_ok[base + r.a]) return false;
+    v = hole->tab_val[base + r.a];
+    if (r.mode == 0) return true;
+    if (!hole->tab_ok[base + r.b]) return false;
+    return apply_op(r.op, v, hole->tab_val[base + r.b], v);
+}
+
+__device__ __forceinline__ u32 ref_vars(const HoleDev* hole, const OperandRef& r) {
+    if (r.mode == 2) return 0xffu;                        // (always a safe answer)
+    return (u32)hole->tab_vars[r.a] | (r.mode == 1 ? (u32)hole->tab_vars[r.b] : 0u);
+}
+
+// Does hole value v satisfy the constraint at probe j (one of the first n_exact)?
+__device__ __forceinline__ bool probe_accepts(const HoleDev* hole, int j, i64 v) {
+    if ((hole->aff_okmask >> j) & 1u) return (u64)v * hole->aff_Aj[j] + hole->aff_Bj[j] == (u64)hole->probe_spec[j];
+    if (v > -(1ll << 62) && v < (1ll << 62)) return v >= hole->rng_lo[j] && v <= hole->rng_hi[j];
+    return true;                                          // (a value of 2^62 or more is left to the whole-domain check)
+}
+
+__device__ __forceinline__ int op_of_slot(int slot) { return slot <= 4 ? slot : slot <= 6 ? slot - 5 + XP_OP_MIN : slot - 7 + XP_OP_SHL; }
+
+// The candidate (operand, leaf) at the probes that have tables, in order; the first failure ends it.
+__device__ __forceinline__ bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
+                                           bool swap, int op, int from, int n_exact, u64& evals) {
+    for (int j = from; j < n_exact; ++j) {
+        ++evals;
+        i64 a, v;
+        if (!ref_value(g, hole, ref, nt, esize, j, a)) return false;
+        const i64 c = var >= 0 ? hole->probe_pt[j][var] : cval;
+        if (!apply_op(op, swap ? c : a, swap ? a : c, v) || !probe_accepts(hole, j, v)) return false;
+    }
+    return true;
+}
+
+// The warp checks one candidate on the whole domain itself (the survivor queue is full).
+__device__ __noinline__ void join_verify(JoinWarp& w, const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, int size, int acc, u64 rank,
+                                         u32 vars, u64& evals) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane == 0) { stage_candidate(w.cand, sk, hole, size, rank); (void)proj_points(sk, hole, vars, &w.cand); }
+    __syncwarp();
+    i64 fail_pid = 0;
+    const bool ok = check_points(w.cand, sk, hole, 0, proj_points(sk, hole, vars, nullptr), evals, &fail_pid);
+    if (ok && lane == 0) {
+        atomicAdd(&plan.acc[acc].match_count[size], 1ull);
+        atomicMin(&plan.acc[acc].min_rank[size], rank);
+    }
+    __syncwarp();
+}
+
+// Candidates that passed the probes (one per lane at most) go to the survivor queue, or are checked
+// by the warp.  Called by all 32 lanes together.
+__device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, const JoinSeg& seg,
+                                             bool pass, u64 rank, u32 vars, JoinCount& n) {
+    u32 m = __ballot_sync(0xffffffffu, pass);
+    if (!m) return;
+    n.passes += (u32)__popc(m);
+    const bool pending = pass && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
+    m = __ballot_sync(0xffffffffu, pending);
+    while (m) {
+        const int src = __ffs((int)m) - 1;
+        m &= m - 1;
+        join_verify(w, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
+    }
+}
+
+// Probes without tables: the candidate is rebuilt in full.
+__device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev* hole, int size, u64 rank, u64& evals) {
+    u32 code[kMaxSize];
+    const int n = unrank(g, hole->start_nt, size, rank, code);
+    return probe_check(g, hole, code, n, evals);
+}
+
+// The candidates in the warp's second queue, one per lane: the probes from `from` on, exactly.  Called by all lanes.
+__device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, int from, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const u32 nc = w.nc;
+    for (u32 at = 0; at < nc; at += 32) {
+        bool pass = false;
+        u64 rank = 0;
+        u32 vars = 0;
+        if (at + lane < nc) {
+            const u32 code = w.c_code[at + lane], pos = w.c_pos[at + lane];
+            const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u);
+            const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code >> 8)];
+            const u64 e = seg.e_begin + w.c_off[at + lane];
+            const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
+            rank = grp.base[swap][slot] + (swap ? (u64)pos * ne + e : e * nl + (u64)pos);
+            if (rank >= seg.rank_begin && rank < seg.rank_end &&
+                XP_CHECKED(e < ne && (u64)pos < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue)) {
+                const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
+                const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
+                pass = exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals);
+                if (pass && hole->n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
+                vars = ref_vars(hole, ref) | (lf.var >= 0 ? 1u << lf.var : 0u);
+            }
+        }
+        join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
+    }
+    __syncwarp();
+    if (lane == 0) w.nc = 0;
+    __syncwarp();
+}
+
+// Lanes with a candidate put it into the second queue (checked when a warp's worth has gathered).  Called by all lanes.
+__device__ __forceinline__ void join_push(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, bool have,
+                                          u32 off, u32 pos, int group, int slot, int swap, int from, JoinCount& n) {
+    const u32 b = __ballot_sync(0xffffffffu, have);
+    if (!b) return;
+    const int lane = threadIdx.x & 31;
+    const u32 nc = w.nc;
+    if (have) {
+        const u32 at = nc + (u32)__popc(b & ((1u << lane) - 1u));      // (nc < 32)
+        w.c_off[at] = off; w.c_pos[at] = pos; w.c_code[at] = ((u32)group << 8) | ((u32)slot << 1) | (u32)swap;
+    }
+    __syncwarp();
+    if (lane == 0) w.nc = nc + (u32)__popc(b);
+    __syncwarp();
+    if (nc + (u32)__popc(b) >= 32u) join_check(w, plan, seg, sk, hole, from, n);
+}
+
+// ---- the conditions ----
+
+struct JoinCtx {                                          // what the conditions need of the hole
+    u32 t0, t1, ut0, ut1;                                 // targets (low words) and their magnitudes (0 where 31 bits do not hold them)
+    float rt0, rt1, rl0, rl1, h0, h1, ft0, ft1;           // 1/|t|, 1/(|t|+1), huge where t = 0, |t|
+    u32 tmod;
+    bool tz, small;                                       // both targets are zero; both are below 2^31
+};
+
+__device__ __forceinline__ bool in_range(u32 c, const GroupCtx& s) { return c - (u32)s.cmin <= (u32)s.cmax - (u32)s.cmin; }
+
+// a * c = t at both probes for some c, given that a0 * t1 = a1 * t0: the operand divides the target.
+__device__ __noinline__ bool factor_exists(i32 a0, i32 a1, const JoinCtx& x, u32 cabs) {
+    if (!x.small) return true;                            // (decided when the suspect is taken up)
+    const u32 u = a0 != 0 ? abs_u32(a0) : abs_u32(a1), t = a0 != 0 ? x.ut0 : x.ut1;
+    if (a0 == 0 && x.ut0 != 0u) return false;
+    return u == 0u ? t == 0u : t % u == 0u && t / u <= cabs;
+}
+
+__device__ __noinline__ bool gcd_exceeds(u32 x, u32 y, u32 least) {      // gcd(x, y) > least (gcd(0, 0) counts as infinite)
+    if (x == 0u && y == 0u) return true;
+    while (y != 0u) {
+        if (y <= least) return false;                     // the divisor sought divides y, and exceeds `least`
+        const u32 r = x % y;
+        x = y; y = r;
+    }
+    return x > least;
+}
+
+// Is there a magnitude m <= cabs with m mod u0 = ut0 and m mod u1 = ut1?  Stepping along the larger of the two.
+__device__ __noinline__ bool residue_exists(u32 u0, u32 u1, u32 ut0, u32 ut1, u32 cabs) {
+    if (u0 <= ut0 || u1 <= ut1) return false;
+    if (u0 < u1) { u32 s = u0; u0 = u1; u1 = s; s = ut0; ut0 = ut1; ut1 = s; }
+    for (u64 m = ut0; m <= cabs; m += u0) if ((u32)m % u1 == ut1) return true;
+    return false;
+}
+
+enum { kSlotAdd = 0, kSlotSub = 1, kSlotMul = 2, kSlotDiv = 3, kSlotMod = 4, kSlotMn = 5, kSlotMx = 6 };
+
+__device__ __forceinline__ bool const_div_fwd(float f0, float f1, const JoinCtx& x, float fc) {       // some |c| in (|a|/(|t|+1), |a|/|t|] at both
+    const float hi = fminf(f0 * x.rt0 + x.h0, f1 * x.rt1 + x.h1) * 1.000002f, lo = fmaxf(f0 * x.rl0, f1 * x.rl1) * 0.999998f;
+    const float c = floorf(fminf(hi, fc));
+    return c >= 1.f && c > lo;
+}
+__device__ __forceinline__ bool const_div_swap(float f0, float f1, const JoinCtx& x, float fc) {      // some |c| in [|t||a|, (|t|+1)|a|) at both
+    const float lo = fmaxf(f0 * x.ft0, f1 * x.ft1) * 0.999998f;
+    const float hi = fminf(f0 * (x.ft0 + 1.f), f1 * (x.ft1 + 1.f)) * 1.000002f;
+    return lo < hi && lo <= fc;
+}
+__device__ __forceinline__ bool const_minmax(i32 a0, i32 a1, const JoinCtx& x, u32 mm, bool mx) {
+    const i32 t0 = (i32)x.t0, t1 = (i32)x.t1;
+    auto f = [&](i32 a, i32 b) { return mx ? (a > b ? a : b) : (a < b ? a : b); };
+    bool h = a0 == t0 && a1 == t1;
+    if (mm & 1u) h |= f(a0, t0) == t0 && f(a1, t0) == t1;
+    if (mm & 2u) h |= f(a0, t1) == t0 && f(a1, t1) == t1;
+    return h;
+}
+
+// One condition on one operand (used again when a suspect is taken up): constants, operator slot, side.
+__device__ __forceinline__ bool const_condition(int slot, int swap, i32 a0, i32 a1, const JoinCtx& x, const GroupCtx& s) {
+    const u32 u0 = abs_u32(a0), u1 = abs_u32(a1);
+    switch (slot) {
+        case kSlotAdd: return (u32)a0 - (u32)a1 == x.t0 - x.t1 && in_range(x.t0 - (u32)a0, s);
+        case kSlotSub: return swap ? (u32)a0 - (u32)a1 == x.t1 - x.t0 && in_range(x.t0 + (u32)a0, s)
+                                   : (u32)a0 - (u32)a1 == x.t0 - x.t1 && in_range((u32)a0 - x.t0, s);
+        case kSlotMul: return (u32)a0 * x.t1 == (u32)a1 * x.t0 && factor_exists(a0, a1, x, s.cabs);
+        case kSlotDiv: return swap ? const_div_swap((float)u0, (float)u1, x, s.fc) : const_div_fwd((float)u0, (float)u1, x, s.fc);
+        case kSlotMod: return swap ? residue_exists(u0, u1, x.ut0, x.ut1, s.cabs)
+                                   : u0 >= x.ut0 && u1 >= x.ut1 && gcd_exceeds(u0 - x.ut0, u1 - x.ut1, x.tmod);
+        case kSlotMn: return const_minmax(a0, a1, x, s.mm, false);
+        case kSlotMx: return const_minmax(a0, a1, x, s.mm, true);
+    }
+    return false;
+}
+
+// The entry's candidates at the two probes, for the operators in f (E op entry) and s (entry op E).
+template <int P>
+__device__ __forceinline__ void entry_conditions(const JoinEntry& e, u32 f, u32 s, const i32 (&a0)[P], const i32 (&a1)[P], const JoinCtx& x, bool (&any)[P]) {
+    if ((f | s) & (1u << kSlotAdd)) {
+        const u32 d0 = x.t0 - e.v0, d1 = x.t1 - e.v1;
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= (u32)a0[p] == d0 && (u32)a1[p] == d1;
+    }
+    if (f & (1u << kSlotSub)) {
+        const u32 d0 = x.t0 + e.v0, d1 = x.t1 + e.v1;
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= (u32)a0[p] == d0 && (u32)a1[p] == d1;
+    }
+    if (s & (1u << kSlotSub)) {
+        const u32 d0 = e.v0 - x.t0, d1 = e.v1 - x.t1;
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= (u32)a0[p] == d0 && (u32)a1[p] == d1;
+    }
+    if ((f | s) & (1u << kSlotMul)) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= (u32)a0[p] * e.v0 == x.t0 && (u32)a1[p] * e.v1 == x.t1;
+    }
+    if ((f & (1u << kSlotDiv)) && e.u0 != 0u && e.u1 != 0u) {              // floor(|a| / |v|) = |t|  <=>  |a| - |t||v| < |v|
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= abs_u32(a0[p]) - e.low0 < e.u0 && abs_u32(a1[p]) - e.low1 < e.u1;
+    }
+    if (s & (1u << kSlotDiv)) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const u32 u0 = abs_u32(a0[p]), u1 = abs_u32(a1[p]);
+            any[p] |= e.u0 - u0 * x.ut0 < u0 && e.u1 - u1 * x.ut1 < u1;    // (a product past 32 bits can only let more through)
+        }
+    }
+    if ((f & (1u << kSlotMod)) && e.cm0 != 0u && e.cm1 != 0u) {            // |v| divides |a| - |t|
+        const u32 k0 = e.k0k1 & 255u, k1 = e.k0k1 >> 8;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const u32 u0 = abs_u32(a0[p]), u1 = abs_u32(a1[p]);
+            any[p] |= u0 >= x.ut0 && rotr32((u0 - x.ut0) * e.inv0, k0) <= e.cm0 && u1 >= x.ut1 && rotr32((u1 - x.ut1) * e.inv1, k1) <= e.cm1;
+        }
+    }
+    if ((s & (1u << kSlotMod)) && e.u0 >= x.ut0 && e.u1 >= x.ut1) {        // |a| divides |v| - |t| and exceeds |t|
+        const u32 y0 = e.u0 - x.ut0, y1 = e.u1 - x.ut1;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const u32 u0 = abs_u32(a0[p]), u1 = abs_u32(a1[p]);
+            if (u0 > x.ut0 && u1 > x.ut1 && (u0 <= y0 || y0 == 0u) && (u1 <= y1 || y1 == 0u)) any[p] |= y0 % u0 == 0u && y1 % u1 == 0u;
+        }
+    }
+    if ((f | s) & (1u << kSlotMn)) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            any[p] |= (a0[p] < (i32)e.v0 ? a0[p] : (i32)e.v0) == (i32)x.t0 && (a1[p] < (i32)e.v1 ? a1[p] : (i32)e.v1) == (i32)x.t1;
+    }
+    if ((f | s) & (1u << kSlotMx)) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            any[p] |= (a0[p] > (i32)e.v0 ? a0[p] : (i32)e.v0) == (i32)x.t0 && (a1[p] > (i32)e.v1 ? a1[p] : (i32)e.v1) == (i32)x.t1;
+    }
+}
+
+// The constants of a group as a set.
+template <int P>
+__device__ __forceinline__ void set_conditions(const GroupCtx& s, const i32 (&a0)[P], const i32 (&a1)[P], const JoinCtx& x, bool (&any)[P]) {
+    const u32 cf = s.cf, cs = s.cs;
+    if ((cf | cs) & ((1u << kSlotAdd) | (1u << kSlotSub))) {
+        const u32 dt = x.t0 - x.t1;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const u32 d = (u32)a0[p] - (u32)a1[p];
+            if (d == dt) {                                // (rarely: most operands part here)
+                if ((cf | cs) & (1u << kSlotAdd)) any[p] |= in_range(x.t0 - (u32)a0[p], s);
+                if (cf & (1u << kSlotSub)) any[p] |= in_range((u32)a0[p] - x.t0, s);
+            }
+            if ((cs & (1u << kSlotSub)) && d == 0u - dt) any[p] |= in_range(x.t0 + (u32)a0[p], s);
+        }
+    }
+    if ((cf | cs) & (1u << kSlotMul)) {
+        const u32 cabs = s.cabs;
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            if ((u32)a0[p] * x.t1 == (u32)a1[p] * x.t0 && ((a0[p] | a1[p]) != 0 || x.tz)) any[p] |= factor_exists(a0[p], a1[p], x, cabs);
+    }
+    if ((cf | cs) & (1u << kSlotDiv)) {
+        const float fc = s.fc;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const float f0 = fabsf((float)a0[p]), f1 = fabsf((float)a1[p]);
+            if (cf & (1u << kSlotDiv)) any[p] |= const_div_fwd(f0, f1, x, fc);
+            if (cs & (1u << kSlotDiv)) any[p] |= const_div_swap(f0, f1, x, fc);
+        }
+    }
+    if (cf & (1u << kSlotMod)) {
+#pragma unroll 1
+        for (int p = 0; p < P; ++p) {
+            const u32 u0 = abs_u32(a0[p]), u1 = abs_u32(a1[p]);
+            if (!any[p] && u0 >= x.ut0 && u1 >= x.ut1) any[p] |= gcd_exceeds(u0 - x.ut0, u1 - x.ut1, x.tmod);
+        }
+    }
+    if (cs & (1u << kSlotMod)) {
+        const u32 cabs = s.cabs;
+#pragma unroll 1
+        for (int p = 0; p < P; ++p)
+            if (!any[p]) any[p] |= residue_exists(abs_u32(a0[p]), abs_u32(a1[p]), x.ut0, x.ut1, cabs);
+    }
+    if ((cf | cs) & (1u << kSlotMn)) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= const_minmax(a0[p], a1[p], x, s.mm, false);
+    }
+    if ((cf | cs) & (1u << kSlotMx)) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) any[p] |= const_minmax(a0[p], a1[p], x, s.mm, true);
+    }
+}
+
+// ---- suspects ----
+
+// First constant of [lo, hi) that is not below v.
+__device__ __forceinline__ i32 const_lower(const ConstDev* c, i32 lo, i32 hi, i64 v) {
+    while (lo < hi) {
+        const i32 mid = (lo + hi) >> 1;
+        if (c[mid].value < v) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// The constants that operator slot `slot` leaves open for an operand: up to two runs of the ascending list.
+__device__ __noinline__ void const_runs(const ConstDev* c, i32 lo, i32 hi, int slot, int swap, i64 a0, i64 a1, i64 t0, i64 t1, u64 tmod, i32 (&run)[4]) {
+    run[0] = run[2] = lo; run[1] = run[3] = lo;
+    auto one = [&](i64 v) { run[0] = const_lower(c, lo, hi, v); run[1] = const_lower(c, run[0], hi, v + 1); };
+    auto magnitudes = [&](u64 from, u64 to) {             // from <= |c| <= to, c != 0
+        if (from < 1) from = 1;
+        const u64 most = 1ull << 31;
+        if (to > most) to = most;
+        if (from > to) return;
+        run[0] = const_lower(c, lo, hi, -(i64)to); run[1] = const_lower(c, run[0], hi, -(i64)from + 1);
+        run[2] = const_lower(c, lo, hi, (i64)from); run[3] = const_lower(c, run[2], hi, (i64)to + 1);
+    };
+    const u64 u0 = (u64)(a0 < 0 ? -a0 : a0), u1 = (u64)(a1 < 0 ? -a1 : a1), v0 = (u64)(t0 < 0 ? -t0 : t0), v1 = (u64)(t1 < 0 ? -t1 : t1);
+    switch (slot) {
+        case kSlotAdd: one(t0 - a0); return;
+        case kSlotSub: one(swap ? t0 + a0 : a0 - t0); return;
+        case kSlotMul: {
+            const i64 a = a0 != 0 ? a0 : a1, t = a0 != 0 ? t0 : t1;
+            if (a0 == 0 && t0 != 0) return;
+            if (a == 0) { if (t == 0) { run[0] = lo; run[1] = hi; } return; }
+            if (t % a == 0) one(t / a);
+            return;
+        }
+        case kSlotDiv:
+            if (!swap) {
+                const u64 l0 = u0 / (v0 + 1) + 1, l1 = u1 / (v1 + 1) + 1;
+                const u64 h0 = v0 ? u0 / v0 : ~0ull, h1 = v1 ? u1 / v1 : ~0ull;
+                magnitudes(l0 > l1 ? l0 : l1, h0 < h1 ? h0 : h1);
+            } else if (u0 != 0 && u1 != 0) {
+                const u64 l0 = v0 * u0, l1 = v1 * u1, h0 = l0 + u0 - 1, h1 = l1 + u1 - 1;
+                const u64 l = l0 > l1 ? l0 : l1, h = h0 < h1 ? h0 : h1;
+                if (l == 0) { run[0] = const_lower(c, lo, hi, -(i64)h); run[1] = const_lower(c, run[0], hi, (i64)h + 1); }      // (0 among them)
+                else magnitudes(l, h);
+            }
+            return;
+        case kSlotMod: if (!swap) { magnitudes(tmod + 1, ~0ull); return; } run[0] = lo; run[1] = hi; return;
+        default: run[0] = lo; run[1] = hi; return;
+    }
+}
+
+// The suspects in the warp's first queue, one per lane.  Called by all 32 lanes together.
+__device__ __noinline__ void join_drain(JoinWarp& w, u32 n_q, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
+                                        const JoinCtx& x, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    n.suspects += n_q;
+    const i64 t0 = hole->join_t0, t1 = hole->join_t1;
+    const u64 tmod = hole->join_tmod;
+    const int from = hole->join_p1 ? 2 : 1;               // probes that the second queue's check starts at
+    for (u32 at = 0; at < n_q; at += 32) {
+        const bool live = at + lane < n_q;
+        const u32 off = live ? w.q_off[at + lane] : 0u;
+        const i32 b0[1] = {live ? w.q_a0[at + lane] : 0}, b1[1] = {live ? w.q_a1[at + lane] : 0};
+        for (int gi = 0; gi < seg.n_groups; ++gi) {
+            const GroupCtx& s = w.grp[gi];
+            const JoinSet* S = s.set;
+            const u32 ef = s.ef, es = s.es;
+            if (ef | es)
+                for (int i = 0; i < s.n_entries; ++i) {
+                    const JoinEntry en = S->e[i];
+                    bool any[1] = {false};
+                    entry_conditions<1>(en, ef, es, b0, b1, x, any);
+                    if (!__any_sync(0xffffffffu, live && any[0])) continue;
+                    for (int swap = 0; swap < 2; ++swap)
+                        for (u32 m = swap ? es : ef; m; m &= m - 1) {
+                            const u32 bit = m & (0u - m);
+                            const int slot = __ffs((int)bit) - 1;
+                            bool one[1] = {false};
+                            entry_conditions<1>(en, swap ? 0u : bit, swap ? bit : 0u, b0, b1, x, one);
+                            bool on = live && one[0];
+                            if (on) {                     // exactly, at both probes
+                                i64 v = 0;
+                                on = apply_op(op_of_slot(slot), swap ? (i64)(i32)en.v0 : b0[0], swap ? b0[0] : (i64)(i32)en.v0, v) && v == t0 &&
+                                     apply_op(op_of_slot(slot), swap ? (i64)(i32)en.v1 : b1[0], swap ? b1[0] : (i64)(i32)en.v1, v) && v == t1;
+                            }
+                            join_push(w, plan, seg, sk, hole, on, off, en.pos, gi, slot, swap, from, n);
+                        }
+                }
+            if (!(s.cf | s.cs)) continue;
+            const i32 clo = S->const_begin, chi = clo + S->n_const;
+            for (int swap = 0; swap < 2; ++swap)
+                for (u32 m = swap ? s.cs : s.cf; m; m &= m - 1) {
+                    const int slot = __ffs((int)m) - 1;
+                    const bool act = live && const_condition(slot, swap, b0[0], b1[0], x, s);
+                    if (!__any_sync(0xffffffffu, act)) continue;
+                    i32 run[4] = {clo, clo, clo, clo};
+                    if (act) const_runs(g->consts, clo, chi, slot, swap, b0[0], b1[0], t0, t1, tmod, run);
+                    const i32 len0 = run[1] - run[0], len = len0 + run[3] - run[2];
+                    for (i32 i = 0; __any_sync(0xffffffffu, act && i < len); ++i) {
+                        bool on = act && i < len;
+                        const ConstDev c = g->consts[on ? (i < len0 ? run[0] + i : run[2] + i - len0) : clo];
+                        if (on) {
+                            i64 v = 0;
+                            on = apply_op(op_of_slot(slot), swap ? c.value : b0[0], swap ? b0[0] : c.value, v) && v == t0 &&
+                                 apply_op(op_of_slot(slot), swap ? c.value : b1[0], swap ? b1[0] : c.value, v) && v == t1;
+                        }
+                        join_push(w, plan, seg, sk, hole, on, off, (u32)c.pos, gi, slot, swap, from, n);
+                    }
+                }
+        }
+    }
+    __syncwarp();
+}
+
+// The exact form: one operand at a time (the same for all lanes), lanes over the leaves, every operator; the first probe
+// here, the others when a warp's worth of candidates has gathered.
+__device__ __noinline__ void join_exact(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, u64 e, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
+    i64 a0, a1 = 0;
+    if (!ref_value(g, hole, ref, seg.nt, seg.esize, 0, a0)) return;
+    const bool two = hole->n_exact >= 2;
+    if (two && !ref_value(g, hole, ref, seg.nt, seg.esize, 1, a1)) return;
+    if (w.nc) join_check(w, plan, seg, sk, hole, hole->join_p1 && hole->join_on ? 2 : 1, n);      // (what waits was held against the pair)
+    for (int gi = 0; gi < seg.n_groups; ++gi) {
+        const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+        const int nl = (int)g->cnt[grp.leaf_nt][1];
+        n.tests += (u64)nl * (u64)(__popc(grp.fmask) + __popc(grp.smask));
+        for (int l0 = 0; l0 < nl; l0 += 32) {
+            const int pos = l0 + lane;
+            const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (pos < nl ? pos : 0)];
+            const i64 c0 = lf.var >= 0 ? hole->probe_pt[0][lf.var] : lf.value, c1 = two && lf.var >= 0 ? hole->probe_pt[1][lf.var] : lf.value;
+            for (int swap = 0; swap < 2; ++swap)
+                for (u32 m = swap ? grp.smask : grp.fmask; m; m &= m - 1) {
+                    const int slot = __ffs((int)m) - 1, op = op_of_slot(slot);
+                    i64 v;
+                    bool hit = pos < nl && apply_op(op, swap ? c0 : a0, swap ? a0 : c0, v) && probe_accepts(hole, 0, v);
+                    if (two && hit) hit = apply_op(op, swap ? c1 : a1, swap ? a1 : c1, v) && probe_accepts(hole, 1, v);
+                    n.suspects += (u32)__popc(__ballot_sync(0xffffffffu, hit));
+                    join_push(w, plan, seg, sk, hole, hit, (u32)(e - seg.e_begin), (u32)pos, gi, slot, swap, two ? 2 : 1, n);
+                }
+        }
+    }
+    if (w.nc) join_check(w, plan, seg, sk, hole, two ? 2 : 1, n);
+}
+
+// ---- operands in rank order ----
+
+// A run of operands of (nt, size) in rank order that one production and pair of sizes builds: entries of the pair
+// table, or (one size above the tables) products of two ranges of them.  The same for all lanes of a warp, so that a
+// lane finds its operand with one division by an invariant.  Mode 2: neither (unranked in full, one by one).
+struct JoinRun {
+    i32 mode, op;
+    const int2* L;
+    const int2* R;
+    u32 l0, r0, cr, inv;                                  // first operands; right operands per left one and 2^32 / that
+    u64 left;                                             // operands to the end of the run
+};
+
+__device__ __noinline__ JoinRun join_run(const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank) {
+    JoinRun c;
+    const int2* pair = reinterpret_cast<const int2*>(hole->tab_pair);
+    const int tmax = hole->tab_max_size;
+    const u64 total = g->cnt[nt][size];
+    c.mode = 2; c.op = 0; c.l0 = c.r0 = 0; c.cr = 1; c.inv = 0xffffffffu; c.L = c.R = pair; c.left = total - rank;
+    if (size <= tmax) { c.mode = 0; c.R = pair + hole->tab_off[nt][size] + rank; return c; }
+    if (tmax < 1 || size < 3) return c;
+    int p = g->bin_begin[nt];
+    const int pe = g->bin_begin[nt + 1];
+    while (p + 1 < pe && g->bins[p + 1].off[size] <= rank) ++p;
+    u64 rem = rank - g->bins[p].off[size];
+    const int lnt = g->bins[p].lnt, rnt = g->bins[p].rnt;
+    u64 cl = 0, cr = 0;
+    int a = 1;
+    for (;; ++a) {
+        cl = g->cnt[lnt][a]; cr = g->cnt[rnt][size - 1 - a];
+        if (rem < cl * cr || a == size - 2) break;
+        rem -= cl * cr;
+    }
+    c.left = cl * cr - rem;
+    if (a > tmax || size - 1 - a > tmax) return c;        // (an operand above the tables: the whole run goes one by one)
+    u64 l, r;
+    divmod_u64(rem, cr, l, r);
+    c.mode = 1; c.op = g->bins[p].op;
+    c.L = pair + hole->tab_off[lnt][a]; c.R = pair + hole->tab_off[rnt][size - 1 - a];
+    c.l0 = (u32)l; c.r0 = (u32)r; c.cr = (u32)cr;
+    c.inv = cr > 1 ? (u32)((1ull << 32) / cr) : 0xffffffffu;
+    return c;
+}
+
+__device__ __forceinline__ bool narrow31(i64 v) { return v > -(1ll << 31) && v < (1ll << 31); }
+
+// An operand's values at the two probes: 0 undefined at one of them, 1 both below 2^31 in magnitude, 2 not.
+__device__ __noinline__ int join_value_slow(const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank, i32& a0, i32& a1) {
+    i64 x, y;
+    if (!operand_value(g, hole, 0, nt, size, rank, x)) return 0;
+    y = x;
+    if (hole->join_p1 && !operand_value(g, hole, hole->join_p1, nt, size, rank, y)) return 0;
+    a0 = (i32)x; a1 = (i32)y;
+    return narrow31(x) && narrow31(y) ? 1 : 2;
+}
+
+// Operator OP on the pairs of P operands.
+template <int OP, int P>
+__device__ __forceinline__ void pair_op(const int2 (&x)[P], const int2 (&y)[P], i32 (&a0)[P], i32 (&a1)[P], u32& alive, u32& wide) {
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        if (OP == XP_OP_DIV || OP == XP_OP_MOD) {         // (magnitudes below 2^31: no overflow)
+            const i32 d0 = y[p].x == 0 ? 1 : y[p].x, d1 = y[p].y == 0 ? 1 : y[p].y;
+            if (y[p].x == 0 || y[p].y == 0) alive &= ~(1u << p);
+            const i32 q0 = x[p].x / d0, q1 = x[p].y / d1;
+            a0[p] = OP == XP_OP_DIV ? q0 : x[p].x - q0 * d0;
+            a1[p] = OP == XP_OP_DIV ? q1 : x[p].y - q1 * d1;
+        } else if (OP == XP_OP_MIN) { a0[p] = min(x[p].x, y[p].x); a1[p] = min(x[p].y, y[p].y); }
+        else if (OP == XP_OP_MAX) { a0[p] = max(x[p].x, y[p].x); a1[p] = max(x[p].y, y[p].y); }
+        else {
+            i64 r0, r1;
+            if (OP == XP_OP_ADD) { r0 = (i64)x[p].x + y[p].x; r1 = (i64)x[p].y + y[p].y; }
+            else if (OP == XP_OP_SUB) { r0 = (i64)x[p].x - y[p].x; r1 = (i64)x[p].y - y[p].y; }
+            else { r0 = (i64)x[p].x * y[p].x; r1 = (i64)x[p].y * y[p].y; }
+            a0[p] = (i32)r0; a1[p] = (i32)r1;
+            if (!narrow31(r0) || !narrow31(r1)) wide |= 1u << p;
+        }
+    }
+}
+
+// Operands at + 32 p + lane of a run (those below n), their values at the two probes.
+template <int P>
+__device__ __forceinline__ void run_values(const JoinRun& c, const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank, u32 at, u32 n,
+                                           i32 (&a0)[P], i32 (&a1)[P], u32& alive, u32& wide) {
+    const u32 lane = threadIdx.x & 31u;
+    alive = wide = 0;
+#pragma unroll
+    for (int p = 0; p < P; ++p) { a0[p] = 0; a1[p] = 0; if (at + 32u * p + lane < n) alive |= 1u << p; }
+    if (c.mode == 0) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const int2 y = (alive >> p) & 1u ? c.R[at + 32u * p + lane] : make_int2(kPairNone, 0);
+            a0[p] = y.x; a1[p] = y.y;
+            if (y.x == kPairNone) { if ((alive >> p) & 1u) wide |= (u32)(y.y != 0) << p; alive &= ~(1u << p); }
+        }
+        return;
+    }
+    if (c.mode == 2) {
+#pragma unroll 1
+        for (int p = 0; p < P; ++p) {
+            if (!((alive >> p) & 1u)) continue;
+            i32 v0 = 0, v1 = 0;
+            const int st = join_value_slow(g, hole, nt, size, rank + at + 32u * p + lane, v0, v1);
+#pragma unroll
+            for (int k = 0; k < P; ++k) if (k == p) { a0[k] = v0; a1[k] = v1; }
+            if (st != 1) { alive &= ~(1u << p); wide |= (u32)(st == 2) << p; }
+        }
+        return;
+    }
+    int2 x[P], y[P];
+    u32 none = 0;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const u32 rel = (alive >> p) & 1u ? c.r0 + at + 32u * p + lane : c.r0;
+        u32 q = __umulhi(rel, c.inv), r = rel - q * c.cr; // the estimate is the quotient or one less
+        if (r >= c.cr) { ++q; r -= c.cr; }
+        x[p] = c.L[c.l0 + q]; y[p] = c.R[r];
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const bool nx = x[p].x == kPairNone, ny = y[p].x == kPairNone;
+        if (nx | ny) {
+            none |= 1u << p;
+            if (!((nx && x[p].y == 0) || (ny && y[p].y == 0)) && ((alive >> p) & 1u)) wide |= 1u << p;      // (defined, but not narrow)
+            x[p] = y[p] = make_int2(1, 1);
+        }
+    }
+    alive &= ~none;
+    u32 w2 = 0;
+    switch (c.op) {
+        case XP_OP_ADD: pair_op<XP_OP_ADD, P>(x, y, a0, a1, alive, w2); break;
+        case XP_OP_SUB: pair_op<XP_OP_SUB, P>(x, y, a0, a1, alive, w2); break;
+        case XP_OP_MUL: pair_op<XP_OP_MUL, P>(x, y, a0, a1, alive, w2); break;
+        case XP_OP_DIV: pair_op<XP_OP_DIV, P>(x, y, a0, a1, alive, w2); break;
+        case XP_OP_MOD: pair_op<XP_OP_MOD, P>(x, y, a0, a1, alive, w2); break;
+        case XP_OP_MIN: pair_op<XP_OP_MIN, P>(x, y, a0, a1, alive, w2); break;
+        case XP_OP_MAX: pair_op<XP_OP_MAX, P>(x, y, a0, a1, alive, w2); break;
+        default: w2 = (1u << P) - 1u; break;              // (shifts: exactly)
+    }
+    w2 &= alive;
+    alive &= ~w2;
+    wide |= w2;
+}
+
+// ---- the kernel ----
+
+__device__ __forceinline__ void join_flush(const PlanDev& plan, int acc, JoinCount& n) {
+    u64 e = n.evals;
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_down_sync(0xffffffffu, e, o);
+    if ((threadIdx.x & 31) == 0 && acc >= 0) {
+        AccDev* a = &plan.acc[acc];
+        if (e) atomicAdd(&a->evals, e);
+        if (n.tests) { atomicAdd(&a->filter_tests, n.tests); atomicAdd(&a->join_tests, n.tests); }
+        if (n.cands) atomicAdd(&a->tile_cands, n.cands);
+        if (n.suspects) atomicAdd(&a->filter_survivors, (u64)n.suspects);
+        if (n.passes) atomicAdd(&a->probe_survivors, (u64)n.passes);
+    }
+    n = JoinCount{0, 0, 0, 0, 0};
+}
+
+// Fills the warp's group contexts for a segment; returns the operand limit, 0 when some leaf set has to go the exact way.
+__device__ __noinline__ u32 join_groups(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const HoleDev* hole, const JoinCtx& x) {
+    const int lane = threadIdx.x & 31;
+    u32 lim = 0x7fffffffu;
+    __syncwarp();
+    if (lane < seg.n_groups) {
+        const JoinGroup& grp = plan.jgroups[seg.first_group + lane];
+        const JoinSet* S = &hole->join_sets[grp.leaf_nt];
+        GroupCtx c;
+        c.set = S;
+        c.cmin = S->cmin; c.cmax = S->cmax; c.cabs = S->cabs; c.mm = S->mm; c.fc = (float)S->cabs; c.n_entries = S->n_entries;
+        c.tests = (S->n_entries + (S->n_const > 0 ? 1 : 0)) * (__popc(grp.fmask) + __popc(grp.smask));
+        u32 cf = grp.fmask, cs = grp.smask, ef = cf, es = cs;
+        // operators that cannot reach the target: quotients, remainders, minima and maxima of narrow operands are narrow;
+        // a remainder is below its divisor; c / a and c % a are at most |c|
+        constexpr u32 kNarrow = (1u << kSlotDiv) | (1u << kSlotMod) | (1u << kSlotMn) | (1u << kSlotMx);
+        if (!x.small) { cf &= ~kNarrow; cs &= ~kNarrow; ef &= ~kNarrow; es &= ~kNarrow; }
+        if (x.tmod >= S->cabs) cf &= ~(1u << kSlotMod);
+        if (x.tmod > S->cabs) cs &= ~((1u << kSlotDiv) | (1u << kSlotMod));
+        if (S->n_const == 0) cf = cs = 0;
+        if (S->n_entries == 0) ef = es = 0;
+        if (hole->join_none) cf = cs = ef = es = 0;
+        c.cf = cf; c.cs = cs; c.ef = ef; c.es = es;
+        w.grp[lane] = c;
+        lim = S->ok ? S->lim : 0u;
+    }
+    __syncwarp();
+    return __reduce_min_sync(0xffffffffu, lim);
+}
+
+// Operands [first, first + count) of a segment against the leaves (count <= the segment's chunk).
+template <int P>
+__device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
+                                         u64 first, u64 count, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    JoinCtx x;
+    {
+        const i64 t0 = hole->join_t0, t1 = hole->join_t1;
+        const u64 v0 = (u64)(t0 < 0 ? -t0 : t0), v1 = (u64)(t1 < 0 ? -t1 : t1), tm = hole->join_tmod;
+        x.t0 = (u32)(u64)t0; x.t1 = (u32)(u64)t1;
+        x.small = (v0 | v1) >> 31 == 0;
+        x.ut0 = x.small ? (u32)v0 : 0u; x.ut1 = x.small ? (u32)v1 : 0u;
+        x.rt0 = hole->join_rt0; x.rt1 = hole->join_rt1; x.rl0 = hole->join_rl0; x.rl1 = hole->join_rl1; x.h0 = hole->join_h0; x.h1 = hole->join_h1;
+        x.ft0 = (float)x.ut0; x.ft1 = (float)x.ut1;
+        x.tmod = tm < 0xffffffffull ? (u32)tm : 0xffffffffu;
+        x.tz = (t0 | t1) == 0;
+    }
+    const u32 lim = join_groups(w, plan, seg, hole, x);
+    u32 tests_each = 0;
+    {
+        u64 pairs = 0;
+        for (int gi = 0; gi < seg.n_groups; ++gi) {
+            const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+            pairs += g->cnt[grp.leaf_nt][1] * (u64)(__popc(grp.fmask) + __popc(grp.smask));
+            tests_each += (u32)w.grp[gi].tests;
+        }
+        n.cands += count * pairs;
+    }
+    if (seg.exact || !hole->join_on || lim == 0u) {
+        for (u64 i = 0; i < count; ++i) join_exact(w, plan, seg, sk, hole, first + i, n);
+        return;
+    }
+    u32 nq = 0;
+    u32 n_alive = 0;
+    for (u64 done = 0; done < count;) {
+        const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done);
+        const u32 n_run = (u32)(c.left < count - done ? c.left : count - done);
+        const u32 off0 = (u32)(first + done - seg.e_begin) + lane;
+        for (u32 at = 0; at < n_run; at += 32u * P) {
+            i32 a0[P], a1[P];
+            u32 alive, wide;
+            run_values<P>(c, g, hole, seg.nt, seg.esize, first + done, at, n_run, a0, a1, alive, wide);
+            bool any[P];
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                any[p] = false;
+                if (((alive >> p) & 1u) && (abs_u32(a0[p]) >= lim || abs_u32(a1[p]) >= lim)) { alive &= ~(1u << p); wide |= 1u << p; }
+            }
+            n_alive += (u32)__popc(alive);
+            for (int gi = 0; gi < seg.n_groups; ++gi) {
+                const GroupCtx& s = w.grp[gi];
+                if (s.cf | s.cs) set_conditions<P>(s, a0, a1, x, any);
+                const u32 ef = s.ef, es = s.es;
+                if (ef | es) {
+                    const JoinEntry* e = s.set->e;
+                    for (int i = 0; i < s.n_entries; ++i) {
+                        const JoinEntry en = e[i];
+                        entry_conditions<P>(en, ef, es, a0, a1, x, any);
+                    }
+                }
+            }
+            u32 hits = 0;
+#pragma unroll
+            for (int p = 0; p < P; ++p) hits |= (u32)any[p] << p;
+            hits &= alive;
+            if (__any_sync(0xffffffffu, hits != 0u)) {
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    const bool h = (hits >> p) & 1u;
+                    const u32 b = __ballot_sync(0xffffffffu, h);
+                    if (h) {
+                        const u32 q = nq + (u32)__popc(b & ((1u << lane) - 1u));
+                        w.q_off[q] = off0 + at + 32u * p; w.q_a0[q] = a0[p]; w.q_a1[q] = a1[p];
+                    }
+                    nq += (u32)__popc(b);
+                }
+                if (nq >= 32u) {                          // whole warps of suspects; the rest waits
+                    const u32 full = nq & ~31u;
+                    join_drain(w, full, plan, seg, sk, hole, x, n);
+                    nq -= full;
+                    u32 o = 0;
+                    i32 v0 = 0, v1 = 0;
+                    if (lane < (int)nq) { o = w.q_off[full + lane]; v0 = w.q_a0[full + lane]; v1 = w.q_a1[full + lane]; }
+                    __syncwarp();
+                    if (lane < (int)nq) { w.q_off[lane] = o; w.q_a0[lane] = v0; w.q_a1[lane] = v1; }
+                    __syncwarp();
+                }
+            }
+            if (__any_sync(0xffffffffu, wide != 0u)) {
+#pragma unroll 1
+                for (int p = 0; p < P; ++p)
+                    for (u32 m = __ballot_sync(0xffffffffu, (wide >> p) & 1u); m; m &= m - 1)
+                        join_exact(w, plan, seg, sk, hole, first + done + at + (u64)(32 * p + __ffs((int)m) - 1), n);
+            }
+        }
+        done += n_run;
+    }
+    n.tests += (u64)tests_each * (u64)__reduce_add_sync(0xffffffffu, n_alive);
+    if (nq) join_drain(w, nq, plan, seg, sk, hole, x, n);
+    if (w.nc) join_check(w, plan, seg, sk, hole, hole->join_p1 ? 2 : 1, n);
+}
+
+// ---- contexts that compare ----
+
+// Operand values at the first kRangeProbes probes sit in registers; leaves are held against those with an early exit.
+constexpr int kRangeProbes = 4;
+
+// v = x op y at one probe for narrow x, y; false when undefined.
+__device__ __forceinline__ bool narrow_op(int slot, i32 x, i32 y, i64& v) {
+    switch (slot) {
+        case kSlotAdd: v = (i64)x + y; return true;
+        case kSlotSub: v = (i64)x - y; return true;
+        case kSlotMul: v = (i64)x * y; return true;
+        case kSlotDiv: if (y == 0) return false; v = y == -1 ? -(i64)x : (i64)(x / y); return true;
+        case kSlotMod: if (y == 0) return false; v = y == -1 ? 0 : (i64)(x % y); return true;
+        case kSlotMn: v = x < y ? x : y; return true;
+        default: v = x > y ? x : y; return true;
+    }
+}
+
+// Operands [first, first + count) of a segment against the leaves, for a hole whose context compares: the value has to
+// lie in [rng_lo, rng_hi] at every probe.
+__device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
+                                          u64 first, u64 count, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    const int np = hole->n_exact, nr = np < kRangeProbes ? np : kRangeProbes;
+    constexpr i64 kMost = 1ll << 62;
+    i64 lo[kRangeProbes], hi[kRangeProbes];
+#pragma unroll
+    for (int j = 0; j < kRangeProbes; ++j) {              // (probes beyond the last repeat the first)
+        const int k = j < nr ? j : 0;
+        lo[j] = hole->rng_lo[k] < -kMost ? -kMost : hole->rng_lo[k];
+        hi[j] = hole->rng_hi[k] > kMost ? kMost : hole->rng_hi[k];
+    }
+    bool sets_ok = (hole->aff_okmask & ((1u << np) - 1u)) == 0u;      // (every probe compares: it does not depend on the point)
+    u64 pairs = 0;
+    for (int gi = 0; gi < seg.n_groups; ++gi) {
+        const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+        pairs += g->cnt[grp.leaf_nt][1] * (u64)(__popc(grp.fmask) + __popc(grp.smask));
+        sets_ok = sets_ok && hole->join_sets[grp.leaf_nt].ok != 0;
+    }
+    n.cands += count * pairs;
+    for (u64 at = 0; at < count; at += 32) {
+        const u64 e = first + at + lane;
+        const bool have = at + lane < count;
+        OperandRef ref;
+        ref.mode = 2; ref.op = 0; ref.a = ref.b = 0;
+        i32 a[kRangeProbes] = {0};
+        // interval of constants c with a + c in range at every probe, and (swapped difference) with c - a in range
+        i64 pl = -kMost, ph = kMost, ml = -kMost, mh = kMost;
+        bool live = false, wide = false;
+        if (have) {
+            ref = operand_ref(g, hole, seg.nt, seg.esize, e);
+            live = true;
+            for (int j = 0; j < np && live && !wide; ++j) {
+                i64 v;
+                live = ref_value(g, hole, ref, seg.nt, seg.esize, j, v);
+                if (!live) break;
+                wide = !narrow31(v);
+                const i64 l = hole->rng_lo[j] < -kMost ? -kMost : hole->rng_lo[j], h = hole->rng_hi[j] > kMost ? kMost : hole->rng_hi[j];
+                pl = pl > l - v ? pl : l - v; ph = ph < h - v ? ph : h - v;
+                ml = ml > l + v ? ml : l + v; mh = mh < h + v ? mh : h + v;
+#pragma unroll
+                for (int k = 0; k < kRangeProbes; ++k) if (k == j || (k >= nr && j == 0)) a[k] = (i32)v;
+            }
+        }
+        if (!sets_ok) wide = live;
+        for (u32 m = __ballot_sync(0xffffffffu, live && wide); m; m &= m - 1)
+            join_exact(w, plan, seg, sk, hole, first + at + (u64)(__ffs((int)m) - 1), n);
+        live = live && !wide;
+        const u32 off = (u32)(e - seg.e_begin);
+        const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
+        if (n_live == 0u) continue;
+        for (int gi = 0; gi < seg.n_groups; ++gi) {
+            const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+            const i32 cb = g->const_begin[grp.leaf_nt], vb = g->var_begin[grp.leaf_nt], ve = g->const_begin[grp.leaf_nt + 1];
+            constexpr u32 kLinear = (1u << kSlotAdd) | (1u << kSlotSub);
+            for (int swap = 0; swap < 2; ++swap) {
+                const u32 mask = swap ? grp.smask : grp.fmask;
+                // constants: sums and differences by the intersection of the probes' intervals
+                for (u32 m = mask & kLinear; m; m &= m - 1) {
+                    const int slot = __ffs((int)m) - 1;
+                    const i64 from = slot == kSlotAdd ? pl : swap ? ml : -ph, to = slot == kSlotAdd ? ph : swap ? mh : -pl;
+                    i32 i0 = cb, i1 = cb;
+                    if (live && from <= to) { i0 = const_lower(g->consts, cb, vb, from); i1 = const_lower(g->consts, i0, vb, to + 1); }
+                    n.tests += n_live;
+                    for (i32 i = 0; __any_sync(0xffffffffu, i0 + i < i1); ++i) {
+                        const bool on = i0 + i < i1;
+                        n.suspects += (u32)__popc(__ballot_sync(0xffffffffu, on));
+                        join_push(w, plan, seg, sk, hole, on, off, on ? (u32)g->consts[i0 + i].pos : 0u, gi, slot, swap, 0, n);
+                    }
+                }
+                // the rest leaf by leaf
+                const u32 others = mask & ~kLinear;
+                for (i32 ci = others ? cb : vb; ci < ve; ++ci) {
+                    const ConstDev c = g->consts[ci];
+                    i32 cv[kRangeProbes];
+#pragma unroll
+                    for (int j = 0; j < kRangeProbes; ++j) cv[j] = (i32)(ci < vb ? c.value : hole->probe_pt[j < nr ? j : 0][c.value]);
+                    for (u32 m = ci < vb ? others : mask; m; m &= m - 1) {
+                        const int slot = __ffs((int)m) - 1;
+                        n.tests += n_live;
+                        bool on = live;
+#pragma unroll
+                        for (int j = 0; j < kRangeProbes; ++j) {
+                            i64 v = 0;
+                            on = on && narrow_op(slot, swap ? cv[j] : a[j], swap ? a[j] : cv[j], v) && v >= lo[j] && v <= hi[j];
+                            if (!__any_sync(0xffffffffu, on)) break;
+                        }
+                        const u32 b = __ballot_sync(0xffffffffu, on);
+                        if (!b) continue;
+                        n.suspects += (u32)__popc(b);
+                        join_push(w, plan, seg, sk, hole, on, off, (u32)c.pos, gi, slot, swap, nr, n);
+                    }
+                }
+                // (what was pushed with different first probes is not mixed in one check)
+                if (w.nc) join_check(w, plan, seg, sk, hole, 0, n);
+            }
+        }
+    }
+}
+
+// Candidates [first, first + count) of (start nonterminal, size) themselves, checked on the probes one by one.
+__device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
+                                           u64 first, u64 count, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    const int n_exact = hole->n_exact;
+    for (u64 at = first; at < first + count; at += 32) {
+        const u64 rank = at + lane;
+        bool pass = false;
+        u32 vars = 0;
+        if (rank < first + count) {
+            const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, rank);
+            pass = true;
+            for (int j = 0; j < n_exact && pass; ++j) {
+                ++n.evals;
+                i64 v;
+                pass = ref_value(g, hole, ref, seg.nt, seg.esize, j, v) && probe_accepts(hole, j, v);
+            }
+            if (pass && n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
+            vars = ref_vars(hole, ref);
+        }
+        const u32 b = __ballot_sync(0xffffffffu, pass);
+        n.suspects += (u32)__popc(b);
+        join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
+    }
+}
+
+template <int P>
+__global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const PlanDev plan) {
+    __shared__ JoinWarp sh[kJoinWarps];
+    JoinWarp& w = sh[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) w.nc = 0;
+    __syncwarp();
+    JoinCount n{0, 0, 0, 0, 0};
+    int acc = -1;
+    const u64 warps = (u64)gridDim.x * kJoinWarps;
+    // the first ticket is the warp's number (warp-in-CTA major, so that a small search spreads over the SMs), the others
+    // come from the counter
+    u64 t = plan.join_base + (u64)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    while (t < plan.n_join) {
+        int lo = 0, k = plan.n_jsegs;
+        while (k > 1) {                                   // last segment with first_ticket <= t: one probe per lane and round
+            const int step = (k + 31) / 32;
+            const int pos = lo + lane * step;
+            const bool le = pos < lo + k && plan.jsegs[pos].first_ticket <= t;
+            const u32 mask = __ballot_sync(0xffffffffu, le);
+            const int j = 31 - __clz((int)(mask | 1u));
+            const int nlo = lo + j * step;
+            k = (lo + k - nlo) < step ? (lo + k - nlo) : step;
+            lo = nlo;
+        }
+        const JoinSeg& seg = plan.jsegs[lo];
+        if (seg.acc != acc) { join_flush(plan, acc, n); acc = seg.acc; }
+        const SketchDev* sk = plan.sketches[seg.sketch];
+        const HoleDev* hole = &sk->holes[seg.hole];
+        const u32 all = hole->n_probe >= 32 ? 0xffffffffu : (1u << hole->n_probe) - 1u;
+        const u64 chunk = seg.chunk, from = (t - seg.first_ticket) * chunk;
+        if ((hole->probe_spec_ok & all) == all && from < seg.e_count) {      // (a spec undefined at a probe: nothing can match)
+            const u64 count = seg.e_count - from < chunk ? seg.e_count - from : chunk;
+            if (seg.kind == kJoinDirect) direct_ticket(w, plan, seg, sk, hole, seg.e_begin + from, count, n);
+            else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, seg.e_begin + from, count, n);
+            else join_ticket<P>(w, plan, seg, sk, hole, seg.e_begin + from, count, n);
+        }
+        u64 next = 0;
+        if (lane == 0) next = atomicAdd(plan.join_ticket, 1ull);
+        t = plan.join_base + warps + __shfl_sync(0xffffffffu, next, 0);
+    }
+    join_flush(plan, acc, n);
+}
+
+}  // namespace xp

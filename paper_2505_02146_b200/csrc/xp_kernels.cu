@@ -1,11 +1,12 @@
 // Device kernels of libxpiler_repair (sm_100a).
 //
-//   prepare_kernel  -- per sketch, once at load: coordinates and spec values of the sample
-//                      points, choice and order of each hole's probe points.
+//   prep_sample_kernel, prepare_kernel -- per sketch, once at load: coordinates and spec values of the
+//                      sample points, choice and order of each hole's probe points.
 //   subvalue_kernel, stage_points_kernel, stage_spec_kernel, coord_bounds_kernel -- per sketch,
 //                      once at load: values (and variable sets) of all small subtrees at the probes;
 //                      points and spec values of a box; coordinate bounds of a table.
-//   eval_kernel     -- the search.  Persistent CTAs take tickets (pieces of the rank space)
+//   join_kernel     -- (xp_join.cuh) the part of the search whose candidates have a leaf at the root.
+//   eval_kernel     -- the rest of the search.  Persistent CTAs take tickets (pieces of the rank space)
 //                      from an atomic counter; no CTA ever waits for another.
 //                        stage 1 (tile segments): probe-point filter over a product of operand tiles,
 //                                 with a second, exact look at probe 1 for what the filter lets through;
@@ -14,13 +15,14 @@
 //   verify_kernel   -- stage 3: check on the whole domain (lane = 2 or 4 points, warp-wide early
 //                      exit), cut into (survivor, chunk of points) items that any warp takes; on a
 //                      box only the sub-box of the variables that occur is visited.
-//   count_kernel    -- survivors that passed every chunk become matches: per-size counts (sum)
-//                      and least rank (min) by atomics.
-//   finish_kernel   -- reduction of the per-size results to the least solution per hole.
+//                      The warp that passes a survivor's last chunk makes it a match: per-size counts
+//                      (sum) and least rank (min) by atomics.
 //   int32_peak_*    -- integer-ALU peak microbenchmarks.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <climits>
+#include <mutex>
 
 #include "xp_device.cuh"
 #include "xp_launch.h"
@@ -119,14 +121,108 @@ __device__ bool ctx_interval(const HoleDev* hole, const i64* pt, i64 spec, i64& 
     return false;
 }
 
-constexpr int kPrepBigSamples = 8192;                    // random candidates of the largest size, held against the first probe
+// The join's targets of a hole (one thread): the hole values that satisfy the constraint at the two probes, exact in
+// 64 bits for values below the operand limits of the leaf sets (the context's factor times such a value cannot wrap).
+__device__ void join_targets(HoleDev* hole) {
+    const u32 ok = hole->probe_spec_ok & hole->aff_okmask;
+    const int np = hole->tab_probes;
+    hole->join_p1 = np >= 2 && ((ok >> 1) & 1u) ? 1 : 0;
+    bool on = np >= 1 && (ok & 1u), none = false;
+    u64 tmod = 0;
+    i64 t[2] = {0, 0};
+    for (int j = 0; j < np && on; ++j) {
+        if (!((ok >> j) & 1u)) continue;
+        const i64 A = (i64)hole->aff_Aj[j], d = (i64)((u64)hole->probe_spec[j] - hole->aff_Bj[j]);
+        if (A == 0 || A <= -(1ll << 31) || A >= (1ll << 31)) { on = false; break; }
+        i64 v = d;
+        bool miss = false;
+        if (A != 1) { miss = d <= -(1ll << 62) || d >= (1ll << 62) || d % A != 0; v = miss ? 0 : d / A; }
+        if (miss) { none = none || j == 0 || j == hole->join_p1; tmod = ~0ull; }
+        else {
+            const u64 m = v < 0 ? 0ull - (u64)v : (u64)v;
+            tmod = m > tmod ? m : tmod;
+        }
+        if (j == 0) t[0] = t[1] = v;
+        if (j == hole->join_p1) t[1] = v;
+    }
+    hole->join_on = on ? 1 : 0;
+    hole->join_none = none ? 1 : 0;
+    hole->join_t0 = t[0]; hole->join_t1 = t[1];
+    hole->join_tmod = tmod;
+    const float m0 = fabsf((float)t[0]), m1 = fabsf((float)t[1]);
+    hole->join_rt0 = t[0] ? 1.f / m0 : 0.f; hole->join_rt1 = t[1] ? 1.f / m1 : 0.f;
+    hole->join_rl0 = 1.f / (m0 + 1.f); hole->join_rl1 = 1.f / (m1 + 1.f);
+    hole->join_h0 = t[0] ? 0.f : 3e38f; hole->join_h1 = t[1] ? 0.f : 3e38f;
+}
+
+// The leaf set of nonterminal nt (one thread): see JoinSet.
+__device__ void join_leaf_set(const GrammarDev* g, HoleDev* hole, int nt) {
+    JoinSet& S = hole->join_sets[nt];
+    const ConstDev* c = g->consts;
+    const int cb = g->const_begin[nt], vb = g->var_begin[nt], ve = g->const_begin[nt + 1];
+    const int p1 = hole->join_p1;
+    const i64 t0 = hole->join_t0, t1 = hole->join_t1;
+    const u64 m0 = t0 < 0 ? 0ull - (u64)t0 : (u64)t0, m1 = t1 < 0 ? 0ull - (u64)t1 : (u64)t1;
+    const bool small = (m0 | m1) >> 31 == 0;              // (otherwise no narrow quotient or remainder is the target)
+    bool ok = true;
+    u64 most = 1;
+    int n = 0;
+    auto magnitude = [](i64 v) { return v < 0 ? 0ull - (u64)v : (u64)v; };
+    auto add = [&](i64 x, i64 y, int pos) {
+        const u64 u0 = magnitude(x), u1 = magnitude(y);
+        most = u0 > most ? u0 : most;
+        most = u1 > most ? u1 : most;
+        if (n >= kJoinEntries || (u0 | u1) >> 31) { ok = false; return; }
+        JoinEntry e;
+        e.v0 = (u32)(u64)x; e.v1 = (u32)(u64)y; e.u0 = (u32)u0; e.u1 = (u32)u1;
+        const u64 l0 = m0 * u0, l1 = m1 * u1;             // (used when the targets are small: below 2^62)
+        e.low0 = small && l0 < (1ull << 31) ? (u32)l0 : 0x80000000u;
+        e.low1 = small && l1 < (1ull << 31) ? (u32)l1 : 0x80000000u;
+        const u32 k0 = e.u0 ? (u32)__ffs((int)e.u0) - 1u : 0u, k1 = e.u1 ? (u32)__ffs((int)e.u1) - 1u : 0u;
+        auto inverse = [](u32 o) { u32 q = o; q *= 2u - o * q; q *= 2u - o * q; q *= 2u - o * q; q *= 2u - o * q; return q; };
+        e.inv0 = inverse(e.u0 ? e.u0 >> k0 : 1u); e.inv1 = inverse(e.u1 ? e.u1 >> k1 : 1u);
+        e.cm0 = small && e.u0 && m0 < e.u0 ? 0xffffffffu / e.u0 : 0u;
+        e.cm1 = small && e.u1 && m1 < e.u1 ? 0xffffffffu / e.u1 : 0u;
+        e.k0k1 = k0 | (k1 << 8);
+        e.pos = (u32)pos;
+        S.e[n++] = e;
+    };
+    for (int i = vb; i < ve; ++i) add(hole->probe_pt[0][c[i].value], hole->probe_pt[p1][c[i].value], c[i].pos);
+    int nc = vb - cb;
+    if (nc <= kJoinFewConsts && n + nc <= kJoinEntries) {
+        for (int i = cb; i < vb; ++i) add(c[i].value, c[i].value, c[i].pos);
+        nc = 0;
+    }
+    i64 lo = 0, hi = 0;
+    if (nc > 0) {
+        lo = c[cb].value; hi = c[vb - 1].value;
+        const u64 a = magnitude(lo), b = magnitude(hi), m = a > b ? a : b;
+        most = m > most ? m : most;
+        if (m >> 31) ok = false;
+    }
+    auto member = [&](i64 v) {
+        int x = cb, y = vb;
+        while (x < y) { const int z = (x + y) >> 1; if (c[z].value < v) x = z + 1; else y = z; }
+        return x < vb && c[x].value == v;
+    };
+    S.n_entries = n; S.n_const = nc; S.const_begin = cb;
+    S.cmin = ok ? (i32)lo : 0; S.cmax = ok ? (i32)hi : 0;
+    S.cabs = ok ? (u32)(magnitude(lo) > magnitude(hi) ? magnitude(lo) : magnitude(hi)) : 0u;
+    S.mm = nc > 0 ? (member(t0) ? 1u : 0u) | (member(t1) ? 2u : 0u) : 0u;
+    // |factor| * |operand| * |leaf| must stay below 2^62
+    const i64 A0 = (i64)hole->aff_Aj[0], A1 = (i64)hole->aff_Aj[p1];
+    u64 A = magnitude(A0) > magnitude(A1) ? magnitude(A0) : magnitude(A1);
+    if (A < 1 || A >> 31) A = 1ull << 31;
+    const u64 lim = ((1ull << 62) - 1) / A / most;
+    S.lim = lim < 0x7fffffffull ? (u32)lim : 0x7fffffffu;
+    S.ok = ok && lim > 0 ? 1 : 0;
+}
 
 // The context at every probe (affine in the hole, or a comparison; one thread per probe), and what
 // the rest of the load and the searches go by.  Called by every thread of the CTA once the n
 // probes (ids, coordinates, spec values) are in place; ncand / pass0: how many sampled candidates
-// the probe choice looked at and how many of them satisfied the first probe; big_hits: how many of
-// the kPrepBigSamples candidates of the largest size did.
-__device__ __forceinline__ void probe_contexts(HoleDev* hole, int n, int ncand, int pass0, int big_hits) {
+// the probe choice looked at and how many of them satisfied the first probe.
+__device__ __forceinline__ void probe_contexts(const GrammarDev* g, HoleDev* hole, int n, int ncand, int pass0) {
     const int t = threadIdx.x;
     if (t < kMaxProbe) {
         u64 A = 0, B = 0;
@@ -153,168 +249,170 @@ __device__ __forceinline__ void probe_contexts(HoleDev* hole, int n, int ncand, 
             if (filter_ok && hole->tab_size_cap > 0 && hole->tab_total > 0) probes = n < hole->tab_probes_cap ? n : hole->tab_probes_cap;
             hole->tab_probes = probes;
             hole->tab_max_size = probes > 0 ? hole->tab_size_cap : 0;
-            hole->big_on = 0;                             // (the kernel that fills the big table turns it on)
+            int exact = 0;                                // probes that the tables decide: spec defined, context affine or a comparison
+            while (exact < probes && ((spec_ok & (amask | rmask)) >> exact & 1u)) ++exact;
+            hole->n_exact = exact;
             // Second look at probe 1 inside the filter: for small searches (its cost is in the operand
             // fills, which large tiles amortise anyway) and wherever the sampled candidates say that
             // probe 0 alone lets many through.
             const bool possible = n >= 2 && probes >= 2 && ((spec_ok & (amask | rmask)) >> 1 & 1u);
-            // (one in 256 of the small sample, or one in 4096 of the large candidates: the dense form of the
-            // loops wins from about there, see kAdaptRate)
-            const bool frequent = (ncand > 0 && (u64)pass0 * 256 >= (u64)ncand) || (u64)big_hits * 4096 >= (u64)kPrepBigSamples;
+            // (one in 256 of the sample: the dense form of the loops wins from about there, see kAdaptRate)
+            const bool frequent = ncand > 0 && (u64)pass0 * 256 >= (u64)ncand;
             hole->second = possible && (hole->small_search || frequent) ? 1 : 0;
             hole->second_ok = possible ? 1 : 0;
+            join_targets(hole);
         }
+    }
+    __syncthreads();
+    if (t < g->n_nt) join_leaf_set(g, hole, t);
+}
+
+// Choice of each hole's probe points, once per sketch.  A sample of small candidates (sizes 1, 3, 5, ranks spread evenly)
+// is run on every sample point (prep_sample_kernel: a bit per sample and candidate); the probes are then picked greedily
+// (prepare_kernel): each next probe is the sample that the fewest of the sampled candidates still alive (satisfying
+// all probes picked so far) also satisfy.  Ties: the second probe should differ from the first in spec value and
+// coordinates (the leaf join's conditions compare the two, and an operand that does not tell them apart passes), then
+// the larger |spec| + sum |coordinate| (large, distinct operand values make coincidences rare).
+// Only the amount of work downstream depends on this choice, never a result.
+//
+// The sampling is spread over 8 CTAs of 16 warps per hole (lane = candidate, warp = 4 samples): as one CTA per hole it
+// was bound by the instruction rate of a single SM (130 to 290 us of a load; now 10).
+constexpr int kPrepCands = 256;
+constexpr int kPrepParts = 16;                          // the samples are split over this many warps
+constexpr int kPrepWords = kPrepCands / 32;
+
+// A sample point's coordinates and spec value, and what it scores in a tie (one thread per sample).
+__device__ __forceinline__ void prep_point(const SketchDev* s, const HoleDev* hole, int t, i64* pt, i64& spec, bool& ok, u64& score) {
+    u64 mag = 0;
+    point_coords(s, s->sample_id[t], pt);
+    for (int d = 0; d < s->n_vars; ++d) mag += (u64)(pt[d] < 0 ? -pt[d] : pt[d]);
+    spec = 0;
+    ok = true;
+    if (hole->spec_table != nullptr) spec = hole->spec_table[s->sample_id[t]];
+    else ok = eval_code(hole->spec, hole->spec_len, pt, 0, spec);
+    const u64 m = (u64)(spec < 0 ? -spec : spec);
+    score = ok ? (m > (1ull << 62) ? (1ull << 62) : m) + mag : 0;
+}
+
+// Sizes that the sample is taken from; returns their number.
+__device__ __forceinline__ int prep_sizes(const GrammarDev* g, const HoleDev* hole, int (&sizes)[3]) {
+    int n = 0;
+    for (int k = 1; k <= 5 && k <= hole->max_size; k += 2)
+        if (g->cnt[hole->start_nt][k] > 0) sizes[n++] = k;
+    return n;
+}
+
+__global__ void __launch_bounds__(32 * kPrepParts) prep_sample_kernel(const LoadJob* jobs, u32* masks) {
+    const SketchDev* s = jobs[blockIdx.y].s;
+    const HoleDev* hole = &s->holes[jobs[blockIdx.y].hole];
+    const GrammarDev* g = s->g;
+    __shared__ i64 s_pt[kProbeSamples][kMaxVars];
+    __shared__ i64 s_spec[kProbeSamples];
+    __shared__ int s_ok[kProbeSamples];
+    const int t = threadIdx.x, lane = t & 31, part = t >> 5, word = blockIdx.x;
+    const int ns = s->n_samples;
+    if (t < ns) {
+        i64 pt[kMaxVars], v;
+        bool ok;
+        u64 score;
+        prep_point(s, hole, t, pt, v, ok, score);
+        for (int d = 0; d < s->n_vars; ++d) s_pt[t][d] = pt[d];
+        s_spec[t] = v;
+        s_ok[t] = ok;
+    }
+    int sizes[3] = {1, 1, 1};
+    const int nsz = prep_sizes(g, hole, sizes);
+    u32 code[kMaxSize];
+    int n = 0;
+    if (nsz > 0) {
+        const int c = word * 32 + lane;
+        const int size = sizes[c % nsz];
+        const u64 cnt = g->cnt[hole->start_nt][size];
+        const u64 per = (u64)(kPrepCands / nsz) + 1, slot = (u64)(c / nsz);
+        if (slot < cnt || cnt >= per)                     // small sizes: every rank once, the rest unused
+            n = unrank(g, hole->start_nt, size, cnt >= per ? slot * (cnt / per) : slot, code);
+    }
+    __syncthreads();
+    u32* out = masks + (u64)blockIdx.y * kProbeSamples * kPrepWords;
+    for (int j = part; j < ns; j += kPrepParts) {
+        i64 v;
+        const bool hit = n > 0 && s_ok[j] && eval_cand(code, n, g->leaves, s_pt[j], v) && ctx_matches(hole, s_pt[j], v, s_spec[j]);
+        const u32 b = __ballot_sync(0xffffffffu, hit);
+        if (lane == 0) out[j * kPrepWords + word] = b;
     }
 }
 
-// Choice of each hole's probe points, once per sketch (one CTA per hole).  Threads evaluate the sample
-// points; then a sample of small candidates (sizes 1, 3, 5, ranks spread evenly) is run on
-// every sample point, giving each a bit set of the samples where it satisfies the constraint.
-// The probes are picked greedily: each next probe is the sample that the fewest of the
-// sampled candidates still alive (satisfying all probes picked so far) also satisfy; ties go
-// to the larger |spec| + sum |coordinate| (large, distinct operand values make coincidences
-// rare).  Only the amount of work downstream depends on this choice, never a result.
-constexpr int kPrepThreads = 1024;
-constexpr int kPrepCands = 1024;
-constexpr int kPrepParts = 4;                           // a sampled candidate's sample points are split over this many threads
-__global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jobs) {
+constexpr int kPrepThreads = 64;                        // one thread per sample
+__global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jobs, const u32* masks) {
     SketchDev* s = jobs[blockIdx.x].s;
     __shared__ i64 s_pt[kProbeSamples][kMaxVars];
     __shared__ i64 s_spec[kProbeSamples];
     __shared__ int s_ok[kProbeSamples];
     __shared__ u64 s_score[kProbeSamples];
-    __shared__ u64 s_sig[kPrepCands];                   // per sampled candidate: bit j = it satisfies sample j
-    __shared__ u32 s_mask[kProbeSamples][kPrepCands / 32];    // the same bits, per sample over the candidates
-    __shared__ u32 s_alive[kPrepCands / 32];            // candidates that satisfy every probe chosen so far
-    __shared__ u32 s_count[kProbeSamples];
-    __shared__ u64 s_chosen;
-    __shared__ int s_best;
-    __shared__ int s_big_hits;
-    const int t = threadIdx.x;
-    const int ns = s->n_samples;
-    const int nv = s->n_vars;
+    __shared__ u32 s_mask[kProbeSamples][kPrepWords + 1];
+    __shared__ int s_n, s_pass0;
+    const int t = threadIdx.x, lane = t & 31;
+    const int ns = s->n_samples, nv = s->n_vars;
     const GrammarDev* g = s->g;
     HoleDev* hole = &s->holes[jobs[blockIdx.x].hole];    // one CTA per hole
     if (t < ns) {
-        i64 pt[kMaxVars];
-        u64 coord_mag = 0;
-        point_coords(s, s->sample_id[t], pt);
-        for (int d = 0; d < nv; ++d) {
-            s_pt[t][d] = pt[d];
-            coord_mag += (u64)(pt[d] < 0 ? -pt[d] : pt[d]);
-        }
-        i64 v = 0;
-        bool ok = true;
-        if (hole->spec_table != nullptr) v = hole->spec_table[s->sample_id[t]];
-        else ok = eval_code(hole->spec, hole->spec_len, pt, 0, v);
-        s_spec[t] = v;
-        s_ok[t] = ok;
-        const u64 mag = (u64)(v < 0 ? -v : v);
-        s_score[t] = ok ? (mag > (1ull << 62) ? (1ull << 62) : mag) + coord_mag : 0;
+        i64 pt[kMaxVars], v;
+        bool ok;
+        u64 score;
+        prep_point(s, hole, t, pt, v, ok, score);
+        for (int d = 0; d < nv; ++d) s_pt[t][d] = pt[d];
+        s_spec[t] = v; s_ok[t] = ok; s_score[t] = score;
+        const u32* m = masks + ((u64)blockIdx.x * kProbeSamples + t) * kPrepWords;
+        for (int w = 0; w < kPrepWords; ++w) s_mask[t][w] = m[w];
     }
-    // behaviour of sampled small candidates on the sample points
-    int sizes[3], nsz = 0;
-    for (int k = 1; k <= 5 && k <= hole->max_size; k += 2)
-        if (g->cnt[hole->start_nt][k] > 0) sizes[nsz++] = k;
-    const int ncand = nsz > 0 ? (s->prep_cands < kPrepCands ? s->prep_cands : kPrepCands) : 0;
-    for (int c = t; c < kPrepCands; c += kPrepThreads) s_sig[c] = 0;
-    if (t == 0) s_chosen = 0;
+    int sizes[3] = {1, 1, 1};
+    const int ncand = prep_sizes(g, hole, sizes) > 0 ? kPrepCands : 0;
     __syncthreads();
-    for (int item = t; item < ncand * kPrepParts; item += kPrepThreads) {
-        const int c = item / kPrepParts, part = item % kPrepParts;
-        const int size = sizes[c % nsz];
-        const u64 cnt = g->cnt[hole->start_nt][size];
-        const u64 per = (u64)(ncand / nsz) + 1;
-        const u64 slot = (u64)(c / nsz);
-        if (slot < cnt || cnt >= per) {                       // small sizes: every rank once, the rest unused
-            const u64 rank = cnt >= per ? slot * (cnt / per) : slot;
-            u32 code[kMaxSize];
-            const int n = unrank(g, hole->start_nt, size, rank, code);
-            u64 sig = 0;
-            for (int j = part; j < ns; j += kPrepParts) {
-                i64 v;
-                if (s_ok[j] && eval_cand(code, n, g->leaves, s_pt[j], v) && ctx_matches(hole, s_pt[j], v, s_spec[j]))
-                    sig |= 1ull << j;
-            }
-            if (sig) atomicOr(&s_sig[c], sig);
-        }
-    }
-    __syncthreads();
-    const int nw = (ncand + 31) / 32;
-    for (int i = t; i < ns * nw; i += kPrepThreads) {         // transpose the bits: per sample, a set of candidates
-        const int j = i / nw, w = i % nw;
-        u32 word = 0;
-        for (int b = 0; b < 32 && w * 32 + b < ncand; ++b) word |= (u32)((s_sig[w * 32 + b] >> j) & 1ull) << b;
-        s_mask[j][w] = word;
-    }
-    if (t < nw) s_alive[t] = (t + 1) * 32 <= ncand ? 0xffffffffu : (1u << (ncand - t * 32)) - 1u;
-    __syncthreads();
-    int n = 0;
-    int pass0 = 0;
-    for (; n < kMaxProbe && n < ns; ++n) {
-        const u64 chosen = s_chosen;
-        if (t < ns) {
-            u32 count = 0xffffffffu;
-            if (!((chosen >> t) & 1ull)) {
-                count = 0;
-                for (int w = 0; w < nw; ++w) count += (u32)__popc(s_alive[w] & s_mask[t][w]);
-            }
-            s_count[t] = count;
-        }
-        __syncthreads();
-        if (t == 0) {
+    if (t < 32) {                                       // one warp picks: two samples per lane
+        u32 alive[kPrepWords];
+        for (int w = 0; w < kPrepWords; ++w) alive[w] = ncand ? 0xffffffffu : 0u;
+        u64 chosen = 0;
+        int n = 0, pass0 = 0, first = 0;
+        u32 spec_ok = 0;
+        for (; n < kMaxProbe && n < ns; ++n) {
+            u64 best_key = ~0ull, best_score = 0;         // key: candidates that pass << 32 | 255 - difference from the first probe
             int best = -1;
-            for (int i = 0; i < ns; ++i) {
+            for (int i = lane; i < ns; i += 32) {
                 if ((chosen >> i) & 1ull) continue;
-                if (best < 0 || s_count[i] < s_count[best] || (s_count[i] == s_count[best] && s_score[i] > s_score[best])) best = i;
+                u32 count = 0;
+                for (int w = 0; w < kPrepWords; ++w) count += (u32)__popc(alive[w] & s_mask[i][w]);
+                u32 diff = 0;
+                if (n == 1) {
+                    for (int d = 0; d < nv; ++d) diff += s_pt[i][d] != s_pt[first][d];
+                    if (s_ok[i] && s_spec[i] != s_spec[first] && s_spec[i] != 0) diff += 16;
+                }
+                const u64 key = ((u64)count << 32) | (255u - diff);
+                if (best < 0 || key < best_key || (key == best_key && s_score[i] > best_score)) { best = i; best_key = key; best_score = s_score[i]; }
             }
-            hole->probe_id[n] = s->sample_id[best];
-            for (int d = 0; d < nv; ++d) hole->probe_pt[n][d] = s_pt[best][d];
-            hole->probe_spec[n] = s_spec[best];
-            if (n == 0) { hole->probe_spec_ok = 0; pass0 = (int)s_count[best]; }
-            if (s_ok[best]) hole->probe_spec_ok |= 1u << n;
-            s_chosen = chosen | (1ull << best);
-            s_best = best;
+            for (int o = 16; o > 0; o >>= 1) {
+                const u64 k2 = __shfl_xor_sync(0xffffffffu, best_key, o), sc2 = __shfl_xor_sync(0xffffffffu, best_score, o);
+                const int b2 = __shfl_xor_sync(0xffffffffu, best, o);
+                if (b2 >= 0 && (best < 0 || k2 < best_key || (k2 == best_key && (sc2 > best_score || (sc2 == best_score && b2 < best))))) {
+                    best = b2; best_key = k2; best_score = sc2;
+                }
+            }
+            chosen |= 1ull << best;
+            if (n == 0) { first = best; pass0 = (int)(best_key >> 32); }
+            if (s_ok[best]) spec_ok |= 1u << n;
+            for (int w = 0; w < kPrepWords; ++w) alive[w] &= s_mask[best][w];
+            if (lane == 0) { hole->probe_id[n] = s->sample_id[best]; hole->probe_spec[n] = s_spec[best]; }
+            if (lane < nv) hole->probe_pt[n][lane] = s_pt[best][lane];
         }
-        __syncthreads();
-        if (t < nw) s_alive[t] &= s_mask[s_best][t];
-        __syncthreads();
-    }
-    if (t == 0) {
-        hole->n_probe = n;
-        if (n == 0) hole->probe_spec_ok = 0;
-        s_big_hits = 0;
-    }
-    __syncthreads();
-    // How often the first probe lets a candidate through is estimated once more on random candidates
-    // of the largest size, where nearly all of a search's work is: the behaviour of expressions of one
-    // to five nodes says little about those of nine.
-    int big_size = hole->max_size;
-    while (big_size > 1 && g->cnt[hole->start_nt][big_size] == 0) --big_size;
-    const bool sample_big = n > 0 && big_size >= 3 && (hole->probe_spec_ok & 1u) && !hole->small_search;      // (a small search takes the second look anyway)
-    if (sample_big) {
-        const u64 cnt = g->cnt[hole->start_nt][big_size];
-        i64 pt0[kMaxVars];
-        for (int d = 0; d < nv; ++d) pt0[d] = hole->probe_pt[0][d];
-        const i64 spec0 = hole->probe_spec[0];
-        for (int c = t; c < kPrepBigSamples; c += kPrepThreads) {
-            u64 x = (u64)(c + 1) * 0x9E3779B97F4A7C15ull;     // (a fixed scramble of the sample's number)
-            x ^= x >> 29; x *= 0xBF58476D1CE4E5B9ull; x ^= x >> 32;
-            u32 code[kMaxSize];
-            const int len = unrank(g, hole->start_nt, big_size, __umul64hi(x, cnt), code);
-            i64 v;
-            if (eval_cand(code, len, g->leaves, pt0, v) && ctx_matches(hole, pt0, v, spec0)) atomicAdd(&s_big_hits, 1);
+        if (lane == 0) {
+            hole->n_probe = n;
+            hole->probe_spec_ok = spec_ok;
+            hole->sample_pass0 = pass0;                   // sampled candidates that satisfy the first probe chosen
+            hole->sample_n = ncand;
+            s_n = n; s_pass0 = pass0;
         }
     }
     __syncthreads();
-    const int big_hits = sample_big ? s_big_hits : 0;
-    if (t == 0) {
-        hole->sample_pass0 = pass0;                       // sampled candidates that satisfy the first probe chosen
-        hole->sample_n = ncand;
-        hole->sample_big = big_hits;
-    }
-    __syncthreads();
-    probe_contexts(hole, n, ncand, pass0, big_hits);
+    probe_contexts(g, hole, s_n, ncand, s_pass0);
 }
 
 // The probes of a hole replaced by the host (xp_sketch_refine: points that ended whole-domain
@@ -338,7 +436,7 @@ __global__ void __launch_bounds__(32) reprobe_kernel(const LoadJob* jobs) {
     const u32 okmask = __ballot_sync(0xffffffffu, ok);
     if (t == 0) hole->probe_spec_ok = okmask;
     __syncthreads();
-    probe_contexts(hole, n, hole->sample_n, hole->sample_pass0, hole->sample_big);
+    probe_contexts(s->g, hole, n, hole->sample_n, hole->sample_pass0);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -867,19 +965,22 @@ __device__ __noinline__ bool check_points(const CandShared& c, const SketchDev* 
     return true;
 }
 
-// A candidate that passed the probes goes into the global queue for the verification kernel.
+// A candidate that passed the probes goes into the global queue for the verification kernel (and,
+// when its check spans more than one chunk of points, on the list of long ones).
 // Returns false if the queue is full: the caller's warp then checks the candidate itself.
-__device__ __forceinline__ bool push_survivor(const PlanDev& plan, const SegDev& seg, u64 rank, u32 vars) {
+__device__ __forceinline__ bool push_survivor(const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, int sketch, int hole_index, int size,
+                                              int acc, u64 rank, u32 vars) {
     // (the counter saturates: once the queue is full nothing is added, so it cannot wrap around
     // and hand out a slot twice however many survivors a search has)
     if (*(volatile const u32*)plan.surv_n >= plan.surv_cap) return false;
     const u32 at = atomicAdd(plan.surv_n, 1u);
     if (at >= plan.surv_cap) return false;
     SurvDev r;
-    r.rank = rank; r.sketch = seg.sketch; r.hole = seg.hole; r.size = seg.size; r.acc = seg.acc;
+    r.rank = rank; r.sketch = sketch; r.hole = hole_index; r.size = size; r.acc = acc;
     r.state = 0; r.vars = vars;
     plan.surv[at] = r;
     if (plan.surv_hist) atomicAdd(&plan.surv_hist[r.acc], 1u);       // (for the hole order the verification walks)
+    if (plan.max_chunks > 1 && proj_points(sk, hole, vars, nullptr) > (i64)kVerifyChunk) plan.surv_long[atomicAdd(plan.surv_long_n, 1u)] = at;
     return true;
 }
 
@@ -936,7 +1037,7 @@ __device__ __noinline__ void linear_ticket(EvalShared& sh, const PlanDev& plan, 
                 u32 vars = 0;
                 for (int k = 0; k < n; ++k)
                     if (!(code[k] & kOpBit)) { const i32 var = g->leaves[code[k]].var; if (var >= 0) vars |= 1u << var; }
-                pending = !push_survivor(plan, seg, rank, vars);
+                pending = !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
             }
         }
         warp_verify_pending(sh, sk, hole, seg.size, pending, rank, my_evals);
@@ -981,11 +1082,6 @@ __device__ __forceinline__ void push_hit(EvalShared& sh, u32 reg_idx, u32 slot, 
 __device__ __noinline__ bool operand_value(const GrammarDev* g, const HoleDev* hole, int pr, int nt, int size, u64 rank, i64& v) {
     const int tmax = hole->tab_max_size;
     const u64 pbase = (u64)pr * hole->tab_total;
-    if (pr == 0 && size == hole->big_size && hole->big_on) {
-        const u64 at = hole->big_off[nt] + rank;
-        v = hole->big_val[at];
-        return hole->big_ok[at] != 0;
-    }
     if (size <= tmax) {
         u64 at = pbase + hole->tab_off[nt][size] + rank;
         if (!XP_CHECKED(pr < hole->tab_probes && hole->tab_off[nt][size] + rank < hole->tab_total && rank < g->cnt[nt][size], kChkTable)) at = 0;
@@ -1047,25 +1143,6 @@ __device__ __noinline__ u32 fill_reg_operands(const GrammarDev* g, const HoleDev
         if (v > -(1ll << 31) && v < (1ll << 31)) fits |= 1u << j;
     };
     int j = 0;
-    if (pr == 0 && size == hole->big_size && hole->big_on) {      // tabulated at the first probe: consecutive entries
-        const u64 at = hole->big_off[nt] + rank;
-        if (n == kNA && (at & 7ull) == 0) {
-            // the usual case: eight aligned entries, fetched with five independent loads
-            const u64 oks = *reinterpret_cast<const u64*>(hole->big_ok + at);
-            const longlong2* src = reinterpret_cast<const longlong2*>(hole->big_val + at);
-            longlong2 v[kNA / 2];
-#pragma unroll
-            for (int k = 0; k < kNA / 2; ++k) v[k] = src[k];
-#pragma unroll
-            for (int k = 0; k < kNA / 2; ++k) {
-                if ((oks >> (16 * k)) & 0xffull) put(2 * k, v[k].x);
-                if ((oks >> (16 * k + 8)) & 0xffull) put(2 * k + 1, v[k].y);
-            }
-            return alive;
-        }
-        for (; j < n; ++j) if (hole->big_ok[at + j]) put(j, hole->big_val[at + j]);
-        return alive;
-    }
     if (size > tmax && tmax >= 1 && size >= 3) {
         int op, lnt, rnt, a;
         u64 l, r;
@@ -1148,87 +1225,64 @@ __global__ void __launch_bounds__(256) stage_spec_kernel(const SketchDev* sk, in
 }
 
 // Bottom-up construction of one size of a hole's subtree-value tables: thread = (nonterminal,
-// rank); the operands' values come from the smaller sizes built by earlier launches.
+// rank) and one group of kSubProbes probes; the operands' values come from the smaller sizes built by
+// earlier launches.  (One thread for several probes: the unranking, two 64-bit divisions, is done once for them.)
+// The first group also writes what does not depend on the probe, and the pair of values the leaf join reads.
+constexpr int kSubProbes = 4;
 __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int size) {
     const SketchDev* sk = jobs[blockIdx.z].s;           // one grid layer per hole of the batch
-    const int hole_index = jobs[blockIdx.z].hole;
-    const int pr = blockIdx.y;                          // one grid row per probe
+    HoleDev* hole = &sk->holes[jobs[blockIdx.z].hole];
+    const int pr0 = blockIdx.y * kSubProbes;            // one grid row per group of probes
     const GrammarDev* g = sk->g;
-    HoleDev* hole = &sk->holes[hole_index];
-    if (pr >= hole->tab_probes || size > hole->tab_max_size) return;      // (the grid is sized for the most there can be)
-    const u64 pbase = (u64)pr * hole->tab_total;
+    if (pr0 >= hole->tab_probes || size > hole->tab_max_size) return;      // (the grid is sized for the most there can be)
+    const int n_pr = hole->tab_probes - pr0 < kSubProbes ? hole->tab_probes - pr0 : kSubProbes;
+    const u64 total = hole->tab_total;
+    // (local copies: the stores below cannot change them, which the compiler cannot know of fields of *hole)
+    i64* __restrict__ tab_val = hole->tab_val;
+    unsigned char* __restrict__ tab_ok = hole->tab_ok;
     u64 idx = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     for (int nt = 0; nt < g->n_nt; ++nt) {
         const u64 c = g->cnt[nt][size];
         if (idx >= c) { idx -= c; continue; }
-        i64 v = 0;
-        bool ok = true;
+        const u64 at = hole->tab_off[nt][size] + idx;
+        LeafDev lf{-1, 0, 0};
+        int op = 0;
+        u64 la = 0, ra = 0;
         u32 vars = 0;
         if (size == 1) {
-            const LeafDev lf = g->leaves[g->leaf_begin[nt] + (i32)idx];
-            v = lf.var >= 0 ? hole->probe_pt[pr][lf.var] : lf.value;
+            lf = g->leaves[g->leaf_begin[nt] + (i32)idx];
             vars = lf.var >= 0 ? 1u << lf.var : 0u;
         } else {
-            int op, lnt, rnt, a;
+            int lnt, rnt, a;
             u64 l, r;
             unrank_root(g, nt, size, idx, op, lnt, rnt, a, l, r);
-            const u64 la = pbase + hole->tab_off[lnt][a] + l, ra = pbase + hole->tab_off[rnt][size - 1 - a] + r;
-            ok = hole->tab_ok[la] && hole->tab_ok[ra] && apply_op(op, hole->tab_val[la], hole->tab_val[ra], v);
-            vars = (u32)hole->tab_vars[hole->tab_off[lnt][a] + l] | (u32)hole->tab_vars[hole->tab_off[rnt][size - 1 - a] + r];
+            la = hole->tab_off[lnt][a] + l; ra = hole->tab_off[rnt][size - 1 - a] + r;
+            if (pr0 == 0) vars = (u32)hole->tab_vars[la] | (u32)hole->tab_vars[ra];
         }
-        const u64 at = pbase + hole->tab_off[nt][size] + idx;
-        hole->tab_val[at] = v;
-        hole->tab_ok[at] = ok ? 1 : 0;
-        if (pr == 0) hole->tab_vars[hole->tab_off[nt][size] + idx] = (unsigned char)vars;
+        i64 v[kSubProbes];
+        bool ok[kSubProbes];
+#pragma unroll
+        for (int k = 0; k < kSubProbes; ++k) {
+            v[k] = 0; ok[k] = true;
+            if (k >= n_pr) continue;
+            const u64 pbase = (u64)(pr0 + k) * total;
+            if (size == 1) v[k] = lf.var >= 0 ? hole->probe_pt[pr0 + k][lf.var] : lf.value;
+            else ok[k] = tab_ok[pbase + la] && tab_ok[pbase + ra] && apply_op(op, tab_val[pbase + la], tab_val[pbase + ra], v[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kSubProbes; ++k)
+            if (k < n_pr) { tab_val[(u64)(pr0 + k) * total + at] = v[k]; tab_ok[(u64)(pr0 + k) * total + at] = ok[k] ? 1 : 0; }
+        if (pr0 == 0) {
+            hole->tab_vars[at] = (unsigned char)vars;
+            const i64 x = v[0], y = hole->join_p1 ? v[1] : v[0];
+            const bool defined = ok[0] && (!hole->join_p1 || ok[1]);
+            const bool narrow = x > -(1ll << 31) && x < (1ll << 31) && y > -(1ll << 31) && y < (1ll << 31);
+            int2 pair;
+            pair.x = defined && narrow ? (i32)x : kPairNone;
+            pair.y = defined ? (narrow ? (i32)y : 1) : 0;
+            reinterpret_cast<int2*>(hole->tab_pair)[at] = pair;
+        }
         return;
-    }
-}
-
-// The big table: values at probe 0 of every subtree of size big_size, from the smaller sizes'
-// tables by one level of unranking.  A thread writes 8 consecutive entries of one nonterminal (the
-// nonterminals' ranges start at multiples of 8): the first is unranked, the others follow by
-// advancing the operand ranks like an odometer (right operand fastest).  The first thread turns
-// the table on for the searches once the launch is under way for a hole whose smaller tables
-// exist (the flag is read by later launches only).
-constexpr int kBigPerThread = 8;
-__global__ void __launch_bounds__(256) bigvalue_kernel(const LoadJob* jobs) {
-    const SketchDev* sk = jobs[blockIdx.y].s;
-    HoleDev* hole = &sk->holes[jobs[blockIdx.y].hole];
-    const int size = hole->big_size;
-    if (size <= 0 || hole->tab_probes < 1 || hole->tab_max_size != hole->tab_size_cap || hole->big_val == nullptr) return;
-    const GrammarDev* g = sk->g;
-    const u64 t = (u64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t == 0) hole->big_on = 1;
-    const u64 at0 = t * (u64)kBigPerThread;
-    if (at0 >= hole->big_total) return;
-    int nt = g->n_nt - 1;                               // the last nonterminal whose range starts at or before at0
-    while (nt > 0 && hole->big_off[nt] > at0) --nt;
-    const u64 c = g->cnt[nt][size], idx = at0 - hole->big_off[nt];
-    if (idx >= c) return;                               // (padding between two nonterminals' ranges)
-    const int n = c - idx < (u64)kBigPerThread ? (int)(c - idx) : kBigPerThread;
-    // (local copies: the stores below cannot change them, which the compiler cannot know of fields of *hole)
-    const i64* __restrict__ tab_val = hole->tab_val;
-    const unsigned char* __restrict__ tab_ok = hole->tab_ok;
-    i64* __restrict__ out_val = hole->big_val + at0;
-    unsigned char* __restrict__ out_ok = hole->big_ok + at0;
-    int j = 0;
-    while (j < n) {
-        int op, lnt, rnt, a;
-        u64 l, r;
-        unrank_root(g, nt, size, idx + j, op, lnt, rnt, a, l, r);
-        const u64 cl = g->cnt[lnt][a], cr = g->cnt[rnt][size - 1 - a];
-        const u64 lbase = hole->tab_off[lnt][a], rbase = hole->tab_off[rnt][size - 1 - a];      // (probe 0: first copy of the tables)
-        while (j < n && l < cl) {                       // until this (production, left size) block ends
-            const bool lok = tab_ok[lbase + l] != 0;
-            const i64 lv = tab_val[lbase + l];
-            for (; j < n && r < cr; ++r, ++j) {
-                i64 v = 0;
-                const bool ok = lok && tab_ok[rbase + r] && apply_op(op, lv, tab_val[rbase + r], v);
-                out_val[j] = v;
-                out_ok[j] = ok ? 1 : 0;
-            }
-            if (r == cr) { r = 0; ++l; }
-        }
     }
 }
 
@@ -1695,7 +1749,7 @@ __device__ __noinline__ void drain_queue(EvalShared& sh, const PlanDev& plan, co
                 ++passes;
                 const u32 vars = sk->project ? operand_vars(g, hole, seg.reg_nt, seg.reg_size, rr) |
                                                operand_vars(g, hole, seg.bc_nt, seg.bc_size, br) : 0xffu;
-                pending = !push_survivor(plan, seg, rank, vars);      // (the hit's own segment: the ticket at hand may be another's)
+                pending = !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);      // (the hit's own segment: the ticket at hand may be another's)
             }
         }
         warp_verify_pending(sh, sk, hole, cand_size, pending, rank, my_evals);
@@ -2164,6 +2218,10 @@ __global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const PlanD
     flush_acc(sh, plan, my_evals);
 }
 
+}  // namespace xp
+#include "xp_join.cuh"
+namespace xp {
+
 // ------------------------------------------------------------------------------------------
 // verify: whole-domain check of the queued survivors
 // ------------------------------------------------------------------------------------------
@@ -2214,18 +2272,6 @@ __global__ void __launch_bounds__(256) surv_scatter_kernel(const PlanDev plan) {
     if (i >= n) return;
     const int acc = plan.surv[i].acc;
     plan.surv_sorted[plan.surv_off[acc] + atomicAdd(&plan.surv_hist[acc], 1u)] = i;
-}
-
-// One thread per queued survivor: those whose (projected) domain has more than one chunk of points
-// go on the list of long survivors.
-__global__ void __launch_bounds__(256) surv_long_kernel(const PlanDev plan) {
-    const u32 pushed = *plan.surv_n;
-    const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
-    const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const SurvDev sv = plan.surv[i];
-    const SketchDev* sk = plan.sketches[sv.sketch];
-    if (proj_points(sk, &sk->holes[sv.hole], sv.vars, nullptr) > (i64)kVerifyChunk) plan.surv_long[atomicAdd(plan.surv_long_n, 1u)] = i;
 }
 
 // ---- whole-domain check of several survivors of one hole together ----
@@ -2433,6 +2479,15 @@ __device__ __noinline__ void verify_batch(VerifyWarp& w, const SketchDev* sk, co
     }
 }
 
+// Notes that a survivor has passed one of its `chunks` chunks; the one that passes last (none has failed) makes it a match.
+__device__ __forceinline__ void chunk_passed(const PlanDev& plan, SurvDev* sv, u32 chunks) {
+    if (atomicAdd(&sv->state, 1u) + 1u != chunks) return;
+    AccDev* a = &plan.acc[sv->acc];
+    atomicAdd(&a->match_count[sv->size], 1ull);
+    atomicMin(&a->min_rank[sv->size], sv->rank);
+}
+__device__ __forceinline__ u32 chunks_of(i64 n_points) { return (u32)((n_points + kVerifyChunk - 1) / kVerifyChunk); }
+
 // One survivor on one chunk, staged by the warp's first lane (boxes with their sub-box projection,
 // programs that do not fit the arena, contexts that never mention the hole).
 __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 si, u64 chunk) {
@@ -2470,7 +2525,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
         ok = check_points(cand, sk, hole, first, last, evals, &fail_pid);
     }
     if (lane == 0) {
-        if (ok) atomicAdd(&sv->state, 1u);
+        if (ok) chunk_passed(plan, sv, chunks_of(np));
         else if (!(atomicOr(&sv->state, kSurvFailed) & kSurvFailed)) record_killer(hole, fail_pid);   // (once per survivor)
         atomicAdd(&plan.acc[sv->acc].evals, (u64)(last - first));     // points of the chunk (an early exit tries fewer)
     }
@@ -2571,7 +2626,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
                     u64 evals = 0;
                     verify_batch(w, sk, hole, now, my_off, len, narrow, first, last, failed, fail_pid, evals);
                     if ((now >> lane) & 1u) {
-                        if (!failed) atomicAdd(&sv->state, 1u);
+                        if (!failed) chunk_passed(plan, sv, chunks_of(sk->n_points));
                         else if (!(atomicOr(&sv->state, kSurvFailed) & kSurvFailed)) record_killer(hole, fail_pid);
                     }
                     if (lane == 0 && evals) atomicAdd(&plan.acc[acc].evals, evals);
@@ -2585,7 +2640,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
     }
 }
 
-// One thread per queued survivor: it is a match if no chunk failed and every chunk passed.
+// One thread per queued survivor of a sketch without points: there is no chunk to pass, it is a match.
 __global__ void count_kernel(const PlanDev plan) {
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
@@ -2593,33 +2648,16 @@ __global__ void count_kernel(const PlanDev plan) {
     if (i >= n) return;
     const SurvDev sv = plan.surv[i];
     const SketchDev* sk = plan.sketches[sv.sketch];
-    const i64 np = proj_points(sk, &sk->holes[sv.hole], sv.vars, nullptr);
-    const u32 chunks = (u32)((np + kVerifyChunk - 1) / kVerifyChunk);
-    if ((sv.state & kSurvFailed) || sv.state != chunks) return;
+    if (sk->n_points != 0) return;
     AccDev* a = &plan.acc[sv.acc];
     atomicAdd(&a->match_count[sv.size], 1ull);
     atomicMin(&a->min_rank[sv.size], sv.rank);
 }
 
-// ------------------------------------------------------------------------------------------
-// finish: least (size, rank) per hole from the per-size minima
-// ------------------------------------------------------------------------------------------
-
-// One warp per accumulator: lane = size; ballot finds the smallest size with a match.
-__global__ void finish_kernel(AccDev* acc, int n_acc, u32* err) {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
 #ifdef XP_CHECKS
-    if (blockIdx.x == 0 && threadIdx.x == 0) *err = atomicExch(&g_check_word, 0u);     // what the checks recorded, if anything
-#else
-    (void)err;
+// What the index checks recorded, if anything, to the word the host reads.
+__global__ void check_kernel(u32* err) { *err = atomicExch(&g_check_word, 0u); }
 #endif
-    if (w >= n_acc) return;
-    AccDev* a = &acc[w];
-    const bool has = lane <= kMaxSize && a->match_count[lane] > 0;
-    const u32 m = __ballot_sync(0xffffffffu, has);
-    if (lane == 0) a->pad = m ? (u64)(__ffs(m) - 1) : 0ull;     // least size (0 = unsolved)
-}
 
 // ------------------------------------------------------------------------------------------
 // integer peak
@@ -2693,15 +2731,14 @@ __global__ void __launch_bounds__(256) int_div_reciprocal_kernel(u32* out, int i
 // launchers
 // ------------------------------------------------------------------------------------------
 
-cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, cudaStream_t stream) {
-    if (n_jobs <= 0) return cudaSuccess;
-    prepare_kernel<<<n_jobs, kPrepThreads, 0, stream>>>(jobs);
-    return cudaGetLastError();
-}
+size_t prepare_scratch_bytes(int n_jobs) { return sizeof(u32) * (size_t)kProbeSamples * kPrepWords * (size_t)n_jobs; }
 
-cudaError_t launch_bigvalues(const LoadJob* jobs, int n_jobs, u64 most_entries, cudaStream_t stream) {
-    if (most_entries == 0 || n_jobs <= 0) return cudaSuccess;
-    bigvalue_kernel<<<dim3((unsigned)((most_entries / kBigPerThread + 255) / 256 + 1), (unsigned)n_jobs), 256, 0, stream>>>(jobs);
+cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, cudaStream_t stream) {
+    if (n_jobs <= 0) return cudaSuccess;
+    prep_sample_kernel<<<dim3(kPrepWords, (unsigned)n_jobs), 32 * kPrepParts, 0, stream>>>(jobs, (u32*)scratch);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    prepare_kernel<<<n_jobs, kPrepThreads, 0, stream>>>(jobs, (const u32*)scratch);
     return cudaGetLastError();
 }
 
@@ -2730,34 +2767,60 @@ cudaError_t launch_stage_spec(const SketchDev* s, int hole_index, i64 n_points, 
 
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int most_probes, u64 most_entries, cudaStream_t stream) {
     if (most_entries == 0 || most_probes <= 0 || n_jobs <= 0) return cudaSuccess;
-    subvalue_kernel<<<dim3((unsigned)((most_entries + 255) / 256), (unsigned)most_probes, (unsigned)n_jobs), 256, 0, stream>>>(jobs, size);
+    subvalue_kernel<<<dim3((unsigned)((most_entries + 255) / 256), (unsigned)((most_probes + kSubProbes - 1) / kSubProbes), (unsigned)n_jobs), 256, 0, stream>>>(jobs, size);
     return cudaGetLastError();
 }
 
-static int resident_ctas(const void* kernel, size_t dynamic_smem = 0) {
-    int dev = 0, sms = 1, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, dynamic_smem) != cudaSuccess || per_sm < 1) per_sm = 1;
-    return sms * per_sm;
+// CTAs of a kernel that fit the device at a time, and the SM count: asked once per device (the queries, and
+// the shared-memory attribute of the verification kernel, cost a microsecond or two each).
+struct Residency { int sms, eval_sparse, eval_dense, verify, join; };
+static const Residency* residency() {
+    static Residency table[64];
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (known[dev].load(std::memory_order_acquire)) return &table[dev];
+    Residency r;
+    auto per_sm = [](const void* kernel, int threads, size_t smem) {
+        int n = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) == cudaSuccess && n > 0 ? n : 1;
+    };
+    const size_t vsmem = sizeof(VerifyWarp) * kVerifyWarps;
+    if (cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
+    if (cudaFuncSetAttribute((const void*)verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsmem) != cudaSuccess) return nullptr;
+    r.eval_sparse = r.sms * per_sm((const void*)eval_kernel<false>, kThreads, 0);
+    r.eval_dense = r.sms * per_sm((const void*)eval_kernel<true>, kThreads, 0);
+    r.verify = r.sms * per_sm((const void*)verify_kernel, kVerifyThreads, vsmem);
+    r.join = r.sms * per_sm((const void*)join_kernel<kJoinP>, kJoinThreads, 0);
+    static std::mutex mu;                                 // (two first calls at the same time compute the same values)
+    std::lock_guard<std::mutex> lock(mu);
+    table[dev] = r;
+    known[dev].store(1, std::memory_order_release);
+    return &table[dev];
 }
+int search_warps() { const Residency* r = residency(); return r ? r->join * kJoinWarps : 1; }
 
-static PlanDev plan_on(char* base, const SearchLayout& L, int n_segs, int n_sketches, u32 max_chunks) {
+static PlanDev plan_on(char* base, const SearchLayout& L) {
     PlanDev pd;
     pd.ticket_base = 0;
     pd.n_tickets = 0;
-    pd.n_segs = n_segs;
-    pd.n_sketches = n_sketches;
+    pd.n_segs = L.n_segs;
+    pd.n_sketches = L.n_sketches;
     pd.ticket = (u64*)base;
     pd.verify_ticket = (u64*)(base + 8);
     pd.surv_n = (u32*)(base + 16);
     pd.err = (u32*)(base + 20);
     pd.segs = (const SegDev*)(base + L.segs);
+    pd.jsegs = (const JoinSeg*)(base + L.jsegs);
+    pd.jgroups = (const JoinGroup*)(base + L.jgroups);
+    pd.n_jsegs = L.n_jsegs; pd.pad0 = 0;
+    pd.join_base = pd.n_join = 0;
+    pd.join_ticket = (u64*)(base + 32);
     pd.sketches = (const SketchDev* const*)(base + L.sketches);
     pd.acc = (AccDev*)(base + L.acc);
     pd.surv = (SurvDev*)(base + L.surv);
     pd.surv_cap = L.surv_cap;
-    pd.max_chunks = max_chunks;
+    pd.max_chunks = L.max_chunks;
     pd.n_acc = L.n_acc;
     const bool order = L.n_acc > 1;                       // (one hole: the queue is in hole order as it is)
     pd.surv_hist = order ? (u32*)(base + L.hist) : nullptr;
@@ -2768,32 +2831,44 @@ static PlanDev plan_on(char* base, const SearchLayout& L, int n_segs, int n_sket
     return pd;
 }
 
-// Stages 1 and 2 for the tickets [t_begin, t_end) of the plan staged at `base`.  A search is one
-// such launch, or several in a row when the host wants to look at a cancel word or a clock in
-// between; `restart` says that the ticket counter has to be set back to zero first (every launch
-// but the first, whose counter the staged copy has just zeroed).
-cudaError_t launch_search_part(char* base, const SearchLayout& L, u64 t_begin, u64 t_end, bool restart, int n_segs,
-                               int n_sketches, u32 max_chunks, cudaStream_t stream, int* n_launches) {
+// The tickets [t_begin, t_end) of the leaf join, or (join false) of the operand tiles and linear pieces, of the
+// plan staged at `base`.  A search is one such launch of each kind that has tickets, or several in a row when
+// the host wants to look at a cancel word or a clock in between; `restart` says that the ticket counter has
+// to be set back to zero first (every launch but the first, whose counter the staged copy has just zeroed).
+cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64 t_begin, u64 t_end, bool restart, cudaStream_t stream,
+                               int* n_launches) {
     if (t_end <= t_begin) return cudaSuccess;
     cudaError_t e;
-    if (restart && (e = cudaMemsetAsync(base, 0, 8, stream)) != cudaSuccess) return e;
-    PlanDev pd = plan_on(base, L, n_segs, n_sketches, max_chunks);
-    pd.ticket_base = t_begin;
-    pd.n_tickets = t_end;
-    const void* kernel = L.dense ? (const void*)eval_kernel<true> : (const void*)eval_kernel<false>;
-    u64 ctas = (u64)resident_ctas(kernel, 0);             // persistent CTAs: one wave
-    if (ctas > t_end - t_begin) ctas = t_end - t_begin;
-    if (L.dense) eval_kernel<true><<<(unsigned)ctas, kThreads, 0, stream>>>(pd);
-    else eval_kernel<false><<<(unsigned)ctas, kThreads, 0, stream>>>(pd);
+    const Residency* R = residency();
+    if (!R) return cudaErrorInvalidDevice;
+    if (restart && (e = cudaMemsetAsync(join ? base + 32 : base, 0, 8, stream)) != cudaSuccess) return e;
+    PlanDev pd = plan_on(base, L);
+    if (join) {
+        pd.join_base = t_begin;
+        pd.n_join = t_end;
+        // a wave of persistent CTAs; a small search gets one warp per ticket on as many SMs as there are tickets
+        u64 ctas = t_end - t_begin;
+        if (ctas > (u64)R->join) ctas = R->join;
+        if (L.join_wide) join_kernel<kJoinP><<<(unsigned)ctas, kJoinThreads, 0, stream>>>(pd);
+        else join_kernel<1><<<(unsigned)ctas, kJoinThreads, 0, stream>>>(pd);
+    } else {
+        pd.ticket_base = t_begin;
+        pd.n_tickets = t_end;
+        u64 ctas = (u64)(L.dense ? R->eval_dense : R->eval_sparse);       // persistent CTAs: one wave
+        if (ctas > t_end - t_begin) ctas = t_end - t_begin;
+        if (L.dense) eval_kernel<true><<<(unsigned)ctas, kThreads, 0, stream>>>(pd);
+        else eval_kernel<false><<<(unsigned)ctas, kThreads, 0, stream>>>(pd);
+    }
     *n_launches += 1;
     return cudaGetLastError();
 }
 
-// Stage 3 and the reductions, after every part of the search has been queued.
-cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, int n_segs, int n_sketches, int n_acc,
-                              u32 max_chunks, cudaStream_t stream, int* n_launches) {
-    PlanDev pd = plan_on(base, L, n_segs, n_sketches, max_chunks);
+// Stage 3, after every part of the search has been queued.
+cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, cudaStream_t stream, int* n_launches) {
+    PlanDev pd = plan_on(base, L);
     cudaError_t e;
+    const Residency* R = residency();
+    if (!R) return cudaErrorInvalidDevice;
     if (any_tickets) {
         if (pd.surv_sorted) {
             surv_scan_kernel<<<1, 1024, 0, stream>>>(pd.surv_hist, pd.surv_off, pd.n_acc);
@@ -2802,30 +2877,27 @@ cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_ticket
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *n_launches += 2;
         }
-        if (max_chunks > 1) {
-            surv_long_kernel<<<(L.surv_cap + 255) / 256, 256, 0, stream>>>(pd);
+        verify_kernel<<<R->verify, kVerifyThreads, sizeof(VerifyWarp) * kVerifyWarps, stream>>>(pd);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        *n_launches += 1;
+        if (L.empty_domain) {
+            count_kernel<<<(L.surv_cap + 255) / 256, 256, 0, stream>>>(pd);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *n_launches += 1;
         }
-        const size_t vsmem = sizeof(VerifyWarp) * kVerifyWarps;
-        if ((e = cudaFuncSetAttribute((const void*)verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsmem)) != cudaSuccess) return e;
-        verify_kernel<<<resident_ctas((const void*)verify_kernel, vsmem), kVerifyThreads, vsmem, stream>>>(pd);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        count_kernel<<<(L.surv_cap + 255) / 256, 256, 0, stream>>>(pd);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        *n_launches += 2;
     }
-    const int warps_per_block = 8;
-    finish_kernel<<<(n_acc + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, stream>>>(pd.acc, n_acc, pd.err);
+#ifdef XP_CHECKS
+    check_kernel<<<1, 1, 0, stream>>>(pd.err);
     *n_launches += 1;
+#endif
     return cudaGetLastError();
 }
 
-cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, int n_segs, int n_sketches, int n_acc,
-                          u32 max_chunks, cudaStream_t stream, int* n_launches) {
-    cudaError_t e = launch_search_part(base, L, 0, n_tickets, false, n_segs, n_sketches, max_chunks, stream, n_launches);
+cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, u64 n_join, cudaStream_t stream, int* n_launches) {
+    cudaError_t e = launch_search_part(base, L, true, 0, n_join, false, stream, n_launches);
+    if (e == cudaSuccess) e = launch_search_part(base, L, false, 0, n_tickets, false, stream, n_launches);
     if (e != cudaSuccess) return e;
-    return launch_search_end(base, L, n_tickets > 0, n_segs, n_sketches, n_acc, max_chunks, stream, n_launches);
+    return launch_search_end(base, L, n_tickets + n_join > 0, stream, n_launches);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -2843,8 +2915,7 @@ static void* g_static_scratch_addr[64];      // per device, filled on the first 
 // Copies the staged head of the plan (counters and accumulators in their start state, which
 // also wipes what the last call left) into the fixed array, runs the search on it, and queues
 // the copy of the accumulators back to `acc_out`.  Allocates nothing.
-cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, int n_segs, int n_acc,
-                                 u32 max_chunks, AccDev* acc_out, cudaStream_t stream) {
+cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, cudaStream_t stream) {
     if (L.total > kStaticScratchBytes) return cudaErrorInvalidValue;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -2860,9 +2931,9 @@ cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n
     e = cudaMemcpyAsync(base, stage, L.head, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return e;
     int launches = 0;
-    e = launch_search(base, L, n_tickets, n_segs, 1, n_acc, max_chunks, stream, &launches);
+    e = launch_search(base, L, n_tickets, n_join, stream, &launches);
     if (e != cudaSuccess) return e;
-    return cudaMemcpyAsync(acc_out, base + L.acc, sizeof(AccDev) * (size_t)n_acc, cudaMemcpyDeviceToHost, stream);
+    return cudaMemcpyAsync(acc_out, base + L.acc, sizeof(AccDev) * (size_t)L.n_acc, cudaMemcpyDeviceToHost, stream);
 }
 
 cudaError_t launch_int32_peak(int which, u32* out, int blocks, int iters, cudaStream_t stream) {

@@ -7,33 +7,36 @@
 
 namespace xp {
 
-cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, cudaStream_t stream);
+size_t prepare_scratch_bytes(int n_jobs);
+cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, cudaStream_t stream);
 cudaError_t launch_reprobe(const LoadJob* jobs, int n_jobs, cudaStream_t stream);
 cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
 cudaError_t launch_stage_points(const SketchDev* s, i64 n_points, i32* coords, cudaStream_t stream);
 cudaError_t launch_stage_spec(const SketchDev* s, int hole_index, i64 n_points, i64* spec, u32* bad, cudaStream_t stream);
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int most_probes, u64 most_entries, cudaStream_t stream);
-cudaError_t launch_bigvalues(const LoadJob* jobs, int n_jobs, u64 most_entries, cudaStream_t stream);
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
-//      build only)   -- zero at launch
-//   segs, sketches, acc: staged from the host;  [0, head) is what the host copies in
+//      build only), 24: long survivors (u32), 32: join ticket (u64)   -- zero at launch
+//   segs, jsegs, jgroups, sketches, acc: staged from the host;  [0, head) is what the host copies in
 //   hist: survivors per accumulator slot, zero at launch (staged);
 //   surv: the survivor queue (surv_cap entries); sort_off, sorted: its hole order -- written by the kernels only
-struct SearchLayout { size_t segs, sketches, acc, hist, head, surv, sort_off, sorted, longs, total; u32 surv_cap; int n_acc;
-                      int dense; /* some hole of the plan takes the second look: launch the search kernel's dense form */ };
+struct SearchLayout {
+    size_t segs, jsegs, jgroups, sketches, acc, hist, head, surv, sort_off, sorted, longs, total;
+    u32 surv_cap, max_chunks;        // max_chunks: chunks of the whole-domain check that the largest domain needs
+    int n_segs, n_jsegs, n_sketches, n_acc;
+    int dense;                       // some hole of the plan takes the second look: launch the search kernel's dense form
+    int join_wide;                   // tickets of the leaf join are long enough for several operands per lane
+    int empty_domain;                // some sketch has no points at all
+};
 
-// The whole search on a staged scratch: eval_kernel, verify_kernel, count_kernel, finish_kernel;
-// or the same in pieces: eval_kernel over one range of tickets at a time, then the rest.
-cudaError_t launch_search_part(char* base, const SearchLayout& L, u64 t_begin, u64 t_end, bool restart, int n_segs,
-                               int n_sketches, u32 max_chunks, cudaStream_t stream, int* n_launches);
-cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, int n_segs, int n_sketches, int n_acc,
-                              u32 max_chunks, cudaStream_t stream, int* n_launches);
-cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, int n_segs, int n_sketches, int n_acc,
-                          u32 max_chunks, cudaStream_t stream, int* n_launches);
+// The whole search on a staged scratch, or the same in pieces: one range of tickets at a time, then the rest.
+cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64 t_begin, u64 t_end, bool restart, cudaStream_t stream,
+                               int* n_launches);
+cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, cudaStream_t stream, int* n_launches);
+cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, u64 n_join, cudaStream_t stream, int* n_launches);
+int search_warps();                                  // warps of the leaf join that run at a time
 constexpr size_t kStaticScratchBytes = 1u << 20;     // fixed scratch of the allocation-free entry point
-cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, int n_segs, int n_acc,
-                                 u32 max_chunks, AccDev* acc_out, cudaStream_t stream);
+cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, cudaStream_t stream);
 cudaError_t launch_int32_peak(int which, u32* out, int blocks, int iters, cudaStream_t stream);
 
 // What the library's other source files may know of a grammar and a loaded sketch (defined in xp_api.cu).
