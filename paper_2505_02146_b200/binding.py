@@ -142,11 +142,12 @@ class xp_joint_view(C.Structure):
 
 
 _lib = None
+_m = None          # the CPython extension that fills the C descriptors (csrc/xp_marshal.c)
 
 
 def load(path: Optional[str] = None):
     """Loads (building first if the sources are newer) the shared library; raises if that fails."""
-    global _lib
+    global _lib, _m
     if _lib is not None:
         return _lib
     # XP_CHECKED_BUILD=1 in the environment selects the variant with index checks compiled in
@@ -187,6 +188,9 @@ def load(path: Optional[str] = None):
     lib.xp_pair_result_free.restype = None
     for name in EXPORTS:
         getattr(lib, name)
+    _build.build_marshal()
+    from . import _marshal
+    _m = _marshal
     _lib = lib
     return lib
 
@@ -197,10 +201,9 @@ def _check(status: int) -> None:
 
 
 def _code(instrs) -> "C.Array":
-    arr = (xp_instr * max(1, len(instrs)))()
-    for i, (k, a, v) in enumerate(instrs):
-        arr[i].kind, arr[i].arg, arr[i].value = k, a, v
-    return arr
+    load()
+    n = len(instrs)
+    return (xp_instr * n).from_buffer_copy(_m.code(instrs)) if n else (xp_instr * 1)()
 
 
 # ------------------------------------------------------------------------------------------
@@ -229,16 +232,9 @@ class GrammarDesc:
 def marshal_grammar(g) -> GrammarDesc:
     """Encodes an ``xp_instances.Grammar`` as the C descriptor ``xp_grammar_create`` takes; a caller that
     creates the same grammar again and again does this once."""
-    nv = len(g.variables)
-    names = [v.name.encode() for v in g.variables]
-    vs = (xp_variable * max(1, nv))()
-    for i, v in enumerate(g.variables):
-        vs[i].name, vs[i].lo, vs[i].hi = names[i], v.lo, v.hi
-    ps = (xp_production * len(g.productions))()
-    for i, p in enumerate(g.productions):
-        q = ps[i]
-        q.lhs, q.kind, q.var, q.op, q.left, q.right, q.value = p.lhs, p.kind, p.var, p.op, p.left, p.right, p.value
-    return GrammarDesc(xp_grammar_desc(nv, vs, g.n_nonterminals, len(g.productions), ps), g, (names, vs, ps))
+    load()
+    address, owner = _m.grammar(g)
+    return GrammarDesc(xp_grammar_desc.from_address(address), g, owner)
 
 
 def xp_grammar_create(g) -> Grammar:
@@ -283,36 +279,9 @@ def _ptr_of(x) -> Tuple[int, int, object]:
     return int(x.data_ptr()), int(x.is_cuda), x      # torch tensor: device memory only, no torch compute
 
 
-def _fill_sketch_desc(desc, sk, coords, spec_tables, keep) -> int:
-    """Marshals one ``xp_instances.Sketch`` into ``desc``; everything that must outlive the call goes to ``keep``."""
-    nh = len(sk.holes)
-    holes = (xp_hole_desc * nh)()
-    keep.append(holes)
-    for i, h in enumerate(sk.holes):
-        d = holes[i]
-        d.start_nt, d.max_size = h.start_nt, h.max_size
-        ctx = _code(h.ctx); keep.append(ctx)
-        d.ctx_len, d.ctx = len(h.ctx), ctx
-        table = (spec_tables or {}).get(i, h.spec_table)
-        if table is not None:
-            if isinstance(table, np.ndarray):
-                table = np.ascontiguousarray(table, dtype=np.int64)
-            d.spec_kind = 1
-            d.spec_table, d.spec_table_on_device, k = _ptr_of(table)
-            keep.append(k)
-        else:
-            se = _code(h.spec_expr); keep.append(se)
-            d.spec_kind, d.spec_len, d.spec_expr = 0, len(h.spec_expr), se
-    co = coords if coords is not None else sk.coords
-    if co is not None:
-        if isinstance(co, np.ndarray):
-            co = np.ascontiguousarray(co, dtype=np.int32)
-        desc.domain_kind = 1
-        desc.n_points = int(co.shape[0])
-        desc.coords, desc.coords_on_device, k = _ptr_of(co)
-        keep.append(k)
-    desc.n_holes, desc.holes = nh, holes
-    return nh
+def _contiguous(a, itemsize: int) -> np.ndarray:
+    """A host array as the descriptors take it: C-contiguous int32 (coordinates) or int64 (spec values)."""
+    return np.ascontiguousarray(a, dtype=np.int32 if itemsize == 4 else np.int64)
 
 
 def xp_sketch_load(gr: Grammar, sk, coords=None, spec_tables: Optional[Dict[int, object]] = None) -> LoadedSketch:
@@ -320,25 +289,19 @@ def xp_sketch_load(gr: Grammar, sk, coords=None, spec_tables: Optional[Dict[int,
     sketch's host tables with contiguous torch CUDA tensors (int32 [n, n_vars] / int64 [n]),
     which the library then uses in place."""
     lib = load()
-    keep = []
-    desc = xp_sketch_desc()
-    nh = _fill_sketch_desc(desc, sk, coords, spec_tables, keep)
+    address, owner, nhs, tensors = _m.sketches((sk,), _contiguous, coords, spec_tables)
     out = C.c_void_p()
-    _check(lib.xp_sketch_load(gr.handle, C.byref(desc), C.byref(out)))
-    return LoadedSketch(out.value, gr, nh, [k for k in keep if not isinstance(k, C.Array)])
+    _check(lib.xp_sketch_load(gr.handle, xp_sketch_desc.from_address(address), C.byref(out)))
+    del owner                                   # (the descriptors are borrowed for the call; device tensors are used in place)
+    return LoadedSketch(out.value, gr, nhs[0], tensors[0])
 
 
 def marshal_sketches(sks: Sequence):
     """The C descriptors (``xp_sketch_desc`` array and what it points to, all in host memory) of a
     list of sketches, for callers that load the same descriptions more than once."""
-    n = len(sks)
-    descs = (xp_sketch_desc * n)()
-    keeps, nhs = [], []
-    for i, sk in enumerate(sks):
-        keep = []
-        nhs.append(_fill_sketch_desc(descs[i], sk, None, None, keep))
-        keeps.append(keep)
-    return descs, nhs, keeps
+    load()
+    address, owner, nhs, tensors = _m.sketches(sks, _contiguous, None, None)
+    return (xp_sketch_desc * len(sks)).from_address(address), nhs, (owner, tensors)
 
 
 def xp_sketch_load_batch(grs: Sequence[Grammar], sks: Sequence, marshalled=None) -> List[LoadedSketch]:
@@ -347,11 +310,12 @@ def xp_sketch_load_batch(grs: Sequence[Grammar], sks: Sequence, marshalled=None)
     lib = load()
     n = len(sks)
     assert len(grs) == n and n > 0
-    descs, nhs, keeps = marshalled if marshalled is not None else marshal_sketches(sks)
+    descs, nhs, keep = marshalled if marshalled is not None else marshal_sketches(sks)
     handles = (C.c_void_p * n)(*[g.handle for g in grs])
     outs = (C.c_void_p * n)()
     _check(lib.xp_sketch_load_batch(handles, descs, n, outs))
-    return [LoadedSketch(outs[i], grs[i], nhs[i], [k for k in keeps[i] if not isinstance(k, C.Array)]) for i in range(n)]
+    tensors = keep[1]
+    return [LoadedSketch(h, g, nh, t) for h, g, nh, t in zip(outs, grs, nhs, tensors)]
 
 
 @dataclass
@@ -379,14 +343,15 @@ class HoleResult:
 def xp_result_get(result_handle: int, hole: int) -> HoleResult:
     v = xp_result_view()
     _check(load().xp_result_get(result_handle, hole, C.byref(v)))
-    K = v.max_size
-    return HoleResult(bool(v.solved), [int(v.cand_count[k]) for k in range(K + 1)],
-                      [int(v.match_count[k]) for k in range(K + 1)], int(v.least_size), int(v.least_rank),
-                      v.least_text.decode() if v.solved else "",
-                      [(v.least_code[i].kind, v.least_code[i].arg, v.least_code[i].value) for i in range(v.least_len)],
-                      int(v.evals_executed), int(v.filter_survivors), int(v.probe_survivors),
-                      int(v.nominal_ops), float(v.kernel_ms), float(v.total_ms), int(v.n_launches),
-                      int(v.filter_tests), int(v.candidates_skipped), int(v.h2d_bytes), int(v.d2h_bytes))
+    return HoleResult(*_m.hole_result(C.addressof(v)))
+
+
+def _opts_of(kw):
+    """(options pointer or None for the defaults, what has to stay alive)."""
+    if not kw:
+        return None, None
+    o, keep = _opts(**kw)
+    return C.byref(o), (o, keep)
 
 
 def _opts(size_min=0, size_max=0, rank_ranges=None, stream=None, workspace=None, flags=0, cancel=None, timeout_ms=0):
@@ -411,18 +376,18 @@ def _opts(size_min=0, size_max=0, rank_ranges=None, stream=None, workspace=None,
 
 
 def xp_workspace_bytes(sketches: Sequence[LoadedSketch], **kw) -> int:
-    o, _keep = _opts(**kw)
+    o, _keep = _opts_of(kw)
     arr = (C.c_void_p * len(sketches))(*[s.handle for s in sketches])
-    return int(load().xp_workspace_bytes(arr, len(sketches), C.byref(o)))
+    return int(load().xp_workspace_bytes(arr, len(sketches), o))
 
 
 def xp_repair(sketch: LoadedSketch, **kw) -> List[HoleResult]:
     """Keyword options: size_min, size_max, rank_ranges=[(hole, size, begin, end)], stream (raw
     cudaStream_t), workspace (torch CUDA uint8 tensor), flags, cancel (a ``ctypes.c_int32`` polled
     between launches), timeout_ms.  Returns one result per hole."""
-    o, _keep = _opts(**kw)
+    o, _keep = _opts_of(kw)
     out = C.c_void_p()
-    _check(load().xp_repair(sketch.handle, C.byref(o), C.byref(out)))
+    _check(load().xp_repair(sketch.handle, o, C.byref(out)))
     try:
         return [xp_result_get(out.value, h) for h in range(sketch.n_holes)]
     finally:
@@ -434,12 +399,12 @@ def xp_repair_batch(sketches: Sequence[LoadedSketch], packed: bool = False, **kw
     where ``summaries`` is ONE ctypes array of ``xp_hole_summary`` (the holes of sketch 0, then of sketch 1,
     ...) filled by a single ``xp_result_pack`` call, and ``view`` is the full ``HoleResult`` of the first
     hole (timings, counters and byte counts of the whole call)."""
-    o, _keep = _opts(**kw)
+    o, _keep = _opts_of(kw)
     lib = load()
     n = len(sketches)
     arr = (C.c_void_p * n)(*[s.handle for s in sketches])
     outs = (C.c_void_p * n)()
-    _check(lib.xp_repair_batch(arr, n, C.byref(o), outs))
+    _check(lib.xp_repair_batch(arr, n, o, outs))
     try:
         if packed:
             total = sum(s.n_holes for s in sketches)
@@ -472,9 +437,9 @@ def xp_repair_static(sketch: LoadedSketch, **kw) -> List[xp_hole_summary]:
     callers that may not allocate device memory at call time.  The summaries are ctypes
     structures owned by the caller (cand_count, match_count, solved, least_size, least_rank,
     least_text).  Keyword options as for ``xp_repair`` (``workspace`` is ignored)."""
-    o, _keep = _opts(**kw)
+    o, _keep = _opts_of(kw)
     out = (xp_hole_summary * sketch.n_holes)()
-    _check(load().xp_repair_static(sketch.handle, C.byref(o), out, sketch.n_holes))
+    _check(load().xp_repair_static(sketch.handle, o, out, sketch.n_holes))
     return list(out)
 
 

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <chrono>
 #include <cstdio>
@@ -124,42 +125,12 @@ void pool_release(void* ptr, size_t bytes, int device) {
 struct xp_sketch;
 static xp_status check_device(const xp_sketch* const* sk, size_t n);
 
-// Page-locked host memory for the staged copies of a load (what goes to the device and what comes
-// back), kept by the library from load to load: copies from and to page-locked memory are queued
-// without the extra pass through the driver's own staging buffer that a copy from ordinary memory
-// takes, which for a batch of thousands of sketches was most of the load's time.  One load uses it
-// at a time (a concurrent load falls back to ordinary memory).
 namespace {
-constexpr size_t kPinnedChunk = 64ull << 20, kPinnedMost = 1ull << 30;
-struct PinnedArena {
-    std::mutex mu;
-    std::vector<char*> chunks;
-    size_t chunk = 0, used = 0;
-    std::mutex take_mu;               // (the threads of one batch load share the arena)
-    void reset() { chunk = 0; used = 0; }
-    char* take(size_t bytes) {
-        std::lock_guard<std::mutex> lock(take_mu);
-        const size_t need = (bytes + 255) & ~(size_t)255;
-        if (need > kPinnedChunk) return nullptr;
-        if (chunk < chunks.size() && used + need > kPinnedChunk) { ++chunk; used = 0; }
-        if (chunk >= chunks.size()) {
-            if ((chunks.size() + 1) * kPinnedChunk > kPinnedMost) return nullptr;
-            void* p = nullptr;
-            if (cudaHostAlloc(&p, kPinnedChunk, cudaHostAllocDefault) != cudaSuccess) { (void)cudaGetLastError(); return nullptr; }
-            chunks.push_back((char*)p);
-        }
-        char* out = chunks[chunk] + used;
-        used += need;
-        return out;
-    }
-};
-PinnedArena g_pinned;
-
 // Page-locked blocks for what a search sends and reads back, and pairs of events that time it: kept from call to
 // call in lists that any thread may use (a copy from ordinary memory goes through the driver's staging buffer and
 // makes the host wait; creating a pair of events takes longer than recording it).  A block that would take the list past
 // kStageKeep bytes is freed when it comes back.
-constexpr size_t kStageKeep = 64ull << 20, kStageLeast = 16ull << 10;
+constexpr size_t kStageKeep = 512ull << 20, kStageLeast = 16ull << 10;
 struct StagePool {
     std::mutex mu;
     std::multimap<size_t, char*> blocks;
@@ -247,7 +218,6 @@ struct xp_grammar {
     u64 cnt[kMaxNt][kMaxSize + 1] = {{0}};
     int ok_size = kMaxSize;          // counts are exact (< 2^63) up to this size
     // device copy, made on first use
-    std::mutex mu;
     GrammarDev* d_g = nullptr;       // one block: header, leaves, binary productions
     size_t d_bytes = 0;
     int d_device = 0;
@@ -410,20 +380,22 @@ extern "C" xp_status xp_grammar_unrank(const xp_grammar* g, int32_t nt, int32_t 
     return XP_OK;
 }
 
-// (staging: page-locked memory of the load at hand, or null; with it the copy is queued on the
-// load's stream like the sketch's own copies and nobody waits for it here)
-static xp_status grammar_to_device(xp_grammar* g, size_t* copied, PinnedArena* staging) {
-    *copied = 0;
-    std::lock_guard<std::mutex> lock(g->mu);
-    if (g->d_g) {
-        // the device copy was made on the device that was current at the first load and serves that device only
-        int dev = -1;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev != g->d_device)
-            return fail(XP_ERR_INVALID_ARG, "the grammar's tables live on device " + std::to_string(g->d_device) +
-                        ", the current device is " + std::to_string(dev) + ": use one grammar handle per device");
-        return XP_OK;
-    }
-    GrammarDev h;
+// Layout of a grammar's tables in one device block: header | leaves | binary productions | constants.
+struct GrammarLayout { size_t leaves, bins, consts, total; };
+static GrammarLayout grammar_layout(const xp_grammar* g) {
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    GrammarLayout l;
+    l.leaves = al(sizeof(GrammarDev));
+    l.bins = l.leaves + al(sizeof(LeafDev) * g->leaves.size());
+    l.consts = l.bins + al(sizeof(BinDev) * g->bins.size());
+    l.total = l.consts + al(sizeof(ConstDev) * g->consts.size());
+    return l;
+}
+
+// The tables as they go to the device block at g->d_g.
+static void grammar_image(const xp_grammar* g, char* out) {
+    const GrammarLayout l = grammar_layout(g);
+    GrammarDev& h = *(GrammarDev*)out;
     memset(&h, 0, sizeof(h));
     h.n_vars = g->n_vars; h.n_nt = g->n_nt;
     h.n_leaves = (int)g->leaves.size(); h.n_bins = (int)g->bins.size();
@@ -432,32 +404,31 @@ static xp_status grammar_to_device(xp_grammar* g, size_t* copied, PinnedArena* s
     memcpy(h.cnt, g->cnt, sizeof(h.cnt));
     memcpy(h.const_begin, g->const_begin, sizeof(h.const_begin));
     memcpy(h.var_begin, g->var_begin, sizeof(h.var_begin));
-    // one device block and one copy: header | leaves | binary productions | constants
-    const size_t off_leaves = (sizeof(GrammarDev) + 255) & ~(size_t)255;
-    const size_t off_bins = off_leaves + ((sizeof(LeafDev) * (g->leaves.size() + 1) + 255) & ~(size_t)255);
-    const size_t off_consts = off_bins + ((sizeof(BinDev) * (g->bins.size() + 1) + 255) & ~(size_t)255);
-    const size_t total = off_consts + sizeof(ConstDev) * (g->consts.size() + 1);
+    const char* block = (const char*)g->d_g;
+    h.leaves = (const LeafDev*)(block + l.leaves);
+    h.bins = (const BinDev*)(block + l.bins);
+    h.consts = (const ConstDev*)(block + l.consts);
+    if (!g->leaves.empty()) memcpy(out + l.leaves, g->leaves.data(), sizeof(LeafDev) * g->leaves.size());
+    if (!g->bins.empty()) memcpy(out + l.bins, g->bins.data(), sizeof(BinDev) * g->bins.size());
+    if (!g->consts.empty()) memcpy(out + l.consts, g->consts.data(), sizeof(ConstDev) * g->consts.size());
+}
+
+// Device memory for a grammar's tables, on first use; *fresh: the caller has to send the image.
+// (Loads hold g_load_mu: nobody else sees a block whose image has not been queued.)
+static xp_status grammar_block(xp_grammar* g, bool* fresh) {
+    *fresh = false;
+    if (g->d_g) {
+        // the device copy was made on the device that was current at the first load and serves that device only
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev != g->d_device)
+            return fail(XP_ERR_INVALID_ARG, "the grammar's tables live on device " + std::to_string(g->d_device) +
+                        ", the current device is " + std::to_string(dev) + ": use one grammar handle per device");
+        return XP_OK;
+    }
     char* block = nullptr;
-    size_t granted = 0;
-    XP_CUDA(pool_alloc((void**)&block, total, &g->d_device, &granted));
-    g->d_bytes = granted;
-    h.leaves = (const LeafDev*)(block + off_leaves);
-    h.bins = (const BinDev*)(block + off_bins);
-    h.consts = (const ConstDev*)(block + off_consts);
-    std::vector<char> stage_own;
-    char* stage = staging ? staging->take(total) : nullptr;
-    const bool queued = stage != nullptr;
-    if (!stage) { stage_own.resize(total); stage = stage_own.data(); }
-    memset(stage, 0, total);
-    memcpy(stage, &h, sizeof(h));
-    if (!g->leaves.empty()) memcpy(stage + off_leaves, g->leaves.data(), sizeof(LeafDev) * g->leaves.size());
-    if (!g->bins.empty()) memcpy(stage + off_bins, g->bins.data(), sizeof(BinDev) * g->bins.size());
-    if (!g->consts.empty()) memcpy(stage + off_consts, g->consts.data(), sizeof(ConstDev) * g->consts.size());
-    cudaError_t e = queued ? cudaMemcpyAsync(block, stage, total, cudaMemcpyHostToDevice, nullptr)
-                           : cudaMemcpy(block, stage, total, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) { pool_release(block, g->d_bytes, g->d_device); return fail(XP_ERR_CUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e)); }
+    XP_CUDA(pool_alloc((void**)&block, grammar_layout(g).total, &g->d_device, &g->d_bytes));
     g->d_g = (GrammarDev*)block;
-    *copied = total;
+    *fresh = true;
     return XP_OK;
 }
 
@@ -505,6 +476,16 @@ struct xp_sketch {
     mutable std::vector<u64> plan_ops;
     mutable u64 plan_tickets = 0;
 };
+
+// What the load's kernels settled for a hole.
+static void hole_decided(HoleHost* h, const LoadOut& o) {
+    // the filter applies where the context at probe 0 is affine in the hole, or a comparison
+    h->filter_ok = o.filter_ok != 0 && o.tab_probes > 0;
+    h->compares = o.filter_ok != 0 && o.aff_ok == 0;
+    h->exact = o.aff_ok != 0 && o.join_on == 0;
+    h->second = o.second != 0;
+    if (o.spec_bad) h->never = true;                      // the spec is undefined at some point
+}
 
 // Checks a postfix expression; returns false when malformed or too deep.
 static bool check_code(const xp_instr* code, int n, int n_vars, bool hole_allowed) {
@@ -559,20 +540,20 @@ static u64 table_entries(const xp_grammar* g, int max_size, u64 (*off)[kMaxSize 
 // load's kernels have run.
 struct LoadState {
     xp_sketch* s = nullptr;
+    const xp_sketch_desc* d = nullptr;
     std::vector<HoleDev> hh;
-    std::vector<char> back_own;      // holes and flags as the kernels left them (ordinary memory, when no page-locked
-    char* back = nullptr;            //   memory could be had); back points at whichever holds them
-    size_t back_bytes = 0;
-    PinnedArena* pinned = nullptr;   // page-locked staging memory of this load, or null
-    size_t off_holes = 0;
-    i64 table_points = 0;            // rows of a table domain (0 for a box)
-    u64 entries_at[kMaxSize + 1] = {0};      // subtree-table entries per size (all nonterminals)
-    int size_cap = 0, probes_cap = 0;        // over the holes
+    std::vector<size_t> off_spec;            // per hole: its spec values in the device block (0: none there)
+    size_t off_coords = 0, head = 0;         // [0, head) of the block is staged on the host
+    bool copy_coords = false, stage = false, stage_box = false;
+    bool grammar_fresh = false;              // this sketch's load sends its grammar's tables
+    size_t grammar_bytes = 0;
+    size_t stage_at = 0;                     // where its part of the staged copy starts (head, then the grammar's tables)
+    size_t piece = 0;
 };
+constexpr size_t kPackMax = 256u << 10;      // host tables up to this size travel in the staged copy
+static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// First half of a load: checks the description, lays out and allocates the sketch's device
-// block, queues the copies of what the host provides and, for a box, the kernels that stage its
-// points and spec values.  Nothing here waits for the device.
+// First part of a load: checks the description, lays out and allocates the sketch's device block.
 static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadState* L) {
     if (!gc || !d) return fail(XP_ERR_INVALID_ARG, "xp_sketch_load: null argument");
     xp_grammar* g = const_cast<xp_grammar*>(gc);
@@ -603,47 +584,39 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             if (n_points > 0 && !hd.spec_table) return fail(XP_ERR_SKETCH, "spec table is null");
         } else return fail(XP_ERR_SKETCH, "bad spec_kind");
     }
-    int ndev = 0;
-    if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) return fail(XP_ERR_CUDA, "no CUDA device is usable");
-    size_t grammar_bytes = 0;
-    xp_status st = grammar_to_device(g, &grammar_bytes, L->pinned);
+    const xp_status st = grammar_block(g, &L->grammar_fresh);
     if (st != XP_OK) return st;
+    if (L->grammar_fresh) L->grammar_bytes = grammar_layout(g).total;
 
     xp_sketch* s = new (std::nothrow) xp_sketch;
     if (!s) return fail(XP_ERR_NOMEM, "out of host memory");
     s->g = g; s->n_holes = d->n_holes; s->n_points = n_points;
-#define XP_CUDA_S(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { xp_sketch_destroy(s); \
-        return fail(e_ == cudaErrorMemoryAllocation ? XP_ERR_NOMEM : XP_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); } } while (0)
-
     // One device block for the whole sketch, laid out here before anything runs: first what the
-    // host provides (sketch, holes, flags, small tables: one staged copy), then what the load's
-    // kernels produce (staged points and specs, subtree tables).  The host then looks at the
-    // device once more, at the end, to read back what the kernels decided.
+    // host provides (sketch, holes, small tables: part of the load's staged copy), then what the load's
+    // kernels produce (staged points and specs, subtree tables).
     const int nh = d->n_holes;
     const size_t np = (size_t)n_points, row = (size_t)(nv ? nv : 1);
-    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    constexpr size_t kPackMax = 256u << 10;              // host tables up to this size travel in the staged copy
     bool i32_ok = true;
     for (int v = 0; v < nv; ++v) i32_ok = i32_ok && g->lo[v] >= INT32_MIN && g->hi[v] <= (i64)INT32_MAX + 1;
-    const bool stage = n_points > 0 && (u64)n_points <= kStageMaxPoints;
-    const bool stage_box = d->domain_kind == XP_DOMAIN_BOX && stage && i32_ok && nv > 0;
-    const bool copy_coords = d->domain_kind == XP_DOMAIN_TABLE && np > 0 && !d->coords_on_device;
+    L->stage = n_points > 0 && (u64)n_points <= kStageMaxPoints;
+    L->stage_box = d->domain_kind == XP_DOMAIN_BOX && L->stage && i32_ok && nv > 0;
+    L->copy_coords = d->domain_kind == XP_DOMAIN_TABLE && np > 0 && !d->coords_on_device;
     const size_t coords_bytes = sizeof(i32) * np * row, spec_bytes = sizeof(i64) * np;
     size_t off = 0;
-    const size_t off_sketch = off;  off += al(sizeof(SketchDev));
-    const size_t off_holes = off;   off += al(sizeof(HoleDev) * nh + sizeof(u32) * nh);       // holes, then one flag each
-    const size_t off_bad = off_holes + sizeof(HoleDev) * nh;
-    size_t off_coords = 0;
-    std::vector<size_t> off_spec(nh, 0), off_tabv(nh, 0), off_tabk(nh, 0), off_tabm(nh, 0), off_pair(nh, 0), off_sets(nh, 0);
-    if (copy_coords && coords_bytes <= kPackMax) { off_coords = off; off += al(coords_bytes); }
+    const size_t off_sketch = off;  off += al256(sizeof(SketchDev));
+    const size_t off_holes = off;   off += al256(sizeof(HoleDev) * nh);
+    L->off_spec.assign(nh, 0);
+    std::vector<size_t>& off_spec = L->off_spec;
+    std::vector<size_t> off_tabv(nh, 0), off_tabk(nh, 0), off_tabm(nh, 0), off_pair(nh, 0), off_sets(nh, 0);
+    if (L->copy_coords && coords_bytes <= kPackMax) { L->off_coords = off; off += al256(coords_bytes); }
     for (int h = 0; h < nh; ++h)
         if (d->holes[h].spec_kind == XP_SPEC_TABLE && np > 0 && !d->holes[h].spec_table_on_device && spec_bytes <= kPackMax) {
-            off_spec[h] = off; off += al(spec_bytes);
+            off_spec[h] = off; off += al256(spec_bytes);
         }
     s->off_kill.assign(nh, 0);
-    for (int h = 0; h < nh; ++h) { s->off_kill[h] = off; off += al((sizeof(i64) + sizeof(u32)) * kKillSlots); }
-    const size_t head = off;                              // [0, head): staged on the host and copied in one piece
-    if ((copy_coords && coords_bytes > kPackMax) || stage_box) { off_coords = off; off += al(coords_bytes); }
+    for (int h = 0; h < nh; ++h) { s->off_kill[h] = off; off += al256((sizeof(i64) + sizeof(u32)) * kKillSlots); }
+    L->head = off;                                        // [0, head): staged on the host
+    if ((L->copy_coords && coords_bytes > kPackMax) || L->stage_box) { L->off_coords = off; off += al256(coords_bytes); }
     std::vector<HoleDev>& hh = L->hh;
     hh.resize(nh);
     for (int h = 0; h < nh; ++h) {
@@ -651,8 +624,8 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
         HoleDev& o = hh[h];
         memset(&o, 0, sizeof(o));
         if (np > 0 && off_spec[h] == 0 &&
-            ((hd.spec_kind == XP_SPEC_TABLE && !hd.spec_table_on_device) || (hd.spec_kind == XP_SPEC_EXPR && stage))) {
-            off_spec[h] = off; off += al(spec_bytes);
+            ((hd.spec_kind == XP_SPEC_TABLE && !hd.spec_table_on_device) || (hd.spec_kind == XP_SPEC_EXPR && L->stage))) {
+            off_spec[h] = off; off += al256(spec_bytes);
         }
         const u64 entries = table_entries(g, hd.max_size, o.tab_off, &o.tab_size_cap);
         u64 probes = kMaxProbe;
@@ -660,12 +633,14 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
         o.tab_total = entries;
         o.tab_probes_cap = entries > 0 ? (i32)probes : 0;
         if (entries > 0) {
-            off_tabv[h] = off; off += al(sizeof(i64) * entries * probes);
-            off_tabk[h] = off; off += al(entries * probes);
-            off_tabm[h] = off; off += al(entries);
-            off_pair[h] = off; off += al(2 * sizeof(i32) * entries);
+            off_tabv[h] = off; off += al256(sizeof(i64) * entries * probes);
+            off_tabk[h] = off; off += al256(entries * probes);
+            off_tabm[h] = off; off += al256(entries);
+            off_pair[h] = off; off += al256(2 * sizeof(i32) * entries);
         }
-        off_sets[h] = off; off += al(sizeof(JoinSet) * (size_t)g->n_nt);
+        off_sets[h] = off; off += al256(sizeof(JoinSet) * (size_t)g->n_nt);
+        if (o.tab_size_cap > s->tab_size_cap) s->tab_size_cap = o.tab_size_cap;
+        if (o.tab_probes_cap > s->tab_probes_cap) s->tab_probes_cap = o.tab_probes_cap;
     }
     size_t arena_granted = 0;
     if (pool_alloc((void**)&s->arena, off, &s->arena_device, &arena_granted) != cudaSuccess) {
@@ -678,19 +653,68 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     char* base = s->arena;
     s->d_s = (SketchDev*)(base + off_sketch);
     s->d_holes = (HoleDev*)(base + off_holes);
+    s->off_holes = off_holes;
+    for (int h = 0; h < nh; ++h) {
+        const xp_hole_desc& hd = d->holes[h];
+        HoleDev& o = hh[h];
+        u64 c = 0;
+        for (int k = 1; k <= hd.max_size; ++k) c += g->cnt[hd.start_nt][k];
+        o.small_search = c <= 100000000ull ? 1 : 0;
+        o.start_nt = hd.start_nt; o.max_size = hd.max_size; o.ctx_len = hd.ctx_len;
+        if (hd.ctx_len) memcpy(o.ctx, hd.ctx, sizeof(xp_instr) * hd.ctx_len);
+        if (hd.spec_kind == XP_SPEC_EXPR) {
+            o.spec_len = hd.spec_len;
+            memcpy(o.spec, hd.spec_expr, sizeof(xp_instr) * hd.spec_len);
+            if (off_spec[h]) o.spec_table = (const i64*)(base + off_spec[h]);       // staged by the load, before anything reads it
+        } else if (np > 0) {
+            o.spec_table = hd.spec_table_on_device ? (const i64*)hd.spec_table : (const i64*)(base + off_spec[h]);
+        }
+        if (o.tab_total > 0) {
+            o.tab_val = (i64*)(base + off_tabv[h]);
+            o.tab_ok = (unsigned char*)(base + off_tabk[h]);
+            o.tab_vars = (unsigned char*)(base + off_tabm[h]);
+            o.tab_pair = (i32*)(base + off_pair[h]);
+        }
+        o.join_sets = (JoinSet*)(base + off_sets[h]);
+        // variables the context and the spec mention (a caller's spec table may depend on all)
+        u32 fv = hd.spec_kind == XP_SPEC_EXPR ? 0u : 0xffffffffu;
+        for (int i = 0; i < hd.ctx_len; ++i) if (hd.ctx[i].kind == XP_I_VAR) fv |= 1u << hd.ctx[i].arg;
+        if (hd.spec_kind == XP_SPEC_EXPR)
+            for (int i = 0; i < hd.spec_len; ++i) if (hd.spec_expr[i].kind == XP_I_VAR) fv |= 1u << hd.spec_expr[i].arg;
+        o.fixed_vars = fv;
+        o.kill_pid = (i64*)(base + s->off_kill[h]);
+        o.kill_cnt = (u32*)(base + s->off_kill[h] + sizeof(i64) * kKillSlots);
+        HoleHost ho;
+        ho.start_nt = hd.start_nt; ho.max_size = hd.max_size;
+        s->holes.push_back(ho);
+    }
+    for (int k = 1; k <= s->tab_size_cap; ++k)
+        for (int nt = 0; nt < g->n_nt; ++nt) s->entries_at[k] += g->cnt[nt][k];
+    L->s = s;
+    L->d = d;
+    return XP_OK;
+}
 
-    SketchDev hs;
+// The sketch's record.
+static void sketch_image(const LoadState* L, SketchDev* out) {
+    const xp_sketch* s = L->s;
+    const xp_grammar* g = s->g;
+    const xp_sketch_desc* d = L->d;
+    const int nv = g->n_vars;
+    const i64 n_points = s->n_points;
+    char* base = s->arena;
+    SketchDev& hs = *out;
     memset(&hs, 0, sizeof(hs));
-    hs.g = g->d_g; hs.n_vars = nv; hs.n_holes = nh; hs.domain_kind = d->domain_kind; hs.n_points = n_points;
+    hs.g = g->d_g; hs.n_vars = nv; hs.n_holes = s->n_holes; hs.domain_kind = d->domain_kind; hs.n_points = n_points;
     hs.holes = s->d_holes;
     for (int v = 0; v < nv; ++v) {
         hs.lo[v] = g->lo[v]; hs.ext[v] = g->hi[v] - g->lo[v];
-        const bool table = d->domain_kind == XP_DOMAIN_TABLE;      // a table's bounds are reduced over its rows below
+        const bool table = d->domain_kind == XP_DOMAIN_TABLE;      // a table's bounds are reduced over its rows by the load
         hs.vmin[v] = table ? LLONG_MAX : g->lo[v];
         hs.vmax[v] = table ? LLONG_MIN : g->hi[v] - 1;
     }
-    if (d->domain_kind == XP_DOMAIN_TABLE && np > 0) hs.coords = d->coords_on_device ? d->coords : (const i32*)(base + off_coords);
-    if (stage_box) { hs.coords = (const i32*)(base + off_coords); hs.project = 1; }
+    if (d->domain_kind == XP_DOMAIN_TABLE && n_points > 0) hs.coords = d->coords_on_device ? d->coords : (const i32*)(base + L->off_coords);
+    if (L->stage_box) { hs.coords = (const i32*)(base + L->off_coords); hs.project = 1; }
     // Sample points the probes are chosen from: box corners first (they expose bound and
     // padding mistakes), then ids spread over the domain by a fixed hash.
     int ns = 0;
@@ -719,217 +743,216 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
         }
     }
     hs.n_samples = ns;
-    for (int h = 0; h < nh; ++h) {
-        u64 c = 0;
-        for (int k = 1; k <= d->holes[h].max_size; ++k) c += g->cnt[d->holes[h].start_nt][k];
-        hh[h].small_search = c <= 100000000ull ? 1 : 0;
-    }
+}
 
-    for (int h = 0; h < nh; ++h) {
-        const xp_hole_desc& hd = d->holes[h];
-        HoleDev& o = hh[h];
-        o.start_nt = hd.start_nt; o.max_size = hd.max_size; o.ctx_len = hd.ctx_len;
-        if (hd.ctx_len) memcpy(o.ctx, hd.ctx, sizeof(xp_instr) * hd.ctx_len);
-        if (hd.spec_kind == XP_SPEC_EXPR) {
-            o.spec_len = hd.spec_len;
-            memcpy(o.spec, hd.spec_expr, sizeof(xp_instr) * hd.spec_len);
-            if (off_spec[h]) o.spec_table = (const i64*)(base + off_spec[h]);       // staged below, before anything reads it
-        } else if (np > 0) {
-            o.spec_table = hd.spec_table_on_device ? (const i64*)hd.spec_table : (const i64*)(base + off_spec[h]);
-        }
-        if (o.tab_total > 0) {
-            o.tab_val = (i64*)(base + off_tabv[h]);
-            o.tab_ok = (unsigned char*)(base + off_tabk[h]);
-            o.tab_vars = (unsigned char*)(base + off_tabm[h]);
-            o.tab_pair = (i32*)(base + off_pair[h]);
-        }
-        o.join_sets = (JoinSet*)(base + off_sets[h]);
-        // variables the context and the spec mention (a caller's spec table may depend on all)
-        u32 fv = hd.spec_kind == XP_SPEC_EXPR ? 0u : 0xffffffffu;
-        for (int i = 0; i < hd.ctx_len; ++i) if (hd.ctx[i].kind == XP_I_VAR) fv |= 1u << hd.ctx[i].arg;
-        if (hd.spec_kind == XP_SPEC_EXPR)
-            for (int i = 0; i < hd.spec_len; ++i) if (hd.spec_expr[i].kind == XP_I_VAR) fv |= 1u << hd.spec_expr[i].arg;
-        o.fixed_vars = fv;
-        o.kill_pid = (i64*)(base + s->off_kill[h]);
-        o.kill_cnt = (u32*)(base + s->off_kill[h] + sizeof(i64) * kKillSlots);
-        HoleHost ho;
-        ho.start_nt = hd.start_nt; ho.max_size = hd.max_size;
-        s->holes.push_back(ho);
-    }
-
-    // the staged copy, then the tables too large for it
-    std::vector<char> stg_own;
-    char* stg = L->pinned ? L->pinned->take(head) : nullptr;
-    if (!stg) { stg_own.resize(head); stg = stg_own.data(); }
-    memset(stg, 0, head);
-    memcpy(&stg[off_sketch], &hs, sizeof(hs));
-    memcpy(&stg[off_holes], hh.data(), sizeof(HoleDev) * nh);
-    if (copy_coords && coords_bytes <= kPackMax) memcpy(&stg[off_coords], d->coords, coords_bytes);
+// Second part: the sketch's share of the staged copy (its head, then its grammar's tables when they are new).
+static void load_fill(const LoadState* L, char* stg) {
+    const xp_sketch* s = L->s;
+    const xp_sketch_desc* d = L->d;
+    const int nh = s->n_holes;
+    const size_t np = (size_t)s->n_points, row = (size_t)(s->g->n_vars ? s->g->n_vars : 1);
+    const size_t coords_bytes = sizeof(i32) * np * row, spec_bytes = sizeof(i64) * np;
+    sketch_image(L, (SketchDev*)stg);
+    memcpy(stg + s->off_holes, L->hh.data(), sizeof(HoleDev) * nh);
+    if (L->copy_coords && coords_bytes <= kPackMax) memcpy(stg + L->off_coords, d->coords, coords_bytes);
     for (int h = 0; h < nh; ++h) {
         const xp_hole_desc& hd = d->holes[h];
         if (hd.spec_kind == XP_SPEC_TABLE && np > 0 && !hd.spec_table_on_device && spec_bytes <= kPackMax)
-            memcpy(&stg[off_spec[h]], hd.spec_table, spec_bytes);
-        memset(&stg[s->off_kill[h]], 0xff, sizeof(i64) * kKillSlots);           // no point noted yet (ids -1, counts 0)
+            memcpy(stg + L->off_spec[h], hd.spec_table, spec_bytes);
+        memset(stg + s->off_kill[h], 0xff, sizeof(i64) * kKillSlots);           // no point noted yet (ids -1, counts 0)
+        memset(stg + s->off_kill[h] + sizeof(i64) * kKillSlots, 0, sizeof(u32) * kKillSlots);
     }
-    s->load_h2d = grammar_bytes + head;
-    XP_CUDA_S(cudaMemcpyAsync(base, stg, head, cudaMemcpyHostToDevice, nullptr));
-    if (copy_coords && coords_bytes > kPackMax) {
-        XP_CUDA_S(cudaMemcpyAsync(base + off_coords, d->coords, coords_bytes, cudaMemcpyHostToDevice, nullptr));
-        s->load_h2d += coords_bytes;
-    }
-    for (int h = 0; h < nh; ++h) {
-        const xp_hole_desc& hd = d->holes[h];
-        if (hd.spec_kind == XP_SPEC_TABLE && np > 0 && !hd.spec_table_on_device && spec_bytes > kPackMax) {
-            XP_CUDA_S(cudaMemcpyAsync(base + off_spec[h], hd.spec_table, spec_bytes, cudaMemcpyHostToDevice, nullptr));
-            s->load_h2d += spec_bytes;
-        }
-    }
-    // The load's kernels, in stream order: points of a box and values of spec expressions (so that
-    // the whole-domain check, and the probe choice, read tables for every kind of domain); bounds of a
-    // table's coordinates; the probe choice; the subtree tables, bottom-up, for as many sizes and
-    // probes as there can be (launches beyond what the probe choice settled on return at once).
-    if (stage_box) XP_CUDA_S(launch_stage_points(s->d_s, n_points, (i32*)(base + off_coords), nullptr));
-    if (stage)
-        for (int h = 0; h < nh; ++h)
-            if (hh[h].spec_len != 0)
-                XP_CUDA_S(launch_stage_spec(s->d_s, h, n_points, (i64*)(base + off_spec[h]), (u32*)(base + off_bad) + h, nullptr));
-    L->s = s;
-    L->off_holes = off_holes;
-    s->off_holes = off_holes;
-    L->table_points = d->domain_kind == XP_DOMAIN_TABLE ? n_points : 0;
-    for (int h = 0; h < nh; ++h) {
-        if (hh[h].tab_size_cap > L->size_cap) L->size_cap = hh[h].tab_size_cap;
-        if (hh[h].tab_probes_cap > L->probes_cap) L->probes_cap = hh[h].tab_probes_cap;
-    }
-    for (int k = 1; k <= kMaxSize; ++k)
-        for (int nt = 0; nt < g->n_nt; ++nt) L->entries_at[k] += g->cnt[nt][k];
-    s->tab_size_cap = L->size_cap; s->tab_probes_cap = L->probes_cap;
-    memcpy(s->entries_at, L->entries_at, sizeof(s->entries_at));
-#undef XP_CUDA_S
-    return XP_OK;
+    if (L->grammar_fresh) grammar_image(s->g, stg + L->head);
 }
+
+// One load at a time: all of them work on the default stream anyway, and a grammar's tables are sent by the first
+// load that needs them.
+static std::mutex g_load_mu;
 
 extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, const xp_sketch_desc* descs, size_t n,
                                           xp_sketch** outs) {
     if (!grammars || !descs || !outs || n == 0) return fail(XP_ERR_INVALID_ARG, "xp_sketch_load_batch: null argument");
     for (size_t i = 0; i < n; ++i) outs[i] = nullptr;
+    std::lock_guard<std::mutex> one(g_load_mu);
     std::vector<LoadState> st(n);
-    std::unique_lock<std::mutex> pin(g_pinned.mu, std::try_to_lock);
-    if (pin.owns_lock()) {
-        g_pinned.reset();
-        for (size_t i = 0; i < n; ++i) st[i].pinned = &g_pinned;
-    }
-    char* jobs_dev = nullptr;
-    size_t jobs_bytes = 0;
-    int jobs_device = 0;
+    char* dev_block = nullptr;
+    size_t dev_bytes = 0;
+    int dev_device = 0;
+    bool sent = false;
     auto undo = [&]() {
         cudaStreamSynchronize(nullptr);                   // nothing may still be writing into the blocks
-        for (size_t i = 0; i < n; ++i) if (st[i].s) xp_sketch_destroy(st[i].s);
-        pool_release(jobs_dev, jobs_bytes, jobs_device);
-    };
-    size_t n_jobs = 0;
-    {
-        // The host part of a load (checks, layout, staging of the tables, queueing of the copies) is
-        // independent from sketch to sketch: large batches spread it over a few threads, each with
-        // the caller's device current.  Everything is queued on the same stream; the batch's kernels
-        // follow once the threads are done.
-        std::vector<xp_status> status(n, XP_OK);
-        std::vector<std::string> message(n);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        unsigned hw = std::thread::hardware_concurrency();
-        size_t n_threads = n / 128;
-        if (n_threads > 8) n_threads = 8;
-        if (hw > 0 && n_threads > hw) n_threads = hw;
-        auto work = [&](size_t t, size_t step) {
-            if (step > 1) cudaSetDevice(dev);
-            for (size_t i = t; i < n; i += step) {
-                status[i] = load_begin(grammars[i], &descs[i], &st[i]);
-                if (status[i] != XP_OK) message[i] = g_last_error;
+        for (size_t i = 0; i < n; ++i) {
+            if (st[i].grammar_fresh && !sent) {           // its tables never went out
+                xp_grammar* g = const_cast<xp_grammar*>(grammars[i]);
+                pool_release(g->d_g, g->d_bytes, g->d_device);
+                g->d_g = nullptr;
             }
-        };
-        if (n_threads < 2) work(0, 1);
-        else {
-            std::vector<std::thread> pool;
-            for (size_t t = 0; t < n_threads; ++t) pool.emplace_back(work, t, n_threads);
-            for (std::thread& th : pool) th.join();
+            if (st[i].s) xp_sketch_destroy(st[i].s);
         }
-        for (size_t i = 0; i < n; ++i)
-            if (status[i] != XP_OK) { undo(); return fail(status[i], "sketch " + std::to_string(i) + ": " + message[i]); }
-        for (size_t i = 0; i < n; ++i) n_jobs += (size_t)st[i].s->n_holes;
-    }
+        pool_release(dev_block, dev_bytes, dev_device);
+    };
 #define XP_CUDA_B(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { undo(); \
         return fail(e_ == cudaErrorMemoryAllocation ? XP_ERR_NOMEM : XP_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); } } while (0)
-    // the batch's kernels: one list of sketches, one list of (sketch, hole) jobs
-    const size_t list_bytes = (sizeof(SketchDev*) * n + 255) & ~(size_t)255;
-    std::vector<char> stage(list_bytes + sizeof(LoadJob) * n_jobs, 0);
-    {
-        size_t j = 0;
-        for (size_t i = 0; i < n; ++i) {
-            ((SketchDev**)stage.data())[i] = st[i].s->d_s;
-            for (int h = 0; h < st[i].s->n_holes; ++h, ++j) {
-                LoadJob job;
-                job.s = st[i].s->d_s; job.hole = h; job.pad = 0;
-                memcpy(&stage[list_bytes + sizeof(LoadJob) * j], &job, sizeof(job));
-            }
+    int ndev = 0;
+    // (a description that is wrong is reported as such also where no device can be used)
+    const bool no_device = cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1;
+    for (size_t i = 0; i < n; ++i) {
+        const xp_status e = load_begin(grammars[i], &descs[i], &st[i]);
+        if (e != XP_OK) {
+            const std::string why = no_device && e == XP_ERR_CUDA ? std::string("no CUDA device is usable") : g_last_error;
+            undo();
+            return fail(e, "sketch " + std::to_string(i) + ": " + why);
         }
     }
-    // (the prepare kernels' scratch follows the lists)
-    constexpr size_t kPiece = 32768;
-    const size_t scratch_at = (stage.size() + 255) & ~(size_t)255;
-    XP_CUDA_B(pool_alloc((void**)&jobs_dev, scratch_at + prepare_scratch_bytes((int)(n_jobs < kPiece ? n_jobs : kPiece)), &jobs_device, &jobs_bytes));
-    XP_CUDA_B(cudaMemcpyAsync(jobs_dev, stage.data(), stage.size(), cudaMemcpyHostToDevice, nullptr));
-    SketchDev* const* d_list = (SketchDev* const*)jobs_dev;
-    const LoadJob* d_jobs = (const LoadJob*)(jobs_dev + list_bytes);
-    // In stream order after the copies and the boxes' staging: bounds of the tables' coordinates;
-    // the probe choice; the subtree tables, bottom-up, for as many sizes and probes as there can be
-    // (blocks beyond what the probe choice settled on for their hole return at once).  Grids are
-    // cut into pieces of at most kPiece jobs (a grid dimension holds 65 535).
-    i64 most_points = 0;
-    int size_cap = 0, probes_cap = 0;
-    u64 most_entries[kMaxSize + 1] = {0};
-    for (size_t i = 0; i < n; ++i) {
-        most_points = st[i].table_points > most_points ? st[i].table_points : most_points;
-        size_cap = st[i].size_cap > size_cap ? st[i].size_cap : size_cap;
-        probes_cap = st[i].probes_cap > probes_cap ? st[i].probes_cap : probes_cap;
-        for (int k = 1; k <= st[i].size_cap; ++k) most_entries[k] = st[i].entries_at[k] > most_entries[k] ? st[i].entries_at[k] : most_entries[k];
+    // The staged copy: the job lists, then the sketches' shares, in pieces of at most kPieceBytes that page-locked memory
+    // holds one by one.  The pieces go to one block of device memory, and a kernel puts the shares in their places:
+    // a few large copies instead of two per sketch (a batch of 1024 sketches: 2048 copies, 10 ms of the copy engine's time).
+    constexpr size_t kPieceBytes = 8ull << 20, kJobs = 32768;
+    size_t n_jobs = 0;
+    for (size_t i = 0; i < n; ++i) n_jobs += (size_t)st[i].s->n_holes;
+    std::vector<LoadCopy> copies;
+    copies.reserve(2 * n);
+    for (size_t i = 0; i < n; ++i) copies.push_back(LoadCopy{st[i].s->arena, 0, st[i].head});
+    for (size_t i = 0; i < n; ++i) if (st[i].grammar_fresh) copies.push_back(LoadCopy{(char*)st[i].s->g->d_g, 0, st[i].grammar_bytes});
+    const size_t at_list = 0, at_jobs = at_list + al256(sizeof(SketchDev*) * n), at_copies = at_jobs + al256(sizeof(LoadJob) * n_jobs);
+    const size_t at_shares = at_copies + al256(sizeof(LoadCopy) * copies.size());
+    std::vector<size_t> piece_at;                         // start of each piece; the lists are in the first
+    size_t at = at_shares;
+    piece_at.push_back(0);
+    for (size_t i = 0, c = n; i < n; ++i) {
+        const size_t share = st[i].head + st[i].grammar_bytes;
+        if (at > piece_at.back() && at + share - piece_at.back() > kPieceBytes) piece_at.push_back(at);
+        st[i].stage_at = at; st[i].piece = piece_at.size() - 1;
+        copies[i].src = at;
+        if (st[i].grammar_fresh) copies[c++].src = at + st[i].head;
+        at += share;
     }
-    for (size_t at = 0; at < n; at += kPiece)
-        XP_CUDA_B(launch_coord_bounds(d_list + at, (int)(n - at < kPiece ? n - at : kPiece), most_points, nullptr));
-    for (size_t at = 0; at < n_jobs; at += kPiece)
-        XP_CUDA_B(launch_prepare(d_jobs + at, (int)(n_jobs - at < kPiece ? n_jobs - at : kPiece), jobs_dev + scratch_at, nullptr));
-    for (int k = 1; k <= size_cap; ++k)
-        for (size_t at = 0; at < n_jobs; at += kPiece)
-            XP_CUDA_B(launch_subvalues(d_jobs + at, (int)(n_jobs - at < kPiece ? n_jobs - at : kPiece), k, probes_cap, most_entries[k], nullptr));
-    // what the kernels decided, per hole
-    for (size_t i = 0; i < n; ++i) {
-        const int nh = st[i].s->n_holes;
-        st[i].back_bytes = sizeof(HoleDev) * nh + sizeof(u32) * nh;
-        st[i].back = st[i].pinned ? st[i].pinned->take(st[i].back_bytes) : nullptr;
-        if (!st[i].back) { st[i].back_own.resize(st[i].back_bytes); st[i].back = st[i].back_own.data(); }
-        XP_CUDA_B(cudaMemcpyAsync(st[i].back, st[i].s->arena + st[i].off_holes, st[i].back_bytes, cudaMemcpyDeviceToHost, nullptr));
-        st[i].s->load_d2h = st[i].back_bytes;
-        st[i].s->load_h2d += sizeof(SketchDev*) + sizeof(LoadJob) * (size_t)nh;       // its lines of the batch's job lists
+    const size_t staged = at;
+    const size_t at_out = al256(staged), at_scratch = at_out + al256(sizeof(LoadOut) * n_jobs);
+    const size_t total = at_scratch + prepare_scratch_bytes((int)(n_jobs < kJobs ? n_jobs : kJobs));
+    XP_CUDA_B(pool_alloc((void**)&dev_block, total, &dev_device, &dev_bytes));
+    StageBlock back(sizeof(LoadOut) * n_jobs);
+    if (!back.p) { undo(); return fail(XP_ERR_NOMEM, "out of host memory"); }
+    {
+        std::vector<StageBlock*> hold;
+        std::vector<std::atomic<size_t>> left(piece_at.size());
+        std::vector<size_t> first(piece_at.size() + 1, n);       // sketches of a piece: [first[p], first[p + 1])
+        for (size_t i = n; i-- > 0;) first[st[i].piece] = i;
+        for (size_t p = piece_at.size(); p-- > 0;) if (first[p] == n && p + 1 < first.size()) first[p] = first[p + 1];
+        auto piece_end = [&](size_t p) { return p + 1 < piece_at.size() ? piece_at[p + 1] : staged; };
+        bool ok = true;
+        for (size_t p = 0; p < piece_at.size() && ok; ++p) {
+            hold.push_back(new (std::nothrow) StageBlock(piece_end(p) - piece_at[p]));
+            ok = hold.back() != nullptr && hold.back()->p != nullptr;
+        }
+        cudaError_t err = cudaSuccess;
+        if (ok) {
+            char* lists = hold[0]->p;
+            size_t j = 0;
+            for (size_t i = 0; i < n; ++i) {
+                ((SketchDev**)(lists + at_list))[i] = st[i].s->d_s;
+                for (int h = 0; h < st[i].s->n_holes; ++h, ++j) ((LoadJob*)(lists + at_jobs))[j] = LoadJob{st[i].s->d_s, h, 0};
+            }
+            memcpy(lists + at_copies, copies.data(), sizeof(LoadCopy) * copies.size());
+            // large batches fill their pieces with a few threads; whoever finishes a piece's last share sends the piece
+            size_t n_threads = n / 64;
+            const unsigned hw = std::thread::hardware_concurrency();
+            if (n_threads > 8) n_threads = 8;
+            if (hw > 0 && n_threads > hw) n_threads = hw;
+            for (size_t p = 0; p < piece_at.size(); ++p) left[p].store(first[p + 1] - first[p]);
+            std::atomic<size_t> next(0);
+            std::atomic<int> bad(0);
+            auto send = [&](size_t p) {
+                const cudaError_t e = cudaMemcpyAsync(dev_block + piece_at[p], hold[p]->p, piece_end(p) - piece_at[p], cudaMemcpyHostToDevice, nullptr);
+                if (e != cudaSuccess) bad.store((int)e);
+            };
+            auto work = [&](bool own) {
+                if (own) cudaSetDevice(dev_device);
+                for (;;) {
+                    const size_t i = next.fetch_add(1);
+                    if (i >= n) break;
+                    const size_t p = st[i].piece;
+                    load_fill(&st[i], hold[p]->p + (st[i].stage_at - piece_at[p]));
+                    if (left[p].fetch_sub(1) == 1) send(p);
+                }
+            };
+            if (n_threads < 2) work(false);
+            else {
+                std::vector<std::thread> pool;
+                for (size_t t = 0; t + 1 < n_threads; ++t) pool.emplace_back(work, true);
+                work(false);
+                for (std::thread& th : pool) th.join();
+            }
+            err = (cudaError_t)bad.load();
+            if (err == cudaSuccess) err = launch_scatter((const LoadCopy*)(dev_block + at_copies), (int)copies.size(), dev_block, nullptr);
+            if (err == cudaSuccess) sent = true;
+        }
+        // (the staging blocks may go back once the copies have been made: they are waited for below, with everything else)
+        struct Hold { std::vector<StageBlock*>& v; ~Hold() { for (StageBlock* b : v) delete b; } } release{hold};
+        if (!ok || err != cudaSuccess) {
+            cudaStreamSynchronize(nullptr);
+            undo();
+            return ok ? fail(XP_ERR_CUDA, std::string("xp_sketch_load: ") + cudaGetErrorString(err)) : fail(XP_ERR_NOMEM, "out of host memory");
+        }
+        // host tables too large for the staged copy
+        i64 most_points = 0, most_box = 0, most_spec = 0;
+        int size_cap = 0, probes_cap = 0;
+        u64 most_entries[kMaxSize + 1] = {0};
+        for (size_t i = 0; i < n; ++i) {
+            const LoadState& L = st[i];
+            xp_sketch* s = L.s;
+            const size_t np = (size_t)s->n_points, row = (size_t)(s->g->n_vars ? s->g->n_vars : 1);
+            const size_t coords_bytes = sizeof(i32) * np * row, spec_bytes = sizeof(i64) * np;
+            s->load_h2d = L.head + L.grammar_bytes + sizeof(SketchDev*) + sizeof(LoadJob) * (size_t)s->n_holes + sizeof(LoadCopy) * (L.grammar_fresh ? 2 : 1);
+            s->load_d2h = sizeof(LoadOut) * (size_t)s->n_holes;
+            if (L.copy_coords && coords_bytes > kPackMax) {
+                XP_CUDA_B(cudaMemcpyAsync(s->arena + L.off_coords, L.d->coords, coords_bytes, cudaMemcpyHostToDevice, nullptr));
+                s->load_h2d += coords_bytes;
+            }
+            for (int h = 0; h < s->n_holes; ++h) {
+                const xp_hole_desc& hd = L.d->holes[h];
+                if (hd.spec_kind == XP_SPEC_TABLE && np > 0 && !hd.spec_table_on_device && spec_bytes > kPackMax) {
+                    XP_CUDA_B(cudaMemcpyAsync(s->arena + L.off_spec[h], hd.spec_table, spec_bytes, cudaMemcpyHostToDevice, nullptr));
+                    s->load_h2d += spec_bytes;
+                }
+                if (hd.spec_kind == XP_SPEC_EXPR && L.stage && s->n_points > most_spec) most_spec = s->n_points;
+            }
+            if (L.d->domain_kind == XP_DOMAIN_TABLE && s->n_points > most_points) most_points = s->n_points;
+            if (L.stage_box && s->n_points > most_box) most_box = s->n_points;
+            if (s->tab_size_cap > size_cap) size_cap = s->tab_size_cap;
+            if (s->tab_probes_cap > probes_cap) probes_cap = s->tab_probes_cap;
+            for (int k = 1; k <= s->tab_size_cap; ++k) most_entries[k] = s->entries_at[k] > most_entries[k] ? s->entries_at[k] : most_entries[k];
+        }
+        // The load's kernels, in stream order, one launch of each for the whole batch: points of the boxes and values of
+        // spec expressions (so that the whole-domain check, and the probe choice, read tables for every kind of domain);
+        // bounds of the tables' coordinates; the probe choice; the subtree tables, bottom-up, for as many sizes and probes
+        // as there can be (blocks beyond what the probe choice settled on for their hole return at once).
+        // Grids are cut into pieces of at most kJobs jobs (a grid dimension holds 65 535).
+        SketchDev* const* d_list = (SketchDev* const*)(dev_block + at_list);
+        const LoadJob* d_jobs = (const LoadJob*)(dev_block + at_jobs);
+        for (size_t q = 0; q < n; q += kJobs) {
+            const int m = (int)(n - q < kJobs ? n - q : kJobs);
+            XP_CUDA_B(launch_stage_points(d_list + q, m, most_box, nullptr));
+            XP_CUDA_B(launch_coord_bounds(d_list + q, m, most_points, nullptr));
+        }
+        for (size_t q = 0; q < n_jobs; q += kJobs) {
+            const int m = (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs);
+            XP_CUDA_B(launch_stage_spec(d_jobs + q, m, most_spec, nullptr));
+            XP_CUDA_B(launch_prepare(d_jobs + q, m, dev_block + at_scratch, (LoadOut*)(dev_block + at_out) + q, nullptr));
+        }
+        for (int k = 1; k <= size_cap; ++k)
+            for (size_t q = 0; q < n_jobs; q += kJobs)
+                XP_CUDA_B(launch_subvalues(d_jobs + q, (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs), k, probes_cap, most_entries[k], nullptr));
+        // what the kernels decided, per hole
+        XP_CUDA_B(cudaMemcpyAsync(back.p, dev_block + at_out, sizeof(LoadOut) * n_jobs, cudaMemcpyDeviceToHost, nullptr));
+        XP_CUDA_B(cudaStreamSynchronize(nullptr));
     }
-    XP_CUDA_B(cudaStreamSynchronize(nullptr));
 #undef XP_CUDA_B
-    pool_release(jobs_dev, jobs_bytes, jobs_device);
+    pool_release(dev_block, dev_bytes, dev_device);
+    const LoadOut* o = (const LoadOut*)back.p;
     for (size_t i = 0; i < n; ++i) {
         xp_sketch* s = st[i].s;
-        const int nh = s->n_holes;
-        for (int h = 0; h < nh; ++h) {
-            HoleDev o;
-            memcpy(&o, &st[i].back[sizeof(HoleDev) * h], sizeof(o));
-            u32 bad = 0;
-            memcpy(&bad, &st[i].back[sizeof(HoleDev) * nh + sizeof(u32) * h], sizeof(bad));
-            // the filter applies where the context at probe 0 is affine in the hole, or a comparison
-            s->holes[h].filter_ok = o.filter_ok != 0 && o.tab_probes > 0;
-            s->holes[h].compares = o.filter_ok != 0 && o.aff_ok == 0;
-            s->holes[h].exact = o.aff_ok != 0 && o.join_on == 0;
-            s->holes[h].never = bad != 0;                 // the spec is undefined at some point
-            s->holes[h].second = o.second != 0;
-            s->n_probes.push_back(o.n_probe);
-        }
+        for (int h = 0; h < s->n_holes; ++h, ++o) { hole_decided(&s->holes[h], *o); s->n_probes.push_back(o->n_probe); }
         outs[i] = s;
     }
     return XP_OK;
@@ -1039,10 +1062,7 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         if (e != cudaSuccess || e2 != cudaSuccess)
             return fail(XP_ERR_CUDA, std::string("xp_sketch_refine: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
         for (int h = 0; h < nh; ++h) {
-            s->holes[h].filter_ok = hh[h].filter_ok != 0 && hh[h].tab_probes > 0;
-            s->holes[h].compares = hh[h].filter_ok != 0 && hh[h].aff_ok == 0;
-            s->holes[h].exact = hh[h].aff_ok != 0 && hh[h].join_on == 0;
-            s->holes[h].second = hh[h].second != 0;
+            hole_decided(&s->holes[h], LoadOut{hh[h].filter_ok, hh[h].tab_probes, hh[h].aff_ok, hh[h].join_on, hh[h].second, hh[h].n_probe, 0u, 0u});
             s->n_probes[h] = hh[h].n_probe;
         }
         std::lock_guard<std::mutex> lock(s->plan_mu);

@@ -137,7 +137,7 @@ struct HoleDev {
     // Variables that the context or the spec expression mention (all of them when the spec is the
     // caller's table).  On a box domain a candidate is checked on the sub-box of these and its
     // own variables only: no other variable can change either side of the constraint.
-    u32 fixed_vars, pad2;
+    u32 fixed_vars, spec_bad;                     // spec_bad: set by the load when the spec is undefined at some point
     // The leaf join: values (a0, a1) at its two probes of every tabulated subtree, 8 bytes each (same index as
     // tab_val; a0 = kPairNone: undefined at one of them (a1 = 0) or not below 2^31 in magnitude (a1 = 1)); the leaf sets
     // of the nonterminals; the targets.  join_on: the context is affine at both probes with a factor that 32 bits hold.
@@ -174,6 +174,12 @@ struct SketchDev {
 
 // One hole of one sketch, for the kernels that run at load over a whole batch of sketches.
 struct LoadJob { SketchDev* s; i32 hole, pad; };
+
+// A piece of a load's staged copy (`src` bytes from its start) and where it belongs.
+struct LoadCopy { char* dst; u64 src, bytes; };
+
+// What the load's kernels settled for a hole, as the host reads it back.
+struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe; u32 spec_bad, pad; };
 
 // Per (sketch, hole) accumulators, zeroed (min_rank to all-ones) by the host before the launch.
 struct AccDev {

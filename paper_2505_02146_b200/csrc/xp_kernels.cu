@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(32 * kPrepParts) prep_sample_kernel(const Load
 }
 
 constexpr int kPrepThreads = 64;                        // one thread per sample
-__global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jobs, const u32* masks) {
+__global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jobs, const u32* masks, LoadOut* out) {
     SketchDev* s = jobs[blockIdx.x].s;
     __shared__ i64 s_pt[kProbeSamples][kMaxVars];
     __shared__ i64 s_spec[kProbeSamples];
@@ -413,6 +413,8 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
     }
     __syncthreads();
     probe_contexts(g, hole, s_n, ncand, s_pass0);
+    if (t == 0)                                         // (thread 0 has written all of these itself)
+        out[blockIdx.x] = LoadOut{hole->filter_ok, hole->tab_probes, hole->aff_ok, hole->join_on, hole->second, hole->n_probe, hole->spec_bad, 0u};
 }
 
 // The probes of a hole replaced by the host (xp_sketch_refine: points that ended whole-domain
@@ -1173,19 +1175,31 @@ __device__ __noinline__ u32 fill_reg_operands(const GrammarDev* g, const HoleDev
     return alive;
 }
 
-// Staging of a box domain at load: the coordinates of every point (int32 rows, like a table
-// domain) and, per hole with a spec expression, the spec's value at every point.  *bad is set
-// if the spec is undefined somewhere (then no candidate can match).
-__global__ void __launch_bounds__(256) stage_points_kernel(const SketchDev* sk, i32* coords) {
-    const i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pid >= sk->n_points) return;
+// The shares of a load's staged copy to their places: one grid row per share, 16 bytes per thread and step (sources
+// and destinations are 256-byte aligned, lengths multiples of 256).
+__global__ void __launch_bounds__(256) scatter_kernel(const LoadCopy* copies, const char* src) {
+    const LoadCopy c = copies[blockIdx.y];
+    const uint4* from = reinterpret_cast<const uint4*>(src + c.src);
+    uint4* to = reinterpret_cast<uint4*>(c.dst);
+    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < c.bytes / 16; i += (u64)gridDim.x * blockDim.x) to[i] = from[i];
+}
+
+// Staging of the box domains of a load: the coordinates of every point (int32 rows, like a table
+// domain) and, per hole with a spec expression, the spec's value at every point.  spec_bad is set
+// if the spec is undefined somewhere (then no candidate can match).  One grid row per sketch or hole.
+__global__ void __launch_bounds__(256) stage_points_kernel(SketchDev* const* list) {
+    const SketchDev* sk = list[blockIdx.y];
+    if (!sk->project) return;
+    i32* coords = const_cast<i32*>(sk->coords);
     const int nv = sk->n_vars;
-    u64 rem = (u64)pid;
-    for (int d = nv - 1; d >= 0; --d) {
-        u64 q, r;
-        divmod_u64(rem, (u64)sk->ext[d], q, r);
-        coords[pid * nv + d] = (i32)(sk->lo[d] + (i64)r);
-        rem = q;
+    for (i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x; pid < sk->n_points; pid += (i64)gridDim.x * blockDim.x) {
+        u64 rem = (u64)pid;
+        for (int d = nv - 1; d >= 0; --d) {
+            u64 q, r;
+            divmod_u64(rem, (u64)sk->ext[d], q, r);
+            coords[pid * nv + d] = (i32)(sk->lo[d] + (i64)r);
+            rem = q;
+        }
     }
 }
 
@@ -1213,15 +1227,18 @@ __global__ void __launch_bounds__(256) coord_bounds_kernel(SketchDev* const* lis
     }
 }
 
-__global__ void __launch_bounds__(256) stage_spec_kernel(const SketchDev* sk, int hole_index, i64* spec, u32* bad) {
-    const i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pid >= sk->n_points) return;
-    const HoleDev* hole = &sk->holes[hole_index];
-    i64 pt[kMaxVars];
-    point_coords(sk, pid, pt);
-    i64 v = 0;
-    if (!eval_code(hole->spec, hole->spec_len, pt, 0, v)) atomicOr(bad, 1u);
-    spec[pid] = v;
+__global__ void __launch_bounds__(256) stage_spec_kernel(const LoadJob* jobs) {
+    const SketchDev* sk = jobs[blockIdx.y].s;
+    HoleDev* hole = &sk->holes[jobs[blockIdx.y].hole];
+    if (hole->spec_len == 0 || hole->spec_table == nullptr) return;
+    i64* spec = const_cast<i64*>(hole->spec_table);
+    for (i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x; pid < sk->n_points; pid += (i64)gridDim.x * blockDim.x) {
+        i64 pt[kMaxVars];
+        point_coords(sk, pid, pt);
+        i64 v = 0;
+        if (!eval_code(hole->spec, hole->spec_len, pt, 0, v)) atomicOr(&hole->spec_bad, 1u);
+        spec[pid] = v;
+    }
 }
 
 // Bottom-up construction of one size of a hole's subtree-value tables: thread = (nonterminal,
@@ -2733,12 +2750,12 @@ __global__ void __launch_bounds__(256) int_div_reciprocal_kernel(u32* out, int i
 
 size_t prepare_scratch_bytes(int n_jobs) { return sizeof(u32) * (size_t)kProbeSamples * kPrepWords * (size_t)n_jobs; }
 
-cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, cudaStream_t stream) {
+cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadOut* out, cudaStream_t stream) {
     if (n_jobs <= 0) return cudaSuccess;
     prep_sample_kernel<<<dim3(kPrepWords, (unsigned)n_jobs), 32 * kPrepParts, 0, stream>>>(jobs, (u32*)scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    prepare_kernel<<<n_jobs, kPrepThreads, 0, stream>>>(jobs, (const u32*)scratch);
+    prepare_kernel<<<n_jobs, kPrepThreads, 0, stream>>>(jobs, (const u32*)scratch, out);
     return cudaGetLastError();
 }
 
@@ -2755,13 +2772,25 @@ cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most
     return cudaGetLastError();
 }
 
-cudaError_t launch_stage_points(const SketchDev* s, i64 n_points, i32* coords, cudaStream_t stream) {
-    stage_points_kernel<<<(unsigned)((n_points + 255) / 256), 256, 0, stream>>>(s, coords);
+cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src, cudaStream_t stream) {
+    for (int at = 0; at < n_copies; at += 65535) {
+        const int m = n_copies - at < 65535 ? n_copies - at : 65535;
+        scatter_kernel<<<dim3(m > 64 ? 4u : 16u, (unsigned)m), 256, 0, stream>>>(copies + at, src);
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_stage_spec(const SketchDev* s, int hole_index, i64 n_points, i64* spec, u32* bad, cudaStream_t stream) {
-    stage_spec_kernel<<<(unsigned)((n_points + 255) / 256), 256, 0, stream>>>(s, hole_index, spec, bad);
+cudaError_t launch_stage_points(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream) {
+    if (most_points <= 0 || n_sketches <= 0) return cudaSuccess;
+    const i64 blocks = (most_points + 255) / 256;
+    stage_points_kernel<<<dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_sketches), 256, 0, stream>>>(list);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_stage_spec(const LoadJob* jobs, int n_jobs, i64 most_points, cudaStream_t stream) {
+    if (most_points <= 0 || n_jobs <= 0) return cudaSuccess;
+    const i64 blocks = (most_points + 255) / 256;
+    stage_spec_kernel<<<dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_jobs), 256, 0, stream>>>(jobs);
     return cudaGetLastError();
 }
 

@@ -8,11 +8,12 @@
 namespace xp {
 
 size_t prepare_scratch_bytes(int n_jobs);
-cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, cudaStream_t stream);
+cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadOut* out, cudaStream_t stream);
+cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src, cudaStream_t stream);
 cudaError_t launch_reprobe(const LoadJob* jobs, int n_jobs, cudaStream_t stream);
 cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
-cudaError_t launch_stage_points(const SketchDev* s, i64 n_points, i32* coords, cudaStream_t stream);
-cudaError_t launch_stage_spec(const SketchDev* s, int hole_index, i64 n_points, i64* spec, u32* bad, cudaStream_t stream);
+cudaError_t launch_stage_points(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
+cudaError_t launch_stage_spec(const LoadJob* jobs, int n_jobs, i64 most_points, cudaStream_t stream);
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int most_probes, u64 most_entries, cudaStream_t stream);
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
