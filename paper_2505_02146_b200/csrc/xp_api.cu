@@ -441,6 +441,9 @@ struct HoleHost {
     bool filter_ok = false;          // the probe filter applies (probe 0 exists, context affine or a comparison there, subtree tables)
     bool never = false;              // the spec is undefined at some point: no candidate can match
     bool exact = false;              // the leaf join's conditions do not apply (a context factor of 2^31 or more, or 0)
+    bool join_on = false;            // the context is affine with a factor of 31 bits
+    bool target_zero = false;        // the hole value wanted is zero at one of the join's two probes
+    int tab_max = 0;                 // subtrees up to this size are tabulated
     bool compares = false;           // the filter works on an interval of hole values (the context compares)
     bool second = false;             // filter hits are looked at once more at probe 1 from the start (hits are frequent)
 };
@@ -473,6 +476,8 @@ struct xp_sketch {
     mutable std::vector<SegDev> plan_segs;
     mutable std::vector<JoinSeg> plan_jsegs;
     mutable std::vector<JoinGroup> plan_jgroups;
+    mutable std::vector<PairSeg> plan_psegs;
+    mutable bool plan_pairs = false;                 // ... with the pair join allowed
     mutable std::vector<u64> plan_ops;
     mutable u64 plan_tickets = 0;
 };
@@ -483,6 +488,9 @@ static void hole_decided(HoleHost* h, const LoadOut& o) {
     h->filter_ok = o.filter_ok != 0 && o.tab_probes > 0;
     h->compares = o.filter_ok != 0 && o.aff_ok == 0;
     h->exact = o.aff_ok != 0 && o.join_on == 0;
+    h->join_on = o.aff_ok != 0 && o.join_on != 0;
+    h->target_zero = o.target_zero != 0;
+    h->tab_max = o.tab_max;
     h->second = o.second != 0;
     if (o.spec_bad) h->never = true;                      // the spec is undefined at some point
 }
@@ -1062,7 +1070,8 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         if (e != cudaSuccess || e2 != cudaSuccess)
             return fail(XP_ERR_CUDA, std::string("xp_sketch_refine: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
         for (int h = 0; h < nh; ++h) {
-            hole_decided(&s->holes[h], LoadOut{hh[h].filter_ok, hh[h].tab_probes, hh[h].aff_ok, hh[h].join_on, hh[h].second, hh[h].n_probe, 0u, 0u});
+            hole_decided(&s->holes[h], LoadOut{hh[h].filter_ok, hh[h].tab_probes, hh[h].aff_ok, hh[h].join_on, hh[h].second, hh[h].n_probe, hh[h].tab_max_size,
+                                                  hh[h].join_t0 == 0 || hh[h].join_t1 == 0, 0u, 0u});
             s->n_probes[h] = hh[h].n_probe;
         }
         std::lock_guard<std::mutex> lock(s->plan_mu);
@@ -1101,6 +1110,7 @@ struct Plan {
     std::vector<SegDev> segs;
     std::vector<JoinSeg> jsegs;
     std::vector<JoinGroup> jgroups;
+    std::vector<PairSeg> psegs;
     std::vector<AccDev> acc;
     std::vector<u64> nominal_ops;    // per accumulator: cost-model operations of the filter stage
     u64 n_tickets = 0, n_join = 0;
@@ -1128,11 +1138,66 @@ static void add_linear(Plan* plan, int sketch, int hole, int acc, int k, u64 lo,
     plan->n_tickets += (hi - lo + (u64)kLinearChunk - 1) / (u64)kLinearChunk;
 }
 
+constexpr size_t kPairMaxSketches = 8;
+constexpr u64 kPairLeast = 1ull << 20;       // pairs from which an index of one side costs less than a test per pair
+constexpr u64 kPairMost = 1ull << 22;        // operands of either side (the size of the subtree tables)
+
+// Does the pair join take the block (production, left size a) of size k?  Both operands tabulated, an operator it knows
+// (products only where neither target is zero: a zero operand would leave its partner open), enough pairs.
+static bool pair_joins(const xp_grammar* g, const HoleHost& ho, const BinDev& bd, int a, int k) {
+    const int b = k - 1 - a;
+    if (!ho.join_on || bd.op > XP_OP_MOD || (bd.op == XP_OP_MUL && ho.target_zero)) return false;
+    if (a > ho.tab_max || b > ho.tab_max) return false;
+    const u64 cl = g->cnt[bd.lnt][a], cr = g->cnt[bd.rnt][b];
+    return cl <= kPairMost && cr <= kPairMost && cl * cr >= kPairLeast;
+}
+
+// Pair-join blocks of (start nonterminal, size k) that ranks [lo, hi) touch: one per (left, right) operand sets.
+static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi) {
+    const size_t first_seg = plan->psegs.size();
+    const int nt = ho.start_nt;
+    for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
+        const BinDev& bd = g->bins[b];
+        u64 base = bd.off[k];
+        for (int a = 1; a <= k - 2; ++a) {
+            const u64 cl = g->cnt[bd.lnt][a], cr = g->cnt[bd.rnt][k - 1 - a];
+            const u64 this_base = base;
+            base += cl * cr;
+            if (a == 1 || a == k - 2 || cl * cr == 0 || !pair_joins(g, ho, bd, a, k)) continue;
+            if (this_base + cl * cr <= lo || this_base >= hi) continue;
+            PairSeg* sg = nullptr;
+            for (size_t i = first_seg; i < plan->psegs.size() && !sg; ++i) {
+                PairSeg& c = plan->psegs[i];
+                if (c.lnt == bd.lnt && c.rnt == bd.rnt && c.la == a && !((c.ops >> bd.op) & 1u)) sg = &c;
+            }
+            if (!sg) {
+                PairSeg c;
+                memset(&c, 0, sizeof(c));
+                c.rank_begin = lo; c.rank_end = hi;
+                c.sketch = sketch; c.hole = hole; c.size = k; c.acc = acc;
+                c.lnt = bd.lnt; c.la = a; c.rnt = bd.rnt; c.ra = k - 1 - a;
+                c.nl = (u32)cl; c.nr = (u32)cr;
+                c.index_right = cr <= cl ? 1 : 0;            // the smaller side is indexed (its chains stay in L2)
+                u32 heads = 1024;
+                while (heads < (c.index_right ? c.nr : c.nl)) heads <<= 1;
+                c.head_mask = heads - 1;
+                // divisors are cut so that some thousand warps have work even for a few blocks of dividends
+                const u64 blocks = (c.nl + 31) / 32;
+                c.pieces = (u32)(blocks >= 4096 ? 1 : blocks >= 512 ? 4 : 16);
+                plan->psegs.push_back(c);
+                sg = &plan->psegs.back();
+            }
+            sg->ops |= 1u << bd.op;
+            sg->base[bd.op] = this_base;
+        }
+    }
+}
+
 constexpr u64 kFamilyMaxWork = 512;          // candidates per register operand below which segments share a fill
 
 // Tile segments of (start nonterminal, size k) restricted to ranks [lo, hi): one per
 // (left size, group of productions with the same operand nonterminals and the same rows).
-static void add_tiles(Plan* plan, const xp_grammar* g, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, int bc_tile) {
+static void add_tiles(Plan* plan, const xp_grammar* g, const HoleHost* pairs, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, int bc_tile) {
     const size_t first_seg = plan->segs.size();
     for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
         const BinDev& bd = g->bins[b];
@@ -1144,6 +1209,7 @@ static void add_tiles(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
             const u64 this_base = base;
             base += block;
             if (a == 1 || a == k - 2) continue;              // (a leaf at the root: add_joins)
+            if (pairs && pair_joins(g, *pairs, bd, a, k)) continue;      // (add_pairs)
             if (this_base + block <= lo || this_base >= hi) continue;
             const u64 wlo = lo > this_base ? lo - this_base : 0;
             const u64 whi = hi - this_base < block ? hi - this_base : block;
@@ -1347,7 +1413,7 @@ static void number_joins(Plan* plan) {
 
 constexpr u64 kTileMinRanks = 4096;          // smaller windows are searched rank by rank
 
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, Plan* plan);
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, bool pairs, Plan* plan);
 
 // A sketch's tables, and the library's scratch, live on the device that was current when the sketch was
 // loaded: a call made with another device current would hand the kernels pointers of the wrong GPU.
@@ -1361,21 +1427,27 @@ static xp_status check_device(const xp_sketch* const* sk, size_t n) {
     return XP_OK;
 }
 
-static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, Plan* plan) {
+// (static_scratch: the call's scratch is the fixed array, which has no room for the pair join's index)
+static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, bool static_scratch, Plan* plan) {
+    // the pair join takes its blocks one after the other, several launches each: a batch keeps to the tiles, which
+    // search all holes in one launch
+    const bool pairs = !static_scratch && n <= kPairMaxSketches;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
         if (!s) return fail(XP_ERR_INVALID_ARG, "null sketch in batch");
-        if (!plain) { plan_sketch(s, i, o, plan); continue; }
+        if (!plain) { plan_sketch(s, i, o, pairs, plan); continue; }
         {
             std::lock_guard<std::mutex> lock(s->plan_mu);
-            if (!s->plan_cached) {
+            if (!s->plan_cached || s->plan_pairs != pairs) {
                 Plan own;
-                plan_sketch(s, 0, o, &own);
+                plan_sketch(s, 0, o, pairs, &own);
                 s->plan_segs = std::move(own.segs);
                 s->plan_jsegs = std::move(own.jsegs);
                 s->plan_jgroups = std::move(own.jgroups);
+                s->plan_psegs = std::move(own.psegs);
+                s->plan_pairs = pairs;
                 s->plan_ops = std::move(own.nominal_ops);
                 s->plan_tickets = own.n_tickets;
                 s->plan_cached = true;
@@ -1397,6 +1469,7 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
         plan->n_tickets += s->plan_tickets;
         const size_t jat = plan->jsegs.size();
         plan->jsegs.insert(plan->jsegs.end(), s->plan_jsegs.begin(), s->plan_jsegs.end());
+        for (const PairSeg& ps : s->plan_psegs) { plan->psegs.push_back(ps); plan->psegs.back().sketch = (i32)i; plan->psegs.back().acc += acc_base; }
         const i32 group_base = (i32)plan->jgroups.size();
         plan->jgroups.insert(plan->jgroups.end(), s->plan_jgroups.begin(), s->plan_jgroups.end());
         for (size_t j = jat; j < plan->jsegs.size(); ++j) {
@@ -1408,7 +1481,7 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
 }
 
 // One sketch's segments, accumulators and tickets, appended to the plan as sketch number i.
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, Plan* plan) {
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, bool pairs, Plan* plan) {
     {
         for (int h = 0; h < s->n_holes; ++h) {
             const HoleHost& ho = s->holes[h];
@@ -1435,7 +1508,8 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 if (!ho.filter_ok || (o->flags & XP_FLAG_NO_FILTER)) { add_linear(plan, (int)i, h, acc, k, lo, hi); continue; }
                 if (k < 3 || (!forced && hi - lo < kTileMinRanks)) { add_direct(plan, ho.start_nt, (int)i, h, acc, k, lo, hi); continue; }
                 add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact);
-                add_tiles(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile);
+                if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi);
+                add_tiles(plan, s->g, pairs ? &ho : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile);
             }
         }
     }
@@ -1450,13 +1524,41 @@ static u32 surv_cap_for(size_t n_sketches) {
 }
 constexpr u32 kSurvCapStatic = 8192;         // ... of a call on the library's fixed scratch
 
+// Scratch of a pair-join block beside its chain heads: counters and histograms (zero at launch), and what kernels fill.
+constexpr size_t kPairZeros = 256 + 2 * 4096;
+static size_t pair_rest_bytes(const PairSeg& c) {
+    const size_t nl = c.nl, nr = c.nr;
+    return align256(sizeof(u32) * (c.index_right ? nr : nl)) + align256(sizeof(u32) * nl) + align256(sizeof(u32) * nr) +
+           ((c.ops & 24u) ? 2 * align256(sizeof(u32) * 1025) + align256(12 * nl) + align256(12 * nr) + 512 : 0);
+}
+static void pair_place(PairSeg& c, char* ones, char* zeros, char* rest) {
+    const size_t nl = c.nl, nr = c.nr;
+    c.head = (u32*)ones;
+    c.counters = (u32*)zeros;
+    c.ticket = (u64*)(zeros + 64);
+    c.hist[0] = (u32*)(zeros + 256); c.hist[1] = (u32*)(zeros + 256 + 4096);
+    auto take = [&](size_t bytes) { char* p = rest; rest += align256(bytes); return p; };
+    c.next = (u32*)take(sizeof(u32) * (c.index_right ? nr : nl));
+    c.wide_l = (u32*)take(sizeof(u32) * nl);
+    c.wide_r = (u32*)take(sizeof(u32) * nr);
+    if (c.ops & 24u)
+        for (int k = 0; k < 2; ++k) {
+            const size_t n = k ? nr : nl;
+            c.start[k] = (u32*)take(sizeof(u32) * 1025);
+            char* p = take(12 * n);
+            c.val[k] = (int2*)p;
+            c.id[k] = (u32*)(p + 8 * n);
+        }
+}
+
 static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size_t n_sketches, u32 surv_cap) {
     SearchLayout w;
     const size_t n_acc = plan.acc.size();
     w.segs = 256;
     w.jsegs = w.segs + align256(sizeof(SegDev) * plan.segs.size());
     w.jgroups = w.jsegs + align256(sizeof(JoinSeg) * plan.jsegs.size());
-    w.sketches = w.jgroups + align256(sizeof(JoinGroup) * plan.jgroups.size());
+    w.psegs = w.jgroups + align256(sizeof(JoinGroup) * plan.jgroups.size());
+    w.sketches = w.psegs + align256(sizeof(PairSeg) * plan.psegs.size());
     w.acc = w.sketches + align256(sizeof(SketchDev*) * (n_sketches + 1));
     w.hist = w.acc + align256(sizeof(AccDev) * (n_acc + 1));
     w.head = w.hist + align256(sizeof(u32) * (n_acc + 1));
@@ -1465,6 +1567,13 @@ static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size
     w.sorted = w.sort_off + align256(sizeof(u32) * (n_acc + 2));
     w.longs = w.sorted + align256(sizeof(u32) * (size_t)surv_cap);
     w.total = w.longs + align256(sizeof(u32) * (size_t)surv_cap);
+    w.n_psegs = (int)plan.psegs.size();
+    w.pair_ones = w.total;
+    for (const PairSeg& c : plan.psegs) w.total += align256(sizeof(u32) * ((size_t)c.head_mask + 1));
+    w.pair_zeros = w.total;
+    for (size_t i = 0; i < plan.psegs.size(); ++i) w.total += kPairZeros;
+    w.pair_rest = w.total;
+    for (const PairSeg& c : plan.psegs) w.total += pair_rest_bytes(c);
     w.n_acc = (int)n_acc; w.n_segs = (int)plan.segs.size(); w.n_jsegs = (int)plan.jsegs.size(); w.n_sketches = (int)n_sketches;
     w.surv_cap = surv_cap;
     w.join_wide = plan.join_wide ? 1 : 0;
@@ -1486,10 +1595,18 @@ static int least_size(const AccDev& a, int max_size) {
 }
 
 // What a call sends to the device in one copy: counters at zero, segments, sketches, accumulators in their start state.
-static void stage_plan(char* stage, const SearchLayout& w, const Plan& plan, const xp_sketch* const* sketches) {
+static void stage_plan(char* stage, char* ws, const SearchLayout& w, Plan& plan, const xp_sketch* const* sketches) {
     memset(stage, 0, 256);
     if (!plan.segs.empty()) memcpy(stage + w.segs, plan.segs.data(), sizeof(SegDev) * plan.segs.size());
     if (!plan.jsegs.empty()) memcpy(stage + w.jsegs, plan.jsegs.data(), sizeof(JoinSeg) * plan.jsegs.size());
+    {
+        char *ones = ws + w.pair_ones, *zeros = ws + w.pair_zeros, *rest = ws + w.pair_rest;
+        for (PairSeg& c : plan.psegs) {
+            pair_place(c, ones, zeros, rest);
+            ones += align256(sizeof(u32) * ((size_t)c.head_mask + 1)); zeros += kPairZeros; rest += pair_rest_bytes(c);
+        }
+        if (!plan.psegs.empty()) memcpy(stage + w.psegs, plan.psegs.data(), sizeof(PairSeg) * plan.psegs.size());
+    }
     if (!plan.jgroups.empty()) memcpy(stage + w.jgroups, plan.jgroups.data(), sizeof(JoinGroup) * plan.jgroups.size());
     for (int i = 0; i < w.n_sketches; ++i) ((const SketchDev**)(stage + w.sketches))[i] = sketches[i]->d_s;
     memcpy(stage + w.acc, plan.acc.data(), sizeof(AccDev) * plan.acc.size());
@@ -1499,7 +1616,7 @@ static void stage_plan(char* stage, const SearchLayout& w, const Plan& plan, con
 extern "C" size_t xp_workspace_bytes(const xp_sketch* const* sketches, size_t n, const xp_repair_opts* opts) {
     if (!sketches || n == 0) return 0;
     Plan plan;
-    if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, &plan) != XP_OK) return 0;
+    if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, false, &plan) != XP_OK) return 0;
     return ws_layout(plan, sketches, n, surv_cap_for(n)).total;
 }
 
@@ -1512,7 +1629,7 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     if (o->cancel && *o->cancel) return fail(XP_ERR_CANCELLED, "cancelled before launch");
     const auto t0 = std::chrono::steady_clock::now();
     Plan plan;
-    xp_status st = build_plan(sketches, n, o, &plan);
+    xp_status st = build_plan(sketches, n, o, false, &plan);
     if (st == XP_OK) st = check_device(sketches, n);
     if (st != XP_OK) return st;
     cudaStream_t stream = (cudaStream_t)o->stream;
@@ -1549,7 +1666,7 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
 #define XP_CUDA_R(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { cudaStreamSynchronize(stream); give_back(); \
         return fail(e_ == cudaErrorMemoryAllocation ? XP_ERR_NOMEM : XP_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); } } while (0)
     if (!stage.p) { give_back(); return fail(XP_ERR_NOMEM, "out of host memory"); }
-    stage_plan(stage.p, w, plan, sketches);
+    stage_plan(stage.p, ws, w, plan, sketches);
     const AccDev* acc = (const AccDev*)(stage.p + w.head);
     u32* check_word = (u32*)(stage.p + w.head + acc_bytes);
     *check_word = 0;
@@ -1578,7 +1695,8 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
         }
     }
     if (stopped == XP_OK) {
-        XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets + plan.n_join > 0, stream, &launches));
+        XP_CUDA_R(launch_pairs(ws, w, plan.psegs.data(), stream, &launches));
+        XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets + plan.n_join + plan.psegs.size() > 0, stream, &launches));
         XP_CUDA_R(cudaEventRecord(ev.e1, stream));
         XP_CUDA_R(cudaMemcpyAsync(stage.p + w.head, ws + w.acc, acc_bytes, cudaMemcpyDeviceToHost, stream));
 #ifdef XP_CHECKS
@@ -1646,7 +1764,7 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
     if (o->n_rank_ranges < 0 || (o->n_rank_ranges > 0 && !o->rank_ranges)) return fail(XP_ERR_INVALID_ARG, "bad rank_ranges");
     if (o->cancel && *o->cancel) return fail(XP_ERR_CANCELLED, "cancelled before launch");
     Plan plan;
-    xp_status st = build_plan(&sketch, 1, o, &plan);
+    xp_status st = build_plan(&sketch, 1, o, true, &plan);
     if (st == XP_OK) st = check_device(&sketch, 1);
     if (st != XP_OK) return st;
     const SearchLayout w = ws_layout(plan, &sketch, 1, kSurvCapStatic);
@@ -1658,7 +1776,7 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
                     "; use xp_repair with a workspace");
     StageBlock stage(w.head + sizeof(AccDev) * plan.acc.size());       // (page-locked host memory that the library keeps)
     if (!stage.p) return fail(XP_ERR_NOMEM, "out of host memory");
-    stage_plan(stage.p, w, plan, &sketch);
+    stage_plan(stage.p, nullptr, w, plan, &sketch);
     const AccDev* acc = (const AccDev*)(stage.p + w.head);
     cudaStream_t stream = (cudaStream_t)o->stream;
     cudaError_t e = launch_search_static(stage.p, w, plan.n_tickets, plan.n_join, (AccDev*)(stage.p + w.head), stream);

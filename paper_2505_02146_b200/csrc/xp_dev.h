@@ -3,6 +3,7 @@
 #pragma once
 
 #include <stdint.h>
+#include <vector_types.h>
 
 #include "xp.h"
 
@@ -179,7 +180,7 @@ struct LoadJob { SketchDev* s; i32 hole, pad; };
 struct LoadCopy { char* dst; u64 src, bytes; };
 
 // What the load's kernels settled for a hole, as the host reads it back.
-struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe; u32 spec_bad, pad; };
+struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe, tab_max, target_zero; u32 spec_bad, pad; };
 
 // Per (sketch, hole) accumulators, zeroed (min_rank to all-ones) by the host before the launch.
 struct AccDev {
@@ -216,6 +217,28 @@ struct JoinSeg {
     u32 chunk;                       // operands per ticket
     i32 pad;
     u64 e_begin, e_count;
+};
+
+// One (left operands, right operands) block of the pair join (csrc/xp_pairs.cuh): every  L op R  of its operators.
+struct PairSeg {
+    u64 rank_begin, rank_end;        // window of ranks searched at this size
+    i32 sketch, hole, size, acc;
+    i32 lnt, la, rnt, ra;            // nonterminal and size of either operand
+    u32 nl, nr;                      // operands
+    u32 ops;                         // operator slots (+ - * / %)
+    i32 index_right;                 // the chains index the right operands (else the left ones)
+    u64 base[5];                     // rank of (0, 0) per operator
+    u32 head_mask, pieces;           // pieces: parts that a warp's divisors are cut into
+    // device scratch of the call
+    u32* head;                       // head_mask + 1, all ones at launch
+    u32* next;
+    u32* counters;                   // [2] wide operands left, right, then the ticket (u64): zero at launch
+    u64* ticket;
+    u32 *wide_l, *wide_r;
+    u32* hist[2];                    // 1024 each, zero at launch
+    u32* start[2];                   // 1025 each
+    u32* id[2];                      // operands by magnitude
+    int2* val[2];
 };
 
 // One contiguous piece of work.  kind 0 (linear): ranks [rank_begin, rank_end) of `size`,
@@ -266,6 +289,7 @@ struct PlanDev {
     const SegDev* segs;              // device
     const JoinSeg* jsegs;            // device
     const JoinGroup* jgroups;        // device
+    const PairSeg* psegs;            // device
     i32 n_jsegs, pad0;
     u64 join_base, n_join;           // tickets of the leaf join that belong to this launch
     u64* join_ticket;                // device counter, zero at launch

@@ -118,14 +118,14 @@ __device__ __forceinline__ bool exact_pair(const GrammarDev* g, const HoleDev* h
 }
 
 // The warp checks one candidate on the whole domain itself (the survivor queue is full).
-__device__ __noinline__ void join_verify(JoinWarp& w, const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, int size, int acc, u64 rank,
+__device__ __noinline__ void join_verify(CandShared& cand, const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, int size, int acc, u64 rank,
                                          u32 vars, u64& evals) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
-    if (lane == 0) { stage_candidate(w.cand, sk, hole, size, rank); (void)proj_points(sk, hole, vars, &w.cand); }
+    if (lane == 0) { stage_candidate(cand, sk, hole, size, rank); (void)proj_points(sk, hole, vars, &cand); }
     __syncwarp();
     i64 fail_pid = 0;
-    const bool ok = check_points(w.cand, sk, hole, 0, proj_points(sk, hole, vars, nullptr), evals, &fail_pid);
+    const bool ok = check_points(cand, sk, hole, 0, proj_points(sk, hole, vars, nullptr), evals, &fail_pid);
     if (ok && lane == 0) {
         atomicAdd(&plan.acc[acc].match_count[size], 1ull);
         atomicMin(&plan.acc[acc].min_rank[size], rank);
@@ -145,7 +145,7 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
     while (m) {
         const int src = __ffs((int)m) - 1;
         m &= m - 1;
-        join_verify(w, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
+        join_verify(w.cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
     }
 }
 

@@ -414,7 +414,8 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
     __syncthreads();
     probe_contexts(g, hole, s_n, ncand, s_pass0);
     if (t == 0)                                         // (thread 0 has written all of these itself)
-        out[blockIdx.x] = LoadOut{hole->filter_ok, hole->tab_probes, hole->aff_ok, hole->join_on, hole->second, hole->n_probe, hole->spec_bad, 0u};
+        out[blockIdx.x] = LoadOut{hole->filter_ok, hole->tab_probes, hole->aff_ok, hole->join_on, hole->second, hole->n_probe, hole->tab_max_size,
+                                  hole->join_t0 == 0 || hole->join_t1 == 0 ? 1 : 0, hole->spec_bad, 0u};
 }
 
 // The probes of a hole replaced by the host (xp_sketch_refine: points that ended whole-domain
@@ -2237,6 +2238,7 @@ __global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const PlanD
 
 }  // namespace xp
 #include "xp_join.cuh"
+#include "xp_pairs.cuh"
 namespace xp {
 
 // ------------------------------------------------------------------------------------------
@@ -2842,6 +2844,7 @@ static PlanDev plan_on(char* base, const SearchLayout& L) {
     pd.segs = (const SegDev*)(base + L.segs);
     pd.jsegs = (const JoinSeg*)(base + L.jsegs);
     pd.jgroups = (const JoinGroup*)(base + L.jgroups);
+    pd.psegs = (const PairSeg*)(base + L.psegs);
     pd.n_jsegs = L.n_jsegs; pd.pad0 = 0;
     pd.join_base = pd.n_join = 0;
     pd.join_ticket = (u64*)(base + 32);
@@ -2890,6 +2893,40 @@ cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64
     }
     *n_launches += 1;
     return cudaGetLastError();
+}
+
+// The pair join, one block after the other: index, then the lookups; sorted operands for / and %.
+cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_segs, cudaStream_t stream, int* n_launches) {
+    if (L.n_psegs == 0) return cudaSuccess;
+    const Residency* R = residency();
+    if (!R) return cudaErrorInvalidDevice;
+    PlanDev pd = plan_on(base, L);
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(base + L.pair_ones, 0xff, L.pair_zeros - L.pair_ones, stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(base + L.pair_zeros, 0, L.pair_rest - L.pair_zeros, stream)) != cudaSuccess) return e;
+    for (int i = 0; i < L.n_psegs; ++i) {
+        const PairSeg& s = host_segs[i];
+        const u32 most = s.nl > s.nr ? s.nl : s.nr, drive = s.index_right ? s.nl : s.nr;
+        auto ctas = [&](u32 n, int per_sm) {
+            const u32 want = (n + kPairThreads - 1) / kPairThreads, cap = (u32)(R->sms * per_sm);
+            return want < cap ? want : cap;
+        };
+        pair_build_kernel<<<(most + kPairThreads - 1) / kPairThreads, kPairThreads, 0, stream>>>(pd, i);
+        pair_hash_kernel<<<ctas(drive, 3), kPairThreads, 0, stream>>>(pd, i);
+        *n_launches += 2;
+        if (s.ops & 24u) {                                // / or %
+            pair_sort_count_kernel<<<dim3(ctas(most, 2), 2), kPairThreads, 0, stream>>>(pd, i);
+            pair_sort_scan_kernel<<<2, kPairBuckets, 0, stream>>>(pd, i);
+            pair_sort_scatter_kernel<<<dim3(ctas(most, 4), 2), kPairThreads, 0, stream>>>(pd, i);
+            const u64 warps = (u64)((s.nl + 31) / 32) * s.pieces, cap = (u64)R->sms * 3 * kPairWarps;
+            pair_div_kernel<<<(unsigned)(((warps < cap ? warps : cap) + kPairWarps - 1) / kPairWarps), kPairThreads, 0, stream>>>(pd, i);
+            *n_launches += 4;
+        }
+        pair_wide_kernel<<<(unsigned)R->sms, kPairThreads, 0, stream>>>(pd, i);
+        *n_launches += 1;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Stage 3, after every part of the search has been queued.

@@ -18,13 +18,14 @@ cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int most
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
 //      build only), 24: long survivors (u32), 32: join ticket (u64)   -- zero at launch
-//   segs, jsegs, jgroups, sketches, acc: staged from the host;  [0, head) is what the host copies in
+//   segs, jsegs, jgroups, psegs, sketches, acc: staged from the host;  [0, head) is what the host copies in
 //   hist: survivors per accumulator slot, zero at launch (staged);
 //   surv: the survivor queue (surv_cap entries); sort_off, sorted: its hole order -- written by the kernels only
 struct SearchLayout {
-    size_t segs, jsegs, jgroups, sketches, acc, hist, head, surv, sort_off, sorted, longs, total;
+    size_t segs, jsegs, jgroups, psegs, sketches, acc, hist, head, surv, sort_off, sorted, longs, total;
+    size_t pair_ones, pair_zeros, pair_rest;      // scratch of the pair join: [pair_ones, pair_zeros) all ones, [pair_zeros, pair_rest) zero at launch
     u32 surv_cap, max_chunks;        // max_chunks: chunks of the whole-domain check that the largest domain needs
-    int n_segs, n_jsegs, n_sketches, n_acc;
+    int n_segs, n_jsegs, n_psegs, n_sketches, n_acc;
     int dense;                       // some hole of the plan takes the second look: launch the search kernel's dense form
     int join_wide;                   // tickets of the leaf join are long enough for several operands per lane
     int empty_domain;                // some sketch has no points at all
@@ -33,6 +34,7 @@ struct SearchLayout {
 // The whole search on a staged scratch, or the same in pieces: one range of tickets at a time, then the rest.
 cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64 t_begin, u64 t_end, bool restart, cudaStream_t stream,
                                int* n_launches);
+cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_segs, cudaStream_t stream, int* n_launches);
 cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, cudaStream_t stream, int* n_launches);
 cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, u64 n_join, cudaStream_t stream, int* n_launches);
 int search_warps();                                  // warps of the leaf join that run at a time

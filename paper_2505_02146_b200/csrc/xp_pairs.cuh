@@ -1,0 +1,389 @@
+// The pair join: candidates  L op R  whose operands both have three nodes or more.
+//
+// The tile kernel tests every pair of two operand sets (config 2's size 7 = 3 + 1 + 3: 92 480^2 pairs and five operators,
+// 4 ms).  Here the pairs that can reach the target (t0, t1) at the join's two probes are found from an index of one set:
+//   pair_build_kernel  -- hash chains over one set, by its values (v0, v1) at the two probes;
+//   pair_hash_kernel   -- + - *: an operand x of the other set asks for its partner's values directly (t - x, x - t, t + x, t / x);
+//   pair_sort_*        -- both sets by magnitude at the first probe (992 buckets of a float's exponent and five mantissa
+//                         bits; order inside a bucket does not matter);
+//   pair_div_kernel    -- / %: a warp takes 32 dividends next to each other in that order and walks only the divisors that
+//                         can reach the target: |r| in (|l|/(|t|+1), |l|/|t|] for a quotient, (|t|, |l| - |t|] for a remainder
+//                         (any above |t| when l is the target itself);
+//   pair_wide_kernel   -- operands that are not narrow (31 bits, or the root of 2^62 / |context factor|), exactly.
+// Candidates that agree at both probes wait in a warp's queue and are checked 32 at a time at the other probes.
+#pragma once
+
+namespace xp {
+
+constexpr int kPairThreads = 256;
+constexpr int kPairWarps = kPairThreads / 32;
+
+struct PairWarp {
+    u32 c_l[64], c_r[64], c_op[64];
+    u32 nc;
+    CandShared cand;
+};
+
+// The lane's candidate against the queue's remaining probes.  Called by all lanes.
+__device__ __noinline__ void pair_check(PairWarp& w, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, int from, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const u32 nc = w.nc;
+    const u64 lo = hole->tab_off[seg.lnt][seg.la], ro = hole->tab_off[seg.rnt][seg.ra];
+    for (u32 at = 0; at < nc; at += 32) {
+        bool pass = false;
+        u64 rank = 0;
+        u32 vars = 0;
+        if (at + lane < nc) {
+            const u32 l = w.c_l[at + lane], r = w.c_r[at + lane];
+            const int slot = (int)w.c_op[at + lane];
+            rank = seg.base[slot] + (u64)l * seg.nr + r;
+            if (rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(l < seg.nl && r < seg.nr && rank < g->cnt[hole->start_nt][seg.size], kChkQueue)) {
+                pass = true;
+                for (int j = from; j < hole->n_exact && pass; ++j) {
+                    ++n.evals;
+                    const u64 b = (u64)j * hole->tab_total;
+                    i64 v;
+                    pass = hole->tab_ok[b + lo + l] && hole->tab_ok[b + ro + r] &&
+                           apply_op(op_of_slot(slot), hole->tab_val[b + lo + l], hole->tab_val[b + ro + r], v) && probe_accepts(hole, j, v);
+                }
+                if (pass && hole->n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
+                vars = (u32)hole->tab_vars[lo + l] | (u32)hole->tab_vars[ro + r];
+            }
+        }
+        u32 m = __ballot_sync(0xffffffffu, pass);
+        if (!m) continue;
+        n.passes += (u32)__popc(m);
+        const bool pending = pass && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
+        m = __ballot_sync(0xffffffffu, pending);
+        while (m) {
+            const int src = __ffs((int)m) - 1;
+            m &= m - 1;
+            join_verify(w.cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
+        }
+    }
+    __syncwarp();
+    if (lane == 0) w.nc = 0;
+    __syncwarp();
+}
+
+__device__ __forceinline__ void pair_push(PairWarp& w, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, bool have, u32 l, u32 r,
+                                          int slot, int from, JoinCount& n) {
+    const u32 b = __ballot_sync(0xffffffffu, have);
+    if (!b) return;
+    const int lane = threadIdx.x & 31;
+    const u32 nc = w.nc;
+    n.suspects += (u32)__popc(b);
+    if (have) {
+        const u32 at = nc + (u32)__popc(b & ((1u << lane) - 1u));
+        w.c_l[at] = l; w.c_r[at] = r; w.c_op[at] = (u32)slot;
+    }
+    __syncwarp();
+    if (lane == 0) w.nc = nc + (u32)__popc(b);
+    __syncwarp();
+    if (nc + (u32)__popc(b) >= 32u) pair_check(w, plan, seg, sk, hole, from, n);
+}
+
+// Entry i of a set: its values at the two probes; 0 undefined, 1 narrow, 2 wide.
+__device__ __forceinline__ int pair_entry(const HoleDev* hole, u64 off, u32 i, u32 lim, int2& v) {
+    v = reinterpret_cast<const int2*>(hole->tab_pair)[off + i];
+    if (v.x == kPairNone) return v.y ? 2 : 0;
+    return abs_u32(v.x) < lim && abs_u32(v.y) < lim ? 1 : 2;
+}
+
+__device__ __forceinline__ u32 pair_slot(int2 v, u32 mask) {
+    u32 h = (u32)v.x * 0x9E3779B1u ^ ((u32)v.y + 0x7F4A7C15u) * 0x85EBCA77u;
+    h ^= h >> 15; h *= 0xC2B2AE3Du; h ^= h >> 13;
+    return h & mask;
+}
+
+// Narrow values stay below this: products with the context's factor must not reach 2^62.
+__device__ __forceinline__ u32 pair_limit(const HoleDev* hole) {
+    const i64 a0 = (i64)hole->aff_Aj[0], a1 = (i64)hole->aff_Aj[hole->join_p1];
+    const u64 m0 = a0 < 0 ? 0ull - (u64)a0 : (u64)a0, m1 = a1 < 0 ? 0ull - (u64)a1 : (u64)a1, A = m0 > m1 ? m0 : m1;
+    if (A <= 1) return 0x7fffffffu;
+    u32 l = 0x7fffffffu;
+    while ((u64)l * l >= (1ull << 62) / A) l >>= 1;       // (a power of two less one: at most a bit below the root)
+    return l;
+}
+
+// Chains of the indexed set (narrow entries), and the lists of wide entries of both sets.
+__global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const PlanDev plan, int index) {
+    const PairSeg& seg = plan.psegs[index];
+    const SketchDev* sk = plan.sketches[seg.sketch];
+    const HoleDev* hole = &sk->holes[seg.hole];
+    const u32 lim = pair_limit(hole);
+    const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int side = 0; side < 2; ++side) {                // 0: left, 1: right
+        const u32 n = side ? seg.nr : seg.nl;
+        if (i >= n) continue;
+        int2 v;
+        const int st = pair_entry(hole, side ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la], i, lim, v);
+        if (st == 2) (side ? seg.wide_r : seg.wide_l)[atomicAdd(&seg.counters[side], 1u)] = i;
+        if (side == seg.index_right && st == 1) seg.next[i] = atomicExch(&seg.head[pair_slot(v, seg.head_mask)], i);
+    }
+}
+
+// + - *: one thread per operand x of the set that is not indexed.
+__global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const PlanDev plan, int index) {
+    __shared__ PairWarp sh[kPairWarps];
+    PairWarp& w = sh[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) w.nc = 0;
+    __syncwarp();
+    const PairSeg& seg = plan.psegs[index];
+    const SketchDev* sk = plan.sketches[seg.sketch];
+    const HoleDev* hole = &sk->holes[seg.hole];
+    JoinCount n{0, 0, 0, 0, 0};
+    const bool ir = seg.index_right != 0;
+    const u32 nx = ir ? seg.nl : seg.nr;
+    const u64 xo = ir ? hole->tab_off[seg.lnt][seg.la] : hole->tab_off[seg.rnt][seg.ra];
+    const u64 yo = ir ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la];
+    const int2* Y = reinterpret_cast<const int2*>(hole->tab_pair) + yo;
+    const u32 lim = pair_limit(hole);
+    const i64 t0 = hole->join_t0, t1 = hole->join_t1;
+    const int from = hole->join_p1 ? 2 : 1;
+    const u32 ops = hole->join_none ? 0u : seg.ops & ((1u << kSlotAdd) | (1u << kSlotSub) | (1u << kSlotMul));
+    for (u32 x0 = (blockIdx.x * kPairWarps + (threadIdx.x >> 5)) * 32u; x0 < nx; x0 += gridDim.x * kPairThreads) {
+        const u32 x = x0 + lane;
+        int2 v = make_int2(0, 0);
+        const bool live = x < nx && pair_entry(hole, xo, x, lim, v) == 1;
+        for (u32 m = ops; m; m &= m - 1) {
+            const int slot = __ffs((int)m) - 1;
+            i64 w0 = 0, w1 = 0;
+            bool ok = live;
+            if (slot == kSlotAdd) { w0 = t0 - v.x; w1 = t1 - v.y; }
+            else if (slot == kSlotSub) {                  // L - R = t
+                if (ir) { w0 = (i64)v.x - t0; w1 = (i64)v.y - t1; } else { w0 = t0 + v.x; w1 = t1 + v.y; }
+            } else {                                      // (the plan leaves products to the tiles where a target is zero)
+                ok = ok && v.x != 0 && v.y != 0 && t0 % (v.x ? v.x : 1) == 0 && t1 % (v.y ? v.y : 1) == 0;
+                if (ok) { w0 = t0 / v.x; w1 = t1 / v.y; }
+            }
+            ok = ok && w0 > -(i64)lim && w0 < (i64)lim && w1 > -(i64)lim && w1 < (i64)lim;
+            n.tests += (u64)__popc(__ballot_sync(0xffffffffu, live));
+            const int2 want = make_int2((i32)w0, (i32)w1);
+            u32 y = ok ? seg.head[pair_slot(want, seg.head_mask)] : 0xffffffffu;
+            while (__any_sync(0xffffffffu, y != 0xffffffffu)) {
+                bool hit = false;
+                u32 at = 0;
+                if (y != 0xffffffffu) {
+                    const int2 q = Y[y];
+                    hit = q.x == want.x && q.y == want.y;
+                    at = y;
+                    y = seg.next[y];
+                }
+                pair_push(w, plan, seg, sk, hole, hit, ir ? x : at, ir ? at : x, slot, from, n);
+            }
+        }
+    }
+    if (w.nc) pair_check(w, plan, seg, sk, hole, from, n);
+    if (blockIdx.x == 0 && threadIdx.x == 0) n.cands += (u64)seg.nl * seg.nr * (u64)__popc(seg.ops);
+    join_flush(plan, seg.acc, n);
+}
+
+// ---- / and % ----
+
+// Bucket of a magnitude below 2^31: exponent and five bits below the leading one (0 for 0).
+__device__ __forceinline__ u32 pair_bucket(u32 u) {
+    if (u == 0u) return 0u;
+    const int e = 31 - __clz((int)u);
+    const u32 frac = e >= 5 ? (u >> (e - 5)) & 31u : (u << (5 - e)) & 31u;
+    return 1u + (u32)e * 32u + frac;
+}
+constexpr int kPairBuckets = 1024;
+
+__global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const PlanDev plan, int index) {
+    __shared__ u32 hist[kPairBuckets];
+    const PairSeg& seg = plan.psegs[index];
+    const int side = blockIdx.y;
+    const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
+    const u32 n = side ? seg.nr : seg.nl, lim = pair_limit(hole);
+    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la];
+    for (int b = threadIdx.x; b < kPairBuckets; b += kPairThreads) hist[b] = 0;
+    __syncthreads();
+    for (u32 i = blockIdx.x * kPairThreads + threadIdx.x; i < n; i += gridDim.x * kPairThreads) {
+        int2 v;
+        if (pair_entry(hole, off, i, lim, v) == 1) atomicAdd(&hist[pair_bucket(abs_u32(v.x))], 1u);
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < kPairBuckets; b += kPairThreads) if (hist[b]) atomicAdd(&seg.hist[side][b], hist[b]);
+}
+
+// One CTA per side: bucket starts (start[kPairBuckets] = entries), and the cursors of the scatter.
+__global__ void __launch_bounds__(kPairBuckets) pair_sort_scan_kernel(const PlanDev plan, int index) {
+    __shared__ u32 part[kPairBuckets];
+    const PairSeg& seg = plan.psegs[index];
+    const int side = blockIdx.x, t = threadIdx.x;
+    const u32 mine = seg.hist[side][t];
+    part[t] = mine;
+    __syncthreads();
+    for (int d = 1; d < kPairBuckets; d <<= 1) {
+        const u32 v = t >= d ? part[t - d] : 0u;
+        __syncthreads();
+        part[t] += v;
+        __syncthreads();
+    }
+    seg.start[side][t] = part[t] - mine;
+    seg.hist[side][t] = part[t] - mine;
+    if (t == kPairBuckets - 1) seg.start[side][kPairBuckets] = part[t];
+}
+
+__global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const PlanDev plan, int index) {
+    const PairSeg& seg = plan.psegs[index];
+    const int side = blockIdx.y, lane = threadIdx.x & 31;
+    const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
+    const u32 n = side ? seg.nr : seg.nl, lim = pair_limit(hole);
+    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la];
+    for (u32 i0 = (blockIdx.x * kPairThreads + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * kPairThreads) {
+        const u32 i = i0 + lane;
+        int2 v = make_int2(0, 0);
+        const bool on = i < n && pair_entry(hole, off, i, lim, v) == 1;
+        const u32 b = on ? pair_bucket(abs_u32(v.x)) : 0xffffffffu;
+        const u32 same = __match_any_sync(0xffffffffu, b);          // one atomic per bucket and warp
+        const int leader = __ffs((int)same) - 1;
+        u32 at = 0;
+        if (on && lane == leader) at = atomicAdd(&seg.hist[side][b], (u32)__popc(same));
+        at = __shfl_sync(0xffffffffu, at, leader) + (u32)__popc(same & ((1u << lane) - 1u));
+        if (!on) continue;
+        seg.id[side][at] = i;
+        seg.val[side][at] = v;
+    }
+}
+
+// First sorted position whose bucket is at least that of magnitude u, and one past the last whose bucket is at most that.
+__device__ __forceinline__ u32 pair_from(const PairSeg& seg, u64 u) { return seg.start[1][u >> 31 ? kPairBuckets : pair_bucket((u32)u)]; }
+__device__ __forceinline__ u32 pair_to(const PairSeg& seg, u64 u) { return seg.start[1][u >> 31 ? kPairBuckets : pair_bucket((u32)u) + 1u]; }
+
+// A ticket: 32 dividends in magnitude order and one piece of the divisors that they may meet.
+__global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const PlanDev plan, int index) {
+    __shared__ PairWarp sh[kPairWarps];
+    PairWarp& w = sh[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) w.nc = 0;
+    __syncwarp();
+    const PairSeg& seg = plan.psegs[index];
+    const SketchDev* sk = plan.sketches[seg.sketch];
+    const HoleDev* hole = &sk->holes[seg.hole];
+    JoinCount n{0, 0, 0, 0, 0};
+    const i64 t0 = hole->join_t0, t1 = hole->join_t1;
+    const u64 m0 = (u64)(t0 < 0 ? -t0 : t0), m1 = (u64)(t1 < 0 ? -t1 : t1);
+    const int from = hole->join_p1 ? 2 : 1;
+    const bool small = ((m0 | m1) >> 31) == 0 && !hole->join_none;      // (otherwise no narrow quotient or remainder is the target)
+    const u32 u0t = (u32)m0, u1t = (u32)m1;
+    const u32 nl = seg.start[0][kPairBuckets], nr = seg.start[1][kPairBuckets];
+    const u32 blocks = (nl + 31u) / 32u, pieces = seg.pieces;
+    const u64 tickets = small ? (u64)blocks * pieces : 0ull;
+    for (;;) {
+        u64 t = 0;
+        if (lane == 0) t = atomicAdd((unsigned long long*)seg.ticket, 1ull);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= tickets) break;
+        const u32 block = blocks - 1u - (u32)(t / pieces), piece = (u32)(t % pieces);      // the largest dividends meet the most divisors: first
+        const u32 li = block * 32u + lane;
+        const bool live = li < nl;
+        const int2 lv = live ? seg.val[0][li] : make_int2(0, 0);
+        const u32 lid = live ? seg.id[0][li] : 0u;
+        const u32 a0 = abs_u32(lv.x), a1 = abs_u32(lv.y);
+        const u32 amin = __reduce_min_sync(0xffffffffu, live ? a0 : 0xffffffffu), amax = __reduce_max_sync(0xffffffffu, a0);
+        for (int which = 0; which < 2; ++which) {
+            if (!((seg.ops >> (which ? kSlotMod : kSlotDiv)) & 1u)) continue;
+            u32 lo, hi;
+            if (which == 0) {                             // quotient
+                lo = pair_from(seg, (u64)amin / (m0 + 1) + 1);
+                hi = m0 ? pair_to(seg, (u64)amax / m0) : nr;
+            } else {                                      // remainder
+                if (amax < u0t) continue;                 // (a remainder is at most its dividend)
+                lo = pair_from(seg, m0 + 1);
+                const bool self = __any_sync(0xffffffffu, live && a0 == u0t);
+                hi = self ? nr : pair_to(seg, (u64)amax - m0);
+            }
+            if (lo >= hi) continue;
+            const u32 len = hi - lo, p0 = lo + (u32)((u64)len * piece / pieces), p1 = lo + (u32)((u64)len * (piece + 1) / pieces);
+            n.tests += (u64)(p1 - p0) * (u64)__popc(__ballot_sync(0xffffffffu, live));
+            const u32 x0 = a0 >= u0t ? a0 - u0t : 1u;
+            const bool can = live && (which == 0 || (a0 >= u0t && a1 >= u1t));
+            for (u32 r0 = p0; r0 < p1; r0 += 32u) {
+                // lanes fetch 32 divisors (and prepare them); all lanes then meet each of them
+                const u32 k = r0 + lane < p1 ? r0 + lane : p1 - 1u;
+                const int2 rv = seg.val[1][k];
+                const u32 b0 = abs_u32(rv.x), b1 = abs_u32(rv.y);
+                u32 q0 = 0, q1 = 0, q2 = 0;
+                if (which == 0) { q0 = u0t * b0; q1 = ((u64)u0t * b0) >> 31 ? 0u : 1u; }
+                else if (b0 > u0t && b1 > u1t) {
+                    const u32 kk = (u32)__ffs((int)b0) - 1u;
+                    q0 = inv_odd(b0 >> kk); q1 = 0xffffffffu / b0; q2 = kk;
+                }
+                const int m = p1 - r0 < 32u ? (int)(p1 - r0) : 32;
+                u32 hits = 0;                             // bit s: this lane's dividend meets divisor s at the first probe
+                if (which == 0) {
+                    for (int s = 0; s < m; ++s) {
+                        const u32 bb = __shfl_sync(0xffffffffu, b0, s), lw = __shfl_sync(0xffffffffu, q0, s), fit = __shfl_sync(0xffffffffu, q1, s);
+                        hits |= (u32)(a0 - lw < bb && fit != 0u) << s;
+                    }
+                } else {
+                    for (int s = 0; s < m; ++s) {
+                        const u32 iv = __shfl_sync(0xffffffffu, q0, s), cm = __shfl_sync(0xffffffffu, q1, s), kk = __shfl_sync(0xffffffffu, q2, s);
+                        hits |= (u32)(rotr32(x0 * iv, kk) <= cm && cm != 0u) << s;
+                    }
+                }
+                if (!can) hits = 0;
+                while (__any_sync(0xffffffffu, hits != 0u)) {
+                    const int s = hits ? __ffs((int)hits) - 1 : 0;
+                    const i32 d0 = __shfl_sync(0xffffffffu, rv.x, s), d1 = __shfl_sync(0xffffffffu, rv.y, s);
+                    bool on = hits != 0u && d0 != 0 && d1 != 0;
+                    hits &= hits - 1;
+                    if (on) {                             // exactly, at both probes
+                        i64 v0, v1;
+                        on = narrow_op(which ? kSlotMod : kSlotDiv, lv.x, d0, v0) && v0 == t0 && narrow_op(which ? kSlotMod : kSlotDiv, lv.y, d1, v1) && v1 == t1;
+                    }
+                    pair_push(w, plan, seg, sk, hole, on, lid, on ? seg.id[1][r0 + (u32)s] : 0u, which ? kSlotMod : kSlotDiv, from, n);
+                }
+            }
+        }
+    }
+    if (w.nc) pair_check(w, plan, seg, sk, hole, from, n);
+    join_flush(plan, seg.acc, n);
+}
+
+// Wide operands: each against the whole other set, lanes over it, from the first probe on, exactly.
+__global__ void __launch_bounds__(kPairThreads) pair_wide_kernel(const PlanDev plan, int index) {
+    __shared__ PairWarp sh[kPairWarps];
+    PairWarp& w = sh[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) w.nc = 0;
+    __syncwarp();
+    const PairSeg& seg = plan.psegs[index];
+    const u32 wl = seg.counters[0], wr = seg.counters[1];
+    if (wl + wr == 0u) return;
+    const SketchDev* sk = plan.sketches[seg.sketch];
+    const HoleDev* hole = &sk->holes[seg.hole];
+    const u32 lim = pair_limit(hole);
+    const u64 lo = hole->tab_off[seg.lnt][seg.la], ro = hole->tab_off[seg.rnt][seg.ra];
+    JoinCount n{0, 0, 0, 0, 0};
+    const u64 nl = wl, total = nl + wr;
+    for (u64 i = blockIdx.x * kPairWarps + (threadIdx.x >> 5); i < total; i += (u64)gridDim.x * kPairWarps) {
+        const bool left = i < nl;
+        const u32 x = left ? seg.wide_l[i] : seg.wide_r[i - nl];
+        if (!hole->tab_ok[(left ? lo : ro) + x]) continue;
+        const i64 xv = hole->tab_val[(left ? lo : ro) + x];
+        const u32 m = left ? seg.nr : seg.nl;
+        for (u32 y0 = 0; y0 < m; y0 += 32u) {
+            const u32 y = y0 + lane;
+            bool on = y < m && hole->tab_ok[(left ? ro : lo) + y] != 0;
+            if (on && !left) { int2 v; on = pair_entry(hole, lo, y, lim, v) == 1; }      // (two wide operands: the left one's turn)
+            const i64 yv = on ? hole->tab_val[(left ? ro : lo) + y] : 0;
+            for (u32 o = seg.ops; o; o &= o - 1) {
+                const int slot = __ffs((int)o) - 1;
+                i64 v;
+                n.tests += (u64)__popc(__ballot_sync(0xffffffffu, on));
+                const bool hit = on && apply_op(op_of_slot(slot), left ? xv : yv, left ? yv : xv, v) && probe_accepts(hole, 0, v);
+                pair_push(w, plan, seg, sk, hole, hit, left ? x : y, left ? y : x, slot, 1, n);
+            }
+        }
+    }
+    if (w.nc) pair_check(w, plan, seg, sk, hole, 1, n);
+    join_flush(plan, seg.acc, n);
+}
+
+}  // namespace xp
