@@ -36,11 +36,39 @@ struct GroupCtx {
     i32 cmin, cmax;
     u32 cabs, mm;
     float fc;
-    i32 n_entries, tests;                                 // tests: what an operand counts for in filter_tests
+    i32 n_entries;
     const JoinSet* set;
 };
 
+// What the conditions need of the hole.
+struct JoinCtx {
+    u32 t0, t1, ut0, ut1;                                 // targets (low words) and their magnitudes (0 where 31 bits do not hold them)
+    float rt0, rt1, rl0, rl1, h0, h1, ft0, ft1;           // 1/|t|, 1/(|t|+1), huge where t = 0, |t|
+    u32 tmod;
+    bool tz, small;                                       // both targets are zero; both are below 2^31
+};
+
+// The entries of all groups as the hot loop tests them (an operand that passes a test of any group is a suspect): sums,
+// differences and products share one comparison each of a mixed pair, three comparisons per variable instead of ten.
+constexpr int kJoinLin = 3 * kJoinEntries * 2;            // most wanted pairs kept (more: the exact form)
+constexpr u32 kPairMix = 0x9E3779B1u;                     // a pair (x, y) is compared as x + kPairMix * y
+struct __align__(16) JoinHot {
+    u32 lin[kJoinLin + 4];                                // a + v, a - v, v - a: the pair that a has to be, mixed
+    u32 mul0[kJoinEntries], mul1[kJoinEntries];           // a * v: a0 * mul0 + a1 * mul1 has to be mul_t
+    u32 mul_t;
+    i32 n_lin, n_mul, n_other, n_set;
+    const JoinEntry* other[kJoinEntries];                 // entries under / % min max, with their operators
+    u32 other_f[kJoinEntries], other_s[kJoinEntries];
+    i32 set[kJoinGroups];                                 // groups whose constants have a condition
+    u32 lim;                                              // operand limit of the segment (0: some leaf set goes the exact way)
+    u32 tests;                                            // what an operand counts for in filter_tests
+    u64 pairs;                                            // candidates per operand
+};
+
 struct JoinWarp {
+    JoinHot hot;
+    JoinCtx x;
+    i32 seg;                                              // segment that grp, x and hot are filled for (-1: none)
     u32 q_off[kJoinQueue];                                // suspects: operand number relative to the segment's first,
     i32 q_a0[kJoinQueue], q_a1[kJoinQueue];               //   its values at the two probes
     u32 c_off[64], c_pos[64], c_code[64];                 // candidates: operand, leaf position, group << 8 | slot << 1 | swapped
@@ -208,13 +236,6 @@ __device__ __forceinline__ void join_push(JoinWarp& w, const PlanDev& plan, cons
 
 // ---- the conditions ----
 
-struct JoinCtx {                                          // what the conditions need of the hole
-    u32 t0, t1, ut0, ut1;                                 // targets (low words) and their magnitudes (0 where 31 bits do not hold them)
-    float rt0, rt1, rl0, rl1, h0, h1, ft0, ft1;           // 1/|t|, 1/(|t|+1), huge where t = 0, |t|
-    u32 tmod;
-    bool tz, small;                                       // both targets are zero; both are below 2^31
-};
-
 __device__ __forceinline__ bool in_range(u32 c, const GroupCtx& s) { return c - (u32)s.cmin <= (u32)s.cmax - (u32)s.cmin; }
 
 // a * c = t at both probes for some c, given that a0 * t1 = a1 * t0: the operand divides the target.
@@ -239,7 +260,8 @@ __device__ __noinline__ bool gcd_exceeds(u32 x, u32 y, u32 least) {      // gcd(
 __device__ __noinline__ bool residue_exists(u32 u0, u32 u1, u32 ut0, u32 ut1, u32 cabs) {
     if (u0 <= ut0 || u1 <= ut1) return false;
     if (u0 < u1) { u32 s = u0; u0 = u1; u1 = s; s = ut0; ut0 = ut1; ut1 = s; }
-    for (u64 m = ut0; m <= cabs; m += u0) if ((u32)m % u1 == ut1) return true;
+    u32 steps = u1;                                       // (the residues repeat after u1 steps)
+    for (u64 m = ut0; m <= cabs && steps > 0u; m += u0, --steps) if ((u32)m % u1 == ut1) return true;
     return false;
 }
 
@@ -342,27 +364,47 @@ __device__ __forceinline__ void entry_conditions(const JoinEntry& e, u32 f, u32 
     }
 }
 
-// The constants of a group as a set.
-template <int P>
+// The constants of a group as a set.  CF, CS: the operators, known at compile time for the usual groups (-1: taken from s).
+template <int P, int CF, int CS>
 __device__ __forceinline__ void set_conditions(const GroupCtx& s, const i32 (&a0)[P], const i32 (&a1)[P], const JoinCtx& x, bool (&any)[P]) {
-    const u32 cf = s.cf, cs = s.cs;
+    const u32 cf = CF < 0 ? s.cf : (u32)CF, cs = CS < 0 ? s.cs : (u32)CS;
     if ((cf | cs) & ((1u << kSlotAdd) | (1u << kSlotSub))) {
-        const u32 dt = x.t0 - x.t1;
+        const u32 dt = x.t0 - x.t1, nt = 0u - dt;
+        const bool rsub = (cs >> kSlotSub) & 1u;
+        bool maybe = false;
 #pragma unroll
         for (int p = 0; p < P; ++p) {
             const u32 d = (u32)a0[p] - (u32)a1[p];
-            if (d == dt) {                                // (rarely: most operands part here)
-                if ((cf | cs) & (1u << kSlotAdd)) any[p] |= in_range(x.t0 - (u32)a0[p], s);
-                if (cf & (1u << kSlotSub)) any[p] |= in_range((u32)a0[p] - x.t0, s);
+            maybe |= d == dt || (rsub && d == nt);
+        }
+        if (maybe) {                                      // (rarely: an operand mostly differs otherwise than the target does)
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const u32 d = (u32)a0[p] - (u32)a1[p];
+                bool h = false;
+                if ((cf | cs) & (1u << kSlotAdd)) h |= d == dt && in_range(x.t0 - (u32)a0[p], s);
+                if (cf & (1u << kSlotSub)) h |= d == dt && in_range((u32)a0[p] - x.t0, s);
+                if (rsub) h |= d == nt && in_range(x.t0 + (u32)a0[p], s);
+                any[p] |= h;
             }
-            if ((cs & (1u << kSlotSub)) && d == 0u - dt) any[p] |= in_range(x.t0 + (u32)a0[p], s);
         }
     }
     if ((cf | cs) & (1u << kSlotMul)) {
-        const u32 cabs = s.cabs;
+        bool maybe = false;
 #pragma unroll
-        for (int p = 0; p < P; ++p)
-            if ((u32)a0[p] * x.t1 == (u32)a1[p] * x.t0 && ((a0[p] | a1[p]) != 0 || x.tz)) any[p] |= factor_exists(a0[p], a1[p], x, cabs);
+        for (int p = 0; p < P; ++p) maybe |= (u32)a0[p] * x.t1 == (u32)a1[p] * x.t0;
+        if (maybe) {
+            const u32 cabs = s.cabs;
+#pragma unroll 1
+            for (int p = 0; p < P; ++p) {
+                i32 v0 = a0[0], v1 = a1[0];
+#pragma unroll
+                for (int k = 1; k < P; ++k) if (k == p) { v0 = a0[k]; v1 = a1[k]; }
+                const bool h = (u32)v0 * x.t1 == (u32)v1 * x.t0 && ((v0 | v1) != 0 || x.tz) && factor_exists(v0, v1, x, cabs);
+#pragma unroll
+                for (int k = 0; k < P; ++k) any[k] |= h && k == p;
+            }
+        }
     }
     if ((cf | cs) & (1u << kSlotDiv)) {
         const float fc = s.fc;
@@ -373,18 +415,20 @@ __device__ __forceinline__ void set_conditions(const GroupCtx& s, const i32 (&a0
             if (cs & (1u << kSlotDiv)) any[p] |= const_div_swap(f0, f1, x, fc);
         }
     }
-    if (cf & (1u << kSlotMod)) {
-#pragma unroll 1
-        for (int p = 0; p < P; ++p) {
-            const u32 u0 = abs_u32(a0[p]), u1 = abs_u32(a1[p]);
-            if (!any[p] && u0 >= x.ut0 && u1 >= x.ut1) any[p] |= gcd_exceeds(u0 - x.ut0, u1 - x.ut1, x.tmod);
-        }
-    }
-    if (cs & (1u << kSlotMod)) {
+    if ((cf | cs) & (1u << kSlotMod)) {
         const u32 cabs = s.cabs;
 #pragma unroll 1
-        for (int p = 0; p < P; ++p)
-            if (!any[p]) any[p] |= residue_exists(abs_u32(a0[p]), abs_u32(a1[p]), x.ut0, x.ut1, cabs);
+        for (int p = 0; p < P; ++p) {
+            i32 v0 = a0[0], v1 = a1[0];
+            bool h = any[0];
+#pragma unroll
+            for (int k = 1; k < P; ++k) if (k == p) { v0 = a0[k]; v1 = a1[k]; h = any[k]; }
+            const u32 u0 = abs_u32(v0), u1 = abs_u32(v1);
+            if (!h && (cf & (1u << kSlotMod)) && u0 >= x.ut0 && u1 >= x.ut1) h = gcd_exceeds(u0 - x.ut0, u1 - x.ut1, x.tmod);
+            if (!h && (cs & (1u << kSlotMod))) h = residue_exists(u0, u1, x.ut0, x.ut1, cabs);
+#pragma unroll
+            for (int k = 0; k < P; ++k) any[k] |= h && k == p;
+        }
     }
     if ((cf | cs) & (1u << kSlotMn)) {
 #pragma unroll
@@ -614,13 +658,14 @@ __device__ __forceinline__ void pair_op(const int2 (&x)[P], const int2 (&y)[P], 
             a1[p] = OP == XP_OP_DIV ? q1 : x[p].y - q1 * d1;
         } else if (OP == XP_OP_MIN) { a0[p] = min(x[p].x, y[p].x); a1[p] = min(x[p].y, y[p].y); }
         else if (OP == XP_OP_MAX) { a0[p] = max(x[p].x, y[p].x); a1[p] = max(x[p].y, y[p].y); }
-        else {
-            i64 r0, r1;
-            if (OP == XP_OP_ADD) { r0 = (i64)x[p].x + y[p].x; r1 = (i64)x[p].y + y[p].y; }
-            else if (OP == XP_OP_SUB) { r0 = (i64)x[p].x - y[p].x; r1 = (i64)x[p].y - y[p].y; }
-            else { r0 = (i64)x[p].x * y[p].x; r1 = (i64)x[p].y * y[p].y; }
+        else if (OP == XP_OP_MUL) {
+            const i64 r0 = (i64)x[p].x * y[p].x, r1 = (i64)x[p].y * y[p].y;
             a0[p] = (i32)r0; a1[p] = (i32)r1;
-            if (!narrow31(r0) || !narrow31(r1)) wide |= 1u << p;
+            if ((i32)(r0 >> 32) != (a0[p] >> 31) || (i32)(r1 >> 32) != (a1[p] >> 31)) wide |= 1u << p;
+        } else {                                          // (-2^31 itself is left to the operand limit)
+            const i32 b0 = OP == XP_OP_ADD ? y[p].x : -y[p].x, b1 = OP == XP_OP_ADD ? y[p].y : -y[p].y;
+            a0[p] = (i32)((u32)x[p].x + (u32)b0); a1[p] = (i32)((u32)x[p].y + (u32)b1);
+            if ((((x[p].x ^ a0[p]) & (b0 ^ a0[p])) | ((x[p].y ^ a1[p]) & (b1 ^ a1[p]))) < 0) wide |= 1u << p;
         }
     }
 }
@@ -705,42 +750,10 @@ __device__ __forceinline__ void join_flush(const PlanDev& plan, int acc, JoinCou
     n = JoinCount{0, 0, 0, 0, 0};
 }
 
-// Fills the warp's group contexts for a segment; returns the operand limit, 0 when some leaf set has to go the exact way.
-__device__ __noinline__ u32 join_groups(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const HoleDev* hole, const JoinCtx& x) {
+// Fills what the warp's loops need of a segment: targets, groups and the merged tests.
+__device__ __noinline__ void join_fill(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const GrammarDev* g, const HoleDev* hole) {
     const int lane = threadIdx.x & 31;
-    u32 lim = 0x7fffffffu;
     __syncwarp();
-    if (lane < seg.n_groups) {
-        const JoinGroup& grp = plan.jgroups[seg.first_group + lane];
-        const JoinSet* S = &hole->join_sets[grp.leaf_nt];
-        GroupCtx c;
-        c.set = S;
-        c.cmin = S->cmin; c.cmax = S->cmax; c.cabs = S->cabs; c.mm = S->mm; c.fc = (float)S->cabs; c.n_entries = S->n_entries;
-        c.tests = (S->n_entries + (S->n_const > 0 ? 1 : 0)) * (__popc(grp.fmask) + __popc(grp.smask));
-        u32 cf = grp.fmask, cs = grp.smask, ef = cf, es = cs;
-        // operators that cannot reach the target: quotients, remainders, minima and maxima of narrow operands are narrow;
-        // a remainder is below its divisor; c / a and c % a are at most |c|
-        constexpr u32 kNarrow = (1u << kSlotDiv) | (1u << kSlotMod) | (1u << kSlotMn) | (1u << kSlotMx);
-        if (!x.small) { cf &= ~kNarrow; cs &= ~kNarrow; ef &= ~kNarrow; es &= ~kNarrow; }
-        if (x.tmod >= S->cabs) cf &= ~(1u << kSlotMod);
-        if (x.tmod > S->cabs) cs &= ~((1u << kSlotDiv) | (1u << kSlotMod));
-        if (S->n_const == 0) cf = cs = 0;
-        if (S->n_entries == 0) ef = es = 0;
-        if (hole->join_none) cf = cs = ef = es = 0;
-        c.cf = cf; c.cs = cs; c.ef = ef; c.es = es;
-        w.grp[lane] = c;
-        lim = S->ok ? S->lim : 0u;
-    }
-    __syncwarp();
-    return __reduce_min_sync(0xffffffffu, lim);
-}
-
-// Operands [first, first + count) of a segment against the leaves (count <= the segment's chunk).
-template <int P>
-__device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
-                                         u64 first, u64 count, JoinCount& n) {
-    const GrammarDev* g = sk->g;
-    const int lane = threadIdx.x & 31;
     JoinCtx x;
     {
         const i64 t0 = hole->join_t0, t1 = hole->join_t1;
@@ -753,21 +766,95 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
         x.tmod = tm < 0xffffffffull ? (u32)tm : 0xffffffffu;
         x.tz = (t0 | t1) == 0;
     }
-    const u32 lim = join_groups(w, plan, seg, hole, x);
-    u32 tests_each = 0;
-    {
-        u64 pairs = 0;
-        for (int gi = 0; gi < seg.n_groups; ++gi) {
-            const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
-            pairs += g->cnt[grp.leaf_nt][1] * (u64)(__popc(grp.fmask) + __popc(grp.smask));
-            tests_each += (u32)w.grp[gi].tests;
+    u32 lim = 0x7fffffffu, tests = 0;
+    u64 pairs = 0;
+    i32 n_lin = 0, n_mul = 0, n_other = 0, n_set = 0;
+    constexpr u32 kNarrow = (1u << kSlotDiv) | (1u << kSlotMod) | (1u << kSlotMn) | (1u << kSlotMx);
+    for (int gi = 0; gi < seg.n_groups; ++gi) {
+        const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+        const JoinSet* S = &hole->join_sets[grp.leaf_nt];
+        const u32 cabs = S->cabs;
+        const int n_entries = S->n_entries, n_const = S->n_const;
+        const int n_ops = __popc(grp.fmask) + __popc(grp.smask);
+        tests += (u32)((n_entries + (n_const > 0 ? 1 : 0)) * n_ops);
+        pairs += g->cnt[grp.leaf_nt][1] * (u64)n_ops;
+        u32 cf = grp.fmask, cs = grp.smask, ef = cf, es = cs;
+        // operators that cannot reach the target: quotients, remainders, minima and maxima of narrow operands are narrow;
+        // a remainder is below its divisor; c / a and c % a are at most |c|
+        if (!x.small) { cf &= ~kNarrow; cs &= ~kNarrow; ef &= ~kNarrow; es &= ~kNarrow; }
+        if (x.tmod >= cabs) cf &= ~(1u << kSlotMod);
+        if (x.tmod > cabs) cs &= ~((1u << kSlotDiv) | (1u << kSlotMod));
+        if (n_const == 0) cf = cs = 0;
+        if (n_entries == 0) ef = es = 0;
+        if (hole->join_none) cf = cs = ef = es = 0;
+        const u32 slim = S->ok ? S->lim : 0u;
+        lim = slim < lim ? slim : lim;
+        if (lane == 0) {
+            GroupCtx c;
+            c.set = S;
+            c.cmin = S->cmin; c.cmax = S->cmax; c.cabs = cabs; c.mm = S->mm; c.fc = (float)cabs; c.n_entries = n_entries;
+            c.cf = cf; c.cs = cs; c.ef = ef; c.es = es;
+            w.grp[gi] = c;
+            if (cf | cs) w.hot.set[n_set] = gi;
         }
-        n.cands += count * pairs;
+        n_set += (cf | cs) != 0u;
+        const bool on = lane < n_entries && (ef | es) != 0u;
+        JoinEntry e;
+        if (on) e = S->e[lane];
+        const u32 below = (1u << lane) - 1u;
+        const int others = __popc(__ballot_sync(0xffffffffu, on && ((ef | es) & kNarrow)));
+        for (int k = 0; k < 3; ++k) {                     // a + v, a - v, v - a
+            const bool want = on && (k == 0 ? ((ef | es) >> kSlotAdd) & 1u : k == 1 ? (ef >> kSlotSub) & 1u : (es >> kSlotSub) & 1u);
+            const u32 b = __ballot_sync(0xffffffffu, want);
+            const int at = n_lin + __popc(b & below);
+            if (want && at < kJoinLin) {
+                const u32 d0 = k == 0 ? x.t0 - e.v0 : k == 1 ? x.t0 + e.v0 : e.v0 - x.t0, d1 = k == 0 ? x.t1 - e.v1 : k == 1 ? x.t1 + e.v1 : e.v1 - x.t1;
+                w.hot.lin[at] = d0 + kPairMix * d1;
+            }
+            n_lin += __popc(b);
+        }
+        {
+            const bool want = on && (((ef | es) >> kSlotMul) & 1u);
+            const u32 b = __ballot_sync(0xffffffffu, want);
+            const int at = n_mul + __popc(b & below);
+            if (want && at < kJoinEntries) { w.hot.mul0[at] = e.v0; w.hot.mul1[at] = kPairMix * e.v1; }
+            n_mul += __popc(b);
+        }
+        if (others) {
+            const int at = n_other + lane;
+            if (on && at < kJoinEntries) { w.hot.other[at] = &S->e[lane]; w.hot.other_f[at] = ef & kNarrow; w.hot.other_s[at] = es & kNarrow; }
+            n_other += others;
+        }
     }
+    __syncwarp();
+    // (more entries than the lists hold: the exact way)
+    if (n_lin > kJoinLin || n_mul > kJoinEntries || n_other > kJoinEntries) lim = 0u;
+    else if (lane < 4 && n_lin > 0) w.hot.lin[n_lin + lane] = w.hot.lin[0];
+    if (lane == 0) {
+        w.x = x;
+        w.hot.mul_t = x.t0 + kPairMix * x.t1;
+        w.hot.n_lin = n_lin; w.hot.n_mul = n_mul; w.hot.n_other = n_other; w.hot.n_set = n_set;
+        w.hot.lim = lim; w.hot.tests = tests; w.hot.pairs = pairs;
+    }
+    __syncwarp();
+}
+
+// Operands [first, first + count) of a segment against the leaves (count <= the segment's chunk).
+template <int P>
+__device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
+                                         u64 first, u64 count, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    n.cands += count * w.hot.pairs;
+    const u32 lim = w.hot.lim;
     if (seg.exact || !hole->join_on || lim == 0u) {
         for (u64 i = 0; i < count; ++i) join_exact(w, plan, seg, sk, hole, first + i, n);
         return;
     }
+    const JoinCtx x = w.x;
+    const int n_lin = w.hot.n_lin, n_mul = w.hot.n_mul, n_other = w.hot.n_other, n_set = w.hot.n_set;
+    const u32 mul_t = w.hot.mul_t;
+    const u32 tests_each = w.hot.tests;
     u32 nq = 0;
     u32 n_alive = 0;
     for (u64 done = 0; done < count;) {
@@ -785,17 +872,36 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
                 if (((alive >> p) & 1u) && (abs_u32(a0[p]) >= lim || abs_u32(a1[p]) >= lim)) { alive &= ~(1u << p); wide |= 1u << p; }
             }
             n_alive += (u32)__popc(alive);
-            for (int gi = 0; gi < seg.n_groups; ++gi) {
-                const GroupCtx& s = w.grp[gi];
-                if (s.cf | s.cs) set_conditions<P>(s, a0, a1, x, any);
-                const u32 ef = s.ef, es = s.es;
-                if (ef | es) {
-                    const JoinEntry* e = s.set->e;
-                    for (int i = 0; i < s.n_entries; ++i) {
-                        const JoinEntry en = e[i];
-                        entry_conditions<P>(en, ef, es, a0, a1, x, any);
-                    }
+            if (n_lin > 0) {
+                u32 h[P];
+#pragma unroll
+                for (int p = 0; p < P; ++p) h[p] = (u32)a0[p] + kPairMix * (u32)a1[p];
+                for (int i = 0; i < n_lin; i += 4) {
+                    const uint4 d = *reinterpret_cast<const uint4*>(&w.hot.lin[i]);
+#pragma unroll
+                    for (int p = 0; p < P; ++p) any[p] |= h[p] == d.x || h[p] == d.y || h[p] == d.z || h[p] == d.w;
                 }
+            }
+            for (int i = 0; i < n_mul; ++i) {
+                const u32 v0 = w.hot.mul0[i], v1 = w.hot.mul1[i];
+#pragma unroll
+                for (int p = 0; p < P; ++p) any[p] |= (u32)a0[p] * v0 + (u32)a1[p] * v1 == mul_t;
+            }
+            for (int i = 0; i < n_other; ++i) {
+                const JoinEntry en = *w.hot.other[i];
+                const u32 f = w.hot.other_f[i], s = w.hot.other_s[i];
+                constexpr u32 kDivMod = (1u << kSlotDiv) | (1u << kSlotMod);
+                if (f == kDivMod && s == kDivMod) entry_conditions<P>(en, kDivMod, kDivMod, a0, a1, x, any);      // (compile-time operators)
+                else entry_conditions<P>(en, f, s, a0, a1, x, any);
+            }
+            for (int i = 0; i < n_set; ++i) {
+                const GroupCtx& s = w.grp[w.hot.set[i]];
+                const u32 cf = s.cf, cs = s.cs;
+                constexpr u32 kRing = (1u << kSlotAdd) | (1u << kSlotSub) | (1u << kSlotMul), kDiv = 1u << kSlotDiv, kMul = 1u << kSlotMul;
+                if (cf == kMul && cs == 0u) set_conditions<P, (int)kMul, 0>(s, a0, a1, x, any);
+                else if (cf == kDiv && cs == 0u) set_conditions<P, (int)kDiv, 0>(s, a0, a1, x, any);
+                else if (cf == (kRing | kDiv) && cs == kRing) set_conditions<P, (int)(kRing | kDiv), (int)kRing>(s, a0, a1, x, any);
+                else set_conditions<P, -1, -1>(s, a0, a1, x, any);
             }
             u32 hits = 0;
 #pragma unroll
@@ -991,7 +1097,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const PlanDev pla
     __shared__ JoinWarp sh[kJoinWarps];
     JoinWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    if (lane == 0) w.nc = 0;
+    if (lane == 0) { w.nc = 0; w.seg = -1; }
     __syncwarp();
     JoinCount n{0, 0, 0, 0, 0};
     int acc = -1;
@@ -1015,6 +1121,11 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const PlanDev pla
         if (seg.acc != acc) { join_flush(plan, acc, n); acc = seg.acc; }
         const SketchDev* sk = plan.sketches[seg.sketch];
         const HoleDev* hole = &sk->holes[seg.hole];
+        if (seg.kind == kJoinLeaf && (hole->aff_ok || seg.exact) && w.seg != lo) {
+            join_fill(w, plan, seg, sk->g, hole);
+            if (lane == 0) w.seg = lo;
+            __syncwarp();
+        }
         const u32 all = hole->n_probe >= 32 ? 0xffffffffu : (1u << hole->n_probe) - 1u;
         const u64 chunk = seg.chunk, from = (t - seg.first_ticket) * chunk;
         if ((hole->probe_spec_ok & all) == all && from < seg.e_count) {      // (a spec undefined at a probe: nothing can match)
