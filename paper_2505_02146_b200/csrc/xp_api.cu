@@ -1585,6 +1585,7 @@ static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size
         for (const HoleHost& h : sk[i]->holes) if (h.second) w.dense = 1;      // (frequent filter hits)
     }
     w.max_chunks = (u32)((most + kVerifyChunk - 1) / kVerifyChunk);
+    w.first_points = (i32)(most < kVerifyChunk ? most : kVerifyChunk);
     return w;
 }
 

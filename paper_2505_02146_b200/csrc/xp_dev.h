@@ -275,7 +275,7 @@ struct SegDev {
 };
 
 // A candidate that passed every probe point and waits for the whole-domain check.  The check
-// is cut into chunks of kVerifyChunk points that any CTA may take; state counts the chunks
+// is cut into chunks of kVerifyChunk points (or pieces of one) that any CTA may take; state counts the pieces
 // that passed, its top bit says that some point failed.
 constexpr int kVerifyChunk = 4096;
 constexpr u32 kSurvFailed = 0x80000000u;
@@ -301,6 +301,7 @@ struct PlanDev {
     u64* verify_ticket;              // device counter, zero at launch
     u32 surv_cap;
     u32 max_chunks;                  // chunks of the largest domain among the sketches
+    i32 first_points;                // points of the first chunk: the largest domain's, at most kVerifyChunk
     u32* err;                        // device word for the checked build's index checks (0: none failed)
     // Survivors in hole order (null when the call has one hole): queued survivors per accumulator slot
     // (counted by eval_kernel), the slots' offsets (a scan of the counts) and, per slot side by side, the

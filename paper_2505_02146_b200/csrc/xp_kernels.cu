@@ -2505,11 +2505,11 @@ __device__ __forceinline__ void chunk_passed(const PlanDev& plan, SurvDev* sv, u
     atomicAdd(&a->match_count[sv->size], 1ull);
     atomicMin(&a->min_rank[sv->size], sv->rank);
 }
-__device__ __forceinline__ u32 chunks_of(i64 n_points) { return (u32)((n_points + kVerifyChunk - 1) / kVerifyChunk); }
+__device__ __forceinline__ u32 chunks_of(i64 n_points, i64 sub) { return (u32)((n_points + sub - 1) / sub); }
 
-// One survivor on one chunk, staged by the warp's first lane (boxes with their sub-box projection,
+// One survivor on the points first .. first + sub, staged by the warp's first lane (boxes with their sub-box projection,
 // programs that do not fit the arena, contexts that never mention the hole).
-__device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 si, u64 chunk) {
+__device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 si, i64 first, i64 sub) {
     const int lane = threadIdx.x & 31;
     CandShared& cand = w.s.cand;
     int skip = 1;
@@ -2520,7 +2520,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
     if (lane == 0) {
         const bool failed = (*(volatile const u32*)&sv->state & kSurvFailed) != 0;
         np = proj_points(sk, hole, sv->vars, nullptr);
-        if ((i64)chunk * kVerifyChunk < np && !failed) {
+        if (first < np && !failed) {
             skip = 0;
             stage_candidate(cand, sk, hole, sv->size, sv->rank);
             proj_points(sk, hole, sv->vars, &cand);
@@ -2532,8 +2532,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
     skip = __shfl_sync(0xffffffffu, skip, 0);
     if (skip) return;
     np = __shfl_sync(0xffffffffu, np, 0);
-    const i64 first = (i64)chunk * kVerifyChunk;
-    const i64 last = first + kVerifyChunk < np ? first + kVerifyChunk : np;
+    const i64 last = first + sub < np ? first + sub : np;
     u64 evals = 0;
     i64 fail_pid = 0;
     bool ok;
@@ -2544,7 +2543,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
         ok = check_points(cand, sk, hole, first, last, evals, &fail_pid);
     }
     if (lane == 0) {
-        if (ok) chunk_passed(plan, sv, chunks_of(np));
+        if (ok) chunk_passed(plan, sv, chunks_of(np, sub));
         else if (!(atomicOr(&sv->state, kSurvFailed) & kSurvFailed)) record_killer(hole, fail_pid);   // (once per survivor)
         atomicAdd(&plan.acc[sv->acc].evals, (u64)(last - first));     // points of the chunk (an early exit tries fewer)
     }
@@ -2555,7 +2554,8 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
 // survivor (blocks in hole order) is taken before any second chunk, so candidates that fail early
 // cost one chunk; the later chunks exist for the long survivors only (surv_long_kernel), which keeps
 // a call whose largest domain has hundreds of chunks from walking hundreds of empty items for every
-// survivor of a small (or projected) domain.  Each WARP takes items on its own: nothing in this kernel synchronises a CTA, and no
+// survivor of a small (or projected) domain.  A call with few survivors cuts the chunks into pieces, down to 128 points,
+// until every warp has an item (three survivors of a 37 123-point table: 341 us as whole chunks).  Each WARP takes items on its own: nothing in this kernel synchronises a CTA, and no
 // warp waits for another.  Within a block the survivors of one hole are handled together when the
 // hole's domain is a table (verify_batch), one after the other otherwise (verify_one).  A survivor
 // that has already failed is skipped.
@@ -2578,7 +2578,12 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
     // The first chunk is walked for every survivor, the later ones for the long survivors only.
     const u64 n_long = plan.max_chunks > 1 ? *plan.surv_long_n : 0u;
     const u64 long_blocks = (n_long + width - 1) / width;
-    const u64 total = n_blocks + long_blocks * (plan.max_chunks - 1);
+    u32 pieces = 1;
+    while (pieces < (u32)(kVerifyChunk / kVStep) && n_blocks * pieces < warps) pieces <<= 1;
+    const i64 sub = kVerifyChunk / pieces;                // points per item
+    const u64 first_parts = plan.first_points >= kVerifyChunk ? pieces : (u64)((plan.first_points + sub - 1) / sub);
+    const u64 first_items = n_blocks * first_parts;
+    const u64 total = first_items + long_blocks * (u64)(plan.max_chunks > 0 ? plan.max_chunks - 1 : 0) * pieces;
     const u64 kBatch = 2;                               // items a warp takes per atomic
     u64 next = 0, batch_end = 0;
     for (;;) {
@@ -2589,9 +2594,9 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
         }
         const u64 t = next++;
         if (t >= total) break;
-        const bool later = t >= n_blocks;
-        const u64 chunk = later ? 1 + (t - n_blocks) / long_blocks : 0;
-        const u64 block = later ? (t - n_blocks) % long_blocks : t;
+        const bool later = t >= first_items;
+        const i64 first = later ? kVerifyChunk + (i64)((t - first_items) / long_blocks) * sub : (i64)(t / n_blocks) * sub;
+        const u64 block = later ? (t - first_items) % long_blocks : t % n_blocks;
         const u64 pos = block * width + lane;
         const bool have = (u32)lane < width && pos < (later ? n_long : n);
         const u32 si = !have ? 0u : later ? plan.surv_long[pos] : plan.surv_sorted ? plan.surv_sorted[pos] : (u32)pos;
@@ -2607,12 +2612,11 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
             const HoleDev* hole = &sk->holes[plan.surv[lsi].hole];
             const bool table = sk->domain_kind == XP_DOMAIN_TABLE && sk->coords != nullptr && hole->spec_table != nullptr &&
                                sk->n_vars <= kVBatchVars;
-            const i64 first = (i64)chunk * kVerifyChunk;
             const bool mine = (run >> lane) & 1u;
             u32 single = 0;                               // survivors of the run that go one by one
             if (!table) single = run;
             else if (first < sk->n_points) {
-                const i64 last = first + kVerifyChunk < sk->n_points ? first + kVerifyChunk : sk->n_points;
+                const i64 last = first + sub < sk->n_points ? first + sub : sk->n_points;
                 SurvDev* sv = &plan.surv[si];
                 const bool live = mine && !(*(volatile const u32*)&sv->state & kSurvFailed);
                 const int want_len = live ? staged_length(hole, sv->size) : 0;
@@ -2645,7 +2649,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
                     u64 evals = 0;
                     verify_batch(w, sk, hole, now, my_off, len, narrow, first, last, failed, fail_pid, evals);
                     if ((now >> lane) & 1u) {
-                        if (!failed) chunk_passed(plan, sv, chunks_of(sk->n_points));
+                        if (!failed) chunk_passed(plan, sv, chunks_of(sk->n_points, sub));
                         else if (!(atomicOr(&sv->state, kSurvFailed) & kSurvFailed)) record_killer(hole, fail_pid);
                     }
                     if (lane == 0 && evals) atomicAdd(&plan.acc[acc].evals, evals);
@@ -2653,7 +2657,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
             }
             for (u32 m = single; m; m &= m - 1) {
                 const int b = __ffs((int)m) - 1;
-                verify_one(plan, w, __shfl_sync(0xffffffffu, si, b), chunk);
+                verify_one(plan, w, __shfl_sync(0xffffffffu, si, b), first, sub);
             }
         }
     }
@@ -2853,6 +2857,7 @@ static PlanDev plan_on(char* base, const SearchLayout& L) {
     pd.surv = (SurvDev*)(base + L.surv);
     pd.surv_cap = L.surv_cap;
     pd.max_chunks = L.max_chunks;
+    pd.first_points = L.first_points;
     pd.n_acc = L.n_acc;
     const bool order = L.n_acc > 1;                       // (one hole: the queue is in hole order as it is)
     pd.surv_hist = order ? (u32*)(base + L.hist) : nullptr;

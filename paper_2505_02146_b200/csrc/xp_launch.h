@@ -24,6 +24,7 @@ cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int most
 struct SearchLayout {
     size_t segs, jsegs, jgroups, psegs, sketches, acc, hist, head, surv, sort_off, sorted, longs, total;
     size_t pair_ones, pair_zeros, pair_rest;      // scratch of the pair join: [pair_ones, pair_zeros) all ones, [pair_zeros, pair_rest) zero at launch
+    i32 first_points;                // points of the largest domain, at most kVerifyChunk
     u32 surv_cap, max_chunks;        // max_chunks: chunks of the whole-domain check that the largest domain needs
     int n_segs, n_jsegs, n_psegs, n_sketches, n_acc;
     int dense;                       // some hole of the plan takes the second look: launch the search kernel's dense form
