@@ -121,101 +121,100 @@ __device__ bool ctx_interval(const HoleDev* hole, const i64* pt, i64 spec, i64& 
     return false;
 }
 
-// The join's targets of a hole (one thread): the hole values that satisfy the constraint at the two probes, exact in
+// The join's targets of a hole: the hole values that satisfy the constraint at the two probes, exact in
 // 64 bits for values below the operand limits of the leaf sets (the context's factor times such a value cannot wrap).
-__device__ void join_targets(HoleDev* hole) {
-    const u32 ok = hole->probe_spec_ok & hole->aff_okmask;
-    const int np = hole->tab_probes;
-    hole->join_p1 = np >= 2 && ((ok >> 1) & 1u) ? 1 : 0;
-    bool on = np >= 1 && (ok & 1u), none = false;
-    u64 tmod = 0;
-    i64 t[2] = {0, 0};
-    for (int j = 0; j < np && on; ++j) {
-        if (!((ok >> j) & 1u)) continue;
-        const i64 A = (i64)hole->aff_Aj[j], d = (i64)((u64)hole->probe_spec[j] - hole->aff_Bj[j]);
-        if (A == 0 || A <= -(1ll << 31) || A >= (1ll << 31)) { on = false; break; }
-        i64 v = d;
-        bool miss = false;
-        if (A != 1) { miss = d <= -(1ll << 62) || d >= (1ll << 62) || d % A != 0; v = miss ? 0 : d / A; }
-        if (miss) { none = none || j == 0 || j == hole->join_p1; tmod = ~0ull; }
-        else {
-            const u64 m = v < 0 ? 0ull - (u64)v : (u64)v;
-            tmod = m > tmod ? m : tmod;
-        }
-        if (j == 0) t[0] = t[1] = v;
-        if (j == hole->join_p1) t[1] = v;
-    }
-    hole->join_on = on ? 1 : 0;
-    hole->join_none = none ? 1 : 0;
-    hole->join_t0 = t[0]; hole->join_t1 = t[1];
-    hole->join_tmod = tmod;
-    const float m0 = fabsf((float)t[0]), m1 = fabsf((float)t[1]);
-    hole->join_rt0 = t[0] ? 1.f / m0 : 0.f; hole->join_rt1 = t[1] ? 1.f / m1 : 0.f;
+// Called by threads 0 .. 15 together, one per probe; np: probes with tables; ok: bit per probe with spec and affine context.
+__device__ __forceinline__ void join_targets(HoleDev* hole, int j, int np, u32 ok, u64 A64, u64 B64) {
+    constexpr u32 kLanes = 0x0000ffffu;
+    const bool mine = j < np && ((ok >> j) & 1u);
+    const int p1 = np >= 2 && ((ok >> 1) & 1u) ? 1 : 0;
+    const i64 A = (i64)A64, d = mine ? (i64)((u64)hole->probe_spec[j] - B64) : 0;
+    const bool bad = mine && (A == 0 || A <= -(1ll << 31) || A >= (1ll << 31));
+    i64 v = d;
+    bool miss = false;
+    if (mine && !bad && A != 1) { miss = d <= -(1ll << 62) || d >= (1ll << 62) || d % A != 0; v = miss ? 0 : d / A; }
+    u64 m = !mine ? 0ull : miss ? ~0ull : v < 0 ? 0ull - (u64)v : (u64)v;
+    for (int o = 8; o > 0; o >>= 1) { const u64 q = __shfl_xor_sync(kLanes, m, o); m = q > m ? q : m; }
+    const u32 any_bad = __ballot_sync(kLanes, bad), missed = __ballot_sync(kLanes, miss);
+    const i64 t0 = __shfl_sync(kLanes, v, 0), t1 = __shfl_sync(kLanes, v, p1);
+    if (j != 0) return;
+    hole->join_p1 = p1;
+    hole->join_on = np >= 1 && (ok & 1u) && any_bad == 0u ? 1 : 0;
+    hole->join_none = (missed & 1u) || ((missed >> p1) & 1u) ? 1 : 0;
+    hole->join_t0 = t0; hole->join_t1 = t1;
+    hole->join_tmod = m;
+    const float m0 = fabsf((float)t0), m1 = fabsf((float)t1);
+    hole->join_rt0 = t0 ? 1.f / m0 : 0.f; hole->join_rt1 = t1 ? 1.f / m1 : 0.f;
     hole->join_rl0 = 1.f / (m0 + 1.f); hole->join_rl1 = 1.f / (m1 + 1.f);
-    hole->join_h0 = t[0] ? 0.f : 3e38f; hole->join_h1 = t[1] ? 0.f : 3e38f;
+    hole->join_h0 = t0 ? 0.f : 3e38f; hole->join_h1 = t1 ? 0.f : 3e38f;
 }
 
-// The leaf set of nonterminal nt (one thread): see JoinSet.
+// The leaf set of nonterminal nt: see JoinSet.  Called by one warp, one lane per entry.
 __device__ void join_leaf_set(const GrammarDev* g, HoleDev* hole, int nt) {
+    const int lane = threadIdx.x & 31;
     JoinSet& S = hole->join_sets[nt];
     const ConstDev* c = g->consts;
     const int cb = g->const_begin[nt], vb = g->var_begin[nt], ve = g->const_begin[nt + 1];
     const int p1 = hole->join_p1;
     const i64 t0 = hole->join_t0, t1 = hole->join_t1;
-    const u64 m0 = t0 < 0 ? 0ull - (u64)t0 : (u64)t0, m1 = t1 < 0 ? 0ull - (u64)t1 : (u64)t1;
-    const bool small = (m0 | m1) >> 31 == 0;              // (otherwise no narrow quotient or remainder is the target)
-    bool ok = true;
-    u64 most = 1;
-    int n = 0;
     auto magnitude = [](i64 v) { return v < 0 ? 0ull - (u64)v : (u64)v; };
-    auto add = [&](i64 x, i64 y, int pos) {
+    const u64 m0 = magnitude(t0), m1 = magnitude(t1);
+    const bool small = (m0 | m1) >> 31 == 0;              // (otherwise no narrow quotient or remainder is the target)
+    const int n_vars = ve - vb;
+    int n_const = vb - cb;
+    const bool few = n_const <= kJoinFewConsts && n_vars + n_const <= kJoinEntries;
+    const int n = n_vars + (few ? n_const : 0);           // entries: the variables, and the constants when there are few
+    u64 most = 1;
+    bool bad = n > kJoinEntries;
+    if (lane < n && !bad) {
+        const ConstDev q = c[lane < n_vars ? vb + lane : cb + lane - n_vars];
+        const i64 x = lane < n_vars ? hole->probe_pt[0][q.value] : q.value, y = lane < n_vars ? hole->probe_pt[p1][q.value] : q.value;
         const u64 u0 = magnitude(x), u1 = magnitude(y);
-        most = u0 > most ? u0 : most;
-        most = u1 > most ? u1 : most;
-        if (n >= kJoinEntries || (u0 | u1) >> 31) { ok = false; return; }
+        most = u0 > u1 ? u0 : u1;
+        most = most ? most : 1;
+        bad = (u0 | u1) >> 31 != 0;
         JoinEntry e;
         e.v0 = (u32)(u64)x; e.v1 = (u32)(u64)y; e.u0 = (u32)u0; e.u1 = (u32)u1;
         const u64 l0 = m0 * u0, l1 = m1 * u1;             // (used when the targets are small: below 2^62)
         e.low0 = small && l0 < (1ull << 31) ? (u32)l0 : 0x80000000u;
         e.low1 = small && l1 < (1ull << 31) ? (u32)l1 : 0x80000000u;
         const u32 k0 = e.u0 ? (u32)__ffs((int)e.u0) - 1u : 0u, k1 = e.u1 ? (u32)__ffs((int)e.u1) - 1u : 0u;
-        auto inverse = [](u32 o) { u32 q = o; q *= 2u - o * q; q *= 2u - o * q; q *= 2u - o * q; q *= 2u - o * q; return q; };
+        auto inverse = [](u32 o) { u32 z = o; z *= 2u - o * z; z *= 2u - o * z; z *= 2u - o * z; z *= 2u - o * z; return z; };
         e.inv0 = inverse(e.u0 ? e.u0 >> k0 : 1u); e.inv1 = inverse(e.u1 ? e.u1 >> k1 : 1u);
         e.cm0 = small && e.u0 && m0 < e.u0 ? 0xffffffffu / e.u0 : 0u;
         e.cm1 = small && e.u1 && m1 < e.u1 ? 0xffffffffu / e.u1 : 0u;
         e.k0k1 = k0 | (k1 << 8);
-        e.pos = (u32)pos;
-        S.e[n++] = e;
-    };
-    for (int i = vb; i < ve; ++i) add(hole->probe_pt[0][c[i].value], hole->probe_pt[p1][c[i].value], c[i].pos);
-    int nc = vb - cb;
-    if (nc <= kJoinFewConsts && n + nc <= kJoinEntries) {
-        for (int i = cb; i < vb; ++i) add(c[i].value, c[i].value, c[i].pos);
-        nc = 0;
+        e.pos = (u32)q.pos;
+        S.e[lane] = e;
     }
-    i64 lo = 0, hi = 0;
-    if (nc > 0) {
-        lo = c[cb].value; hi = c[vb - 1].value;
-        const u64 a = magnitude(lo), b = magnitude(hi), m = a > b ? a : b;
-        most = m > most ? m : most;
-        if (m >> 31) ok = false;
-    }
-    auto member = [&](i64 v) {
+    if (few) n_const = 0;
+    const i64 lo = n_const > 0 ? c[cb].value : 0, hi = n_const > 0 ? c[vb - 1].value : 0;
+    const u64 cabs = magnitude(lo) > magnitude(hi) ? magnitude(lo) : magnitude(hi);
+    most = cabs > most ? cabs : most;
+    bad = bad || cabs >> 31 != 0;
+    for (int o = 16; o > 0; o >>= 1) { const u64 q = __shfl_xor_sync(0xffffffffu, most, o); most = q > most ? q : most; }
+    const bool ok = !__any_sync(0xffffffffu, bad);
+    bool member = false;                                  // lanes 0 and 1: is the target at probe 0 / 1 one of the constants?
+    if (lane < 2 && n_const > 0) {
+        const i64 v = lane ? t1 : t0;
         int x = cb, y = vb;
         while (x < y) { const int z = (x + y) >> 1; if (c[z].value < v) x = z + 1; else y = z; }
-        return x < vb && c[x].value == v;
-    };
-    S.n_entries = n; S.n_const = nc; S.const_begin = cb;
-    S.cmin = ok ? (i32)lo : 0; S.cmax = ok ? (i32)hi : 0;
-    S.cabs = ok ? (u32)(magnitude(lo) > magnitude(hi) ? magnitude(lo) : magnitude(hi)) : 0u;
-    S.mm = nc > 0 ? (member(t0) ? 1u : 0u) | (member(t1) ? 2u : 0u) : 0u;
-    // |factor| * |operand| * |leaf| must stay below 2^62
-    const i64 A0 = (i64)hole->aff_Aj[0], A1 = (i64)hole->aff_Aj[p1];
-    u64 A = magnitude(A0) > magnitude(A1) ? magnitude(A0) : magnitude(A1);
-    if (A < 1 || A >> 31) A = 1ull << 31;
-    const u64 lim = ((1ull << 62) - 1) / A / most;
-    S.lim = lim < 0x7fffffffull ? (u32)lim : 0x7fffffffu;
-    S.ok = ok && lim > 0 ? 1 : 0;
+        member = x < vb && c[x].value == v;
+    }
+    const u32 mm = __ballot_sync(0xffffffffu, member);
+    if (lane == 0) {
+        S.n_entries = n > kJoinEntries ? 0 : n; S.n_const = n_const; S.const_begin = cb;
+        S.cmin = ok ? (i32)lo : 0; S.cmax = ok ? (i32)hi : 0;
+        S.cabs = ok ? (u32)cabs : 0u;
+        S.mm = mm;
+        // |factor| * |operand| * |leaf| must stay below 2^62
+        const u64 A0 = magnitude((i64)hole->aff_Aj[0]), A1 = magnitude((i64)hole->aff_Aj[p1]);
+        u64 A = A0 > A1 ? A0 : A1;
+        if (A < 1 || A >> 31) A = 1ull << 31;
+        const u64 lim = ((1ull << 62) - 1) / A / most;
+        S.lim = lim < 0x7fffffffull ? (u32)lim : 0x7fffffffu;
+        S.ok = ok && lim > 0 ? 1 : 0;
+    }
 }
 
 // The context at every probe (affine in the hole, or a comparison; one thread per probe), and what
@@ -235,6 +234,12 @@ __device__ __forceinline__ void probe_contexts(const GrammarDev* g, HoleDev* hol
         hole->rng_lo[t] = lo;
         hole->rng_hi[t] = hi;
         const u32 amask = __ballot_sync(0x0000ffffu, aff), rmask = __ballot_sync(0x0000ffffu, rng);
+        {
+            const u32 spec_ok = hole->probe_spec_ok;
+            const bool filter = n > 0 && ((amask & 1u) || (rmask & spec_ok & 1u)) && hole->tab_size_cap > 0 && hole->tab_total > 0;
+            const int np = filter ? (n < hole->tab_probes_cap ? n : hole->tab_probes_cap) : 0;
+            join_targets(hole, t, np, spec_ok & amask, A, B);
+        }
         if (t == 0) {
             hole->aff_ok = aff ? 1 : 0;
             hole->aff_A = aff ? A : 0;
@@ -260,11 +265,10 @@ __device__ __forceinline__ void probe_contexts(const GrammarDev* g, HoleDev* hol
             const bool frequent = ncand > 0 && (u64)pass0 * 256 >= (u64)ncand;
             hole->second = possible && (hole->small_search || frequent) ? 1 : 0;
             hole->second_ok = possible ? 1 : 0;
-            join_targets(hole);
         }
     }
     __syncthreads();
-    if (t < g->n_nt) join_leaf_set(g, hole, t);
+    if (t < 32) for (int nt = 0; nt < g->n_nt; ++nt) join_leaf_set(g, hole, nt);
 }
 
 // Choice of each hole's probe points, once per sketch.  A sample of small candidates (sizes 1, 3, 5, ranks spread evenly)
@@ -275,11 +279,13 @@ __device__ __forceinline__ void probe_contexts(const GrammarDev* g, HoleDev* hol
 // the larger |spec| + sum |coordinate| (large, distinct operand values make coincidences rare).
 // Only the amount of work downstream depends on this choice, never a result.
 //
-// The sampling is spread over 8 CTAs of 16 warps per hole (lane = candidate, warp = 4 samples): as one CTA per hole it
-// was bound by the instruction rate of a single SM (130 to 290 us of a load; now 10).
+// The sampling is spread over 64 CTAs of 4 warps per hole (lane = candidate, warp = 2 samples): as one CTA per hole it
+// was bound by the instruction rate of a single SM (130 to 290 us of a load).  The context is brought to an affine map
+// or an interval once per sample instead of being interpreted for every candidate.
 constexpr int kPrepCands = 256;
-constexpr int kPrepParts = 16;                          // the samples are split over this many warps
 constexpr int kPrepWords = kPrepCands / 32;
+constexpr int kPrepWarps = 4, kPrepEach = 2;            // warps per CTA, samples per warp
+constexpr int kPrepSplit = kProbeSamples / (kPrepWarps * kPrepEach);
 
 // A sample point's coordinates and spec value, and what it scores in a tie (one thread per sample).
 __device__ __forceinline__ void prep_point(const SketchDev* s, const HoleDev* hole, int t, i64* pt, i64& spec, bool& ok, u64& score) {
@@ -302,23 +308,31 @@ __device__ __forceinline__ int prep_sizes(const GrammarDev* g, const HoleDev* ho
     return n;
 }
 
-__global__ void __launch_bounds__(32 * kPrepParts) prep_sample_kernel(const LoadJob* jobs, u32* masks) {
-    const SketchDev* s = jobs[blockIdx.y].s;
-    const HoleDev* hole = &s->holes[jobs[blockIdx.y].hole];
+__global__ void __launch_bounds__(32 * kPrepWarps) prep_sample_kernel(const LoadJob* jobs, u32* masks) {
+    constexpr int kHere = kPrepWarps * kPrepEach;        // samples of this CTA
+    const SketchDev* s = jobs[blockIdx.z].s;
+    const HoleDev* hole = &s->holes[jobs[blockIdx.z].hole];
     const GrammarDev* g = s->g;
-    __shared__ i64 s_pt[kProbeSamples][kMaxVars];
-    __shared__ i64 s_spec[kProbeSamples];
-    __shared__ int s_ok[kProbeSamples];
-    const int t = threadIdx.x, lane = t & 31, part = t >> 5, word = blockIdx.x;
+    __shared__ i64 s_pt[kHere][kMaxVars], s_spec[kHere], s_lo[kHere], s_hi[kHere];
+    __shared__ u64 s_A[kHere], s_B[kHere];
+    __shared__ int s_form[kHere];                        // 0: no constraint can hold; 1: affine; 2: interval; 3: interpret
+    const int t = threadIdx.x, lane = t & 31, word = blockIdx.x, first = blockIdx.y * kHere;
     const int ns = s->n_samples;
-    if (t < ns) {
-        i64 pt[kMaxVars], v;
-        bool ok;
-        u64 score;
-        prep_point(s, hole, t, pt, v, ok, score);
-        for (int d = 0; d < s->n_vars; ++d) s_pt[t][d] = pt[d];
-        s_spec[t] = v;
-        s_ok[t] = ok;
+    if (t < kHere) {
+        int form = 0;
+        if (first + t < ns) {
+            i64 pt[kMaxVars], v;
+            bool ok;
+            u64 score;
+            prep_point(s, hole, first + t, pt, v, ok, score);
+            for (int d = 0; d < s->n_vars; ++d) s_pt[t][d] = pt[d];
+            s_spec[t] = v;
+            u64 A = 0, B = 0;
+            i64 lo = 1, hi = 0;
+            if (ok) form = ctx_affine(hole, pt, A, B) ? 1 : ctx_interval(hole, pt, v, lo, hi) ? 2 : 3;
+            s_A[t] = A; s_B[t] = B; s_lo[t] = lo; s_hi[t] = hi;
+        }
+        s_form[t] = form;
     }
     int sizes[3] = {1, 1, 1};
     const int nsz = prep_sizes(g, hole, sizes);
@@ -333,12 +347,18 @@ __global__ void __launch_bounds__(32 * kPrepParts) prep_sample_kernel(const Load
             n = unrank(g, hole->start_nt, size, cnt >= per ? slot * (cnt / per) : slot, code);
     }
     __syncthreads();
-    u32* out = masks + (u64)blockIdx.y * kProbeSamples * kPrepWords;
-    for (int j = part; j < ns; j += kPrepParts) {
-        i64 v;
-        const bool hit = n > 0 && s_ok[j] && eval_cand(code, n, g->leaves, s_pt[j], v) && ctx_matches(hole, s_pt[j], v, s_spec[j]);
+    u32* out = masks + (u64)blockIdx.z * kProbeSamples * kPrepWords;
+    for (int k = 0; k < kPrepEach; ++k) {
+        const int j = (t >> 5) * kPrepEach + k;
+        if (first + j >= ns) break;
+        const int form = s_form[j];
+        i64 v = 0;
+        bool hit = form != 0 && n > 0 && eval_cand(code, n, g->leaves, s_pt[j], v);
+        if (form == 1) hit = hit && (u64)v * s_A[j] + s_B[j] == (u64)s_spec[j];
+        else if (form == 2) hit = hit && v >= s_lo[j] && v <= s_hi[j];
+        else hit = hit && ctx_matches(hole, s_pt[j], v, s_spec[j]);
         const u32 b = __ballot_sync(0xffffffffu, hit);
-        if (lane == 0) out[j * kPrepWords + word] = b;
+        if (lane == 0) out[(first + j) * kPrepWords + word] = b;
     }
 }
 
@@ -375,6 +395,9 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
         int n = 0, pass0 = 0, first = 0;
         u32 spec_ok = 0;
         for (; n < kMaxProbe && n < ns; ++n) {
+            u32 left = 0;
+            for (int w = 0; w < kPrepWords; ++w) left |= alive[w];
+            if (n >= 2 && left == 0u) break;              // no sampled candidate is left: by score alone, all at once below
             u64 best_key = ~0ull, best_score = 0;         // key: candidates that pass << 32 | 255 - difference from the first probe
             int best = -1;
             for (int i = lane; i < ns; i += 32) {
@@ -402,6 +425,23 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
             for (int w = 0; w < kPrepWords; ++w) alive[w] &= s_mask[best][w];
             if (lane == 0) { hole->probe_id[n] = s->sample_id[best]; hole->probe_spec[n] = s_spec[best]; }
             if (lane < nv) hole->probe_pt[n][lane] = s_pt[best][lane];
+        }
+        const int most = ns < kMaxProbe ? ns : kMaxProbe;
+        if (n < most) {
+            u32 more = 0;
+            for (int i = lane; i < ns; i += 32) {
+                if ((chosen >> i) & 1ull) continue;
+                int before = 0;
+                for (int k = 0; k < ns; ++k)
+                    before += !((chosen >> k) & 1ull) && (s_score[k] > s_score[i] || (s_score[k] == s_score[i] && k < i));
+                if (n + before >= most) continue;
+                const int at = n + before;
+                hole->probe_id[at] = s->sample_id[i]; hole->probe_spec[at] = s_spec[i];
+                for (int d = 0; d < nv; ++d) hole->probe_pt[at][d] = s_pt[i][d];
+                more |= (u32)(s_ok[i] != 0) << at;
+            }
+            spec_ok |= __reduce_or_sync(0xffffffffu, more);
+            n = most;
         }
         if (lane == 0) {
             hole->n_probe = n;
@@ -2758,7 +2798,7 @@ size_t prepare_scratch_bytes(int n_jobs) { return sizeof(u32) * (size_t)kProbeSa
 
 cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadOut* out, cudaStream_t stream) {
     if (n_jobs <= 0) return cudaSuccess;
-    prep_sample_kernel<<<dim3(kPrepWords, (unsigned)n_jobs), 32 * kPrepParts, 0, stream>>>(jobs, (u32*)scratch);
+    prep_sample_kernel<<<dim3(kPrepWords, kPrepSplit, (unsigned)n_jobs), 32 * kPrepWarps, 0, stream>>>(jobs, (u32*)scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     prepare_kernel<<<n_jobs, kPrepThreads, 0, stream>>>(jobs, (const u32*)scratch, out);
