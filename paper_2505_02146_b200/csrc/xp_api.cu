@@ -561,6 +561,113 @@ struct LoadState {
 constexpr size_t kPackMax = 256u << 10;      // host tables up to this size travel in the staged copy
 static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
+// Which variables can decide whether a hole value satisfies the constraint?  Where the context is an affine map of the
+// hole, A h + B = spec, it is those of A and of D = spec - B, taken as polynomials over the variables (coefficients modulo
+// 2^64, so + - * are exact) with every other subexpression as an atom of its own: terms that both sides share cancel
+// (c * 3136 + HOLE * 56 + col against c * 3136 + row * 56 + col leaves the variables of row).  On a box the whole-domain
+// check then runs over those and the candidate's own variables only.  Subexpressions that may be undefined keep theirs.
+namespace {
+struct Poly { std::map<std::vector<int>, u64> t; };       // monomial (sorted atoms) -> coefficient, none zero
+struct PolyAtoms { std::map<std::string, int> ids; std::vector<u32> vars; u32 may_fail = 0; };
+constexpr size_t kPolyTerms = 64;
+
+void poly_add(Poly& a, const Poly& b, u64 f) {
+    for (const auto& m : b.t) {
+        const u64 c = (a.t[m.first] += f * m.second);
+        if (c == 0) a.t.erase(m.first);
+    }
+}
+bool poly_mul(const Poly& a, const Poly& b, Poly& out) {
+    out.t.clear();
+    for (const auto& x : a.t)
+        for (const auto& y : b.t) {
+            std::vector<int> m(x.first);
+            m.insert(m.end(), y.first.begin(), y.first.end());
+            if (m.size() > 8) return false;
+            std::sort(m.begin(), m.end());
+            const u64 c = (out.t[m] += x.second * y.second);
+            if (c == 0) out.t.erase(m);
+            if (out.t.size() > kPolyTerms) return false;
+        }
+    return true;
+}
+std::string poly_key(const Poly& p) {
+    std::string s;
+    for (const auto& m : p.t) {
+        s += std::to_string(m.second) + ":";
+        for (int a : m.first) s += std::to_string(a) + ",";
+        s += ";";
+    }
+    return s;
+}
+u32 poly_vars(const Poly& p, const PolyAtoms& atoms) {
+    u32 v = 0;
+    for (const auto& m : p.t) for (int a : m.first) v |= atoms.vars[a];
+    return v;
+}
+// code = A h + B; false when it is not of that form (or too large to follow).
+bool poly_affine(const xp_instr* code, int n, PolyAtoms& atoms, Poly& A, Poly& B) {
+    struct E { Poly a, b; };
+    std::vector<E> st;
+    for (int i = 0; i < n; ++i) {
+        const xp_instr& c = code[i];
+        if (c.kind != XP_I_OP) {
+            E e;
+            if (c.kind == XP_I_HOLE) e.a.t[{}] = 1;
+            else if (c.kind == XP_I_VAR) e.b.t[{c.arg}] = 1;
+            else if (c.value != 0) e.b.t[{}] = (u64)c.value;
+            st.push_back(std::move(e));
+            continue;
+        }
+        E y = std::move(st.back()); st.pop_back();
+        E x = std::move(st.back()); st.pop_back();
+        E r;
+        if (c.arg == XP_OP_ADD || c.arg == XP_OP_SUB) {
+            const u64 f = c.arg == XP_OP_ADD ? 1ull : ~0ull;
+            r = std::move(x);
+            poly_add(r.a, y.a, f); poly_add(r.b, y.b, f);
+            if (r.a.t.size() > kPolyTerms || r.b.t.size() > kPolyTerms) return false;
+        } else if (c.arg == XP_OP_MUL) {
+            if (!x.a.t.empty() && !y.a.t.empty()) return false;
+            const Poly& h = x.a.t.empty() ? y.a : x.a;
+            const Poly& k = x.a.t.empty() ? x.b : y.b;
+            if (!poly_mul(h, k, r.a) || !poly_mul(x.b, y.b, r.b)) return false;
+        } else {
+            if (!x.a.t.empty() || !y.a.t.empty()) return false;      // (the hole under another operator)
+            const u32 v = poly_vars(x.b, atoms) | poly_vars(y.b, atoms);
+            const std::string key = std::to_string(c.arg) + "(" + poly_key(x.b) + "|" + poly_key(y.b) + ")";
+            auto it = atoms.ids.find(key);
+            if (it == atoms.ids.end()) { it = atoms.ids.insert({key, (int)atoms.vars.size()}).first; atoms.vars.push_back(v); }
+            const bool divides = c.arg == XP_OP_DIV || c.arg == XP_OP_MOD, shifts = c.arg == XP_OP_SHL || c.arg == XP_OP_SHR;
+            const bool constant = y.b.t.empty() || (y.b.t.size() == 1 && y.b.t.begin()->first.empty());
+            const u64 value = y.b.t.empty() || !constant ? 0ull : y.b.t.begin()->second;
+            if ((divides && (!constant || value == 0)) || (shifts && (!constant || value > 63))) atoms.may_fail |= v;
+            r.b.t[{it->second}] = 1;
+        }
+        st.push_back(std::move(r));
+    }
+    A = std::move(st.back().a); B = std::move(st.back().b);
+    return true;
+}
+}  // namespace
+
+// Variables that the constraint of a hole with a spec expression depends on beside the hole's value (bits).  Below
+// kPolyPoints points the check is short whatever the variables, and the algebra would cost the load more than it saves.
+constexpr i64 kPolyPoints = 1 << 15;
+static u32 constraint_vars(const xp_hole_desc& hd, int n_vars, i64 n_points) {
+    u32 fv = 0;
+    for (int i = 0; i < hd.ctx_len; ++i) if (hd.ctx[i].kind == XP_I_VAR) fv |= 1u << hd.ctx[i].arg;
+    for (int i = 0; i < hd.spec_len; ++i) if (hd.spec_expr[i].kind == XP_I_VAR) fv |= 1u << hd.spec_expr[i].arg;
+    if (hd.ctx_len == 0 || n_points < kPolyPoints) return fv;
+    PolyAtoms atoms;
+    for (int v = 0; v < n_vars; ++v) atoms.vars.push_back(1u << v);
+    Poly A, B, none, D;
+    if (!poly_affine(hd.ctx, hd.ctx_len, atoms, A, B) || A.t.empty()) return fv;
+    if (!poly_affine(hd.spec_expr, hd.spec_len, atoms, none, D)) return fv;
+    poly_add(D, B, ~0ull);
+    return fv & (poly_vars(A, atoms) | poly_vars(D, atoms) | atoms.may_fail);
+}
+
 // First part of a load: checks the description, lays out and allocates the sketch's device block.
 static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadState* L) {
     if (!gc || !d) return fail(XP_ERR_INVALID_ARG, "xp_sketch_load: null argument");
@@ -684,11 +791,8 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             o.tab_pair = (i32*)(base + off_pair[h]);
         }
         o.join_sets = (JoinSet*)(base + off_sets[h]);
-        // variables the context and the spec mention (a caller's spec table may depend on all)
-        u32 fv = hd.spec_kind == XP_SPEC_EXPR ? 0u : 0xffffffffu;
-        for (int i = 0; i < hd.ctx_len; ++i) if (hd.ctx[i].kind == XP_I_VAR) fv |= 1u << hd.ctx[i].arg;
-        if (hd.spec_kind == XP_SPEC_EXPR)
-            for (int i = 0; i < hd.spec_len; ++i) if (hd.spec_expr[i].kind == XP_I_VAR) fv |= 1u << hd.spec_expr[i].arg;
+        // variables that decide beside the candidate's own (a caller's spec table may depend on all)
+        const u32 fv = hd.spec_kind != XP_SPEC_EXPR ? 0xffffffffu : constraint_vars(hd, nv, n_points);
         o.fixed_vars = fv;
         o.kill_pid = (i64*)(base + s->off_kill[h]);
         o.kill_cnt = (u32*)(base + s->off_kill[h] + sizeof(i64) * kKillSlots);

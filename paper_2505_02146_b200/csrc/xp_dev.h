@@ -135,8 +135,8 @@ struct HoleDev {
     i64* tab_val;                                 // device
     unsigned char* tab_ok;                        // device
     unsigned char* tab_vars;                      // device, one copy: bit v set if variable v occurs in the subtree
-    // Variables that the context or the spec expression mention (all of them when the spec is the
-    // caller's table).  On a box domain a candidate is checked on the sub-box of these and its
+    // Variables that can decide whether a hole value satisfies the constraint (all of them when the spec is the
+    // caller's table; see constraint_vars).  On a box domain a candidate is checked on the sub-box of these and its
     // own variables only: no other variable can change either side of the constraint.
     u32 fixed_vars, spec_bad;                     // spec_bad: set by the load when the spec is undefined at some point
     // The leaf join: values (a0, a1) at its two probes of every tabulated subtree, 8 bytes each (same index as
