@@ -132,65 +132,6 @@ __device__ __forceinline__ bool probe_accepts(const HoleDev* hole, int j, i64 v)
 
 __device__ __forceinline__ int op_of_slot(int slot) { return slot <= 4 ? slot : slot <= 6 ? slot - 5 + XP_OP_MIN : slot - 7 + XP_OP_SHL; }
 
-// Candidates checked one by one look at the probes four at a time: their table entries lie in four places that nothing has
-// touched before, and one probe after the other a candidate that passes 16 probes waits 16 times for memory (the direct
-// tickets of a small search: 20.7 -> 18.6 us).  Candidates of the join mostly end at the next probe and keep the plain order.
-constexpr int kProbeStep = 4;
-
-// An operand's values at the probes j0 .. j0 + 3 (those below n); returns the mask of those it is defined at.
-__device__ __forceinline__ u32 ref_value4(const GrammarDev* g, const HoleDev* hole, const OperandRef& r, int nt, int size, int j0, int n, i64 (&v)[kProbeStep]) {
-    u32 ok = 0;
-    if (r.mode == 2) {
-#pragma unroll 1
-        for (int k = 0; k < kProbeStep; ++k) {
-            i64 x = 0;
-            if (j0 + k < n && ref_value_full(g, hole, nt, size, r.a, j0 + k, x)) ok |= 1u << k;
-#pragma unroll
-            for (int q = 0; q < kProbeStep; ++q) if (q == k) v[q] = x;
-        }
-        return ok;
-    }
-    const u64 total = hole->tab_total;
-    const bool in = XP_CHECKED(n <= hole->tab_probes && r.a < total && r.b < total, kChkTable);
-    i64 y[kProbeStep];
-#pragma unroll
-    for (int k = 0; k < kProbeStep; ++k) {
-        v[k] = 0; y[k] = 0;
-        if (j0 + k < n && in) {
-            const u64 at = (u64)(j0 + k) * total;
-            ok |= (u32)(hole->tab_ok[at + r.a] != 0) << k;
-            v[k] = hole->tab_val[at + r.a];
-            if (r.mode == 1) { if (!hole->tab_ok[at + r.b]) ok &= ~(1u << k); y[k] = hole->tab_val[at + r.b]; }
-        }
-    }
-    if (r.mode == 1) {
-#pragma unroll 1
-        for (int k = 0; k < kProbeStep; ++k) {
-            i64 x = v[0], z = y[0];
-#pragma unroll
-            for (int q = 1; q < kProbeStep; ++q) if (q == k) { x = v[q]; z = y[q]; }
-            if (((ok >> k) & 1u) && !apply_op(r.op, x, z, x)) ok &= ~(1u << k);
-#pragma unroll
-            for (int q = 0; q < kProbeStep; ++q) if (q == k) v[q] = x;
-        }
-    }
-    return ok;
-}
-
-// Do the values v at the probes j0 .. j0 + 3 (those below n) satisfy the constraint?
-__device__ __forceinline__ bool probes_accept(const HoleDev* hole, int j0, int n, const i64 (&v)[kProbeStep]) {
-    const u32 aff = hole->aff_okmask >> j0;
-    bool ok = true;
-#pragma unroll
-    for (int k = 0; k < kProbeStep; ++k) {
-        if (j0 + k >= n) continue;
-        const int j = j0 + k;
-        if ((aff >> k) & 1u) ok = ok && (u64)v[k] * hole->aff_Aj[j] + hole->aff_Bj[j] == (u64)hole->probe_spec[j];
-        else if (v[k] > -(1ll << 62) && v[k] < (1ll << 62)) ok = ok && v[k] >= hole->rng_lo[j] && v[k] <= hole->rng_hi[j];
-    }
-    return ok;
-}
-
 // The candidate (operand, leaf) at the probes that have tables, in order; the first failure ends it.
 __device__ __forceinline__ bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
                                            bool swap, int op, int from, int n_exact, u64& evals) {
@@ -1137,11 +1078,10 @@ __device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, con
         if (rank < first + count) {
             const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, rank);
             pass = true;
-            for (int j0 = 0; j0 < n_exact && pass; j0 += kProbeStep) {
-                const int here = n_exact - j0 < kProbeStep ? n_exact - j0 : kProbeStep;
-                n.evals += (u64)here;
-                i64 v[kProbeStep];
-                pass = ref_value4(g, hole, ref, seg.nt, seg.esize, j0, n_exact, v) == (1u << here) - 1u && probes_accept(hole, j0, n_exact, v);
+            for (int j = 0; j < n_exact && pass; ++j) {
+                ++n.evals;
+                i64 v;
+                pass = ref_value(g, hole, ref, seg.nt, seg.esize, j, v) && probe_accepts(hole, j, v);
             }
             if (pass && n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
             vars = ref_vars(hole, ref);
