@@ -1091,6 +1091,16 @@ HoleSpec sketch_hole(const xp_sketch* s, int hole) {
     return HoleSpec{s->holes[hole].start_nt, s->holes[hole].max_size};
 }
 const HoleDev* sketch_hole_dev(const xp_sketch* s, int hole) { return s->d_holes + hole; }
+StageMemory::StageMemory(size_t bytes) : p(nullptr), block(new (std::nothrow) StageBlock(bytes)) { if (block) p = ((StageBlock*)block)->p; }
+StageMemory::~StageMemory() { delete (StageBlock*)block; }
+StageEvents::StageEvents() : e0(nullptr), e1(nullptr), pair(new (std::nothrow) EventPair) {}
+StageEvents::~StageEvents() { delete (EventPair*)pair; }
+cudaError_t StageEvents::open() {
+    if (!pair) return cudaErrorMemoryAllocation;
+    const cudaError_t e = ((EventPair*)pair)->open();
+    e0 = ((EventPair*)pair)->e0; e1 = ((EventPair*)pair)->e1;
+    return e;
+}
 cudaError_t device_alloc(void** out, size_t bytes, int* device, size_t* granted) { return pool_alloc(out, bytes, device, granted); }
 void device_release(void* ptr, size_t granted, int device) { pool_release(ptr, granted, device); }
 }  // namespace xp

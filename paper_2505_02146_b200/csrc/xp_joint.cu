@@ -2,18 +2,25 @@
 //
 //   joint_probe_kernel   -- coordinates and spec values of the probe points (the first sample points
 //                           of the sketch: box corners first, then ids spread by a fixed hash).
+// A context that is affine in both parts, A0 h0 + A1 h1 + B (the usual one: a stride and an offset), is searched from
+// one side: the pair satisfies the probes iff A1 h1 = spec - B - A0 h0 at all of them.
+//   joint_key_kernel     -- thread = candidate of one part: its side of that equation at every probe, hashed to 64 bits.
+//                           Part 1 goes into hash chains; part 0 then walks the chain of its own key and lists
+//                           the partners.  N0 + N1 candidates are evaluated instead of N0 * N1 pairs.
+//   joint_check_kernel   -- a warp per listed pair: the whole domain, lane = point, vote exit.
+// Any other context (and a list that ran over):
 //   joint_values_kernel  -- value at every probe of every candidate of either part (every size up
 //                           to its bound): thread = (table entry, probe).
 //   joint_pairs_kernel   -- one (size of part 0, size of part 1) block of the pair space: thread =
 //                           pair, rank of part 1 fastest; the constraint is evaluated at the probes
 //                           from the tables, first failure ends the pair; the pairs of a warp that
-//                           pass every probe are checked on the whole domain by the warp together
-//                           (lane = point, vote exit).  Matches go into per-total-size counts (sum)
-//                           and least keys (min) by atomics.
+//                           pass every probe are checked on the whole domain by the warp together.
+// Matches go into per-total-size counts (sum) and least keys (min) by atomics.
 // No CTA or warp waits for another.
 #include <cuda_runtime.h>
 
 #include <chrono>
+#include <cstddef>
 #include <cstring>
 #include <new>
 #include <string>
@@ -43,10 +50,56 @@ struct JointDev {
     u64 tab_total[2];
     i64* tab_val[2];                                      // device, [probe][entry]
     unsigned char* tab_ok[2];
+    // the search from one side: context coefficients per probe, part 1's chains, the listed pairs
+    u64 A0[kJointProbes], A1[kJointProbes], B[kJointProbes];
+    u32 undefined, head_mask;                             // undefined: bit j: a hole-free part of the context is undefined at probe j
+    u32* head;                                            // device, all ones at launch
+    u32* next;
+    u64* key;
+    uint2* list;                                          // device, kJointList entries (candidate of part 0, of part 1)
+    // results, read back together
     u64 match_count[kJointTotal + 1];
     u64 min_key[kJointTotal + 1];                         // size of part 0 << 48 | rank 0 << 24 | rank 1 (all-ones: none)
-    u64 evals, survivors;
+    u64 evals, survivors, listed;
 };
+constexpr u64 kJointList = 1ull << 20;                    // pairs that pass the probes, at most (more: the other form)
+
+// The context at one point as A0 h0 + A1 h1 + B in wrap-around arithmetic (its form was checked on the host); false when
+// a hole-free operand is undefined there.
+__device__ bool joint_affine_at(const xp_instr* code, int n, const i64* pt, u64& A0, u64& A1, u64& B) {
+    u64 a[kMaxStack], b[kMaxStack], c[kMaxStack];
+    u32 has = 0;
+    int sp = 0;
+    for (int i = 0; i < n; ++i) {
+        const xp_instr q = code[i];
+        if (q.kind != XP_I_OP) {
+            a[sp] = q.kind == XP_I_HOLE && q.arg == 0 ? 1ull : 0ull;
+            b[sp] = q.kind == XP_I_HOLE && q.arg == 1 ? 1ull : 0ull;
+            c[sp] = q.kind == XP_I_VAR ? (u64)pt[q.arg] : q.kind == XP_I_CONST ? (u64)q.value : 0ull;
+            has = (has & ~(1u << sp)) | ((u32)(q.kind == XP_I_HOLE) << sp);
+            ++sp;
+            continue;
+        }
+        --sp;
+        const bool hy = (has >> sp) & 1u, hx = (has >> (sp - 1)) & 1u;
+        if (!hx && !hy) {
+            i64 r;
+            if (!apply_op(q.arg, (i64)c[sp - 1], (i64)c[sp], r)) return false;
+            c[sp - 1] = (u64)r;
+            continue;
+        }
+        if (q.arg == XP_OP_ADD) { a[sp - 1] += a[sp]; b[sp - 1] += b[sp]; c[sp - 1] += c[sp]; }
+        else if (q.arg == XP_OP_SUB) { a[sp - 1] -= a[sp]; b[sp - 1] -= b[sp]; c[sp - 1] -= c[sp]; }
+        else {                                            // a product with one hole-free side
+            const u64 f = hx ? c[sp] : c[sp - 1];
+            const int k = hx ? sp - 1 : sp;
+            a[sp - 1] = a[k] * f; b[sp - 1] = b[k] * f; c[sp - 1] = c[k] * f;
+        }
+        has |= 1u << (sp - 1);
+    }
+    A0 = a[0]; A1 = b[0]; B = c[0];
+    return true;
+}
 
 // Value of the joint context at one point from the values of its two parts.
 __device__ __forceinline__ bool eval_joint(const xp_instr* code, int n, const i64* pt, i64 h0, i64 h1, i64& out) {
@@ -69,7 +122,7 @@ __device__ __forceinline__ bool eval_joint(const xp_instr* code, int n, const i6
     return true;
 }
 
-__global__ void joint_probe_kernel(JointDev* J) {
+__global__ void joint_probe_kernel(JointDev* J, int affine) {
     const int t = threadIdx.x;
     const SketchDev* sk = J->sk;
     bool ok = false;
@@ -87,6 +140,58 @@ __global__ void joint_probe_kernel(JointDev* J) {
     }
     const u32 m = __ballot_sync(0xffffffffu, ok);
     if (t == 0) J->spec_ok = m;
+    if (!affine) return;
+    bool undef = false;
+    if (t < J->n_probe) undef = !joint_affine_at(J->ctx, J->ctx_len, J->probe_pt[t], J->A0[t], J->A1[t], J->B[t]);
+    const u32 u = __ballot_sync(0xffffffffu, undef);
+    if (t == 0) J->undefined = u;
+}
+
+// Size and rank of candidate number e of a part.
+__device__ __forceinline__ int joint_locate(const JointDev* J, int part, u64 e, u64& rank) {
+    int s = 1;
+    while (s < J->max_size[part] && J->tab_off[part][s + 1] <= e) ++s;
+    rank = e - J->tab_off[part][s];
+    return s;
+}
+
+__global__ void __launch_bounds__(128) joint_key_kernel(JointDev* J, int part) {
+    const SketchDev* sk = J->sk;
+    const GrammarDev* g = sk->g;
+    const u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    const int np = J->n_probe;
+    const u32 all = np >= 32 ? 0xffffffffu : (1u << np) - 1u;
+    if ((J->spec_ok & all) != all || (J->undefined & all) != 0u) return;      // nothing can match
+    u32 ran = 0;
+    u64 key = 0x243F6A8885A308D3ull;
+    bool ok = e < J->tab_total[part];
+    if (ok) {
+        u64 rank;
+        const int s = joint_locate(J, part, e, rank);
+        u32 code[kMaxSize];
+        const int n = unrank(g, J->start_nt[part], s, rank, code);
+        for (int j = 0; j < np && ok; ++j) {
+            i64 h;
+            ++ran;
+            ok = eval_cand(code, n, g->leaves, J->probe_pt[j], h);
+            const u64 v = part ? J->A1[j] * (u64)h : (u64)J->probe_spec[j] - J->B[j] - J->A0[j] * (u64)h;
+            key = (key ^ v) * 0x9E3779B97F4A7C15ull;
+            key ^= key >> 29;
+        }
+    }
+    if (ok) {
+        u32* head = &J->head[(u32)(key >> 32) & J->head_mask];
+        if (part) { J->key[e] = key; J->next[e] = atomicExch(head, (u32)e); }
+        else
+            for (u32 y = *head; y != 0xffffffffu; y = J->next[y])
+                if (J->key[y] == key) {                   // (an equal key that is no match fails on the domain, probes among it)
+                    const u64 at = atomicAdd((unsigned long long*)&J->listed, 1ull);
+                    if (at >= kJointList) break;          // (the host takes the other form)
+                    J->list[at] = make_uint2((u32)e, y);
+                }
+    }
+    for (int o = 16; o > 0; o >>= 1) ran += __shfl_down_sync(0xffffffffu, ran, o);
+    if ((threadIdx.x & 31) == 0 && ran) atomicAdd((unsigned long long*)&J->evals, (u64)ran);
 }
 
 __global__ void __launch_bounds__(256) joint_values_kernel(JointDev* J, int part, int size) {
@@ -177,9 +282,42 @@ __global__ void __launch_bounds__(256) joint_pairs_kernel(JointDev* J, int s0, i
     }
 }
 
+// A warp per listed pair.
+__global__ void __launch_bounds__(256) joint_check_kernel(JointDev* J) {
+    const u64 n = J->listed;
+    if (n > kJointList) return;                           // (the list ran over: the host takes the other form)
+    u64 evals = 0;
+    for (u64 i = (u64)blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += (u64)gridDim.x * 8) {
+        u64 r0, r1;
+        const int s0 = joint_locate(J, 0, J->list[i].x, r0), s1 = joint_locate(J, 1, J->list[i].y, r1);
+        if (joint_check_domain(J, s0, r0, s1, r1, evals) && (threadIdx.x & 31) == 0) {
+            atomicAdd(&J->match_count[s0 + s1], 1ull);
+            atomicMin(&J->min_key[s0 + s1], ((u64)s0 << 48) | (r0 << 24) | r1);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) evals += __shfl_down_sync(0xffffffffu, evals, o);
+    if ((threadIdx.x & 31) == 0 && evals) atomicAdd(&J->evals, evals);
+}
+
 }  // namespace xp
 
 using namespace xp;
+
+// Is the context affine in both parts whatever the point: no hole under an operator but + - *, none times another?
+static bool joint_is_affine(const xp_instr* code, int n) {
+    bool has[kMaxStack + 1];
+    int sp = 0;
+    for (int i = 0; i < n; ++i) {
+        if (code[i].kind != XP_I_OP) { has[sp++] = code[i].kind == XP_I_HOLE; continue; }
+        --sp;
+        const bool x = has[sp - 1], y = has[sp];
+        if (x || y) {
+            if (code[i].arg > XP_OP_MUL || (code[i].arg == XP_OP_MUL && x && y)) return false;
+            has[sp - 1] = true;
+        }
+    }
+    return true;
+}
 
 struct xp_joint_result {
     int solved = 0, max_total = 0, least_total = 0, least_size[2] = {0, 0};
@@ -275,76 +413,110 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
         return XP_OK;
     }
     const int n_probe = (int)(si.n_points < kJointProbes ? si.n_points : kJointProbes);
-    // one device block: the record, the spec table (if it is the host's), the value tables
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const bool copy_spec = d->spec_kind == XP_SPEC_TABLE && si.n_points > 0 && !d->spec_table_on_device;
-    size_t off = al(sizeof(JointDev));
-    const size_t off_spec = off;
-    if (copy_spec) off += al(sizeof(i64) * (size_t)si.n_points);
-    size_t off_val[2], off_ok[2];
-    for (int k = 0; k < 2; ++k) {
-        off_val[k] = off; off += al(sizeof(i64) * entries[k] * (size_t)(n_probe ? n_probe : 1));
-        off_ok[k] = off; off += al(entries[k] * (size_t)(n_probe ? n_probe : 1));
-    }
-    char* block = nullptr;
-    size_t granted = 0;
-    int bdev = 0;
-    if (device_alloc((void**)&block, off, &bdev, &granted) != cudaSuccess) {
-        (void)cudaGetLastError();
-        delete r;
-        return set_error(XP_ERR_NOMEM, "xp_repair_joint: device memory for the value tables");
-    }
-    h.sk = si.d_s; h.n_probe = n_probe; h.ctx_len = d->ctx_len;
-    memcpy(h.ctx, d->ctx, sizeof(xp_instr) * d->ctx_len);
-    if (d->spec_kind == XP_SPEC_EXPR) { h.spec_len = d->spec_len; memcpy(h.spec, d->spec_expr, sizeof(xp_instr) * d->spec_len); }
-    else if (si.n_points > 0) h.spec_table = copy_spec ? (const i64*)(block + off_spec) : (const i64*)d->spec_table;
-    for (int k = 0; k < 2; ++k) { h.tab_val[k] = (i64*)(block + off_val[k]); h.tab_ok[k] = (unsigned char*)(block + off_ok[k]); }
-    for (int t = 0; t <= kJointTotal; ++t) h.min_key[t] = ~0ull;
-    JointDev* dJ = (JointDev*)block;
+    const bool affine = joint_is_affine(d->ctx, d->ctx_len);
+    const size_t result_at = offsetof(JointDev, match_count), result_bytes = sizeof(JointDev) - result_at;
+    StageMemory stage(sizeof(JointDev));
+    StageEvents ev;
     cudaStream_t stream = opts ? (cudaStream_t)opts->stream : nullptr;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    cudaError_t e = cudaMemcpyAsync(dJ, &h, sizeof(h), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess && copy_spec) e = cudaMemcpyAsync(block + off_spec, d->spec_table, sizeof(i64) * (size_t)si.n_points, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaEventCreate(&e0);
-    if (e == cudaSuccess) e = cudaEventCreate(&e1);
-    if (e == cudaSuccess) e = cudaEventRecord(e0, stream);
-    int launches = 0;
-    if (e == cudaSuccess && n_probe > 0) {
-        joint_probe_kernel<<<1, 32, 0, stream>>>(dJ);
-        ++launches;
-        e = cudaGetLastError();
-        for (int k = 0; k < 2 && e == cudaSuccess; ++k)
-            for (int s = 1; s <= d->max_size[k] && e == cudaSuccess; ++s) {
-                const u64 c = grammar_cnt(si.g, d->start_nt[k], s);
-                if (c == 0) continue;
-                joint_values_kernel<<<dim3((unsigned)((c + 255) / 256), (unsigned)n_probe), 256, 0, stream>>>(dJ, k, s);
-                ++launches;
-                e = cudaGetLastError();
-            }
-        int sms = 148;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        for (int t = 2; t <= r->max_total && e == cudaSuccess; ++t)          // total size ascending (any order gives the same sums and minima)
-            for (int s0 = 1; s0 < t && e == cudaSuccess; ++s0) {
-                const int s1 = t - s0;
-                if (s0 > d->max_size[0] || s1 > d->max_size[1]) continue;
-                const u64 n0 = grammar_cnt(si.g, d->start_nt[0], s0), n1 = grammar_cnt(si.g, d->start_nt[1], s1);
-                if (n0 == 0 || n1 == 0) continue;
-                const u64 want = (n0 * n1 + 255) / 256, most = (u64)sms * 8;
-                joint_pairs_kernel<<<(unsigned)(want < most ? want : most), 256, 0, stream>>>(dJ, s0, s1, n0, n1);
-                ++launches;
-                e = cudaGetLastError();
-            }
-    }
-    JointDev back;
-    if (e == cudaSuccess) e = cudaEventRecord(e1, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&back, dJ, sizeof(back), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream); else cudaStreamSynchronize(stream);
     float ms = 0.f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    if (e0) cudaEventDestroy(e0);
-    if (e1) cudaEventDestroy(e1);
-    device_release(block, granted, bdev);
-    if (e != cudaSuccess) { delete r; return set_error(XP_ERR_CUDA, (std::string("xp_repair_joint: ") + cudaGetErrorString(e)).c_str()); }
+    int launches = 0, sms = 148;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!stage.p) { delete r; return set_error(XP_ERR_NOMEM, "out of host memory"); }
+    JointDev& back = *(JointDev*)stage.p;
+    // The search from one side first where the context allows it; the pair by pair form otherwise, or when more pairs
+    // pass the probes than the list holds.
+    for (int form = affine ? 0 : 1; form < 2; ++form) {
+        // one device block: the record, the spec table (if it is the host's), then the form's tables
+        size_t off = al(sizeof(JointDev));
+        const size_t off_spec = off;
+        if (copy_spec) off += al(sizeof(i64) * (size_t)si.n_points);
+        size_t off_val[2] = {0, 0}, off_ok[2] = {0, 0}, off_head = 0, off_next = 0, off_key = 0, off_list = 0;
+        u32 heads = 1024;
+        while (heads < entries[1]) heads <<= 1;
+        if (form == 0) {
+            off_head = off; off += al(sizeof(u32) * heads);
+            off_next = off; off += al(sizeof(u32) * entries[1]);
+            off_key = off; off += al(sizeof(u64) * entries[1]);
+            off_list = off; off += al(sizeof(uint2) * kJointList);
+        } else
+            for (int k = 0; k < 2; ++k) {
+                off_val[k] = off; off += al(sizeof(i64) * entries[k] * (size_t)n_probe);
+                off_ok[k] = off; off += al(entries[k] * (size_t)n_probe);
+            }
+        char* block = nullptr;
+        size_t granted = 0;
+        int bdev = 0;
+        if (device_alloc((void**)&block, off, &bdev, &granted) != cudaSuccess) {
+            (void)cudaGetLastError();
+            delete r;
+            return set_error(XP_ERR_NOMEM, "xp_repair_joint: device memory for the tables");
+        }
+        h.sk = si.d_s; h.n_probe = n_probe; h.ctx_len = d->ctx_len;
+        memcpy(h.ctx, d->ctx, sizeof(xp_instr) * d->ctx_len);
+        if (d->spec_kind == XP_SPEC_EXPR) { h.spec_len = d->spec_len; memcpy(h.spec, d->spec_expr, sizeof(xp_instr) * d->spec_len); }
+        else if (si.n_points > 0) h.spec_table = copy_spec ? (const i64*)(block + off_spec) : (const i64*)d->spec_table;
+        for (int k = 0; k < 2; ++k) { h.tab_val[k] = (i64*)(block + off_val[k]); h.tab_ok[k] = (unsigned char*)(block + off_ok[k]); }
+        h.head = (u32*)(block + off_head); h.next = (u32*)(block + off_next); h.key = (u64*)(block + off_key); h.list = (uint2*)(block + off_list);
+        h.head_mask = heads - 1;
+        for (int t = 0; t <= kJointTotal; ++t) h.min_key[t] = ~0ull;
+        JointDev* dJ = (JointDev*)block;
+        memcpy(stage.p, &h, sizeof(h));
+        cudaError_t e = ev.e0 ? cudaSuccess : ev.open();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dJ, stage.p, sizeof(h), cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess && copy_spec) e = cudaMemcpyAsync(block + off_spec, d->spec_table, sizeof(i64) * (size_t)si.n_points, cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess && form == 0) e = cudaMemsetAsync(block + off_head, 0xff, sizeof(u32) * heads, stream);
+        if (e == cudaSuccess) e = cudaEventRecord(ev.e0, stream);
+        if (e == cudaSuccess) {
+            joint_probe_kernel<<<1, 32, 0, stream>>>(dJ, form == 0 ? 1 : 0);
+            ++launches;
+            e = cudaGetLastError();
+        }
+        if (form == 0) {
+            for (int part = 1; part >= 0 && e == cudaSuccess; --part) {
+                if (entries[part] == 0) continue;
+                joint_key_kernel<<<(unsigned)((entries[part] + 127) / 128), 128, 0, stream>>>(dJ, part);
+                ++launches;
+                e = cudaGetLastError();
+            }
+            if (e == cudaSuccess) {
+                joint_check_kernel<<<(unsigned)sms * 4, 256, 0, stream>>>(dJ);
+                ++launches;
+                e = cudaGetLastError();
+            }
+        } else {
+            for (int k = 0; k < 2 && e == cudaSuccess; ++k)
+                for (int s = 1; s <= d->max_size[k] && e == cudaSuccess; ++s) {
+                    const u64 c = grammar_cnt(si.g, d->start_nt[k], s);
+                    if (c == 0) continue;
+                    joint_values_kernel<<<dim3((unsigned)((c + 255) / 256), (unsigned)n_probe), 256, 0, stream>>>(dJ, k, s);
+                    ++launches;
+                    e = cudaGetLastError();
+                }
+            for (int t = 2; t <= r->max_total && e == cudaSuccess; ++t)      // total size ascending (any order gives the same sums and minima)
+                for (int s0 = 1; s0 < t && e == cudaSuccess; ++s0) {
+                    const int s1 = t - s0;
+                    if (s0 > d->max_size[0] || s1 > d->max_size[1]) continue;
+                    const u64 n0 = grammar_cnt(si.g, d->start_nt[0], s0), n1 = grammar_cnt(si.g, d->start_nt[1], s1);
+                    if (n0 == 0 || n1 == 0) continue;
+                    const u64 want = (n0 * n1 + 255) / 256, most = (u64)sms * 8;
+                    joint_pairs_kernel<<<(unsigned)(want < most ? want : most), 256, 0, stream>>>(dJ, s0, s1, n0, n1);
+                    ++launches;
+                    e = cudaGetLastError();
+                }
+        }
+        float part_ms = 0.f;
+        if (e == cudaSuccess) e = cudaEventRecord(ev.e1, stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(stage.p + result_at, (char*)dJ + result_at, result_bytes, cudaMemcpyDeviceToHost, stream);
+        const cudaError_t e2 = cudaStreamSynchronize(stream);
+        if (e == cudaSuccess) e = e2;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&part_ms, ev.e0, ev.e1);
+        device_release(block, granted, bdev);
+        if (e != cudaSuccess) { delete r; return set_error(XP_ERR_CUDA, (std::string("xp_repair_joint: ") + cudaGetErrorString(e)).c_str()); }
+        ms += part_ms;
+        if (form == 0 && back.listed <= kJointList) { back.survivors = back.listed; break; }
+    }
     for (int t = 2; t <= r->max_total; ++t) {
         r->match[t] = back.match_count[t];
         if (!r->solved && back.match_count[t] > 0) {

@@ -59,5 +59,23 @@ const HoleDev* sketch_hole_dev(const xp_sketch* s, int hole); // device pointer
 cudaError_t device_alloc(void** out, size_t bytes, int* device, size_t* granted);     // the library's device pool
 void device_release(void* ptr, size_t granted, int device);
 xp_status set_error(xp_status st, const char* msg);
+// Page-locked host memory and a pair of timing events from the library's pools (given back when the holder goes).
+struct StageMemory {
+    StageMemory(size_t bytes);
+    ~StageMemory();
+    char* p;                         // null: out of host memory
+    void* block;
+    StageMemory(const StageMemory&) = delete;
+    StageMemory& operator=(const StageMemory&) = delete;
+};
+struct StageEvents {
+    StageEvents();
+    ~StageEvents();
+    cudaError_t open();
+    cudaEvent_t e0, e1;
+    void* pair;
+    StageEvents(const StageEvents&) = delete;
+    StageEvents& operator=(const StageEvents&) = delete;
+};
 
 }  // namespace xp
