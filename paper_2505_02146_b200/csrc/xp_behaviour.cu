@@ -3,23 +3,26 @@
 //
 // Representatives of every (nonterminal, size) live side by side in device memory: their
 // signatures (n_sig int64 values each) and a 16-byte record (operator or leaf, the two operand
-// representatives).  One pass per (size, nonterminal), in chunks of kChunk candidates:
-//   beh_sig_kernel     -- thread = candidate of the pruned space: finds its (production, left size)
-//                         block, reads the operands' signatures, writes its own to the chunk buffer;
-//   beh_insert_kernel  -- puts the candidate into the nonterminal's hash table (open addressing, one
-//                         64-bit word per class: 24 bits of the signature's hash, a kind bit, an id).
-//                         A word with the same 24 bits is confirmed by comparing the signatures
-//                         themselves.  A class that a representative already owns drops the candidate;
+// representatives).  One pass per (size, nonterminal), in chunks of kBehChunk candidates:
+//   beh_insert_kernel  -- thread = candidate of the pruned space: finds its (production, left size) block, computes its
+//                         signature in registers from the operands' (which stay in cache: a few thousand rows serve
+//                         millions of candidates) and puts it into the nonterminal's hash table (open addressing, one
+//                         64-bit word per class: 24 bits of the signature's hash, a kind bit, an id).  A word with the same
+//                         24 bits is confirmed by comparing the signatures themselves (another candidate's is computed
+//                         again).  A class that a representative already owns drops the candidate;
 //                         among the chunk's candidates the smallest index takes the word (compare-and-
 //                         swap that only ever lowers it: no thread waits for another);
 //   beh_flag_kernel    -- a candidate is new iff its class's word carries its own index; counts per block;
 //   beh_scan_kernel    -- exclusive scan of the block counts (one CTA);
 //   beh_append_kernel  -- the new ones, in candidate order, become representatives: signature and
 //                         record are appended, and the class's word now names the representative.
+// A table starts small and grows with the passes (beh_rehash_kernel puts the representatives into the larger one), so that a
+// call clears what it uses and not what its bound would allow.
 // Then the representatives of the hole's nonterminal are held against the constraint at the
 // signature points (beh_match_kernel) and the few that satisfy it are checked on the whole domain,
 // in order (beh_verify_kernel: thread = point, the representative's tree walked with a small stack).
-// The passes are bound by memory traffic: a candidate moves about 2 * 8 * n_sig + 16 bytes.
+// Candidates' signatures used to be written to memory, read back twice and compared from there: 290 us of a million
+// candidates with 12 points.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -50,29 +53,32 @@ struct BehDev {
     const SketchDev* sk;
     const HoleDev* hole;
     i32 n_sig, n_nt;
-    u32 spec_ok, err;                                     // err: a probe sequence ran its limit (table too full)
+    u32 spec_ok, pad0;
     i64 sig_id[XP_MAX_SIG];
     i64 sig_pt[XP_MAX_SIG][kMaxVars];
     i64 sig_spec[XP_MAX_SIG];
     i64* rep_sig;                                         // [max_reps][n_sig]
     RepDesc* rep_desc;
     u64* table;                                           // [n_nt][table_size]
-    u64 table_size;                                       // a power of two
-    i64* buf_sig;                                         // chunk buffers: [kBehChunk][n_sig]
-    unsigned char* buf_def;
-    u32* buf_flag;
-    u64* buf_slot;
+    u64 table_size;                                       // a power of two: the most a nonterminal's table may have
+    u64* buf_slot;                                        // per candidate of the chunk: slot of its class (kNoSlot: dropped)
     u32* block_count;                                     // per block of the chunk: new candidates, then their exclusive scan
+    // results, read back from here on
     u64 chunk_new;                                        // new representatives of the chunk at hand
+    u32 err, pad;                                         // err: a probe sequence ran its limit (table too full)
     u64 match_count;
-    u32 match_n, verify_fail;
+    u32 match_n, pad2;
     u32 match_id[kMatchCap];
+    u32 verify_fail, n_nodes;                             // whole-domain check of one representative, and its tree in preorder
+    RepDesc node[kMaxSize];
 };
+constexpr u64 kNoSlot = ~0ull;
+constexpr u64 kBehTable = 1ull << 17;                     // slots a table starts with (1 MB: cleared in 2 us)
 
 struct BehBlock { u64 first, cr, lbase, rbase; i32 op, pad; };
 struct BehPass {
     i32 nt, size, n_blocks, leaf_first;                   // size 1: candidates are the leaves leaf_first ...
-    u64 n_cand;
+    u64 n_cand, mask;                                     // mask: the table's size at this pass, less one
     BehBlock blocks[kBehBlocks];
 };
 
@@ -80,12 +86,6 @@ __device__ __forceinline__ u64 sig_hash(const i64* s, int n) {
     u64 h = 0x243F6A8885A308D3ull;
     for (int j = 0; j < n; ++j) { h = (h ^ (u64)s[j]) * 0x9E3779B97F4A7C15ull; h ^= h >> 29; }
     return h;
-}
-
-__device__ __forceinline__ bool sig_equal(const i64* a, const i64* b, int n) {
-    bool eq = true;
-    for (int j = 0; j < n; ++j) eq = eq && a[j] == b[j];
-    return eq;
 }
 
 __global__ void beh_points_kernel(BehDev* B) {
@@ -108,94 +108,152 @@ __global__ void beh_points_kernel(BehDev* B) {
     if (t == 0) B->spec_ok = m;
 }
 
-__global__ void __launch_bounds__(kBehThreads) beh_sig_kernel(BehDev* B, const BehPass P, u64 chunk_first, u32 chunk_n) {
+// Candidate idx of the pass: its operator and its operands (size 1: its leaf).
+struct BehOperands { i32 op; LeafDev leaf; u64 l, r; };
+__device__ __forceinline__ BehOperands beh_operands(const BehDev* B, const BehPass& P, u64 idx) {
+    BehOperands o;
+    o.op = -1; o.l = o.r = 0;
+    o.leaf = LeafDev{-1, 0, 0};
+    if (P.size == 1) { o.leaf = B->sk->g->leaves[P.leaf_first + (i32)idx]; return o; }
+    int b = 0;
+    while (b + 1 < P.n_blocks && P.blocks[b + 1].first <= idx) ++b;
+    const BehBlock& k = P.blocks[b];
+    u64 l, r;
+    divmod_u64(idx - k.first, k.cr, l, r);
+    o.op = k.op; o.l = k.lbase + l; o.r = k.rbase + r;
+    return o;
+}
+
+// Operator OP on two signatures, point by point, given to f(j, value); returns whether all are defined.  The operator is
+// chosen once per candidate (beh_signature): with the choice inside the unrolled loop the kernel was ten times the size and
+// waited for its instructions.
+template <int OP, int NS, typename F>
+__device__ __forceinline__ bool beh_apply(const i64* __restrict__ ls, const i64* __restrict__ rs, int ns, F f) {
+    bool ok = true;
+#pragma unroll
+    for (int j = 0; j < NS; ++j)
+        if (j < ns) {
+            i64 v = 0;
+            ok = apply_op(OP, ls[j], rs[j], v) && ok;
+            f(j, v);
+        }
+    return ok;
+}
+template <int NS, typename F>
+__device__ __forceinline__ bool beh_signature(const BehDev* B, const BehOperands& o, int ns, F f) {
+    const i64* ls = B->rep_sig + o.l * ns;
+    const i64* rs = B->rep_sig + o.r * ns;
+    switch (o.op) {
+        case -1:
+#pragma unroll
+            for (int j = 0; j < NS; ++j) if (j < ns) f(j, o.leaf.var >= 0 ? B->sig_pt[j][o.leaf.var] : o.leaf.value);
+            return true;
+        case XP_OP_ADD: return beh_apply<XP_OP_ADD, NS>(ls, rs, ns, f);
+        case XP_OP_SUB: return beh_apply<XP_OP_SUB, NS>(ls, rs, ns, f);
+        case XP_OP_MUL: return beh_apply<XP_OP_MUL, NS>(ls, rs, ns, f);
+        case XP_OP_DIV: return beh_apply<XP_OP_DIV, NS>(ls, rs, ns, f);
+        case XP_OP_MOD: return beh_apply<XP_OP_MOD, NS>(ls, rs, ns, f);
+        case XP_OP_MIN: return beh_apply<XP_OP_MIN, NS>(ls, rs, ns, f);
+        case XP_OP_MAX: return beh_apply<XP_OP_MAX, NS>(ls, rs, ns, f);
+        case XP_OP_SHL: return beh_apply<XP_OP_SHL, NS>(ls, rs, ns, f);
+        default: return beh_apply<XP_OP_SHR, NS>(ls, rs, ns, f);
+    }
+}
+
+// Is the signature behind a table word (a representative's, or another candidate's of the pass) equal to `mine`?
+template <int NS>
+__device__ __forceinline__ bool beh_same(const BehDev* B, const BehPass& P, u64 word, const i64 (&mine)[NS], int ns) {
+    const u64 id = word & kIdMask;
+    bool eq = true;
+    if (!(word & kKindCand)) {
+        const i64* s = B->rep_sig + id * ns;
+#pragma unroll
+        for (int j = 0; j < NS; ++j) if (j < ns) eq = eq && s[j] == mine[j];
+        return eq;
+    }
+    (void)beh_signature<NS>(B, beh_operands(B, P, id), ns, [&](int j, i64 v) { eq = eq && v == mine[j]; });
+    return eq;
+}
+
+template <int NS>                                         // n_sig <= NS: the signature stays in registers
+__global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, const BehPass P, u64 chunk_first, u32 chunk_n) {
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= chunk_n) return;
-    const u64 idx = chunk_first + c;
     const int ns = B->n_sig;
-    i64* out = B->buf_sig + (u64)c * ns;
-    bool defined = true;
-    if (P.size == 1) {
-        const LeafDev lf = B->sk->g->leaves[P.leaf_first + (i32)idx];
-        for (int j = 0; j < ns; ++j) out[j] = lf.var >= 0 ? B->sig_pt[j][lf.var] : lf.value;
-    } else {
-        int b = 0;
-        while (b + 1 < P.n_blocks && P.blocks[b + 1].first <= idx) ++b;
-        const BehBlock& k = P.blocks[b];
-        const u64 rem = idx - k.first, l = rem / k.cr, r = rem - l * k.cr;
-        const i64* ls = B->rep_sig + (k.lbase + l) * ns;
-        const i64* rs = B->rep_sig + (k.rbase + r) * ns;
-        for (int j = 0; j < ns; ++j) {
-            i64 v = 0;
-            defined = apply_op(k.op, ls[j], rs[j], v) && defined;
-            out[j] = v;
-        }
-    }
-    B->buf_def[c] = defined ? 1 : 0;
-}
-
-// Signature behind a table word: a representative's, or a candidate's of the chunk at hand.
-__device__ __forceinline__ const i64* sig_of(const BehDev* B, u64 word, u64 chunk_first) {
-    const u64 id = word & kIdMask;
-    return (word & kKindCand) ? B->buf_sig + (id - chunk_first) * B->n_sig : B->rep_sig + id * B->n_sig;
-}
-
-__global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, int nt, u64 chunk_first, u32 chunk_n) {
-    const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= chunk_n || !B->buf_def[c]) return;
-    const int ns = B->n_sig;
-    const i64* mine = B->buf_sig + (u64)c * ns;
-    const u64 h = sig_hash(mine, ns), mask = B->table_size - 1;
-    const u64 me = ((h & 0xffffffull) << 40) | kKindCand | (chunk_first + c);
-    u64* tab = B->table + (u64)nt * B->table_size;
-    u64 slot = (h >> 24) & mask;
-    for (u64 step = 0; step <= mask; ++step, slot = (slot + 1) & mask) {
-        u64 w = tab[slot];
-        bool other_class = false;
-        // A failed compare-and-swap means that another thread has just changed the word (claimed it,
-        // or lowered it within this class), never that one must be waited for; the limit only guards
-        // against a mistake in this routine.
-        for (int tries = 0; tries < (1 << 20) && !other_class; ++tries) {
-            if (w == kEmpty) {
-                const u64 old = atomicCAS((unsigned long long*)&tab[slot], kEmpty, me);
-                if (old == kEmpty) return;
+    const BehOperands o = beh_operands(B, P, chunk_first + c);
+    i64 mine[NS];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) mine[j] = 0;
+    const bool defined = beh_signature<NS>(B, o, ns, [&](int j, i64 v) { mine[j] = v; });
+    u64 h = 0x243F6A8885A308D3ull;                        // (sig_hash)
+#pragma unroll
+    for (int j = 0; j < NS; ++j) if (j < ns) { h = (h ^ (u64)mine[j]) * 0x9E3779B97F4A7C15ull; h ^= h >> 29; }
+    u64 place = kNoSlot;
+    if (defined) {
+        const u64 me = ((h & 0xffffffull) << 40) | kKindCand | (chunk_first + c);
+        u64* tab = B->table + (u64)P.nt * B->table_size;
+        u64 slot = (h >> 24) & P.mask;
+        bool done = false;
+        for (u64 step = 0; step <= P.mask && !done; ++step, slot = (slot + 1) & P.mask) {
+            u64 w = tab[slot];
+            bool other_class = false;
+            // A failed compare-and-swap means that another thread has just changed the word (claimed it,
+            // or lowered it within this class), never that one must be waited for; the limit only guards
+            // against a mistake in this routine.
+            for (int tries = 0; tries < (1 << 20); ++tries) {
+                if (w == kEmpty) {
+                    const u64 old = atomicCAS((unsigned long long*)&tab[slot], kEmpty, me);
+                    if (old == kEmpty) { place = slot; done = true; break; }
+                    w = old;
+                    continue;
+                }
+                if ((w >> 40) != (me >> 40) || !beh_same<NS>(B, P, w, mine, ns)) { other_class = true; break; }
+                if (!(w & kKindCand) || w <= me) { done = true; break; }      // a representative, or an earlier candidate, owns the class
+                const u64 old = atomicCAS((unsigned long long*)&tab[slot], w, me);
+                if (old == w) { place = slot; done = true; break; }
                 w = old;
-                continue;
             }
-            if ((w >> 40) != (me >> 40) || !sig_equal(mine, sig_of(B, w, chunk_first), ns)) { other_class = true; break; }
-            if (!(w & kKindCand) || w <= me) return;      // a representative, or an earlier candidate, owns the class
-            const u64 old = atomicCAS((unsigned long long*)&tab[slot], w, me);
-            if (old == w) return;
-            w = old;
+            if (!done && !other_class) break;             // (the limit ran out)
         }
-        if (!other_class) break;                          // (the limit ran out)
+        if (!done) atomicOr(&B->err, 1u);
     }
-    atomicOr(&B->err, 1u);
+    B->buf_slot[c] = place;
 }
 
 __global__ void __launch_bounds__(kBehThreads) beh_flag_kernel(BehDev* B, int nt, u64 chunk_first, u32 chunk_n) {
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     bool is_new = false;
-    if (c < chunk_n && B->buf_def[c]) {
-        const int ns = B->n_sig;
-        const i64* mine = B->buf_sig + (u64)c * ns;
-        const u64 h = sig_hash(mine, ns), mask = B->table_size - 1;
-        const u64 me = ((h & 0xffffffull) << 40) | kKindCand | (chunk_first + c);
-        const u64* tab = B->table + (u64)nt * B->table_size;
-        u64 slot = (h >> 24) & mask;
-        for (u64 step = 0; step <= mask; ++step, slot = (slot + 1) & mask) {
-            const u64 w = tab[slot];
-            if (w == kEmpty) { atomicOr(&B->err, 2u); break; }          // (cannot happen: the class was inserted)
-            if ((w >> 40) == (me >> 40) && sig_equal(mine, sig_of(B, w, chunk_first), ns)) {
-                is_new = w == me;
-                B->buf_slot[c] = slot;
-                break;
-            }
+    if (c < chunk_n) {
+        const u64 slot = B->buf_slot[c];
+        if (slot != kNoSlot) {                            // it has held its class's word: does it still?
+            is_new = (B->table[(u64)nt * B->table_size + slot] & ((1ull << 40) - 1)) == (kKindCand | (chunk_first + c));
+            if (!is_new) B->buf_slot[c] = kNoSlot;
         }
     }
-    if (c < chunk_n) B->buf_flag[c] = is_new ? 1u : 0u;
     const int n = __syncthreads_count(is_new);
     if (threadIdx.x == 0) B->block_count[blockIdx.x] = (u32)n;
+}
+
+// A nonterminal's representatives, by size.
+struct BehRanges { i32 n; i32 pad; u64 first[kMaxSize], count[kMaxSize], total; };
+__device__ __forceinline__ u64 range_id(const BehRanges& R, u64 i) {
+    int k = 0;
+    while (k + 1 < R.n && i >= R.count[k]) { i -= R.count[k]; ++k; }
+    return R.first[k] + i;
+}
+
+// Representatives of a nonterminal into its (cleared) table.
+__global__ void __launch_bounds__(kBehThreads) beh_rehash_kernel(BehDev* B, int nt, u64 mask, const BehRanges R) {
+    const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= R.total) return;
+    const u64 id = range_id(R, i);
+    const u64 h = sig_hash(B->rep_sig + id * B->n_sig, B->n_sig);
+    const u64 word = ((h & 0xffffffull) << 40) | id;
+    u64* tab = B->table + (u64)nt * B->table_size;
+    u64 slot = (h >> 24) & mask;
+    for (u64 step = 0; step <= mask; ++step, slot = (slot + 1) & mask)       // (their signatures differ: the first free slot)
+        if (atomicCAS((unsigned long long*)&tab[slot], kEmpty, word) == kEmpty) return;
+    atomicOr(&B->err, 1u);
 }
 
 __global__ void __launch_bounds__(1024) beh_scan_kernel(BehDev* B, int n_blocks) {
@@ -222,7 +280,7 @@ __global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, cons
     __shared__ u32 warp_sum[kBehThreads / 32];
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool is_new = c < chunk_n && B->buf_flag[c] != 0;
+    const bool is_new = c < chunk_n && B->buf_slot[c] != kNoSlot;
     const u32 bal = __ballot_sync(0xffffffffu, is_new);
     if (lane == 0) warp_sum[warp] = (u32)__popc(bal);
     __syncthreads();
@@ -231,40 +289,35 @@ __global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, cons
     for (int w = 0; w < warp; ++w) pos += warp_sum[w];
     const u64 gid = rep_base + pos;
     const int ns = B->n_sig;
-    const i64* mine = B->buf_sig + (u64)c * ns;
-    i64* dst = B->rep_sig + gid * ns;
-    for (int j = 0; j < ns; ++j) dst[j] = mine[j];
     const u64 idx = chunk_first + c;
+    const BehOperands o = beh_operands(B, P, idx);
+    i64* dst = B->rep_sig + gid * ns;
+    (void)beh_signature<XP_MAX_SIG>(B, o, ns, [&](int j, i64 v) { dst[j] = v; });
     RepDesc d;
     d.size = (u32)P.size;
     if (P.size == 1) { d.op_or_leaf = kLeafBit | (u32)(P.leaf_first + (i32)idx); d.left = d.right = 0; }
-    else {
-        int b = 0;
-        while (b + 1 < P.n_blocks && P.blocks[b + 1].first <= idx) ++b;
-        const BehBlock& k = P.blocks[b];
-        const u64 rem = idx - k.first, l = rem / k.cr, r = rem - l * k.cr;
-        d.op_or_leaf = (u32)k.op; d.left = (u32)(k.lbase + l); d.right = (u32)(k.rbase + r);
-    }
+    else { d.op_or_leaf = (u32)o.op; d.left = (u32)o.l; d.right = (u32)o.r; }
     B->rep_desc[gid] = d;
     u64* tab = B->table + (u64)P.nt * B->table_size;
     const u64 slot = B->buf_slot[c];
     tab[slot] = (tab[slot] & ~((1ull << 40) - 1)) | gid;  // the class's word now names the representative
 }
 
-// Representatives [first, first + n) of the hole's nonterminal against the constraint at the signature points.
-__global__ void __launch_bounds__(kBehThreads) beh_match_kernel(BehDev* B, u64 first, u64 n) {
+// All of them against the constraint at the signature points.
+__global__ void __launch_bounds__(kBehThreads) beh_match_kernel(BehDev* B, const BehRanges R) {
     const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= R.total) return;
+    const u64 id = range_id(R, i);
     const int ns = B->n_sig;
     const u32 all = ns >= 32 ? 0xffffffffu : (1u << ns) - 1u;
     if ((B->spec_ok & all) != all) return;                // the spec is undefined at a signature point: nothing satisfies it
-    const i64* s = B->rep_sig + (first + i) * ns;
+    const i64* s = B->rep_sig + id * ns;
     bool ok = true;
     for (int j = 0; j < ns && ok; ++j) ok = ctx_matches(B->hole, B->sig_pt[j], s[j], B->sig_spec[j]);
     if (!ok) return;
     atomicAdd((unsigned long long*)&B->match_count, 1ull);
     const u32 at = atomicAdd(&B->match_n, 1u);
-    if (at < (u32)kMatchCap) B->match_id[at] = (u32)(first + i);
+    if (at < (u32)kMatchCap) B->match_id[at] = (u32)id;
 }
 
 // Value of representative `gid` at one point: its tree is walked with an explicit stack.
@@ -303,6 +356,17 @@ __device__ bool rep_value(const BehDev* B, u32 gid, const i64* pt, i64& out) {
 __global__ void __launch_bounds__(kBehThreads) beh_verify_kernel(BehDev* B, u32 gid) {
     const SketchDev* sk = B->sk;
     const HoleDev* hole = B->hole;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {            // its tree, for the text: nodes in preorder
+        u32 todo[kMaxSize + 1];
+        int n = 0, k = 0;
+        todo[n++] = gid;
+        while (n > 0 && k < kMaxSize) {
+            const RepDesc d = B->rep_desc[todo[--n]];
+            B->node[k++] = d;
+            if (!(d.op_or_leaf & kLeafBit) && n + 2 <= kMaxSize + 1) { todo[n++] = d.right; todo[n++] = d.left; }
+        }
+        B->n_nodes = (u32)k;
+    }
     for (i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x; pid < sk->n_points; pid += (i64)gridDim.x * blockDim.x) {
         if (*(volatile u32*)&B->verify_fail) return;
         i64 pt[kMaxVars];
@@ -343,16 +407,13 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
     const u64 max_reps = d->max_representatives ? d->max_representatives : (1ull << 22);
     if (max_reps >= (1ull << 31)) return set_error(XP_ERR_TOO_LARGE, "xp_behaviours: max_representatives must stay below 2^31");
     u64 tsize = 1024;
-    while (tsize < 2 * max_reps + 2 * kBehChunk) tsize <<= 1;
+    while (tsize < 2 * max_reps + 2 * kBehChunk) tsize <<= 1;      // (at least kBehTable)
     // one device block
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     size_t off = al(sizeof(BehDev));
     const size_t o_sig = off;   off += al(sizeof(i64) * max_reps * ns);
     const size_t o_desc = off;  off += al(sizeof(RepDesc) * max_reps);
     const size_t o_tab = off;   off += al(sizeof(u64) * tsize * n_nt);
-    const size_t o_bsig = off;  off += al(sizeof(i64) * kBehChunk * ns);
-    const size_t o_bdef = off;  off += al(kBehChunk);
-    const size_t o_bflag = off; off += al(sizeof(u32) * kBehChunk);
     const size_t o_bslot = off; off += al(sizeof(u64) * kBehChunk);
     const size_t o_bcnt = off;  off += al(sizeof(u32) * (kBehChunk / kBehThreads + 1));
     char* block = nullptr;
@@ -362,26 +423,35 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
         (void)cudaGetLastError();
         return set_error(XP_ERR_NOMEM, ("xp_behaviours: device memory (" + std::to_string(off) + " bytes)").c_str());
     }
-    BehDev h;
+    StageMemory stage(2 * sizeof(BehDev));                // what goes out, and what comes back behind it
+    StageEvents ev;
+    if (!stage.p) { device_release(block, granted, bdev); return set_error(XP_ERR_NOMEM, "out of host memory"); }
+    BehDev& h = *(BehDev*)stage.p;
+    BehDev& back = *(BehDev*)(stage.p + sizeof(BehDev));
     memset(&h, 0, sizeof(h));
     h.sk = si.d_s; h.hole = sketch_hole_dev(sketch, d->hole); h.n_sig = ns; h.n_nt = n_nt;
     for (int j = 0; j < ns; ++j) h.sig_id[j] = d->sig_points[j];
     h.rep_sig = (i64*)(block + o_sig); h.rep_desc = (RepDesc*)(block + o_desc);
     h.table = (u64*)(block + o_tab); h.table_size = tsize;
-    h.buf_sig = (i64*)(block + o_bsig); h.buf_def = (unsigned char*)(block + o_bdef);
-    h.buf_flag = (u32*)(block + o_bflag); h.buf_slot = (u64*)(block + o_bslot); h.block_count = (u32*)(block + o_bcnt);
+    h.buf_slot = (u64*)(block + o_bslot); h.block_count = (u32*)(block + o_bcnt);
     BehDev* dB = (BehDev*)block;
     cudaStream_t stream = opts ? (cudaStream_t)opts->stream : nullptr;
+    constexpr size_t kBackAt = offsetof(BehDev, chunk_new);
     Cuda cu;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    cu(cudaEventCreate(&e0));
-    cu(cudaEventCreate(&e1));
+    cu(ev.open());
     cu(cudaMemcpyAsync(dB, &h, sizeof(h), cudaMemcpyHostToDevice, stream));
-    cu(cudaMemsetAsync(block + o_tab, 0xff, sizeof(u64) * tsize * n_nt, stream));
-    cu(cudaEventRecord(e0, stream));
+    if (cu.ok()) cu(cudaEventRecord(ev.e0, stream));
     int launches = 0;
     if (cu.ok()) { beh_points_kernel<<<1, 32, 0, stream>>>(dB); ++launches; cu(cudaGetLastError()); }
     std::vector<std::vector<u64>> count(n_nt, std::vector<u64>(K + 1, 0)), base(n_nt, std::vector<u64>(K + 1, 0));
+    std::vector<u64> table(n_nt, 0), held(n_nt, 0);       // per nonterminal: size of its table so far, representatives in it
+    auto ranges_of = [&](int nt) {
+        BehRanges R;
+        memset(&R, 0, sizeof(R));
+        for (int s = 1; s <= K; ++s)
+            if (count[nt][s] > 0) { R.first[R.n] = base[nt][s]; R.count[R.n++] = count[nt][s]; R.total += count[nt][s]; }
+        return R;
+    };
     u64 n_reps = 0, bytes = 0;
     xp_status st = XP_OK;
     std::string why;
@@ -409,14 +479,27 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
             for (u64 first = 0; first < P.n_cand && cu.ok() && st == XP_OK; first += kBehChunk) {
                 const u32 n = (u32)(P.n_cand - first < kBehChunk ? P.n_cand - first : kBehChunk);
                 const int nb = (int)((n + kBehThreads - 1) / kBehThreads);
-                beh_sig_kernel<<<nb, kBehThreads, 0, stream>>>(dB, P, first, n);
-                beh_insert_kernel<<<nb, kBehThreads, 0, stream>>>(dB, nt, first, n);
+                // room for every candidate of the chunk at half the slots
+                u64 want = table[nt] ? table[nt] : kBehTable;
+                while (want < 2 * (held[nt] + n)) want <<= 1;
+                if (want > tsize) want = tsize;
+                if (want != table[nt]) {
+                    cu(cudaMemsetAsync((u64*)(block + o_tab) + tsize * nt, 0xff, sizeof(u64) * want, stream));
+                    const BehRanges R = ranges_of(nt);
+                    if (R.total > 0 && cu.ok()) {
+                        beh_rehash_kernel<<<(unsigned)((R.total + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream>>>(dB, nt, want - 1, R);
+                        ++launches;
+                    }
+                    table[nt] = want;
+                }
+                P.mask = table[nt] - 1;
+                if (ns <= 8) beh_insert_kernel<8><<<nb, kBehThreads, 0, stream>>>(dB, P, first, n);
+                else beh_insert_kernel<XP_MAX_SIG><<<nb, kBehThreads, 0, stream>>>(dB, P, first, n);
                 beh_flag_kernel<<<nb, kBehThreads, 0, stream>>>(dB, nt, first, n);
                 beh_scan_kernel<<<1, 1024, 0, stream>>>(dB, nb);
-                launches += 4;
+                launches += 3;
                 cu(cudaGetLastError());
-                BehDev back;
-                cu(cudaMemcpyAsync(&back, dB, offsetof(BehDev, match_count), cudaMemcpyDeviceToHost, stream));
+                cu(cudaMemcpyAsync(&back.chunk_new, (char*)dB + kBackAt, 2 * sizeof(u64), cudaMemcpyDeviceToHost, stream));
                 cu(cudaStreamSynchronize(stream));
                 if (!cu.ok()) break;
                 if (back.err) { st = XP_ERR_TOO_LARGE; why = "xp_behaviours: the hash table is too full (raise max_representatives)"; break; }
@@ -429,6 +512,7 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
                 ++launches;
                 cu(cudaGetLastError());
                 n_reps += back.chunk_new;
+                held[nt] += back.chunk_new;
                 count[nt][s] += back.chunk_new;
                 bytes += back.chunk_new * (u64)(2 * 8 * ns + 24);
             }
@@ -437,15 +521,10 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
     // the hole's representatives against the constraint, then the whole-domain checks in order
     std::vector<u32> ids;
     if (cu.ok() && st == XP_OK) {
-        for (int s = 1; s <= K; ++s)
-            if (count[hs.start_nt][s] > 0) {
-                const u64 n = count[hs.start_nt][s];
-                beh_match_kernel<<<(unsigned)((n + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream>>>(dB, base[hs.start_nt][s], n);
-                ++launches;
-            }
+        const BehRanges R = ranges_of(hs.start_nt);
+        if (R.total > 0) { beh_match_kernel<<<(unsigned)((R.total + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream>>>(dB, R); ++launches; }
         cu(cudaGetLastError());
-        BehDev back;
-        cu(cudaMemcpyAsync(&back, dB, sizeof(back), cudaMemcpyDeviceToHost, stream));
+        cu(cudaMemcpyAsync(&back.chunk_new, (char*)dB + kBackAt, sizeof(BehDev) - kBackAt, cudaMemcpyDeviceToHost, stream));
         cu(cudaStreamSynchronize(stream));
         if (cu.ok()) {
             out->sig_matches = back.match_count;
@@ -459,39 +538,42 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
         for (int s = 1; s <= K; ++s)
             if (gid >= base[hs.start_nt][s] && gid < base[hs.start_nt][s] + count[hs.start_nt][s]) { *size = s; *index = gid - base[hs.start_nt][s]; }
     };
-    std::function<bool(u32, std::string&)> text_of = [&](u32 gid, std::string& t) -> bool {
-        RepDesc r;
-        if (cudaMemcpy(&r, (char*)block + o_desc + sizeof(RepDesc) * gid, sizeof(r), cudaMemcpyDeviceToHost) != cudaSuccess) return false;
+    // text of the tree that the last whole-domain check left in `back` (nodes in preorder)
+    std::function<void(u32&, std::string&)> text_of = [&](u32& at, std::string& t) {
+        if (at >= back.n_nodes) return;
+        const RepDesc r = back.node[at++];
         if (r.op_or_leaf & kLeafBit) {
             const LeafDev& lf = gh.leaves[r.op_or_leaf & ~kLeafBit];
             t += lf.var >= 0 ? std::string(gh.var_names[lf.var]) : std::to_string((long long)lf.value);
-            return true;
+            return;
         }
         static const char* const kText[] = {"+", "-", "*", "/", "%", "<", "<=", "==", "!=", "min", "max", "&&", "||", "<<", ">>"};
         const bool call = r.op_or_leaf == XP_OP_MIN || r.op_or_leaf == XP_OP_MAX;
         t += call ? std::string(kText[r.op_or_leaf]) + "(" : std::string("(");
-        if (!text_of(r.left, t)) return false;
+        text_of(at, t);
         t += call ? "," : kText[r.op_or_leaf];
-        if (!text_of(r.right, t)) return false;
+        text_of(at, t);
         t += ")";
-        return true;
     };
+    int sms = 148;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    constexpr size_t kCheckAt = offsetof(BehDev, verify_fail);
     for (size_t k = 0; k < ids.size() && cu.ok() && st == XP_OK && !out->solved; ++k) {
-        cu(cudaMemsetAsync((char*)dB + offsetof(BehDev, verify_fail), 0, sizeof(u32), stream));
-        int sms = 148;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (k > 0) cu(cudaMemsetAsync((char*)dB + kCheckAt, 0, sizeof(u32), stream));
         const i64 want = (si.n_points + kBehThreads - 1) / kBehThreads;
-        if (want > 0) { beh_verify_kernel<<<(unsigned)(want < sms * 8 ? want : sms * 8), kBehThreads, 0, stream>>>(dB, ids[k]); ++launches; }
+        beh_verify_kernel<<<(unsigned)(want < 1 ? 1 : want < sms * 8 ? want : sms * 8), kBehThreads, 0, stream>>>(dB, ids[k]);
+        ++launches;
         cu(cudaGetLastError());
-        u32 fail = 0;
-        cu(cudaMemcpyAsync(&fail, (char*)dB + offsetof(BehDev, verify_fail), sizeof(fail), cudaMemcpyDeviceToHost, stream));
+        cu(cudaMemcpyAsync(&back.verify_fail, (char*)dB + kCheckAt, sizeof(BehDev) - kCheckAt, cudaMemcpyDeviceToHost, stream));
         cu(cudaStreamSynchronize(stream));
         if (!cu.ok()) break;
+        const u32 fail = back.verify_fail;
         std::string t;
         int size = 0;
         u64 index = 0;
         locate(ids[k], &size, &index);
-        if (k == 0 || !fail) text_of(ids[k], t);
+        u32 node = 0;
+        text_of(node, t);
         if (k == 0) {
             out->hit = 1; out->hit_size = size; out->hit_index = index; out->hit_verified = fail ? 0 : 1;
             snprintf(out->hit_text, sizeof(out->hit_text), "%s", t.c_str());
@@ -502,10 +584,8 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
         }
     }
     float ms = 0.f;
-    if (cu.ok()) { cu(cudaEventRecord(e1, stream)); cu(cudaEventSynchronize(e1)); cu(cudaEventElapsedTime(&ms, e0, e1)); }
+    if (cu.ok()) { cu(cudaEventRecord(ev.e1, stream)); cu(cudaEventSynchronize(ev.e1)); cu(cudaEventElapsedTime(&ms, ev.e0, ev.e1)); }
     else cudaStreamSynchronize(stream);
-    if (e0) cudaEventDestroy(e0);
-    if (e1) cudaEventDestroy(e1);
     device_release(block, granted, bdev);
     if (!cu.ok()) return set_error(XP_ERR_CUDA, (std::string("xp_behaviours: ") + cudaGetErrorString(cu.e)).c_str());
     if (st != XP_OK) return set_error(st, why.c_str());
