@@ -249,6 +249,11 @@ static void build_counts(xp_grammar* g) {
     }
 }
 
+static u32 reciprocal(i64 v) {       // (ConstDev::recip)
+    const u64 m = v < 0 ? 0ull - (u64)v : (u64)v;
+    return m == 0 || m >> 31 ? 0u : m == 1 ? 0xffffffffu : (u32)((1ull << 32) / m);
+}
+
 extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** out) {
     if (!d || !out) return fail(XP_ERR_INVALID_ARG, "xp_grammar_create: null argument");
     *out = nullptr;
@@ -299,11 +304,11 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
     for (int nt = 0; nt < g->n_nt; ++nt) {
         const int lb = g->leaf_begin[nt], le = g->leaf_begin[nt + 1];
         g->const_begin[nt] = (int)g->consts.size();
-        for (int i = lb; i < le; ++i) if (g->leaves[i].var < 0) g->consts.push_back(ConstDev{g->leaves[i].value, i - lb, 0});
+        for (int i = lb; i < le; ++i) if (g->leaves[i].var < 0) g->consts.push_back(ConstDev{g->leaves[i].value, i - lb, reciprocal(g->leaves[i].value)});
         std::sort(g->consts.begin() + g->const_begin[nt], g->consts.end(), [](const ConstDev& a, const ConstDev& b) {
             return a.value != b.value ? a.value < b.value : a.pos < b.pos; });
         g->var_begin[nt] = (int)g->consts.size();
-        for (int i = lb; i < le; ++i) if (g->leaves[i].var >= 0) g->consts.push_back(ConstDev{g->leaves[i].var, i - lb, 0});
+        for (int i = lb; i < le; ++i) if (g->leaves[i].var >= 0) g->consts.push_back(ConstDev{g->leaves[i].var, i - lb, 0u});
     }
     g->const_begin[g->n_nt] = (int)g->consts.size();
     build_counts(g);

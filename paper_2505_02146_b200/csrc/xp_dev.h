@@ -82,7 +82,9 @@ struct JoinSet {                      // the leaves of one nonterminal, for one 
     JoinEntry e[kJoinEntries];
 };
 
-struct ConstDev { i64 value; i32 pos, pad; };    // a constant leaf of a nonterminal (position among its leaves)
+// A constant leaf of a nonterminal (position among its leaves); recip: floor(2^32 / |value|), 2^32 - 1 for 1, 0 for 0 and
+// values of 2^31 or more.
+struct ConstDev { i64 value; i32 pos; u32 recip; };
 
 struct HoleDev {
     i32 start_nt, max_size, ctx_len, spec_len;   // spec_len == 0: the spec is a table

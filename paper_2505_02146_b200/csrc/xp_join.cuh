@@ -17,8 +17,9 @@
 // one (a suspect) waits in the warp's first queue until 32 have gathered; then every lane takes one, finds the leaves its
 // conditions leave open (binary search among the sorted constants) and holds each against both probes.  What is left
 // goes to a second queue, and 32 at a time (a lane each, none idle) are checked exactly, in 64 bits, at the other probes.
-// A context that compares asks for an interval of values at every probe: sums and differences with a constant
-// are decided by intersecting the intervals over all probes, the other operators leaf by leaf with an early exit.
+// A context that compares asks for an interval of values at every probe.  Every operator but % is monotone in a constant
+// (on either side of zero, for a / c): its constants are one or two runs, the intersection of the probes' intervals
+// (range_runs); remainders are tested constant by constant at the first probe with reciprocals.
 // Operands of JoinSet::lim or more and shifts take the exact form: one operand at a time, lanes over the leaves.
 // Warps work on their own; nothing here waits for another warp.
 #pragma once
@@ -131,6 +132,65 @@ __device__ __forceinline__ bool probe_accepts(const HoleDev* hole, int j, i64 v)
 }
 
 __device__ __forceinline__ int op_of_slot(int slot) { return slot <= 4 ? slot : slot <= 6 ? slot - 5 + XP_OP_MIN : slot - 7 + XP_OP_SHL; }
+
+// Candidates checked one by one look at the probes four at a time: their table entries lie in four places that nothing has
+// touched before, and one probe after the other a candidate that passes 16 probes waits 16 times for memory (the direct
+// tickets of a small search: 20.7 -> 18.6 us).  Candidates of the join mostly end at the next probe and keep the plain order.
+constexpr int kProbeStep = 4;
+
+// An operand's values at the probes j0 .. j0 + 3 (those below n); returns the mask of those it is defined at.
+__device__ __forceinline__ u32 ref_value4(const GrammarDev* g, const HoleDev* hole, const OperandRef& r, int nt, int size, int j0, int n, i64 (&v)[kProbeStep]) {
+    u32 ok = 0;
+    if (r.mode == 2) {
+#pragma unroll 1
+        for (int k = 0; k < kProbeStep; ++k) {
+            i64 x = 0;
+            if (j0 + k < n && ref_value_full(g, hole, nt, size, r.a, j0 + k, x)) ok |= 1u << k;
+#pragma unroll
+            for (int q = 0; q < kProbeStep; ++q) if (q == k) v[q] = x;
+        }
+        return ok;
+    }
+    const u64 total = hole->tab_total;
+    const bool in = XP_CHECKED(n <= hole->tab_probes && r.a < total && r.b < total, kChkTable);
+    i64 y[kProbeStep];
+#pragma unroll
+    for (int k = 0; k < kProbeStep; ++k) {
+        v[k] = 0; y[k] = 0;
+        if (j0 + k < n && in) {
+            const u64 at = (u64)(j0 + k) * total;
+            ok |= (u32)(hole->tab_ok[at + r.a] != 0) << k;
+            v[k] = hole->tab_val[at + r.a];
+            if (r.mode == 1) { if (!hole->tab_ok[at + r.b]) ok &= ~(1u << k); y[k] = hole->tab_val[at + r.b]; }
+        }
+    }
+    if (r.mode == 1) {
+#pragma unroll 1
+        for (int k = 0; k < kProbeStep; ++k) {
+            i64 x = v[0], z = y[0];
+#pragma unroll
+            for (int q = 1; q < kProbeStep; ++q) if (q == k) { x = v[q]; z = y[q]; }
+            if (((ok >> k) & 1u) && !apply_op(r.op, x, z, x)) ok &= ~(1u << k);
+#pragma unroll
+            for (int q = 0; q < kProbeStep; ++q) if (q == k) v[q] = x;
+        }
+    }
+    return ok;
+}
+
+// Do the values v at the probes j0 .. j0 + 3 (those below n) satisfy the constraint?
+__device__ __forceinline__ bool probes_accept(const HoleDev* hole, int j0, int n, const i64 (&v)[kProbeStep]) {
+    const u32 aff = hole->aff_okmask >> j0;
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < kProbeStep; ++k) {
+        if (j0 + k >= n) continue;
+        const int j = j0 + k;
+        if ((aff >> k) & 1u) ok = ok && (u64)v[k] * hole->aff_Aj[j] + hole->aff_Bj[j] == (u64)hole->probe_spec[j];
+        else if (v[k] > -(1ll << 62) && v[k] < (1ll << 62)) ok = ok && v[k] >= hole->rng_lo[j] && v[k] <= hole->rng_hi[j];
+    }
+    return ok;
+}
 
 // The candidate (operand, leaf) at the probes that have tables, in order; the first failure ends it.
 __device__ __forceinline__ bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
@@ -962,6 +1022,60 @@ __device__ __forceinline__ bool narrow_op(int slot, i32 x, i32 y, i64& v) {
     }
 }
 
+// The constants c of the ascending list [cb, vb) for which  a op c  (swap: c op a) can lie in [lo, hi] at all of the
+// kRangeProbes probes, as up to two runs.  For * / min and max; a necessary condition: bounds are taken in double
+// precision and widened by more than its rounding.
+__device__ __noinline__ void range_runs(const ConstDev* c, i32 cb, i32 vb, int slot, int swap, const i32 (&a)[kRangeProbes], const i64 (&lo)[kRangeProbes],
+                                        const i64 (&hi)[kRangeProbes], i32 (&run)[4]) {
+    run[0] = run[1] = run[2] = run[3] = cb;
+    constexpr i64 kEnd = (1ll << 31) + 1;
+    constexpr double kEps = 1e-15;
+    auto clip = [](double x) { return (i64)(x < -2147483650.0 ? -2147483650.0 : x > 2147483650.0 ? 2147483650.0 : x); };
+    if (slot == kSlotDiv && !swap) {                      // floor(|a| / |c|) in an interval that depends on the signs
+        i64 f[2] = {1, 1}, t[2] = {kEnd, kEnd};           // |c| for c > 0 and c < 0
+        for (int j = 0; j < kRangeProbes; ++j) {
+            const double u = fabs((double)a[j]);
+            for (int k = 0; k < 2; ++k) {
+                const bool same = (a[j] >= 0) == (k == 0);
+                const i64 L = same ? lo[j] : -hi[j], H = same ? hi[j] : -lo[j];
+                if (H < 0) { t[k] = 0; continue; }
+                const i64 from = clip(floor(u / ((double)H + 1.0) * (1.0 - kEps))) + 1;
+                f[k] = from > f[k] ? from : f[k];
+                if (L > 0) { const i64 to = clip(floor(u / (double)L * (1.0 + kEps))); t[k] = to < t[k] ? to : t[k]; }
+            }
+        }
+        if (f[0] <= t[0]) { run[0] = const_lower(c, cb, vb, f[0]); run[1] = const_lower(c, run[0], vb, t[0] + 1); }
+        if (f[1] <= t[1]) { run[2] = const_lower(c, cb, vb, -t[1]); run[3] = const_lower(c, run[2], vb, -f[1] + 1); }
+        return;
+    }
+    i64 f = -kEnd, t = kEnd;
+    for (int j = 0; j < kRangeProbes; ++j) {
+        const i64 l = lo[j], h = hi[j], v = a[j];
+        i64 from = -kEnd, to = kEnd;
+        if (slot == kSlotMul) {
+            if (v == 0) { if (l > 0 || h < 0) return; }
+            else {
+                const double q0 = (double)(v > 0 ? l : h) / (double)v, q1 = (double)(v > 0 ? h : l) / (double)v;
+                from = clip(ceil(q0 - fabs(q0) * kEps)); to = clip(floor(q1 + fabs(q1) * kEps));
+            }
+        } else if (slot == kSlotDiv) {                    // c / a
+            if (v == 0) return;
+            const i64 m = v < 0 ? -v : v;
+            i64 L = v > 0 ? l : -h, H = v > 0 ? h : -l;   // c / |a| in [L, H]
+            L = L < -kEnd ? -kEnd : L > kEnd ? kEnd : L; H = H < -kEnd ? -kEnd : H > kEnd ? kEnd : H;
+            from = L > 0 ? L * m : (L - 1) * m + 1; to = H < 0 ? H * m : (H + 1) * m - 1;
+        } else if (slot == kSlotMn) {
+            if (v < l) return;
+            from = l; if (v > h) to = h;
+        } else {
+            if (v > h) return;
+            to = h; if (v < l) from = l;
+        }
+        f = from > f ? from : f; t = to < t ? to : t;
+    }
+    if (f <= t) { run[0] = const_lower(c, cb, vb, f); run[1] = const_lower(c, run[0], vb, t + 1); }
+}
+
 // Operands [first, first + count) of a segment against the leaves, for a hole whose context compares: the value has to
 // lie in [rng_lo, rng_hi] at every probe.
 __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
@@ -1016,53 +1130,94 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         const u32 off = (u32)(e - seg.e_begin);
         const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
         if (n_live == 0u) continue;
+        auto accepted = [&](int slot, int swap, const i32 (&cv)[kRangeProbes]) {      // at the first nr probes
+            bool ok = true;
+#pragma unroll 1
+            for (int j = 0; j < nr && ok; ++j) {
+                i32 x = a[0], y = cv[0];
+                i64 l = lo[0], h = hi[0], v = 0;
+#pragma unroll
+                for (int k = 1; k < kRangeProbes; ++k) if (k == j) { x = a[k]; y = cv[k]; l = lo[k]; h = hi[k]; }
+                ok = narrow_op(slot, swap ? y : x, swap ? x : y, v) && v >= l && v <= h;
+            }
+            return ok;
+        };
+        auto give = [&](bool on, u32 pos, int gi, int slot, int swap) {
+            const u32 b = __ballot_sync(0xffffffffu, on);
+            if (!b) return;
+            n.suspects += (u32)__popc(b);
+            join_push(w, plan, seg, sk, hole, on, off, pos, gi, slot, swap, 0, n);
+        };
+        const u32 ua = abs_u32(a[0]), ra = ua <= 1u ? 0xffffffffu : 0xffffffffu / ua;
+        // remainders at the first probe: |value| in [mlo, mhi] for a value of a's sign / of a positive / negative constant's sign
+        auto clip31 = [](i64 v) { return (u32)(v < 0 ? 0 : v > 0x7fffffffll ? 0x7fffffffll : v); };
+        const u32 plo = clip31(lo[0]), phi = clip31(hi[0]), nlo = clip31(-hi[0]), nhi = clip31(-lo[0]);
+        const bool can_p = hi[0] >= 0, can_n = lo[0] <= 0;       // some value >= 0 / <= 0 is in range
         for (int gi = 0; gi < seg.n_groups; ++gi) {
             const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
             const i32 cb = g->const_begin[grp.leaf_nt], vb = g->var_begin[grp.leaf_nt], ve = g->const_begin[grp.leaf_nt + 1];
-            constexpr u32 kLinear = (1u << kSlotAdd) | (1u << kSlotSub);
             for (int swap = 0; swap < 2; ++swap) {
                 const u32 mask = swap ? grp.smask : grp.fmask;
-                // constants: sums and differences by the intersection of the probes' intervals
-                for (u32 m = mask & kLinear; m; m &= m - 1) {
+                n.tests += (u64)n_live * (u64)(__popc(mask) * (1 + ve - vb));
+                for (u32 m = cb < vb ? mask & ~(1u << kSlotMod) : 0u; m; m &= m - 1) {
                     const int slot = __ffs((int)m) - 1;
-                    const i64 from = slot == kSlotAdd ? pl : swap ? ml : -ph, to = slot == kSlotAdd ? ph : swap ? mh : -pl;
-                    i32 i0 = cb, i1 = cb;
-                    if (live && from <= to) { i0 = const_lower(g->consts, cb, vb, from); i1 = const_lower(g->consts, i0, vb, to + 1); }
-                    n.tests += n_live;
-                    for (i32 i = 0; __any_sync(0xffffffffu, i0 + i < i1); ++i) {
-                        const bool on = i0 + i < i1;
-                        n.suspects += (u32)__popc(__ballot_sync(0xffffffffu, on));
-                        join_push(w, plan, seg, sk, hole, on, off, on ? (u32)g->consts[i0 + i].pos : 0u, gi, slot, swap, 0, n);
+                    i32 run[4] = {cb, cb, cb, cb};
+                    if (slot <= kSlotSub) {               // by the intersection over all probes
+                        const i64 from = slot == kSlotAdd ? pl : swap ? ml : -ph, to = slot == kSlotAdd ? ph : swap ? mh : -pl;
+                        if (live && from <= to) { run[0] = const_lower(g->consts, cb, vb, from); run[1] = const_lower(g->consts, run[0], vb, to + 1); }
+                    } else if (live) range_runs(g->consts, cb, vb, slot, swap, a, lo, hi, run);
+                    const i32 len0 = run[1] - run[0], len = len0 + run[3] - run[2];
+                    for (i32 i = 0; __any_sync(0xffffffffu, i < len); ++i) {
+                        bool on = i < len;
+                        const ConstDev c = g->consts[on ? (i < len0 ? run[0] + i : run[2] + i - len0) : cb];
+                        if (on && slot > kSlotSub) {
+                            const i32 cv[kRangeProbes] = {(i32)c.value, (i32)c.value, (i32)c.value, (i32)c.value};
+                            on = accepted(slot, swap, cv);
+                        }
+                        give(on, (u32)c.pos, gi, slot, swap);
                     }
                 }
-                // the rest leaf by leaf
-                const u32 others = mask & ~kLinear;
-                for (i32 ci = others ? cb : vb; ci < ve; ++ci) {
+                if (((mask >> kSlotMod) & 1u) && cb < vb) {
+                    const u32 alo = a[0] >= 0 ? plo : nlo, ahi = a[0] >= 0 ? phi : nhi;
+                    const bool can = live && (swap ? ua != 0u : a[0] >= 0 ? can_p : can_n);
+                    if (__any_sync(0xffffffffu, can))
+                        for (i32 ci = cb; ci < vb; ++ci) {
+                            const ConstDev c = g->consts[ci];
+                            const u32 uc = abs_u32((i32)c.value);
+                            u32 r, l = alo, h = ahi;
+                            bool on = can;
+                            if (!swap) {
+                                if (uc == 0u) continue;
+                                r = ua - __umulhi(ua, c.recip) * uc;
+                                if (r >= uc) r -= uc;
+                            } else {
+                                r = uc - __umulhi(uc, ra) * ua;
+                                if (r >= ua) r -= ua;
+                                if (c.value >= 0) { l = plo; h = phi; on = on && can_p; } else { l = nlo; h = nhi; on = on && can_n; }
+                            }
+                            on = on && r - l <= h - l;
+                            if (!__any_sync(0xffffffffu, on)) continue;
+                            if (on) {
+                                const i32 cv[kRangeProbes] = {(i32)c.value, (i32)c.value, (i32)c.value, (i32)c.value};
+                                on = accepted(kSlotMod, swap, cv);
+                            }
+                            give(on, (u32)c.pos, gi, kSlotMod, swap);
+                        }
+                }
+                for (i32 ci = vb; ci < ve; ++ci) {        // variables one by one
                     const ConstDev c = g->consts[ci];
                     i32 cv[kRangeProbes];
 #pragma unroll
-                    for (int j = 0; j < kRangeProbes; ++j) cv[j] = (i32)(ci < vb ? c.value : hole->probe_pt[j < nr ? j : 0][c.value]);
-                    for (u32 m = ci < vb ? others : mask; m; m &= m - 1) {
+                    for (int j = 0; j < kRangeProbes; ++j) cv[j] = (i32)hole->probe_pt[j < nr ? j : 0][c.value];
+                    for (u32 m = mask; m; m &= m - 1) {
                         const int slot = __ffs((int)m) - 1;
-                        n.tests += n_live;
-                        bool on = live;
-#pragma unroll
-                        for (int j = 0; j < kRangeProbes; ++j) {
-                            i64 v = 0;
-                            on = on && narrow_op(slot, swap ? cv[j] : a[j], swap ? a[j] : cv[j], v) && v >= lo[j] && v <= hi[j];
-                            if (!__any_sync(0xffffffffu, on)) break;
-                        }
-                        const u32 b = __ballot_sync(0xffffffffu, on);
-                        if (!b) continue;
-                        n.suspects += (u32)__popc(b);
-                        join_push(w, plan, seg, sk, hole, on, off, (u32)c.pos, gi, slot, swap, nr, n);
+                        give(live && accepted(slot, swap, cv), (u32)c.pos, gi, slot, swap);
                     }
                 }
-                // (what was pushed with different first probes is not mixed in one check)
-                if (w.nc) join_check(w, plan, seg, sk, hole, 0, n);
             }
         }
     }
+    if (w.nc) join_check(w, plan, seg, sk, hole, 0, n);
 }
 
 // Candidates [first, first + count) of (start nonterminal, size) themselves, checked on the probes one by one.
@@ -1078,10 +1233,11 @@ __device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, con
         if (rank < first + count) {
             const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, rank);
             pass = true;
-            for (int j = 0; j < n_exact && pass; ++j) {
-                ++n.evals;
-                i64 v;
-                pass = ref_value(g, hole, ref, seg.nt, seg.esize, j, v) && probe_accepts(hole, j, v);
+            for (int j0 = 0; j0 < n_exact && pass; j0 += kProbeStep) {
+                const int here = n_exact - j0 < kProbeStep ? n_exact - j0 : kProbeStep;
+                n.evals += (u64)here;
+                i64 v[kProbeStep];
+                pass = ref_value4(g, hole, ref, seg.nt, seg.esize, j0, n_exact, v) == (1u << here) - 1u && probes_accept(hole, j0, n_exact, v);
             }
             if (pass && n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
             vars = ref_vars(hole, ref);
