@@ -73,7 +73,7 @@ struct JoinWarp {
     u32 q_off[kJoinQueue];                                // suspects: operand number relative to the segment's first,
     i32 q_a0[kJoinQueue], q_a1[kJoinQueue];               //   its values at the two probes
     u32 c_off[64], c_pos[64], c_code[64];                 // candidates: operand, leaf position, group << 8 | slot << 1 | swapped
-    u32 nc;                                               // candidates waiting
+    u32 nq, nc;                                           // suspects and candidates waiting (of segment `seg`)
     GroupCtx grp[kJoinGroups];
     CandShared cand;                                      // candidate of a whole-domain check that the warp does itself
 };
@@ -551,12 +551,25 @@ __device__ __noinline__ void const_runs(const ConstDev* c, i32 lo, i32 hi, int s
     }
 }
 
+// v = x op y at one probe for narrow x, y; false when undefined.
+__device__ __forceinline__ bool narrow_op(int slot, i32 x, i32 y, i64& v) {
+    switch (slot) {
+        case kSlotAdd: v = (i64)x + y; return true;
+        case kSlotSub: v = (i64)x - y; return true;
+        case kSlotMul: v = (i64)x * y; return true;
+        case kSlotDiv: if (y == 0) return false; v = y == -1 ? -(i64)x : (i64)(x / y); return true;
+        case kSlotMod: if (y == 0) return false; v = y == -1 ? 0 : (i64)(x % y); return true;
+        case kSlotMn: v = x < y ? x : y; return true;
+        default: v = x > y ? x : y; return true;
+    }
+}
+
 // The suspects in the warp's first queue, one per lane.  Called by all 32 lanes together.
-__device__ __noinline__ void join_drain(JoinWarp& w, u32 n_q, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
-                                        const JoinCtx& x, JoinCount& n) {
+__device__ __noinline__ void join_drain(JoinWarp& w, u32 n_q, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
     __syncwarp();
+    const JoinCtx& x = w.x;
     n.suspects += n_q;
     const i64 t0 = hole->join_t0, t1 = hole->join_t1;
     const u64 tmod = hole->join_tmod;
@@ -564,52 +577,62 @@ __device__ __noinline__ void join_drain(JoinWarp& w, u32 n_q, const PlanDev& pla
     for (u32 at = 0; at < n_q; at += 32) {
         const bool live = at + lane < n_q;
         const u32 off = live ? w.q_off[at + lane] : 0u;
-        const i32 b0[1] = {live ? w.q_a0[at + lane] : 0}, b1[1] = {live ? w.q_a1[at + lane] : 0};
+        const i32 b0 = live ? w.q_a0[at + lane] : 0, b1 = live ? w.q_a1[at + lane] : 0;
+        auto holds = [&](int slot, int swap, i32 x0, i32 x1, i32 c0, i32 c1) {       // exactly, at both probes
+            i64 v = 0;
+            return narrow_op(slot, swap ? c0 : x0, swap ? x0 : c0, v) && v == t0 && narrow_op(slot, swap ? c1 : x1, swap ? x1 : c1, v) && v == t1;
+        };
         for (int gi = 0; gi < seg.n_groups; ++gi) {
             const GroupCtx& s = w.grp[gi];
             const JoinSet* S = s.set;
-            const u32 ef = s.ef, es = s.es;
-            if (ef | es)
+            if (s.ef | s.es)
                 for (int i = 0; i < s.n_entries; ++i) {
-                    const JoinEntry en = S->e[i];
-                    bool any[1] = {false};
-                    entry_conditions<1>(en, ef, es, b0, b1, x, any);
-                    if (!__any_sync(0xffffffffu, live && any[0])) continue;
+                    const i32 v0 = (i32)S->e[i].v0, v1 = (i32)S->e[i].v1;
+                    const u32 pos = S->e[i].pos;
                     for (int swap = 0; swap < 2; ++swap)
-                        for (u32 m = swap ? es : ef; m; m &= m - 1) {
-                            const u32 bit = m & (0u - m);
-                            const int slot = __ffs((int)bit) - 1;
-                            bool one[1] = {false};
-                            entry_conditions<1>(en, swap ? 0u : bit, swap ? bit : 0u, b0, b1, x, one);
-                            bool on = live && one[0];
-                            if (on) {                     // exactly, at both probes
-                                i64 v = 0;
-                                on = apply_op(op_of_slot(slot), swap ? (i64)(i32)en.v0 : b0[0], swap ? b0[0] : (i64)(i32)en.v0, v) && v == t0 &&
-                                     apply_op(op_of_slot(slot), swap ? (i64)(i32)en.v1 : b1[0], swap ? b1[0] : (i64)(i32)en.v1, v) && v == t1;
-                            }
-                            join_push(w, plan, seg, sk, hole, on, off, en.pos, gi, slot, swap, from, n);
+#pragma unroll 1
+                        for (u32 m = swap ? s.es : s.ef; m; m &= m - 1) {
+                            const int slot = __ffs((int)m) - 1;
+                            join_push(w, plan, seg, sk, hole, live && holds(slot, swap, b0, b1, v0, v1), off, pos, gi, slot, swap, from, n);
                         }
                 }
             if (!(s.cf | s.cs)) continue;
             const i32 clo = S->const_begin, chi = clo + S->n_const;
             for (int swap = 0; swap < 2; ++swap)
+#pragma unroll 1
                 for (u32 m = swap ? s.cs : s.cf; m; m &= m - 1) {
                     const int slot = __ffs((int)m) - 1;
-                    const bool act = live && const_condition(slot, swap, b0[0], b1[0], x, s);
+                    const bool act = live && const_condition(slot, swap, b0, b1, x, s);
                     if (!__any_sync(0xffffffffu, act)) continue;
                     i32 run[4] = {clo, clo, clo, clo};
-                    if (act) const_runs(g->consts, clo, chi, slot, swap, b0[0], b1[0], t0, t1, tmod, run);
+                    if (act) const_runs(g->consts, clo, chi, slot, swap, b0, b1, t0, t1, tmod, run);
                     const i32 len0 = run[1] - run[0], len = len0 + run[3] - run[2];
-                    for (i32 i = 0; __any_sync(0xffffffffu, act && i < len); ++i) {
-                        bool on = act && i < len;
-                        const ConstDev c = g->consts[on ? (i < len0 ? run[0] + i : run[2] + i - len0) : clo];
-                        if (on) {
-                            i64 v = 0;
-                            on = apply_op(op_of_slot(slot), swap ? c.value : b0[0], swap ? b0[0] : c.value, v) && v == t0 &&
-                                 apply_op(op_of_slot(slot), swap ? c.value : b1[0], swap ? b1[0] : c.value, v) && v == t1;
+                    // A lane per suspect, or, where few suspects have long runs (a remainder leaves every constant above the
+                    // target open), the suspects one after the other with the lanes over their constants.
+                    const i32 longest = (i32)__reduce_max_sync(0xffffffffu, (u32)len);
+                    const i32 steps = (i32)__reduce_add_sync(0xffffffffu, (u32)((len + 31) / 32));
+                    if (longest <= steps) {
+                        for (i32 i = 0; i < longest; ++i) {
+                            bool on = i < len;
+                            const ConstDev c = g->consts[on ? (i < len0 ? run[0] + i : run[2] + i - len0) : clo];
+                            if (on) on = holds(slot, swap, b0, b1, (i32)c.value, (i32)c.value);
+                            join_push(w, plan, seg, sk, hole, on, off, (u32)c.pos, gi, slot, swap, from, n);
                         }
-                        join_push(w, plan, seg, sk, hole, on, off, (u32)c.pos, gi, slot, swap, from, n);
-                    }
+                    } else
+                        for (u32 q = __ballot_sync(0xffffffffu, len > 0); q; q &= q - 1) {
+                            const int src = __ffs((int)q) - 1;
+                            const i32 r0 = __shfl_sync(0xffffffffu, run[0], src), r2 = __shfl_sync(0xffffffffu, run[2], src);
+                            const i32 n0 = __shfl_sync(0xffffffffu, len0, src), nn = __shfl_sync(0xffffffffu, len, src);
+                            const i32 x0 = __shfl_sync(0xffffffffu, b0, src), x1 = __shfl_sync(0xffffffffu, b1, src);
+                            const u32 o = __shfl_sync(0xffffffffu, off, src);
+                            for (i32 i0 = 0; i0 < nn; i0 += 32) {
+                                const i32 i = i0 + lane;
+                                bool on = i < nn;
+                                const ConstDev c = g->consts[on ? (i < n0 ? r0 + i : r2 + i - n0) : clo];
+                                if (on) on = holds(slot, swap, x0, x1, (i32)c.value, (i32)c.value);
+                                join_push(w, plan, seg, sk, hole, on, o, (u32)c.pos, gi, slot, swap, from, n);
+                            }
+                        }
                 }
         }
     }
@@ -915,7 +938,7 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     const int n_lin = w.hot.n_lin, n_mul = w.hot.n_mul, n_other = w.hot.n_other, n_set = w.hot.n_set;
     const u32 mul_t = w.hot.mul_t;
     const u32 tests_each = w.hot.tests;
-    u32 nq = 0;
+    u32 nq = w.nq;
     u32 n_alive = 0;
     for (u64 done = 0; done < count;) {
         const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done);
@@ -980,7 +1003,7 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
                 }
                 if (nq >= 32u) {                          // whole warps of suspects; the rest waits
                     const u32 full = nq & ~31u;
-                    join_drain(w, full, plan, seg, sk, hole, x, n);
+                    join_drain(w, full, plan, seg, sk, hole, n);
                     nq -= full;
                     u32 o = 0;
                     i32 v0 = 0, v1 = 0;
@@ -1000,27 +1023,26 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
         done += n_run;
     }
     n.tests += (u64)tests_each * (u64)__reduce_add_sync(0xffffffffu, n_alive);
-    if (nq) join_drain(w, nq, plan, seg, sk, hole, x, n);
+    if (lane == 0) w.nq = nq;                             // (fewer than 32: they wait for the warp's next ticket of this segment)
+    __syncwarp();
+}
+
+// What waits in the warp's queues when it leaves segment `index`.
+__device__ __noinline__ void join_leave(JoinWarp& w, const PlanDev& plan, int index, JoinCount& n) {
+    const JoinSeg& seg = plan.jsegs[index];
+    const SketchDev* sk = plan.sketches[seg.sketch];
+    const HoleDev* hole = &sk->holes[seg.hole];
+    if (w.nq) join_drain(w, w.nq, plan, seg, sk, hole, n);
     if (w.nc) join_check(w, plan, seg, sk, hole, hole->join_p1 ? 2 : 1, n);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) { w.nq = 0; w.seg = -1; }
+    __syncwarp();
 }
 
 // ---- contexts that compare ----
 
 // Operand values at the first kRangeProbes probes sit in registers; leaves are held against those with an early exit.
 constexpr int kRangeProbes = 4;
-
-// v = x op y at one probe for narrow x, y; false when undefined.
-__device__ __forceinline__ bool narrow_op(int slot, i32 x, i32 y, i64& v) {
-    switch (slot) {
-        case kSlotAdd: v = (i64)x + y; return true;
-        case kSlotSub: v = (i64)x - y; return true;
-        case kSlotMul: v = (i64)x * y; return true;
-        case kSlotDiv: if (y == 0) return false; v = y == -1 ? -(i64)x : (i64)(x / y); return true;
-        case kSlotMod: if (y == 0) return false; v = y == -1 ? 0 : (i64)(x % y); return true;
-        case kSlotMn: v = x < y ? x : y; return true;
-        default: v = x > y ? x : y; return true;
-    }
-}
 
 // The constants c of the ascending list [cb, vb) for which  a op c  (swap: c op a) can lie in [lo, hi] at all of the
 // kRangeProbes probes, as up to two runs.  For * / min and max; a necessary condition: bounds are taken in double
@@ -1253,7 +1275,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const PlanDev pla
     __shared__ JoinWarp sh[kJoinWarps];
     JoinWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    if (lane == 0) { w.nc = 0; w.seg = -1; }
+    if (lane == 0) { w.nq = 0; w.nc = 0; w.seg = -1; }
     __syncwarp();
     JoinCount n{0, 0, 0, 0, 0};
     int acc = -1;
@@ -1274,6 +1296,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const PlanDev pla
             lo = nlo;
         }
         const JoinSeg& seg = plan.jsegs[lo];
+        if (w.seg >= 0 && w.seg != lo) join_leave(w, plan, w.seg, n);
         if (seg.acc != acc) { join_flush(plan, acc, n); acc = seg.acc; }
         const SketchDev* sk = plan.sketches[seg.sketch];
         const HoleDev* hole = &sk->holes[seg.hole];
@@ -1294,6 +1317,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const PlanDev pla
         if (lane == 0) next = atomicAdd(plan.join_ticket, 1ull);
         t = plan.join_base + warps + __shfl_sync(0xffffffffu, next, 0);
     }
+    if (w.seg >= 0) join_leave(w, plan, w.seg, n);
     join_flush(plan, acc, n);
 }
 
