@@ -1434,7 +1434,7 @@ static JoinSeg new_join_seg(int sketch, int hole, int acc, int k, u64 lo, u64 hi
 // Leaf-join segments of (start nonterminal, size k >= 3) restricted to ranks [lo, hi): one per operand nonterminal, with
 // a group per leaf nonterminal, for every operator with a leaf of it on either side of such an operand.  Copies of one
 // production open segments of their own; so do shifts, which only the exact form knows.
-static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool exact) {
+static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool exact, bool compares) {
     struct Open { JoinSeg seg; std::vector<JoinGroup> groups; };
     std::vector<Open> open;
     for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
@@ -1467,7 +1467,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
             if (!at) {
                 Open c;
                 c.seg = new_join_seg(sketch, hole, acc, k, lo, hi);
-                c.seg.kind = kJoinLeaf; c.seg.nt = ent; c.seg.esize = k - 2; c.seg.exact = ex ? 1 : 0;
+                c.seg.kind = kJoinLeaf; c.seg.nt = ent; c.seg.esize = k - 2; c.seg.exact = ex ? 1 : 0; c.seg.heavy = ex || compares ? 1 : 0;
                 c.seg.e_begin = e0; c.seg.e_count = e1 - e0;
                 open.push_back(c);
                 at = &open.back();
@@ -1516,6 +1516,9 @@ static void add_direct(Plan* plan, int nt, int sketch, int hole, int acc, int k,
 // warps spend their time taking tickets.  64 steps at most.
 static void number_joins(Plan* plan) {
     if (plan->jsegs.empty()) return;
+    // the heavy tickets of a few large sketches first, so that none of them is a call's last (batches are long enough to even out)
+    if (plan->jsegs.size() <= 64)
+        std::stable_sort(plan->jsegs.begin(), plan->jsegs.end(), [](const JoinSeg& a, const JoinSeg& b) { return a.heavy > b.heavy; });
     u64 steps = 0;
     for (const JoinSeg& c : plan->jsegs) steps += c.exact ? c.e_count : (c.e_count + 31) / 32;
     u64 per = steps / ((u64)search_warps() * 4);
@@ -1626,7 +1629,7 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, b
                 const bool forced = (o->flags & XP_FLAG_ALWAYS_FILTER) != 0;
                 if (!ho.filter_ok || (o->flags & XP_FLAG_NO_FILTER)) { add_linear(plan, (int)i, h, acc, k, lo, hi); continue; }
                 if (k < 3 || (!forced && hi - lo < kTileMinRanks)) { add_direct(plan, ho.start_nt, (int)i, h, acc, k, lo, hi); continue; }
-                add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact);
+                add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact, ho.compares);
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi);
                 add_tiles(plan, s->g, pairs ? &ho : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile);
             }

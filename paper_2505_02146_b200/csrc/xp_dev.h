@@ -217,7 +217,7 @@ struct JoinSeg {
     i32 first_group;
     i32 exact;                       // the operators have no condition (shifts): every candidate is evaluated on its own
     u32 chunk;                       // operands per ticket
-    i32 pad;
+    i32 heavy;                       // an operand costs many times the usual (exact form, contexts that compare): these go first
     u64 e_begin, e_count;
 };
 

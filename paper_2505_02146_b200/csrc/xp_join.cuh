@@ -1098,6 +1098,30 @@ __device__ __noinline__ void range_runs(const ConstDev* c, i32 cb, i32 vb, int s
     if (f <= t) { run[0] = const_lower(c, cb, vb, f); run[1] = const_lower(c, run[0], vb, t + 1); }
 }
 
+// Is  x op y  in range at all of the kRangeProbes probes?  The operator is chosen once, the probes are straight-line code.
+template <int SLOT>
+__device__ __forceinline__ bool range_holds(const i32 (&x)[kRangeProbes], const i32 (&y)[kRangeProbes], const i64 (&lo)[kRangeProbes], const i64 (&hi)[kRangeProbes]) {
+    bool ok = true;
+#pragma unroll
+    for (int j = 0; j < kRangeProbes; ++j) {
+        i64 v = 0;
+        ok = narrow_op(SLOT, x[j], y[j], v) && ok && v >= lo[j] && v <= hi[j];
+    }
+    return ok;
+}
+__device__ __forceinline__ bool range_accepts(int slot, const i32 (&x)[kRangeProbes], const i32 (&y)[kRangeProbes], const i64 (&lo)[kRangeProbes],
+                                              const i64 (&hi)[kRangeProbes]) {
+    switch (slot) {
+        case kSlotAdd: return range_holds<kSlotAdd>(x, y, lo, hi);
+        case kSlotSub: return range_holds<kSlotSub>(x, y, lo, hi);
+        case kSlotMul: return range_holds<kSlotMul>(x, y, lo, hi);
+        case kSlotDiv: return range_holds<kSlotDiv>(x, y, lo, hi);
+        case kSlotMod: return range_holds<kSlotMod>(x, y, lo, hi);
+        case kSlotMn: return range_holds<kSlotMn>(x, y, lo, hi);
+        default: return range_holds<kSlotMx>(x, y, lo, hi);
+    }
+}
+
 // Operands [first, first + count) of a segment against the leaves, for a hole whose context compares: the value has to
 // lie in [rng_lo, rng_hi] at every probe.
 __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
@@ -1153,16 +1177,10 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
         if (n_live == 0u) continue;
         auto accepted = [&](int slot, int swap, const i32 (&cv)[kRangeProbes]) {      // at the first nr probes
-            bool ok = true;
-#pragma unroll 1
-            for (int j = 0; j < nr && ok; ++j) {
-                i32 x = a[0], y = cv[0];
-                i64 l = lo[0], h = hi[0], v = 0;
+            i32 x[kRangeProbes], y[kRangeProbes];
 #pragma unroll
-                for (int k = 1; k < kRangeProbes; ++k) if (k == j) { x = a[k]; y = cv[k]; l = lo[k]; h = hi[k]; }
-                ok = narrow_op(slot, swap ? y : x, swap ? x : y, v) && v >= l && v <= h;
-            }
-            return ok;
+            for (int j = 0; j < kRangeProbes; ++j) { x[j] = swap ? cv[j] : a[j]; y[j] = swap ? a[j] : cv[j]; }
+            return range_accepts(slot, x, y, lo, hi);
         };
         auto give = [&](bool on, u32 pos, int gi, int slot, int swap) {
             const u32 b = __ballot_sync(0xffffffffu, on);
@@ -1170,11 +1188,24 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
             n.suspects += (u32)__popc(b);
             join_push(w, plan, seg, sk, hole, on, off, pos, gi, slot, swap, 0, n);
         };
-        const u32 ua = abs_u32(a[0]), ra = ua <= 1u ? 0xffffffffu : 0xffffffffu / ua;
-        // remainders at the first probe: |value| in [mlo, mhi] for a value of a's sign / of a positive / negative constant's sign
-        auto clip31 = [](i64 v) { return (u32)(v < 0 ? 0 : v > 0x7fffffffll ? 0x7fffffffll : v); };
-        const u32 plo = clip31(lo[0]), phi = clip31(hi[0]), nlo = clip31(-hi[0]), nhi = clip31(-lo[0]);
-        const bool can_p = hi[0] >= 0, can_n = lo[0] <= 0;       // some value >= 0 / <= 0 is in range
+        // Remainders: magnitude in [mag, mag + span] for a value >= 0 (0) or <= 0 (1); kNever where no such value is in range.
+        constexpr u32 kNever = 0x80000000u;
+        auto bound = [](i64 l, i64 h, u32& from, u32& span) {
+            if (h < 0 || l > 0x7fffffffll) { from = kNever; span = 0; return; }
+            from = l < 0 ? 0u : (u32)l;
+            span = (u32)(h > 0x7fffffffll ? 0x7fffffffll : h) - from;
+            if (h < (i64)from) { from = kNever; span = 0; }
+        };
+        u32 ua[kRangeProbes], ra[kRangeProbes], pm[kRangeProbes], ps[kRangeProbes], nm[kRangeProbes], ns[kRangeProbes];
+        bool none0 = false;                               // some a is zero (no remainder by it)
+#pragma unroll
+        for (int j = 0; j < kRangeProbes; ++j) {
+            ua[j] = abs_u32(a[j]);
+            ra[j] = ua[j] <= 1u ? 0xffffffffu : 0xffffffffu / ua[j];
+            none0 = none0 || ua[j] == 0u;
+            bound(lo[j], hi[j], pm[j], ps[j]);
+            bound(-hi[j], -lo[j], nm[j], ns[j]);
+        }
         for (int gi = 0; gi < seg.n_groups; ++gi) {
             const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
             const i32 cb = g->const_begin[grp.leaf_nt], vb = g->var_begin[grp.leaf_nt], ve = g->const_begin[grp.leaf_nt + 1];
@@ -1200,30 +1231,40 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
                     }
                 }
                 if (((mask >> kSlotMod) & 1u) && cb < vb) {
-                    const u32 alo = a[0] >= 0 ? plo : nlo, ahi = a[0] >= 0 ? phi : nhi;
-                    const bool can = live && (swap ? ua != 0u : a[0] >= 0 ? can_p : can_n);
-                    if (__any_sync(0xffffffffu, can))
-                        for (i32 ci = cb; ci < vb; ++ci) {
+                    if (!swap) {                          // a % c: the sign of a
+                        u32 m[kRangeProbes], sp[kRangeProbes];
+                        bool can = live;
+#pragma unroll
+                        for (int j = 0; j < kRangeProbes; ++j) {
+                            m[j] = a[j] >= 0 ? pm[j] : nm[j]; sp[j] = a[j] >= 0 ? ps[j] : ns[j];
+                            can = can && m[j] != kNever;
+                        }
+                        if (__any_sync(0xffffffffu, can))
+                            for (i32 ci = cb; ci < vb; ++ci) {
+                                const ConstDev c = g->consts[ci];
+                                const u32 uc = abs_u32((i32)c.value);
+                                if (uc == 0u) continue;
+                                bool on = can;
+#pragma unroll
+                                for (int j = 0; j < kRangeProbes; ++j) {
+                                    u32 r = ua[j] - __umulhi(ua[j], c.recip) * uc;
+                                    if (r >= uc) r -= uc;
+                                    on = on && r - m[j] <= sp[j];
+                                }
+                                give(on, (u32)c.pos, gi, kSlotMod, 0);
+                            }
+                    } else if (__any_sync(0xffffffffu, live && !none0))
+                        for (i32 ci = cb; ci < vb; ++ci) {      // c % a: the sign of c
                             const ConstDev c = g->consts[ci];
                             const u32 uc = abs_u32((i32)c.value);
-                            u32 r, l = alo, h = ahi;
-                            bool on = can;
-                            if (!swap) {
-                                if (uc == 0u) continue;
-                                r = ua - __umulhi(ua, c.recip) * uc;
-                                if (r >= uc) r -= uc;
-                            } else {
-                                r = uc - __umulhi(uc, ra) * ua;
-                                if (r >= ua) r -= ua;
-                                if (c.value >= 0) { l = plo; h = phi; on = on && can_p; } else { l = nlo; h = nhi; on = on && can_n; }
+                            bool on = live && !none0;
+#pragma unroll
+                            for (int j = 0; j < kRangeProbes; ++j) {
+                                u32 r = uc - __umulhi(uc, ra[j]) * ua[j];
+                                if (r >= ua[j]) r -= ua[j];
+                                on = on && (c.value >= 0 ? r - pm[j] <= ps[j] : r - nm[j] <= ns[j]);
                             }
-                            on = on && r - l <= h - l;
-                            if (!__any_sync(0xffffffffu, on)) continue;
-                            if (on) {
-                                const i32 cv[kRangeProbes] = {(i32)c.value, (i32)c.value, (i32)c.value, (i32)c.value};
-                                on = accepted(kSlotMod, swap, cv);
-                            }
-                            give(on, (u32)c.pos, gi, kSlotMod, swap);
+                            give(on, (u32)c.pos, gi, kSlotMod, 1);
                         }
                 }
                 for (i32 ci = vb; ci < ve; ++ci) {        // variables one by one
