@@ -1044,22 +1044,25 @@ __device__ __noinline__ void join_leave(JoinWarp& w, const PlanDev& plan, int in
 // Operand values at the first kRangeProbes probes sit in registers; leaves are held against those with an early exit.
 constexpr int kRangeProbes = 4;
 
-// The constants c of the ascending list [cb, vb) for which  a op c  (swap: c op a) can lie in [lo, hi] at all of the
-// kRangeProbes probes, as up to two runs.  For * / min and max; a necessary condition: bounds are taken in double
-// precision and widened by more than its rounding.
-__device__ __noinline__ void range_runs(const ConstDev* c, i32 cb, i32 vb, int slot, int swap, const i32 (&a)[kRangeProbes], const i64 (&lo)[kRangeProbes],
-                                        const i64 (&hi)[kRangeProbes], i32 (&run)[4]) {
+// The constants c of the ascending list [cb, vb) for which  a op c  (swap: c op a) can lie in the hole's interval at all np
+// probes (a: the operand's values there), as up to two runs.  For * / min and max; a necessary condition: bounds are taken
+// in double precision and widened by more than its rounding.  (With four probes instead of all the runs were so much
+// longer that testing them was most of the ticket.)
+__device__ __noinline__ void range_runs(const HoleDev* hole, int np, const ConstDev* c, i32 cb, i32 vb, int slot, int swap, const i32 (&a)[kMaxProbe],
+                                        i32 (&run)[4]) {
+    constexpr i64 kMost = 1ll << 62;
     run[0] = run[1] = run[2] = run[3] = cb;
     constexpr i64 kEnd = (1ll << 31) + 1;
     constexpr double kEps = 1e-15;
     auto clip = [](double x) { return (i64)(x < -2147483650.0 ? -2147483650.0 : x > 2147483650.0 ? 2147483650.0 : x); };
     if (slot == kSlotDiv && !swap) {                      // floor(|a| / |c|) in an interval that depends on the signs
         i64 f[2] = {1, 1}, t[2] = {kEnd, kEnd};           // |c| for c > 0 and c < 0
-        for (int j = 0; j < kRangeProbes; ++j) {
+        for (int j = 0; j < np && (f[0] <= t[0] || f[1] <= t[1]); ++j) {
             const double u = fabs((double)a[j]);
+            const i64 l = hole->rng_lo[j] < -kMost ? -kMost : hole->rng_lo[j], h = hole->rng_hi[j] > kMost ? kMost : hole->rng_hi[j];
             for (int k = 0; k < 2; ++k) {
                 const bool same = (a[j] >= 0) == (k == 0);
-                const i64 L = same ? lo[j] : -hi[j], H = same ? hi[j] : -lo[j];
+                const i64 L = same ? l : -h, H = same ? h : -l;
                 if (H < 0) { t[k] = 0; continue; }
                 const i64 from = clip(floor(u / ((double)H + 1.0) * (1.0 - kEps))) + 1;
                 f[k] = from > f[k] ? from : f[k];
@@ -1071,8 +1074,8 @@ __device__ __noinline__ void range_runs(const ConstDev* c, i32 cb, i32 vb, int s
         return;
     }
     i64 f = -kEnd, t = kEnd;
-    for (int j = 0; j < kRangeProbes; ++j) {
-        const i64 l = lo[j], h = hi[j], v = a[j];
+    for (int j = 0; j < np && f <= t; ++j) {
+        const i64 l = hole->rng_lo[j] < -kMost ? -kMost : hole->rng_lo[j], h = hole->rng_hi[j] > kMost ? kMost : hole->rng_hi[j], v = a[j];
         i64 from = -kEnd, to = kEnd;
         if (slot == kSlotMul) {
             if (v == 0) { if (l > 0 || h < 0) return; }
@@ -1129,6 +1132,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
     const int np = hole->n_exact, nr = np < kRangeProbes ? np : kRangeProbes;
+    static_assert(kRangeProbes == kProbeStep, "the first step's values are the range probes'");
     constexpr i64 kMost = 1ll << 62;
     i64 lo[kRangeProbes], hi[kRangeProbes];
 #pragma unroll
@@ -1150,23 +1154,32 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         const bool have = at + lane < count;
         OperandRef ref;
         ref.mode = 2; ref.op = 0; ref.a = ref.b = 0;
-        i32 a[kRangeProbes] = {0};
+        i32 a[kRangeProbes] = {0}, every[kMaxProbe];      // its values at the first probes, and at all of them
         // interval of constants c with a + c in range at every probe, and (swapped difference) with c - a in range
         i64 pl = -kMost, ph = kMost, ml = -kMost, mh = kMost;
         bool live = false, wide = false;
         if (have) {
             ref = operand_ref(g, hole, seg.nt, seg.esize, e);
             live = true;
-            for (int j = 0; j < np && live && !wide; ++j) {
-                i64 v;
-                live = ref_value(g, hole, ref, seg.nt, seg.esize, j, v);
-                if (!live) break;
-                wide = !narrow31(v);
-                const i64 l = hole->rng_lo[j] < -kMost ? -kMost : hole->rng_lo[j], h = hole->rng_hi[j] > kMost ? kMost : hole->rng_hi[j];
-                pl = pl > l - v ? pl : l - v; ph = ph < h - v ? ph : h - v;
-                ml = ml > l + v ? ml : l + v; mh = mh < h + v ? mh : h + v;
+            for (int j0 = 0; j0 < np && live && !wide; j0 += kProbeStep) {
+                i64 val[kProbeStep];
+                const int here = np - j0 < kProbeStep ? np - j0 : kProbeStep;
+                live = ref_value4(g, hole, ref, seg.nt, seg.esize, j0, np, val) == (1u << here) - 1u;
 #pragma unroll
-                for (int k = 0; k < kRangeProbes; ++k) if (k == j || (k >= nr && j == 0)) a[k] = (i32)v;
+                for (int q = 0; q < kProbeStep; ++q) {
+                    if (q >= here) continue;
+                    const int j = j0 + q;
+                    const i64 v = val[q];
+                    wide = wide || !narrow31(v);
+                    every[j] = (i32)v;
+                    const i64 l = hole->rng_lo[j] < -kMost ? -kMost : hole->rng_lo[j], h = hole->rng_hi[j] > kMost ? kMost : hole->rng_hi[j];
+                    pl = pl > l - v ? pl : l - v; ph = ph < h - v ? ph : h - v;
+                    ml = ml > l + v ? ml : l + v; mh = mh < h + v ? mh : h + v;
+                    if (j0 == 0) {
+#pragma unroll
+                        for (int k = 0; k < kRangeProbes; ++k) if (k == q || (k >= nr && q == 0)) a[k] = (i32)v;
+                    }
+                }
             }
         }
         if (!sets_ok) wide = live;
@@ -1218,7 +1231,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
                     if (slot <= kSlotSub) {               // by the intersection over all probes
                         const i64 from = slot == kSlotAdd ? pl : swap ? ml : -ph, to = slot == kSlotAdd ? ph : swap ? mh : -pl;
                         if (live && from <= to) { run[0] = const_lower(g->consts, cb, vb, from); run[1] = const_lower(g->consts, run[0], vb, to + 1); }
-                    } else if (live) range_runs(g->consts, cb, vb, slot, swap, a, lo, hi, run);
+                    } else if (live) range_runs(hole, np, g->consts, cb, vb, slot, swap, every, run);
                     const i32 len0 = run[1] - run[0], len = len0 + run[3] - run[2];
                     for (i32 i = 0; __any_sync(0xffffffffu, i < len); ++i) {
                         bool on = i < len;
@@ -1240,31 +1253,51 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
                             can = can && m[j] != kNever;
                         }
                         if (__any_sync(0xffffffffu, can))
-                            for (i32 ci = cb; ci < vb; ++ci) {
-                                const ConstDev c = g->consts[ci];
-                                const u32 uc = abs_u32((i32)c.value);
-                                if (uc == 0u) continue;
-                                bool on = can;
+                            for (i32 c0 = cb; c0 < vb; c0 += 32) {      // 32 constants without a branch, then those with a hit
+                                const int nc = vb - c0 < 32 ? vb - c0 : 32;
+                                u32 hits = 0;
+#pragma unroll 4
+                                for (int k = 0; k < nc; ++k) {
+                                    const ConstDev c = g->consts[c0 + k];
+                                    const u32 uc = abs_u32((i32)c.value);
+                                    u32 on = uc != 0u;
 #pragma unroll
-                                for (int j = 0; j < kRangeProbes; ++j) {
-                                    u32 r = ua[j] - __umulhi(ua[j], c.recip) * uc;
-                                    if (r >= uc) r -= uc;
-                                    on = on && r - m[j] <= sp[j];
+                                    for (int j = 0; j < kRangeProbes; ++j) {
+                                        u32 r = ua[j] - __umulhi(ua[j], c.recip) * uc;
+                                        r = r >= uc ? r - uc : r;
+                                        on &= (u32)(r - m[j] <= sp[j]);
+                                    }
+                                    hits |= on << k;
                                 }
-                                give(on, (u32)c.pos, gi, kSlotMod, 0);
+                                if (!can) hits = 0;
+                                for (u32 q = __reduce_or_sync(0xffffffffu, hits); q; q &= q - 1) {
+                                    const int k = __ffs((int)q) - 1;
+                                    give((hits >> k) & 1u, (u32)g->consts[c0 + k].pos, gi, kSlotMod, 0);
+                                }
                             }
                     } else if (__any_sync(0xffffffffu, live && !none0))
-                        for (i32 ci = cb; ci < vb; ++ci) {      // c % a: the sign of c
-                            const ConstDev c = g->consts[ci];
-                            const u32 uc = abs_u32((i32)c.value);
-                            bool on = live && !none0;
+                        for (i32 c0 = cb; c0 < vb; c0 += 32) {          // c % a: the sign of c
+                            const int nc = vb - c0 < 32 ? vb - c0 : 32;
+                            u32 hits = 0;
+#pragma unroll 4
+                            for (int k = 0; k < nc; ++k) {
+                                const ConstDev c = g->consts[c0 + k];
+                                const u32 uc = abs_u32((i32)c.value);
+                                const bool pos = c.value >= 0;
+                                u32 on = 1u;
 #pragma unroll
-                            for (int j = 0; j < kRangeProbes; ++j) {
-                                u32 r = uc - __umulhi(uc, ra[j]) * ua[j];
-                                if (r >= ua[j]) r -= ua[j];
-                                on = on && (c.value >= 0 ? r - pm[j] <= ps[j] : r - nm[j] <= ns[j]);
+                                for (int j = 0; j < kRangeProbes; ++j) {
+                                    u32 r = uc - __umulhi(uc, ra[j]) * ua[j];
+                                    r = r >= ua[j] ? r - ua[j] : r;
+                                    on &= (u32)(r - (pos ? pm[j] : nm[j]) <= (pos ? ps[j] : ns[j]));
+                                }
+                                hits |= on << k;
                             }
-                            give(on, (u32)c.pos, gi, kSlotMod, 1);
+                            if (!live || none0) hits = 0;
+                            for (u32 q = __reduce_or_sync(0xffffffffu, hits); q; q &= q - 1) {
+                                const int k = __ffs((int)q) - 1;
+                                give((hits >> k) & 1u, (u32)g->consts[c0 + k].pos, gi, kSlotMod, 1);
+                            }
                         }
                 }
                 for (i32 ci = vb; ci < ve; ++ci) {        // variables one by one
