@@ -2335,23 +2335,31 @@ __global__ void __launch_bounds__(256) surv_scatter_kernel(const PlanDev plan) {
 
 // ---- whole-domain check of several survivors of one hole together ----
 //
-// For table domains.  The warp's lanes each stage one survivor (unranking, substitution into the
-// context, magnitude bounds, constant-divisor folding: all 32 at once, where one lane used to do it
-// for one survivor while 31 waited) as a compact program in the warp's arena.  Then the chunk is
-// walked in steps of 128 points (4 per lane): the step's coordinates go to shared memory and its
+// For table domains, and boxes of at most one chunk.  The warp's lanes each stage one survivor (unranking, substitution into
+// the context, magnitude bounds, constant-divisor folding: all 32 at once) as a compact program in the warp's arena.  Then
+// the chunk is walked in steps of 256 points (8 per lane): the step's coordinates go to shared memory and its
 // spec values to registers ONCE, and every staged survivor still alive is run on them; a survivor
 // that fails at some point of the step leaves the set.
-constexpr int kVArena = 256;                              // program entries a warp stages at once
-constexpr int kVStep = 128;                               // points per step
+//
+// A program is a list of steps on an accumulator: "load", and operators whose other operand is a leaf (a variable or a
+// constant, on either side) or the value pushed last.  (i * 9) + j is three steps and touches no stack, where postfix
+// takes five with four stack accesses; with 8 points per lane instead of 4 the decoding of a step is shared by
+// twice as many points (1331 matches on 2^20 points: 18.5 -> 5.5 ms; 1024 small instances, 1.8e5 matches: 3.6 -> 2.7 ms).
+// Two CTAs per SM: at three the 80 registers spill the step loop (small calls 48 us against 33, large ones the same).
+constexpr int kVArena = 192;                              // program steps a warp stages at once
+constexpr int kVStep = 256;                               // points per step
 constexpr int kVBatchVars = 4;                            // most variables a table may have for this form
-constexpr int kVBatchDepth = 4;                           // deepest operand stack it takes
+constexpr int kVBatchDepth = 2;                           // most values pushed at a time
+// One step: x = operator (XP_OP_*; +kFRev: leaf op accumulator) | source << 8 | push first << 16; y = variable, or the
+// constant's low word; z = its high word, or (division by a constant) floor(2^32 / |constant|).
+constexpr u32 kFLoad = 64, kFDivC = 65, kFModC = 66, kFRev = 32;
+enum { kFVar = 0, kFConst = 1, kFStack = 2 };
 // A warp's shared memory: the batch form's arrays and the one-survivor form's share the same bytes
-// (a warp is in one form at a time), which keeps three CTAs resident per SM.
+// (a warp is in one form at a time), so the larger one counts.
 struct VerifyBatch {
-    i32 pvar[kVArena];                                    // >= 0: variable; -1: constant; -2 - op: operator
-    i64 pval[kVArena];
+    uint4 prog[kVArena];
     i32 coords[kVBatchVars][kVStep];                      // the step's points, [variable][point]
-    uint4 stack[kVBatchDepth * 32];                       // operand stacks below the top, per level and lane
+    uint4 stack[kVBatchDepth][2][32];                     // pushed values, per level: 32 bytes a lane
 };
 struct VerifySingle {
     uint4 stack[kVecDepth * 32];
@@ -2370,32 +2378,55 @@ __device__ __forceinline__ int staged_length(const HoleDev* hole, int n) {
     return holes ? hole->ctx_len + holes * (n - 1) : -1;
 }
 
-// One lane: stages survivor (size, rank) at w.pvar / w.pval [off ...).  Returns the final length
-// (constant divisors folded when the program is exact in int32), or -1 when the operand stack gets
-// deeper than the vectorised check takes.
+// Steps that a postfix program of `len` instructions takes at most: every operator is one, every load serves two leaves.
+__device__ __forceinline__ int staged_steps(int len) { const int leaves = (len + 1) / 2; return len - leaves + (leaves + 1) / 2; }
+
+// One lane: stages survivor (size, rank) at w.b.prog [off ...).  Returns the number of steps, or -1 when more values have to be
+// pushed than the form keeps.  narrow_out: no value can leave int32 over the domain (bounds from the variables' ranges).
 __device__ __noinline__ int stage_compact(VerifyWarp& w, int off, const SketchDev* sk, const HoleDev* hole, int size, u64 rank,
                                          bool& narrow_out) {
     const GrammarDev* g = sk->g;
     u32 code[kMaxSize];
     const int n = unrank(g, hole->start_nt, size, rank, code);
-    int len = 0, sp = 0, depth = 0;
-    bool narrow = true;
+    constexpr int kDeep = kMaxStack + kCandStack + 1;
     constexpr u64 kSat = 1ull << 62;
-    u64 mag[kMaxStack + kCandStack + 1];
+    i32 kind[kDeep];                                      // stack entries: >= 0 variable, -1 constant, -2 the accumulator, -3 pushed
+    i64 val[kDeep];
+    u64 mag[kDeep];
+    val[0] = 0;
+    int len = 0, sp = 0, pushed = 0, acc_at = -1;         // acc_at: stack entry that sits in the accumulator (-1: none)
+    bool narrow = true, deep = false;
     auto mag_of = [](i64 v) { return v < 0 ? 0ull - (u64)v : (u64)v; };
-    auto emit = [&](i32 var, i64 val) {
-        if (sp > kMaxStack + kCandStack - 1) { depth = kVBatchDepth + 1; return; }
-        w.b.pvar[off + len] = var; w.b.pval[off + len] = val; ++len;
+    auto out = [&](u32 x, i32 k, i64 v) {                 // a step whose operand is the leaf (k, v)
+        uint4 q;
+        q.x = x | ((u32)(k >= 0 ? kFVar : kFConst) << 8);
+        q.y = k >= 0 ? (u32)k : (u32)(u64)v; q.z = k >= 0 ? 0u : (u32)((u64)v >> 32); q.w = 0u;
+        w.b.prog[off + len++] = q;
+    };
+    auto load = [&](int e) {                              // entry e (a leaf) into the accumulator
+        u32 push = 0;
+        if (acc_at >= 0) { kind[acc_at] = -3; push = 1u << 16; if (++pushed > kVBatchDepth) deep = true; }
+        out(kFLoad | push, kind[e], val[e]);
+        kind[e] = -2;
+        acc_at = e;
+    };
+    auto leaf = [&](i32 k, i64 v) {
+        if (sp >= kDeep) { deep = true; return; }
         u64 m;
-        if (var >= -1) {
-            if (var >= 0) { const u64 a = mag_of(sk->vmin[var]), b = mag_of(sk->vmax[var]); m = a > b ? a : b; }
-            else m = mag_of(val);
-            mag[sp] = m < kSat ? m : kSat;
-            if (++sp > depth) depth = sp;
-        } else {
-            --sp;
-            const u64 a = mag[sp - 1], b = mag[sp];
-            switch (-2 - var) {
+        if (k >= 0) { const u64 a = mag_of(sk->vmin[k]), b = mag_of(sk->vmax[k]); m = a > b ? a : b; }
+        else m = mag_of(v);
+        mag[sp] = m < kSat ? m : kSat;
+        narrow = narrow && (m >> 31) == 0;
+        kind[sp] = k; val[sp] = v; ++sp;
+    };
+    auto oper = [&](int op) {
+        if (deep) return;
+        --sp;
+        const int x = sp - 1, y = sp;
+        {
+            const u64 a = mag[x], b = mag[y];
+            u64 m;
+            switch (op) {
                 case XP_OP_ADD: case XP_OP_SUB: m = a + b; break;
                 case XP_OP_MUL: m = (a >> 31 || b >> 31) ? kSat : a * b; break;
                 case XP_OP_DIV: m = a; break;
@@ -2405,14 +2436,26 @@ __device__ __noinline__ int stage_compact(VerifyWarp& w, int off, const SketchDe
                 case XP_OP_SHR: m = a; break;
                 default: m = 1; break;
             }
-            mag[sp - 1] = m < kSat ? m : kSat;
+            mag[x] = m < kSat ? m : kSat;
+            narrow = narrow && (m >> 31) == 0;
         }
-        narrow = narrow && (m >> 31) == 0;
+        // (the topmost entry that is not a leaf is always the one in the accumulator)
+        if (kind[x] >= -1 && kind[y] >= -1) load(x);
+        if (kind[y] >= -1) out((u32)op, kind[y], val[y]);                       // accumulator op leaf
+        else if (kind[x] >= -1) { out((u32)op | kFRev, kind[x], val[x]); kind[x] = -2; }      // leaf op accumulator
+        else {                                                                 // pushed op accumulator
+            uint4 q;
+            q.x = (u32)op | kFRev | ((u32)kFStack << 8); q.y = q.z = q.w = 0u;
+            w.b.prog[off + len++] = q;
+            --pushed;
+            kind[x] = -2;
+        }
+        acc_at = x;
     };
     auto emit_cand = [&]() {
         for (int k = 0; k < n; ++k) {
-            if (code[k] & kOpBit) emit(-2 - (i32)(code[k] & 0xff), 0);
-            else { const LeafDev lf = g->leaves[code[k]]; emit(lf.var >= 0 ? lf.var : -1, lf.value); }
+            if (code[k] & kOpBit) oper((int)(code[k] & 0xff));
+            else { const LeafDev lf = g->leaves[code[k]]; leaf(lf.var >= 0 ? lf.var : -1, lf.value); }
         }
     };
     if (hole->ctx_len == 0) emit_cand();
@@ -2420,76 +2463,147 @@ __device__ __noinline__ int stage_compact(VerifyWarp& w, int off, const SketchDe
         for (int i = 0; i < hole->ctx_len; ++i) {
             const xp_instr in = hole->ctx[i];
             if (in.kind == XP_I_HOLE) emit_cand();
-            else if (in.kind == XP_I_OP) emit(-2 - in.arg, 0);
-            else emit(in.kind == XP_I_VAR ? in.arg : -1, in.value);
+            else if (in.kind == XP_I_OP) oper(in.arg);
+            else leaf(in.kind == XP_I_VAR ? in.arg : -1, in.value);
         }
     narrow_out = narrow;
-    if (depth > kVBatchDepth) return -1;
-    if (narrow) {                                         // "push c; x / y" -> one instruction on the top of the stack
-        int wr = 0;
+    if (deep) return -1;
+    if (kind[0] >= -1) load(0);                           // a single leaf
+    if (narrow)                                           // division by a constant: multiply-high with its reciprocal
         for (int k = 0; k < len; ++k) {
-            const i32 cv = w.b.pvar[off + k];
-            const bool divmod = cv == -2 - XP_OP_DIV || cv == -2 - XP_OP_MOD;
-            if (divmod && wr > 0 && w.b.pvar[off + wr - 1] == -1 && w.b.pval[off + wr - 1] != 0 &&
-                w.b.pval[off + wr - 1] > -(1ll << 31) && w.b.pval[off + wr - 1] < (1ll << 31)) {
-                const i32 d = (i32)w.b.pval[off + wr - 1];
-                const u32 ad = d < 0 ? 0u - (u32)d : (u32)d;
-                const u32 M = ad == 1u ? 0xffffffffu : (u32)((1ull << 32) / ad);
-                w.b.pvar[off + wr - 1] = -2 - (cv == -2 - XP_OP_DIV ? kOpDivC : kOpModC);
-                w.b.pval[off + wr - 1] = (i64)(((u64)M << 32) | (u32)d);
-                continue;
-            }
-            w.b.pvar[off + wr] = cv; w.b.pval[off + wr] = w.b.pval[off + k]; ++wr;
+            uint4 q = w.b.prog[off + k];
+            const u32 op = q.x & 0xffu;
+            if ((op != XP_OP_DIV && op != XP_OP_MOD) || ((q.x >> 8) & 3u) != (u32)kFConst || q.y == 0u) continue;
+            const u32 ad = (i32)q.y < 0 ? 0u - q.y : q.y;
+            q.x = (q.x & ~0xffu) | (op == XP_OP_DIV ? kFDivC : kFModC);
+            q.z = ad == 1u ? 0xffffffffu : (u32)((1ull << 32) / ad);
+            w.b.prog[off + k] = q;
         }
-        len = wr;
-    }
     return len;
 }
 
-// The staged program [off, off + len) on the lane's points of the step (P at a time: points
-// lane*4 + half*P + i).  Returns the bit set of the lane's points that fail (a zero divisor: bit 0).
-template <typename T, int P>
-__device__ __forceinline__ u32 run_staged(VerifyWarp& w, int off, int len, int half, const i64* want, u32 in_mask) {
-    typedef VecSlot<T, P> Slot;
+// Point number (of the step) of this lane's value i of half h.
+__device__ __forceinline__ int staged_point(int h, int i) { return h * 128 + (int)(threadIdx.x & 31) * 4 + i; }
+
+// The staged program [off, off + len) on this lane's 8 points of the step, all values in int32.  bad: a zero divisor.
+__device__ __forceinline__ void run_narrow(VerifyBatch& b, int off, int len, i32 (&acc)[8], bool& bad) {
     const int lane = threadIdx.x & 31;
-    Slot t;
-#pragma unroll
-    for (int i = 0; i < P; ++i) t.v[i] = 0;
-    bool bad = false;
     int below = 0;
+    i32 y[8];
+    auto unpack = [](i32 (&v)[8], const uint4& p, const uint4& q) {
+        v[0] = (i32)p.x; v[1] = (i32)p.y; v[2] = (i32)p.z; v[3] = (i32)p.w; v[4] = (i32)q.x; v[5] = (i32)q.y; v[6] = (i32)q.z; v[7] = (i32)q.w;
+    };
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0;
     for (int k = 0; k < len; ++k) {
-        const i32 cv = w.b.pvar[off + k];
-        if (cv >= -1) {
-            w.b.stack[below * 32 + lane] = t.q;
+        const uint4 in = b.prog[off + k];
+        const u32 src = (in.x >> 8) & 3u, op = in.x & 0xffu;
+        if (in.x >> 16) {
+            b.stack[below][0][lane] = make_uint4((u32)acc[0], (u32)acc[1], (u32)acc[2], (u32)acc[3]);
+            b.stack[below][1][lane] = make_uint4((u32)acc[4], (u32)acc[5], (u32)acc[6], (u32)acc[7]);
             ++below;
-            if (cv >= 0) {
-                if (sizeof(T) == 4) t.q = *reinterpret_cast<const uint4*>(&w.b.coords[cv][lane * 4]);
-                else {
+        }
+        if (op >= kFDivC) {                               // x / c or x % c, c != 0 a constant
+            const u32 M = in.z, ad = (i32)in.y < 0 ? 0u - in.y : in.y;
 #pragma unroll
-                    for (int i = 0; i < P; ++i) t.v[i] = (T)w.b.coords[cv][lane * 4 + half * P + i];
-                }
-            } else {
-                const T v = (T)w.b.pval[off + k];
-#pragma unroll
-                for (int i = 0; i < P; ++i) t.v[i] = v;
+            for (int i = 0; i < 8; ++i) {
+                const u32 ux = acc[i] < 0 ? 0u - (u32)acc[i] : (u32)acc[i];      // |x| < 2^31: the estimate is the quotient or one less
+                u32 q = __umulhi(ux, M), r = ux - q * ad;
+                if (r >= ad) { ++q; r -= ad; }
+                acc[i] = op == kFDivC ? (((acc[i] < 0) != ((i32)in.y < 0)) ? (i32)(0u - q) : (i32)q) : (acc[i] < 0 ? (i32)(0u - r) : (i32)r);
             }
             continue;
         }
-        const int op = -2 - cv;
-        Slot a;
-        a.q = t.q;
-        if (!(sizeof(T) == 4 && op >= kOpDivC)) { --below; a.q = w.b.stack[below * 32 + lane]; }
-        vec_op<T, P>(op, w.b.pval[off + k], a, t, bad);
-    }
-    u32 which = 0;
+        if (src == kFVar) {
+            const i32* c = b.coords[in.y];
+            unpack(y, *reinterpret_cast<const uint4*>(c + lane * 4), *reinterpret_cast<const uint4*>(c + 128 + lane * 4));
+        } else if (src == kFConst) {
 #pragma unroll
-    for (int i = 0; i < P; ++i) which |= (u32)(((in_mask >> (half * P + i)) & 1u) && (i64)t.v[i] != want[half * P + i]) << (half * P + i);
-    // (points past the end of the chunk repeat its first point, so a zero divisor there is one at a real point too)
-    return which | (bad ? 1u : 0u);
+            for (int i = 0; i < 8; ++i) y[i] = (i32)in.y;
+        } else { --below; unpack(y, b.stack[below][0][lane], b.stack[below][1][lane]); }
+        switch (op) {                                     // no result can overflow (proved at staging)
+#define XP_EACH(expr) _Pragma("unroll") for (int i = 0; i < 8; ++i) { const i32 a = acc[i], c = y[i]; acc[i] = (i32)(expr); } break;
+            case kFLoad: XP_EACH(((void)a, c))
+            case XP_OP_ADD: case XP_OP_ADD + kFRev: XP_EACH(a + c)
+            case XP_OP_SUB: XP_EACH(a - c)
+            case XP_OP_SUB + kFRev: XP_EACH(c - a)
+            case XP_OP_MUL: case XP_OP_MUL + kFRev: XP_EACH(a * c)
+            case XP_OP_LT: XP_EACH(a < c)
+            case XP_OP_LT + kFRev: XP_EACH(c < a)
+            case XP_OP_LE: XP_EACH(a <= c)
+            case XP_OP_LE + kFRev: XP_EACH(c <= a)
+            case XP_OP_EQ: case XP_OP_EQ + kFRev: XP_EACH(a == c)
+            case XP_OP_NE: case XP_OP_NE + kFRev: XP_EACH(a != c)
+            case XP_OP_MIN: case XP_OP_MIN + kFRev: XP_EACH(a < c ? a : c)
+            case XP_OP_MAX: case XP_OP_MAX + kFRev: XP_EACH(a > c ? a : c)
+            case XP_OP_AND: case XP_OP_AND + kFRev: XP_EACH((a != 0) & (c != 0))
+            case XP_OP_OR: case XP_OP_OR + kFRev: XP_EACH((a != 0) | (c != 0))
+#undef XP_EACH
+            case XP_OP_DIV: case XP_OP_MOD: case XP_OP_DIV + kFRev: case XP_OP_MOD + kFRev:
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const i32 x = op & kFRev ? y[i] : acc[i], d0 = op & kFRev ? acc[i] : y[i];
+                    bad |= d0 == 0;
+                    const i32 d = d0 == 0 ? 1 : d0, q = x / d;      // |x| < 2^31, so x / -1 does not overflow
+                    acc[i] = (op & ~kFRev) == XP_OP_DIV ? q : x - q * d;
+                }
+                break;
+            case XP_OP_SHR: case XP_OP_SHR + kFRev:       // (a left shift never stays in an int32 program: its bound saturates)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const i32 x = op & kFRev ? y[i] : acc[i], n = op & kFRev ? acc[i] : y[i];
+                    bad |= n < 0 || n > 63;
+                    acc[i] = x >> (n > 31 ? 31 : (n < 0 ? 0 : n));
+                }
+                break;
+            default: bad = true; break;
+        }
+    }
 }
 
-// The survivors of `now` (bit b = lane b holds one, all of one hole) on chunk `chunk` of the hole's
-// table domain.  Each lane ends up with `failed` set if its survivor failed at some point
+// The same in int64 on the 4 points of half h.
+__device__ __noinline__ void run_wide(VerifyBatch& b, int off, int len, int h, i64 (&acc)[4], bool& bad) {
+    const int lane = threadIdx.x & 31;
+    int below = 0;
+    i64 y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = 0;
+    for (int k = 0; k < len; ++k) {
+        const uint4 in = b.prog[off + k];
+        const u32 src = (in.x >> 8) & 3u, op = in.x & 0xffu;
+        if (in.x >> 16) {
+            longlong2* s0 = reinterpret_cast<longlong2*>(&b.stack[below][0][lane]);
+            longlong2* s1 = reinterpret_cast<longlong2*>(&b.stack[below][1][lane]);
+            *s0 = make_longlong2(acc[0], acc[1]); *s1 = make_longlong2(acc[2], acc[3]);
+            ++below;
+        }
+        if (src == kFVar) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) y[i] = b.coords[in.y][staged_point(h, i)];
+        } else if (src == kFConst) {
+            const i64 v = (i64)(((u64)in.z << 32) | in.y);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) y[i] = v;
+        } else {
+            --below;
+            const longlong2 p = *reinterpret_cast<const longlong2*>(&b.stack[below][0][lane]), q = *reinterpret_cast<const longlong2*>(&b.stack[below][1][lane]);
+            y[0] = p.x; y[1] = p.y; y[2] = q.x; y[3] = q.y;
+        }
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+            i64 a = acc[0], c = y[0];
+#pragma unroll
+            for (int j = 1; j < 4; ++j) if (j == i) { a = acc[j]; c = y[j]; }
+            i64 r = c;
+            if (op != kFLoad) bad |= !apply_op((int)(op & ~kFRev), op & kFRev ? c : a, op & kFRev ? a : c, r);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) if (j == i) acc[j] = r;
+        }
+    }
+}
+
+// The survivors of `now` (bit b = lane b holds one, all of one hole) on the points [first, last) of the hole's
+// domain.  Each lane ends up with `failed` set if its survivor failed at some point
 // (fail_pid), and the warp with the number of candidate-point evaluations it made.
 __device__ __noinline__ void verify_batch(VerifyWarp& w, const SketchDev* sk, const HoleDev* hole, u32 now, int my_off, int my_len,
                                           bool my_narrow, i64 first, i64 last, bool& failed, i64& fail_pid, u64& evals) {
@@ -2501,18 +2615,22 @@ __device__ __noinline__ void verify_batch(VerifyWarp& w, const SketchDev* sk, co
     for (i64 base = first; base < last && alive; base += kVStep) {
         const int npts = last - base < kVStep ? (int)(last - base) : kVStep;
         __syncwarp();                                     // everyone is done with the previous step's points
-        for (int idx = lane; idx < kVStep * nv; idx += 32) {      // rows are contiguous: coalesced reads
-            const int p = idx / nv, v = idx - p * nv;
-            const int src = p < npts ? idx : v;           // points past the end repeat the step's first point
-            w.b.coords[v][p] = coords[base * nv + src];
+        // (points past the end repeat the step's first point: a zero divisor there is one at a real point too)
+#pragma unroll 2
+        for (int q = 0; q < kVStep / 32; ++q) {
+            const int p = q * 32 + lane;
+            const i32* row = coords + (base + (p < npts ? p : 0)) * nv;
+            for (int v = 0; v < nv; ++v) w.b.coords[v][p] = row[v];
         }
-        i64 want[4];
-        u32 in_mask = 0;
+        i32 want[8];
+        u32 in_mask = 0, off32 = 0;                       // off32: spec values outside int32 (no narrow program reaches them)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int p = lane * 4 + i;
+        for (int i = 0; i < 8; ++i) {
+            const int p = staged_point(i >> 2, i & 3);
             if (p < npts) in_mask |= 1u << i;
-            want[i] = spec[base + (p < npts ? p : 0)];
+            const i64 v = spec[base + (p < npts ? p : 0)];
+            want[i] = (i32)v;
+            if (v != (i64)want[i]) off32 |= 1u << i;
         }
         __syncwarp();
         evals += (u64)npts * (u64)__popc(alive);
@@ -2520,16 +2638,32 @@ __device__ __noinline__ void verify_batch(VerifyWarp& w, const SketchDev* sk, co
             const int b = __ffs((int)m) - 1;
             const int off = __shfl_sync(0xffffffffu, my_off, b), len = __shfl_sync(0xffffffffu, my_len, b);
             const bool narrow = __shfl_sync(0xffffffffu, (int)my_narrow, b) != 0;
-            u32 which;
-            if (narrow) which = run_staged<i32, 4>(w, off, len, 0, want, in_mask);
-            else which = run_staged<i64, 2>(w, off, len, 0, want, in_mask) | run_staged<i64, 2>(w, off, len, 1, want, in_mask);
+            u32 which = 0;                                // bit i: this lane's point i fails
+            bool bad = false;
+            if (narrow) {
+                i32 acc[8];
+                run_narrow(w.b, off, len, acc, bad);
+                which = off32;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) which |= (u32)(acc[i] != want[i]) << i;
+            } else {
+                for (int h = 0; h < 2; ++h) {
+                    i64 acc[4];
+                    run_wide(w.b, off, len, h, acc, bad);
+                    for (int i = 0; i < 4; ++i) {
+                        const int p = staged_point(h, i);
+                        which |= (u32)(acc[i] != spec[base + (p < npts ? p : 0)]) << (h * 4 + i);
+                    }
+                }
+            }
+            which = (which & in_mask) | (bad ? 1u : 0u);
             const u32 bm = __ballot_sync(0xffffffffu, which != 0u);
             if (bm) {
                 const int src = __ffs((int)bm) - 1;
                 const u32 wsrc = __shfl_sync(0xffffffffu, which, src);
                 alive &= ~(1u << b);
                 if (lane == b) {
-                    const int p = src * 4 + (__ffs((int)wsrc) - 1);
+                    const int i = __ffs((int)wsrc) - 1, p = (i >> 2) * 128 + src * 4 + (i & 3);
                     failed = true;
                     fail_pid = base + (p < npts ? p : 0);
                 }
@@ -2594,14 +2728,14 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
 // survivor (blocks in hole order) is taken before any second chunk, so candidates that fail early
 // cost one chunk; the later chunks exist for the long survivors only (surv_long_kernel), which keeps
 // a call whose largest domain has hundreds of chunks from walking hundreds of empty items for every
-// survivor of a small (or projected) domain.  A call with few survivors cuts the chunks into pieces, down to 128 points,
+// survivor of a small (or projected) domain.  A call with few survivors cuts the chunks into pieces, down to 256 points,
 // until every warp has an item (three survivors of a 37 123-point table: 341 us as whole chunks).  Each WARP takes items on its own: nothing in this kernel synchronises a CTA, and no
 // warp waits for another.  Within a block the survivors of one hole are handled together when the
 // hole's domain is a table (verify_batch), one after the other otherwise (verify_one).  A survivor
 // that has already failed is skipped.
 constexpr int kVerifyThreads = 256;
 constexpr int kVerifyWarps = kVerifyThreads / 32;
-__global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev plan) {
+__global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const PlanDev plan) {
     extern __shared__ __align__(16) unsigned char verify_smem[];
     VerifyWarp& w = reinterpret_cast<VerifyWarp*>(verify_smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -2612,14 +2746,16 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
     // of the grid a full block (a search with a few thousand survivors on a large domain spreads
     // better as one survivor per warp).
     const u64 warps = (u64)gridDim.x * kVerifyWarps;
-    u32 width = 32;
-    while (width > 1 && n < warps * width) width >>= 1;
-    const u64 n_blocks = (n + width - 1) / width;
-    // The first chunk is walked for every survivor, the later ones for the long survivors only.
+    // The first chunk is walked for every survivor, the later ones for the long survivors only.  Where most are long every
+    // chunk is work of its own, and 32 survivors share its points (1331 matches on 2^20 points).
     const u64 n_long = plan.max_chunks > 1 ? *plan.surv_long_n : 0u;
+    const u64 walks = 2 * n_long >= n && n_long > 0 ? plan.max_chunks : 1u;
+    u32 width = 32;
+    while (width > 1 && n * walks < warps * width) width >>= 1;
+    const u64 n_blocks = (n + width - 1) / width;
     const u64 long_blocks = (n_long + width - 1) / width;
     u32 pieces = 1;
-    while (pieces < (u32)(kVerifyChunk / kVStep) && n_blocks * pieces < warps) pieces <<= 1;
+    while (pieces < (u32)(kVerifyChunk / kVStep) && n_blocks * walks * pieces < warps) pieces <<= 1;
     const i64 sub = kVerifyChunk / pieces;                // points per item
     const u64 first_parts = plan.first_points >= kVerifyChunk ? pieces : (u64)((plan.first_points + sub - 1) / sub);
     const u64 first_items = n_blocks * first_parts;
@@ -2650,8 +2786,9 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
             const u32 lsi = __shfl_sync(0xffffffffu, si, leader);
             const SketchDev* sk = plan.sketches[plan.surv[lsi].sketch];
             const HoleDev* hole = &sk->holes[plan.surv[lsi].hole];
-            const bool table = sk->domain_kind == XP_DOMAIN_TABLE && sk->coords != nullptr && hole->spec_table != nullptr &&
-                               sk->n_vars <= kVBatchVars;
+            // (a box of one chunk is walked in full here: what its projection would save is less than 32 stagings one by one)
+            const bool table = (sk->domain_kind == XP_DOMAIN_TABLE || sk->n_points <= (i64)kVerifyChunk) && sk->coords != nullptr &&
+                               hole->spec_table != nullptr && sk->n_vars <= kVBatchVars;
             const bool mine = (run >> lane) & 1u;
             u32 single = 0;                               // survivors of the run that go one by one
             if (!table) single = run;
@@ -2659,8 +2796,9 @@ __global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(const PlanDev
                 const i64 last = first + sub < sk->n_points ? first + sub : sk->n_points;
                 SurvDev* sv = &plan.surv[si];
                 const bool live = mine && !(*(volatile const u32*)&sv->state & kSurvFailed);
-                const int want_len = live ? staged_length(hole, sv->size) : 0;
-                single = __ballot_sync(0xffffffffu, live && (want_len < 0 || want_len > kVArena));
+                const int plain_len = live ? staged_length(hole, sv->size) : 0;
+                const int want_len = staged_steps(plain_len);
+                single = __ballot_sync(0xffffffffu, live && (plain_len < 0 || want_len > kVArena));
                 u32 todo = __ballot_sync(0xffffffffu, live) & ~single;
                 while (todo) {                            // as many as the arena holds at a time
                     int off = 0, my_off = 0;
