@@ -1,0 +1,155 @@
+"""The search's kernels at the sizes where each can go wrong, against the CPU oracle, bit for bit (whole numbers
+throughout: the tolerance is zero)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import oracle
+from tests.util import assert_same, check_sketch
+from xp_instances import Hole, JointHole, Sketch, Variable, constant_set, free_grammar, parse_expr
+from tests.test_behaviours_gpu import _check as check_behaviours
+from tests.test_joint_gpu import _check as check_joint
+
+IJ = [Variable("i", 0, 9), Variable("j", -3, 6)]
+W = 1 << 33
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("consts,ops,ctx,spec", [
+    (constant_set(-30, 30), "+-*/%", "", "(i*7)+j"),                   # more constants than a lane's registers hold
+    (constant_set(-30, 30), "+-*/%", "", "(i/3)*-5"),
+    (constant_set(-30, 30), "+-*/%", "", "(i+j)%11"),
+    ([2], "+-*/%", "", "(i*2)-j"),                                     # one constant
+    ([], "+-*/%", "", "(i*j)+j"),                                      # none
+    ([0, 1, -1], "+-*/%", "", "0"),                                    # zero target: every product with a zero operand
+    ([W, -W, 3, 2**31 - 1, -2**31], "+-*/%", "", f"(i*{W})+j"),        # operands and targets outside int32
+    ([W, 5, 2**62, -2**63], "+-*/%", "", f"(j*{W})/5"),
+    ([1, 2, 7], ["+", "min", "max", "<<", ">>"], "", "min(i<<2,7)"),
+    ([1, 2, 70], ["-", "<<", ">>"], "", "(i<<1)>>2"),                  # shifts that are undefined
+    (constant_set(-9, 9), "+-*/%", "(HOLE*3)+(i*16)", "((i+j)*3)+(i*16)"),
+    (constant_set(-9, 9), "+-*/%", "HOLE/4", "(i*9)/4"),               # a context that loses values
+    (constant_set(-9, 9), "+-*/%", "HOLE*HOLE", "(i-j)*(i-j)"),
+    (constant_set(-9, 9), "+-*/%", "(HOLE%5)+(j/(i-4))", "((i*j)%5)+(j/(i-4))"),
+    (constant_set(-40, 40), "+-*/%", "HOLE<=i", "(j*2)<=i"),           # comparisons: runs of constants
+    (constant_set(-40, 40), "+-*/%", "(i-3)<(HOLE*-2)", "(i-3)<(j/2)"),
+    ([W, 3, -W], "+-*/%", f"HOLE<(i*{W})", f"(j*{W})<(i*{W})"),
+    (constant_set(-9, 9), "+-*/%", "", "i/0"),                         # never defined
+])
+def test_a_leaf_at_the_root(xp, consts, ops, ctx, spec):
+    g = free_grammar(IJ, consts, ops=list(ops))
+    sk = Sketch(g, [Hole(0, 5, ctx=parse_expr(ctx, IJ) if ctx else [], spec_expr=parse_expr(spec, IJ))], name=f"{ctx} = {spec}")
+    n = check_sketch(xp, sk)[0].cand_count
+    b, e = n[3] // 3 + 1, n[5] - n[5] // 3 - 1                          # windows whose ends lie inside blocks
+    check_sketch(xp, sk, windows={1: (0, 1), 3: (1, b), 5: (n[5] // 7 + 1, e)})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("top", [12, 11])                               # 1125^2 pairs of size 3: an index; 980^2: a test per pair
+@pytest.mark.parametrize("spec", ["(i*3)+(j*2)", "(i+2)*(j-1)", "(i*5)/(j+4)", "(i+j)%(j+5)", "j-j", "(i*1048576)*(j*65536)"])
+def test_two_operands_of_three_nodes(xp, top, spec):
+    g = free_grammar(IJ, list(range(0, top)) + [65536])
+    sk = Sketch(g, [Hole(0, 7, spec_expr=parse_expr(spec, IJ))], name=spec)
+    g7 = oracle.counts(g, 0, 7)[7]
+    check_sketch(xp, sk, windows={7: (0, 1_500_000)})                   # the first blocks: a leaf left, then pairs
+    check_sketch(xp, sk, windows={7: (g7 // 2 - 700_000, g7 // 2 + 700_001)})
+    check_sketch(xp, sk, windows={5: (3, 40_000), 7: (g7 - 1_500_000, g7 - 1)})
+
+
+DEEP = "((i+1)*2)-(((j+1)*3)-(((i-j)+1)-(((i*j)+2)-HOLE)))"
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("points", [1, 31, 255, 256, 257, 4096, 4097, 9000])
+@pytest.mark.parametrize("ctx", ["", "((i*2)+(j*3))*((HOLE+1)+(i*j))", DEEP, f"(HOLE*{W})+i", "(17-HOLE)/-3", "((HOLE%7)+(i/(j+1)))-(5%(i+1))",
+                                 "max(HOLE,i)<(min(j,3)+4)"])
+def test_whole_domain_check_of_many_matches(xp, points, ctx):
+    """Programs with pushed values, too deep ones, values outside int32, constant and variable divisors; tables that end
+    inside a step, a piece and a chunk; and boxes of at most one chunk."""
+    g = free_grammar(IJ, [0, 1, 2])
+    context = parse_expr(ctx, IJ) if ctx else []
+    S = parse_expr(ctx.replace("HOLE", "(i+j)") if ctx else "i+j", IJ)
+    rng = np.random.default_rng(points)
+    coords = np.stack([rng.integers(0, 200, size=points), rng.integers(0, 30, size=points)], axis=1).astype(np.int32)
+    check_sketch(xp, Sketch(g, [Hole(0, 5, ctx=context, spec_expr=S)], coords, name=f"table {points}: {ctx}"))
+    vs = [Variable("i", 0, points if points < 300 else 64), Variable("j", 0, 1 if points < 300 else points // 64)]
+    check_sketch(xp, Sketch(free_grammar(vs, [0, 1, 2]), [Hole(0, 5, ctx=context, spec_expr=S)], name=f"box {points}: {ctx}"))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ctx,spec", [
+    ("((c*3136)+(HOLE*56))+w", "((c*3136)+((r+1)*56))+w"),              # the shared terms cancel
+    ("((c*3136)+(HOLE*56))+w", "((c*3136)+(r*56))+(w*2)"),              # one does not
+    ("(HOLE*(w+1))+(c/2)", "((r*2)*(w+1))+(c/2)"),                      # a variable in the factor; a common quotient
+    ("(HOLE*4)+(w/(c-3))", "(r*4)+(w/(c-3))"),                          # undefined where c is 3
+    ("((HOLE+c)*(HOLE+1))-(c*HOLE)", "((r+c)*(r+1))-(c*r)"),            # not affine
+    ("(HOLE*4611686018427387904)+(c*r)", "(r*4611686018427387904)+(r*c)"),
+])
+def test_variables_that_cancel_on_a_large_box(xp, ctx, spec):
+    vs = [Variable("c", 0, 11), Variable("r", 0, 56), Variable("w", 0, 57)]
+    g = free_grammar(vs, [0, 1, 2], ops=["+", "*", "/"])
+    check_sketch(xp, Sketch(g, [Hole(0, 3, ctx=parse_expr(ctx, vs), spec_expr=parse_expr(spec, vs))], name=ctx))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ctx,spec,K", [
+    ("(HOLE0*16)+HOLE1", "((i+2)*16)+(j*3)", (3, 5)),
+    ("(HOLE0*3)-(HOLE1*i)", "((i/2)*3)-(j*i)", (3, 3)),                 # the factor of a part is zero at some points
+    ("(HOLE0*(12/(i-3)))+HOLE1", "j", (3, 3)),                          # the context is undefined at some points
+    (f"(HOLE0*{W})+HOLE1", f"((i*j)*{W})+i", (3, 3)),
+    ("(HOLE0*0)+(HOLE1*0)", "0", (5, 3)),                               # more pairs pass than the list holds
+])
+def test_joint_search_from_one_side(xp, ctx, spec, K):
+    g = free_grammar(IJ, [1, 2, 3, 16])
+    sk = Sketch(g, [Hole(0, 1, spec_expr=parse_expr("i", IJ))], name=ctx)
+    check_joint(xp, sk, JointHole((0, 0), K, parse_expr(ctx, IJ), spec_expr=parse_expr(spec, IJ)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_sig", [1, 2, 9, 16])
+def test_behaviour_tables_grow(xp, n_sig):
+    """Two hundred thousand behaviours (nine and more signature points): the tables are enlarged between passes."""
+    g = free_grammar(IJ, [1, 2, 3, 5, 7, 11, 13, 17, 19, 23, 29, 31])
+    sk = Sketch(g, [Hole(0, 7, spec_expr=parse_expr("((i*5)+j)%7", IJ))], name="grow")
+    check_behaviours(xp, sk, [(k * 7) % 81 for k in range(n_sig)])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [3, 130])
+def test_batch_load_in_pieces(xp, n):
+    """Tables of some 10^4 points each: the staged copy spans several pieces; from 128 sketches on threads fill them.  Two
+    grammars are shared, so one load sends a grammar's tables for all sketches of it."""
+    vs = [Variable("i", 0, 256), Variable("j", 0, 64)]
+    models = [free_grammar(vs, [1, 2, 3]), free_grammar(vs, [2, 5])]
+    rng = np.random.default_rng(n)
+    sks = []
+    for k in range(n):
+        points = int(rng.integers(1, 16000)) if k else 32768            # (the first: exactly the largest that is staged)
+        coords = np.stack([rng.integers(0, 256, size=points), rng.integers(0, 64, size=points)], axis=1).astype(np.int32)
+        a, b = coords[:, 0].astype(np.int64), coords[:, 1].astype(np.int64)
+        sks.append(Sketch(models[k % 2], [Hole(0, 3, spec_table=[a + b, a * 2, a // 5, b - a][k % 4])], coords))
+    grs = [xp.xp_grammar_create(m) for m in models]
+    got = xp.xp_repair_batch(xp.xp_sketch_load_batch([grs[k % 2] for k in range(n)], sks))
+    for k in range(n):
+        assert_same(got[k][0], oracle.repair_hole(sks[k]), f"sketch {k}")
+
+
+@pytest.mark.parametrize("bad", ["kind", "pair", "value", "attr"])
+def test_descriptors_from_models(bad):
+    """Integers of any kind, arrays of other types and strides, and what is refused."""
+    from paper_2505_02146_b200 import binding as B
+    B.load()
+    g = free_grammar([Variable("i", np.int64(0), np.int32(9))], [np.int64(-5), 1])
+    made = B.marshal_grammar(g)
+    d = made.desc
+    assert (d.n_vars, d.vars[0].name, d.vars[0].hi, d.n_productions) == (1, b"i", 9, 8)
+    assert [d.productions[k].value for k in range(3) if d.productions[k].kind == 1] == [-5, 1]
+    wide = np.arange(40, dtype=np.int64).reshape(10, 4)[::2, :1]
+    spec = np.arange(10, dtype=np.int16)[::2]
+    descs, nhs, keep = B.marshal_sketches([Sketch(g, [Hole(0, 3, ctx=parse_expr("HOLE+i", g.variables), spec_table=spec)], wide)])
+    assert nhs == [1] and descs[0].n_points == 5 and descs[0].holes[0].ctx_len == 3
+    assert list((C.c_int32 * 5).from_address(descs[0].coords)) == [0, 8, 16, 24, 32]
+    assert list((C.c_int64 * 5).from_address(descs[0].holes[0].spec_table)) == [0, 2, 4, 6, 8]
+    hole = Hole(0, 3, spec_expr={"kind": [("x", 0, 0)], "pair": [(0, 0)], "value": [(0, 0, 2**70)], "attr": [7]}[bad])
+    with pytest.raises((TypeError, ValueError, OverflowError)):
+        B.marshal_sketches([Sketch(g, [hole])])
