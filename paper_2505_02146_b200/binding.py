@@ -9,7 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
-from dataclasses import dataclass
+from dataclasses import dataclass, fields
 from typing import Dict, List, Optional, Sequence, Tuple
 
 import numpy as np
@@ -142,7 +142,8 @@ class xp_joint_view(C.Structure):
 
 
 _lib = None
-_m = None          # the CPython extension that fills the C descriptors (csrc/xp_marshal.c)
+_m = None          # the CPython extension that fills the C descriptors and makes the objects (csrc/xp_marshal.c)
+_at = {}           # addresses of the library's functions that the extension calls itself
 
 
 def load(path: Optional[str] = None):
@@ -191,6 +192,8 @@ def load(path: Optional[str] = None):
     _build.build_marshal()
     from . import _marshal
     _m = _marshal
+    for name in ("xp_grammar_create", "xp_grammar_destroy", "xp_sketch_destroy", "xp_result_get", "xp_result_free"):
+        _at[name] = C.cast(getattr(lib, name), vp).value
     _lib = lib
     return lib
 
@@ -214,12 +217,8 @@ class Grammar:
     """Owns an ``xp_grammar*``."""
 
     def __init__(self, handle: int, model):
-        self.handle, self.model = handle, model
-
-    def __del__(self):
-        if getattr(self, "handle", None) and _lib is not None:
-            _lib.xp_grammar_destroy(self.handle)
-            self.handle = None
+        load()
+        self._own, self.handle, self.model = _m.handle(_at["xp_grammar_destroy"], handle), handle, model
 
 
 class GrammarDesc:
@@ -241,10 +240,14 @@ def xp_grammar_create(g) -> Grammar:
     """``g``: an ``xp_instances.Grammar`` (variables with ranges, productions in canonical order), or the
     descriptor ``marshal_grammar`` made of one."""
     lib = load()
-    d = g if isinstance(g, GrammarDesc) else marshal_grammar(g)
-    out = C.c_void_p()
-    _check(lib.xp_grammar_create(C.byref(d.desc), C.byref(out)))
-    return Grammar(out.value, d.model)
+    if isinstance(g, GrammarDesc):
+        out = C.c_void_p()
+        _check(lib.xp_grammar_create(C.byref(g.desc), C.byref(out)))
+        return Grammar(out.value, g.model)
+    made = _m.grammar_create(_at["xp_grammar_create"], _at["xp_grammar_destroy"], Grammar, g)
+    if made.__class__ is int:
+        _check(made)
+    return made
 
 
 def xp_grammar_count(gr: Grammar, nt: int, max_size: int) -> List[int]:
@@ -264,12 +267,9 @@ class LoadedSketch:
     """Owns an ``xp_sketch*`` and keeps the grammar and any device tensors it refers to alive."""
 
     def __init__(self, handle: int, grammar: Grammar, n_holes: int, keep):
-        self.handle, self.grammar, self.n_holes, self._keep = handle, grammar, n_holes, keep
-
-    def __del__(self):
-        if getattr(self, "handle", None) and _lib is not None:
-            _lib.xp_sketch_destroy(self.handle)
-            self.handle = None
+        load()
+        self._own, self.handle = _m.handle(_at["xp_sketch_destroy"], handle), handle
+        self.grammar, self.n_holes, self._keep = grammar, n_holes, keep
 
 
 def _ptr_of(x) -> Tuple[int, int, object]:
@@ -314,8 +314,7 @@ def xp_sketch_load_batch(grs: Sequence[Grammar], sks: Sequence, marshalled=None)
     handles = (C.c_void_p * n)(*[g.handle for g in grs])
     outs = (C.c_void_p * n)()
     _check(lib.xp_sketch_load_batch(handles, descs, n, outs))
-    tensors = keep[1]
-    return [LoadedSketch(h, g, nh, t) for h, g, nh, t in zip(outs, grs, nhs, tensors)]
+    return _m.loaded(_at["xp_sketch_destroy"], C.addressof(outs), LoadedSketch, grs, nhs, keep[1])
 
 
 @dataclass
@@ -340,10 +339,19 @@ class HoleResult:
     d2h_bytes: int = 0
 
 
+_HOLE_FIELDS = tuple(f.name for f in fields(HoleResult))
+
+
+def _hole_results(result_handle: int, first: int, n: int) -> List[HoleResult]:
+    out = _m.hole_results(_at["xp_result_get"], HoleResult, _HOLE_FIELDS, result_handle or 0, first, n)
+    if out.__class__ is int:
+        _check(out)
+    return out
+
+
 def xp_result_get(result_handle: int, hole: int) -> HoleResult:
-    v = xp_result_view()
-    _check(load().xp_result_get(result_handle, hole, C.byref(v)))
-    return HoleResult(*_m.hole_result(C.addressof(v)))
+    load()
+    return _hole_results(result_handle, hole, 1)[0]
 
 
 def _opts_of(kw):
@@ -389,7 +397,7 @@ def xp_repair(sketch: LoadedSketch, **kw) -> List[HoleResult]:
     out = C.c_void_p()
     _check(load().xp_repair(sketch.handle, o, C.byref(out)))
     try:
-        return [xp_result_get(out.value, h) for h in range(sketch.n_holes)]
+        return _hole_results(out.value, 0, sketch.n_holes)
     finally:
         load().xp_result_free(out.value)
 
@@ -412,10 +420,9 @@ def xp_repair_batch(sketches: Sequence[LoadedSketch], packed: bool = False, **kw
             got = C.c_size_t()
             _check(lib.xp_result_pack(outs, n, out, total, C.byref(got)))
             return out, xp_result_get(outs[0], 0)
-        return [[xp_result_get(outs[i], h) for h in range(sketches[i].n_holes)] for i in range(n)]
+        return [_hole_results(h, 0, s.n_holes) for h, s in zip(outs, sketches)]
     finally:
-        for i in range(n):
-            lib.xp_result_free(outs[i])
+        _m.free_all(_at["xp_result_free"], C.addressof(outs), n)
 
 
 def xp_sketch_info_get(sketch: LoadedSketch) -> xp_sketch_info:

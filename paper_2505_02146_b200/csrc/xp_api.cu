@@ -208,7 +208,6 @@ struct xp_grammar {
     int n_vars = 0, n_nt = 0;
     std::vector<std::string> names;
     std::vector<i64> lo, hi;
-    std::vector<xp_production> prods;
     std::vector<LeafDev> leaves;
     std::vector<BinDev> bins;
     std::vector<ConstDev> consts;    // per nonterminal: its constants ascending, then its variables (see GrammarDev::consts)
@@ -232,13 +231,21 @@ static void build_counts(xp_grammar* g) {
         for (int nt = 0; nt < g->n_nt && !overflow; ++nt) {
             unsigned __int128 total = 0;
             if (s == 1) total = (unsigned)(g->leaf_begin[nt + 1] - g->leaf_begin[nt]);
+            unsigned __int128 block = 0;                  // trees of the previous production's operands (most productions share them)
             for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1] && !overflow; ++b) {
                 BinDev& bd = g->bins[b];
                 bd.off[s] = (u64)total;
-                for (int a = 1; a <= s - 2 && !overflow; ++a) {
-                    total += (unsigned __int128)g->cnt[bd.lnt][a] * g->cnt[bd.rnt][s - 1 - a];
-                    overflow = (total >> 63) != 0;
+                if (b == g->bin_begin[nt] || bd.lnt != (&bd)[-1].lnt || bd.rnt != (&bd)[-1].rnt) {
+                    block = 0;
+                    const u64 *l = g->cnt[bd.lnt], *r = g->cnt[bd.rnt];
+                    for (int a = 1; a <= s - 2 && !overflow; ++a) {
+                        if (l[a] == 0 || r[s - 1 - a] == 0) continue;
+                        block += (unsigned __int128)l[a] * r[s - 1 - a];
+                        overflow = (block >> 63) != 0;
+                    }
                 }
+                total += block;
+                overflow = overflow || (total >> 63) != 0;
             }
             g->cnt[nt][s] = (u64)total;
         }
@@ -271,6 +278,7 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
         g->lo.push_back(d->vars[i].lo);
         g->hi.push_back(d->vars[i].hi);
     }
+    size_t n_leaves = 0, n_bins = 0;
     for (int i = 0; i < d->n_productions; ++i) {
         const xp_production& p = d->productions[i];
         bool ok = p.lhs >= 0 && p.lhs < g->n_nt;
@@ -278,12 +286,16 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
         else if (p.kind == XP_PROD_BIN) ok = ok && ((p.op >= XP_OP_ADD && p.op <= XP_OP_MOD) || p.op == XP_OP_MIN || p.op == XP_OP_MAX || p.op == XP_OP_SHL || p.op == XP_OP_SHR) && p.left >= 0 && p.left < g->n_nt && p.right >= 0 && p.right < g->n_nt;
         else if (p.kind != XP_PROD_CONST) ok = false;
         if (!ok) { delete g; return fail(XP_ERR_GRAMMAR, "production " + std::to_string(i) + " is malformed"); }
-        g->prods.push_back(p);
+        ++(p.kind == XP_PROD_BIN ? n_bins : n_leaves);
     }
+    g->leaves.reserve(n_leaves);
+    g->consts.reserve(n_leaves);
+    g->bins.reserve(n_bins);
     for (int nt = 0; nt < g->n_nt; ++nt) {          // leaves and binaries grouped per nonterminal, order kept
         g->leaf_begin[nt] = (int)g->leaves.size();
         g->bin_begin[nt] = (int)g->bins.size();
-        for (const xp_production& p : g->prods) {
+        for (int i = 0; i < d->n_productions; ++i) {
+            const xp_production& p = d->productions[i];
             if (p.lhs != nt) continue;
             if (p.kind == XP_PROD_BIN) {
                 BinDev b;
@@ -305,8 +317,9 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
         const int lb = g->leaf_begin[nt], le = g->leaf_begin[nt + 1];
         g->const_begin[nt] = (int)g->consts.size();
         for (int i = lb; i < le; ++i) if (g->leaves[i].var < 0) g->consts.push_back(ConstDev{g->leaves[i].value, i - lb, reciprocal(g->leaves[i].value)});
-        std::sort(g->consts.begin() + g->const_begin[nt], g->consts.end(), [](const ConstDev& a, const ConstDev& b) {
-            return a.value != b.value ? a.value < b.value : a.pos < b.pos; });
+        auto before = [](const ConstDev& a, const ConstDev& b) { return a.value != b.value ? a.value < b.value : a.pos < b.pos; };
+        const auto first = g->consts.begin() + g->const_begin[nt];
+        if (!std::is_sorted(first, g->consts.end(), before)) std::sort(first, g->consts.end(), before);
         g->var_begin[nt] = (int)g->consts.size();
         for (int i = lb; i < le; ++i) if (g->leaves[i].var >= 0) g->consts.push_back(ConstDev{g->leaves[i].var, i - lb, 0u});
     }

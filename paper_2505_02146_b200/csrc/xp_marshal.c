@@ -1,12 +1,16 @@
 /* CPython extension of the binding: walks grammar and sketch models and fills the C descriptors of include/xp.h.
  *
  * A batch load marshals thousands of productions and holes; done field by field through ctypes that took longer than the
- * GPU's part of the load (1024 small sketches: 40 ms).  Nothing here evaluates, counts or ranks candidates.
+ * GPU's part of the load (1024 small sketches: 40 ms); so do Python-level constructors, finalisers and ctypes calls per
+ * object (1024 grammars, loads and results: 21.7 -> 18.8 ms).  Nothing here evaluates, counts or ranks candidates.
  *
  *   grammar(g)                         -> (address of an xp_grammar_desc, owner)
  *   sketches(list, conv, coords, specs) -> (address of the xp_sketch_desc array, owner, holes per sketch, device tensors per sketch)
  *   code(list)                         -> bytes of xp_instr
- *   hole_result(address of an xp_result_view) -> tuple of a hole result's fields
+ *   grammar_create(create, destroy, class, g), loaded(destroy, addresses, class, grammars, holes, tensors),
+ *   hole_results(get, class, fields, result, first, n)  -> instances of the binding's classes, made without running Python code;
+ *                                         the functions of the library are passed as addresses
+ *   handle(destroy, address), free_all(destroy, addresses, n)
  *
  * The owner object frees the memory behind the address; it also holds the arrays the descriptors point into.
  */
@@ -18,7 +22,8 @@
 #include "xp.h"
 
 static PyObject *s_variables, *s_name, *s_lo, *s_hi, *s_n_nonterminals, *s_productions, *s_lhs, *s_kind, *s_var, *s_op, *s_left, *s_right, *s_value,
-    *s_holes, *s_coords, *s_start_nt, *s_max_size, *s_ctx, *s_spec_expr, *s_spec_table, *s_data_ptr, *s_is_cuda, *s_shape;
+    *s_holes, *s_coords, *s_start_nt, *s_max_size, *s_ctx, *s_spec_expr, *s_spec_table, *s_data_ptr, *s_is_cuda, *s_shape,
+    *s_own, *s_handle, *s_model, *s_grammar, *s_n_holes, *s_keep;
 
 /* What a marshalled description owns: one block of memory and a list of the objects it points into. */
 typedef struct { PyObject_HEAD void* mem; PyObject* held; } Owner;
@@ -100,43 +105,52 @@ static PyObject* m_code(PyObject* self, PyObject* arg) {
     return out;
 }
 
-static PyObject* m_grammar(PyObject* self, PyObject* g) {
-    (void)self;
-    PyObject *vars = NULL, *prods = NULL, *ret = NULL, *tmp;
-    Owner* o = NULL;
-    tmp = PyObject_GetAttr(g, s_variables);
-    if (!tmp) return NULL;
-    vars = PySequence_Fast(tmp, "variables is a list");
-    Py_DECREF(tmp);
-    tmp = vars ? PyObject_GetAttr(g, s_productions) : NULL;
-    if (!tmp) goto done;
-    prods = PySequence_Fast(tmp, "productions is a list");
-    Py_DECREF(tmp);
-    if (!prods) goto done;
-    const Py_ssize_t nv = PySequence_Fast_GET_SIZE(vars), np = PySequence_Fast_GET_SIZE(prods);
-    o = new_owner(sizeof(xp_grammar_desc) + sizeof(xp_variable) * (size_t)nv + sizeof(xp_production) * (size_t)np);
-    if (!o) goto done;
-    xp_grammar_desc* d = (xp_grammar_desc*)o->mem;
+/* A grammar model's lists, and its descriptor in memory that follows them: sizes first, then the fields. */
+typedef struct { PyObject *vars, *prods; Py_ssize_t nv, np; } GrammarLists;
+
+static int grammar_lists(PyObject* g, GrammarLists* l) {
+    l->vars = l->prods = NULL;
+    for (int k = 0; k < 2; ++k) {
+        PyObject* tmp = PyObject_GetAttr(g, k ? s_productions : s_variables);
+        if (!tmp) return -1;
+        PyObject* f = PySequence_Fast(tmp, k ? "productions is a list" : "variables is a list");
+        Py_DECREF(tmp);
+        if (!f) return -1;
+        if (k) l->prods = f;
+        else l->vars = f;
+    }
+    l->nv = PySequence_Fast_GET_SIZE(l->vars);
+    l->np = PySequence_Fast_GET_SIZE(l->prods);
+    return 0;
+}
+
+static size_t grammar_bytes(const GrammarLists* l) {
+    return sizeof(xp_grammar_desc) + sizeof(xp_production) * (size_t)l->np + (sizeof(xp_variable) + sizeof(PyObject*)) * (size_t)l->nv;
+}
+
+/* Fills `mem` (zeroed).  names[i] receives the name object that vars[i].name points into. */
+static int fill_grammar(PyObject* g, const GrammarLists* l, void* mem, PyObject*** names_out) {
+    xp_grammar_desc* d = (xp_grammar_desc*)mem;
     xp_production* p = (xp_production*)(d + 1);
-    xp_variable* v = (xp_variable*)(p + np);
-    d->n_vars = (int32_t)nv;
+    xp_variable* v = (xp_variable*)(p + l->np);
+    PyObject** names = (PyObject**)(v + l->nv);
+    *names_out = names;
+    d->n_vars = (int32_t)l->nv;
     d->vars = v;
     d->n_nonterminals = (int32_t)int_attr(g, s_n_nonterminals);
-    d->n_productions = (int32_t)np;
+    d->n_productions = (int32_t)l->np;
     d->productions = p;
-    for (Py_ssize_t i = 0; i < nv; ++i) {
-        PyObject* x = PySequence_Fast_GET_ITEM(vars, i);
-        PyObject* name = PyObject_GetAttr(x, s_name);
-        PyObject* utf = name ? PyUnicode_AsUTF8String(name) : NULL;
-        Py_XDECREF(name);
-        if (!utf || PyList_Append(o->held, utf) < 0) { Py_XDECREF(utf); goto done; }
-        v[i].name = PyBytes_AS_STRING(utf);
-        Py_DECREF(utf);                                  /* (the list holds it) */
+    for (Py_ssize_t i = 0; i < l->nv; ++i) {
+        PyObject* x = PySequence_Fast_GET_ITEM(l->vars, i);
+        names[i] = PyObject_GetAttr(x, s_name);
+        if (names[i] && !PyUnicode_Check(names[i])) PyErr_SetString(PyExc_TypeError, "a variable's name is a string");
+        v[i].name = names[i] && PyUnicode_Check(names[i]) ? PyUnicode_AsUTF8(names[i]) : NULL;
+        if (!v[i].name) return -1;
         v[i].lo = int_attr(x, s_lo);
         v[i].hi = int_attr(x, s_hi);
     }
-    for (Py_ssize_t i = 0; i < np; ++i) {
-        PyObject* x = PySequence_Fast_GET_ITEM(prods, i);
+    for (Py_ssize_t i = 0; i < l->np; ++i) {
+        PyObject* x = PySequence_Fast_GET_ITEM(l->prods, i);
         const int32_t kind = (int32_t)int_attr(x, s_kind);
         p[i].kind = kind;
         p[i].lhs = (int32_t)int_attr(x, s_lhs);
@@ -146,13 +160,156 @@ static PyObject* m_grammar(PyObject* self, PyObject* g) {
         p[i].left = (int32_t)int_attr(x, s_left);
         p[i].right = (int32_t)int_attr(x, s_right);
     }
-    if (PyErr_Occurred()) goto done;
-    ret = Py_BuildValue("(KO)", (unsigned long long)(size_t)o->mem, (PyObject*)o);
-done:
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+static PyObject* m_grammar(PyObject* self, PyObject* g) {
+    (void)self;
+    PyObject *ret = NULL, **names = NULL;
+    GrammarLists l;
+    Owner* o = grammar_lists(g, &l) == 0 ? new_owner(grammar_bytes(&l)) : NULL;
+    if (o) {
+        int rc = fill_grammar(g, &l, o->mem, &names);
+        for (Py_ssize_t i = 0; i < l.nv; ++i) {
+            if (names[i] && PyList_Append(o->held, names[i]) < 0) rc = -1;
+            Py_XDECREF(names[i]);                        /* (the list holds it) */
+        }
+        if (rc == 0) ret = Py_BuildValue("(KO)", (unsigned long long)(size_t)o->mem, (PyObject*)o);
+    }
     Py_XDECREF((PyObject*)o);
-    Py_XDECREF(vars);
-    Py_XDECREF(prods);
+    Py_XDECREF(l.vars);
+    Py_XDECREF(l.prods);
     return ret;
+}
+
+/* Something the library made: destroyed with this object. */
+typedef struct { PyObject_HEAD void (*destroy)(void*); void* at; } Handle;
+
+static void handle_dealloc(Handle* h) {
+    void (*destroy)(void*) = h->destroy;
+    void* at = h->at;
+    Py_TYPE(h)->tp_free((PyObject*)h);
+    if (!at || !destroy) return;
+    Py_BEGIN_ALLOW_THREADS
+    destroy(at);
+    Py_END_ALLOW_THREADS
+}
+
+static PyTypeObject HandleType = {
+    PyVarObject_HEAD_INIT(NULL, 0).tp_name = "_marshal.Handle", .tp_basicsize = sizeof(Handle), .tp_flags = Py_TPFLAGS_DEFAULT,
+    .tp_dealloc = (destructor)handle_dealloc, .tp_doc = "Something the library made; destroyed with this object.",
+};
+
+static PyObject* new_handle(unsigned long long destroy, void* at) {
+    Handle* h = PyObject_New(Handle, &HandleType);
+    if (!h) return NULL;
+    h->destroy = (void (*)(void*))(size_t)destroy;
+    h->at = at;
+    return (PyObject*)h;
+}
+
+static PyObject* m_handle(PyObject* self, PyObject* args) {
+    (void)self;
+    unsigned long long destroy, at;
+    if (!PyArg_ParseTuple(args, "KK", &destroy, &at)) return NULL;
+    return new_handle(destroy, (void*)(size_t)at);
+}
+
+/* obj.name = value; takes the reference (NULL: an exception is set). */
+static int put(PyObject* obj, PyObject* name, PyObject* value) {
+    const int rc = value ? PyObject_SetAttr(obj, name, value) : -1;
+    Py_XDECREF(value);
+    return rc;
+}
+
+/* An instance of `cls` without a call of its __init__. */
+static PyObject* blank(PyObject* cls) {
+    PyObject* none = PyTuple_New(0);
+    PyObject* obj = none ? ((PyTypeObject*)cls)->tp_new((PyTypeObject*)cls, none, NULL) : NULL;
+    Py_XDECREF(none);
+    return obj;
+}
+
+/* A new instance of the Python class `cls` that owns the library object `at`. */
+static PyObject* owning(PyObject* cls, unsigned long long destroy, void* at) {
+    PyObject* own = new_handle(destroy, at);             /* (first: whatever fails from here on, `at` is destroyed) */
+    if (!own) return NULL;
+    PyObject* obj = blank(cls);
+    if (!obj) { Py_DECREF(own); return NULL; }
+    if (put(obj, s_own, own) < 0 || put(obj, s_handle, PyLong_FromVoidPtr(at)) < 0) Py_CLEAR(obj);
+    return obj;
+}
+
+static PyObject* m_grammar_create(PyObject* self, PyObject* args) {
+    (void)self;
+    unsigned long long create, destroy;
+    PyObject *cls, *g, *ret = NULL, **names = NULL;
+    if (!PyArg_ParseTuple(args, "KKO!O", &create, &destroy, &PyType_Type, &cls, &g)) return NULL;
+    GrammarLists l;
+    _Alignas(16) char room[4096];                        /* (most grammars fit) */
+    void* mem = NULL;
+    if (grammar_lists(g, &l) == 0) {
+        const size_t bytes = grammar_bytes(&l);
+        mem = bytes <= sizeof(room) ? memset(room, 0, bytes) : calloc(1, bytes);
+        if (!mem) PyErr_NoMemory();
+        else {
+            void* at = NULL;
+            if (fill_grammar(g, &l, mem, &names) == 0) {
+                const int st = ((int (*)(const xp_grammar_desc*, void**))(size_t)create)((const xp_grammar_desc*)mem, &at);
+                if (st != 0) ret = PyLong_FromLong(st);
+                else {
+                    ret = owning(cls, destroy, at);
+                    if (ret && put(ret, s_model, Py_NewRef(g)) < 0) Py_CLEAR(ret);
+                }
+            }
+            for (Py_ssize_t i = 0; i < l.nv; ++i) Py_XDECREF(names[i]);
+            if (mem != (void*)room) free(mem);
+        }
+    }
+    Py_XDECREF(l.vars);
+    Py_XDECREF(l.prods);
+    return ret;
+}
+
+/* Instances of `cls` for n loaded sketches. */
+static PyObject* m_loaded(PyObject* self, PyObject* args) {
+    (void)self;
+    unsigned long long destroy, address;
+    PyObject *cls, *grs, *nhs, *keeps;
+    if (!PyArg_ParseTuple(args, "KKO!OO!O!", &destroy, &address, &PyType_Type, &cls, &grs, &PyList_Type, &nhs, &PyList_Type, &keeps)) return NULL;
+    void** at = (void**)(size_t)address;
+    const Py_ssize_t n = PyList_GET_SIZE(nhs);
+    PyObject* seq = PySequence_Fast(grs, "grammars is a list");
+    PyObject* out = seq ? PyList_New(n) : NULL;
+    int rc = out ? 0 : -1;
+    if (rc == 0 && (PySequence_Fast_GET_SIZE(seq) != n || PyList_GET_SIZE(keeps) != n)) {
+        PyErr_SetString(PyExc_ValueError, "lists of one length were expected");
+        rc = -1;
+    }
+    for (Py_ssize_t i = 0; out && i < n; ++i) {
+        PyObject* obj = owning(cls, destroy, at[i]);     /* (also after a failure: every sketch gets its owner) */
+        if (!obj) { rc = -1; continue; }
+        PyList_SET_ITEM(out, i, obj);
+        if (rc < 0) continue;
+        if (put(obj, s_grammar, Py_NewRef(PySequence_Fast_GET_ITEM(seq, i))) < 0 || put(obj, s_n_holes, Py_NewRef(PyList_GET_ITEM(nhs, i))) < 0 ||
+            put(obj, s_keep, Py_NewRef(PyList_GET_ITEM(keeps, i))) < 0) rc = -1;
+    }
+    Py_XDECREF(seq);
+    if (rc < 0) Py_CLEAR(out);
+    return out;
+}
+
+/* destroy(address[0 .. n)) */
+static PyObject* m_free_all(PyObject* self, PyObject* args) {
+    (void)self;
+    unsigned long long destroy, address;
+    Py_ssize_t n;
+    if (!PyArg_ParseTuple(args, "KKn", &destroy, &address, &n)) return NULL;
+    void** at = (void**)(size_t)address;
+    Py_BEGIN_ALLOW_THREADS
+    for (Py_ssize_t i = 0; i < n; ++i) ((void (*)(void*))(size_t)destroy)(at[i]);
+    Py_END_ALLOW_THREADS
+    Py_RETURN_NONE;
 }
 
 /* Address and row count of an array with `itemsize`-byte integers; *held receives the object that has to stay alive.
@@ -332,36 +489,63 @@ done:
     return ret;
 }
 
-static PyObject* m_hole_result(PyObject* self, PyObject* arg) {
+/* The results of holes [first, first + n) of a result handle as a list of `cls` (whose fields are `names`); the status where
+ * the library refuses one. */
+static PyObject* m_hole_results(PyObject* self, PyObject* args) {
     (void)self;
-    const xp_result_view* v = (const xp_result_view*)(size_t)PyLong_AsUnsignedLongLong(arg);
-    if (!v) return NULL;
-    const Py_ssize_t K = v->max_size + 1;
-    PyObject *cand = PyList_New(K), *match = PyList_New(K), *code = PyList_New(v->least_len);
-    if (!cand || !match || !code) {
-        Py_XDECREF(cand);
-        Py_XDECREF(match);
-        Py_XDECREF(code);
-        return NULL;
+    unsigned long long get, handle;
+    PyObject *cls, *names;
+    int first, n;
+    if (!PyArg_ParseTuple(args, "KO!O!Kii", &get, &PyType_Type, &cls, &PyTuple_Type, &names, &handle, &first, &n)) return NULL;
+    PyObject* out = PyList_New(n > 0 ? n : 0);
+    for (int h = 0; out && h < n; ++h) {
+        xp_result_view v;
+        memset(&v, 0, sizeof(v));
+        const int st = ((int (*)(void*, int32_t, xp_result_view*))(size_t)get)((void*)(size_t)handle, first + h, &v);
+        if (st != 0) {
+            Py_DECREF(out);
+            return PyLong_FromLong(st);
+        }
+        const Py_ssize_t K = v.max_size + 1;
+        PyObject *cand = PyList_New(K), *match = PyList_New(K), *code = PyList_New(v.least_len);
+        for (Py_ssize_t k = 0; cand && match && k < K; ++k) {
+            PyList_SET_ITEM(cand, k, PyLong_FromUnsignedLongLong(v.cand_count[k]));
+            PyList_SET_ITEM(match, k, PyLong_FromUnsignedLongLong(v.match_count[k]));
+        }
+        for (Py_ssize_t k = 0; code && k < v.least_len; ++k)
+            PyList_SET_ITEM(code, k, Py_BuildValue("(iiL)", (int)v.least_code[k].kind, (int)v.least_code[k].arg, (long long)v.least_code[k].value));
+        PyObject* field[] = {PyBool_FromLong(v.solved), cand, match, PyLong_FromLong(v.least_size), PyLong_FromUnsignedLongLong(v.least_rank),
+                             PyUnicode_FromString(v.solved ? v.least_text : ""), code, PyLong_FromUnsignedLongLong(v.evals_executed),
+                             PyLong_FromUnsignedLongLong(v.filter_survivors), PyLong_FromUnsignedLongLong(v.probe_survivors),
+                             PyLong_FromUnsignedLongLong(v.nominal_ops), PyFloat_FromDouble(v.kernel_ms), PyFloat_FromDouble(v.total_ms),
+                             PyLong_FromLong(v.n_launches), PyLong_FromUnsignedLongLong(v.filter_tests),
+                             PyLong_FromUnsignedLongLong(v.candidates_skipped), PyLong_FromUnsignedLongLong(v.h2d_bytes),
+                             PyLong_FromUnsignedLongLong(v.d2h_bytes)};
+        const Py_ssize_t nf = (Py_ssize_t)(sizeof(field) / sizeof(field[0]));
+        PyObject* obj = PyTuple_GET_SIZE(names) == nf ? blank(cls) : NULL;
+        if (!obj && !PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "a hole result has other fields");
+        int rc = obj ? 0 : -1;
+        for (Py_ssize_t k = 0; k < nf; ++k) {
+            if (rc == 0) rc = put(obj, PyTuple_GET_ITEM(names, k), field[k]);
+            else Py_XDECREF(field[k]);
+        }
+        if (rc < 0) {
+            Py_XDECREF(obj);
+            Py_CLEAR(out);
+        } else PyList_SET_ITEM(out, h, obj);
     }
-    for (Py_ssize_t k = 0; k < K; ++k) {
-        PyList_SET_ITEM(cand, k, PyLong_FromUnsignedLongLong(v->cand_count[k]));
-        PyList_SET_ITEM(match, k, PyLong_FromUnsignedLongLong(v->match_count[k]));
-    }
-    for (Py_ssize_t k = 0; k < v->least_len; ++k)
-        PyList_SET_ITEM(code, k, Py_BuildValue("(iiL)", (int)v->least_code[k].kind, (int)v->least_code[k].arg, (long long)v->least_code[k].value));
-    return Py_BuildValue("(NNNiKsNKKKKddiKKKK)", PyBool_FromLong(v->solved), cand, match, (int)v->least_size, (unsigned long long)v->least_rank,
-                         v->solved ? v->least_text : "", code, (unsigned long long)v->evals_executed, (unsigned long long)v->filter_survivors,
-                         (unsigned long long)v->probe_survivors, (unsigned long long)v->nominal_ops, v->kernel_ms, v->total_ms, (int)v->n_launches,
-                         (unsigned long long)v->filter_tests, (unsigned long long)v->candidates_skipped, (unsigned long long)v->h2d_bytes,
-                         (unsigned long long)v->d2h_bytes);
+    return out;
 }
 
 static PyMethodDef methods[] = {
     {"grammar", m_grammar, METH_O, "Grammar model -> (descriptor address, owner)."},
     {"sketches", m_sketches, METH_VARARGS, "Sketch models -> (descriptors' address, owner, holes per sketch, device tensors per sketch)."},
     {"code", m_code, METH_O, "Postfix list -> xp_instr bytes."},
-    {"hole_result", m_hole_result, METH_O, "Address of an xp_result_view -> tuple."},
+    {"handle", m_handle, METH_VARARGS, "(address of a destroy function, address) -> owner."},
+    {"grammar_create", m_grammar_create, METH_VARARGS, "Grammar model -> instance of a class, or the status of the library's refusal."},
+    {"loaded", m_loaded, METH_VARARGS, "Addresses of loaded sketches -> instances of a class."},
+    {"free_all", m_free_all, METH_VARARGS, "Destroys an array of library objects."},
+    {"hole_results", m_hole_results, METH_VARARGS, "Results of a handle's holes -> instances of a class."},
     {NULL, NULL, 0, NULL},
 };
 
@@ -373,11 +557,12 @@ PyMODINIT_FUNC PyInit__marshal(void) {
         {&s_productions, "productions"}, {&s_lhs, "lhs"}, {&s_kind, "kind"}, {&s_var, "var"}, {&s_op, "op"}, {&s_left, "left"},
         {&s_right, "right"}, {&s_value, "value"}, {&s_holes, "holes"}, {&s_coords, "coords"}, {&s_start_nt, "start_nt"},
         {&s_max_size, "max_size"}, {&s_ctx, "ctx"}, {&s_spec_expr, "spec_expr"}, {&s_spec_table, "spec_table"},
-        {&s_data_ptr, "data_ptr"}, {&s_is_cuda, "is_cuda"}, {&s_shape, "shape"}};
+        {&s_data_ptr, "data_ptr"}, {&s_is_cuda, "is_cuda"}, {&s_shape, "shape"}, {&s_own, "_own"},
+        {&s_handle, "handle"}, {&s_model, "model"}, {&s_grammar, "grammar"}, {&s_n_holes, "n_holes"}, {&s_keep, "_keep"}};
     for (size_t i = 0; i < sizeof(names) / sizeof(names[0]); ++i) {
         *names[i].to = PyUnicode_InternFromString(names[i].name);
         if (!*names[i].to) return NULL;
     }
-    if (PyType_Ready(&OwnerType) < 0) return NULL;
+    if (PyType_Ready(&OwnerType) < 0 || PyType_Ready(&HandleType) < 0) return NULL;
     return PyModule_Create(&module);
 }
