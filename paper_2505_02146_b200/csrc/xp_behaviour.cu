@@ -176,7 +176,7 @@ __device__ __forceinline__ bool beh_same(const BehDev* B, const BehPass& P, u64 
 }
 
 template <int NS>                                         // n_sig <= NS: the signature stays in registers
-__global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, const BehPass P, u64 chunk_first, u32 chunk_n) {
+__global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n) {
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= chunk_n) return;
     const int ns = B->n_sig;
@@ -243,7 +243,7 @@ __device__ __forceinline__ u64 range_id(const BehRanges& R, u64 i) {
 }
 
 // Representatives of a nonterminal into its (cleared) table.
-__global__ void __launch_bounds__(kBehThreads) beh_rehash_kernel(BehDev* B, int nt, u64 mask, const BehRanges R) {
+__global__ void __launch_bounds__(kBehThreads) beh_rehash_kernel(BehDev* B, int nt, u64 mask, const __grid_constant__ BehRanges R) {
     const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= R.total) return;
     const u64 id = range_id(R, i);
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(1024) beh_scan_kernel(BehDev* B, int n_blocks)
     if (t == 1023) B->chunk_new = part[1023];
 }
 
-__global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, const BehPass P, u64 chunk_first, u32 chunk_n, u64 rep_base) {
+__global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n, u64 rep_base) {
     __shared__ u32 warp_sum[kBehThreads / 32];
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, cons
 }
 
 // All of them against the constraint at the signature points.
-__global__ void __launch_bounds__(kBehThreads) beh_match_kernel(BehDev* B, const BehRanges R) {
+__global__ void __launch_bounds__(kBehThreads) beh_match_kernel(BehDev* B, const __grid_constant__ BehRanges R) {
     const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= R.total) return;
     const u64 id = range_id(R, i);

@@ -2213,7 +2213,7 @@ __device__ __noinline__ void tile_ticket(EvalShared& sh, const PlanDev& plan, co
 #define XP_MIN_CTAS 3
 #endif
 template <bool DENSE>
-__global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const PlanDev plan) {
+__global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const __grid_constant__ PlanDev plan) {
     __shared__ EvalShared sh;
     u64 my_evals = 0;
     if (threadIdx.x <= kMaxSize) { sh.match_count[threadIdx.x] = 0; sh.min_rank[threadIdx.x] = ~0ull; }
@@ -2324,7 +2324,7 @@ __global__ void __launch_bounds__(1024) surv_scan_kernel(u32* hist, u32* off, in
     if (t == 1023) off[n_acc] = part[1023];
 }
 
-__global__ void __launch_bounds__(256) surv_scatter_kernel(const PlanDev plan) {
+__global__ void __launch_bounds__(256) surv_scatter_kernel(const __grid_constant__ PlanDev plan) {
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
     const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2735,7 +2735,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
 // that has already failed is skipped.
 constexpr int kVerifyThreads = 256;
 constexpr int kVerifyWarps = kVerifyThreads / 32;
-__global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const PlanDev plan) {
+__global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const __grid_constant__ PlanDev plan) {
     extern __shared__ __align__(16) unsigned char verify_smem[];
     VerifyWarp& w = reinterpret_cast<VerifyWarp*>(verify_smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -2842,7 +2842,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const PlanDev
 }
 
 // One thread per queued survivor of a sketch without points: there is no chunk to pass, it is a match.
-__global__ void count_kernel(const PlanDev plan) {
+__global__ void count_kernel(const __grid_constant__ PlanDev plan) {
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
     const u32 i = blockIdx.x * blockDim.x + threadIdx.x;

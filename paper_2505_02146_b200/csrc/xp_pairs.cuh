@@ -109,7 +109,7 @@ __device__ __forceinline__ u32 pair_limit(const HoleDev* hole) {
 }
 
 // Chains of the indexed set (narrow entries), and the lists of wide entries of both sets.
-__global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const __grid_constant__ PlanDev plan, int index) {
     const PairSeg& seg = plan.psegs[index];
     const SketchDev* sk = plan.sketches[seg.sketch];
     const HoleDev* hole = &sk->holes[seg.hole];
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const PlanDev 
 }
 
 // + - *: one thread per operand x of the set that is not indexed.
-__global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const __grid_constant__ PlanDev plan, int index) {
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -193,7 +193,7 @@ __device__ __forceinline__ u32 pair_bucket(u32 u) {
 }
 constexpr int kPairBuckets = 1024;
 
-__global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const __grid_constant__ PlanDev plan, int index) {
     __shared__ u32 hist[kPairBuckets];
     const PairSeg& seg = plan.psegs[index];
     const int side = blockIdx.y;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const Pla
 }
 
 // One CTA per side: bucket starts (start[kPairBuckets] = entries), and the cursors of the scatter.
-__global__ void __launch_bounds__(kPairBuckets) pair_sort_scan_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairBuckets) pair_sort_scan_kernel(const __grid_constant__ PlanDev plan, int index) {
     __shared__ u32 part[kPairBuckets];
     const PairSeg& seg = plan.psegs[index];
     const int side = blockIdx.x, t = threadIdx.x;
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kPairBuckets) pair_sort_scan_kernel(const Plan
     if (t == kPairBuckets - 1) seg.start[side][kPairBuckets] = part[t];
 }
 
-__global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const __grid_constant__ PlanDev plan, int index) {
     const PairSeg& seg = plan.psegs[index];
     const int side = blockIdx.y, lane = threadIdx.x & 31;
     const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
@@ -256,7 +256,7 @@ __device__ __forceinline__ u32 pair_from(const PairSeg& seg, u64 u) { return seg
 __device__ __forceinline__ u32 pair_to(const PairSeg& seg, u64 u) { return seg.start[1][u >> 31 ? kPairBuckets : pair_bucket((u32)u) + 1u]; }
 
 // A ticket: 32 dividends in magnitude order and one piece of the divisors that they may meet.
-__global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_constant__ PlanDev plan, int index) {
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const PlanDev
 }
 
 // Wide operands: each against the whole other set, lanes over it, from the first probe on, exactly.
-__global__ void __launch_bounds__(kPairThreads) pair_wide_kernel(const PlanDev plan, int index) {
+__global__ void __launch_bounds__(kPairThreads) pair_wide_kernel(const __grid_constant__ PlanDev plan, int index) {
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
