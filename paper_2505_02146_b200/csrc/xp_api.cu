@@ -895,6 +895,14 @@ static void load_fill(const LoadState* L, char* stg) {
     if (L->grammar_fresh) grammar_image(s->g, stg + L->head);
 }
 
+// The launches that make subtree tables: sizes 1 and 3 together, then one after the other (even sizes have no trees).
+static cudaError_t make_tables(const LoadJob* jobs, int n_jobs, int size_cap, int probes_cap, const u64* entries_at) {
+    if (size_cap < 1) return cudaSuccess;
+    cudaError_t e = launch_subvalues(jobs, n_jobs, 1, 3, probes_cap, entries_at[1] + (size_cap >= 3 ? entries_at[3] : 0), nullptr);
+    for (int k = 5; k <= size_cap && e == cudaSuccess; k += 2) e = launch_subvalues(jobs, n_jobs, k, k, probes_cap, entries_at[k], nullptr);
+    return e;
+}
+
 // One load at a time: all of them work on the default stream anyway, and a grammar's tables are sent by the first
 // load that needs them.
 static std::mutex g_load_mu;
@@ -1025,7 +1033,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             return ok ? fail(XP_ERR_CUDA, std::string("xp_sketch_load: ") + cudaGetErrorString(err)) : fail(XP_ERR_NOMEM, "out of host memory");
         }
         // host tables too large for the staged copy
-        i64 most_points = 0, most_box = 0, most_spec = 0;
+        i64 most_points = 0, most_staged = 0;
         int size_cap = 0, probes_cap = 0;
         u64 most_entries[kMaxSize + 1] = {0};
         for (size_t i = 0; i < n; ++i) {
@@ -1045,10 +1053,10 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
                     XP_CUDA_B(cudaMemcpyAsync(s->arena + L.off_spec[h], hd.spec_table, spec_bytes, cudaMemcpyHostToDevice, nullptr));
                     s->load_h2d += spec_bytes;
                 }
-                if (hd.spec_kind == XP_SPEC_EXPR && L.stage && s->n_points > most_spec) most_spec = s->n_points;
+                if (hd.spec_kind == XP_SPEC_EXPR && L.stage && s->n_points > most_staged) most_staged = s->n_points;
             }
             if (L.d->domain_kind == XP_DOMAIN_TABLE && s->n_points > most_points) most_points = s->n_points;
-            if (L.stage_box && s->n_points > most_box) most_box = s->n_points;
+            if (L.stage_box && s->n_points > most_staged) most_staged = s->n_points;
             if (s->tab_size_cap > size_cap) size_cap = s->tab_size_cap;
             if (s->tab_probes_cap > probes_cap) probes_cap = s->tab_probes_cap;
             for (int k = 1; k <= s->tab_size_cap; ++k) most_entries[k] = s->entries_at[k] > most_entries[k] ? s->entries_at[k] : most_entries[k];
@@ -1062,19 +1070,18 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         const LoadJob* d_jobs = (const LoadJob*)(dev_block + at_jobs);
         for (size_t q = 0; q < n; q += kJobs) {
             const int m = (int)(n - q < kJobs ? n - q : kJobs);
-            XP_CUDA_B(launch_stage_points(d_list + q, m, most_box, nullptr));
             XP_CUDA_B(launch_coord_bounds(d_list + q, m, most_points, nullptr));
         }
         for (size_t q = 0; q < n_jobs; q += kJobs) {
             const int m = (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs);
-            XP_CUDA_B(launch_stage_spec(d_jobs + q, m, most_spec, nullptr));
-            XP_CUDA_B(launch_prepare(d_jobs + q, m, dev_block + at_scratch, (LoadOut*)(dev_block + at_out) + q, nullptr));
+            XP_CUDA_B(launch_stage(d_jobs + q, m, most_staged, nullptr));
+            // (what it decides per hole goes straight to page-locked memory: a few bytes, and no copy to queue behind the tables)
+            LoadOut* out = (LoadOut*)(back.locked ? back.p : dev_block + at_out);
+            XP_CUDA_B(launch_prepare(d_jobs + q, m, dev_block + at_scratch, out + q, nullptr));
         }
-        for (int k = 1; k <= size_cap; ++k)
-            for (size_t q = 0; q < n_jobs; q += kJobs)
-                XP_CUDA_B(launch_subvalues(d_jobs + q, (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs), k, probes_cap, most_entries[k], nullptr));
-        // what the kernels decided, per hole
-        XP_CUDA_B(cudaMemcpyAsync(back.p, dev_block + at_out, sizeof(LoadOut) * n_jobs, cudaMemcpyDeviceToHost, nullptr));
+        for (size_t q = 0; q < n_jobs; q += kJobs)
+            XP_CUDA_B(make_tables(d_jobs + q, (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs), size_cap, probes_cap, most_entries));
+        if (!back.locked) XP_CUDA_B(cudaMemcpyAsync(back.p, dev_block + at_out, sizeof(LoadOut) * n_jobs, cudaMemcpyDeviceToHost, nullptr));
         XP_CUDA_B(cudaStreamSynchronize(nullptr));
     }
 #undef XP_CUDA_B
@@ -1194,8 +1201,7 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         cudaError_t e = cudaMemcpyAsync(s->arena + s->off_holes, hh.data(), sizeof(HoleDev) * nh, cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(LoadJob) * jobs.size(), cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = launch_reprobe((const LoadJob*)jobs_dev, (int)jobs.size(), nullptr);
-        for (int k = 1; k <= s->tab_size_cap && e == cudaSuccess; ++k)
-            e = launch_subvalues((const LoadJob*)jobs_dev, (int)jobs.size(), k, s->tab_probes_cap, s->entries_at[k], nullptr);
+        if (e == cudaSuccess) e = make_tables((const LoadJob*)jobs_dev, (int)jobs.size(), s->tab_size_cap, s->tab_probes_cap, s->entries_at);
         if (e == cudaSuccess) e = cudaMemcpyAsync(hh.data(), s->arena + s->off_holes, sizeof(HoleDev) * nh, cudaMemcpyDeviceToHost, nullptr);
         const cudaError_t e2 = cudaStreamSynchronize(nullptr);
         pool_release(jobs_dev, jobs_bytes, jobs_device);

@@ -89,6 +89,7 @@ __device__ __forceinline__ u64 sig_hash(const i64* s, int n) {
 }
 
 __global__ void beh_points_kernel(BehDev* B) {
+    chain_wait();
     const int t = threadIdx.x;
     const SketchDev* sk = B->sk;
     bool ok = false;
@@ -177,6 +178,7 @@ __device__ __forceinline__ bool beh_same(const BehDev* B, const BehPass& P, u64 
 
 template <int NS>                                         // n_sig <= NS: the signature stays in registers
 __global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n) {
+    chain_wait();
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= chunk_n) return;
     const int ns = B->n_sig;
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, cons
 }
 
 __global__ void __launch_bounds__(kBehThreads) beh_flag_kernel(BehDev* B, int nt, u64 chunk_first, u32 chunk_n) {
+    chain_wait();
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     bool is_new = false;
     if (c < chunk_n) {
@@ -244,6 +247,7 @@ __device__ __forceinline__ u64 range_id(const BehRanges& R, u64 i) {
 
 // Representatives of a nonterminal into its (cleared) table.
 __global__ void __launch_bounds__(kBehThreads) beh_rehash_kernel(BehDev* B, int nt, u64 mask, const __grid_constant__ BehRanges R) {
+    chain_wait();
     const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= R.total) return;
     const u64 id = range_id(R, i);
@@ -257,6 +261,7 @@ __global__ void __launch_bounds__(kBehThreads) beh_rehash_kernel(BehDev* B, int 
 }
 
 __global__ void __launch_bounds__(1024) beh_scan_kernel(BehDev* B, int n_blocks) {
+    chain_wait();
     __shared__ u32 part[1024];
     const int t = threadIdx.x;
     const int per = (n_blocks + 1023) / 1024;
@@ -277,6 +282,7 @@ __global__ void __launch_bounds__(1024) beh_scan_kernel(BehDev* B, int n_blocks)
 }
 
 __global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n, u64 rep_base) {
+    chain_wait();
     __shared__ u32 warp_sum[kBehThreads / 32];
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -305,6 +311,7 @@ __global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, cons
 
 // All of them against the constraint at the signature points.
 __global__ void __launch_bounds__(kBehThreads) beh_match_kernel(BehDev* B, const __grid_constant__ BehRanges R) {
+    chain_wait();
     const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= R.total) return;
     const u64 id = range_id(R, i);
@@ -354,6 +361,7 @@ __device__ bool rep_value(const BehDev* B, u32 gid, const i64* pt, i64& out) {
 }
 
 __global__ void __launch_bounds__(kBehThreads) beh_verify_kernel(BehDev* B, u32 gid) {
+    chain_wait();
     const SketchDev* sk = B->sk;
     const HoleDev* hole = B->hole;
     if (blockIdx.x == 0 && threadIdx.x == 0) {            // its tree, for the text: nodes in preorder
@@ -442,7 +450,7 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
     cu(cudaMemcpyAsync(dB, &h, sizeof(h), cudaMemcpyHostToDevice, stream));
     if (cu.ok()) cu(cudaEventRecord(ev.e0, stream));
     int launches = 0;
-    if (cu.ok()) { beh_points_kernel<<<1, 32, 0, stream>>>(dB); ++launches; cu(cudaGetLastError()); }
+    if (cu.ok()) { chain(beh_points_kernel, 1, 32, 0, stream, dB); ++launches; cu(cudaGetLastError()); }
     std::vector<std::vector<u64>> count(n_nt, std::vector<u64>(K + 1, 0)), base(n_nt, std::vector<u64>(K + 1, 0));
     std::vector<u64> table(n_nt, 0), held(n_nt, 0);       // per nonterminal: size of its table so far, representatives in it
     auto ranges_of = [&](int nt) {
@@ -487,16 +495,16 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
                     cu(cudaMemsetAsync((u64*)(block + o_tab) + tsize * nt, 0xff, sizeof(u64) * want, stream));
                     const BehRanges R = ranges_of(nt);
                     if (R.total > 0 && cu.ok()) {
-                        beh_rehash_kernel<<<(unsigned)((R.total + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream>>>(dB, nt, want - 1, R);
+                        chain(beh_rehash_kernel, (unsigned)((R.total + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream, dB, nt, want - 1, R);
                         ++launches;
                     }
                     table[nt] = want;
                 }
                 P.mask = table[nt] - 1;
-                if (ns <= 8) beh_insert_kernel<8><<<nb, kBehThreads, 0, stream>>>(dB, P, first, n);
-                else beh_insert_kernel<XP_MAX_SIG><<<nb, kBehThreads, 0, stream>>>(dB, P, first, n);
-                beh_flag_kernel<<<nb, kBehThreads, 0, stream>>>(dB, nt, first, n);
-                beh_scan_kernel<<<1, 1024, 0, stream>>>(dB, nb);
+                if (ns <= 8) chain(beh_insert_kernel<8>, nb, kBehThreads, 0, stream, dB, P, first, n);
+                else chain(beh_insert_kernel<XP_MAX_SIG>, nb, kBehThreads, 0, stream, dB, P, first, n);
+                chain(beh_flag_kernel, nb, kBehThreads, 0, stream, dB, nt, first, n);
+                chain(beh_scan_kernel, 1, 1024, 0, stream, dB, nb);
                 launches += 3;
                 cu(cudaGetLastError());
                 cu(cudaMemcpyAsync(&back.chunk_new, (char*)dB + kBackAt, 2 * sizeof(u64), cudaMemcpyDeviceToHost, stream));
@@ -508,7 +516,7 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
                     why = "xp_behaviours: more than " + std::to_string(max_reps) + " representatives (size " + std::to_string(s) + ")";
                     break;
                 }
-                beh_append_kernel<<<nb, kBehThreads, 0, stream>>>(dB, P, first, n, n_reps);
+                chain(beh_append_kernel, nb, kBehThreads, 0, stream, dB, P, first, n, n_reps);
                 ++launches;
                 cu(cudaGetLastError());
                 n_reps += back.chunk_new;
@@ -522,7 +530,7 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
     std::vector<u32> ids;
     if (cu.ok() && st == XP_OK) {
         const BehRanges R = ranges_of(hs.start_nt);
-        if (R.total > 0) { beh_match_kernel<<<(unsigned)((R.total + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream>>>(dB, R); ++launches; }
+        if (R.total > 0) { chain(beh_match_kernel, (unsigned)((R.total + kBehThreads - 1) / kBehThreads), kBehThreads, 0, stream, dB, R); ++launches; }
         cu(cudaGetLastError());
         cu(cudaMemcpyAsync(&back.chunk_new, (char*)dB + kBackAt, sizeof(BehDev) - kBackAt, cudaMemcpyDeviceToHost, stream));
         cu(cudaStreamSynchronize(stream));
@@ -561,7 +569,7 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
     for (size_t k = 0; k < ids.size() && cu.ok() && st == XP_OK && !out->solved; ++k) {
         if (k > 0) cu(cudaMemsetAsync((char*)dB + kCheckAt, 0, sizeof(u32), stream));
         const i64 want = (si.n_points + kBehThreads - 1) / kBehThreads;
-        beh_verify_kernel<<<(unsigned)(want < 1 ? 1 : want < sms * 8 ? want : sms * 8), kBehThreads, 0, stream>>>(dB, ids[k]);
+        chain(beh_verify_kernel, (unsigned)(want < 1 ? 1 : want < sms * 8 ? want : sms * 8), kBehThreads, 0, stream, dB, ids[k]);
         ++launches;
         cu(cudaGetLastError());
         cu(cudaMemcpyAsync(&back.verify_fail, (char*)dB + kCheckAt, sizeof(BehDev) - kCheckAt, cudaMemcpyDeviceToHost, stream));

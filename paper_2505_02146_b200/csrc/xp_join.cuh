@@ -1346,6 +1346,7 @@ __device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, con
 
 template <int P>
 __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_constant__ PlanDev plan) {
+    chain_wait();
     __shared__ JoinWarp sh[kJoinWarps];
     JoinWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;

@@ -123,6 +123,7 @@ __device__ __forceinline__ bool eval_joint(const xp_instr* code, int n, const i6
 }
 
 __global__ void joint_probe_kernel(JointDev* J, int affine) {
+    chain_wait();
     const int t = threadIdx.x;
     const SketchDev* sk = J->sk;
     bool ok = false;
@@ -156,6 +157,7 @@ __device__ __forceinline__ int joint_locate(const JointDev* J, int part, u64 e, 
 }
 
 __global__ void __launch_bounds__(128) joint_key_kernel(JointDev* J, int part) {
+    chain_wait();
     const SketchDev* sk = J->sk;
     const GrammarDev* g = sk->g;
     const u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x;
@@ -195,6 +197,7 @@ __global__ void __launch_bounds__(128) joint_key_kernel(JointDev* J, int part) {
 }
 
 __global__ void __launch_bounds__(256) joint_values_kernel(JointDev* J, int part, int size) {
+    chain_wait();
     const SketchDev* sk = J->sk;
     const GrammarDev* g = sk->g;
     const int nt = J->start_nt[part];
@@ -240,6 +243,7 @@ __device__ __noinline__ bool joint_check_domain(const JointDev* J, int s0, u64 r
 }
 
 __global__ void __launch_bounds__(256) joint_pairs_kernel(JointDev* J, int s0, int s1, u64 n0, u64 n1) {
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const u64 pairs = n0 * n1;
     const u64 stride = (u64)gridDim.x * blockDim.x;
@@ -284,6 +288,7 @@ __global__ void __launch_bounds__(256) joint_pairs_kernel(JointDev* J, int s0, i
 
 // A warp per listed pair.
 __global__ void __launch_bounds__(256) joint_check_kernel(JointDev* J) {
+    chain_wait();
     const u64 n = J->listed;
     if (n > kJointList) return;                           // (the list ran over: the host takes the other form)
     u64 evals = 0;
@@ -469,19 +474,19 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
         if (e == cudaSuccess && form == 0) e = cudaMemsetAsync(block + off_head, 0xff, sizeof(u32) * heads, stream);
         if (e == cudaSuccess) e = cudaEventRecord(ev.e0, stream);
         if (e == cudaSuccess) {
-            joint_probe_kernel<<<1, 32, 0, stream>>>(dJ, form == 0 ? 1 : 0);
+            chain(joint_probe_kernel, 1, 32, 0, stream, dJ, form == 0 ? 1 : 0);
             ++launches;
             e = cudaGetLastError();
         }
         if (form == 0) {
             for (int part = 1; part >= 0 && e == cudaSuccess; --part) {
                 if (entries[part] == 0) continue;
-                joint_key_kernel<<<(unsigned)((entries[part] + 127) / 128), 128, 0, stream>>>(dJ, part);
+                chain(joint_key_kernel, (unsigned)((entries[part] + 127) / 128), 128, 0, stream, dJ, part);
                 ++launches;
                 e = cudaGetLastError();
             }
             if (e == cudaSuccess) {
-                joint_check_kernel<<<(unsigned)sms * 4, 256, 0, stream>>>(dJ);
+                chain(joint_check_kernel, (unsigned)sms * 4, 256, 0, stream, dJ);
                 ++launches;
                 e = cudaGetLastError();
             }
@@ -490,7 +495,7 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
                 for (int s = 1; s <= d->max_size[k] && e == cudaSuccess; ++s) {
                     const u64 c = grammar_cnt(si.g, d->start_nt[k], s);
                     if (c == 0) continue;
-                    joint_values_kernel<<<dim3((unsigned)((c + 255) / 256), (unsigned)n_probe), 256, 0, stream>>>(dJ, k, s);
+                    chain(joint_values_kernel, dim3((unsigned)((c + 255) / 256), (unsigned)n_probe), 256, 0, stream, dJ, k, s);
                     ++launches;
                     e = cudaGetLastError();
                 }
@@ -501,7 +506,7 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
                     const u64 n0 = grammar_cnt(si.g, d->start_nt[0], s0), n1 = grammar_cnt(si.g, d->start_nt[1], s1);
                     if (n0 == 0 || n1 == 0) continue;
                     const u64 want = (n0 * n1 + 255) / 256, most = (u64)sms * 8;
-                    joint_pairs_kernel<<<(unsigned)(want < most ? want : most), 256, 0, stream>>>(dJ, s0, s1, n0, n1);
+                    chain(joint_pairs_kernel, (unsigned)(want < most ? want : most), 256, 0, stream, dJ, s0, s1, n0, n1);
                     ++launches;
                     e = cudaGetLastError();
                 }

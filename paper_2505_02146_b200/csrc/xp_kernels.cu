@@ -2,7 +2,7 @@
 //
 //   prep_sample_kernel, prepare_kernel -- per sketch, once at load: coordinates and spec values of the
 //                      sample points, choice and order of each hole's probe points.
-//   subvalue_kernel, stage_points_kernel, stage_spec_kernel, coord_bounds_kernel -- per sketch,
+//   subvalue_kernel, stage_kernel, coord_bounds_kernel -- per sketch,
 //                      once at load: values (and variable sets) of all small subtrees at the probes;
 //                      points and spec values of a box; coordinate bounds of a table.
 //   join_kernel     -- (xp_join.cuh) the part of the search whose candidates have a leaf at the root.
@@ -309,6 +309,7 @@ __device__ __forceinline__ int prep_sizes(const GrammarDev* g, const HoleDev* ho
 }
 
 __global__ void __launch_bounds__(32 * kPrepWarps) prep_sample_kernel(const LoadJob* jobs, u32* masks) {
+    chain_wait();
     constexpr int kHere = kPrepWarps * kPrepEach;        // samples of this CTA
     const SketchDev* s = jobs[blockIdx.z].s;
     const HoleDev* hole = &s->holes[jobs[blockIdx.z].hole];
@@ -364,6 +365,7 @@ __global__ void __launch_bounds__(32 * kPrepWarps) prep_sample_kernel(const Load
 
 constexpr int kPrepThreads = 64;                        // one thread per sample
 __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jobs, const u32* masks, LoadOut* out) {
+    chain_wait();
     SketchDev* s = jobs[blockIdx.x].s;
     __shared__ i64 s_pt[kProbeSamples][kMaxVars];
     __shared__ i64 s_spec[kProbeSamples];
@@ -1219,27 +1221,96 @@ __device__ __noinline__ u32 fill_reg_operands(const GrammarDev* g, const HoleDev
 // The shares of a load's staged copy to their places: one grid row per share, 16 bytes per thread and step (sources
 // and destinations are 256-byte aligned, lengths multiples of 256).
 __global__ void __launch_bounds__(256) scatter_kernel(const LoadCopy* copies, const char* src) {
+    chain_wait();
     const LoadCopy c = copies[blockIdx.y];
     const uint4* from = reinterpret_cast<const uint4*>(src + c.src);
     uint4* to = reinterpret_cast<uint4*>(c.dst);
     for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < c.bytes / 16; i += (u64)gridDim.x * blockDim.x) to[i] = from[i];
 }
 
-// Staging of the box domains of a load: the coordinates of every point (int32 rows, like a table
-// domain) and, per hole with a spec expression, the spec's value at every point.  spec_bad is set
-// if the spec is undefined somewhere (then no candidate can match).  One grid row per sketch or hole.
-__global__ void __launch_bounds__(256) stage_points_kernel(SketchDev* const* list) {
-    const SketchDev* sk = list[blockIdx.y];
-    if (!sk->project) return;
+// Value of a spec expression at kStageEach points (pt[variable][point]); false where it is undefined.  The instructions are
+// decoded once for all of them.
+constexpr int kStageEach = 4;
+__device__ __forceinline__ bool eval_code_at(const xp_instr* __restrict__ code, int n, const i64 (*pt)[kStageEach], int n_pt, i64* out) {
+    i64 st[kMaxStack][kStageEach];
+    int sp = 0;
+    bool ok = true;
+    for (int i = 0; i < n; ++i) {
+        const xp_instr c = code[i];
+        if (c.kind == XP_I_OP) {
+            --sp;
+            i64 *x = st[sp - 1], *y = st[sp];
+            if (c.arg <= XP_OP_MUL) {
+#pragma unroll
+                for (int k = 0; k < kStageEach; ++k) {
+                    const u64 u = (u64)x[k], v = (u64)y[k];
+                    x[k] = (i64)(c.arg == XP_OP_ADD ? u + v : c.arg == XP_OP_SUB ? u - v : u * v);
+                }
+            } else {
+#pragma unroll 1
+                for (int k = 0; k < n_pt; ++k) {
+                    i64 r;
+                    if (apply_op(c.arg, x[k], y[k], r)) x[k] = r;
+                    else ok = false;
+                }
+            }
+        } else {
+            if (!XP_CHECKED(sp < kMaxStack, kChkStack)) return false;
+#pragma unroll
+            for (int k = 0; k < kStageEach; ++k) st[sp][k] = c.kind == XP_I_VAR ? pt[c.arg][k] : c.value;
+            ++sp;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kStageEach; ++k) out[k] = st[0][k];
+    return ok;
+}
+
+// Staging of a load: for a box the coordinates of every point (int32 rows, like a table domain; written for the sketch's first
+// hole) and, per hole with a spec expression, the spec's value at every point.  spec_bad is set
+// if the spec is undefined somewhere (then no candidate can match).  One grid row per hole.
+// Bound by the interpreter's chain of local and constant loads, hence kStageEach points per thread (load of three holes of
+// 1.8 million points: 265 -> 239 us), and by the launches where domains are small, hence one kernel.
+__global__ void __launch_bounds__(256) stage_kernel(const LoadJob* jobs) {
+    chain_wait();
+    const LoadJob job = jobs[blockIdx.y];
+    const SketchDev* sk = job.s;
+    HoleDev* hole = &sk->holes[job.hole];
+    const bool rows = job.hole == 0 && sk->project, values = hole->spec_len != 0 && hole->spec_table != nullptr;
+    if (!rows && !values) return;
+    i64* spec = const_cast<i64*>(hole->spec_table);
     i32* coords = const_cast<i32*>(sk->coords);
     const int nv = sk->n_vars;
-    for (i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x; pid < sk->n_points; pid += (i64)gridDim.x * blockDim.x) {
-        u64 rem = (u64)pid;
-        for (int d = nv - 1; d >= 0; --d) {
-            u64 q, r;
-            divmod_u64(rem, (u64)sk->ext[d], q, r);
-            coords[pid * nv + d] = (i32)(sk->lo[d] + (i64)r);
-            rem = q;
+    const bool box = sk->project || coords == nullptr;
+    const i64 n = sk->n_points, step = (i64)gridDim.x * 256 * kStageEach;
+    for (i64 at = (i64)blockIdx.x * 256 * kStageEach + threadIdx.x; at < n; at += step) {
+        i64 pt[kMaxVars][kStageEach];
+        int n_pt = 0;
+#pragma unroll
+        for (int k = 0; k < kStageEach; ++k) {
+            i64 pid = at + 256 * k;
+            if (pid < n) n_pt = k + 1;
+            else pid = at;                                // (past the end: the first point again)
+            if (box) {
+                u64 rem = (u64)pid;
+                for (int d = nv - 1; d >= 0; --d) {
+                    u64 q, r;
+                    divmod_u64(rem, (u64)sk->ext[d], q, r);
+                    pt[d][k] = sk->lo[d] + (i64)r;
+                    rem = q;
+                }
+            } else {
+                for (int d = 0; d < nv; ++d) pt[d][k] = coords[pid * nv + d];
+            }
+        }
+        if (rows)
+            for (int k = 0; k < n_pt; ++k)
+                for (int d = 0; d < nv; ++d) coords[(at + 256 * k) * nv + d] = (i32)pt[d][k];
+        if (values) {
+            i64 v[kStageEach];
+            if (!eval_code_at(hole->spec, hole->spec_len, pt, n_pt, v)) atomicOr(&hole->spec_bad, 1u);
+#pragma unroll
+            for (int k = 0; k < kStageEach; ++k) if (k < n_pt) spec[at + 256 * k] = v[k];
         }
     }
 }
@@ -1248,6 +1319,7 @@ __global__ void __launch_bounds__(256) stage_points_kernel(SketchDev* const* lis
 // sketch (whose vmin / vmax start at the extreme values).  Warp shuffles, then one atomic pair
 // per warp and variable.
 __global__ void __launch_bounds__(256) coord_bounds_kernel(SketchDev* const* list) {
+    chain_wait();
     SketchDev* sk = list[blockIdx.y];                   // one grid row per sketch of the batch
     if (sk->domain_kind != XP_DOMAIN_TABLE) return;
     const int nv = sk->n_vars;
@@ -1268,26 +1340,14 @@ __global__ void __launch_bounds__(256) coord_bounds_kernel(SketchDev* const* lis
     }
 }
 
-__global__ void __launch_bounds__(256) stage_spec_kernel(const LoadJob* jobs) {
-    const SketchDev* sk = jobs[blockIdx.y].s;
-    HoleDev* hole = &sk->holes[jobs[blockIdx.y].hole];
-    if (hole->spec_len == 0 || hole->spec_table == nullptr) return;
-    i64* spec = const_cast<i64*>(hole->spec_table);
-    for (i64 pid = (i64)blockIdx.x * blockDim.x + threadIdx.x; pid < sk->n_points; pid += (i64)gridDim.x * blockDim.x) {
-        i64 pt[kMaxVars];
-        point_coords(sk, pid, pt);
-        i64 v = 0;
-        if (!eval_code(hole->spec, hole->spec_len, pt, 0, v)) atomicOr(&hole->spec_bad, 1u);
-        spec[pid] = v;
-    }
-}
-
-// Bottom-up construction of one size of a hole's subtree-value tables: thread = (nonterminal,
+// Bottom-up construction of a hole's subtree-value tables: thread = (size, nonterminal,
 // rank) and one group of kSubProbes probes; the operands' values come from the smaller sizes built by
-// earlier launches.  (One thread for several probes: the unranking, two 64-bit divisions, is done once for them.)
+// earlier launches.  The first launch makes sizes 1 and 3: the operands of size 3 are leaves, whose values come from the
+// probes themselves.  (One thread for several probes: the unranking, two 64-bit divisions, is done once for them.)
 // The first group also writes what does not depend on the probe, and the pair of values the leaf join reads.
 constexpr int kSubProbes = 4;
-__global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int size) {
+__global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int size, int last) {
+    chain_wait();
     const SketchDev* sk = jobs[blockIdx.z].s;           // one grid layer per hole of the batch
     HoleDev* hole = &sk->holes[jobs[blockIdx.z].hole];
     const int pr0 = blockIdx.y * kSubProbes;            // one grid row per group of probes
@@ -1299,6 +1359,8 @@ __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int 
     i64* __restrict__ tab_val = hole->tab_val;
     unsigned char* __restrict__ tab_ok = hole->tab_ok;
     u64 idx = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    const i32 most = hole->tab_max_size < last ? hole->tab_max_size : last;
+    for (; size <= most; size += 2)                       // (every node has no or two children: only odd sizes)
     for (int nt = 0; nt < g->n_nt; ++nt) {
         const u64 c = g->cnt[nt][size];
         if (idx >= c) { idx -= c; continue; }
@@ -1307,6 +1369,7 @@ __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int 
         int op = 0;
         u64 la = 0, ra = 0;
         u32 vars = 0;
+        LeafDev rf{-1, 0, 0};
         if (size == 1) {
             lf = g->leaves[g->leaf_begin[nt] + (i32)idx];
             vars = lf.var >= 0 ? 1u << lf.var : 0u;
@@ -1314,8 +1377,13 @@ __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int 
             int lnt, rnt, a;
             u64 l, r;
             unrank_root(g, nt, size, idx, op, lnt, rnt, a, l, r);
-            la = hole->tab_off[lnt][a] + l; ra = hole->tab_off[rnt][size - 1 - a] + r;
-            if (pr0 == 0) vars = (u32)hole->tab_vars[la] | (u32)hole->tab_vars[ra];
+            if (size == 3) {
+                lf = g->leaves[g->leaf_begin[lnt] + (i32)l]; rf = g->leaves[g->leaf_begin[rnt] + (i32)r];
+                vars = (lf.var >= 0 ? 1u << lf.var : 0u) | (rf.var >= 0 ? 1u << rf.var : 0u);
+            } else {
+                la = hole->tab_off[lnt][a] + l; ra = hole->tab_off[rnt][size - 1 - a] + r;
+                if (pr0 == 0) vars = (u32)hole->tab_vars[la] | (u32)hole->tab_vars[ra];
+            }
         }
         i64 v[kSubProbes];
         bool ok[kSubProbes];
@@ -1324,7 +1392,9 @@ __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int 
             v[k] = 0; ok[k] = true;
             if (k >= n_pr) continue;
             const u64 pbase = (u64)(pr0 + k) * total;
-            if (size == 1) v[k] = lf.var >= 0 ? hole->probe_pt[pr0 + k][lf.var] : lf.value;
+            auto leaf = [&](const LeafDev& f) { return f.var >= 0 ? hole->probe_pt[pr0 + k][f.var] : f.value; };
+            if (size == 1) v[k] = leaf(lf);
+            else if (size == 3) ok[k] = apply_op(op, leaf(lf), leaf(rf), v[k]);
             else ok[k] = tab_ok[pbase + la] && tab_ok[pbase + ra] && apply_op(op, tab_val[pbase + la], tab_val[pbase + ra], v[k]);
         }
 #pragma unroll
@@ -2214,6 +2284,7 @@ __device__ __noinline__ void tile_ticket(EvalShared& sh, const PlanDev& plan, co
 #endif
 template <bool DENSE>
 __global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const __grid_constant__ PlanDev plan) {
+    chain_wait();
     __shared__ EvalShared sh;
     u64 my_evals = 0;
     if (threadIdx.x <= kMaxSize) { sh.match_count[threadIdx.x] = 0; sh.min_rank[threadIdx.x] = ~0ull; }
@@ -2305,6 +2376,7 @@ __device__ __noinline__ void record_killer(const HoleDev* hole, i64 pid) {
 
 // One CTA: exclusive scan of hist[0 .. n_acc) into off[0 .. n_acc]; hist is cleared for the scatter.
 __global__ void __launch_bounds__(1024) surv_scan_kernel(u32* hist, u32* off, int n_acc) {
+    chain_wait();
     __shared__ u32 part[1024];
     const int t = threadIdx.x;
     const int per = (n_acc + 1023) / 1024;
@@ -2325,6 +2397,7 @@ __global__ void __launch_bounds__(1024) surv_scan_kernel(u32* hist, u32* off, in
 }
 
 __global__ void __launch_bounds__(256) surv_scatter_kernel(const __grid_constant__ PlanDev plan) {
+    chain_wait();
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
     const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2736,6 +2809,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
 constexpr int kVerifyThreads = 256;
 constexpr int kVerifyWarps = kVerifyThreads / 32;
 __global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const __grid_constant__ PlanDev plan) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char verify_smem[];
     VerifyWarp& w = reinterpret_cast<VerifyWarp*>(verify_smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -2843,6 +2917,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const __grid_
 
 // One thread per queued survivor of a sketch without points: there is no chunk to pass, it is a match.
 __global__ void count_kernel(const __grid_constant__ PlanDev plan) {
+    chain_wait();
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
     const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2936,10 +3011,10 @@ size_t prepare_scratch_bytes(int n_jobs) { return sizeof(u32) * (size_t)kProbeSa
 
 cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadOut* out, cudaStream_t stream) {
     if (n_jobs <= 0) return cudaSuccess;
-    prep_sample_kernel<<<dim3(kPrepWords, kPrepSplit, (unsigned)n_jobs), 32 * kPrepWarps, 0, stream>>>(jobs, (u32*)scratch);
+    chain(prep_sample_kernel, dim3(kPrepWords, kPrepSplit, (unsigned)n_jobs), 32 * kPrepWarps, 0, stream, jobs, (u32*)scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    prepare_kernel<<<n_jobs, kPrepThreads, 0, stream>>>(jobs, (const u32*)scratch, out);
+    chain(prepare_kernel, n_jobs, kPrepThreads, 0, stream, jobs, (const u32*)scratch, out);
     return cudaGetLastError();
 }
 
@@ -2952,35 +3027,28 @@ cudaError_t launch_reprobe(const LoadJob* jobs, int n_jobs, cudaStream_t stream)
 cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream) {
     if (most_points <= 0 || n_sketches <= 0) return cudaSuccess;
     const i64 blocks = (most_points + 255) / 256;
-    coord_bounds_kernel<<<dim3((unsigned)(blocks < 64 ? blocks : 64), (unsigned)n_sketches), 256, 0, stream>>>(list);
+    chain(coord_bounds_kernel, dim3((unsigned)(blocks < 64 ? blocks : 64), (unsigned)n_sketches), 256, 0, stream, list);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src, cudaStream_t stream) {
     for (int at = 0; at < n_copies; at += 65535) {
         const int m = n_copies - at < 65535 ? n_copies - at : 65535;
-        scatter_kernel<<<dim3(m > 64 ? 4u : 16u, (unsigned)m), 256, 0, stream>>>(copies + at, src);
+        chain(scatter_kernel, dim3(m > 64 ? 4u : 16u, (unsigned)m), 256, 0, stream, copies + at, src);
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_stage_points(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream) {
-    if (most_points <= 0 || n_sketches <= 0) return cudaSuccess;
-    const i64 blocks = (most_points + 255) / 256;
-    stage_points_kernel<<<dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_sketches), 256, 0, stream>>>(list);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_stage_spec(const LoadJob* jobs, int n_jobs, i64 most_points, cudaStream_t stream) {
+cudaError_t launch_stage(const LoadJob* jobs, int n_jobs, i64 most_points, cudaStream_t stream) {
     if (most_points <= 0 || n_jobs <= 0) return cudaSuccess;
-    const i64 blocks = (most_points + 255) / 256;
-    stage_spec_kernel<<<dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_jobs), 256, 0, stream>>>(jobs);
+    const i64 blocks = (most_points + 256 * kStageEach - 1) / (256 * kStageEach);
+    chain(stage_kernel, dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_jobs), 256, 0, stream, jobs);
     return cudaGetLastError();
 }
 
-cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int most_probes, u64 most_entries, cudaStream_t stream) {
+cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last, int most_probes, u64 most_entries, cudaStream_t stream) {
     if (most_entries == 0 || most_probes <= 0 || n_jobs <= 0) return cudaSuccess;
-    subvalue_kernel<<<dim3((unsigned)((most_entries + 255) / 256), (unsigned)((most_probes + kSubProbes - 1) / kSubProbes), (unsigned)n_jobs), 256, 0, stream>>>(jobs, size);
+    chain(subvalue_kernel, dim3((unsigned)((most_entries + 255) / 256), (unsigned)((most_probes + kSubProbes - 1) / kSubProbes), (unsigned)n_jobs), 256, 0, stream, jobs, size, last);
     return cudaGetLastError();
 }
 
@@ -3064,15 +3132,15 @@ cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64
         // a wave of persistent CTAs; a small search gets one warp per ticket on as many SMs as there are tickets
         u64 ctas = t_end - t_begin;
         if (ctas > (u64)R->join) ctas = R->join;
-        if (L.join_wide) join_kernel<kJoinP><<<(unsigned)ctas, kJoinThreads, 0, stream>>>(pd);
-        else join_kernel<1><<<(unsigned)ctas, kJoinThreads, 0, stream>>>(pd);
+        if (L.join_wide) chain(join_kernel<kJoinP>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
+        else chain(join_kernel<1>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
     } else {
         pd.ticket_base = t_begin;
         pd.n_tickets = t_end;
         u64 ctas = (u64)(L.dense ? R->eval_dense : R->eval_sparse);       // persistent CTAs: one wave
         if (ctas > t_end - t_begin) ctas = t_end - t_begin;
-        if (L.dense) eval_kernel<true><<<(unsigned)ctas, kThreads, 0, stream>>>(pd);
-        else eval_kernel<false><<<(unsigned)ctas, kThreads, 0, stream>>>(pd);
+        if (L.dense) chain(eval_kernel<true>, (unsigned)ctas, kThreads, 0, stream, pd);
+        else chain(eval_kernel<false>, (unsigned)ctas, kThreads, 0, stream, pd);
     }
     *n_launches += 1;
     return cudaGetLastError();
@@ -3094,18 +3162,18 @@ cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_
             const u32 want = (n + kPairThreads - 1) / kPairThreads, cap = (u32)(R->sms * per_sm);
             return want < cap ? want : cap;
         };
-        pair_build_kernel<<<(most + kPairThreads - 1) / kPairThreads, kPairThreads, 0, stream>>>(pd, i);
-        pair_hash_kernel<<<ctas(drive, 3), kPairThreads, 0, stream>>>(pd, i);
+        chain(pair_build_kernel, (most + kPairThreads - 1) / kPairThreads, kPairThreads, 0, stream, pd, i);
+        chain(pair_hash_kernel, ctas(drive, 3), kPairThreads, 0, stream, pd, i);
         *n_launches += 2;
         if (s.ops & 24u) {                                // / or %
-            pair_sort_count_kernel<<<dim3(ctas(most, 2), 2), kPairThreads, 0, stream>>>(pd, i);
-            pair_sort_scan_kernel<<<2, kPairBuckets, 0, stream>>>(pd, i);
-            pair_sort_scatter_kernel<<<dim3(ctas(most, 4), 2), kPairThreads, 0, stream>>>(pd, i);
+            chain(pair_sort_count_kernel, dim3(ctas(most, 2), 2), kPairThreads, 0, stream, pd, i);
+            chain(pair_sort_scan_kernel, 2, kPairBuckets, 0, stream, pd, i);
+            chain(pair_sort_scatter_kernel, dim3(ctas(most, 4), 2), kPairThreads, 0, stream, pd, i);
             const u64 warps = (u64)((s.nl + 31) / 32) * s.pieces, cap = (u64)R->sms * 3 * kPairWarps;
-            pair_div_kernel<<<(unsigned)(((warps < cap ? warps : cap) + kPairWarps - 1) / kPairWarps), kPairThreads, 0, stream>>>(pd, i);
+            chain(pair_div_kernel, (unsigned)(((warps < cap ? warps : cap) + kPairWarps - 1) / kPairWarps), kPairThreads, 0, stream, pd, i);
             *n_launches += 4;
         }
-        pair_wide_kernel<<<(unsigned)R->sms, kPairThreads, 0, stream>>>(pd, i);
+        chain(pair_wide_kernel, (unsigned)R->sms, kPairThreads, 0, stream, pd, i);
         *n_launches += 1;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -3120,17 +3188,17 @@ cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_ticket
     if (!R) return cudaErrorInvalidDevice;
     if (any_tickets) {
         if (pd.surv_sorted) {
-            surv_scan_kernel<<<1, 1024, 0, stream>>>(pd.surv_hist, pd.surv_off, pd.n_acc);
+            chain(surv_scan_kernel, 1, 1024, 0, stream, pd.surv_hist, pd.surv_off, pd.n_acc);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            surv_scatter_kernel<<<(L.surv_cap + 255) / 256, 256, 0, stream>>>(pd);
+            chain(surv_scatter_kernel, (L.surv_cap + 255) / 256, 256, 0, stream, pd);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *n_launches += 2;
         }
-        verify_kernel<<<R->verify, kVerifyThreads, sizeof(VerifyWarp) * kVerifyWarps, stream>>>(pd);
+        chain(verify_kernel, R->verify, kVerifyThreads, sizeof(VerifyWarp) * kVerifyWarps, stream, pd);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *n_launches += 1;
         if (L.empty_domain) {
-            count_kernel<<<(L.surv_cap + 255) / 256, 256, 0, stream>>>(pd);
+            chain(count_kernel, (L.surv_cap + 255) / 256, 256, 0, stream, pd);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *n_launches += 1;
         }

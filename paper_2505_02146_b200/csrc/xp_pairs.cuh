@@ -110,6 +110,7 @@ __device__ __forceinline__ u32 pair_limit(const HoleDev* hole) {
 
 // Chains of the indexed set (narrow entries), and the lists of wide entries of both sets.
 __global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     const PairSeg& seg = plan.psegs[index];
     const SketchDev* sk = plan.sketches[seg.sketch];
     const HoleDev* hole = &sk->holes[seg.hole];
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const __grid_c
 
 // + - *: one thread per operand x of the set that is not indexed.
 __global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -194,6 +196,7 @@ __device__ __forceinline__ u32 pair_bucket(u32 u) {
 constexpr int kPairBuckets = 1024;
 
 __global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     __shared__ u32 hist[kPairBuckets];
     const PairSeg& seg = plan.psegs[index];
     const int side = blockIdx.y;
@@ -212,6 +215,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const __g
 
 // One CTA per side: bucket starts (start[kPairBuckets] = entries), and the cursors of the scatter.
 __global__ void __launch_bounds__(kPairBuckets) pair_sort_scan_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     __shared__ u32 part[kPairBuckets];
     const PairSeg& seg = plan.psegs[index];
     const int side = blockIdx.x, t = threadIdx.x;
@@ -230,6 +234,7 @@ __global__ void __launch_bounds__(kPairBuckets) pair_sort_scan_kernel(const __gr
 }
 
 __global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     const PairSeg& seg = plan.psegs[index];
     const int side = blockIdx.y, lane = threadIdx.x & 31;
     const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
@@ -257,6 +262,7 @@ __device__ __forceinline__ u32 pair_to(const PairSeg& seg, u64 u) { return seg.s
 
 // A ticket: 32 dividends in magnitude order and one piece of the divisors that they may meet.
 __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -348,6 +354,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
 
 // Wide operands: each against the whole other set, lanes over it, from the first probe on, exactly.
 __global__ void __launch_bounds__(kPairThreads) pair_wide_kernel(const __grid_constant__ PlanDev plan, int index) {
+    chain_wait();
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
