@@ -1070,11 +1070,11 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         const LoadJob* d_jobs = (const LoadJob*)(dev_block + at_jobs);
         for (size_t q = 0; q < n; q += kJobs) {
             const int m = (int)(n - q < kJobs ? n - q : kJobs);
+            XP_CUDA_B(launch_stage(d_list + q, m, most_staged, nullptr));
             XP_CUDA_B(launch_coord_bounds(d_list + q, m, most_points, nullptr));
         }
         for (size_t q = 0; q < n_jobs; q += kJobs) {
             const int m = (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs);
-            XP_CUDA_B(launch_stage(d_jobs + q, m, most_staged, nullptr));
             // (what it decides per hole goes straight to page-locked memory: a few bytes, and no copy to queue behind the tables)
             LoadOut* out = (LoadOut*)(back.locked ? back.p : dev_block + at_out);
             XP_CUDA_B(launch_prepare(d_jobs + q, m, dev_block + at_scratch, out + q, nullptr));

@@ -1228,87 +1228,120 @@ __global__ void __launch_bounds__(256) scatter_kernel(const LoadCopy* copies, co
     for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < c.bytes / 16; i += (u64)gridDim.x * blockDim.x) to[i] = from[i];
 }
 
-// Value of a spec expression at kStageEach points (pt[variable][point]); false where it is undefined.  The instructions are
-// decoded once for all of them.
+// Value of a spec expression at the kStageEach points of a thread; false where it is undefined.  The instructions are
+// decoded once for all of them, the top of the stack stays in registers, and a leaf goes straight into the operator that
+// follows it: the stack proper (local memory, whose stores all go through to L2) is touched where a subtree waits for another.
 constexpr int kStageEach = 4;
-__device__ __forceinline__ bool eval_code_at(const xp_instr* __restrict__ code, int n, const i64 (*pt)[kStageEach], int n_pt, i64* out) {
+struct StagePoints { i64 lo[kMaxVars]; i32 digit[kMaxVars][kStageEach][256]; };      // coordinate = lo + digit
+__device__ __forceinline__ bool eval_code_at(const xp_instr* __restrict__ code, int n, const StagePoints& pts, int n_pt, i64 (&acc)[kStageEach]) {
     i64 st[kMaxStack][kStageEach];
     int sp = 0;
-    bool ok = true;
+    bool ok = true, have = false;
+#pragma unroll
+    for (int k = 0; k < kStageEach; ++k) acc[k] = 0;
     for (int i = 0; i < n; ++i) {
         const xp_instr c = code[i];
-        if (c.kind == XP_I_OP) {
-            --sp;
-            i64 *x = st[sp - 1], *y = st[sp];
-            if (c.arg <= XP_OP_MUL) {
+        i64 y[kStageEach];
+        int op = c.arg;
+        if (c.kind != XP_I_OP) {
 #pragma unroll
-                for (int k = 0; k < kStageEach; ++k) {
-                    const u64 u = (u64)x[k], v = (u64)y[k];
-                    x[k] = (i64)(c.arg == XP_OP_ADD ? u + v : c.arg == XP_OP_SUB ? u - v : u * v);
+            for (int k = 0; k < kStageEach; ++k) y[k] = c.kind == XP_I_VAR ? pts.lo[c.arg] + pts.digit[c.arg][k][threadIdx.x] : c.value;
+            if (!have || i + 1 >= n || code[i + 1].kind != XP_I_OP) {
+                if (!XP_CHECKED(sp < kMaxStack, kChkStack)) return false;
+                if (have) {
+#pragma unroll
+                    for (int k = 0; k < kStageEach; ++k) st[sp][k] = acc[k];
+                    ++sp;
                 }
-            } else {
-#pragma unroll 1
-                for (int k = 0; k < n_pt; ++k) {
-                    i64 r;
-                    if (apply_op(c.arg, x[k], y[k], r)) x[k] = r;
-                    else ok = false;
-                }
+#pragma unroll
+                for (int k = 0; k < kStageEach; ++k) acc[k] = y[k];
+                have = true;
+                continue;
+            }
+            op = code[++i].arg;
+        } else {
+            --sp;
+#pragma unroll
+            for (int k = 0; k < kStageEach; ++k) { y[k] = acc[k]; acc[k] = st[sp][k]; }
+        }
+        if (op <= XP_OP_MUL) {
+#pragma unroll
+            for (int k = 0; k < kStageEach; ++k) {
+                const u64 u = (u64)acc[k], v = (u64)y[k];
+                acc[k] = (i64)(op == XP_OP_ADD ? u + v : op == XP_OP_SUB ? u - v : u * v);
             }
         } else {
-            if (!XP_CHECKED(sp < kMaxStack, kChkStack)) return false;
 #pragma unroll
-            for (int k = 0; k < kStageEach; ++k) st[sp][k] = c.kind == XP_I_VAR ? pt[c.arg][k] : c.value;
-            ++sp;
+            for (int k = 0; k < kStageEach; ++k) {
+                i64 r = 0;
+                if (!apply_op(op, acc[k], y[k], r) && k < n_pt) ok = false;
+                acc[k] = r;
+            }
         }
     }
-#pragma unroll
-    for (int k = 0; k < kStageEach; ++k) out[k] = st[0][k];
     return ok;
 }
 
-// Staging of a load: for a box the coordinates of every point (int32 rows, like a table domain; written for the sketch's first
-// hole) and, per hole with a spec expression, the spec's value at every point.  spec_bad is set
-// if the spec is undefined somewhere (then no candidate can match).  One grid row per hole.
-// Bound by the interpreter's chain of local and constant loads, hence kStageEach points per thread (load of three holes of
-// 1.8 million points: 265 -> 239 us), and by the launches where domains are small, hence one kernel.
-__global__ void __launch_bounds__(256) stage_kernel(const LoadJob* jobs) {
+// Staging of a load: for a box the coordinates of every point (int32 rows, like a table domain) and, per hole with a spec
+// expression, the spec's value at every point.  spec_bad is set
+// if the spec is undefined somewhere (then no candidate can match).  One grid row per sketch, kStageEach points per thread:
+// a point's digits are taken once for all holes, by multiplication with reciprocals (what is staged has at most 2^26 points).
+// Bound by the interpreter, and by launches where domains are small, hence one kernel for both (three holes of 1.8 million
+// points: 120 us as two kernels with local stacks, now 61; 80 MB are written, which takes 12).
+static_assert(kStageMaxPoints <= 1ull << 31, "point numbers and extents of a staged box are 32-bit");
+__global__ void __launch_bounds__(256) stage_kernel(SketchDev* const* list) {
     chain_wait();
-    const LoadJob job = jobs[blockIdx.y];
-    const SketchDev* sk = job.s;
-    HoleDev* hole = &sk->holes[job.hole];
-    const bool rows = job.hole == 0 && sk->project, values = hole->spec_len != 0 && hole->spec_table != nullptr;
-    if (!rows && !values) return;
-    i64* spec = const_cast<i64*>(hole->spec_table);
+    __shared__ xp_instr s_code[kMaxCode];
+    __shared__ u32 s_ext[kMaxVars], s_inv[kMaxVars];
+    __shared__ StagePoints pts;
+    const SketchDev* sk = list[blockIdx.y];
+    const i64 n = sk->n_points;
+    const int nv = sk->n_vars, nh = sk->n_holes;
+    const bool rows = sk->project;
     i32* coords = const_cast<i32*>(sk->coords);
-    const int nv = sk->n_vars;
-    const bool box = sk->project || coords == nullptr;
-    const i64 n = sk->n_points, step = (i64)gridDim.x * 256 * kStageEach;
-    for (i64 at = (i64)blockIdx.x * 256 * kStageEach + threadIdx.x; at < n; at += step) {
-        i64 pt[kMaxVars][kStageEach];
+    const bool box = rows || coords == nullptr;
+    if (n > (i64)kStageMaxPoints) return;                 // (another sketch of the batch is staged, not this one)
+    if (threadIdx.x < nv) {
+        const u32 e = (u32)sk->ext[threadIdx.x];
+        s_ext[threadIdx.x] = e;
+        s_inv[threadIdx.x] = e <= 1u ? 0xffffffffu : (u32)((1ull << 32) / e);
+        pts.lo[threadIdx.x] = box ? sk->lo[threadIdx.x] : 0;
+    }
+    __syncthreads();
+    const i64 step = (i64)gridDim.x * 256 * kStageEach;
+    for (i64 first = (i64)blockIdx.x * 256 * kStageEach; first < n; first += step) {
+        const i64 at = first + threadIdx.x;               // (the loop is uniform in a block: threads past the end take its first point)
         int n_pt = 0;
 #pragma unroll
-        for (int k = 0; k < kStageEach; ++k) {
+        for (int k = 0; k < kStageEach; ++k) {            // (every thread reads back what it wrote itself)
             i64 pid = at + 256 * k;
             if (pid < n) n_pt = k + 1;
-            else pid = at;                                // (past the end: the first point again)
+            else pid = first;
             if (box) {
-                u64 rem = (u64)pid;
+                u32 rem = (u32)pid;
                 for (int d = nv - 1; d >= 0; --d) {
-                    u64 q, r;
-                    divmod_u64(rem, (u64)sk->ext[d], q, r);
-                    pt[d][k] = sk->lo[d] + (i64)r;
+                    const u32 e = s_ext[d];
+                    u32 q = __umulhi(rem, s_inv[d]), r = rem - q * e;      // (the estimate is the quotient or one less)
+                    if (r >= e) { ++q; r -= e; }
+                    pts.digit[d][k][threadIdx.x] = (i32)r;
+                    if (rows && n_pt > k) coords[pid * nv + d] = (i32)(pts.lo[d] + (i64)r);
                     rem = q;
                 }
             } else {
-                for (int d = 0; d < nv; ++d) pt[d][k] = coords[pid * nv + d];
+                for (int d = 0; d < nv; ++d) pts.digit[d][k][threadIdx.x] = coords[pid * nv + d];
             }
         }
-        if (rows)
-            for (int k = 0; k < n_pt; ++k)
-                for (int d = 0; d < nv; ++d) coords[(at + 256 * k) * nv + d] = (i32)pt[d][k];
-        if (values) {
+        for (int h = 0; h < nh; ++h) {
+            HoleDev* hole = &sk->holes[h];
+            const int len = hole->spec_len;
+            i64* spec = const_cast<i64*>(hole->spec_table);
+            if (len == 0 || spec == nullptr) continue;
+            __syncthreads();                              // (the code of the hole before is done with)
+            for (int i = threadIdx.x; i < len; i += 256) s_code[i] = hole->spec[i];
+            __syncthreads();
+            if (n_pt == 0) continue;
             i64 v[kStageEach];
-            if (!eval_code_at(hole->spec, hole->spec_len, pt, n_pt, v)) atomicOr(&hole->spec_bad, 1u);
+            if (!eval_code_at(s_code, len, pts, n_pt, v)) atomicOr(&hole->spec_bad, 1u);
 #pragma unroll
             for (int k = 0; k < kStageEach; ++k) if (k < n_pt) spec[at + 256 * k] = v[k];
         }
@@ -1345,15 +1378,20 @@ __global__ void __launch_bounds__(256) coord_bounds_kernel(SketchDev* const* lis
 // earlier launches.  The first launch makes sizes 1 and 3: the operands of size 3 are leaves, whose values come from the
 // probes themselves.  (One thread for several probes: the unranking, two 64-bit divisions, is done once for them.)
 // The first group also writes what does not depend on the probe, and the pair of values the leaf join reads.
+// `groups`: groups of probes per thread; all of them where the entries alone fill the chip (the unranking is then done once per
+// entry: 1024 holes of 6 160 entries at 16 probes: 970 -> 537 us, of which the 940 MB written take 140), one in small loads.
 constexpr int kSubProbes = 4;
-__global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int size, int last) {
+__global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int size, int last, int groups) {
     chain_wait();
     const SketchDev* sk = jobs[blockIdx.z].s;           // one grid layer per hole of the batch
     HoleDev* hole = &sk->holes[jobs[blockIdx.z].hole];
-    const int pr0 = blockIdx.y * kSubProbes;            // one grid row per group of probes
+    const int first = blockIdx.y * groups * kSubProbes;  // one grid row per `groups` groups of probes
     const GrammarDev* g = sk->g;
-    if (pr0 >= hole->tab_probes || size > hole->tab_max_size) return;      // (the grid is sized for the most there can be)
-    const int n_pr = hole->tab_probes - pr0 < kSubProbes ? hole->tab_probes - pr0 : kSubProbes;
+    const int n_probes = hole->tab_probes, p1 = hole->join_p1;
+    if (first >= n_probes || size > hole->tab_max_size) return;      // (the grid is sized for the most there can be)
+    __shared__ i64 s_pt[kMaxProbe][kMaxVars];
+    if (threadIdx.x < kMaxProbe * kMaxVars) s_pt[threadIdx.x / kMaxVars][threadIdx.x % kMaxVars] = hole->probe_pt[threadIdx.x / kMaxVars][threadIdx.x % kMaxVars];
+    __syncthreads();
     const u64 total = hole->tab_total;
     // (local copies: the stores below cannot change them, which the compiler cannot know of fields of *hole)
     i64* __restrict__ tab_val = hole->tab_val;
@@ -1365,11 +1403,10 @@ __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int 
         const u64 c = g->cnt[nt][size];
         if (idx >= c) { idx -= c; continue; }
         const u64 at = hole->tab_off[nt][size] + idx;
-        LeafDev lf{-1, 0, 0};
+        LeafDev lf{-1, 0, 0}, rf{-1, 0, 0};
         int op = 0;
         u64 la = 0, ra = 0;
         u32 vars = 0;
-        LeafDev rf{-1, 0, 0};
         if (size == 1) {
             lf = g->leaves[g->leaf_begin[nt] + (i32)idx];
             vars = lf.var >= 0 ? 1u << lf.var : 0u;
@@ -1382,33 +1419,37 @@ __global__ void __launch_bounds__(256) subvalue_kernel(const LoadJob* jobs, int 
                 vars = (lf.var >= 0 ? 1u << lf.var : 0u) | (rf.var >= 0 ? 1u << rf.var : 0u);
             } else {
                 la = hole->tab_off[lnt][a] + l; ra = hole->tab_off[rnt][size - 1 - a] + r;
-                if (pr0 == 0) vars = (u32)hole->tab_vars[la] | (u32)hole->tab_vars[ra];
+                if (first == 0) vars = (u32)hole->tab_vars[la] | (u32)hole->tab_vars[ra];
             }
         }
-        i64 v[kSubProbes];
-        bool ok[kSubProbes];
+#pragma unroll 1
+        for (int pr0 = first; pr0 < first + groups * kSubProbes && pr0 < n_probes; pr0 += kSubProbes) {
+            const int n_pr = n_probes - pr0 < kSubProbes ? n_probes - pr0 : kSubProbes;
+            i64 v[kSubProbes];
+            bool ok[kSubProbes];
 #pragma unroll
-        for (int k = 0; k < kSubProbes; ++k) {
-            v[k] = 0; ok[k] = true;
-            if (k >= n_pr) continue;
-            const u64 pbase = (u64)(pr0 + k) * total;
-            auto leaf = [&](const LeafDev& f) { return f.var >= 0 ? hole->probe_pt[pr0 + k][f.var] : f.value; };
-            if (size == 1) v[k] = leaf(lf);
-            else if (size == 3) ok[k] = apply_op(op, leaf(lf), leaf(rf), v[k]);
-            else ok[k] = tab_ok[pbase + la] && tab_ok[pbase + ra] && apply_op(op, tab_val[pbase + la], tab_val[pbase + ra], v[k]);
-        }
+            for (int k = 0; k < kSubProbes; ++k) {
+                v[k] = 0; ok[k] = true;
+                if (k >= n_pr) continue;
+                const u64 pbase = (u64)(pr0 + k) * total;
+                auto leaf = [&](const LeafDev& f) { return f.var >= 0 ? s_pt[pr0 + k][f.var] : f.value; };
+                if (size == 1) v[k] = leaf(lf);
+                else if (size == 3) ok[k] = apply_op(op, leaf(lf), leaf(rf), v[k]);
+                else ok[k] = tab_ok[pbase + la] && tab_ok[pbase + ra] && apply_op(op, tab_val[pbase + la], tab_val[pbase + ra], v[k]);
+            }
 #pragma unroll
-        for (int k = 0; k < kSubProbes; ++k)
-            if (k < n_pr) { tab_val[(u64)(pr0 + k) * total + at] = v[k]; tab_ok[(u64)(pr0 + k) * total + at] = ok[k] ? 1 : 0; }
-        if (pr0 == 0) {
-            hole->tab_vars[at] = (unsigned char)vars;
-            const i64 x = v[0], y = hole->join_p1 ? v[1] : v[0];
-            const bool defined = ok[0] && (!hole->join_p1 || ok[1]);
-            const bool narrow = x > -(1ll << 31) && x < (1ll << 31) && y > -(1ll << 31) && y < (1ll << 31);
-            int2 pair;
-            pair.x = defined && narrow ? (i32)x : kPairNone;
-            pair.y = defined ? (narrow ? (i32)y : 1) : 0;
-            reinterpret_cast<int2*>(hole->tab_pair)[at] = pair;
+            for (int k = 0; k < kSubProbes; ++k)
+                if (k < n_pr) { tab_val[(u64)(pr0 + k) * total + at] = v[k]; tab_ok[(u64)(pr0 + k) * total + at] = ok[k] ? 1 : 0; }
+            if (pr0 == 0) {
+                hole->tab_vars[at] = (unsigned char)vars;
+                const i64 x = v[0], y = p1 ? v[1] : v[0];
+                const bool defined = ok[0] && (!p1 || ok[1]);
+                const bool narrow = x > -(1ll << 31) && x < (1ll << 31) && y > -(1ll << 31) && y < (1ll << 31);
+                int2 pair;
+                pair.x = defined && narrow ? (i32)x : kPairNone;
+                pair.y = defined ? (narrow ? (i32)y : 1) : 0;
+                reinterpret_cast<int2*>(hole->tab_pair)[at] = pair;
+            }
         }
         return;
     }
@@ -3039,16 +3080,18 @@ cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src
     return cudaGetLastError();
 }
 
-cudaError_t launch_stage(const LoadJob* jobs, int n_jobs, i64 most_points, cudaStream_t stream) {
-    if (most_points <= 0 || n_jobs <= 0) return cudaSuccess;
+cudaError_t launch_stage(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream) {
+    if (most_points <= 0 || n_sketches <= 0) return cudaSuccess;
     const i64 blocks = (most_points + 256 * kStageEach - 1) / (256 * kStageEach);
-    chain(stage_kernel, dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_jobs), 256, 0, stream, jobs);
+    chain(stage_kernel, dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_sketches), 256, 0, stream, list);
     return cudaGetLastError();
 }
 
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last, int most_probes, u64 most_entries, cudaStream_t stream) {
     if (most_entries == 0 || most_probes <= 0 || n_jobs <= 0) return cudaSuccess;
-    chain(subvalue_kernel, dim3((unsigned)((most_entries + 255) / 256), (unsigned)((most_probes + kSubProbes - 1) / kSubProbes), (unsigned)n_jobs), 256, 0, stream, jobs, size, last);
+    const int all = (most_probes + kSubProbes - 1) / kSubProbes;
+    const int groups = (u64)n_jobs * most_entries >= 148ull * 2048 ? all : 1;
+    chain(subvalue_kernel, dim3((unsigned)((most_entries + 255) / 256), (unsigned)((all + groups - 1) / groups), (unsigned)n_jobs), 256, 0, stream, jobs, size, last, groups);
     return cudaGetLastError();
 }
 

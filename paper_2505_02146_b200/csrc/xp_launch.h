@@ -36,7 +36,7 @@ cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadO
 cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src, cudaStream_t stream);
 cudaError_t launch_reprobe(const LoadJob* jobs, int n_jobs, cudaStream_t stream);
 cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
-cudaError_t launch_stage(const LoadJob* jobs, int n_jobs, i64 most_points, cudaStream_t stream);
+cudaError_t launch_stage(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last, int most_probes, u64 most_entries, cudaStream_t stream);
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
