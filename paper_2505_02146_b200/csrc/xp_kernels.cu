@@ -2458,14 +2458,17 @@ __global__ void __launch_bounds__(256) surv_scatter_kernel(const __grid_constant
 // A program is a list of steps on an accumulator: "load", and operators whose other operand is a leaf (a variable or a
 // constant, on either side) or the value pushed last.  (i * 9) + j is three steps and touches no stack, where postfix
 // takes five with four stack accesses; with 8 points per lane instead of 4 the decoding of a step is shared by
-// twice as many points (1331 matches on 2^20 points: 18.5 -> 5.5 ms; 1024 small instances, 1.8e5 matches: 3.6 -> 2.7 ms).
+// twice as many points.  Bound by the instruction rate (1331 matches on 2^20 points: 18.5 -> 4.3 ms; 1024 small instances,
+// 1.8e5 matches: 3.6 -> 1.5 ms, where the divisions are exact multiplications and the constants never copied).
 // Two CTAs per SM: at three the 80 registers spill the step loop (small calls 48 us against 33, large ones the same).
 constexpr int kVArena = 192;                              // program steps a warp stages at once
 constexpr int kVStep = 256;                               // points per step
 constexpr int kVBatchVars = 4;                            // most variables a table may have for this form
 constexpr int kVBatchDepth = 2;                           // most values pushed at a time
 // One step: x = operator (XP_OP_*; +kFRev: leaf op accumulator) | source << 8 | push first << 16; y = variable, or the
-// constant's low word; z = its high word, or (division by a constant) floor(2^32 / |constant|).
+// constant's low word; z = its high word.  Division by a constant c of two and more in magnitude: z, w = multiplier and shift of the
+// exact quotient of a 31-bit dividend (Granlund and Montgomery, Division by Invariant Integers using Multiplication: with
+// l = ceil(log2 |c|), floor(x / |c|) = (x * ceil(2^(31 + l) / |c|)) >> (31 + l) for every x < 2^31).
 constexpr u32 kFLoad = 64, kFDivC = 65, kFModC = 66, kFRev = 32;
 enum { kFVar = 0, kFConst = 1, kFStack = 2 };
 // A warp's shared memory: the batch form's arrays and the one-survivor form's share the same bytes
@@ -2589,8 +2592,15 @@ __device__ __noinline__ int stage_compact(VerifyWarp& w, int off, const SketchDe
             const u32 op = q.x & 0xffu;
             if ((op != XP_OP_DIV && op != XP_OP_MOD) || ((q.x >> 8) & 3u) != (u32)kFConst || q.y == 0u) continue;
             const u32 ad = (i32)q.y < 0 ? 0u - q.y : q.y;
-            q.x = (q.x & ~0xffu) | (op == XP_OP_DIV ? kFDivC : kFModC);
-            q.z = ad == 1u ? 0xffffffffu : (u32)((1ull << 32) / ad);
+            if (ad == 1u) {                               // x / c = x * c, x % c = x * 0
+                q.x = (q.x & ~0xffu) | (u32)XP_OP_MUL;
+                if (op == XP_OP_MOD) q.y = 0u;
+            } else {
+                const int l = 32 - __clz((int)(ad - 1u));
+                q.x = (q.x & ~0xffu) | (op == XP_OP_DIV ? kFDivC : kFModC);
+                q.z = (u32)(((1ull << (31 + l)) + ad - 1u) / ad);
+                q.w = (u32)(l - 1);
+            }
             w.b.prog[off + k] = q;
         }
     return len;
@@ -2600,6 +2610,7 @@ __device__ __noinline__ int stage_compact(VerifyWarp& w, int off, const SketchDe
 __device__ __forceinline__ int staged_point(int h, int i) { return h * 128 + (int)(threadIdx.x & 31) * 4 + i; }
 
 // The staged program [off, off + len) on this lane's 8 points of the step, all values in int32.  bad: a zero divisor.
+// (The first step is always a load.  Sums and products with a constant have a form of their own: no copies of the constant.)
 __device__ __forceinline__ void run_narrow(VerifyBatch& b, int off, int len, i32 (&acc)[8], bool& bad) {
     const int lane = threadIdx.x & 31;
     int below = 0;
@@ -2607,31 +2618,57 @@ __device__ __forceinline__ void run_narrow(VerifyBatch& b, int off, int len, i32
     auto unpack = [](i32 (&v)[8], const uint4& p, const uint4& q) {
         v[0] = (i32)p.x; v[1] = (i32)p.y; v[2] = (i32)p.z; v[3] = (i32)p.w; v[4] = (i32)q.x; v[5] = (i32)q.y; v[6] = (i32)q.z; v[7] = (i32)q.w;
     };
+    auto fetch = [&](i32 (&v)[8], u32 var) {
+        const i32* c = b.coords[var] + lane * 4;
+        unpack(v, *reinterpret_cast<const uint4*>(c), *reinterpret_cast<const uint4*>(c + 128));
+    };
+    {
+        const uint4 in = b.prog[off];
+        if (((in.x >> 8) & 3u) == (u32)kFVar) fetch(acc, in.y);
+        else {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0;
-    for (int k = 0; k < len; ++k) {
+            for (int i = 0; i < 8; ++i) acc[i] = (i32)in.y;
+        }
+    }
+#pragma unroll 1
+    for (int k = 1; k < len; ++k) {
         const uint4 in = b.prog[off + k];
         const u32 src = (in.x >> 8) & 3u, op = in.x & 0xffu;
+        if (src == (u32)kFConst) {
+            const u32 c = in.y;
+#define XP_EACH(expr) { _Pragma("unroll") for (int i = 0; i < 8; ++i) { const u32 a = (u32)acc[i]; acc[i] = (i32)(expr); } continue; }
+            if (op == XP_OP_MUL || op == XP_OP_MUL + kFRev) XP_EACH(a * c)
+            if (op == XP_OP_ADD || op == XP_OP_ADD + kFRev) XP_EACH(a + c)
+            if (op == XP_OP_SUB) XP_EACH(a - c)
+            if (op == XP_OP_SUB + kFRev) XP_EACH(c - a)
+#undef XP_EACH
+            if (op >= kFDivC) {                           // x / c or x % c, |c| >= 2 a constant
+                const u32 M = in.z, sh = in.w, ad = (i32)c < 0 ? 0u - c : c;
+                if (op == kFDivC) {
+                    const i32 sc = (i32)c >> 31;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const i32 q = (i32)(__umulhi((u32)abs(acc[i]), M) >> sh), sg = (acc[i] >> 31) ^ sc;
+                        acc[i] = (q ^ sg) - sg;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const u32 x = (u32)abs(acc[i]);
+                        const i32 r = (i32)(x - (__umulhi(x, M) >> sh) * ad), sg = acc[i] >> 31;
+                        acc[i] = (r ^ sg) - sg;
+                    }
+                }
+                continue;
+            }
+        }
         if (in.x >> 16) {
             b.stack[below][0][lane] = make_uint4((u32)acc[0], (u32)acc[1], (u32)acc[2], (u32)acc[3]);
             b.stack[below][1][lane] = make_uint4((u32)acc[4], (u32)acc[5], (u32)acc[6], (u32)acc[7]);
             ++below;
         }
-        if (op >= kFDivC) {                               // x / c or x % c, c != 0 a constant
-            const u32 M = in.z, ad = (i32)in.y < 0 ? 0u - in.y : in.y;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const u32 ux = acc[i] < 0 ? 0u - (u32)acc[i] : (u32)acc[i];      // |x| < 2^31: the estimate is the quotient or one less
-                u32 q = __umulhi(ux, M), r = ux - q * ad;
-                if (r >= ad) { ++q; r -= ad; }
-                acc[i] = op == kFDivC ? (((acc[i] < 0) != ((i32)in.y < 0)) ? (i32)(0u - q) : (i32)q) : (acc[i] < 0 ? (i32)(0u - r) : (i32)r);
-            }
-            continue;
-        }
-        if (src == kFVar) {
-            const i32* c = b.coords[in.y];
-            unpack(y, *reinterpret_cast<const uint4*>(c + lane * 4), *reinterpret_cast<const uint4*>(c + 128 + lane * 4));
-        } else if (src == kFConst) {
+        if (src == (u32)kFVar) fetch(y, in.y);
+        else if (src == (u32)kFConst) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) y[i] = (i32)in.y;
         } else { --below; unpack(y, b.stack[below][0][lane], b.stack[below][1][lane]); }
@@ -2757,6 +2794,11 @@ __device__ __noinline__ void verify_batch(VerifyWarp& w, const SketchDev* sk, co
             if (narrow) {
                 i32 acc[8];
                 run_narrow(w.b, off, len, acc, bad);
+                // (points past the end repeat a real point, so they differ only where that one does)
+                u32 diff = off32 | (u32)bad;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) diff |= (u32)(acc[i] ^ want[i]);
+                if (!__any_sync(0xffffffffu, diff != 0u)) continue;
                 which = off32;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) which |= (u32)(acc[i] != want[i]) << i;
@@ -2871,19 +2913,16 @@ __global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const __grid_
     const u64 long_blocks = (n_long + width - 1) / width;
     u32 pieces = 1;
     while (pieces < (u32)(kVerifyChunk / kVStep) && n_blocks * walks * pieces < warps) pieces <<= 1;
+    // (full blocks: four items a warp even out the last wave; below 1024 points the staging would cost more than that)
+    while (pieces < (u32)(kVerifyChunk / 1024) && n_blocks * walks * pieces < 4 * warps) pieces <<= 1;
     const i64 sub = kVerifyChunk / pieces;                // points per item
     const u64 first_parts = plan.first_points >= kVerifyChunk ? pieces : (u64)((plan.first_points + sub - 1) / sub);
     const u64 first_items = n_blocks * first_parts;
     const u64 total = first_items + long_blocks * (u64)(plan.max_chunks > 0 ? plan.max_chunks - 1 : 0) * pieces;
-    const u64 kBatch = 2;                               // items a warp takes per atomic
-    u64 next = 0, batch_end = 0;
     for (;;) {
-        if (next == batch_end) {
-            if (lane == 0) next = atomicAdd(plan.verify_ticket, kBatch);
-            next = __shfl_sync(0xffffffffu, next, 0);
-            batch_end = next + kBatch;
-        }
-        const u64 t = next++;
+        u64 t = 0;
+        if (lane == 0) t = atomicAdd(plan.verify_ticket, 1ull);
+        t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= total) break;
         const bool later = t >= first_items;
         const i64 first = later ? kVerifyChunk + (i64)((t - first_items) / long_blocks) * sub : (i64)(t / n_blocks) * sub;
