@@ -567,8 +567,13 @@ static u64 table_entries(const xp_grammar* g, int max_size, u64 (*off)[kMaxSize 
 struct LoadState {
     xp_sketch* s = nullptr;
     const xp_sketch_desc* d = nullptr;
-    std::vector<HoleDev> hh;
-    std::vector<size_t> off_spec;            // per hole: its spec values in the device block (0: none there)
+    struct Hole {                            // what begin settles per hole; the record itself is made in its place in the staged copy
+        size_t off_spec = 0;                 // its spec values in the device block (0: none there)
+        size_t off_tabv = 0, off_tabk = 0, off_tabm = 0, off_pair = 0, off_sets = 0;
+        u64 entries = 0;
+        int probes = 0;
+    };
+    std::vector<Hole> hole;
     size_t off_coords = 0, head = 0;         // [0, head) of the block is staged on the host
     bool copy_coords = false, stage = false, stage_box = false;
     bool grammar_fresh = false;              // this sketch's load sends its grammar's tables
@@ -738,42 +743,38 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     size_t off = 0;
     const size_t off_sketch = off;  off += al256(sizeof(SketchDev));
     const size_t off_holes = off;   off += al256(sizeof(HoleDev) * nh);
-    L->off_spec.assign(nh, 0);
-    std::vector<size_t>& off_spec = L->off_spec;
-    std::vector<size_t> off_tabv(nh, 0), off_tabk(nh, 0), off_tabm(nh, 0), off_pair(nh, 0), off_sets(nh, 0);
+    L->hole.resize(nh);
     if (L->copy_coords && coords_bytes <= kPackMax) { L->off_coords = off; off += al256(coords_bytes); }
     for (int h = 0; h < nh; ++h)
         if (d->holes[h].spec_kind == XP_SPEC_TABLE && np > 0 && !d->holes[h].spec_table_on_device && spec_bytes <= kPackMax) {
-            off_spec[h] = off; off += al256(spec_bytes);
+            L->hole[h].off_spec = off; off += al256(spec_bytes);
         }
     s->off_kill.assign(nh, 0);
     for (int h = 0; h < nh; ++h) { s->off_kill[h] = off; off += al256((sizeof(i64) + sizeof(u32)) * kKillSlots); }
     L->head = off;                                        // [0, head): staged on the host
     if ((L->copy_coords && coords_bytes > kPackMax) || L->stage_box) { L->off_coords = off; off += al256(coords_bytes); }
-    std::vector<HoleDev>& hh = L->hh;
-    hh.resize(nh);
     for (int h = 0; h < nh; ++h) {
         const xp_hole_desc& hd = d->holes[h];
-        HoleDev& o = hh[h];
-        memset(&o, 0, sizeof(o));
-        if (np > 0 && off_spec[h] == 0 &&
+        LoadState::Hole& o = L->hole[h];
+        if (np > 0 && o.off_spec == 0 &&
             ((hd.spec_kind == XP_SPEC_TABLE && !hd.spec_table_on_device) || (hd.spec_kind == XP_SPEC_EXPR && L->stage))) {
-            off_spec[h] = off; off += al256(spec_bytes);
+            o.off_spec = off; off += al256(spec_bytes);
         }
-        const u64 entries = table_entries(g, hd.max_size, o.tab_off, &o.tab_size_cap);
+        int size_cap = 0;
+        const u64 entries = table_entries(g, hd.max_size, nullptr, &size_cap);
         u64 probes = kMaxProbe;
         while (probes > 1 && entries * 9 * probes > kTabBudgetBytes) --probes;
-        o.tab_total = entries;
-        o.tab_probes_cap = entries > 0 ? (i32)probes : 0;
+        o.entries = entries;
+        o.probes = entries > 0 ? (int)probes : 0;
         if (entries > 0) {
-            off_tabv[h] = off; off += al256(sizeof(i64) * entries * probes);
-            off_tabk[h] = off; off += al256(entries * probes);
-            off_tabm[h] = off; off += al256(entries);
-            off_pair[h] = off; off += al256(2 * sizeof(i32) * entries);
+            o.off_tabv = off; off += al256(sizeof(i64) * entries * probes);
+            o.off_tabk = off; off += al256(entries * probes);
+            o.off_tabm = off; off += al256(entries);
+            o.off_pair = off; off += al256(2 * sizeof(i32) * entries);
         }
-        off_sets[h] = off; off += al256(sizeof(JoinSet) * (size_t)g->n_nt);
-        if (o.tab_size_cap > s->tab_size_cap) s->tab_size_cap = o.tab_size_cap;
-        if (o.tab_probes_cap > s->tab_probes_cap) s->tab_probes_cap = o.tab_probes_cap;
+        o.off_sets = off; off += al256(sizeof(JoinSet) * (size_t)g->n_nt);
+        if (size_cap > s->tab_size_cap) s->tab_size_cap = size_cap;
+        if (o.probes > s->tab_probes_cap) s->tab_probes_cap = o.probes;
     }
     size_t arena_granted = 0;
     if (pool_alloc((void**)&s->arena, off, &s->arena_device, &arena_granted) != cudaSuccess) {
@@ -787,42 +788,50 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     s->d_s = (SketchDev*)(base + off_sketch);
     s->d_holes = (HoleDev*)(base + off_holes);
     s->off_holes = off_holes;
-    for (int h = 0; h < nh; ++h) {
-        const xp_hole_desc& hd = d->holes[h];
-        HoleDev& o = hh[h];
-        u64 c = 0;
-        for (int k = 1; k <= hd.max_size; ++k) c += g->cnt[hd.start_nt][k];
-        o.small_search = c <= 100000000ull ? 1 : 0;
-        o.start_nt = hd.start_nt; o.max_size = hd.max_size; o.ctx_len = hd.ctx_len;
-        if (hd.ctx_len) memcpy(o.ctx, hd.ctx, sizeof(xp_instr) * hd.ctx_len);
-        if (hd.spec_kind == XP_SPEC_EXPR) {
-            o.spec_len = hd.spec_len;
-            memcpy(o.spec, hd.spec_expr, sizeof(xp_instr) * hd.spec_len);
-            if (off_spec[h]) o.spec_table = (const i64*)(base + off_spec[h]);       // staged by the load, before anything reads it
-        } else if (np > 0) {
-            o.spec_table = hd.spec_table_on_device ? (const i64*)hd.spec_table : (const i64*)(base + off_spec[h]);
-        }
-        if (o.tab_total > 0) {
-            o.tab_val = (i64*)(base + off_tabv[h]);
-            o.tab_ok = (unsigned char*)(base + off_tabk[h]);
-            o.tab_vars = (unsigned char*)(base + off_tabm[h]);
-            o.tab_pair = (i32*)(base + off_pair[h]);
-        }
-        o.join_sets = (JoinSet*)(base + off_sets[h]);
-        // variables that decide beside the candidate's own (a caller's spec table may depend on all)
-        const u32 fv = hd.spec_kind != XP_SPEC_EXPR ? 0xffffffffu : constraint_vars(hd, nv, n_points);
-        o.fixed_vars = fv;
-        o.kill_pid = (i64*)(base + s->off_kill[h]);
-        o.kill_cnt = (u32*)(base + s->off_kill[h] + sizeof(i64) * kKillSlots);
-        HoleHost ho;
-        ho.start_nt = hd.start_nt; ho.max_size = hd.max_size;
-        s->holes.push_back(ho);
-    }
+    s->holes.resize(nh);
+    for (int h = 0; h < nh; ++h) { s->holes[h].start_nt = d->holes[h].start_nt; s->holes[h].max_size = d->holes[h].max_size; }
     for (int k = 1; k <= s->tab_size_cap; ++k)
         for (int nt = 0; nt < g->n_nt; ++nt) s->entries_at[k] += g->cnt[nt][k];
     L->s = s;
     L->d = d;
     return XP_OK;
+}
+
+// A hole's record.
+static void hole_image(const LoadState* L, int h, HoleDev* out) {
+    const xp_sketch* s = L->s;
+    const xp_grammar* g = s->g;
+    const xp_hole_desc& hd = L->d->holes[h];
+    const LoadState::Hole& at = L->hole[h];
+    char* base = s->arena;
+    HoleDev& o = *out;
+    memset(&o, 0, sizeof(o));
+    table_entries(g, hd.max_size, o.tab_off, &o.tab_size_cap);
+    o.tab_total = at.entries;
+    o.tab_probes_cap = at.probes;
+    u64 c = 0;
+    for (int k = 1; k <= hd.max_size; ++k) c += g->cnt[hd.start_nt][k];
+    o.small_search = c <= 100000000ull ? 1 : 0;
+    o.start_nt = hd.start_nt; o.max_size = hd.max_size; o.ctx_len = hd.ctx_len;
+    if (hd.ctx_len) memcpy(o.ctx, hd.ctx, sizeof(xp_instr) * hd.ctx_len);
+    if (hd.spec_kind == XP_SPEC_EXPR) {
+        o.spec_len = hd.spec_len;
+        memcpy(o.spec, hd.spec_expr, sizeof(xp_instr) * hd.spec_len);
+        if (at.off_spec) o.spec_table = (const i64*)(base + at.off_spec);       // staged by the load, before anything reads it
+    } else if (s->n_points > 0) {
+        o.spec_table = hd.spec_table_on_device ? (const i64*)hd.spec_table : (const i64*)(base + at.off_spec);
+    }
+    if (at.entries > 0) {
+        o.tab_val = (i64*)(base + at.off_tabv);
+        o.tab_ok = (unsigned char*)(base + at.off_tabk);
+        o.tab_vars = (unsigned char*)(base + at.off_tabm);
+        o.tab_pair = (i32*)(base + at.off_pair);
+    }
+    o.join_sets = (JoinSet*)(base + at.off_sets);
+    // variables that decide beside the candidate's own (a caller's spec table may depend on all)
+    o.fixed_vars = hd.spec_kind != XP_SPEC_EXPR ? 0xffffffffu : constraint_vars(hd, g->n_vars, s->n_points);
+    o.kill_pid = (i64*)(base + s->off_kill[h]);
+    o.kill_cnt = (u32*)(base + s->off_kill[h] + sizeof(i64) * kKillSlots);
 }
 
 // The sketch's record.
@@ -848,6 +857,14 @@ static void sketch_image(const LoadState* L, SketchDev* out) {
     // Sample points the probes are chosen from: box corners first (they expose bound and
     // padding mistakes), then ids spread over the domain by a fixed hash.
     int ns = 0;
+    unsigned char slot[4 * kProbeSamples] = {0};          // which ids are there: open addressing, number of the sample plus one
+    auto add = [&](i64 id) {
+        unsigned at = (unsigned)(mix64((u64)id) >> 32) % (4 * kProbeSamples);
+        for (; slot[at]; at = (at + 1) % (4 * kProbeSamples)) if (hs.sample_id[slot[at] - 1] == id) return;
+        hs.sample_id[ns++] = id;
+        slot[at] = (unsigned char)ns;
+    };
+    static_assert(kProbeSamples < 256, "a sample's number fits a byte");
     if (n_points > 0) {
         if (d->domain_kind == XP_DOMAIN_BOX) {
             const int ncorner = 1 << (nv < 5 ? nv : 5);
@@ -858,18 +875,13 @@ static void sketch_image(const LoadState* L, SketchDev* out) {
                     const i64 c = (v < 5 && ((m >> v) & 1)) ? ext - 1 : 0;
                     id = id * ext + c;
                 }
-                bool dup = false;
-                for (int k = 0; k < ns; ++k) dup = dup || hs.sample_id[k] == id;
-                if (!dup) hs.sample_id[ns++] = id;
+                add(id);
             }
         } else {
-            for (i64 id = 0; id < n_points && ns < 4; ++id) hs.sample_id[ns++] = id;
+            for (i64 id = 0; id < n_points && ns < 4; ++id) add(id);
         }
         for (u64 k = 0; ns < kProbeSamples && k < 4 * kProbeSamples; ++k) {
-            const i64 id = (i64)(mix64(k) % (u64)n_points);
-            bool dup = false;
-            for (int j = 0; j < ns; ++j) dup = dup || hs.sample_id[j] == id;
-            if (!dup) hs.sample_id[ns++] = id;
+            add((i64)(mix64(k) % (u64)n_points));
         }
     }
     hs.n_samples = ns;
@@ -883,12 +895,12 @@ static void load_fill(const LoadState* L, char* stg) {
     const size_t np = (size_t)s->n_points, row = (size_t)(s->g->n_vars ? s->g->n_vars : 1);
     const size_t coords_bytes = sizeof(i32) * np * row, spec_bytes = sizeof(i64) * np;
     sketch_image(L, (SketchDev*)stg);
-    memcpy(stg + s->off_holes, L->hh.data(), sizeof(HoleDev) * nh);
+    for (int h = 0; h < nh; ++h) hole_image(L, h, (HoleDev*)(stg + s->off_holes) + h);
     if (L->copy_coords && coords_bytes <= kPackMax) memcpy(stg + L->off_coords, d->coords, coords_bytes);
     for (int h = 0; h < nh; ++h) {
         const xp_hole_desc& hd = d->holes[h];
         if (hd.spec_kind == XP_SPEC_TABLE && np > 0 && !hd.spec_table_on_device && spec_bytes <= kPackMax)
-            memcpy(stg + L->off_spec[h], hd.spec_table, spec_bytes);
+            memcpy(stg + L->hole[h].off_spec, hd.spec_table, spec_bytes);
         memset(stg + s->off_kill[h], 0xff, sizeof(i64) * kKillSlots);           // no point noted yet (ids -1, counts 0)
         memset(stg + s->off_kill[h] + sizeof(i64) * kKillSlots, 0, sizeof(u32) * kKillSlots);
     }
@@ -993,7 +1005,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             }
             memcpy(lists + at_copies, copies.data(), sizeof(LoadCopy) * copies.size());
             // large batches fill their pieces with a few threads; whoever finishes a piece's last share sends the piece
-            size_t n_threads = n / 64;
+            size_t n_threads = staged / (1u << 20) < n / 8 ? staged / (1u << 20) : n / 8;      // (starting a thread takes as long as filling some 300 KB)
             const unsigned hw = std::thread::hardware_concurrency();
             if (n_threads > 8) n_threads = 8;
             if (hw > 0 && n_threads > hw) n_threads = hw;
@@ -1050,7 +1062,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             for (int h = 0; h < s->n_holes; ++h) {
                 const xp_hole_desc& hd = L.d->holes[h];
                 if (hd.spec_kind == XP_SPEC_TABLE && np > 0 && !hd.spec_table_on_device && spec_bytes > kPackMax) {
-                    XP_CUDA_B(cudaMemcpyAsync(s->arena + L.off_spec[h], hd.spec_table, spec_bytes, cudaMemcpyHostToDevice, nullptr));
+                    XP_CUDA_B(cudaMemcpyAsync(s->arena + L.hole[h].off_spec, hd.spec_table, spec_bytes, cudaMemcpyHostToDevice, nullptr));
                     s->load_h2d += spec_bytes;
                 }
                 if (hd.spec_kind == XP_SPEC_EXPR && L.stage && s->n_points > most_staged) most_staged = s->n_points;
