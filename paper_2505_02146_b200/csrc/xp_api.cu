@@ -226,7 +226,7 @@ struct xp_grammar {
 // is the number of size-s trees of its nonterminal that come before it.  Sizes from the first
 // one at which a count reaches 2^63 are marked unusable (ok_size).
 static void build_counts(xp_grammar* g) {
-    for (int s = 1; s <= kMaxSize; ++s) {
+    for (int s = 1; s <= kMaxSize; s += 2) {              // (every node has no or two children: no trees of even size)
         bool overflow = g->ok_size < s;
         for (int nt = 0; nt < g->n_nt && !overflow; ++nt) {
             unsigned __int128 total = 0;
@@ -238,8 +238,7 @@ static void build_counts(xp_grammar* g) {
                 if (b == g->bin_begin[nt] || bd.lnt != (&bd)[-1].lnt || bd.rnt != (&bd)[-1].rnt) {
                     block = 0;
                     const u64 *l = g->cnt[bd.lnt], *r = g->cnt[bd.rnt];
-                    for (int a = 1; a <= s - 2 && !overflow; ++a) {
-                        if (l[a] == 0 || r[s - 1 - a] == 0) continue;
+                    for (int a = 1; a <= s - 2 && !overflow; a += 2) {
                         block += (unsigned __int128)l[a] * r[s - 1 - a];
                         overflow = (block >> 63) != 0;
                     }
@@ -258,7 +257,10 @@ static void build_counts(xp_grammar* g) {
 
 static u32 reciprocal(i64 v) {       // (ConstDev::recip)
     const u64 m = v < 0 ? 0ull - (u64)v : (u64)v;
-    return m == 0 || m >> 31 ? 0u : m == 1 ? 0xffffffffu : (u32)((1ull << 32) / m);
+    if (m == 0 || m >> 31) return 0u;
+    if (m == 1) return 0xffffffffu;
+    const u32 d = (u32)m, q = 0xffffffffu / d;            // (2^32 - 1: one less where d divides 2^32)
+    return q + ((d & (d - 1)) == 0 ? 1u : 0u);
 }
 
 extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** out) {
@@ -272,9 +274,11 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
     if (!g) return fail(XP_ERR_NOMEM, "out of host memory");
     g->n_vars = d->n_vars;
     g->n_nt = d->n_nonterminals;
+    g->names.reserve(d->n_vars); g->lo.reserve(d->n_vars); g->hi.reserve(d->n_vars);
     for (int i = 0; i < d->n_vars; ++i) {
         if (d->vars[i].hi < d->vars[i].lo) { delete g; return fail(XP_ERR_GRAMMAR, "variable range with hi < lo"); }
-        g->names.push_back(d->vars[i].name ? d->vars[i].name : ("v" + std::to_string(i)));
+        if (d->vars[i].name) g->names.emplace_back(d->vars[i].name);
+        else g->names.push_back("v" + std::to_string(i));
         g->lo.push_back(d->vars[i].lo);
         g->hi.push_back(d->vars[i].hi);
     }
@@ -1128,7 +1132,9 @@ HoleSpec sketch_hole(const xp_sketch* s, int hole) {
     return HoleSpec{s->holes[hole].start_nt, s->holes[hole].max_size};
 }
 const HoleDev* sketch_hole_dev(const xp_sketch* s, int hole) { return s->d_holes + hole; }
-StageMemory::StageMemory(size_t bytes) : p(nullptr), block(new (std::nothrow) StageBlock(bytes)) { if (block) p = ((StageBlock*)block)->p; }
+StageMemory::StageMemory(size_t bytes) : p(nullptr), locked(false), block(new (std::nothrow) StageBlock(bytes)) {
+    if (block) { p = ((StageBlock*)block)->p; locked = ((StageBlock*)block)->locked; }
+}
 StageMemory::~StageMemory() { delete (StageBlock*)block; }
 StageEvents::StageEvents() : e0(nullptr), e1(nullptr), pair(new (std::nothrow) EventPair) {}
 StageEvents::~StageEvents() { delete (EventPair*)pair; }

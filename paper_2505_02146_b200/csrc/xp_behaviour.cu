@@ -10,10 +10,10 @@
 //                         64-bit word per class: 24 bits of the signature's hash, a kind bit, an id).  A word with the same
 //                         24 bits is confirmed by comparing the signatures themselves (another candidate's is computed
 //                         again).  A class that a representative already owns drops the candidate;
-//                         among the chunk's candidates the smallest index takes the word (compare-and-
-//                         swap that only ever lowers it: no thread waits for another);
-//   beh_flag_kernel    -- a candidate is new iff its class's word carries its own index; counts per block;
-//   beh_scan_kernel    -- exclusive scan of the block counts (one CTA);
+//                         among the chunk's candidates the smallest index takes the word (an atomic minimum:
+//                         no thread waits for another);
+//   beh_flag_kernel    -- a candidate is new iff its class's word carries its own index; counts per block, and their exclusive
+//                         scan by the block that finishes last;
 //   beh_append_kernel  -- the new ones, in candidate order, become representatives: signature and
 //                         record are appended, and the class's word now names the representative.
 // A table starts small and grows with the passes (beh_rehash_kernel puts the representatives into the larger one), so that a
@@ -63,6 +63,8 @@ struct BehDev {
     u64 table_size;                                       // a power of two: the most a nonterminal's table may have
     u64* buf_slot;                                        // per candidate of the chunk: slot of its class (kNoSlot: dropped)
     u32* block_count;                                     // per block of the chunk: new candidates, then their exclusive scan
+    u64* told;                                            // page-locked: chunk_new and err as the host reads them (null: by copy)
+    u32 blocks_done, pad1;                                // blocks of the flag kernel that have counted, zero between passes
     // results, read back from here on
     u64 chunk_new;                                        // new representatives of the chunk at hand
     u32 err, pad;                                         // err: a probe sequence ran its limit (table too full)
@@ -75,7 +77,10 @@ struct BehDev {
 constexpr u64 kNoSlot = ~0ull;
 constexpr u64 kBehTable = 1ull << 17;                     // slots a table starts with (1 MB: cleared in 2 us)
 
-struct BehBlock { u64 first, cr, lbase, rbase; i32 op, pad; };
+// mirror: the operator commutes and both operands are of one nonterminal, so that exchanging them gives a candidate of
+// the same behaviour -- 1: always an earlier one (the smaller operand on the left), 2: an earlier one where the left
+// operand's number is the larger, 0: none such.
+struct BehBlock { u64 first, cr, lbase, rbase; i32 op, mirror; };
 struct BehPass {
     i32 nt, size, n_blocks, leaf_first;                   // size 1: candidates are the leaves leaf_first ...
     u64 n_cand, mask;                                     // mask: the table's size at this pass, less one
@@ -110,10 +115,10 @@ __global__ void beh_points_kernel(BehDev* B) {
 }
 
 // Candidate idx of the pass: its operator and its operands (size 1: its leaf).
-struct BehOperands { i32 op; LeafDev leaf; u64 l, r; };
+struct BehOperands { i32 op, mirror; LeafDev leaf; u64 l, r; };
 __device__ __forceinline__ BehOperands beh_operands(const BehDev* B, const BehPass& P, u64 idx) {
     BehOperands o;
-    o.op = -1; o.l = o.r = 0;
+    o.op = -1; o.mirror = 0; o.l = o.r = 0;
     o.leaf = LeafDev{-1, 0, 0};
     if (P.size == 1) { o.leaf = B->sk->g->leaves[P.leaf_first + (i32)idx]; return o; }
     int b = 0;
@@ -121,7 +126,7 @@ __device__ __forceinline__ BehOperands beh_operands(const BehDev* B, const BehPa
     const BehBlock& k = P.blocks[b];
     u64 l, r;
     divmod_u64(idx - k.first, k.cr, l, r);
-    o.op = k.op; o.l = k.lbase + l; o.r = k.rbase + r;
+    o.op = k.op; o.mirror = k.mirror; o.l = k.lbase + l; o.r = k.rbase + r;
     return o;
 }
 
@@ -176,13 +181,18 @@ __device__ __forceinline__ bool beh_same(const BehDev* B, const BehPass& P, u64 
     return eq;
 }
 
-template <int NS>                                         // n_sig <= NS: the signature stays in registers
-__global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n) {
+// (n_sig <= NS: the signature stays in registers.)  Bound by the latency of the table and of the operands' signatures in L2: four
+// CTAs per SM cost 50 bytes of spills and are faster than three (1.07 million candidates of 12 points: 196 -> 183 us).  A
+// candidate whose mirror image comes earlier cannot be the first of its class and is not evaluated (183 -> 171 us), and a class is
+// compared once per slot however often its word is lowered meanwhile (171 -> 137 us).
+template <int NS>
+__global__ void __launch_bounds__(kBehThreads, 4) beh_insert_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n) {
     chain_wait();
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= chunk_n) return;
     const int ns = B->n_sig;
     const BehOperands o = beh_operands(B, P, chunk_first + c);
+    if (o.mirror == 1 || (o.mirror == 2 && o.l > o.r)) { B->buf_slot[c] = kNoSlot; return; }
     i64 mine[NS];
 #pragma unroll
     for (int j = 0; j < NS; ++j) mine[j] = 0;
@@ -198,30 +208,25 @@ __global__ void __launch_bounds__(kBehThreads) beh_insert_kernel(BehDev* B, cons
         bool done = false;
         for (u64 step = 0; step <= P.mask && !done; ++step, slot = (slot + 1) & P.mask) {
             u64 w = tab[slot];
-            bool other_class = false;
-            // A failed compare-and-swap means that another thread has just changed the word (claimed it,
-            // or lowered it within this class), never that one must be waited for; the limit only guards
-            // against a mistake in this routine.
-            for (int tries = 0; tries < (1 << 20); ++tries) {
-                if (w == kEmpty) {
-                    const u64 old = atomicCAS((unsigned long long*)&tab[slot], kEmpty, me);
-                    if (old == kEmpty) { place = slot; done = true; break; }
-                    w = old;
-                    continue;
-                }
-                if ((w >> 40) != (me >> 40) || !beh_same<NS>(B, P, w, mine, ns)) { other_class = true; break; }
-                if (!(w & kKindCand) || w <= me) { done = true; break; }      // a representative, or an earlier candidate, owns the class
-                const u64 old = atomicCAS((unsigned long long*)&tab[slot], w, me);
-                if (old == w) { place = slot; done = true; break; }
+            if (w == kEmpty) {
+                const u64 old = atomicCAS((unsigned long long*)&tab[slot], kEmpty, me);
+                if (old == kEmpty) { place = slot; done = true; break; }
                 w = old;
             }
-            if (!done && !other_class) break;             // (the limit ran out)
+            if ((w >> 40) != (me >> 40) || !beh_same<NS>(B, P, w, mine, ns)) continue;
+            // A slot's class never changes, so what the word has become meanwhile needs no second look: a representative's word
+            // and an earlier candidate's are smaller than this one and stay.
+            done = true;
+            if ((w & kKindCand) && w > me && atomicMin((unsigned long long*)&tab[slot], me) > me) place = slot;
         }
         if (!done) atomicOr(&B->err, 1u);
     }
     B->buf_slot[c] = place;
 }
 
+// Which candidates of the chunk own their class, counted per block; the block that finishes last scans the counts and
+// tells the host how many there are (a launch and a copy fewer per pass: with the append queued before the host looks,
+// 410 -> 388 us at four passes).
 __global__ void __launch_bounds__(kBehThreads) beh_flag_kernel(BehDev* B, int nt, u64 chunk_first, u32 chunk_n) {
     chain_wait();
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -234,7 +239,37 @@ __global__ void __launch_bounds__(kBehThreads) beh_flag_kernel(BehDev* B, int nt
         }
     }
     const int n = __syncthreads_count(is_new);
-    if (threadIdx.x == 0) B->block_count[blockIdx.x] = (u32)n;
+    __shared__ u32 part[kBehThreads];
+    __shared__ bool s_last;
+    const int t = threadIdx.x;
+    if (t == 0) {
+        B->block_count[blockIdx.x] = (u32)n;
+        __threadfence();
+        s_last = atomicAdd(&B->blocks_done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int n_blocks = (int)gridDim.x, per = (n_blocks + kBehThreads - 1) / kBehThreads;
+    const int lo = t * per < n_blocks ? t * per : n_blocks, hi = lo + per < n_blocks ? lo + per : n_blocks;
+    u32 sum = 0;
+    for (int i = lo; i < hi; ++i) sum += __ldcg(&B->block_count[i]);
+    part[t] = sum;
+    __syncthreads();
+    for (int d = 1; d < kBehThreads; d <<= 1) {
+        const u32 v = t >= d ? part[t - d] : 0u;
+        __syncthreads();
+        part[t] += v;
+        __syncthreads();
+    }
+    u32 run = part[t] - sum;
+    for (int i = lo; i < hi; ++i) { const u32 h = __ldcg(&B->block_count[i]); B->block_count[i] = run; run += h; }
+    if (t == 0) {
+        const u32 total = part[kBehThreads - 1];
+        B->chunk_new = total;
+        B->blocks_done = 0u;
+        if (B->told) { B->told[0] = total; B->told[1] = B->err; }
+    }
 }
 
 // A nonterminal's representatives, by size.
@@ -260,29 +295,9 @@ __global__ void __launch_bounds__(kBehThreads) beh_rehash_kernel(BehDev* B, int 
     atomicOr(&B->err, 1u);
 }
 
-__global__ void __launch_bounds__(1024) beh_scan_kernel(BehDev* B, int n_blocks) {
+__global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n, u64 rep_base, u64 max_reps) {
     chain_wait();
-    __shared__ u32 part[1024];
-    const int t = threadIdx.x;
-    const int per = (n_blocks + 1023) / 1024;
-    const int lo = t * per < n_blocks ? t * per : n_blocks, hi = lo + per < n_blocks ? lo + per : n_blocks;
-    u32 sum = 0;
-    for (int i = lo; i < hi; ++i) sum += B->block_count[i];
-    part[t] = sum;
-    __syncthreads();
-    for (int d = 1; d < 1024; d <<= 1) {
-        const u32 v = t >= d ? part[t - d] : 0u;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
-    }
-    u32 run = part[t] - sum;
-    for (int i = lo; i < hi; ++i) { const u32 h = B->block_count[i]; B->block_count[i] = run; run += h; }
-    if (t == 1023) B->chunk_new = part[1023];
-}
-
-__global__ void __launch_bounds__(kBehThreads) beh_append_kernel(BehDev* B, const __grid_constant__ BehPass P, u64 chunk_first, u32 chunk_n, u64 rep_base) {
-    chain_wait();
+    if (B->err || rep_base + B->chunk_new > max_reps) return;      // (the host has not looked yet: it will give up)
     __shared__ u32 warp_sum[kBehThreads / 32];
     const u32 c = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -432,7 +447,7 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
         return set_error(XP_ERR_NOMEM, ("xp_behaviours: device memory (" + std::to_string(off) + " bytes)").c_str());
     }
     StageMemory stage(2 * sizeof(BehDev));                // what goes out, and what comes back behind it
-    StageEvents ev;
+    StageEvents ev, counted;
     if (!stage.p) { device_release(block, granted, bdev); return set_error(XP_ERR_NOMEM, "out of host memory"); }
     BehDev& h = *(BehDev*)stage.p;
     BehDev& back = *(BehDev*)(stage.p + sizeof(BehDev));
@@ -446,7 +461,9 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
     cudaStream_t stream = opts ? (cudaStream_t)opts->stream : nullptr;
     constexpr size_t kBackAt = offsetof(BehDev, chunk_new);
     Cuda cu;
+    h.told = stage.locked ? &back.chunk_new : nullptr;
     cu(ev.open());
+    cu(counted.open());
     cu(cudaMemcpyAsync(dB, &h, sizeof(h), cudaMemcpyHostToDevice, stream));
     if (cu.ok()) cu(cudaEventRecord(ev.e0, stream));
     int launches = 0;
@@ -477,6 +494,8 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
                         if (P.n_blocks == kBehBlocks) { st = XP_ERR_TOO_LARGE; why = "xp_behaviours: more than 64 (production, left size) blocks in one pass"; break; }
                         BehBlock& k = P.blocks[P.n_blocks++];
                         k.first = P.n_cand; k.cr = cr; k.lbase = base[gh.bins[b].lnt][a]; k.rbase = base[gh.bins[b].rnt][s - 1 - a]; k.op = gh.bins[b].op;
+                        const bool commutes = k.op == XP_OP_ADD || k.op == XP_OP_MUL || k.op == XP_OP_MIN || k.op == XP_OP_MAX;
+                        k.mirror = !commutes || gh.bins[b].lnt != gh.bins[b].rnt || 2 * a < s - 1 ? 0 : 2 * a == s - 1 ? 2 : 1;
                         P.n_cand += cl * cr;
                         if (P.n_cand >= kKindCand) { st = XP_ERR_TOO_LARGE; why = "xp_behaviours: 2^39 candidates or more in one pass"; break; }
                     }
@@ -504,11 +523,12 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
                 if (ns <= 8) chain(beh_insert_kernel<8>, nb, kBehThreads, 0, stream, dB, P, first, n);
                 else chain(beh_insert_kernel<XP_MAX_SIG>, nb, kBehThreads, 0, stream, dB, P, first, n);
                 chain(beh_flag_kernel, nb, kBehThreads, 0, stream, dB, nt, first, n);
-                chain(beh_scan_kernel, 1, 1024, 0, stream, dB, nb);
+                if (!stage.locked) cu(cudaMemcpyAsync(&back.chunk_new, (char*)dB + kBackAt, 2 * sizeof(u64), cudaMemcpyDeviceToHost, stream));
+                cu(cudaEventRecord(counted.e0, stream));
+                chain(beh_append_kernel, nb, kBehThreads, 0, stream, dB, P, first, n, n_reps, max_reps);
                 launches += 3;
                 cu(cudaGetLastError());
-                cu(cudaMemcpyAsync(&back.chunk_new, (char*)dB + kBackAt, 2 * sizeof(u64), cudaMemcpyDeviceToHost, stream));
-                cu(cudaStreamSynchronize(stream));
+                cu(cudaEventSynchronize(counted.e0));     // (the append runs on while the host prepares the next pass)
                 if (!cu.ok()) break;
                 if (back.err) { st = XP_ERR_TOO_LARGE; why = "xp_behaviours: the hash table is too full (raise max_representatives)"; break; }
                 if (n_reps + back.chunk_new > max_reps) {
@@ -516,9 +536,6 @@ extern "C" xp_status xp_behaviours(const xp_sketch* sketch, const xp_behaviour_d
                     why = "xp_behaviours: more than " + std::to_string(max_reps) + " representatives (size " + std::to_string(s) + ")";
                     break;
                 }
-                chain(beh_append_kernel, nb, kBehThreads, 0, stream, dB, P, first, n, n_reps);
-                ++launches;
-                cu(cudaGetLastError());
                 n_reps += back.chunk_new;
                 held[nt] += back.chunk_new;
                 count[nt][s] += back.chunk_new;

@@ -87,6 +87,7 @@ struct StageMemory {
     StageMemory(size_t bytes);
     ~StageMemory();
     char* p;                         // null: out of host memory
+    bool locked;                     // page-locked: kernels may write to it
     void* block;
     StageMemory(const StageMemory&) = delete;
     StageMemory& operator=(const StageMemory&) = delete;
