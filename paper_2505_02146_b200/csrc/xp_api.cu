@@ -1856,9 +1856,10 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     }
     if (stopped == XP_OK) {
         XP_CUDA_R(launch_pairs(ws, w, plan.psegs.data(), stream, &launches));
-        XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets + plan.n_join + plan.psegs.size() > 0, stream, &launches));
+        bool told = false;
+        XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets + plan.n_join + plan.psegs.size() > 0, stage.locked ? (AccDev*)(stage.p + w.head) : nullptr, &told, stream, &launches));
         XP_CUDA_R(cudaEventRecord(ev.e1, stream));
-        XP_CUDA_R(cudaMemcpyAsync(stage.p + w.head, ws + w.acc, acc_bytes, cudaMemcpyDeviceToHost, stream));
+        if (!told) XP_CUDA_R(cudaMemcpyAsync(stage.p + w.head, ws + w.acc, acc_bytes, cudaMemcpyDeviceToHost, stream));
 #ifdef XP_CHECKS
         XP_CUDA_R(cudaMemcpyAsync(check_word, ws + 20, sizeof(*check_word), cudaMemcpyDeviceToHost, stream));
 #endif
@@ -1939,7 +1940,7 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
     stage_plan(stage.p, nullptr, w, plan, &sketch);
     const AccDev* acc = (const AccDev*)(stage.p + w.head);
     cudaStream_t stream = (cudaStream_t)o->stream;
-    cudaError_t e = launch_search_static(stage.p, w, plan.n_tickets, plan.n_join, (AccDev*)(stage.p + w.head), stream);
+    cudaError_t e = launch_search_static(stage.p, w, plan.n_tickets, plan.n_join, (AccDev*)(stage.p + w.head), stage.locked, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);         // (before the staging block goes back, whatever happened)
     if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) return fail(XP_ERR_CUDA, std::string("xp_repair_static: ") + cudaGetErrorString(e));

@@ -316,6 +316,8 @@ struct PlanDev {
     // listed after the search so that the later chunks are walked for them alone.
     u32* surv_long;                  // device, surv_cap
     u32* surv_long_n;                // device counter, zero at launch
+    u32* verify_done;                // device counter of finished CTAs of the verification kernel, zero at launch
+    AccDev* told;                    // page-locked: where the CTA that finishes last puts the accumulators (null: the host copies them)
 };
 
 }  // namespace xp

@@ -2993,6 +2993,19 @@ __global__ void __launch_bounds__(kVerifyThreads, 2) verify_kernel(const __grid_
             }
         }
     }
+    if (plan.told == nullptr) return;
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(plan.verify_done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const u64* from = reinterpret_cast<const u64*>(plan.acc);
+    u64* to = reinterpret_cast<u64*>(plan.told);
+    for (u32 i = threadIdx.x; i < (u32)plan.n_acc * (u32)(sizeof(AccDev) / 8); i += kVerifyThreads) to[i] = __ldcg(from + i);
 }
 
 // One thread per queued survivor of a sketch without points: there is no chunk to pass, it is a match.
@@ -3193,6 +3206,8 @@ static PlanDev plan_on(char* base, const SearchLayout& L) {
     pd.surv_sorted = order ? (u32*)(base + L.sorted) : nullptr;
     pd.surv_long = (u32*)(base + L.longs);
     pd.surv_long_n = (u32*)(base + 24);
+    pd.verify_done = (u32*)(base + 40);
+    pd.told = nullptr;
     return pd;
 }
 
@@ -3262,9 +3277,13 @@ cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_
     return cudaSuccess;
 }
 
-// Stage 3, after every part of the search has been queued.
-cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, cudaStream_t stream, int* n_launches) {
+// Stage 3, after every part of the search has been queued.  acc_out: page-locked memory for the accumulators (or null).  Where
+// there are few of them the verification kernel writes them there itself (*told): a copy of some hundred bytes takes the
+// stream as long as one of 20 KB, 4 to 5 us of a small call.
+cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, AccDev* acc_out, bool* told, cudaStream_t stream, int* n_launches) {
     PlanDev pd = plan_on(base, L);
+    *told = acc_out != nullptr && any_tickets && !L.empty_domain && L.n_acc <= 64;
+    if (*told) pd.told = acc_out;
     cudaError_t e;
     const Residency* R = residency();
     if (!R) return cudaErrorInvalidDevice;
@@ -3292,11 +3311,12 @@ cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_ticket
     return cudaGetLastError();
 }
 
-cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, u64 n_join, cudaStream_t stream, int* n_launches) {
+static cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, bool* told, cudaStream_t stream,
+                                 int* n_launches) {
     cudaError_t e = launch_search_part(base, L, true, 0, n_join, false, stream, n_launches);
     if (e == cudaSuccess) e = launch_search_part(base, L, false, 0, n_tickets, false, stream, n_launches);
     if (e != cudaSuccess) return e;
-    return launch_search_end(base, L, n_tickets + n_join > 0, stream, n_launches);
+    return launch_search_end(base, L, n_tickets + n_join > 0, acc_out, told, stream, n_launches);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -3314,7 +3334,7 @@ static void* g_static_scratch_addr[64];      // per device, filled on the first 
 // Copies the staged head of the plan (counters and accumulators in their start state, which
 // also wipes what the last call left) into the fixed array, runs the search on it, and queues
 // the copy of the accumulators back to `acc_out`.  Allocates nothing.
-cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, cudaStream_t stream) {
+cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, bool locked, cudaStream_t stream) {
     if (L.total > kStaticScratchBytes) return cudaErrorInvalidValue;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -3330,8 +3350,9 @@ cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n
     e = cudaMemcpyAsync(base, stage, L.head, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return e;
     int launches = 0;
-    e = launch_search(base, L, n_tickets, n_join, stream, &launches);
-    if (e != cudaSuccess) return e;
+    bool told = false;
+    e = launch_search(base, L, n_tickets, n_join, locked ? acc_out : nullptr, &told, stream, &launches);
+    if (e != cudaSuccess || told) return e;
     return cudaMemcpyAsync(acc_out, base + L.acc, sizeof(AccDev) * (size_t)L.n_acc, cudaMemcpyDeviceToHost, stream);
 }
 

@@ -40,7 +40,7 @@ cudaError_t launch_stage(SketchDev* const* list, int n_sketches, i64 most_points
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last, int most_probes, u64 most_entries, cudaStream_t stream);
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
-//      build only), 24: long survivors (u32), 32: join ticket (u64)   -- zero at launch
+//      build only), 24: long survivors (u32), 32: join ticket (u64), 40: finished verification CTAs (u32)   -- zero at launch
 //   segs, jsegs, jgroups, psegs, sketches, acc: staged from the host;  [0, head) is what the host copies in
 //   hist: survivors per accumulator slot, zero at launch (staged);
 //   surv: the survivor queue (surv_cap entries); sort_off, sorted: its hole order -- written by the kernels only
@@ -59,11 +59,10 @@ struct SearchLayout {
 cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64 t_begin, u64 t_end, bool restart, cudaStream_t stream,
                                int* n_launches);
 cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_segs, cudaStream_t stream, int* n_launches);
-cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, cudaStream_t stream, int* n_launches);
-cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_tickets, u64 n_join, cudaStream_t stream, int* n_launches);
+cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, AccDev* acc_out, bool* told, cudaStream_t stream, int* n_launches);
 int search_warps();                                  // warps of the leaf join that run at a time
 constexpr size_t kStaticScratchBytes = 1u << 20;     // fixed scratch of the allocation-free entry point
-cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, cudaStream_t stream);
+cudaError_t launch_search_static(const void* stage, const SearchLayout& L, u64 n_tickets, u64 n_join, AccDev* acc_out, bool locked, cudaStream_t stream);
 cudaError_t launch_int32_peak(int which, u32* out, int blocks, int iters, cudaStream_t stream);
 
 // What the library's other source files may know of a grammar and a loaded sketch (defined in xp_api.cu).
