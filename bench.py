@@ -37,24 +37,16 @@ WORKLOADS = {
 HEADLINE = "config4"
 DIVISION_COST = None
 
-# Counters of one eval_kernel launch per workload, from the ncu captures summarised under profiles/
-# (dram = dram__bytes_read.sum + dram__bytes_write.sum, thread_inst = smsp__thread_inst_executed.sum).
-# They describe the kernel sources whose hash is given; bench.py reports them (roofline.traffic,
-# roofline.frac_executed) only while the sources still have that hash.
-NCU_CAPTURE = {
-    "kernel_hash": "c59191fc30a2a131",
-    "date": "2026-12-01",
-    "config2": {"dram_bytes": 2.658e9, "thread_inst": 4.216e11},
-    "config4": {"dram_bytes": 6.484e9, "thread_inst": 8.183e11},
-    # (captured on 1024 of the 4096 instances and multiplied by 4: the instances are independent draws)
-    "config5": {"dram_bytes": 1.162e9, "thread_inst": 6.580e10},
-}
+# Counters of the search kernels per step and workload, from ncu captures (dram = dram__bytes_read.sum +
+# dram__bytes_write.sum, thread_inst = smsp__thread_inst_executed.sum).  They describe the kernel sources whose hash is
+# given; bench.py reports them (roofline.traffic, roofline.frac_executed) only while the sources still have that hash.
+NCU_CAPTURE = {"kernel_hash": None, "date": None}
 
 
 def kernel_hash() -> str:
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2505_02146_b200", "csrc")
-    for name in ("xp_dev.h", "xp_device.cuh", "xp_kernels.cu"):
+    for name in ("xp_dev.h", "xp_device.cuh", "xp_kernels.cu", "xp_join.cuh", "xp_pairs.cuh"):
         h.update(open(os.path.join(csrc, name), "rb").read())
     return h.hexdigest()[:16]
 
@@ -296,10 +288,10 @@ def roofline(m, steps, world, peak_add, peak_mad, name):
            "frac_cost_model": (m["model_ops"] / world) / kern_s / peak_add if m.get("model_ops") else None,
            "traffic": cap.get("dram_bytes") if fresh else None,
            "division_cost": DIVISION_COST,
-           "kernel": "eval_kernel",
+           "kernel": "join_kernel",
            "peak_source": "measured live: independent 32-bit add chains (xp_int32_peak); multiply-add chains reach %.0f" % (peak_mad / 1e9),
            "model": "frac: 2 x candidate-point evaluations that ran (one 32-bit operation + one comparison each) / kernel time / peak; "
-                    "frac_executed: thread instructions of eval_kernel per launch (ncu capture %s, kernel sources %s) / live kernel time / peak; "
+                    "frac_executed: thread instructions of the search kernels per step (ncu capture %s, kernel sources %s) / live kernel time / peak; "
                     "frac_cost_model: the library's nominal_ops (a straightforward 32-bit evaluator with a 7-operation reciprocal division)"
                     % (NCU_CAPTURE.get("date"), NCU_CAPTURE.get("kernel_hash"))}
     return out

@@ -2882,7 +2882,7 @@ __device__ __noinline__ void verify_one(const PlanDev& plan, VerifyWarp& w, u32 
 
 // Items are (chunk of points, block of up to 32 survivors), chunk-major: the first chunk of every
 // survivor (blocks in hole order) is taken before any second chunk, so candidates that fail early
-// cost one chunk; the later chunks exist for the long survivors only (surv_long_kernel), which keeps
+// cost one chunk; the later chunks exist for the long survivors only (listed as they are queued), which keeps
 // a call whose largest domain has hundreds of chunks from walking hundreds of empty items for every
 // survivor of a small (or projected) domain.  A call with few survivors cuts the chunks into pieces, down to 256 points,
 // until every warp has an item (three survivors of a 37 123-point table: 341 us as whole chunks).  Each WARP takes items on its own: nothing in this kernel synchronises a CTA, and no
