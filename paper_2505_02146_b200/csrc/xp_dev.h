@@ -222,6 +222,7 @@ struct JoinSeg {
 };
 
 // One (left operands, right operands) block of the pair join (csrc/xp_pairs.cuh): every  L op R  of its operators.
+constexpr u32 kPairWalk = 64;        // divisors that a warp of the division kernel meets in one go
 struct PairSeg {
     u64 rank_begin, rank_end;        // window of ranks searched at this size
     i32 sketch, hole, size, acc;
@@ -230,12 +231,13 @@ struct PairSeg {
     u32 ops;                         // operator slots (+ - * / %)
     i32 index_right;                 // the chains index the right operands (else the left ones)
     u64 base[5];                     // rank of (0, 0) per operator
-    u32 head_mask, pieces;           // pieces: parts that a warp's divisors are cut into
+    u32 head_mask, far_cap;          // far_cap: room in `far`
     // device scratch of the call
     u32* head;                       // head_mask + 1, all ones at launch
     u32* next;
-    u32* counters;                   // [2] wide operands left, right, then the ticket (u64): zero at launch
-    u64* ticket;
+    u32* counters;                   // [2] wide operands left, right, [2] entries of `far` (may run past far_cap); zero at launch
+    u64* ticket;                     // [2] of the division kernel's two launches, zero at launch
+    uint2* far;                      // (block of dividends | remainder << 31, first divisor): what a long walk left for the second launch
     u32 *wide_l, *wide_r;
     u32* hist[2];                    // 1024 each, zero at launch
     u32* start[2];                   // 1025 each

@@ -260,8 +260,23 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const _
 __device__ __forceinline__ u32 pair_from(const PairSeg& seg, u64 u) { return seg.start[1][u >> 31 ? kPairBuckets : pair_bucket((u32)u)]; }
 __device__ __forceinline__ u32 pair_to(const PairSeg& seg, u64 u) { return seg.start[1][u >> 31 ? kPairBuckets : pair_bucket((u32)u) + 1u]; }
 
-// A ticket: 32 dividends in magnitude order and one piece of the divisors that they may meet.
-__global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_constant__ PlanDev plan, int index) {
+// The sorted divisors [lo, hi) that the dividends with magnitudes amin .. amax (self: one of them is the target's) may meet.
+__device__ __forceinline__ void pair_span(const PairSeg& seg, int which, u64 m0, u32 amin, u32 amax, bool self, u32 nr, u32& lo, u32& hi) {
+    if (which == 0) {                                     // quotient
+        lo = pair_from(seg, (u64)amin / (m0 + 1) + 1);
+        hi = m0 ? pair_to(seg, (u64)amax / m0) : nr;
+    } else {                                              // remainder (at most its dividend)
+        lo = pair_from(seg, m0 + 1);
+        hi = amax < m0 ? lo : self ? nr : pair_to(seg, (u64)amax - m0);
+    }
+}
+
+// 32 dividends next to each other in magnitude order, and the divisors that they may meet.  Blocks differ by three
+// orders of magnitude in how many those are (a dividend that is the target itself leaves the remainder of every larger
+// divisor open), and one such walk by one warp was the kernel's whole time: a warp meets kPairWalk divisors at most and lists the
+// rest, which the second launch (phase 1) takes piece by piece (92 480 x 92 480 pairs: 780 -> 105 us; with walks of 512
+// divisors 730: where most of a walk agrees at both probes, every 32 divisors are 32 exact checks).
+__global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_constant__ PlanDev plan, int index, int phase) {
     chain_wait();
     __shared__ PairWarp sh[kPairWarps];
     PairWarp& w = sh[threadIdx.x >> 5];
@@ -278,35 +293,43 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
     const bool small = ((m0 | m1) >> 31) == 0 && !hole->join_none;      // (otherwise no narrow quotient or remainder is the target)
     const u32 u0t = (u32)m0, u1t = (u32)m1;
     const u32 nl = seg.start[0][kPairBuckets], nr = seg.start[1][kPairBuckets];
-    const u32 blocks = (nl + 31u) / 32u, pieces = seg.pieces;
-    const u64 tickets = small ? (u64)blocks * pieces : 0ull;
+    const u32 blocks = (nl + 31u) / 32u, n_far = seg.counters[2] < seg.far_cap ? seg.counters[2] : seg.far_cap;
+    const u64 tickets = !small ? 0ull : phase ? (u64)n_far : (u64)blocks;
     for (;;) {
         u64 t = 0;
-        if (lane == 0) t = atomicAdd((unsigned long long*)seg.ticket, 1ull);
+        if (lane == 0) t = atomicAdd((unsigned long long*)&seg.ticket[phase], 1ull);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= tickets) break;
-        const u32 block = blocks - 1u - (u32)(t / pieces), piece = (u32)(t % pieces);      // the largest dividends meet the most divisors: first
-        const u32 li = block * 32u + lane;
+        uint2 far = make_uint2(blocks - 1u - (u32)t, 0u);     // (the largest dividends meet the most divisors: first)
+        if (phase) far = seg.far[t];
+        const u32 li = (far.x & 0x7fffffffu) * 32u + lane;
         const bool live = li < nl;
         const int2 lv = live ? seg.val[0][li] : make_int2(0, 0);
         const u32 lid = live ? seg.id[0][li] : 0u;
         const u32 a0 = abs_u32(lv.x), a1 = abs_u32(lv.y);
         const u32 amin = __reduce_min_sync(0xffffffffu, live ? a0 : 0xffffffffu), amax = __reduce_max_sync(0xffffffffu, a0);
-        for (int which = 0; which < 2; ++which) {
+        const bool self = __any_sync(0xffffffffu, live && a0 == u0t);
+        const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
+        for (int which = phase ? (int)(far.x >> 31) : 0; which < (phase ? (int)(far.x >> 31) + 1 : 2); ++which) {
             if (!((seg.ops >> (which ? kSlotMod : kSlotDiv)) & 1u)) continue;
             u32 lo, hi;
-            if (which == 0) {                             // quotient
-                lo = pair_from(seg, (u64)amin / (m0 + 1) + 1);
-                hi = m0 ? pair_to(seg, (u64)amax / m0) : nr;
-            } else {                                      // remainder
-                if (amax < u0t) continue;                 // (a remainder is at most its dividend)
-                lo = pair_from(seg, m0 + 1);
-                const bool self = __any_sync(0xffffffffu, live && a0 == u0t);
-                hi = self ? nr : pair_to(seg, (u64)amax - m0);
-            }
+            pair_span(seg, which, m0, amin, amax, self, nr, lo, hi);
             if (lo >= hi) continue;
-            const u32 len = hi - lo, p0 = lo + (u32)((u64)len * piece / pieces), p1 = lo + (u32)((u64)len * (piece + 1) / pieces);
-            n.tests += (u64)(p1 - p0) * (u64)__popc(__ballot_sync(0xffffffffu, live));
+            u32 p0 = lo, p1 = hi;
+            if (phase) { p0 = far.y; p1 = hi - p0 < kPairWalk ? hi : p0 + kPairWalk; }
+            else if (hi - lo > kPairWalk) {               // the first piece here, the others listed (where the list is full: all that is left)
+                const u32 more = (hi - lo - 1u) / kPairWalk;
+                u32 at = 0;
+                if (lane == 0) at = atomicAdd(&seg.counters[2], more);
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (at <= seg.far_cap && more <= seg.far_cap - at) {
+                    for (u32 k = lane; k < more; k += 32u) seg.far[at + k] = make_uint2(far.x | ((u32)which << 31), lo + (k + 1u) * kPairWalk);
+                    p1 = lo + kPairWalk;
+                } else if (lane == 0 && at < seg.far_cap)
+                    for (u32 k = at; k < seg.far_cap; ++k) seg.far[k] = make_uint2(far.x | ((u32)which << 31), 0xffffffffu);      // (taken, nothing to do)
+            }
+            if (p0 >= p1) continue;
+            n.tests += (u64)(p1 - p0) * (u64)n_live;
             const u32 x0 = a0 >= u0t ? a0 - u0t : 1u;
             const bool can = live && (which == 0 || (a0 >= u0t && a1 >= u1t));
             for (u32 r0 = p0; r0 < p1; r0 += 32u) {
