@@ -546,7 +546,25 @@ __device__ __noinline__ void const_runs(const ConstDev* c, i32 lo, i32 hi, int s
                 else magnitudes(l, h);
             }
             return;
-        case kSlotMod: if (!swap) { magnitudes(tmod + 1, ~0ull); return; } run[0] = lo; run[1] = hi; return;
+        case kSlotMod:
+            // a % c: |c| exceeds every target and divides |a| - |t| at both probes, so it is a divisor of their greatest common
+            // one, and that one itself where its half is no longer above the targets.  c % a: |c| is |t| plus a multiple of
+            // |a|, so |t| itself where one |a| more is beyond every constant.  (With every constant
+            // above the target open: join of the large table 9.00 -> 8.91 ms, of the four-variable nest 1.96 -> 1.92.)
+            if (!swap) {
+                u64 g = u0 - v0, r = u1 - v1;
+                if (u0 < v0 || u1 < v1) return;
+                while (r) { const u64 q = (u32)g % (u32)r; g = r; r = q; }      // (both below 2^31)
+                magnitudes(g && g / 2 <= tmod ? g : tmod + 1, g ? g : ~0ull);
+                if (g && g <= tmod) { run[1] = run[0]; run[3] = run[2]; }
+                return;
+            }
+            {
+                const u64 big = u0 > u1 ? u0 : u1, at = u0 > u1 ? v0 : v1;
+                const u64 m0 = (u64)(c[lo].value < 0 ? -c[lo].value : c[lo].value), m1 = (u64)(c[hi - 1].value < 0 ? -c[hi - 1].value : c[hi - 1].value);
+                if (at + big > (m0 > m1 ? m0 : m1)) { if (at) magnitudes(at, at); else one(0); return; }
+            }
+            run[0] = lo; run[1] = hi; return;
         default: run[0] = lo; run[1] = hi; return;
     }
 }
