@@ -958,7 +958,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             return fail(e, "sketch " + std::to_string(i) + ": " + why);
         }
     }
-    // The staged copy: the job lists, then the sketches' shares, in pieces of at most kPieceBytes that page-locked memory
+    // The staged copy: the job lists, then the sketches' shares, in pieces of about kPieceBytes that page-locked memory
     // holds one by one.  The pieces go to one block of device memory, and a kernel puts the shares in their places:
     // a few large copies instead of two per sketch (a batch of 1024 sketches: 2048 copies, 10 ms of the copy engine's time).
     constexpr size_t kPieceBytes = 8ull << 20, kJobs = 32768;
@@ -975,7 +975,9 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     piece_at.push_back(0);
     for (size_t i = 0, c = n; i < n; ++i) {
         const size_t share = st[i].head + st[i].grammar_bytes;
-        if (at > piece_at.back() && at + share - piece_at.back() > kPieceBytes) piece_at.push_back(at);
+        // (a piece is closed only when it holds a sketch: whoever fills the last one sends it; the lists, and a share of any
+        // size, may make a piece larger than that)
+        if (i > 0 && at + share - piece_at.back() > kPieceBytes) piece_at.push_back(at);
         st[i].stage_at = at; st[i].piece = piece_at.size() - 1;
         copies[i].src = at;
         if (st[i].grammar_fresh) copies[c++].src = at + st[i].head;
@@ -992,7 +994,6 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         std::vector<std::atomic<size_t>> left(piece_at.size());
         std::vector<size_t> first(piece_at.size() + 1, n);       // sketches of a piece: [first[p], first[p + 1])
         for (size_t i = n; i-- > 0;) first[st[i].piece] = i;
-        for (size_t p = piece_at.size(); p-- > 0;) if (first[p] == n && p + 1 < first.size()) first[p] = first[p + 1];
         auto piece_end = [&](size_t p) { return p + 1 < piece_at.size() ? piece_at[p + 1] : staged; };
         bool ok = true;
         for (size_t p = 0; p < piece_at.size() && ok; ++p) {

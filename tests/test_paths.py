@@ -153,3 +153,24 @@ def test_descriptors_from_models(bad):
     hole = Hole(0, 3, spec_expr={"kind": [("x", 0, 0)], "pair": [(0, 0)], "value": [(0, 0, 2**70)], "attr": [7]}[bad])
     with pytest.raises((TypeError, ValueError, OverflowError)):
         B.marshal_sketches([Sketch(g, [hole])])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("holes,points", [(40, 32768), (1200, 0)])
+def test_a_first_share_larger_than_a_piece(xp, holes, points):
+    """One sketch whose share of the staged copy (host tables of 256 KB each, or a thousand hole records) is larger than a
+    piece: the lists in front of it travel with it."""
+    g = free_grammar(IJ, [1, 2])
+    specs = ["i+j", "i*2", "j-1", "2-i", "i/2", "j%2", "i"]
+    if points:
+        rng = np.random.default_rng(points)
+        coords = np.stack([rng.integers(0, 200, size=points), rng.integers(-30, 30, size=points)], axis=1).astype(np.int32)
+        i, j = coords[:, 0].astype(np.int64), coords[:, 1].astype(np.int64)
+        tables = [i + j, i * 2, j - 1, 2 - i, i // 2, np.fmod(j, 2), i]
+        sk = Sketch(g, [Hole(0, 3, spec_table=tables[h % 7]) for h in range(holes)], coords)
+    else:
+        sk = Sketch(g, [Hole(0, 3, spec_expr=parse_expr(specs[h % 7], IJ)) for h in range(holes)])
+    want = [oracle.repair_hole(sk, h) for h in range(7)]
+    got = xp.xp_repair(xp.xp_sketch_load(xp.xp_grammar_create(g), sk))
+    for h in range(holes):
+        assert_same(got[h], want[h % 7], f"hole {h}")
