@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -470,6 +471,17 @@ struct HoleHost {
     bool second = false;             // filter hits are looked at once more at probe 1 from the start (hits are frequent)
 };
 
+struct Plan {
+    std::vector<SegDev> segs;
+    std::vector<JoinSeg> jsegs;
+    std::vector<JoinGroup> jgroups;
+    std::vector<PairSeg> psegs;
+    std::vector<AccDev> acc;
+    std::vector<u64> nominal_ops;    // per accumulator: cost-model operations of the filter stage
+    u64 n_tickets = 0, n_join = 0;
+    bool join_wide = false;          // several operands per lane and step
+};
+
 struct xp_sketch {
     xp_grammar* g = nullptr;
     int n_holes = 0;
@@ -493,15 +505,10 @@ struct xp_sketch {
     // if it were the only sketch of the call: built on the first such call and copied, with ticket, sketch
     // and accumulator numbers shifted, into the plan of every later one (a batch of thousands of small
     // sketches would otherwise spend longer planning than some of its searches take).
+    // Two of them, with and without the pair join: each is built once, under the lock, and only read from then on
+    // (calls on several threads copy them at the same time); a refinement, during which no search may run, drops both.
     mutable std::mutex plan_mu;
-    mutable bool plan_cached = false;
-    mutable std::vector<SegDev> plan_segs;
-    mutable std::vector<JoinSeg> plan_jsegs;
-    mutable std::vector<JoinGroup> plan_jgroups;
-    mutable std::vector<PairSeg> plan_psegs;
-    mutable bool plan_pairs = false;                 // ... with the pair join allowed
-    mutable std::vector<u64> plan_ops;
-    mutable u64 plan_tickets = 0;
+    mutable std::unique_ptr<const Plan> plan_kept[2];
 };
 
 // What the load's kernels settled for a hole.
@@ -1232,7 +1239,7 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
             s->n_probes[h] = hh[h].n_probe;
         }
         std::lock_guard<std::mutex> lock(s->plan_mu);
-        s->plan_cached = false;                           // (the plan depends on which holes the filter serves)
+        for (auto& kept : s->plan_kept) kept.reset();     // (the plan depends on which holes the filter serves)
     } else {
         XP_CUDA(cudaStreamSynchronize(nullptr));
     }
@@ -1261,17 +1268,6 @@ struct xp_result {
     double kernel_ms = 0, total_ms = 0;
     int n_launches = 0;
     u64 h2d_bytes = 0, d2h_bytes = 0;
-};
-
-struct Plan {
-    std::vector<SegDev> segs;
-    std::vector<JoinSeg> jsegs;
-    std::vector<JoinGroup> jgroups;
-    std::vector<PairSeg> psegs;
-    std::vector<AccDev> acc;
-    std::vector<u64> nominal_ops;    // per accumulator: cost-model operations of the filter stage
-    u64 n_tickets = 0, n_join = 0;
-    bool join_wide = false;          // several operands per lane and step
 };
 
 // Scratch of calls that bring no workspace: one block per process, reused while no other call
@@ -1598,40 +1594,37 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
         const xp_sketch* s = sk[i];
         if (!s) return fail(XP_ERR_INVALID_ARG, "null sketch in batch");
         if (!plain) { plan_sketch(s, i, o, pairs, plan); continue; }
+        const Plan* own;
         {
             std::lock_guard<std::mutex> lock(s->plan_mu);
-            if (!s->plan_cached || s->plan_pairs != pairs) {
-                Plan own;
-                plan_sketch(s, 0, o, pairs, &own);
-                s->plan_segs = std::move(own.segs);
-                s->plan_jsegs = std::move(own.jsegs);
-                s->plan_jgroups = std::move(own.jgroups);
-                s->plan_psegs = std::move(own.psegs);
-                s->plan_pairs = pairs;
-                s->plan_ops = std::move(own.nominal_ops);
-                s->plan_tickets = own.n_tickets;
-                s->plan_cached = true;
+            std::unique_ptr<const Plan>& kept = s->plan_kept[pairs ? 1 : 0];
+            if (!kept) {
+                std::unique_ptr<Plan> made(new Plan);
+                plan_sketch(s, 0, o, pairs, made.get());
+                made->acc.clear();                        // (made per call, below)
+                kept = std::move(made);
             }
+            own = kept.get();
         }
         const int acc_base = (int)plan->acc.size();
         AccDev a;
         memset(&a, 0, sizeof(a));
         for (int k = 0; k <= kMaxSize; ++k) a.min_rank[k] = ~0ull;
-        for (int h = 0; h < s->n_holes; ++h) { plan->acc.push_back(a); plan->nominal_ops.push_back(s->plan_ops[h]); }
+        for (int h = 0; h < s->n_holes; ++h) { plan->acc.push_back(a); plan->nominal_ops.push_back(own->nominal_ops[h]); }
         const size_t at = plan->segs.size();
-        plan->segs.insert(plan->segs.end(), s->plan_segs.begin(), s->plan_segs.end());
+        plan->segs.insert(plan->segs.end(), own->segs.begin(), own->segs.end());
         for (size_t j = at; j < plan->segs.size(); ++j) {
             SegDev& c = plan->segs[j];
             c.first_ticket += plan->n_tickets;
             c.sketch = (i32)i;
             c.acc += acc_base;
         }
-        plan->n_tickets += s->plan_tickets;
+        plan->n_tickets += own->n_tickets;
         const size_t jat = plan->jsegs.size();
-        plan->jsegs.insert(plan->jsegs.end(), s->plan_jsegs.begin(), s->plan_jsegs.end());
-        for (const PairSeg& ps : s->plan_psegs) { plan->psegs.push_back(ps); plan->psegs.back().sketch = (i32)i; plan->psegs.back().acc += acc_base; }
+        plan->jsegs.insert(plan->jsegs.end(), own->jsegs.begin(), own->jsegs.end());
+        for (const PairSeg& ps : own->psegs) { plan->psegs.push_back(ps); plan->psegs.back().sketch = (i32)i; plan->psegs.back().acc += acc_base; }
         const i32 group_base = (i32)plan->jgroups.size();
-        plan->jgroups.insert(plan->jgroups.end(), s->plan_jgroups.begin(), s->plan_jgroups.end());
+        plan->jgroups.insert(plan->jgroups.end(), own->jgroups.begin(), own->jgroups.end());
         for (size_t j = jat; j < plan->jsegs.size(); ++j) {
             plan->jsegs[j].sketch = (i32)i; plan->jsegs[j].acc += acc_base; plan->jsegs[j].first_group += group_base;
         }

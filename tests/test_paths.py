@@ -1,6 +1,7 @@
 """The search's kernels at the sizes where each can go wrong, against the CPU oracle, bit for bit (whole numbers
 throughout: the tolerance is zero)."""
 import ctypes as C
+import threading
 
 import numpy as np
 import pytest
@@ -174,3 +175,31 @@ def test_a_first_share_larger_than_a_piece(xp, holes, points):
     got = xp.xp_repair(xp.xp_sketch_load(xp.xp_grammar_create(g), sk))
     for h in range(holes):
         assert_same(got[h], want[h % 7], f"hole {h}")
+
+
+@pytest.mark.gpu
+def test_one_sketch_under_both_plans_from_several_threads(xp):
+    """xp_repair may take blocks to the pair join, xp_repair_static and a batch of more than eight sketches may not: two plans of
+    one sketch, used in turn and at the same time."""
+    g = free_grammar(IJ, list(range(0, 12)) + [65536])
+    load = lambda spec: xp.xp_sketch_load(xp.xp_grammar_create(g), Sketch(g, [Hole(0, 7, spec_expr=parse_expr(spec, IJ))]))
+    ls, others = load("(i*3)+(j*2)"), [load("i+j") for _ in range(8)]
+    ref = xp.xp_repair(ls)[0]
+    key = lambda r, K=7: ([int(c) for c in r.match_count][:K + 1], r.least_size, int(r.least_rank))
+    calls = [lambda: key(xp.xp_repair(ls)[0]), lambda: key(xp.xp_repair_static(ls)[0]), lambda: key(xp.xp_repair_batch([ls] + others)[0][0])]
+    for _ in range(3):
+        for call in calls:
+            assert call() == key(ref)
+    bad = []
+
+    def work(call):
+        for _ in range(40):
+            r = call()
+            if r != key(ref):
+                bad.append(r)
+    threads = [threading.Thread(target=work, args=(c,)) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
