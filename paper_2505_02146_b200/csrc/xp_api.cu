@@ -1293,7 +1293,6 @@ static void add_linear(Plan* plan, int sketch, int hole, int acc, int k, u64 lo,
 
 constexpr size_t kPairMaxSketches = 8;
 constexpr u64 kPairLeast = 1ull << 20;       // pairs from which an index of one side costs less than a test per pair
-constexpr u64 kPairFar = 1ull << 18;         // most entries of the division kernel's second launch (2 MB)
 constexpr u64 kPairMost = 1ull << 22;        // operands of either side (the size of the subtree tables)
 
 // Does the pair join take the block (production, left size a) of size k?  Both operands tabulated, an operator it knows
@@ -1335,8 +1334,7 @@ static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
                 u32 heads = 1024;
                 while (heads < (c.index_right ? c.nr : c.nl)) heads <<= 1;
                 c.head_mask = heads - 1;
-                const u64 far = 2ull * ((c.nl + 31) / 32) * (c.nr / kPairWalk);      // (every block with every divisor)
-                c.far_cap = (u32)(far < kPairFar ? far : kPairFar);
+                c.far_pieces = pair_pieces(c.nl, c.nr);
                 plan->psegs.push_back(c);
                 sg = &plan->psegs.back();
             }
@@ -1682,7 +1680,7 @@ constexpr size_t kPairZeros = 256 + 2 * 4096;
 static size_t pair_rest_bytes(const PairSeg& c) {
     const size_t nl = c.nl, nr = c.nr;
     return align256(sizeof(u32) * (c.index_right ? nr : nl)) + align256(sizeof(u32) * nl) + align256(sizeof(u32) * nr) +
-           ((c.ops & 24u) ? align256(sizeof(uint2) * (size_t)c.far_cap) + 2 * align256(sizeof(u32) * 1025) + align256(12 * nl) + align256(12 * nr) + 512 : 0);
+           ((c.ops & 24u) ? align256(sizeof(uint2) * (size_t)pair_list_entries(c.nl, c.nr)) + 2 * align256(sizeof(u32) * 1025) + align256(12 * nl) + align256(12 * nr) + 512 : 0);
 }
 static void pair_place(PairSeg& c, char* ones, char* zeros, char* rest) {
     const size_t nl = c.nl, nr = c.nr;
@@ -1695,7 +1693,7 @@ static void pair_place(PairSeg& c, char* ones, char* zeros, char* rest) {
     c.wide_l = (u32*)take(sizeof(u32) * nl);
     c.wide_r = (u32*)take(sizeof(u32) * nr);
     if (c.ops & 24u) {
-        c.far = (uint2*)take(sizeof(uint2) * (size_t)c.far_cap);
+        c.far = (uint2*)take(sizeof(uint2) * (size_t)pair_list_entries(c.nl, c.nr));
         for (int k = 0; k < 2; ++k) {
             const size_t n = k ? nr : nl;
             c.start[k] = (u32*)take(sizeof(u32) * 1025);

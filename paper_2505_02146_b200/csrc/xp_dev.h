@@ -222,7 +222,28 @@ struct JoinSeg {
 };
 
 // One (left operands, right operands) block of the pair join (csrc/xp_pairs.cuh): every  L op R  of its operators.
-constexpr u32 kPairWalk = 64;        // divisors that a warp of the division kernel meets in one go
+//
+// The division kernel's walks: a block of 32 dividends may have any number of divisors to meet.  A walk is cut into pieces of
+// kPairWalk divisors, or longer ones where it would give more than `pieces` beside the first; the first is walked at once, the
+// others are listed for a second launch.  The list holds 2 * blocks * pieces entries, which is the most that all walks together
+// can list: no reservation runs past its end, whatever the operands are.
+#ifdef __CUDACC__
+#define XP_HD __host__ __device__
+#else
+#define XP_HD
+#endif
+constexpr u32 kPairWalk = 64;        // divisors that a warp of the division kernel meets in one go, at least
+constexpr u32 kPairList = 1u << 20;  // entries of the list that `pieces` aims at (8 MB)
+XP_HD inline u32 pair_blocks(u32 nl) { return (nl + 31u) / 32u; }
+XP_HD inline u32 pair_pieces(u32 nl, u32 nr) {
+    const u32 share = nl ? kPairList / (2u * pair_blocks(nl)) : 0u, most = share > 8u ? share : 8u, all = nr ? (nr - 1u) / kPairWalk : 0u;
+    return all < most ? all : most;
+}
+XP_HD inline u64 pair_list_entries(u32 nl, u32 nr) { return 2ull * pair_blocks(nl) * pair_pieces(nl, nr); }
+XP_HD inline u32 pair_piece(u32 span, u32 pieces) {      // divisors per piece of a walk over `span` of them, a multiple of 32
+    const u32 even = ((span + pieces) / (pieces + 1u) + 31u) & ~31u;
+    return even > kPairWalk ? even : kPairWalk;
+}
 struct PairSeg {
     u64 rank_begin, rank_end;        // window of ranks searched at this size
     i32 sketch, hole, size, acc;
@@ -231,13 +252,13 @@ struct PairSeg {
     u32 ops;                         // operator slots (+ - * / %)
     i32 index_right;                 // the chains index the right operands (else the left ones)
     u64 base[5];                     // rank of (0, 0) per operator
-    u32 head_mask, far_cap;          // far_cap: room in `far`
+    u32 head_mask, far_pieces;       // far_pieces: pieces that a walk lists at most (pair_pieces)
     // device scratch of the call
     u32* head;                       // head_mask + 1, all ones at launch
     u32* next;
-    u32* counters;                   // [2] wide operands left, right, [2] entries of `far` (may run past far_cap); zero at launch
+    u32* counters;                   // [2] wide operands left, right, [1] entries of `far`; zero at launch
     u64* ticket;                     // [2] of the division kernel's two launches, zero at launch
-    uint2* far;                      // (block of dividends | remainder << 31, first divisor): what a long walk left for the second launch
+    uint2* far;                      // (block of dividends | remainder << 31, first divisor): the pieces of long walks that the second launch takes
     u32 *wide_l, *wide_r;
     u32* hist[2];                    // 1024 each, zero at launch
     u32* start[2];                   // 1025 each

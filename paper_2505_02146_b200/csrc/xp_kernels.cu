@@ -3268,7 +3268,7 @@ cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_
             chain(pair_sort_scatter_kernel, dim3(ctas(most, 4), 2), kPairThreads, 0, stream, pd, i);
             const u64 warps = (u64)((s.nl + 31) / 32), cap = (u64)R->sms * 3 * kPairWarps;
             chain(pair_div_kernel, (unsigned)(((warps < cap ? warps : cap) + kPairWarps - 1) / kPairWarps), kPairThreads, 0, stream, pd, i, 0);
-            if (s.far_cap > 0) {
+            if (s.far_pieces > 0) {
                 chain(pair_div_kernel, (unsigned)R->sms * 3u, kPairThreads, 0, stream, pd, i, 1);
                 *n_launches += 1;
             }

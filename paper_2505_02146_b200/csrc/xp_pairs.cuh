@@ -273,9 +273,9 @@ __device__ __forceinline__ void pair_span(const PairSeg& seg, int which, u64 m0,
 
 // 32 dividends next to each other in magnitude order, and the divisors that they may meet.  Blocks differ by three
 // orders of magnitude in how many those are (a dividend that is the target itself leaves the remainder of every larger
-// divisor open), and one such walk by one warp was the kernel's whole time: a warp meets kPairWalk divisors at most and lists the
-// rest, which the second launch (phase 1) takes piece by piece (92 480 x 92 480 pairs: 780 -> 105 us; with walks of 512
-// divisors 730: where most of a walk agrees at both probes, every 32 divisors are 32 exact checks).
+// divisor open), and one such walk by one warp was the kernel's whole time: a warp meets one piece of kPairWalk divisors (or more,
+// see pair_pieces) and lists the others, which the second launch (phase 1) takes one by one (92 480 x 92 480 pairs: 780 ->
+// 105 us; with walks of 512 divisors 730: where most of a walk agrees at both probes, every 32 divisors are 32 exact checks).
 __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_constant__ PlanDev plan, int index, int phase) {
     chain_wait();
     __shared__ PairWarp sh[kPairWarps];
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
     const bool small = ((m0 | m1) >> 31) == 0 && !hole->join_none;      // (otherwise no narrow quotient or remainder is the target)
     const u32 u0t = (u32)m0, u1t = (u32)m1;
     const u32 nl = seg.start[0][kPairBuckets], nr = seg.start[1][kPairBuckets];
-    const u32 blocks = (nl + 31u) / 32u, n_far = seg.counters[2] < seg.far_cap ? seg.counters[2] : seg.far_cap;
+    const u32 blocks = (nl + 31u) / 32u, n_far = seg.counters[2];
     const u64 tickets = !small ? 0ull : phase ? (u64)n_far : (u64)blocks;
     for (;;) {
         u64 t = 0;
@@ -315,20 +315,18 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
             u32 lo, hi;
             pair_span(seg, which, m0, amin, amax, self, nr, lo, hi);
             if (lo >= hi) continue;
-            u32 p0 = lo, p1 = hi;
-            if (phase) { p0 = far.y; p1 = hi - p0 < kPairWalk ? hi : p0 + kPairWalk; }
-            else if (hi - lo > kPairWalk) {               // the first piece here, the others listed (where the list is full: all that is left)
-                const u32 more = (hi - lo - 1u) / kPairWalk;
+            const u32 piece = pair_piece(hi - lo, seg.far_pieces);
+            u32 p0 = lo;
+            if (phase) p0 = far.y;
+            else if (hi - lo > piece) {                   // the first piece here, the others listed
+                const u32 more = (hi - lo - 1u) / piece;
                 u32 at = 0;
                 if (lane == 0) at = atomicAdd(&seg.counters[2], more);
                 at = __shfl_sync(0xffffffffu, at, 0);
-                if (at <= seg.far_cap && more <= seg.far_cap - at) {
-                    for (u32 k = lane; k < more; k += 32u) seg.far[at + k] = make_uint2(far.x | ((u32)which << 31), lo + (k + 1u) * kPairWalk);
-                    p1 = lo + kPairWalk;
-                } else if (lane == 0 && at < seg.far_cap)
-                    for (u32 k = at; k < seg.far_cap; ++k) seg.far[k] = make_uint2(far.x | ((u32)which << 31), 0xffffffffu);      // (taken, nothing to do)
+                if (XP_CHECKED((u64)at + more <= pair_list_entries(seg.nl, seg.nr), kChkQueue))
+                    for (u32 k = lane; k < more; k += 32u) seg.far[at + k] = make_uint2(far.x | ((u32)which << 31), lo + (k + 1u) * piece);
             }
-            if (p0 >= p1) continue;
+            const u32 p1 = hi - p0 < piece ? hi : p0 + piece;
             n.tests += (u64)(p1 - p0) * (u64)n_live;
             const u32 x0 = a0 >= u0t ? a0 - u0t : 1u;
             const bool can = live && (which == 0 || (a0 >= u0t && a1 >= u1t));

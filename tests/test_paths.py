@@ -1,12 +1,15 @@
 """The search's kernels at the sizes where each can go wrong, against the CPU oracle, bit for bit (whole numbers
 throughout: the tolerance is zero)."""
 import ctypes as C
+import os
+import subprocess
 import threading
 
 import numpy as np
 import pytest
 
 import oracle
+from tests.conftest import ROOT
 from tests.util import assert_same, check_sketch
 from xp_instances import Hole, JointHole, Sketch, Variable, constant_set, free_grammar, parse_expr
 from tests.test_behaviours_gpu import _check as check_behaviours
@@ -203,3 +206,57 @@ def test_one_sketch_under_both_plans_from_several_threads(xp):
     for t in threads:
         t.join()
     assert not bad
+
+
+def test_the_list_of_long_walks_holds_every_piece(tmp_path):
+    """Division kernel of the pair join: all walks together never list more pieces than the list has room for (nor than 32
+    bits count), and the pieces of a walk cover it."""
+    src = tmp_path / "walks.cpp"
+    src.write_text(r"""
+#include <cstdio>
+#include "xp_dev.h"
+using namespace xp;
+int main() {
+    const u32 sizes[] = {1, 31, 32, 33, 63, 64, 65, 129, 1125, 9245, 92480, 3150592, 1u << 22};
+    for (u32 nl : sizes) for (u32 nr : sizes) {
+        const u32 pieces = pair_pieces(nl, nr);
+        const u64 room = pair_list_entries(nl, nr);
+        const u32 spans[] = {1, 2, 31, 32, 33, 63, 64, 65, 96, 97, nr / 3 + 1, nr / 2 + 1, nr - nr / 7, nr - 1, nr};
+        u64 most = 0;
+        for (u32 span : spans) {
+            if (span < 1 || span > nr) continue;
+            const u32 piece = pair_piece(span, pieces), more = span > piece ? (span - 1) / piece : 0;
+            if (piece < kPairWalk || piece % 32 || (u64)more * piece >= span || (u64)(more + 1) * piece < span) { printf("%u %u span %u piece %u\n", nl, nr, span, piece); return 1; }
+            if (more > most) most = more;
+        }
+        if (2ull * ((nl + 31) / 32) * most > room || room >> 31) { printf("%u %u: %llu in %llu\n", nl, nr, 2ull * ((nl + 31) / 32) * most, room); return 1; }
+    }
+    return 0;
+}
+""")
+    exe = tmp_path / "walks"
+    subprocess.check_call(["g++", "-std=c++17", "-I" + os.path.join(ROOT, "paper_2505_02146_b200", "csrc"), "-I" + os.path.join(ROOT, "include"),
+                           "-I/usr/local/cuda/include", str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)], capture_output=True, text=True).stdout == ""
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("spec", ["((k*13)+i)/60", "(i+(k*9))%37", "(i/50)+(k/7)"])
+def test_walks_of_small_targets(xp, spec):
+    """A small target at the first probe leaves most divisors open: walks of 92 480 divisors.  Against the operand tiles,
+    which a batch of more than eight sketches keeps to, and the oracle in windows."""
+    vs = [Variable("i", 0, 64), Variable("j", 0, 256), Variable("k", 0, 8)]
+    g = free_grammar(vs, constant_set(-64, 64, [128, 256, 512, 1024]))
+    sk = Sketch(g, [Hole(0, 7, spec_expr=parse_expr(spec, vs))], name=spec)
+    n = oracle.counts(g, 0, 7)
+    load = lambda s: xp.xp_sketch_load(xp.xp_grammar_create(s.grammar), s)
+    ls = load(sk)
+    small = free_grammar(IJ, [1])
+    others = [load(Sketch(small, [Hole(0, 3, spec_expr=parse_expr("i+j", IJ))])) for _ in range(8)]
+    at = 3 * n[7] // 5 + n[1] * n[5]                                     # the first quotient of two operands of three nodes
+    kw = dict(rank_ranges=[(0, 7, at, at + 300_000_000)], size_min=7)
+    a, b = xp.xp_repair(ls)[0], xp.xp_repair_batch([ls] + others)[0][0]
+    assert (a.match_count, a.least_size, a.least_rank) == (b.match_count, b.least_size, b.least_rank)
+    a, b = xp.xp_repair(ls, **kw)[0], xp.xp_repair_batch([ls] + others, **kw)[0][0]
+    assert (a.match_count, a.solved, a.least_rank) == (b.match_count, b.solved, b.least_rank)
+    check_sketch(xp, sk, windows={7: (at + 12_345_678, at + 13_345_678)})
