@@ -1584,8 +1584,9 @@ static xp_status check_device(const xp_sketch* const* sk, size_t n) {
 // (static_scratch: the call's scratch is the fixed array, which has no room for the pair join's index)
 static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, bool static_scratch, Plan* plan) {
     // the pair join takes its blocks one after the other, several launches each: a batch keeps to the tiles, which
-    // search all holes in one launch
-    const bool pairs = !static_scratch && n <= kPairMaxSketches;
+    // search all holes in one launch.  So does a call with a cancel word or a time limit: its launches are bounded, and the
+    // host looks at both between them; a pair join's launch covers a whole block.
+    const bool pairs = !static_scratch && n <= kPairMaxSketches && !o->cancel && o->timeout_ms <= 0;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {

@@ -4,6 +4,7 @@ import ctypes as C
 import os
 import subprocess
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -260,3 +261,24 @@ def test_walks_of_small_targets(xp, spec):
     a, b = xp.xp_repair(ls, **kw)[0], xp.xp_repair_batch([ls] + others, **kw)[0][0]
     assert (a.match_count, a.solved, a.least_rank) == (b.match_count, b.solved, b.least_rank)
     check_sketch(xp, sk, windows={7: (at + 12_345_678, at + 13_345_678)})
+
+
+@pytest.mark.gpu
+def test_cancel_word_and_time_limit_between_two_operands_of_three_nodes(xp):
+    """450 000 operands of three nodes a side: blocks that the pair join takes whole, unless a call wants to be stopped."""
+    vs = [Variable("i", 0, 64), Variable("j", 0, 256), Variable("k", 0, 8)]
+    g = free_grammar(vs, constant_set(-148, 148))
+    n = oracle.counts(g, 0, 7)
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), Sketch(g, [Hole(0, 7, spec_expr=parse_expr("((i*13)+j)+(k*5)", vs))]))
+    blocks = dict(rank_ranges=[(0, 7, n[7] // 5 + n[1] * n[5], n[7] // 5 + n[1] * n[5] + n[3] * n[3])], size_min=7)
+    with pytest.raises(xp.XpError) as e:
+        xp.xp_repair(ls, timeout_ms=3, **blocks)
+    assert e.value.status == 7
+    word = C.c_int32(0)
+    threading.Timer(0.005, lambda: setattr(word, "value", 1)).start()
+    t0 = time.perf_counter()
+    with pytest.raises(xp.XpError) as e:
+        xp.xp_repair(ls, cancel=word, **dict(blocks, rank_ranges=None))
+    assert e.value.status == 8 and "between launches" in str(e.value) and time.perf_counter() - t0 < 2.0
+    a, b = xp.xp_repair(ls, cancel=C.c_int32(0), timeout_ms=60_000, **blocks)[0], xp.xp_repair(ls, **blocks)[0]
+    assert (a.match_count, a.least_rank) == (b.match_count, b.least_rank) and a.n_launches > b.n_launches
