@@ -1467,7 +1467,7 @@ static JoinSeg new_join_seg(int sketch, int hole, int acc, int k, u64 lo, u64 hi
 // a group per leaf nonterminal, for every operator with a leaf of it on either side of such an operand.  Copies of one
 // production open segments of their own; so do shifts, which only the exact form knows.
 static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool exact, bool compares) {
-    struct Open { JoinSeg seg; std::vector<JoinGroup> groups; };
+    struct Open { JoinSeg seg; bool shifts; std::vector<JoinGroup> groups; };
     std::vector<Open> open;
     for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
         const BinDev& bd = g->bins[b];
@@ -1486,18 +1486,19 @@ static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
             if (!swap) { e0 = wlo / cr; e1 = (whi + cr - 1) / cr; }
             else if (wlo / cr == (whi - 1) / cr) { e0 = wlo % cr; e1 = (whi - 1) % cr + 1; }
             const int slot = slot_of_op(bd.op);
-            const bool ex = exact || slot >= 7;
+            const bool shifts = slot >= 7, ex = exact || shifts;      // (how many segments there are does not depend on `exact`)
             Open* at = nullptr;
             JoinGroup* grp = nullptr;
             for (size_t i = 0; i < open.size() && !at; ++i) {
                 Open& c = open[i];
-                if (c.seg.nt != ent || (c.seg.exact != 0) != ex) continue;
+                if (c.seg.nt != ent || c.shifts != shifts) continue;
                 grp = nullptr;
                 for (JoinGroup& q : c.groups) if (q.leaf_nt == lnt) grp = &q;
                 if (grp ? !(((swap ? grp->smask : grp->fmask) >> slot) & 1u) : c.groups.size() < (size_t)kJoinGroups) at = &c;
             }
             if (!at) {
                 Open c;
+                c.shifts = shifts;
                 c.seg = new_join_seg(sketch, hole, acc, k, lo, hi);
                 c.seg.kind = kJoinLeaf; c.seg.nt = ent; c.seg.esize = k - 2; c.seg.exact = ex ? 1 : 0; c.seg.heavy = ex || compares ? 1 : 0;
                 c.seg.e_begin = e0; c.seg.e_count = e1 - e0;
@@ -1581,12 +1582,12 @@ static xp_status check_device(const xp_sketch* const* sk, size_t n) {
     return XP_OK;
 }
 
-// (static_scratch: the call's scratch is the fixed array, which has no room for the pair join's index)
-static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, bool static_scratch, Plan* plan) {
+// (may_pair: the call's scratch has room for the pair join's index)
+static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, bool may_pair, Plan* plan) {
     // the pair join takes its blocks one after the other, several launches each: a batch keeps to the tiles, which
     // search all holes in one launch.  So does a call with a cancel word or a time limit: its launches are bounded, and the
     // host looks at both between them; a pair join's launch covers a whole block.
-    const bool pairs = !static_scratch && n <= kPairMaxSketches && !o->cancel && o->timeout_ms <= 0;
+    const bool pairs = may_pair && n <= kPairMaxSketches && !o->cancel && o->timeout_ms <= 0;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
@@ -1771,7 +1772,7 @@ static void stage_plan(char* stage, char* ws, const SearchLayout& w, Plan& plan,
 extern "C" size_t xp_workspace_bytes(const xp_sketch* const* sketches, size_t n, const xp_repair_opts* opts) {
     if (!sketches || n == 0) return 0;
     Plan plan;
-    if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, false, &plan) != XP_OK) return 0;
+    if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, true, &plan) != XP_OK) return 0;
     return ws_layout(plan, sketches, n, surv_cap_for(n)).total;
 }
 
@@ -1784,13 +1785,21 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     if (o->cancel && *o->cancel) return fail(XP_ERR_CANCELLED, "cancelled before launch");
     const auto t0 = std::chrono::steady_clock::now();
     Plan plan;
-    xp_status st = build_plan(sketches, n, o, false, &plan);
+    xp_status st = build_plan(sketches, n, o, true, &plan);
     if (st == XP_OK) st = check_device(sketches, n);
     if (st != XP_OK) return st;
     cudaStream_t stream = (cudaStream_t)o->stream;
 
-    const SearchLayout w = ws_layout(plan, sketches, n, surv_cap_for(n));
+    SearchLayout w = ws_layout(plan, sketches, n, surv_cap_for(n));
     char* ws = (char*)o->workspace;
+    if (ws && o->workspace_bytes < w.total && !plan.psegs.empty()) {
+        // A refinement can change which blocks the pair join may take (a target that is no longer zero), and so what a call
+        // needs: a caller's workspace made before it holds the plan without the pair join.
+        plan = Plan();
+        st = build_plan(sketches, n, o, false, &plan);
+        if (st != XP_OK) return st;
+        w = ws_layout(plan, sketches, n, surv_cap_for(n));
+    }
     bool own_ws = false, cached_ws = false;
     if (ws) {
         if (o->workspace_bytes < w.total || ((uintptr_t)ws & 255)) return fail(XP_ERR_NOMEM, "workspace too small or misaligned");
@@ -1920,7 +1929,7 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
     if (o->n_rank_ranges < 0 || (o->n_rank_ranges > 0 && !o->rank_ranges)) return fail(XP_ERR_INVALID_ARG, "bad rank_ranges");
     if (o->cancel && *o->cancel) return fail(XP_ERR_CANCELLED, "cancelled before launch");
     Plan plan;
-    xp_status st = build_plan(&sketch, 1, o, true, &plan);
+    xp_status st = build_plan(&sketch, 1, o, false, &plan);
     if (st == XP_OK) st = check_device(&sketch, 1);
     if (st != XP_OK) return st;
     const SearchLayout w = ws_layout(plan, &sketch, 1, kSurvCapStatic);

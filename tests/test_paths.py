@@ -282,3 +282,30 @@ def test_cancel_word_and_time_limit_between_two_operands_of_three_nodes(xp):
     assert e.value.status == 8 and "between launches" in str(e.value) and time.perf_counter() - t0 < 2.0
     a, b = xp.xp_repair(ls, cancel=C.c_int32(0), timeout_ms=60_000, **blocks)[0], xp.xp_repair(ls, **blocks)[0]
     assert (a.match_count, a.least_rank) == (b.match_count, b.least_rank) and a.n_launches > b.n_launches
+
+
+@pytest.mark.gpu
+def test_a_workspace_made_before_a_refinement(xp):
+    """Products of two operands of three nodes go to the pair join where no target is zero.  Here every sampled point but the
+    first wants 0; the points that end the survivors want 5 and become probes, and the search needs more scratch than before."""
+    import torch
+    vs = [Variable("a", 0, 9), Variable("b", 0, 9)]
+    g = free_grammar(vs, constant_set(1, 40), ops=["*"])
+    coords = np.zeros((6000, 2), dtype=np.int32)
+    coords[:, 1] = np.arange(6000) % 7
+    coords[0] = (2, 3)
+    spec = np.zeros(6000, dtype=np.int64)
+    spec[0] = 6
+    spec[100:106] = 5
+    sk = Sketch(g, [Hole(0, 7, spec_table=spec)], coords)
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
+    need = xp.xp_workspace_bytes([ls])
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    before = xp.xp_repair(ls, workspace=ws)[0]
+    assert before.probe_survivors > 0 and xp.xp_sketch_refine(ls) >= 1
+    assert xp.xp_workspace_bytes([ls]) > need                           # (or this test does not test what it says)
+    assert_same(xp.xp_repair(ls, workspace=ws)[0], before)
+    assert_same(xp.xp_repair(ls)[0], before)
+    with pytest.raises(xp.XpError) as e:                                # too small for any plan: refused as ever
+        xp.xp_repair(ls, workspace=ws[:need // 2])
+    assert e.value.status == 5
