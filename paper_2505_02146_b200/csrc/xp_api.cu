@@ -1525,14 +1525,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
         c.seg.first_group = (i32)plan->jgroups.size();
         c.seg.n_groups = (i32)c.groups.size();
         plan->jgroups.insert(plan->jgroups.end(), c.groups.begin(), c.groups.end());
-        JoinSeg sg = c.seg;
-        u64 left = sg.e_count;
-        const u64 most = 1ull << 31;                         // (a suspect's number inside its segment takes 32 bits)
-        while (left > 0) {
-            sg.e_count = left < most ? left : most;
-            plan->jsegs.push_back(sg);
-            sg.e_begin += sg.e_count; left -= sg.e_count;
-        }
+        plan->jsegs.push_back(c.seg);
     }
 }
 

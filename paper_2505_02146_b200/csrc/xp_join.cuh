@@ -70,7 +70,8 @@ struct JoinWarp {
     JoinHot hot;
     JoinCtx x;
     i32 seg;                                              // segment that grp, x and hot are filled for (-1: none)
-    u32 q_off[kJoinQueue];                                // suspects: operand number relative to the segment's first,
+    u64 base;                                             // operand that the queues' numbers count from
+    u32 q_off[kJoinQueue];                                // suspects: operand number relative to `base`,
     i32 q_a0[kJoinQueue], q_a1[kJoinQueue];               //   its values at the two probes
     u32 c_off[64], c_pos[64], c_code[64];                 // candidates: operand, leaf position, group << 8 | slot << 1 | swapped
     u32 nq, nc;                                           // suspects and candidates waiting (of segment `seg`)
@@ -258,7 +259,7 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
             const u32 code = w.c_code[at + lane], pos = w.c_pos[at + lane];
             const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u);
             const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code >> 8)];
-            const u64 e = seg.e_begin + w.c_off[at + lane];
+            const u64 e = w.base + w.c_off[at + lane];
             const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
             rank = grp.base[swap][slot] + (swap ? (u64)pos * ne + e : e * nl + (u64)pos);
             if (rank >= seg.rank_begin && rank < seg.rank_end &&
@@ -714,7 +715,7 @@ __device__ __noinline__ void join_exact(JoinWarp& w, const PlanDev& plan, const 
                     bool hit = pos < nl && apply_op(op, swap ? c0 : a0, swap ? a0 : c0, v) && probe_accepts(hole, 0, v);
                     if (two && hit) hit = apply_op(op, swap ? c1 : a1, swap ? a1 : c1, v) && probe_accepts(hole, 1, v);
                     n.suspects += (u32)__popc(__ballot_sync(0xffffffffu, hit));
-                    join_push(w, plan, seg, sk, hole, hit, (u32)(e - seg.e_begin), (u32)pos, gi, slot, swap, two ? 2 : 1, n);
+                    join_push(w, plan, seg, sk, hole, hit, (u32)(e - w.base), (u32)pos, gi, slot, swap, two ? 2 : 1, n);
                 }
         }
     }
@@ -992,7 +993,7 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     for (u64 done = 0; done < count;) {
         const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done);
         const u32 n_run = (u32)(c.left < count - done ? c.left : count - done);
-        const u32 off0 = (u32)(first + done - seg.e_begin) + lane;
+        const u32 off0 = (u32)(first + done - w.base) + lane;
         for (u32 at = 0; at < n_run; at += 32u * P) {
             i32 a0[P], a1[P];
             u32 alive, wide;
@@ -1235,7 +1236,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         for (u32 m = __ballot_sync(0xffffffffu, live && wide); m; m &= m - 1)
             join_exact(w, plan, seg, sk, hole, first + at + (u64)(__ffs((int)m) - 1), n);
         live = live && !wide;
-        const u32 off = (u32)(e - seg.e_begin);
+        const u32 off = (u32)(e - w.base);
         const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
         if (n_live == 0u) continue;
         auto accepted = [&](int slot, int swap, const i32 (&cv)[kRangeProbes]) {      // at the first nr probes
@@ -1420,22 +1421,24 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
             lo = nlo;
         }
         const JoinSeg& seg = plan.jsegs[lo];
-        if (w.seg >= 0 && w.seg != lo) join_leave(w, plan, w.seg, n);
+        const u64 chunk = seg.chunk, from = (t - seg.first_ticket) * chunk, first = seg.e_begin + from;
+        // (what waits in the queues is numbered in 32 bits, and a warp's tickets ascend)
+        if (w.seg >= 0 && (w.seg != lo || (first + chunk - w.base) >> 32)) join_leave(w, plan, w.seg, n);
         if (seg.acc != acc) { join_flush(plan, acc, n); acc = seg.acc; }
         const SketchDev* sk = plan.sketches[seg.sketch];
         const HoleDev* hole = &sk->holes[seg.hole];
-        if (seg.kind == kJoinLeaf && (hole->aff_ok || seg.exact) && w.seg != lo) {
-            join_fill(w, plan, seg, sk->g, hole);
-            if (lane == 0) w.seg = lo;
+        if (seg.kind == kJoinLeaf && w.seg != lo) {
+            const bool fill = hole->aff_ok || seg.exact;
+            if (fill) join_fill(w, plan, seg, sk->g, hole);
+            if (lane == 0) { w.base = first; if (fill) w.seg = lo; }
             __syncwarp();
         }
         const u32 all = hole->n_probe >= 32 ? 0xffffffffu : (1u << hole->n_probe) - 1u;
-        const u64 chunk = seg.chunk, from = (t - seg.first_ticket) * chunk;
         if ((hole->probe_spec_ok & all) == all && from < seg.e_count) {      // (a spec undefined at a probe: nothing can match)
             const u64 count = seg.e_count - from < chunk ? seg.e_count - from : chunk;
-            if (seg.kind == kJoinDirect) direct_ticket(w, plan, seg, sk, hole, seg.e_begin + from, count, n);
-            else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, seg.e_begin + from, count, n);
-            else join_ticket<P>(w, plan, seg, sk, hole, seg.e_begin + from, count, n);
+            if (seg.kind == kJoinDirect) direct_ticket(w, plan, seg, sk, hole, first, count, n);
+            else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, first, count, n);
+            else join_ticket<P>(w, plan, seg, sk, hole, first, count, n);
         }
         u64 next = 0;
         if (lane == 0) next = atomicAdd(plan.join_ticket, 1ull);

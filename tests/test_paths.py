@@ -309,3 +309,26 @@ def test_a_workspace_made_before_a_refinement(xp):
     with pytest.raises(xp.XpError) as e:                                # too small for any plan: refused as ever
         xp.xp_repair(ls, workspace=ws[:need // 2])
     assert e.value.status == 5
+
+
+@pytest.mark.gpu
+def test_more_operands_than_32_bits_count(xp):
+    """The plan of a search does not grow with the number of its operands (4e14 of size 9 here), and a warp that passes 2^32
+    operands of a segment loses none: 1.1e10 operands against the same in five windows."""
+    vs = [Variable("i", 0, 64), Variable("j", 0, 256), Variable("k", 0, 8)]
+    g = free_grammar(vs, constant_set(-64, 64, [128, 256, 512, 1024]))
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), Sketch(g, [Hole(0, 11, spec_expr=parse_expr("(i*13)+j", vs))]))
+    assert xp.xp_workspace_bytes([ls], size_min=11) < 4 << 20
+    with pytest.raises(xp.XpError) as e:
+        xp.xp_repair(ls, timeout_ms=20, size_min=11)
+    assert e.value.status == 7
+    g = free_grammar(vs, constant_set(-31, 30))
+    n = oracle.counts(g, 0, 9)
+    sk = Sketch(g, [Hole(0, 9, spec_expr=parse_expr("i+((j*7)%(i+3))", vs))])
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
+    run = lambda b, e: xp.xp_repair(ls, rank_ranges=[(0, 9, b, e)], size_min=9)[0]
+    cuts = [n[7] * k // 5 for k in range(6)]                            # i + (every operand of size 7)
+    parts = [run(b, e) for b, e in zip(cuts, cuts[1:])]
+    whole = run(0, n[7])
+    assert n[7] > 2 * 2**32 and whole.match_count[9] == sum(p.match_count[9] for p in parts) > 0
+    assert whole.least_rank == min(p.least_rank for p in parts if p.solved) > 2**32
