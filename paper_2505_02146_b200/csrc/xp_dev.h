@@ -224,23 +224,27 @@ struct JoinSeg {
 // One (left operands, right operands) block of the pair join (csrc/xp_pairs.cuh): every  L op R  of its operators.
 //
 // The division kernel's walks: a block of 32 dividends may have any number of divisors to meet.  A walk is cut into pieces of
-// kPairWalk divisors, or longer ones where it would give more than `pieces` beside the first; the first is walked at once, the
-// others are listed for a second launch.  The list holds 2 * blocks * pieces entries, which is the most that all walks together
-// can list: no reservation runs past its end, whatever the operands are.
+// kPairWalk divisors; the first is walked at once, the others are listed for a second launch.  They go to a list of kPairShort
+// entries while it has room, and otherwise, in longer pieces, at most `pieces` a walk, to a second list of
+// 2 * blocks * pieces entries, which is the most that all walks together can list: neither list is written past its end
+// and neither counter passes it, whatever the operands are.  (Short pieces as long as they fit: where most of a walk
+// agrees at both probes, every 32 divisors are 32 exact checks, and with pieces of 512 one such search took 60 ms longer.)
 #ifdef __CUDACC__
 #define XP_HD __host__ __device__
 #else
 #define XP_HD
 #endif
 constexpr u32 kPairWalk = 64;        // divisors that a warp of the division kernel meets in one go, at least
-constexpr u32 kPairList = 1u << 20;  // entries of the list that `pieces` aims at (8 MB)
+constexpr u32 kPairShort = 1u << 18; // entries of the list of short pieces (2 MB)
+constexpr u32 kPairLong = 1u << 20;  // entries of the list of long ones that `pieces` aims at (8 MB)
+XP_HD inline bool pair_fits(u32 taken, u32 more) { return taken <= kPairShort && more <= kPairShort - taken; }
 XP_HD inline u32 pair_blocks(u32 nl) { return (nl + 31u) / 32u; }
 XP_HD inline u32 pair_pieces(u32 nl, u32 nr) {
-    const u32 share = nl ? kPairList / (2u * pair_blocks(nl)) : 0u, most = share > 8u ? share : 8u, all = nr ? (nr - 1u) / kPairWalk : 0u;
+    const u32 share = nl ? kPairLong / (2u * pair_blocks(nl)) : 0u, most = share > 8u ? share : 8u, all = nr ? (nr - 1u) / kPairWalk : 0u;
     return all < most ? all : most;
 }
-XP_HD inline u64 pair_list_entries(u32 nl, u32 nr) { return 2ull * pair_blocks(nl) * pair_pieces(nl, nr); }
-XP_HD inline u32 pair_piece(u32 span, u32 pieces) {      // divisors per piece of a walk over `span` of them, a multiple of 32
+XP_HD inline u64 pair_list_entries(u32 nl, u32 nr) { return kPairShort + 2ull * pair_blocks(nl) * pair_pieces(nl, nr); }      // both lists
+XP_HD inline u32 pair_piece(u32 span, u32 pieces) {      // divisors per long piece of a walk over `span` of them, a multiple of 32
     const u32 even = ((span + pieces) / (pieces + 1u) + 31u) & ~31u;
     return even > kPairWalk ? even : kPairWalk;
 }
@@ -252,13 +256,14 @@ struct PairSeg {
     u32 ops;                         // operator slots (+ - * / %)
     i32 index_right;                 // the chains index the right operands (else the left ones)
     u64 base[5];                     // rank of (0, 0) per operator
-    u32 head_mask, far_pieces;       // far_pieces: pieces that a walk lists at most (pair_pieces)
+    u32 head_mask, far_pieces;       // far_pieces: long pieces that a walk lists at most (pair_pieces)
     // device scratch of the call
     u32* head;                       // head_mask + 1, all ones at launch
     u32* next;
-    u32* counters;                   // [2] wide operands left, right, [1] entries of `far`; zero at launch
+    u32* counters;                   // [2] wide operands left, right, [2] entries of the two lists; zero at launch
     u64* ticket;                     // [2] of the division kernel's two launches, zero at launch
-    uint2* far;                      // (block of dividends | remainder << 31, first divisor): the pieces of long walks that the second launch takes
+    uint2* far;                      // (block of dividends | long piece << 30 | remainder << 31, first divisor): what the second launch takes; the list of
+                                     // short pieces, then that of long ones
     u32 *wide_l, *wide_r;
     u32* hist[2];                    // 1024 each, zero at launch
     u32* start[2];                   // 1025 each

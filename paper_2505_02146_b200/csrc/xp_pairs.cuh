@@ -273,9 +273,9 @@ __device__ __forceinline__ void pair_span(const PairSeg& seg, int which, u64 m0,
 
 // 32 dividends next to each other in magnitude order, and the divisors that they may meet.  Blocks differ by three
 // orders of magnitude in how many those are (a dividend that is the target itself leaves the remainder of every larger
-// divisor open), and one such walk by one warp was the kernel's whole time: a warp meets one piece of kPairWalk divisors (or more,
-// see pair_pieces) and lists the others, which the second launch (phase 1) takes one by one (92 480 x 92 480 pairs: 780 ->
-// 105 us; with walks of 512 divisors 730: where most of a walk agrees at both probes, every 32 divisors are 32 exact checks).
+// divisor open), and one such walk by one warp was the kernel's whole time: a warp meets one piece of the walk and lists the
+// others (see pair_pieces), which the second launch (phase 1) takes one by one (92 480 x 92 480 pairs: 780 -> 105 us; with
+// walks of 512 divisors 730: where most of a walk agrees at both probes, every 32 divisors are 32 exact checks).
 __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_constant__ PlanDev plan, int index, int phase) {
     chain_wait();
     __shared__ PairWarp sh[kPairWarps];
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
     const bool small = ((m0 | m1) >> 31) == 0 && !hole->join_none;      // (otherwise no narrow quotient or remainder is the target)
     const u32 u0t = (u32)m0, u1t = (u32)m1;
     const u32 nl = seg.start[0][kPairBuckets], nr = seg.start[1][kPairBuckets];
-    const u32 blocks = (nl + 31u) / 32u, n_far = seg.counters[2];
+    const u32 blocks = (nl + 31u) / 32u, n_short = phase ? seg.counters[2] : 0u, n_far = phase ? n_short + seg.counters[3] : 0u;
     const u64 tickets = !small ? 0ull : phase ? (u64)n_far : (u64)blocks;
     for (;;) {
         u64 t = 0;
@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= tickets) break;
         uint2 far = make_uint2(blocks - 1u - (u32)t, 0u);     // (the largest dividends meet the most divisors: first)
-        if (phase) far = seg.far[t];
-        const u32 li = (far.x & 0x7fffffffu) * 32u + lane;
+        if (phase) far = seg.far[t < n_short ? t : kPairShort + (t - n_short)];
+        const u32 li = (far.x & 0x3fffffffu) * 32u + lane;
         const bool live = li < nl;
         const int2 lv = live ? seg.val[0][li] : make_int2(0, 0);
         const u32 lid = live ? seg.id[0][li] : 0u;
@@ -315,16 +315,30 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_div_kernel(const __grid_
             u32 lo, hi;
             pair_span(seg, which, m0, amin, amax, self, nr, lo, hi);
             if (lo >= hi) continue;
-            const u32 piece = pair_piece(hi - lo, seg.far_pieces);
-            u32 p0 = lo;
-            if (phase) p0 = far.y;
-            else if (hi - lo > piece) {                   // the first piece here, the others listed
-                const u32 more = (hi - lo - 1u) / piece;
-                u32 at = 0;
-                if (lane == 0) at = atomicAdd(&seg.counters[2], more);
+            u32 piece = kPairWalk, p0 = lo;
+            if (phase) {
+                p0 = far.y;
+                if ((far.x >> 30) & 1u) piece = pair_piece(hi - lo, seg.far_pieces);
+            } else if (hi - lo > piece) {                 // the first piece here, the others listed
+                u32 more = (hi - lo - 1u) / piece, at = 0, is_long = 0;
+                if (lane == 0) {
+                    at = *(volatile u32*)&seg.counters[2];
+                    for (;;) {                            // (a failed exchange means that another warp has listed its walk)
+                        is_long = pair_fits(at, more) ? 0u : 1u;
+                        const u32 seen = is_long ? at : atomicCAS(&seg.counters[2], at, at + more);
+                        if (seen == at) break;
+                        at = seen;
+                    }
+                }
+                is_long = __shfl_sync(0xffffffffu, is_long, 0);
+                if (is_long) {
+                    piece = pair_piece(hi - lo, seg.far_pieces);
+                    more = (hi - lo - 1u) / piece;
+                    if (lane == 0) at = kPairShort + atomicAdd(&seg.counters[3], more);
+                }
                 at = __shfl_sync(0xffffffffu, at, 0);
                 if (XP_CHECKED((u64)at + more <= pair_list_entries(seg.nl, seg.nr), kChkQueue))
-                    for (u32 k = lane; k < more; k += 32u) seg.far[at + k] = make_uint2(far.x | ((u32)which << 31), lo + (k + 1u) * piece);
+                    for (u32 k = lane; k < more; k += 32u) seg.far[at + k] = make_uint2(far.x | (is_long << 30) | ((u32)which << 31), lo + (k + 1u) * piece);
             }
             const u32 p1 = hi - p0 < piece ? hi : p0 + piece;
             n.tests += (u64)(p1 - p0) * (u64)n_live;

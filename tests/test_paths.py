@@ -230,7 +230,8 @@ int main() {
             if (piece < kPairWalk || piece % 32 || (u64)more * piece >= span || (u64)(more + 1) * piece < span) { printf("%u %u span %u piece %u\n", nl, nr, span, piece); return 1; }
             if (more > most) most = more;
         }
-        if (2ull * ((nl + 31) / 32) * most > room || room >> 31) { printf("%u %u: %llu in %llu\n", nl, nr, 2ull * ((nl + 31) / 32) * most, room); return 1; }
+        if (!pair_fits(0, kPairShort) || !pair_fits(kPairShort, 0) || pair_fits(kPairShort, 1) || pair_fits(5, kPairShort - 4) || pair_fits(~0u, 7)) return 2;
+        if (kPairShort + 2ull * ((nl + 31) / 32) * most > room || room >> 31) { printf("%u %u: %llu in %llu\n", nl, nr, 2ull * ((nl + 31) / 32) * most, room); return 1; }
     }
     return 0;
 }
@@ -238,7 +239,8 @@ int main() {
     exe = tmp_path / "walks"
     subprocess.check_call(["g++", "-std=c++17", "-I" + os.path.join(ROOT, "paper_2505_02146_b200", "csrc"), "-I" + os.path.join(ROOT, "include"),
                            "-I/usr/local/cuda/include", str(src), "-o", str(exe)])
-    assert subprocess.run([str(exe)], capture_output=True, text=True).stdout == ""
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert (r.returncode, r.stdout) == (0, "")
 
 
 @pytest.mark.gpu
