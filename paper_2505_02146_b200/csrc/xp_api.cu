@@ -463,8 +463,8 @@ struct HoleHost {
     int start_nt = 0, max_size = 0;
     bool filter_ok = false;          // the probe filter applies (probe 0 exists, context affine or a comparison there, subtree tables)
     bool never = false;              // the spec is undefined at some point: no candidate can match
-    bool exact = false;              // the leaf join's conditions do not apply (a context factor of 2^31 or more, or 0)
-    bool join_on = false;            // the context is affine with a factor of 31 bits
+    bool exact = false;              // the leaf join's conditions do not apply (a context factor of 0, or with more than 31 zero bits at its end)
+    bool join_on = false;            // the context is affine, and they do
     bool target_zero = false;        // the hole value wanted is zero at one of the join's two probes
     int tab_max = 0;                 // subtrees up to this size are tabulated
     bool compares = false;           // the filter works on an interval of hole values (the context compares)

@@ -143,9 +143,11 @@ struct HoleDev {
     u32 fixed_vars, spec_bad;                     // spec_bad: set by the load when the spec is undefined at some point
     // The leaf join: values (a0, a1) at its two probes of every tabulated subtree, 8 bytes each (same index as
     // tab_val; a0 = kPairNone: undefined at one of them (a1 = 0) or not below 2^31 in magnitude (a1 = 1)); the leaf sets
-    // of the nonterminals; the targets.  join_on: the context is affine at both probes with a factor that 32 bits hold.
+    // of the nonterminals; the targets.  join_on: the context is affine at both probes with a factor that has
+    // at most 31 zero bits at its end.
     i32 join_on, join_p1;                         // second probe (0 when there is only one that serves)
     i32 join_none, n_exact;                       // no value below the operand limit can be the target; probes checked from the tables
+    i32 join_shift, pad5;                         // zero bits at the end of the context's factor (the larger of the two probes')
     i64 join_t0, join_t1;                         // hole values that satisfy the constraint at the two probes
     u64 join_tmod;                                // largest |target| over the probes: a remainder's divisor must exceed it
     float join_rt0, join_rt1, join_rl0, join_rl1; // 1 / |target| (0 for 0), 1 / (|target| + 1)

@@ -121,25 +121,37 @@ __device__ bool ctx_interval(const HoleDev* hole, const i64* pt, i64 spec, i64& 
     return false;
 }
 
-// The join's targets of a hole: the hole values that satisfy the constraint at the two probes, exact in
-// 64 bits for values below the operand limits of the leaf sets (the context's factor times such a value cannot wrap).
+// The join's targets of a hole: the values h that satisfy A h + B = spec at the two probes.  In wrap-around arithmetic that is
+// A h = d modulo 2^64, with A = odd * 2^z: d has to end in z zeros, and then h = (d / 2^z) / odd modulo 2^(64-z), one value
+// among those below 2^(63-z) in magnitude.  The operand limits of the leaf sets keep every result there (join_shift: the larger z of
+// the two probes), so any factor but 0 will do, and large odd ones cost nothing.
 // Called by threads 0 .. 15 together, one per probe; np: probes with tables; ok: bit per probe with spec and affine context.
-__device__ __forceinline__ void join_targets(HoleDev* hole, int j, int np, u32 ok, u64 A64, u64 B64) {
+constexpr int kJoinShift = 31;       // largest z (the conditions compare 32 bits of a value that is known modulo 2^(64-z))
+__device__ __forceinline__ void join_targets(HoleDev* hole, int j, int np, u32 ok, u64 A, u64 B) {
     constexpr u32 kLanes = 0x0000ffffu;
-    const bool mine = j < np && ((ok >> j) & 1u);
-    const int p1 = np >= 2 && ((ok >> 1) & 1u) ? 1 : 0;
-    const i64 A = (i64)A64, d = mine ? (i64)((u64)hole->probe_spec[j] - B64) : 0;
-    const bool bad = mine && (A == 0 || A <= -(1ll << 31) || A >= (1ll << 31));
-    i64 v = d;
+    const int z = A ? __ffsll((i64)A) - 1 : 64;
+    const bool mine = j < np && ((ok >> j) & 1u) && z <= kJoinShift;
+    const u32 good = __ballot_sync(kLanes, mine);
+    const int p1 = (good >> 1) & 1u ? 1 : 0;
+    const u64 d = mine ? (u64)hole->probe_spec[j] - B : 0ull;
+    i64 v = 0;
     bool miss = false;
-    if (mine && !bad && A != 1) { miss = d <= -(1ll << 62) || d >= (1ll << 62) || d % A != 0; v = miss ? 0 : d / A; }
+    if (mine) {
+        const u64 odd = A >> z;
+        u64 inv = odd;                                    // (three bits; each of Newton's steps doubles them)
+        for (int k = 0; k < 5; ++k) inv *= 2ull - odd * inv;
+        miss = (d & ((1ull << z) - 1ull)) != 0;
+        if (!miss) v = (i64)(((d >> z) * inv) << z) >> z;
+    }
     u64 m = !mine ? 0ull : miss ? ~0ull : v < 0 ? 0ull - (u64)v : (u64)v;
     for (int o = 8; o > 0; o >>= 1) { const u64 q = __shfl_xor_sync(kLanes, m, o); m = q > m ? q : m; }
-    const u32 any_bad = __ballot_sync(kLanes, bad), missed = __ballot_sync(kLanes, miss);
+    const u32 missed = __ballot_sync(kLanes, miss);
     const i64 t0 = __shfl_sync(kLanes, v, 0), t1 = __shfl_sync(kLanes, v, p1);
+    const int z0 = __shfl_sync(kLanes, z, 0), z1 = __shfl_sync(kLanes, z, p1);
     if (j != 0) return;
     hole->join_p1 = p1;
-    hole->join_on = np >= 1 && (ok & 1u) && any_bad == 0u ? 1 : 0;
+    hole->join_on = (i32)(good & 1u);
+    hole->join_shift = z0 > z1 ? z0 : z1;
     hole->join_none = (missed & 1u) || ((missed >> p1) & 1u) ? 1 : 0;
     hole->join_t0 = t0; hole->join_t1 = t1;
     hole->join_tmod = m;
@@ -207,11 +219,9 @@ __device__ void join_leaf_set(const GrammarDev* g, HoleDev* hole, int nt) {
         S.cmin = ok ? (i32)lo : 0; S.cmax = ok ? (i32)hi : 0;
         S.cabs = ok ? (u32)cabs : 0u;
         S.mm = mm;
-        // |factor| * |operand| * |leaf| must stay below 2^62
-        const u64 A0 = magnitude((i64)hole->aff_Aj[0]), A1 = magnitude((i64)hole->aff_Aj[p1]);
-        u64 A = A0 > A1 ? A0 : A1;
-        if (A < 1 || A >> 31) A = 1ull << 31;
-        const u64 lim = ((1ull << 62) - 1) / A / most;
+        // |operand| * |leaf| must stay below 2^(62 - join_shift): see join_targets
+        const int z = hole->join_on ? hole->join_shift : 0;
+        const u64 lim = ((1ull << (62 - z)) - 1) / most;
         S.lim = lim < 0x7fffffffull ? (u32)lim : 0x7fffffffu;
         S.ok = ok && lim > 0 ? 1 : 0;
     }

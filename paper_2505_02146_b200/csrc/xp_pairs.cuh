@@ -9,7 +9,7 @@
 //   pair_div_kernel    -- / %: a warp takes 32 dividends next to each other in that order and walks only the divisors that
 //                         can reach the target: |r| in (|l|/(|t|+1), |l|/|t|] for a quotient, (|t|, |l| - |t|] for a remainder
 //                         (any above |t| when l is the target itself);
-//   pair_wide_kernel   -- operands that are not narrow (31 bits, or the root of 2^62 / |context factor|), exactly.
+//   pair_wide_kernel   -- operands that are not narrow (31 bits, or fewer where the context's factor ends in zero bits), exactly.
 // Candidates that agree at both probes wait in a warp's queue and are checked 32 at a time at the other probes.
 #pragma once
 
@@ -98,13 +98,11 @@ __device__ __forceinline__ u32 pair_slot(int2 v, u32 mask) {
     return h & mask;
 }
 
-// Narrow values stay below this: products with the context's factor must not reach 2^62.
+// Narrow values stay below this: products of two must not reach 2^(62 - join_shift) (see join_targets).
 __device__ __forceinline__ u32 pair_limit(const HoleDev* hole) {
-    const i64 a0 = (i64)hole->aff_Aj[0], a1 = (i64)hole->aff_Aj[hole->join_p1];
-    const u64 m0 = a0 < 0 ? 0ull - (u64)a0 : (u64)a0, m1 = a1 < 0 ? 0ull - (u64)a1 : (u64)a1, A = m0 > m1 ? m0 : m1;
-    if (A <= 1) return 0x7fffffffu;
+    const int z = hole->join_shift;
     u32 l = 0x7fffffffu;
-    while ((u64)l * l >= (1ull << 62) / A) l >>= 1;       // (a power of two less one: at most a bit below the root)
+    while ((u64)l * l >= 1ull << (62 - z)) l >>= 1;       // (a power of two less one: at most a bit below the root)
     return l;
 }
 

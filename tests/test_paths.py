@@ -334,3 +334,20 @@ def test_more_operands_than_32_bits_count(xp):
     whole = run(0, n[7])
     assert n[7] > 2 * 2**32 and whole.match_count[9] == sum(p.match_count[9] for p in parts) > 0
     assert whole.least_rank == min(p.least_rank for p in parts if p.solved) > 2**32
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("factor", ["3000000000", "-3000000001", "2147483648", "3221225472", "4294967296", "8589934593", "5497558138880",
+                                    "4611686018427387904", "-9223372036854775808", "9223372036854775807", "i", "(i-4)", "(j*1048576)"])
+def test_factors_of_the_context(xp, factor):
+    """Odd and even factors beyond 31 bits (even ones leave more than one hole value open modulo 2^64), and factors that are zero
+    at some of the points: leaf join, pair join and tiles against the oracle."""
+    c = [0, 1, 2, 3, 5, 7, -1, -4, 65536]
+    for g, size, spec in ((free_grammar(IJ, constant_set(-20, 20) + [65536, 2**31 - 1]), 5, "(i*7)+j"), (free_grammar(IJ, c), 5, "(i/3)-(j%5)"),
+                          (free_grammar(IJ, list(range(0, 12)) + [65536]), 7, "(i*3)+(j*2)")):
+        sk = Sketch(g, [Hole(0, size, ctx=parse_expr(f"(HOLE*{factor})+(j*3)", IJ), spec_expr=parse_expr(f"(({spec})*{factor})+(j*3)", IJ))], name=f"{factor} {spec}")
+        n = oracle.counts(g, 0, size)[size]
+        if size == 5:
+            check_sketch(xp, sk)
+        else:
+            check_sketch(xp, sk, windows={7: (n // 2 - 300_000, n // 2 + 300_001), 5: (3, 400_000)})
