@@ -216,6 +216,7 @@ struct xp_grammar {
     int leaf_begin[kMaxNt + 1] = {0};
     int bin_begin[kMaxNt + 1] = {0};
     u64 cnt[kMaxNt][kMaxSize + 1] = {{0}};
+    u32 wide_leaf = 0;               // nonterminals with a leaf that may be 2^31 or more in magnitude
     int ok_size = kMaxSize;          // counts are exact (< 2^63) up to this size
     // device copy, made on first use
     GrammarDev* d_g = nullptr;       // one block: header, leaves, binary productions
@@ -329,6 +330,12 @@ extern "C" xp_status xp_grammar_create(const xp_grammar_desc* d, xp_grammar** ou
         for (int i = lb; i < le; ++i) if (g->leaves[i].var >= 0) g->consts.push_back(ConstDev{g->leaves[i].var, i - lb, 0u});
     }
     g->const_begin[g->n_nt] = (int)g->consts.size();
+    for (int nt = 0; nt < g->n_nt; ++nt)
+        for (int i = g->leaf_begin[nt]; i < g->leaf_begin[nt + 1]; ++i) {
+            const LeafDev& l = g->leaves[i];
+            const i64 lo = l.var >= 0 ? g->lo[l.var] : l.value, hi = l.var >= 0 ? g->hi[l.var] : l.value + (l.value < 0);
+            if (lo <= INT32_MIN || hi > (l.var >= 0 ? 1ll << 31 : (1ll << 31) - 1)) g->wide_leaf |= 1u << nt;
+        }
     build_counts(g);
     *out = g;
     return XP_OK;
@@ -1500,7 +1507,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
                 Open c;
                 c.shifts = shifts;
                 c.seg = new_join_seg(sketch, hole, acc, k, lo, hi);
-                c.seg.kind = kJoinLeaf; c.seg.nt = ent; c.seg.esize = k - 2; c.seg.exact = ex ? 1 : 0; c.seg.heavy = ex || compares ? 1 : 0;
+                c.seg.kind = kJoinLeaf; c.seg.nt = ent; c.seg.esize = k - 2; c.seg.exact = ex ? kExactMany : 0; c.seg.heavy = ex || compares ? 1 : 0;
                 c.seg.e_begin = e0; c.seg.e_count = e1 - e0;
                 open.push_back(c);
                 at = &open.back();
@@ -1524,6 +1531,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
     for (Open& c : open) {
         c.seg.first_group = (i32)plan->jgroups.size();
         c.seg.n_groups = (i32)c.groups.size();
+        for (const JoinGroup& q : c.groups) if ((g->wide_leaf >> q.leaf_nt) & 1u) { c.seg.exact = kExactMany; c.seg.heavy = 1; }
         plan->jgroups.insert(plan->jgroups.end(), c.groups.begin(), c.groups.end());
         plan->jsegs.push_back(c.seg);
     }
@@ -1537,24 +1545,28 @@ static void add_direct(Plan* plan, int nt, int sketch, int hole, int acc, int k,
     plan->jsegs.push_back(sg);
 }
 
-// Tickets of the leaf join.  A step is 32 operands (one per lane); in the exact form one operand.  A ticket takes so
+// Tickets of the leaf join.  A step is 32 operands (one per lane).  A ticket takes so
 // many steps that every warp of the device gets about four: fewer and the last wave is uneven, more and the
-// warps spend their time taking tickets.  64 steps at most.
+// warps spend their time taking tickets.  64 steps at most.  In the exact form a ticket is one step, which costs as much as some
+// hundred others; with fewer steps than two for every warp it is one operand, so that the warps share those.
 static void number_joins(Plan* plan) {
     if (plan->jsegs.empty()) return;
     // the heavy tickets of a few large sketches first, so that none of them is a call's last (batches are long enough to even out)
     if (plan->jsegs.size() <= 64)
         std::stable_sort(plan->jsegs.begin(), plan->jsegs.end(), [](const JoinSeg& a, const JoinSeg& b) { return a.heavy > b.heavy; });
-    u64 steps = 0;
-    for (const JoinSeg& c : plan->jsegs) steps += c.exact ? c.e_count : (c.e_count + 31) / 32;
-    u64 per = steps / ((u64)search_warps() * 4);
+    u64 steps = 0, exact_steps = 0;
+    for (const JoinSeg& c : plan->jsegs) (c.exact ? exact_steps : steps) += (c.e_count + 31) / 32;
+    const u64 warps = (u64)search_warps();
+    const i32 form = exact_steps < 2 * warps ? kExactFew : kExactMany;
+    u64 per = steps / (warps * 4);
     if (per < 1) per = 1;
     if (per > 64) per = 64;
     if (per >= 4) per &= ~3ull;
     plan->join_wide = per >= 4;
     for (JoinSeg& c : plan->jsegs) {
+        if (c.exact) c.exact = form;
         c.first_ticket = plan->n_join;
-        c.chunk = (u32)(c.exact ? per : per * 32);
+        c.chunk = (u32)(c.exact ? (form == kExactFew ? 1 : 32) : per * 32);
         plan->n_join += (c.e_count + c.chunk - 1) / c.chunk;
     }
 }

@@ -205,6 +205,7 @@ constexpr i32 kPairNone = (i32)0x80000000u;
 // A piece of the leaf join's work: operands e_begin .. e_begin + e_count of (nt, esize), each against the leaves of
 // n_groups nonterminals.  kJoinDirect: candidates of (nt, esize) themselves, e_begin .. , checked on the probes one by one.
 enum { kJoinLeaf = 0, kJoinDirect = 1 };
+enum { kExactFew = 1, kExactMany = 2 };      // a warp per operand; a lane per operand
 constexpr int kJoinGroups = 8;        // most groups of a segment
 struct JoinGroup {
     i32 leaf_nt, pad;
@@ -217,7 +218,7 @@ struct JoinSeg {
     i32 sketch, hole, size, kind;
     i32 acc, nt, esize, n_groups;
     i32 first_group;
-    i32 exact;                       // the operators have no condition (shifts): every candidate is evaluated on its own
+    i32 exact;                       // kExactFew, kExactMany: there is no condition (shifts, a leaf of 2^31 or more), every candidate is evaluated on its own
     u32 chunk;                       // operands per ticket
     i32 heavy;                       // an operand costs many times the usual (exact form, contexts that compare): these go first
     u64 e_begin, e_count;

@@ -20,7 +20,8 @@
 // A context that compares asks for an interval of values at every probe.  Every operator but % is monotone in a constant
 // (on either side of zero, for a / c): its constants are one or two runs, the intersection of the probes' intervals
 // (range_runs); remainders are tested constant by constant at the first probe with reciprocals.
-// Operands of JoinSet::lim or more and shifts take the exact form: one operand at a time, lanes over the leaves.
+// Operands of JoinSet::lim or more, leaf sets with a wider leaf and shifts take the exact form, in 64 bits: 32 operands at a time, a
+// lane each (they too wait in a queue), or, where a segment has few operands, one at a time, lanes over the leaves.
 // Warps work on their own; nothing here waits for another warp.
 #pragma once
 
@@ -74,7 +75,8 @@ struct JoinWarp {
     u32 q_off[kJoinQueue];                                // suspects: operand number relative to `base`,
     i32 q_a0[kJoinQueue], q_a1[kJoinQueue];               //   its values at the two probes
     u32 c_off[64], c_pos[64], c_code[64];                 // candidates: operand, leaf position, group << 8 | slot << 1 | swapped
-    u32 nq, nc;                                           // suspects and candidates waiting (of segment `seg`)
+    u32 w_off[kJoinQueue];                                // wide operands
+    u32 nq, nc, nw;                                       // suspects, candidates and wide operands waiting (of segment `seg`)
     GroupCtx grp[kJoinGroups];
     CandShared cand;                                      // candidate of a whole-domain check that the warp does itself
 };
@@ -326,7 +328,7 @@ __device__ __noinline__ bool residue_exists(u32 u0, u32 u1, u32 ut0, u32 ut1, u3
     return false;
 }
 
-enum { kSlotAdd = 0, kSlotSub = 1, kSlotMul = 2, kSlotDiv = 3, kSlotMod = 4, kSlotMn = 5, kSlotMx = 6 };
+enum { kSlotAdd = 0, kSlotSub = 1, kSlotMul = 2, kSlotDiv = 3, kSlotMod = 4, kSlotMn = 5, kSlotMx = 6, kSlotShl = 7, kSlotShr = 8 };
 
 __device__ __forceinline__ bool const_div_fwd(float f0, float f1, const JoinCtx& x, float fc) {       // some |c| in (|a|/(|t|+1), |a|/|t|] at both
     const float hi = fminf(f0 * x.rt0 + x.h0, f1 * x.rt1 + x.h1) * 1.000002f, lo = fmaxf(f0 * x.rl0, f1 * x.rl1) * 0.999998f;
@@ -689,8 +691,8 @@ __device__ __noinline__ void join_drain(JoinWarp& w, u32 n_q, const PlanDev& pla
     __syncwarp();
 }
 
-// The exact form: one operand at a time (the same for all lanes), lanes over the leaves, every operator; the first probe
-// here, the others when a warp's worth of candidates has gathered.
+// The exact form where a segment has few operands (kExactFew): one at a time (the same for all lanes), lanes over the leaves, every
+// operator; the first two probes here, the others when a warp's worth of candidates has gathered.
 __device__ __noinline__ void join_exact(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, u64 e, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
@@ -720,6 +722,97 @@ __device__ __noinline__ void join_exact(JoinWarp& w, const PlanDev& plan, const 
         }
     }
     if (w.nc) join_check(w, plan, seg, sk, hole, two ? 2 : 1, n);
+}
+
+// What a probe demands of a candidate's value, in registers.
+struct ProbeWant { bool affine; u64 A, D; i64 lo, hi; };
+__device__ __forceinline__ ProbeWant probe_want(const HoleDev* hole, int j) {
+    ProbeWant p;
+    p.affine = (hole->aff_okmask >> j) & 1u;
+    p.A = hole->aff_Aj[j]; p.D = (u64)hole->probe_spec[j] - hole->aff_Bj[j];
+    p.lo = hole->rng_lo[j]; p.hi = hole->rng_hi[j];
+    return p;
+}
+__device__ __forceinline__ bool wanted(const ProbeWant& p, i64 v) {      // (probe_accepts)
+    if (p.affine) return (u64)v * p.A == p.D;
+    return v <= -(1ll << 62) || v >= (1ll << 62) || (v >= p.lo && v <= p.hi);
+}
+
+// For which of the operators `ops` is the result of operand a and leaf c what the probe wants?  Bit = slot for a op c, 16 + slot for
+// c op a.  In 64 bits, one division for quotient and remainder; `ops` is the same for all lanes.
+__device__ __forceinline__ u32 exact_bits(i64 a, i64 c, u32 ops, const ProbeWant& p) {
+    auto both = [](int slot) { return 0x10001u << slot; };
+    u32 b = 0;
+    i64 v;
+    if (ops & both(kSlotAdd)) { (void)apply_op(XP_OP_ADD, a, c, v); if (wanted(p, v)) b |= both(kSlotAdd); }
+    if (ops & (1u << kSlotSub)) { (void)apply_op(XP_OP_SUB, a, c, v); if (wanted(p, v)) b |= 1u << kSlotSub; }
+    if (ops & (0x10000u << kSlotSub)) { (void)apply_op(XP_OP_SUB, c, a, v); if (wanted(p, v)) b |= 0x10000u << kSlotSub; }
+    if (ops & both(kSlotMul)) { (void)apply_op(XP_OP_MUL, a, c, v); if (wanted(p, v)) b |= both(kSlotMul); }
+    if (ops & both(kSlotMn)) { if (wanted(p, a < c ? a : c)) b |= both(kSlotMn); }
+    if (ops & both(kSlotMx)) { if (wanted(p, a > c ? a : c)) b |= both(kSlotMx); }
+#pragma unroll 1
+    for (int swap = 0; swap < 2; ++swap) {
+        const u32 o = swap ? ops >> 16 : ops & 0xffffu;
+        const i64 x = swap ? c : a, y = swap ? a : c;
+        u32 q = 0;
+        if ((o & ((1u << kSlotDiv) | (1u << kSlotMod))) && apply_op(XP_OP_DIV, x, y, v)) {
+            if (wanted(p, v)) q |= 1u << kSlotDiv;
+            if (wanted(p, (i64)((u64)x - (u64)v * (u64)y))) q |= 1u << kSlotMod;
+        }
+        if ((o & (1u << kSlotShl)) && apply_op(XP_OP_SHL, x, y, v) && wanted(p, v)) q |= 1u << kSlotShl;
+        if ((o & (1u << kSlotShr)) && apply_op(XP_OP_SHR, x, y, v) && wanted(p, v)) q |= 1u << kSlotShr;
+        b |= swap ? q << 16 : q;
+    }
+    return b & ops;
+}
+
+// The exact form for 32 operands, one per lane (live: this lane has one): every leaf, every operator, at the first two probes; the
+// others when a warp's worth of candidates has gathered (from probe `from` on).  Called by all 32 lanes together.  Bound by the
+// 64-bit arithmetic.  (One operand at a time, each lookup and each vote was waited for: size 7, 63 leaves with shifts 72 -> 27 ms;
+// 36 leaves with one of 2^33 16.3 -> 3.1 ms.)
+__device__ __noinline__ void join_exact32(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, u64 e, bool live,
+                                          int from, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const bool two = hole->n_exact >= 2;
+    i64 a0 = 0, a1 = 0;
+    if (live) {
+        const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
+        live = ref_value(g, hole, ref, seg.nt, seg.esize, 0, a0) && (!two || ref_value(g, hole, ref, seg.nt, seg.esize, 1, a1));
+    }
+    const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
+    if (n_live == 0u) return;
+    const ProbeWant p0 = probe_want(hole, 0), p1 = probe_want(hole, two ? 1 : 0);
+    const u32 off = (u32)(e - w.base);
+    for (int gi = 0; gi < seg.n_groups; ++gi) {
+        const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+        const int nl = (int)g->cnt[grp.leaf_nt][1], lb = g->leaf_begin[grp.leaf_nt];
+        const u32 ops = grp.fmask | (grp.smask << 16);
+        n.tests += (u64)nl * (u64)__popc(ops) * n_live;
+        for (int l = 0; l < nl; ++l) {
+            const LeafDev lf = g->leaves[lb + l];
+            u32 hits = live ? exact_bits(a0, lf.var >= 0 ? hole->probe_pt[0][lf.var] : lf.value, ops, p0) : 0u;
+            if (!__any_sync(0xffffffffu, hits != 0u)) continue;
+            if (two && hits) hits &= exact_bits(a1, lf.var >= 0 ? hole->probe_pt[1][lf.var] : lf.value, ops, p1);
+#pragma unroll 1
+            for (u32 m = __reduce_or_sync(0xffffffffu, hits); m; m &= m - 1) {
+                const int bit = __ffs((int)m) - 1;
+                const u32 b = __ballot_sync(0xffffffffu, (hits >> bit) & 1u);
+                n.suspects += (u32)__popc(b);
+                join_push(w, plan, seg, sk, hole, (hits >> bit) & 1u, off, (u32)l, gi, bit & 15, bit >> 4, from, n);
+            }
+        }
+    }
+}
+
+// The first n_w wide operands of the warp's queue, 32 at a time.
+__device__ __noinline__ void join_wide(JoinWarp& w, u32 n_w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, JoinCount& n) {
+    const u32 lane = threadIdx.x & 31u;
+    __syncwarp();
+    for (u32 at = 0; at < n_w; at += 32u) {
+        const bool live = at + lane < n_w;
+        join_exact32(w, plan, seg, sk, hole, w.base + (live ? w.w_off[at + lane] : 0u), live, hole->join_p1 ? 2 : 1, n);
+    }
+    __syncwarp();
 }
 
 // ---- operands in rank order ----
@@ -980,15 +1073,19 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     const int lane = threadIdx.x & 31;
     n.cands += count * w.hot.pairs;
     const u32 lim = w.hot.lim;
-    if (seg.exact || !hole->join_on || lim == 0u) {
+    if (seg.exact == kExactFew) {
         for (u64 i = 0; i < count; ++i) join_exact(w, plan, seg, sk, hole, first + i, n);
+        return;
+    }
+    if (seg.exact || !hole->join_on || lim == 0u) {
+        for (u64 i = 0; i < count; i += 32u) join_exact32(w, plan, seg, sk, hole, first + i + lane, i + lane < count, hole->join_p1 ? 2 : 1, n);
         return;
     }
     const JoinCtx x = w.x;
     const int n_lin = w.hot.n_lin, n_mul = w.hot.n_mul, n_other = w.hot.n_other, n_set = w.hot.n_set;
     const u32 mul_t = w.hot.mul_t;
     const u32 tests_each = w.hot.tests;
-    u32 nq = w.nq;
+    u32 nq = w.nq, nw = w.nw;
     u32 n_alive = 0;
     for (u64 done = 0; done < count;) {
         const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done);
@@ -1064,16 +1161,28 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
                 }
             }
             if (__any_sync(0xffffffffu, wide != 0u)) {
-#pragma unroll 1
-                for (int p = 0; p < P; ++p)
-                    for (u32 m = __ballot_sync(0xffffffffu, (wide >> p) & 1u); m; m &= m - 1)
-                        join_exact(w, plan, seg, sk, hole, first + done + at + (u64)(32 * p + __ffs((int)m) - 1), n);
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    const bool h = (wide >> p) & 1u;
+                    const u32 b = __ballot_sync(0xffffffffu, h);
+                    if (h) w.w_off[nw + (u32)__popc(b & ((1u << lane) - 1u))] = off0 + at + 32u * p;
+                    nw += (u32)__popc(b);
+                }
+                if (nw >= 32u) {
+                    const u32 full = nw & ~31u;
+                    join_wide(w, full, plan, seg, sk, hole, n);
+                    nw -= full;
+                    const u32 o = lane < (int)nw ? w.w_off[full + lane] : 0u;
+                    __syncwarp();
+                    if (lane < (int)nw) w.w_off[lane] = o;
+                    __syncwarp();
+                }
             }
         }
         done += n_run;
     }
     n.tests += (u64)tests_each * (u64)__reduce_add_sync(0xffffffffu, n_alive);
-    if (lane == 0) w.nq = nq;                             // (fewer than 32: they wait for the warp's next ticket of this segment)
+    if (lane == 0) { w.nq = nq; w.nw = nw; }              // (fewer than 32: they wait for the warp's next ticket of this segment)
     __syncwarp();
 }
 
@@ -1083,9 +1192,10 @@ __device__ __noinline__ void join_leave(JoinWarp& w, const PlanDev& plan, int in
     const SketchDev* sk = plan.sketches[seg.sketch];
     const HoleDev* hole = &sk->holes[seg.hole];
     if (w.nq) join_drain(w, w.nq, plan, seg, sk, hole, n);
+    if (w.nw) join_wide(w, w.nw, plan, seg, sk, hole, n);
     if (w.nc) join_check(w, plan, seg, sk, hole, hole->join_p1 ? 2 : 1, n);
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) { w.nq = 0; w.seg = -1; }
+    if ((threadIdx.x & 31) == 0) { w.nq = w.nw = 0; w.seg = -1; }
     __syncwarp();
 }
 
@@ -1233,8 +1343,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
             }
         }
         if (!sets_ok) wide = live;
-        for (u32 m = __ballot_sync(0xffffffffu, live && wide); m; m &= m - 1)
-            join_exact(w, plan, seg, sk, hole, first + at + (u64)(__ffs((int)m) - 1), n);
+        if (__any_sync(0xffffffffu, live && wide)) join_exact32(w, plan, seg, sk, hole, e, live && wide, 0, n);
         live = live && !wide;
         const u32 off = (u32)(e - w.base);
         const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
@@ -1400,7 +1509,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
     __shared__ JoinWarp sh[kJoinWarps];
     JoinWarp& w = sh[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    if (lane == 0) { w.nq = 0; w.nc = 0; w.seg = -1; }
+    if (lane == 0) { w.nq = w.nc = w.nw = 0; w.seg = -1; }
     __syncwarp();
     JoinCount n{0, 0, 0, 0, 0};
     int acc = -1;

@@ -351,3 +351,31 @@ def test_factors_of_the_context(xp, factor):
             check_sketch(xp, sk)
         else:
             check_sketch(xp, sk, windows={7: (n // 2 - 300_000, n // 2 + 300_001), 5: (3, 400_000)})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("consts,ops,ctx,spec", [
+    (list(range(0, 18)), ["+", "*", "<<", ">>"], "", "((i<<3)+j)*2"),
+    (list(range(0, 17)) + [63, 64, -1], ["-", "%", "<<", ">>"], "", "(i<<2)-(j>>1)"),
+    (list(range(1, 18)) + [W], "+-*/%", "", f"((i*{W})+j)-3"),
+    (list(range(1, 18)) + [W, 2**31 - 1, -2**31], "+-*/%", "(HOLE*3)+i", f"(j*{W})/5"),
+    (list(range(1, 18)) + [2**31 - 1], "+-*/%", "", "(i*2147483647)+(j*3)"),      # narrow leaves, wide operands
+    (list(range(1, 18)) + [2**30], ["+", "-", "*", "min", "max", "/"], "", "(i*1073741824)/(j+7)"),
+    (list(range(0, 18)) + [W], ["+", "-", "<<"], "j<HOLE", "i-2"),
+])
+def test_many_operands_in_the_exact_form(xp, consts, ops, ctx, spec):
+    """Some 4e5 operands of size 5: shifts, leaves and operands of 2^31 or more, 32 at a time; windows at the first block of each
+    production, across the end of its blocks with a leaf on the left, and at its end."""
+    g = free_grammar(IJ, consts, ops=list(ops))
+    text = ctx.replace("HOLE", f"({spec})") if ctx else spec
+    sk = Sketch(g, [Hole(0, 7, ctx=parse_expr(ctx, IJ) if ctx else [], spec_expr=parse_expr(text, IJ))], name=text)
+    n = oracle.counts(g, 0, 7)
+    per = n[7] // len(ops)
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
+    for p in range(len(ops)):
+        for at in (p * per, p * per + n[1] * n[5] - 100_000, (p + 1) * per - 200_000):
+            w = (max(at, 0), min(at + 200_000, n[7]))
+            got = xp.xp_repair(ls, rank_ranges=[(0, 7, *w)], size_min=7)[0]
+            want = oracle.repair_hole(sk, rank_ranges={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: w})
+            assert (got.match_count[7], got.solved) == (want.match_count[7], want.solved), w
+            assert not want.solved or (got.least_rank, got.least_text) == (want.least_rank, want.least_text)
