@@ -62,6 +62,31 @@ struct GrammarDev {
 // probes (a0, a1) and asks, per operator, for which leaves the result can be the target at both.  Constants have the
 // same value at both probes, so one condition on (a0, a1) decides all of them at once; the variables, and constants
 // when there are only a few, are entries that are tested one by one.
+//
+// Least m with m mod u0 = t0 and m mod u1 = t1, ~0 when there is none (u0 > t0, u1 > t1, both below 2^31): m = t0 + u0 k with
+// u0 k = t1 - t0 modulo u1, solved by the extended Euclidean algorithm.
+#ifdef __CUDACC__
+#define XP_HD __host__ __device__
+#else
+#define XP_HD
+#endif
+constexpr u32 kResidueSteps = 24;     // as many steps cost about what that algorithm does
+XP_HD inline u64 residue_least(u32 u0, u32 u1, u32 t0, u32 t1) {
+    u32 g = u1, r = u0 % u1;
+    i32 x = 0, y = 1;                 // y u0 = r, x u0 = g (modulo u1)
+    while (r != 0u) {
+        const u32 q = g / r, s = g - q * r;
+        const i32 z = x - (i32)q * y;
+        g = r; r = s;
+        x = y; y = z;
+    }
+    const i64 d = (i64)t1 - (i64)t0;
+    if (d % (i64)g != 0) return ~0ull;
+    const u32 n = u1 / g;             // k is known modulo n
+    const i64 inv = x < 0 ? (i64)x + (i64)n : (i64)x, e = (d / (i64)g) % (i64)n;
+    const u64 k = (u64)(inv % (i64)n) * (u64)(e < 0 ? e + (i64)n : e) % (u64)n;
+    return (u64)t0 + (u64)u0 * k;
+}
 constexpr int kOpSlots = 9;           // + - * / % min max << >> (in this order; the last two only in the exact form)
 constexpr int kJoinEntries = 12;      // most leaves of a nonterminal that are tested one by one
 constexpr int kJoinFewConsts = 4;     // constants up to this many are entries too
@@ -232,11 +257,6 @@ struct JoinSeg {
 // 2 * blocks * pieces entries, which is the most that all walks together can list: neither list is written past its end
 // and neither counter passes it, whatever the operands are.  (Short pieces as long as they fit: where most of a walk
 // agrees at both probes, every 32 divisors are 32 exact checks, and with pieces of 512 one such search took 60 ms longer.)
-#ifdef __CUDACC__
-#define XP_HD __host__ __device__
-#else
-#define XP_HD
-#endif
 constexpr u32 kPairWalk = 64;        // divisors that a warp of the division kernel meets in one go, at least
 constexpr u32 kPairShort = 1u << 18; // entries of the list of short pieces (2 MB)
 constexpr u32 kPairLong = 1u << 20;  // entries of the list of long ones that `pieces` aims at (8 MB)

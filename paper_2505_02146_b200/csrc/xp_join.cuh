@@ -319,10 +319,13 @@ __device__ __noinline__ bool gcd_exceeds(u32 x, u32 y, u32 least) {      // gcd(
     return x > least;
 }
 
-// Is there a magnitude m <= cabs with m mod u0 = ut0 and m mod u1 = ut1?  Stepping along the larger of the two.
+// Is there a magnitude m <= cabs with m mod u0 = ut0 and m mod u1 = ut1?  Stepping along the larger of the two where that is a few
+// steps, otherwise by the least such m.  (With a constant of 2^31 - 1 the steps, up to 46 000 an operand, were the search: 69 leaves, size 7,
+// 118 -> 10 ms.)
 __device__ __noinline__ bool residue_exists(u32 u0, u32 u1, u32 ut0, u32 ut1, u32 cabs) {
     if (u0 <= ut0 || u1 <= ut1) return false;
     if (u0 < u1) { u32 s = u0; u0 = u1; u1 = s; s = ut0; ut0 = ut1; ut1 = s; }
+    if (u1 > kResidueSteps && cabs / u0 > kResidueSteps) return residue_least(u0, u1, ut0, ut1) <= cabs;
     u32 steps = u1;                                       // (the residues repeat after u1 steps)
     for (u64 m = ut0; m <= cabs && steps > 0u; m += u0, --steps) if ((u32)m % u1 == ut1) return true;
     return false;

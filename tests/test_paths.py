@@ -209,14 +209,46 @@ def test_one_sketch_under_both_plans_from_several_threads(xp):
     assert not bad
 
 
+def run_on_host(tmp_path, name, body):
+    """Compiles and runs a C++ program over the structures and rules that host and kernels share."""
+    src, exe = tmp_path / f"{name}.cpp", tmp_path / name
+    src.write_text('#include <cstdio>\n#include "xp_dev.h"\nusing namespace xp;\n' + body)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I" + os.path.join(ROOT, "paper_2505_02146_b200", "csrc"), "-I" + os.path.join(ROOT, "include"),
+                           "-I/usr/local/cuda/include", str(src), "-o", str(exe)])
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert (r.returncode, r.stdout) == (0, "")
+
+
+def test_least_number_with_two_residues(tmp_path):
+    run_on_host(tmp_path, "residues", r"""
+static u64 plain(u64 u0, u64 u1, u64 t0, u64 t1) { for (u64 k = 0; k < u1; ++k) if ((t0 + u0 * k) % u1 == t1) return t0 + u0 * k; return ~0ull; }
+static bool same(u32 u0, u32 u1, u32 t0, u32 t1) {
+    if (residue_least(u0, u1, t0, t1) == plain(u0, u1, t0, t1)) return true;
+    printf("%u %u %u %u\n", u0, u1, t0, t1);
+    return false;
+}
+int main() {
+    for (u32 u0 = 1; u0 < 26; ++u0) for (u32 u1 = 1; u1 < 26; ++u1)
+        for (u32 t0 = 0; t0 < u0; ++t0) for (u32 t1 = 0; t1 < u1; ++t1) if (!same(u0, u1, t0, t1)) return 1;
+    const u32 big = 0x7fffffffu;
+    u64 x = 1;
+    auto next = [&]() { x = x * 6364136223846793005ull + 1442695040888963407ull; return (u32)(x >> 33); };
+    for (int n = 0; n < 2000; ++n) {
+        const u32 u1 = 1 + next() % 3000, f = 1 + next() % 40, u0 = n % 3 ? 1 + next() % (big - 1) : u1 * f;
+        if (!same(u0, u1, next() % u0, next() % u1)) return 1;
+        const u32 v0 = 1 + next() % (big - 1), v1 = 1 + next() % (big - 1), m = next();      // m itself is one: the least is no larger, and has its residues
+        const u64 l = residue_least(v0, v1, m % v0, m % v1);
+        if (l > m || l % v0 != m % v0 || l % v1 != m % v1) { printf("%u %u of %u\n", v0, v1, m); return 1; }
+    }
+    return 0;
+}
+""")
+
+
 def test_the_list_of_long_walks_holds_every_piece(tmp_path):
     """Division kernel of the pair join: all walks together never list more pieces than the list has room for (nor than 32
     bits count), and the pieces of a walk cover it."""
-    src = tmp_path / "walks.cpp"
-    src.write_text(r"""
-#include <cstdio>
-#include "xp_dev.h"
-using namespace xp;
+    run_on_host(tmp_path, "walks", r"""
 int main() {
     const u32 sizes[] = {1, 31, 32, 33, 63, 64, 65, 129, 1125, 9245, 92480, 3150592, 1u << 22};
     for (u32 nl : sizes) for (u32 nr : sizes) {
@@ -236,11 +268,6 @@ int main() {
     return 0;
 }
 """)
-    exe = tmp_path / "walks"
-    subprocess.check_call(["g++", "-std=c++17", "-I" + os.path.join(ROOT, "paper_2505_02146_b200", "csrc"), "-I" + os.path.join(ROOT, "include"),
-                           "-I/usr/local/cuda/include", str(src), "-o", str(exe)])
-    r = subprocess.run([str(exe)], capture_output=True, text=True)
-    assert (r.returncode, r.stdout) == (0, "")
 
 
 @pytest.mark.gpu
@@ -360,6 +387,7 @@ def test_factors_of_the_context(xp, factor):
     (list(range(1, 18)) + [W], "+-*/%", "", f"((i*{W})+j)-3"),
     (list(range(1, 18)) + [W, 2**31 - 1, -2**31], "+-*/%", "(HOLE*3)+i", f"(j*{W})/5"),
     (list(range(1, 18)) + [2**31 - 1], "+-*/%", "", "(i*2147483647)+(j*3)"),      # narrow leaves, wide operands
+    (list(range(1, 18)) + [2**31 - 1, 1000003], "%+*-/", "", "1000003%((i*37)+(j+90))"),     # residues of large constants
     (list(range(1, 18)) + [2**30], ["+", "-", "*", "min", "max", "/"], "", "(i*1073741824)/(j+7)"),
     (list(range(0, 18)) + [W], ["+", "-", "<<"], "j<HOLE", "i-2"),
 ])
