@@ -1673,12 +1673,13 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, b
     }
 }
 
-constexpr u32 kSurvCap = 65536;              // survivor queue entries of a call with its own workspace (at least)
-
-// Batches get 256 entries per sketch, up to 2^20.
-static u32 surv_cap_for(size_t n_sketches) {
+// Survivor queue entries of a call with its own workspace.  A survivor that finds the queue full is checked by the warp that has it, alone
+// and at once, at some ten times the cost (a loop bound in a guard, 133 503 survivors on 65 536 points: 254 ms with 65 536
+// entries, 13 with 2^20).  A caller's workspace made for fewer entries is taken with as many as it holds, from surv_least on.
+constexpr u32 kSurvMost = 1u << 20;          // (42 MB)
+static u32 surv_least(size_t n_sketches) {
     const size_t want = n_sketches * 256;
-    return (u32)(want < kSurvCap ? kSurvCap : (want > (1u << 20) ? (1u << 20) : want));
+    return (u32)(want < 65536 ? 65536 : (want > kSurvMost ? kSurvMost : want));
 }
 constexpr u32 kSurvCapStatic = 8192;         // ... of a call on the library's fixed scratch
 
@@ -1778,7 +1779,7 @@ extern "C" size_t xp_workspace_bytes(const xp_sketch* const* sketches, size_t n,
     if (!sketches || n == 0) return 0;
     Plan plan;
     if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, true, &plan) != XP_OK) return 0;
-    return ws_layout(plan, sketches, n, surv_cap_for(n)).total;
+    return ws_layout(plan, sketches, n, kSurvMost).total;
 }
 
 extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n, const xp_repair_opts* opts,
@@ -1795,15 +1796,23 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     if (st != XP_OK) return st;
     cudaStream_t stream = (cudaStream_t)o->stream;
 
-    SearchLayout w = ws_layout(plan, sketches, n, surv_cap_for(n));
+    SearchLayout w = ws_layout(plan, sketches, n, kSurvMost);
     char* ws = (char*)o->workspace;
+    auto shrink = [&]() {                                 // to the caller's workspace, if the queue can be made small enough
+        for (u32 cap = kSurvMost; w.total > o->workspace_bytes && cap > surv_least(n);) {
+            cap = cap / 2 > surv_least(n) ? cap / 2 : surv_least(n);
+            w = ws_layout(plan, sketches, n, cap);
+        }
+    };
+    if (ws) shrink();
     if (ws && o->workspace_bytes < w.total && !plan.psegs.empty()) {
         // A refinement can change which blocks the pair join may take (a target that is no longer zero), and so what a call
         // needs: a caller's workspace made before it holds the plan without the pair join.
         plan = Plan();
         st = build_plan(sketches, n, o, false, &plan);
         if (st != XP_OK) return st;
-        w = ws_layout(plan, sketches, n, surv_cap_for(n));
+        w = ws_layout(plan, sketches, n, kSurvMost);
+        shrink();
     }
     bool own_ws = false, cached_ws = false;
     if (ws) {

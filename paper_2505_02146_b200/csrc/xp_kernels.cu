@@ -2451,10 +2451,10 @@ __global__ void __launch_bounds__(256) surv_scatter_kernel(const __grid_constant
     chain_wait();
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
-    const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int acc = plan.surv[i].acc;
-    plan.surv_sorted[plan.surv_off[acc] + atomicAdd(&plan.surv_hist[acc], 1u)] = i;
+    for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int acc = plan.surv[i].acc;
+        plan.surv_sorted[plan.surv_off[acc] + atomicAdd(&plan.surv_hist[acc], 1u)] = i;
+    }
 }
 
 // ---- whole-domain check of several survivors of one hole together ----
@@ -3023,14 +3023,13 @@ __global__ void count_kernel(const __grid_constant__ PlanDev plan) {
     chain_wait();
     const u32 pushed = *plan.surv_n;
     const u32 n = pushed < plan.surv_cap ? pushed : plan.surv_cap;
-    const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const SurvDev sv = plan.surv[i];
-    const SketchDev* sk = plan.sketches[sv.sketch];
-    if (sk->n_points != 0) return;
-    AccDev* a = &plan.acc[sv.acc];
-    atomicAdd(&a->match_count[sv.size], 1ull);
-    atomicMin(&a->min_rank[sv.size], sv.rank);
+    for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const SurvDev sv = plan.surv[i];
+        if (plan.sketches[sv.sketch]->n_points != 0) continue;
+        AccDev* a = &plan.acc[sv.acc];
+        atomicAdd(&a->match_count[sv.size], 1ull);
+        atomicMin(&a->min_rank[sv.size], sv.rank);
+    }
 }
 
 #ifdef XP_CHECKS
@@ -3302,10 +3301,11 @@ cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_ticket
     const Residency* R = residency();
     if (!R) return cudaErrorInvalidDevice;
     if (any_tickets) {
+        const u32 queue = (L.surv_cap + 255) / 256, surv_ctas = queue < 256u ? queue : 256u;      // (one wave; the kernels stride)
         if (pd.surv_sorted) {
             chain(surv_scan_kernel, 1, 1024, 0, stream, pd.surv_hist, pd.surv_off, pd.n_acc);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            chain(surv_scatter_kernel, (L.surv_cap + 255) / 256, 256, 0, stream, pd);
+            chain(surv_scatter_kernel, surv_ctas, 256, 0, stream, pd);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *n_launches += 2;
         }
@@ -3313,7 +3313,7 @@ cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_ticket
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *n_launches += 1;
         if (L.empty_domain) {
-            chain(count_kernel, (L.surv_cap + 255) / 256, 256, 0, stream, pd);
+            chain(count_kernel, surv_ctas, 256, 0, stream, pd);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *n_launches += 1;
         }

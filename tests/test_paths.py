@@ -335,8 +335,9 @@ def test_a_workspace_made_before_a_refinement(xp):
     assert xp.xp_workspace_bytes([ls]) > need                           # (or this test does not test what it says)
     assert_same(xp.xp_repair(ls, workspace=ws)[0], before)
     assert_same(xp.xp_repair(ls)[0], before)
+    assert_same(xp.xp_repair(ls, workspace=ws[:need - 40 * (2**20 - 65536)])[0], before)      # (with the shortest survivor queue)
     with pytest.raises(xp.XpError) as e:                                # too small for any plan: refused as ever
-        xp.xp_repair(ls, workspace=ws[:need // 2])
+        xp.xp_repair(ls, workspace=ws[:1 << 20])
     assert e.value.status == 5
 
 
@@ -407,3 +408,24 @@ def test_many_operands_in_the_exact_form(xp, consts, ops, ctx, spec):
             want = oracle.repair_hole(sk, rank_ranges={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: w})
             assert (got.match_count[7], got.solved) == (want.match_count[7], want.solved), w
             assert not want.solved or (got.least_rank, got.least_text) == (want.least_rank, want.least_text)
+
+
+@pytest.mark.gpu
+def test_more_survivors_than_the_queue_of_a_small_workspace_holds(xp):
+    """A workspace made for 65 536 survivors, as callers have had, is taken with what it holds: the warps check the others themselves."""
+    import torch
+    vs = [Variable("i", 0, 16), Variable("j", 0, 16)]
+    g = free_grammar(vs, constant_set(-12, 12))
+    sk = Sketch(g, [Hole(0, 5, spec_expr=parse_expr("0", vs))])
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
+    want = oracle.repair_hole(sk)
+    assert want.match_count[5] > 65536
+    need = xp.xp_workspace_bytes([ls])
+    small = need - 40 * (2**20 - 65536)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    for size in (need, small + 1_000_000, small):
+        assert_same(xp.xp_repair(ls, workspace=ws[:size])[0], want, f"{size} bytes")
+    assert_same(xp.xp_repair(ls)[0], want)
+    with pytest.raises(xp.XpError) as e:
+        xp.xp_repair(ls, workspace=ws[:small - 256])
+    assert e.value.status == 5
