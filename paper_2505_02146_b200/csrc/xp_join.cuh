@@ -818,6 +818,31 @@ __device__ __noinline__ void join_wide(JoinWarp& w, u32 n_w, const PlanDev& plan
     __syncwarp();
 }
 
+// Wide operands (bit p of `wide`: number off + 32 p) into their queue; whole warps of them are taken up.  Called by all lanes.
+__device__ __noinline__ void join_push_wide(JoinWarp& w, u32 wide, u32 off, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
+                                            JoinCount& n) {
+    const int lane = threadIdx.x & 31;
+    u32 nw = w.nw;
+    for (u32 any = __reduce_or_sync(0xffffffffu, wide); any; any &= any - 1) {
+        const int p = __ffs((int)any) - 1;
+        const bool h = (wide >> p) & 1u;
+        const u32 b = __ballot_sync(0xffffffffu, h);
+        if (h) w.w_off[nw + (u32)__popc(b & ((1u << lane) - 1u))] = off + 32u * (u32)p;
+        nw += (u32)__popc(b);
+    }
+    if (nw >= 32u) {
+        const u32 full = nw & ~31u;
+        join_wide(w, full, plan, seg, sk, hole, n);
+        nw -= full;
+        const u32 o = lane < (int)nw ? w.w_off[full + lane] : 0u;
+        __syncwarp();
+        if (lane < (int)nw) w.w_off[lane] = o;
+    }
+    __syncwarp();
+    if (lane == 0) w.nw = nw;
+    __syncwarp();
+}
+
 // ---- operands in rank order ----
 
 // A run of operands of (nt, size) in rank order that one production and pair of sizes builds: entries of the pair
@@ -1088,7 +1113,7 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     const int n_lin = w.hot.n_lin, n_mul = w.hot.n_mul, n_other = w.hot.n_other, n_set = w.hot.n_set;
     const u32 mul_t = w.hot.mul_t;
     const u32 tests_each = w.hot.tests;
-    u32 nq = w.nq, nw = w.nw;
+    u32 nq = w.nq;
     u32 n_alive = 0;
     for (u64 done = 0; done < count;) {
         const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done);
@@ -1163,29 +1188,12 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
                     __syncwarp();
                 }
             }
-            if (__any_sync(0xffffffffu, wide != 0u)) {
-#pragma unroll
-                for (int p = 0; p < P; ++p) {
-                    const bool h = (wide >> p) & 1u;
-                    const u32 b = __ballot_sync(0xffffffffu, h);
-                    if (h) w.w_off[nw + (u32)__popc(b & ((1u << lane) - 1u))] = off0 + at + 32u * p;
-                    nw += (u32)__popc(b);
-                }
-                if (nw >= 32u) {
-                    const u32 full = nw & ~31u;
-                    join_wide(w, full, plan, seg, sk, hole, n);
-                    nw -= full;
-                    const u32 o = lane < (int)nw ? w.w_off[full + lane] : 0u;
-                    __syncwarp();
-                    if (lane < (int)nw) w.w_off[lane] = o;
-                    __syncwarp();
-                }
-            }
+            if (__any_sync(0xffffffffu, wide != 0u)) join_push_wide(w, wide, off0 + at, plan, seg, sk, hole, n);
         }
         done += n_run;
     }
     n.tests += (u64)tests_each * (u64)__reduce_add_sync(0xffffffffu, n_alive);
-    if (lane == 0) { w.nq = nq; w.nw = nw; }              // (fewer than 32: they wait for the warp's next ticket of this segment)
+    if (lane == 0) w.nq = nq;                             // (fewer than 32: they wait for the warp's next ticket of this segment)
     __syncwarp();
 }
 
