@@ -165,8 +165,10 @@ enum { XP_CANCEL_TICKETS = 8192 };
 enum {
     XP_FLAG_NO_FILTER = 1u,             /* skip the probe-point filter stage (every candidate is unranked
                                            and checked on its own); same results, for testing */
-    XP_FLAG_ALWAYS_FILTER = 2u          /* use the filter stage also for rank windows too small to gain
+    XP_FLAG_ALWAYS_FILTER = 2u,         /* use the filter stage also for rank windows too small to gain
                                            from it; same results, for testing */
+    XP_FLAG_ALWAYS_PAIR = 4u            /* index the operands of every block of two larger operands that can be (at most 8
+                                           sketches a call), however small; same results, for testing */
 };
 
 typedef struct xp_grammar xp_grammar;

@@ -512,10 +512,10 @@ struct xp_sketch {
     // if it were the only sketch of the call: built on the first such call and copied, with ticket, sketch
     // and accumulator numbers shifted, into the plan of every later one (a batch of thousands of small
     // sketches would otherwise spend longer planning than some of its searches take).
-    // Two of them, with and without the pair join: each is built once, under the lock, and only read from then on
-    // (calls on several threads copy them at the same time); a refinement, during which no search may run, drops both.
+    // One per form (PlanForm): each is built once, under the lock, and only read from then on
+    // (calls on several threads copy them at the same time); a refinement, during which no search may run, drops them.
     mutable std::mutex plan_mu;
-    mutable std::unique_ptr<const Plan> plan_kept[2];
+    mutable std::unique_ptr<const Plan> plan_kept[4];
 };
 
 // What the load's kernels settled for a hole.
@@ -1298,37 +1298,58 @@ static void add_linear(Plan* plan, int sketch, int hole, int acc, int k, u64 lo,
     plan->n_tickets += (hi - lo + (u64)kLinearChunk - 1) / (u64)kLinearChunk;
 }
 
-constexpr size_t kPairMaxSketches = 8;
-constexpr u64 kPairLeast = 1ull << 20;       // pairs from which an index of one side costs less than a test per pair
+constexpr size_t kPairMaxSketches = 8;       // (each block has scratch of its own: 12 MB for 92 480 operands a side)
 constexpr u64 kPairMost = 1ull << 22;        // operands of either side (the size of the subtree tables)
+// Pairs from which the pair join is taken.  It costs a block some ten launches one after the other, where the tiles of all blocks and
+// sketches are one launch (size 7, tiles / pair join: one sketch 0.15 / 0.16 ms at 2.6e7 pairs a block, 0.39 / 0.25 at 1.3e8;
+// four 0.75 / 0.81 at 1.3e8, 1.67 / 1.36 at 4.2e8).
+constexpr u64 kPairLeast = 1ull << 26, kPairLeastBatch = 1ull << 28;
+constexpr u64 kPairLeastRing = 1ull << 20;   // ... of a nonterminal without / and % there: half the launches (a ragged table, 2.4e6 pairs: 0.36 / 0.34 ms)
+constexpr size_t kPairFew = 2;               // sketches up to which kPairLeast holds
+// A rank window cuts a block to some of its left operands, but the other side is indexed whole: a block with fewer rows than this,
+// or thereabouts, is done as tiles before the index is made (450 000 operands a side, remainders: 2 222 rows 0.26 ms, the index 1.9).
+constexpr u64 kPairEach = 1ull << 12;
+constexpr u64 kRangeMost = 1ull << 18;       // operands of a hole whose context compares from which the tiles take a leaf at the root too
 
-// Does the pair join take the block (production, left size a) of size k?  Both operands tabulated, an operator it knows
-// (products only where neither target is zero: a zero operand would leave its partner open), enough pairs.
+// Does the pair join know the block (production, left size a) of size k?  Both operands tabulated, an operator it has
+// (products only where neither target is zero: a zero operand would leave its partner open).
 static bool pair_joins(const xp_grammar* g, const HoleHost& ho, const BinDev& bd, int a, int k) {
     const int b = k - 1 - a;
     if (!ho.join_on || bd.op > XP_OP_MOD || (bd.op == XP_OP_MUL && ho.target_zero)) return false;
     if (a > ho.tab_max || b > ho.tab_max) return false;
-    const u64 cl = g->cnt[bd.lnt][a], cr = g->cnt[bd.rnt][b];
-    return cl <= kPairMost && cr <= kPairMost && cl * cr >= kPairLeast;
+    return g->cnt[bd.lnt][a] <= kPairMost && g->cnt[bd.rnt][b] <= kPairMost;
 }
 
-// Pair-join blocks of (start nonterminal, size k) that ranks [lo, hi) touch: one per (left, right) operand sets.
-static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi) {
+// Pair-join blocks of (start nonterminal, size k) that ranks [lo, hi) touch: one per (left, right) operand sets.  taken: per
+// production of the nonterminal a bit for every left size whose block is here and not for the tiles.
+static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi, u64 least, std::vector<u32>* taken) {
     const size_t first_seg = plan->psegs.size();
     const int nt = ho.start_nt;
+    taken->assign((size_t)(g->bin_begin[nt + 1] - g->bin_begin[nt]), 0u);
+    bool divides = false;
+    for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
+        const BinDev& bd = g->bins[b];
+        if (bd.op != XP_OP_DIV && bd.op != XP_OP_MOD) continue;
+        for (int a = 2; a < k - 2; ++a) divides = divides || (g->cnt[bd.lnt][a] > 0 && g->cnt[bd.rnt][k - 1 - a] > 0);
+    }
+    if (!divides && least > kPairLeastRing) least = kPairLeastRing;
     for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
         const BinDev& bd = g->bins[b];
         u64 base = bd.off[k];
         for (int a = 1; a <= k - 2; ++a) {
-            const u64 cl = g->cnt[bd.lnt][a], cr = g->cnt[bd.rnt][k - 1 - a];
+            const u64 cl = g->cnt[bd.lnt][a], cr = g->cnt[bd.rnt][k - 1 - a], block = cl * cr;
             const u64 this_base = base;
-            base += cl * cr;
-            if (a == 1 || a == k - 2 || cl * cr == 0 || !pair_joins(g, ho, bd, a, k)) continue;
-            if (this_base + cl * cr <= lo || this_base >= hi) continue;
+            base += block;
+            if (a == 1 || a == k - 2 || block == 0 || !pair_joins(g, ho, bd, a, k)) continue;
+            if (this_base + block <= lo || this_base >= hi) continue;
+            const u64 wlo = lo > this_base ? lo - this_base : 0, whi = hi - this_base < block ? hi - this_base : block;
+            const u64 l0 = wlo / cr, nl = (whi + cr - 1) / cr - l0;      // left operands that the window covers
+            if (nl * cr < least || (least > 1 && nl < cl && nl * cr < kPairEach * (nl + cr))) continue;
+            taken->at(b - g->bin_begin[nt]) |= 1u << a;
             PairSeg* sg = nullptr;
             for (size_t i = first_seg; i < plan->psegs.size() && !sg; ++i) {
                 PairSeg& c = plan->psegs[i];
-                if (c.lnt == bd.lnt && c.rnt == bd.rnt && c.la == a && !((c.ops >> bd.op) & 1u)) sg = &c;
+                if (c.lnt == bd.lnt && c.rnt == bd.rnt && c.la == a && c.l_begin == l0 && c.nl == nl && !((c.ops >> bd.op) & 1u)) sg = &c;
             }
             if (!sg) {
                 PairSeg c;
@@ -1336,8 +1357,8 @@ static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
                 c.rank_begin = lo; c.rank_end = hi;
                 c.sketch = sketch; c.hole = hole; c.size = k; c.acc = acc;
                 c.lnt = bd.lnt; c.la = a; c.rnt = bd.rnt; c.ra = k - 1 - a;
-                c.nl = (u32)cl; c.nr = (u32)cr;
-                c.index_right = cr <= cl ? 1 : 0;            // the smaller side is indexed (its chains stay in L2)
+                c.l_begin = (u32)l0; c.nl = (u32)nl; c.nr = (u32)cr;
+                c.index_right = cr <= nl ? 1 : 0;            // the smaller side is indexed (its chains stay in L2)
                 u32 heads = 1024;
                 while (heads < (c.index_right ? c.nr : c.nl)) heads <<= 1;
                 c.head_mask = heads - 1;
@@ -1346,16 +1367,19 @@ static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
                 sg = &plan->psegs.back();
             }
             sg->ops |= 1u << bd.op;
-            sg->base[bd.op] = this_base;
+            sg->base[bd.op] = this_base + l0 * cr;
         }
     }
 }
 
 constexpr u64 kFamilyMaxWork = 512;          // candidates per register operand below which segments share a fill
+constexpr u64 kTileTickets = 148;            // tickets that a segment of a small call is cut into, if it has the operands
 
 // Tile segments of (start nonterminal, size k) restricted to ranks [lo, hi): one per
 // (left size, group of productions with the same operand nonterminals and the same rows).
-static void add_tiles(Plan* plan, const xp_grammar* g, const HoleHost* pairs, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, int bc_tile) {
+// taken: blocks that the pair join has (null: none); few: the call has so few sketches that a ticket for every SM is wanted;
+// leaves: blocks with a leaf as an operand too.
+static void add_tiles(Plan* plan, const xp_grammar* g, const std::vector<u32>* taken, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, int bc_tile, bool few, bool leaves) {
     const size_t first_seg = plan->segs.size();
     for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
         const BinDev& bd = g->bins[b];
@@ -1366,8 +1390,8 @@ static void add_tiles(Plan* plan, const xp_grammar* g, const HoleHost* pairs, in
             if (block == 0) continue;
             const u64 this_base = base;
             base += block;
-            if (a == 1 || a == k - 2) continue;              // (a leaf at the root: add_joins)
-            if (pairs && pair_joins(g, *pairs, bd, a, k)) continue;      // (add_pairs)
+            if ((a == 1 || a == k - 2) && !leaves) continue; // (a leaf at the root: add_joins)
+            if (taken && ((taken->at(b - g->bin_begin[nt]) >> a) & 1u)) continue;      // (add_pairs)
             if (this_base + block <= lo || this_base >= hi) continue;
             const u64 wlo = lo > this_base ? lo - this_base : 0;
             const u64 whi = hi - this_base < block ? hi - this_base : block;
@@ -1407,6 +1431,17 @@ static void add_tiles(Plan* plan, const xp_grammar* g, const HoleHost* pairs, in
             if (bd.op == XP_OP_SHL || bd.op == XP_OP_SHR) sg->generic = 1;
         }
     }
+    // A small segment of a small call: narrower broadcast tiles, until there are as many tickets as SMs.  (Its few tickets ran on as many
+    // SMs: four sketches of 12 leaves, size 7, 0.28 -> 0.12 ms; one of 5 leaves, size 9, where most of a tile hits, 1.86 -> 0.65.)
+    if (few)
+        for (size_t i = first_seg; i < plan->segs.size(); ++i) {
+            SegDev& c = plan->segs[i];
+            if ((u64)c.reg_tiles * c.bc_tiles >= kTileTickets || c.bc_count * (u64)c.n_ops < kFamilyMaxWork) continue;
+            const u64 share = (c.bc_count * c.reg_tiles + kTileTickets - 1) / kTileTickets, tile = (share + 15) & ~15ull;
+            if (tile >= (u64)c.bc_tile) continue;
+            c.bc_tile = (i32)tile;
+            c.bc_tiles = (u32)((c.bc_count + tile - 1) / tile);
+        }
     // Families: segments with the same register-side operands and a single broadcast tile are
     // put next to each other; the first takes the tickets (one per register tile) and visits
     // the others, so the register operands are fetched once for all of them.
@@ -1573,7 +1608,10 @@ static void number_joins(Plan* plan) {
 
 constexpr u64 kTileMinRanks = 4096;          // smaller windows are searched rank by rank
 
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, bool pairs, Plan* plan);
+// What a plan may use: kFormMany, a batch: no pair join; the others, at most kPairMaxSketches sketches: narrow tiles where a block is small, and
+// without the pair join, with it from kPairLeastBatch pairs on, or from kPairLeast on.
+enum PlanForm { kFormMany = 0, kFormTiles = 1, kFormPairsSome = 2, kFormPairs = 3 };
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, Plan* plan);
 
 // A sketch's tables, and the library's scratch, live on the device that was current when the sketch was
 // loaded: a call made with another device current would hand the kernels pointers of the wrong GPU.
@@ -1592,20 +1630,21 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
     // the pair join takes its blocks one after the other, several launches each: a batch keeps to the tiles, which
     // search all holes in one launch.  So does a call with a cancel word or a time limit: its launches are bounded, and the
     // host looks at both between them; a pair join's launch covers a whole block.
-    const bool pairs = may_pair && n <= kPairMaxSketches && !o->cancel && o->timeout_ms <= 0;
+    const bool pairs = may_pair && !o->cancel && o->timeout_ms <= 0;
+    const PlanForm form = n > kPairMaxSketches ? kFormMany : !pairs ? kFormTiles : n > kPairFew ? kFormPairsSome : kFormPairs;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
         if (!s) return fail(XP_ERR_INVALID_ARG, "null sketch in batch");
-        if (!plain) { plan_sketch(s, i, o, pairs, plan); continue; }
+        if (!plain) { plan_sketch(s, i, o, form, plan); continue; }
         const Plan* own;
         {
             std::lock_guard<std::mutex> lock(s->plan_mu);
-            std::unique_ptr<const Plan>& kept = s->plan_kept[pairs ? 1 : 0];
+            std::unique_ptr<const Plan>& kept = s->plan_kept[form];
             if (!kept) {
                 std::unique_ptr<Plan> made(new Plan);
-                plan_sketch(s, 0, o, pairs, made.get());
+                plan_sketch(s, 0, o, form, made.get());
                 made->acc.clear();                        // (made per call, below)
                 kept = std::move(made);
             }
@@ -1639,7 +1678,8 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
 }
 
 // One sketch's segments, accumulators and tickets, appended to the plan as sketch number i.
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, bool pairs, Plan* plan) {
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, Plan* plan) {
+    std::vector<u32> taken;
     {
         for (int h = 0; h < s->n_holes; ++h) {
             const HoleHost& ho = s->holes[h];
@@ -1665,9 +1705,13 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, b
                 const bool forced = (o->flags & XP_FLAG_ALWAYS_FILTER) != 0;
                 if (!ho.filter_ok || (o->flags & XP_FLAG_NO_FILTER)) { add_linear(plan, (int)i, h, acc, k, lo, hi); continue; }
                 if (k < 3 || (!forced && hi - lo < kTileMinRanks)) { add_direct(plan, ho.start_nt, (int)i, h, acc, k, lo, hi); continue; }
-                add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact, ho.compares);
-                if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi);
-                add_tiles(plan, s->g, pairs ? &ho : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile);
+                // (A range of hole values: the join's interval arithmetic per operand against a test per candidate.  27 leaves, size 7, 984 000
+                // operands, four specs: 13.4, 26.5, 10.2, 14.4 ms by the join, 14.9, 19.8, 10.7, 8.2 as tiles; 40 leaves, size 5: 0.4 against 1.4.)
+                const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
+                if (!leaves) add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact, ho.compares);
+                const bool pairs = form >= kFormPairsSome;
+                if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
+                add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany, leaves);
             }
         }
     }

@@ -275,10 +275,10 @@ struct PairSeg {
     u64 rank_begin, rank_end;        // window of ranks searched at this size
     i32 sketch, hole, size, acc;
     i32 lnt, la, rnt, ra;            // nonterminal and size of either operand
-    u32 nl, nr;                      // operands
+    u32 l_begin, nl, nr;             // first of the left operands (a rank window may leave some out), and how many there are
     u32 ops;                         // operator slots (+ - * / %)
     i32 index_right;                 // the chains index the right operands (else the left ones)
-    u64 base[5];                     // rank of (0, 0) per operator
+    u64 base[5];                     // rank of (l_begin, 0) per operator
     u32 head_mask, far_pieces;       // far_pieces: long pieces that a walk lists at most (pair_pieces)
     // device scratch of the call
     u32* head;                       // head_mask + 1, all ones at launch

@@ -24,13 +24,16 @@ struct PairWarp {
     CandShared cand;
 };
 
+// Table entry of the first left operand.
+__device__ __forceinline__ u64 pair_left(const HoleDev* hole, const PairSeg& seg) { return hole->tab_off[seg.lnt][seg.la] + seg.l_begin; }
+
 // The lane's candidate against the queue's remaining probes.  Called by all lanes.
 __device__ __noinline__ void pair_check(PairWarp& w, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, int from, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
     __syncwarp();
     const u32 nc = w.nc;
-    const u64 lo = hole->tab_off[seg.lnt][seg.la], ro = hole->tab_off[seg.rnt][seg.ra];
+    const u64 lo = pair_left(hole, seg), ro = hole->tab_off[seg.rnt][seg.ra];
     for (u32 at = 0; at < nc; at += 32) {
         bool pass = false;
         u64 rank = 0;
@@ -118,7 +121,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const __grid_c
         const u32 n = side ? seg.nr : seg.nl;
         if (i >= n) continue;
         int2 v;
-        const int st = pair_entry(hole, side ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la], i, lim, v);
+        const int st = pair_entry(hole, side ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg), i, lim, v);
         if (st == 2) (side ? seg.wide_r : seg.wide_l)[atomicAdd(&seg.counters[side], 1u)] = i;
         if (side == seg.index_right && st == 1) seg.next[i] = atomicExch(&seg.head[pair_slot(v, seg.head_mask)], i);
     }
@@ -138,8 +141,8 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const __grid
     JoinCount n{0, 0, 0, 0, 0};
     const bool ir = seg.index_right != 0;
     const u32 nx = ir ? seg.nl : seg.nr;
-    const u64 xo = ir ? hole->tab_off[seg.lnt][seg.la] : hole->tab_off[seg.rnt][seg.ra];
-    const u64 yo = ir ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la];
+    const u64 xo = ir ? pair_left(hole, seg) : hole->tab_off[seg.rnt][seg.ra];
+    const u64 yo = ir ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg);
     const int2* Y = reinterpret_cast<const int2*>(hole->tab_pair) + yo;
     const u32 lim = pair_limit(hole);
     const i64 t0 = hole->join_t0, t1 = hole->join_t1;
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const __g
     const int side = blockIdx.y;
     const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
     const u32 n = side ? seg.nr : seg.nl, lim = pair_limit(hole);
-    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la];
+    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg);
     for (int b = threadIdx.x; b < kPairBuckets; b += kPairThreads) hist[b] = 0;
     __syncthreads();
     for (u32 i = blockIdx.x * kPairThreads + threadIdx.x; i < n; i += gridDim.x * kPairThreads) {
@@ -237,7 +240,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const _
     const int side = blockIdx.y, lane = threadIdx.x & 31;
     const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
     const u32 n = side ? seg.nr : seg.nl, lim = pair_limit(hole);
-    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : hole->tab_off[seg.lnt][seg.la];
+    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg);
     for (u32 i0 = (blockIdx.x * kPairThreads + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * kPairThreads) {
         const u32 i = i0 + lane;
         int2 v = make_int2(0, 0);
@@ -399,7 +402,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_wide_kernel(const __grid_co
     const SketchDev* sk = plan.sketches[seg.sketch];
     const HoleDev* hole = &sk->holes[seg.hole];
     const u32 lim = pair_limit(hole);
-    const u64 lo = hole->tab_off[seg.lnt][seg.la], ro = hole->tab_off[seg.rnt][seg.ra];
+    const u64 lo = pair_left(hole, seg), ro = hole->tab_off[seg.rnt][seg.ra];
     JoinCount n{0, 0, 0, 0, 0};
     const u64 nl = wl, total = nl + wr;
     for (u64 i = blockIdx.x * kPairWarps + (threadIdx.x >> 5); i < total; i += (u64)gridDim.x * kPairWarps) {

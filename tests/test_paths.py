@@ -328,16 +328,17 @@ def test_a_workspace_made_before_a_refinement(xp):
     spec[100:106] = 5
     sk = Sketch(g, [Hole(0, 7, spec_table=spec)], coords)
     ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
-    need = xp.xp_workspace_bytes([ls])
+    flag = dict(flags=xp.XP_FLAG_ALWAYS_PAIR)                          # (a block this small goes to the tiles)
+    need = xp.xp_workspace_bytes([ls], **flag)
     ws = torch.empty(need, dtype=torch.uint8, device="cuda")
-    before = xp.xp_repair(ls, workspace=ws)[0]
+    before = xp.xp_repair(ls, workspace=ws, **flag)[0]
     assert before.probe_survivors > 0 and xp.xp_sketch_refine(ls) >= 1
-    assert xp.xp_workspace_bytes([ls]) > need                           # (or this test does not test what it says)
-    assert_same(xp.xp_repair(ls, workspace=ws)[0], before)
-    assert_same(xp.xp_repair(ls)[0], before)
-    assert_same(xp.xp_repair(ls, workspace=ws[:need - 40 * (2**20 - 65536)])[0], before)      # (with the shortest survivor queue)
+    assert xp.xp_workspace_bytes([ls], **flag) > need                           # (or this test does not test what it says)
+    assert_same(xp.xp_repair(ls, workspace=ws, **flag)[0], before)
+    assert_same(xp.xp_repair(ls, **flag)[0], before)
+    assert_same(xp.xp_repair(ls, workspace=ws[:need - 40 * (2**20 - 65536)], **flag)[0], before)      # (with the shortest survivor queue)
     with pytest.raises(xp.XpError) as e:                                # too small for any plan: refused as ever
-        xp.xp_repair(ls, workspace=ws[:1 << 20])
+        xp.xp_repair(ls, workspace=ws[:1 << 20], **flag)
     assert e.value.status == 5
 
 
@@ -429,3 +430,33 @@ def test_more_survivors_than_the_queue_of_a_small_workspace_holds(xp):
     with pytest.raises(xp.XpError) as e:
         xp.xp_repair(ls, workspace=ws[:small - 256])
     assert e.value.status == 5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("spec", ["(i*3)+(j*2)", "(i+2)*(j-1)", "(i*5)/(j+4)", "(i+j)%(j+5)", "j-j", "(i*1048576)*(j*65536)"])
+def test_indexed_operands_in_rank_windows(xp, spec):
+    """The pair join of blocks that a window cuts to some of their left operands, small ones too."""
+    g = free_grammar(IJ, list(range(0, 12)) + [65536])
+    sk = Sketch(g, [Hole(0, 7, spec_expr=parse_expr(spec, IJ))], name=spec)
+    n = oracle.counts(g, 0, 7)
+    flag = dict(flags=xp.XP_FLAG_ALWAYS_PAIR)
+    per, mid = n[7] // 5, n[1] * n[5]                                   # a production's first pair of two operands of three nodes
+    for p in range(5):
+        at = p * per + mid
+        check_sketch(xp, sk, windows={7: (at + 5 * n[3] + 17, at + 9 * n[3] + 3), 5: (3, 40_000)}, **flag)
+    check_sketch(xp, sk, windows={7: (per + mid + 1000 * n[3] + 5, 2 * per + mid + 100 * n[3])}, **flag)      # ends of one block, starts of the next
+    check_sketch(xp, sk, windows={7: (0, 100_000)}, **flag)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ctx,spec", [("j<HOLE", "i*2"), ("HOLE<=(i-j)", "(i%7)-3"), ("(j-HOLE)<4", "i/3")])
+def test_many_operands_under_a_comparison(xp, ctx, spec):
+    """Operand tiles with a leaf on either side, for a hole whose context compares."""
+    g = free_grammar(IJ, list(range(-6, 11)))
+    sk = Sketch(g, [Hole(0, 7, ctx=parse_expr(ctx, IJ), spec_expr=parse_expr(ctx.replace("HOLE", f"({spec})"), IJ))], name=ctx)
+    n = oracle.counts(g, 0, 7)
+    assert n[5] > 2**18
+    for p in range(5):
+        at = p * (n[7] // 5)
+        check_sketch(xp, sk, windows={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: (at + 7, at + 100_000)})
+    check_sketch(xp, sk, windows={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: (n[7] - 100_000, n[7])})
