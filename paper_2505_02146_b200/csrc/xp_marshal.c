@@ -23,7 +23,7 @@
 
 static PyObject *s_variables, *s_name, *s_lo, *s_hi, *s_n_nonterminals, *s_productions, *s_lhs, *s_kind, *s_var, *s_op, *s_left, *s_right, *s_value,
     *s_holes, *s_coords, *s_start_nt, *s_max_size, *s_ctx, *s_spec_expr, *s_spec_table, *s_data_ptr, *s_is_cuda, *s_shape,
-    *s_own, *s_handle, *s_model, *s_grammar, *s_n_holes, *s_keep;
+    *s_dtype, *s_own, *s_handle, *s_model, *s_grammar, *s_n_holes, *s_keep;
 
 /* What a marshalled description owns: one block of memory and a list of the objects it points into. */
 typedef struct { PyObject_HEAD void* mem; PyObject* held; } Owner;
@@ -52,22 +52,39 @@ static Owner* new_owner(size_t bytes) {
     return o;
 }
 
-/* obj.name as an integer; -1 with an exception set on failure. */
-static long long int_attr(PyObject* obj, PyObject* name) {
-    PyObject* v = PyObject_GetAttr(obj, name);
-    if (!v) return -1;
-    const long long r = PyLong_AsLongLong(v);
-    if (r == -1 && PyErr_Occurred() && PyErr_ExceptionMatches(PyExc_TypeError)) {      /* numpy integers and the like */
-        PyErr_Clear();
-        PyObject* w = PyNumber_Long(v);
-        Py_DECREF(v);
-        if (!w) return -1;
-        const long long q = PyLong_AsLongLong(w);
-        Py_DECREF(w);
-        return q;
+/* An integer (int, numpy integer, anything with __index__; no floats, no texts) between -2^63 and 2^64 - 1 as 64 bits: an unsigned
+ * constant wraps, as it does in the C structures.  Returns -1 with an exception set on failure. */
+static inline int as_int64(PyObject* v, long long* out) {
+    if (PyLong_CheckExact(v)) {
+        int over = 0;
+        *out = PyLong_AsLongLongAndOverflow(v, &over);
+        if (over == 0) return 0;
     }
-    Py_DECREF(v);
-    return r;
+    PyObject* i = PyNumber_Index(v);
+    if (!i) return -1;
+    int over = 0;
+    long long r = PyLong_AsLongLongAndOverflow(i, &over);
+    if (over > 0) r = (long long)PyLong_AsUnsignedLongLong(i);
+    else if (over < 0) PyErr_SetString(PyExc_OverflowError, "an integer below -2^63");
+    Py_DECREF(i);
+    *out = r;
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+static inline int get_int64(PyObject* obj, PyObject* name, int64_t* out) {
+    PyObject* v = PyObject_GetAttr(obj, name);
+    long long r = 0;
+    const int rc = v ? as_int64(v, &r) : -1;
+    Py_XDECREF(v);
+    *out = r;
+    return rc;
+}
+
+static inline int get_int32(PyObject* obj, PyObject* name, int32_t* out) {      /* (the low 32 bits: as the C structures take an int) */
+    int64_t r = 0;
+    const int rc = get_int64(obj, name, &r);
+    *out = (int32_t)r;
+    return rc;
 }
 
 static int fill_instrs(PyObject* seq, xp_instr* out, Py_ssize_t n) {
@@ -79,14 +96,11 @@ static int fill_instrs(PyObject* seq, xp_instr* out, Py_ssize_t n) {
             PyErr_SetString(PyExc_ValueError, "an instruction is a (kind, arg, value) tuple");
             return -1;
         }
-        long long v[3];
-        for (int k = 0; k < 3; ++k) {
-            PyObject* x = PyNumber_Index(PySequence_Fast_GET_ITEM(t, k));
-            v[k] = x ? PyLong_AsLongLong(x) : -1;
-            Py_XDECREF(x);
-        }
+        long long v[3] = {0, 0, 0};
+        int rc = 0;
+        for (int k = 0; k < 3 && rc == 0; ++k) rc = as_int64(PySequence_Fast_GET_ITEM(t, k), &v[k]);
         Py_DECREF(t);
-        if (PyErr_Occurred()) return -1;
+        if (rc < 0) return -1;
         out[i].kind = (int32_t)v[0];
         out[i].arg = (int32_t)v[1];
         out[i].value = v[2];
@@ -137,7 +151,7 @@ static int fill_grammar(PyObject* g, const GrammarLists* l, void* mem, PyObject*
     *names_out = names;
     d->n_vars = (int32_t)l->nv;
     d->vars = v;
-    d->n_nonterminals = (int32_t)int_attr(g, s_n_nonterminals);
+    if (get_int32(g, s_n_nonterminals, &d->n_nonterminals) < 0) return -1;
     d->n_productions = (int32_t)l->np;
     d->productions = p;
     for (Py_ssize_t i = 0; i < l->nv; ++i) {
@@ -145,22 +159,17 @@ static int fill_grammar(PyObject* g, const GrammarLists* l, void* mem, PyObject*
         names[i] = PyObject_GetAttr(x, s_name);
         if (names[i] && !PyUnicode_Check(names[i])) PyErr_SetString(PyExc_TypeError, "a variable's name is a string");
         v[i].name = names[i] && PyUnicode_Check(names[i]) ? PyUnicode_AsUTF8(names[i]) : NULL;
-        if (!v[i].name) return -1;
-        v[i].lo = int_attr(x, s_lo);
-        v[i].hi = int_attr(x, s_hi);
+        if (!v[i].name || get_int64(x, s_lo, &v[i].lo) < 0 || get_int64(x, s_hi, &v[i].hi) < 0) return -1;
     }
     for (Py_ssize_t i = 0; i < l->np; ++i) {
         PyObject* x = PySequence_Fast_GET_ITEM(l->prods, i);
-        const int32_t kind = (int32_t)int_attr(x, s_kind);
-        p[i].kind = kind;
-        p[i].lhs = (int32_t)int_attr(x, s_lhs);
-        if (kind == XP_PROD_CONST) { p[i].value = int_attr(x, s_value); continue; }      /* (each kind reads its own fields) */
-        if (kind == XP_PROD_VAR) { p[i].var = (int32_t)int_attr(x, s_var); continue; }
-        p[i].op = (int32_t)int_attr(x, s_op);
-        p[i].left = (int32_t)int_attr(x, s_left);
-        p[i].right = (int32_t)int_attr(x, s_right);
+        if (get_int32(x, s_kind, &p[i].kind) < 0 || get_int32(x, s_lhs, &p[i].lhs) < 0) return -1;
+        const int rc = p[i].kind == XP_PROD_CONST ? get_int64(x, s_value, &p[i].value)      /* (each kind reads its own fields) */
+                     : p[i].kind == XP_PROD_VAR ? get_int32(x, s_var, &p[i].var)
+                     : get_int32(x, s_op, &p[i].op) < 0 || get_int32(x, s_left, &p[i].left) < 0 ? -1 : get_int32(x, s_right, &p[i].right);
+        if (rc < 0) return -1;
     }
-    return PyErr_Occurred() ? -1 : 0;
+    return 0;
 }
 
 static PyObject* m_grammar(PyObject* self, PyObject* g) {
@@ -255,7 +264,10 @@ static PyObject* m_grammar_create(PyObject* self, PyObject* args) {
         else {
             void* at = NULL;
             if (fill_grammar(g, &l, mem, &names) == 0) {
-                const int st = ((int (*)(const xp_grammar_desc*, void**))(size_t)create)((const xp_grammar_desc*)mem, &at);
+                int st;
+                Py_BEGIN_ALLOW_THREADS                   /* (what `mem` points into is held by `names`) */
+                st = ((int (*)(const xp_grammar_desc*, void**))(size_t)create)((const xp_grammar_desc*)mem, &at);
+                Py_END_ALLOW_THREADS
                 if (st != 0) ret = PyLong_FromLong(st);
                 else {
                     ret = owning(cls, destroy, at);
@@ -318,7 +330,9 @@ static PyObject* m_free_all(PyObject* self, PyObject* args) {
 static int array_at(PyObject* a, Py_ssize_t itemsize, PyObject* conv, const void** ptr, int32_t* on_device, long long* rows, PyObject** held) {
     Py_buffer b;
     *on_device = 0;
-    if (PyObject_CheckBuffer(a)) {
+    static PyTypeObject* array_type = NULL;              /* the type seen last that is an array and not just any buffer */
+    if (Py_TYPE(a) != array_type && PyObject_CheckBuffer(a) && PyObject_HasAttr(a, s_dtype)) array_type = (PyTypeObject*)Py_NewRef(Py_TYPE(a));
+    if (Py_TYPE(a) == array_type) {
         Py_INCREF(a);
         for (int tries = 0; tries < 2; ++tries) {
             if (PyObject_GetBuffer(a, &b, PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) == 0) {
@@ -364,10 +378,10 @@ static int array_at(PyObject* a, Py_ssize_t itemsize, PyObject* conv, const void
     return 0;
 }
 
-static PyObject* get_list(PyObject* obj, PyObject* name) {       /* obj.name as a fast sequence (None: empty) */
+static PyObject* get_list(PyObject* obj, PyObject* name, int may_be_none) {       /* obj.name as a fast sequence (None, where it may be: empty) */
     PyObject* v = PyObject_GetAttr(obj, name);
     if (!v) return NULL;
-    if (v == Py_None) {
+    if (v == Py_None && may_be_none) {
         Py_DECREF(v);
         return PyList_New(0);
     }
@@ -388,13 +402,13 @@ static PyObject* m_sketches(PyObject* self, PyObject* args) {
     /* first walk: how many holes and instructions */
     size_t n_holes = 0, n_instr = 0;
     for (Py_ssize_t i = 0; i < n; ++i) {
-        PyObject* holes = get_list(PySequence_Fast_GET_ITEM(seq, i), s_holes);
+        PyObject* holes = get_list(PySequence_Fast_GET_ITEM(seq, i), s_holes, 0);
         if (!holes) goto done;
         const Py_ssize_t nh = PySequence_Fast_GET_SIZE(holes);
         n_holes += (size_t)nh;
         for (Py_ssize_t h = 0; h < nh; ++h)
             for (int k = 0; k < 2; ++k) {
-                PyObject* c = get_list(PySequence_Fast_GET_ITEM(holes, h), k ? s_spec_expr : s_ctx);
+                PyObject* c = get_list(PySequence_Fast_GET_ITEM(holes, h), k ? s_spec_expr : s_ctx, k);
                 if (!c) { Py_DECREF(holes); goto done; }
                 n_instr += (size_t)PySequence_Fast_GET_SIZE(c);
                 Py_DECREF(c);
@@ -414,7 +428,7 @@ static PyObject* m_sketches(PyObject* self, PyObject* args) {
         PyObject* dev = PyList_New(0);
         if (!dev) goto done;
         PyList_SET_ITEM(devs, i, dev);
-        PyObject* holes = get_list(sk, s_holes);
+        PyObject* holes = get_list(sk, s_holes, 0);
         if (!holes) goto done;
         const Py_ssize_t nh = PySequence_Fast_GET_SIZE(holes);
         PyList_SET_ITEM(nhs, i, PyLong_FromSsize_t(nh));
@@ -423,8 +437,7 @@ static PyObject* m_sketches(PyObject* self, PyObject* args) {
         int bad = 0;
         for (Py_ssize_t h = 0; h < nh && !bad; ++h, ++hd) {
             PyObject* ho = PySequence_Fast_GET_ITEM(holes, h);
-            hd->start_nt = (int32_t)int_attr(ho, s_start_nt);
-            hd->max_size = (int32_t)int_attr(ho, s_max_size);
+            if (get_int32(ho, s_start_nt, &hd->start_nt) < 0 || get_int32(ho, s_max_size, &hd->max_size) < 0) { bad = 1; break; }
             PyObject* table = NULL;
             if (specs_arg != Py_None) {
                 PyObject* key = PyLong_FromSsize_t(h);
@@ -436,7 +449,7 @@ static PyObject* m_sketches(PyObject* self, PyObject* args) {
             if (!table) { bad = 1; break; }
             for (int k = 0; k < 2 && !bad; ++k) {
                 if (k == 1 && table != Py_None) break;   /* a table: the expression is not looked at */
-                PyObject* c = get_list(ho, k ? s_spec_expr : s_ctx);
+                PyObject* c = get_list(ho, k ? s_spec_expr : s_ctx, 0);
                 const Py_ssize_t len = c ? PySequence_Fast_GET_SIZE(c) : 0;
                 if (!c || len > code_end - code || fill_instrs(c, code, len) < 0) bad = 1;
                 else if (k) { hd->spec_kind = XP_SPEC_EXPR; hd->spec_len = (int32_t)len; hd->spec_expr = code; }
@@ -557,7 +570,7 @@ PyMODINIT_FUNC PyInit__marshal(void) {
         {&s_productions, "productions"}, {&s_lhs, "lhs"}, {&s_kind, "kind"}, {&s_var, "var"}, {&s_op, "op"}, {&s_left, "left"},
         {&s_right, "right"}, {&s_value, "value"}, {&s_holes, "holes"}, {&s_coords, "coords"}, {&s_start_nt, "start_nt"},
         {&s_max_size, "max_size"}, {&s_ctx, "ctx"}, {&s_spec_expr, "spec_expr"}, {&s_spec_table, "spec_table"},
-        {&s_data_ptr, "data_ptr"}, {&s_is_cuda, "is_cuda"}, {&s_shape, "shape"}, {&s_own, "_own"},
+        {&s_data_ptr, "data_ptr"}, {&s_is_cuda, "is_cuda"}, {&s_shape, "shape"}, {&s_dtype, "dtype"}, {&s_own, "_own"},
         {&s_handle, "handle"}, {&s_model, "model"}, {&s_grammar, "grammar"}, {&s_n_holes, "n_holes"}, {&s_keep, "_keep"}};
     for (size_t i = 0; i < sizeof(names) / sizeof(names[0]); ++i) {
         *names[i].to = PyUnicode_InternFromString(names[i].name);

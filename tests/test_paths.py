@@ -139,6 +139,33 @@ def test_batch_load_in_pieces(xp, n):
         assert_same(got[k][0], oracle.repair_hole(sks[k]), f"sketch {k}")
 
 
+def test_integers_of_descriptors():
+    """What the C structures take as an integer: no float, no text, unsigned 64-bit constants by their bits; and the first error is the one reported."""
+    import array
+    from paper_2505_02146_b200 import binding as B
+    from xp_instances.model import Grammar, Production
+    B.load()
+    vs = [Variable("i", 0, 9)]
+    big = free_grammar(vs, [2**63, 2**64 - 1, -2**63])
+    d = B.marshal_grammar(big).desc
+    assert [d.productions[k].value for k in (1, 2, 3)] == [-2**63, -1, -2**63]
+    ok = [Production(0, 0, var=0), Production(0, 1, value=3)]
+    for variables, prods in (([Variable("i", 0.0, 9)], ok), ([Variable("i", 0, "9")], ok), ([Variable("i", 0, 2.5)], ok), (vs, [Production(0, 1, value=1.5)]),
+                             (vs, [Production(0, 1, value="7")]), (vs, [Production(0.0, 0)]), (vs, [Production(0, 0, var="0")]), (vs, [Production(0, 2, op=None)])):
+        with pytest.raises(TypeError):
+            B.marshal_grammar(Grammar(variables, 1, prods))
+    with pytest.raises(OverflowError):
+        B.marshal_grammar(free_grammar(vs, [2**64]))
+    with pytest.raises(AttributeError, match="lo"):                     # (not a later one)
+        B.marshal_grammar(Grammar([type("V", (), {"name": "i"})()], 1, [object()]))
+    g = free_grammar(vs, [1])
+    rows = np.zeros((3, 1), dtype=np.int32)
+    for hole, coords in ((Hole(0, 3, ctx=None, spec_expr=parse_expr("i", vs)), None), (Hole(0, 3), None), (Hole(0, 3.0, spec_expr=parse_expr("i", vs)), None),
+                         (Hole(0, 3, spec_table=array.array("q", [1, 2, 3])), rows), (Hole(0, 3, spec_expr=[(1, 0, 1.0)]), None)):
+        with pytest.raises((TypeError, AttributeError)):
+            B.marshal_sketches([Sketch(g, [hole], coords)])
+
+
 @pytest.mark.parametrize("bad", ["kind", "pair", "value", "attr"])
 def test_descriptors_from_models(bad):
     """Integers of any kind, arrays of other types and strides, and what is refused."""
