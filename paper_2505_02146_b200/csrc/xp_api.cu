@@ -6,6 +6,7 @@
 #include <atomic>
 #include <climits>
 #include <chrono>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -14,6 +15,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -222,6 +224,7 @@ struct xp_grammar {
     GrammarDev* d_g = nullptr;       // one block: header, leaves, binary productions
     size_t d_bytes = 0;
     int d_device = 0;
+    bool d_pending = false;          // some load has taken the block and not yet queued the tables (under g_load_mu)
 };
 
 // cnt[nt][s] by the recurrence over productions and left sizes; off[s] of a binary production
@@ -444,7 +447,7 @@ static void grammar_image(const xp_grammar* g, char* out) {
 }
 
 // Device memory for a grammar's tables, on first use; *fresh: the caller has to send the image.
-// (Loads hold g_load_mu: nobody else sees a block whose image has not been queued.)
+// (Under g_load_mu; a grammar whose block another load has taken and not yet filled is waited for before.)
 static xp_status grammar_block(xp_grammar* g, bool* fresh) {
     *fresh = false;
     if (g->d_g) {
@@ -595,6 +598,7 @@ struct LoadState {
     size_t off_coords = 0, head = 0;         // [0, head) of the block is staged on the host
     bool copy_coords = false, stage = false, stage_box = false;
     bool grammar_fresh = false;              // this sketch's load sends its grammar's tables
+    i64 n_points = 0;
     size_t grammar_bytes = 0;
     size_t stage_at = 0;                     // where its part of the staged copy starts (head, then the grammar's tables)
     size_t piece = 0;
@@ -709,10 +713,9 @@ static u32 constraint_vars(const xp_hole_desc& hd, int n_vars, i64 n_points) {
     return fv & (poly_vars(A, atoms) | poly_vars(D, atoms) | atoms.may_fail);
 }
 
-// First part of a load: checks the description, lays out and allocates the sketch's device block.
-static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadState* L) {
-    if (!gc || !d) return fail(XP_ERR_INVALID_ARG, "xp_sketch_load: null argument");
-    xp_grammar* g = const_cast<xp_grammar*>(gc);
+// First part of a load: checks the description.
+static xp_status load_check(const xp_grammar* g, const xp_sketch_desc* d, LoadState* L) {
+    if (!g || !d) return fail(XP_ERR_INVALID_ARG, "xp_sketch_load: null argument");
     if (d->n_holes < 1 || !d->holes) return fail(XP_ERR_SKETCH, "a sketch needs at least one hole");
     if (d->domain_kind != XP_DOMAIN_BOX && d->domain_kind != XP_DOMAIN_TABLE) return fail(XP_ERR_SKETCH, "bad domain_kind");
     const int nv = g->n_vars;
@@ -740,10 +743,15 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             if (n_points > 0 && !hd.spec_table) return fail(XP_ERR_SKETCH, "spec table is null");
         } else return fail(XP_ERR_SKETCH, "bad spec_kind");
     }
-    const xp_status st = grammar_block(g, &L->grammar_fresh);
-    if (st != XP_OK) return st;
-    if (L->grammar_fresh) L->grammar_bytes = grammar_layout(g).total;
+    L->n_points = n_points;
+    return XP_OK;
+}
 
+// Second part: lays out and allocates the sketch's device block.
+static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadState* L) {
+    xp_grammar* g = const_cast<xp_grammar*>(gc);
+    const int nv = g->n_vars;
+    const i64 n_points = L->n_points;
     xp_sketch* s = new (std::nothrow) xp_sketch;
     if (!s) return fail(XP_ERR_NOMEM, "out of host memory");
     s->g = g; s->n_holes = d->n_holes; s->n_points = n_points;
@@ -905,7 +913,7 @@ static void sketch_image(const LoadState* L, SketchDev* out) {
     hs.n_samples = ns;
 }
 
-// Second part: the sketch's share of the staged copy (its head, then its grammar's tables when they are new).
+// Third part: the sketch's share of the staged copy (its head, then its grammar's tables when they are new).
 static void load_fill(const LoadState* L, char* stg) {
     const xp_sketch* s = L->s;
     const xp_sketch_desc* d = L->d;
@@ -933,30 +941,41 @@ static cudaError_t make_tables(const LoadJob* jobs, int n_jobs, int size_cap, in
     return e;
 }
 
-// One load at a time: all of them work on the default stream anyway, and a grammar's tables are sent by the first
-// load that needs them.
+// Loads of several threads run side by side (their kernels follow one another on the default stream).  A grammar's tables are sent by
+// the first load that needs them, and others may queue kernels that read them once that copy has been queued: a load takes the
+// blocks of all its new grammars at one time, when no grammar of its list is on its way in another load, and waits for that
+// holding none.
 static std::mutex g_load_mu;
+static std::condition_variable g_load_cv;
+static std::mutex g_fill_mu;
 
 extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, const xp_sketch_desc* descs, size_t n,
                                           xp_sketch** outs) {
     if (!grammars || !descs || !outs || n == 0) return fail(XP_ERR_INVALID_ARG, "xp_sketch_load_batch: null argument");
     for (size_t i = 0; i < n; ++i) outs[i] = nullptr;
-    std::lock_guard<std::mutex> one(g_load_mu);
     std::vector<LoadState> st(n);
     char* dev_block = nullptr;
     size_t dev_bytes = 0;
     int dev_device = 0;
     bool sent = false;
+    bool claimed = false;                                 // grammars of this load are on their way
+    auto settle = [&]() {                                 // they have been sent, or never will be
+        if (!claimed) return;
+        claimed = false;
+        std::lock_guard<std::mutex> lock(g_load_mu);
+        for (size_t i = 0; i < n; ++i) {
+            if (!st[i].grammar_fresh) continue;
+            xp_grammar* g = const_cast<xp_grammar*>(grammars[i]);
+            if (!sent) { pool_release(g->d_g, g->d_bytes, g->d_device); g->d_g = nullptr; }
+            g->d_pending = false;
+        }
+        g_load_cv.notify_all();
+    };
+    struct Settle { decltype(settle)& f; ~Settle() { f(); } } at_the_end{settle};      // (whatever way the call ends)
     auto undo = [&]() {
         cudaStreamSynchronize(nullptr);                   // nothing may still be writing into the blocks
-        for (size_t i = 0; i < n; ++i) {
-            if (st[i].grammar_fresh && !sent) {           // its tables never went out
-                xp_grammar* g = const_cast<xp_grammar*>(grammars[i]);
-                pool_release(g->d_g, g->d_bytes, g->d_device);
-                g->d_g = nullptr;
-            }
-            if (st[i].s) xp_sketch_destroy(st[i].s);
-        }
+        settle();
+        for (size_t i = 0; i < n; ++i) if (st[i].s) xp_sketch_destroy(st[i].s);
         pool_release(dev_block, dev_bytes, dev_device);
     };
 #define XP_CUDA_B(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { undo(); \
@@ -964,13 +983,36 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     int ndev = 0;
     // (a description that is wrong is reported as such also where no device can be used)
     const bool no_device = cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1;
+    auto refuse = [&](xp_status e, size_t i) {
+        const std::string why = no_device && e == XP_ERR_CUDA ? std::string("no CUDA device is usable") : g_last_error;
+        undo();
+        return fail(e, "sketch " + std::to_string(i) + ": " + why);
+    };
+    for (size_t i = 0; i < n; ++i) {
+        const xp_status e = load_check(grammars[i], &descs[i], &st[i]);
+        if (e != XP_OK) return refuse(e, i);
+    }
+    {
+        xp_status e = XP_OK;
+        size_t i = 0;
+        {
+            std::unique_lock<std::mutex> lock(g_load_mu);
+            g_load_cv.wait(lock, [&]() {
+                for (size_t k = 0; k < n; ++k) if (grammars[k]->d_pending) return false;
+                return true;
+            });
+            claimed = true;
+            for (; i < n && e == XP_OK; ++i) {
+                xp_grammar* g = const_cast<xp_grammar*>(grammars[i]);
+                e = grammar_block(g, &st[i].grammar_fresh);
+                if (st[i].grammar_fresh) { g->d_pending = true; st[i].grammar_bytes = grammar_layout(g).total; }
+            }
+        }
+        if (e != XP_OK) return refuse(e, i - 1);
+    }
     for (size_t i = 0; i < n; ++i) {
         const xp_status e = load_begin(grammars[i], &descs[i], &st[i]);
-        if (e != XP_OK) {
-            const std::string why = no_device && e == XP_ERR_CUDA ? std::string("no CUDA device is usable") : g_last_error;
-            undo();
-            return fail(e, "sketch " + std::to_string(i) + ": " + why);
-        }
+        if (e != XP_OK) return refuse(e, i);
     }
     // The staged copy: the job lists, then the sketches' shares, in pieces of about kPieceBytes that page-locked memory
     // holds one by one.  The pieces go to one block of device memory, and a kernel puts the shares in their places:
@@ -1047,14 +1089,19 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             };
             if (n_threads < 2) work(false);
             else {
+                std::lock_guard<std::mutex> alone(g_fill_mu);        // (one load at a time spreads over the cores: four at once, 200 sketches each, 1.3 -> 2.0 ms a load)
                 std::vector<std::thread> pool;
-                for (size_t t = 0; t + 1 < n_threads; ++t) pool.emplace_back(work, true);
+                pool.reserve(n_threads);
+                try {
+                    for (size_t t = 0; t + 1 < n_threads; ++t) pool.emplace_back(work, true);
+                } catch (const std::system_error&) {      // (no more threads to be had: those there are do the work)
+                }
                 work(false);
                 for (std::thread& th : pool) th.join();
             }
             err = (cudaError_t)bad.load();
             if (err == cudaSuccess) err = launch_scatter((const LoadCopy*)(dev_block + at_copies), (int)copies.size(), dev_block, nullptr);
-            if (err == cudaSuccess) sent = true;
+            if (err == cudaSuccess) { sent = true; settle(); }
         }
         // (the staging blocks may go back once the copies have been made: they are waited for below, with everything else)
         struct Hold { std::vector<StageBlock*>& v; ~Hold() { for (StageBlock* b : v) delete b; } } release{hold};

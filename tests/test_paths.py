@@ -487,3 +487,35 @@ def test_many_operands_under_a_comparison(xp, ctx, spec):
         at = p * (n[7] // 5)
         check_sketch(xp, sk, windows={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: (at + 7, at + 100_000)})
     check_sketch(xp, sk, windows={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: (n[7] - 100_000, n[7])})
+
+
+@pytest.mark.gpu
+def test_threads_that_load_the_same_new_grammars(xp):
+    """Two grammars that nobody has loaded yet, in batches that name them in either order, from six threads at once: each load finds the
+    tables in place, and none waits for another for good."""
+    vs = [Variable("i", 0, 50), Variable("j", 0, 40)]
+    models = [free_grammar(vs, [1, 2, 3]), free_grammar(vs, [2, 5])]
+    rng = np.random.default_rng(1)
+    coords = np.stack([rng.integers(0, 50, size=9000), rng.integers(0, 40, size=9000)], axis=1).astype(np.int32)
+    table = coords[:, 0].astype(np.int64) * 2 + coords[:, 1]
+    sks = [Sketch(m, [Hole(0, 5, spec_table=table)], coords) for m in models]
+    want = [oracle.repair_hole(s) for s in sks]
+    for _ in range(8):
+        grs = [xp.xp_grammar_create(m) for m in models]
+        got, failed = [], []
+
+        def work(k):
+            try:
+                order = [k % 2, 1 - k % 2, k % 2]
+                for which, r in zip(order, xp.xp_repair_batch(xp.xp_sketch_load_batch([grs[o] for o in order], [sks[o] for o in order]))):
+                    got.append((which, r[0]))
+            except Exception as e:      # noqa: BLE001
+                failed.append(e)
+        threads = [threading.Thread(target=work, args=(k,)) for k in range(6)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join(60)
+        assert not failed and len(got) == 18
+        for which, r in got:
+            assert_same(r, want[which])
