@@ -479,6 +479,11 @@ struct HoleHost {
     int tab_max = 0;                 // subtrees up to this size are tabulated
     bool compares = false;           // the filter works on an interval of hole values (the context compares)
     bool second = false;             // filter hits are looked at once more at probe 1 from the start (hits are frequent)
+    int cls_size = 0;                // operands of this size are in classes, cls_n of each nonterminal (0: none)
+    u32 cls_n[kMaxNt] = {0};
+    // What the load makes classes of: the size, and for which contexts (0: none); a grammar's subtrees of that size, and of one nonterminal at most.
+    int cls_top = 0, cls_want = 0;
+    u64 cls_entries = 0, cls_most = 0;
 };
 
 struct Plan {
@@ -531,6 +536,8 @@ static void hole_decided(HoleHost* h, const LoadOut& o) {
     h->target_zero = o.target_zero != 0;
     h->tab_max = o.tab_max;
     h->second = o.second != 0;
+    h->cls_size = o.cls_size;
+    memcpy(h->cls_n, o.cls_n, sizeof(h->cls_n));
     if (o.spec_bad) h->never = true;                      // the spec is undefined at some point
 }
 
@@ -583,6 +590,26 @@ static u64 table_entries(const xp_grammar* g, int max_size, u64 (*off)[kMaxSize 
     return total;
 }
 
+// Is a hole's search made of enough combinations of its largest tabulated subtrees that they are put into classes first?  Where an
+// operand of the search is itself above the tables, each of them is met at least a hundred times; where the context compares, an
+// operand costs some ten thousand instructions against some hundred here.  Otherwise every operand is met once, and would be here too.
+constexpr u64 kClassLeast = 4096;            // subtrees from which it pays
+static void class_plan(const xp_grammar* g, const xp_hole_desc& hd, HoleHost* h) {
+    int tmax = 0, top = 0, need = 0;
+    (void)table_entries(g, hd.max_size, nullptr, &tmax);
+    for (int nt = 0; nt < g->n_nt; ++nt)
+        for (int k = 1; k <= hd.max_size - 2; ++k)
+            if (g->cnt[nt][k] > 0) { need = k > need ? k : need; if (k <= tmax) top = k > top ? k : top; }
+    if (top < 3) return;
+    u64 all = 0, most = 0;
+    for (int nt = 0; nt < g->n_nt; ++nt) { const u64 c = g->cnt[nt][top]; all += c; most = c > most ? c : most; }
+    if (all < kClassLeast) return;
+    bool compares = false;
+    for (int i = 0; i < hd.ctx_len; ++i) compares = compares || (hd.ctx[i].kind == XP_I_OP && (hd.ctx[i].arg == XP_OP_LT || hd.ctx[i].arg == XP_OP_LE));
+    h->cls_want = (need > top ? kClassAffine | kClassCompare : 0) | (compares ? kClassCompare : 0);
+    if (h->cls_want) { h->cls_top = top; h->cls_entries = all; h->cls_most = most; }
+}
+
 // One sketch on its way through a load: everything between its description and the moment the
 // load's kernels have run.
 struct LoadState {
@@ -590,7 +617,7 @@ struct LoadState {
     const xp_sketch_desc* d = nullptr;
     struct Hole {                            // what begin settles per hole; the record itself is made in its place in the staged copy
         size_t off_spec = 0;                 // its spec values in the device block (0: none there)
-        size_t off_tabv = 0, off_tabk = 0, off_tabm = 0, off_pair = 0, off_sets = 0;
+        size_t off_tabv = 0, off_tabk = 0, off_tabm = 0, off_pair = 0, off_sets = 0, off_cls = 0;
         u64 entries = 0;
         int probes = 0;
     };
@@ -770,6 +797,7 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     const size_t off_sketch = off;  off += al256(sizeof(SketchDev));
     const size_t off_holes = off;   off += al256(sizeof(HoleDev) * nh);
     L->hole.resize(nh);
+    s->holes.resize(nh);
     if (L->copy_coords && coords_bytes <= kPackMax) { L->off_coords = off; off += al256(coords_bytes); }
     for (int h = 0; h < nh; ++h)
         if (d->holes[h].spec_kind == XP_SPEC_TABLE && np > 0 && !d->holes[h].spec_table_on_device && spec_bytes <= kPackMax) {
@@ -798,6 +826,8 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             o.off_tabm = off; off += al256(entries);
             o.off_pair = off; off += al256(2 * sizeof(i32) * entries);
         }
+        class_plan(g, hd, &s->holes[h]);
+        if (const size_t c = s->holes[h].cls_entries) { o.off_cls = off; off += al256(8 * c) + al256(4 * (c + kMaxNt + 1)) + al256(4 * c); }
         o.off_sets = off; off += al256(sizeof(JoinSet) * (size_t)g->n_nt);
         if (size_cap > s->tab_size_cap) s->tab_size_cap = size_cap;
         if (o.probes > s->tab_probes_cap) s->tab_probes_cap = o.probes;
@@ -814,7 +844,6 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
     s->d_s = (SketchDev*)(base + off_sketch);
     s->d_holes = (HoleDev*)(base + off_holes);
     s->off_holes = off_holes;
-    s->holes.resize(nh);
     for (int h = 0; h < nh; ++h) { s->holes[h].start_nt = d->holes[h].start_nt; s->holes[h].max_size = d->holes[h].max_size; }
     for (int k = 1; k <= s->tab_size_cap; ++k)
         for (int nt = 0; nt < g->n_nt; ++nt) s->entries_at[k] += g->cnt[nt][k];
@@ -852,6 +881,14 @@ static void hole_image(const LoadState* L, int h, HoleDev* out) {
         o.tab_ok = (unsigned char*)(base + at.off_tabk);
         o.tab_vars = (unsigned char*)(base + at.off_tabm);
         o.tab_pair = (i32*)(base + at.off_pair);
+    }
+    if (at.off_cls) {
+        const HoleHost& hh = s->holes[h];
+        const size_t c = hh.cls_entries;
+        o.cls_top = hh.cls_top; o.cls_want = hh.cls_want;
+        o.cls_pair = (int2*)(base + at.off_cls);
+        o.cls_start = (u32*)(base + at.off_cls + al256(8 * c));
+        o.cls_mem = (u32*)(base + at.off_cls + al256(8 * c) + al256(4 * (c + kMaxNt + 1)));
     }
     o.join_sets = (JoinSet*)(base + at.off_sets);
     // variables that decide beside the candidate's own (a caller's spec table may depend on all)
@@ -938,6 +975,19 @@ static cudaError_t make_tables(const LoadJob* jobs, int n_jobs, int size_cap, in
     if (size_cap < 1) return cudaSuccess;
     cudaError_t e = launch_subvalues(jobs, n_jobs, 1, 3, probes_cap, entries_at[1] + (size_cap >= 3 ? entries_at[3] : 0), nullptr);
     for (int k = 5; k <= size_cap && e == cudaSuccess; k += 2) e = launch_subvalues(jobs, n_jobs, k, k, probes_cap, entries_at[k], nullptr);
+    return e;
+}
+
+// The classes of the holes of a sketch that are to have them, one hole after the other in the same scratch.
+static size_t classes_scratch(const xp_sketch* s) {
+    size_t most = 0;
+    for (const HoleHost& h : s->holes) { const size_t b = class_scratch_bytes(h.cls_entries); most = b > most ? b : most; }
+    return most;
+}
+static cudaError_t make_classes(const xp_sketch* s, char* scratch, LoadOut* out) {
+    cudaError_t e = cudaSuccess;
+    for (int h = 0; h < s->n_holes && e == cudaSuccess; ++h)
+        if (s->holes[h].cls_entries > 0) e = launch_classes(s->d_s, h, scratch, s->holes[h].cls_entries, s->holes[h].cls_most, s->g->n_nt, out ? out + h : nullptr, nullptr);
     return e;
 }
 
@@ -1044,7 +1094,10 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     }
     const size_t staged = at;
     const size_t at_out = al256(staged), at_scratch = at_out + al256(sizeof(LoadOut) * n_jobs);
-    const size_t total = at_scratch + prepare_scratch_bytes((int)(n_jobs < kJobs ? n_jobs : kJobs));
+    const size_t at_classes = at_scratch + al256(prepare_scratch_bytes((int)(n_jobs < kJobs ? n_jobs : kJobs)));
+    size_t class_bytes = 0;
+    for (size_t i = 0; i < n; ++i) { const size_t b = classes_scratch(st[i].s); class_bytes = b > class_bytes ? b : class_bytes; }
+    const size_t total = at_classes + class_bytes;
     XP_CUDA_B(pool_alloc((void**)&dev_block, total, &dev_device, &dev_bytes));
     StageBlock back(sizeof(LoadOut) * n_jobs);
     if (!back.p) { undo(); return fail(XP_ERR_NOMEM, "out of host memory"); }
@@ -1161,6 +1214,10 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         }
         for (size_t q = 0; q < n_jobs; q += kJobs)
             XP_CUDA_B(make_tables(d_jobs + q, (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs), size_cap, probes_cap, most_entries));
+        if (class_bytes > 0) {
+            LoadOut* out = (LoadOut*)(back.locked ? back.p : dev_block + at_out);
+            for (size_t i = 0; i < n; out += st[i].s->n_holes, ++i) XP_CUDA_B(make_classes(st[i].s, dev_block + at_classes, out));
+        }
         if (!back.locked) XP_CUDA_B(cudaMemcpyAsync(back.p, dev_block + at_out, sizeof(LoadOut) * n_jobs, cudaMemcpyDeviceToHost, nullptr));
         XP_CUDA_B(cudaStreamSynchronize(nullptr));
     }
@@ -1279,19 +1336,24 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         char* jobs_dev = nullptr;
         size_t jobs_bytes = 0;
         int jobs_device = 0;
-        XP_CUDA(pool_alloc((void**)&jobs_dev, sizeof(LoadJob) * jobs.size(), &jobs_device, &jobs_bytes));
+        const size_t at_classes = al256(sizeof(LoadJob) * jobs.size()), class_bytes = classes_scratch(s);
+        XP_CUDA(pool_alloc((void**)&jobs_dev, at_classes + class_bytes, &jobs_device, &jobs_bytes));
+        for (HoleDev& o : hh) memset(o.cls_count, 0, sizeof(o.cls_count));      // (holes without a promoted point are numbered again too)
         cudaError_t e = cudaMemcpyAsync(s->arena + s->off_holes, hh.data(), sizeof(HoleDev) * nh, cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(LoadJob) * jobs.size(), cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = launch_reprobe((const LoadJob*)jobs_dev, (int)jobs.size(), nullptr);
         if (e == cudaSuccess) e = make_tables((const LoadJob*)jobs_dev, (int)jobs.size(), s->tab_size_cap, s->tab_probes_cap, s->entries_at);
+        if (e == cudaSuccess && class_bytes > 0) e = make_classes(s, jobs_dev + at_classes, nullptr);
         if (e == cudaSuccess) e = cudaMemcpyAsync(hh.data(), s->arena + s->off_holes, sizeof(HoleDev) * nh, cudaMemcpyDeviceToHost, nullptr);
         const cudaError_t e2 = cudaStreamSynchronize(nullptr);
         pool_release(jobs_dev, jobs_bytes, jobs_device);
         if (e != cudaSuccess || e2 != cudaSuccess)
             return fail(XP_ERR_CUDA, std::string("xp_sketch_refine: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
         for (int h = 0; h < nh; ++h) {
-            hole_decided(&s->holes[h], LoadOut{hh[h].filter_ok, hh[h].tab_probes, hh[h].aff_ok, hh[h].join_on, hh[h].second, hh[h].n_probe, hh[h].tab_max_size,
-                                                  hh[h].join_t0 == 0 || hh[h].join_t1 == 0, 0u, 0u});
+            LoadOut o{hh[h].filter_ok, hh[h].tab_probes, hh[h].aff_ok, hh[h].join_on, hh[h].second, hh[h].n_probe, hh[h].tab_max_size,
+                      hh[h].join_t0 == 0 || hh[h].join_t1 == 0, 0u, hh[h].cls_size, {0}};
+            memcpy(o.cls_n, hh[h].cls_n, sizeof(o.cls_n));
+            hole_decided(&s->holes[h], o);
             s->n_probes[h] = hh[h].n_probe;
         }
         std::lock_guard<std::mutex> lock(s->plan_mu);
@@ -1554,10 +1616,26 @@ static JoinSeg new_join_seg(int sketch, int hole, int acc, int k, u64 lo, u64 hi
     return sg;
 }
 
+// Operands of (nt, size) counted by class (class_operand walks them in the same order); without classes, all of them.
+static u64 class_operands(const xp_grammar* g, const HoleHost& ho, int nt, int size) {
+    if (ho.cls_size == 0 || size < ho.cls_size) return g->cnt[nt][size];
+    auto side = [&](int n, int k) { return k == ho.cls_size ? (u64)ho.cls_n[n] : g->cnt[n][k]; };
+    if (size <= ho.tab_max) return side(nt, size);
+    u64 sum = 0;
+    for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b)
+        for (int a = 1; a <= size - 2; ++a) {
+            const int l = g->bins[b].lnt, r = g->bins[b].rnt, z = size - 1 - a;
+            sum += a > ho.tab_max || z > ho.tab_max ? g->cnt[l][a] * g->cnt[r][z] : side(l, a) * side(r, z);
+        }
+    return sum;
+}
+
 // Leaf-join segments of (start nonterminal, size k >= 3) restricted to ranks [lo, hi): one per operand nonterminal, with
 // a group per leaf nonterminal, for every operator with a leaf of it on either side of such an operand.  Copies of one
 // production open segments of their own; so do shifts, which only the exact form knows.
-static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool exact, bool compares) {
+static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi) {
+    const int nt = ho.start_nt;
+    const bool exact = ho.exact, compares = ho.compares;
     struct Open { JoinSeg seg; bool shifts; std::vector<JoinGroup> groups; };
     std::vector<Open> open;
     for (int b = g->bin_begin[nt]; b < g->bin_begin[nt + 1]; ++b) {
@@ -1616,6 +1694,11 @@ static void add_joins(Plan* plan, const xp_grammar* g, int nt, int sketch, int h
         c.seg.first_group = (i32)plan->jgroups.size();
         c.seg.n_groups = (i32)c.groups.size();
         for (const JoinGroup& q : c.groups) if ((g->wide_leaf >> q.leaf_nt) & 1u) { c.seg.exact = kExactMany; c.seg.heavy = 1; }
+        // (a rank window may cover fewer operands than there are combinations of classes)
+        if (!c.seg.exact && ho.cls_size > 0 && c.seg.esize >= ho.cls_size) {
+            const u64 m = class_operands(g, ho, c.seg.nt, c.seg.esize);
+            if (m < c.seg.e_count) { c.seg.classes = 1; c.seg.e_begin = 0; c.seg.e_count = m; }
+        }
         plan->jgroups.insert(plan->jgroups.end(), c.groups.begin(), c.groups.end());
         plan->jsegs.push_back(c.seg);
     }
@@ -1756,8 +1839,8 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 if (k < 3 || (!forced && hi - lo < kTileMinRanks)) { add_direct(plan, ho.start_nt, (int)i, h, acc, k, lo, hi); continue; }
                 // (A range of hole values: the join's interval arithmetic per operand against a test per candidate.  27 leaves, size 7, 984 000
                 // operands, four specs: 13.4, 26.5, 10.2, 14.4 ms by the join, 14.9, 19.8, 10.7, 8.2 as tiles; 40 leaves, size 5: 0.4 against 1.4.)
-                const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
-                if (!leaves) add_joins(plan, s->g, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.exact, ho.compares);
+                const bool leaves = ho.compares && class_operands(s->g, ho, ho.start_nt, k - 2) > kRangeMost;
+                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi);
                 const bool pairs = form >= kFormPairsSome;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
                 add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany, leaves);

@@ -179,6 +179,17 @@ struct HoleDev {
     float join_h0, join_h1;                       // a huge number where the target is 0, else 0
     JoinSet* join_sets;                           // device, one per nonterminal
     i32* tab_pair;                                // device
+    // Operand classes (csrc/xp_classes.cuh): the subtrees of cls_size nodes, the largest size with any in the tables, by their
+    // values at the first n_exact probes.  Class c of nonterminal nt: the pair of values that its members share
+    // (cls_pair), and their ranks cls_mem[cls_start[c] .. cls_start[c + 1]).  Subtrees undefined at one of those probes are in
+    // none.  A nonterminal's share of the arrays starts at tab_off[nt][cls_size] - tab_off[0][cls_size] (of cls_start, nt further on).
+    i32 cls_top, cls_want;                        // host: that size, and for which contexts classes are made (kClassAffine, kClassCompare)
+    i32 cls_size, pad6;                           // 0: there are none
+    u32 cls_n[kMaxNt];
+    u64 cls_count[kMaxNt];                        // members << 32 | classes while they are numbered, zero before
+    int2* cls_pair;                               // device
+    u32* cls_start;                               // device
+    u32* cls_mem;                                 // device
     // Points that ended a survivor's whole-domain check (a candidate that passed every probe and then
     // failed somewhere): a small open-addressed table of point ids (-1: free) with the number of
     // survivors each has ended.  Written by verify_kernel, read and cleared by xp_sketch_refine, which
@@ -187,6 +198,7 @@ struct HoleDev {
     u32* kill_cnt;                                // device, kKillSlots entries
 };
 constexpr int kKillSlots = 64;
+enum { kClassAffine = 1, kClassCompare = 2 };
 
 struct SketchDev {
     const GrammarDev* g;                          // device
@@ -209,7 +221,7 @@ struct LoadJob { SketchDev* s; i32 hole, pad; };
 struct LoadCopy { char* dst; u64 src, bytes; };
 
 // What the load's kernels settled for a hole, as the host reads it back.
-struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe, tab_max, target_zero; u32 spec_bad, pad; };
+struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe, tab_max, target_zero; u32 spec_bad; i32 cls_size; u32 cls_n[kMaxNt]; };
 
 // Per (sketch, hole) accumulators, zeroed (min_rank to all-ones) by the host before the launch.
 struct AccDev {
@@ -246,6 +258,7 @@ struct JoinSeg {
     i32 exact;                       // kExactFew, kExactMany: there is no condition (shifts, a leaf of 2^31 or more), every candidate is evaluated on its own
     u32 chunk;                       // operands per ticket
     i32 heavy;                       // an operand costs many times the usual (exact form, contexts that compare): these go first
+    i32 classes, pad;                // operands are counted by class: e_begin = 0, e_count combinations of classes (class_operands)
     u64 e_begin, e_count;
 };
 

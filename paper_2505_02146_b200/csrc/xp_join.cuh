@@ -247,6 +247,43 @@ __device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev*
     return probe_check(g, hole, code, n, evals);
 }
 
+// Candidates of a segment that counts by class, one per lane (pass: this lane has one, and it satisfies the probes with tables):
+// every member of the class is a candidate of its own, 32 at a time over all lanes' members.  Called by all lanes.
+__device__ __noinline__ void join_members(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, bool pass, u64 e, u32 pos,
+                                          u32 code, JoinCount& n) {
+    if (!__any_sync(0xffffffffu, pass)) return;
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    u64 incl = pass ? class_operand(g, hole, seg.nt, seg.esize, e).members() : 0ull;
+    for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+    const u64 total = __shfl_sync(0xffffffffu, incl, 31);
+    for (u64 k0 = 0; k0 < total; k0 += 32u) {
+        const u64 k = k0 + (u64)lane < total ? k0 + (u64)lane : total - 1u;
+        int src = 0;                                      // the lane whose member this is: the first with incl > k
+        for (int step = 16; step > 0; step >>= 1) { const u64 v = __shfl_sync(0xffffffffu, incl, src + step - 1); if (v <= k) src += step; }
+        const u64 before = __shfl_sync(0xffffffffu, incl, src ? src - 1 : 0), e2 = __shfl_sync(0xffffffffu, e, src);
+        const u32 pos2 = __shfl_sync(0xffffffffu, pos, src), code2 = __shfl_sync(0xffffffffu, code, src);
+        bool ok = false;
+        u64 rank = 0;
+        u32 vars = 0;
+        if (k0 + (u64)lane < total) {
+            const int swap = (int)(code2 & 1u), slot = (int)((code2 >> 1) & 15u);
+            const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code2 >> 8)];
+            const u64 member = class_operand(g, hole, seg.nt, seg.esize, e2).rank(src ? k - before : k);
+            const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
+            rank = grp.base[swap][slot] + (swap ? (u64)pos2 * ne + member : member * nl + (u64)pos2);
+            ok = rank >= seg.rank_begin && rank < seg.rank_end &&
+                 XP_CHECKED(member < ne && (u64)pos2 < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
+            if (ok && hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, rank, n.evals);
+            if (ok) {
+                const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos2];
+                vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, member)) | (lf.var >= 0 ? 1u << lf.var : 0u);
+            }
+        }
+        join_survive(w, plan, sk, hole, seg, ok, rank, vars, n);
+    }
+}
+
 // The candidates in the warp's second queue, one per lane: the probes from `from` on, exactly.  Called by all lanes.
 __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, int from, JoinCount& n) {
     const GrammarDev* g = sk->g;
@@ -257,6 +294,19 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
         bool pass = false;
         u64 rank = 0;
         u32 vars = 0;
+        if (seg.classes) {                                // a member's values are its class's: one check for all of them
+            u64 e = 0;
+            u32 code = 0, pos = 0;
+            if (at + lane < nc) {
+                code = w.c_code[at + lane]; pos = w.c_pos[at + lane]; e = w.base + w.c_off[at + lane];
+                const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, class_operand(g, hole, seg.nt, seg.esize, e).rank(0));
+                const LeafDev lf = g->leaves[g->leaf_begin[plan.jgroups[seg.first_group + (int)(code >> 8)].leaf_nt] + (int)pos];
+                pass = exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, (code & 1u) != 0u, op_of_slot((int)((code >> 1) & 15u)), from,
+                                  hole->n_exact, n.evals);
+            }
+            join_members(w, plan, seg, sk, hole, pass, e, pos, code, n);
+            continue;
+        }
         if (at + lane < nc) {
             const u32 code = w.c_code[at + lane], pos = w.c_pos[at + lane];
             const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u);
@@ -779,7 +829,7 @@ __device__ __noinline__ void join_exact32(JoinWarp& w, const PlanDev& plan, cons
     const bool two = hole->n_exact >= 2;
     i64 a0 = 0, a1 = 0;
     if (live) {
-        const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
+        const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, seg.classes ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e);
         live = ref_value(g, hole, ref, seg.nt, seg.esize, 0, a0) && (!two || ref_value(g, hole, ref, seg.nt, seg.esize, 1, a1));
     }
     const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
@@ -854,34 +904,52 @@ struct JoinRun {
     const int2* R;
     u32 l0, r0, cr, inv;                                  // first operands; right operands per left one and 2^32 / that
     u64 left;                                             // operands to the end of the run
+    u64 rank;                                             // (mode 2) rank of the first
 };
 
-__device__ __noinline__ JoinRun join_run(const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank) {
+// The run that operand number `rank` of (nt, size) is in; classes: the number counts by class (class_operand).
+__device__ __noinline__ JoinRun join_run(const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank, bool classes) {
     JoinRun c;
     const int2* pair = reinterpret_cast<const int2*>(hole->tab_pair);
     const int tmax = hole->tab_max_size;
     const u64 total = g->cnt[nt][size];
-    c.mode = 2; c.op = 0; c.l0 = c.r0 = 0; c.cr = 1; c.inv = 0xffffffffu; c.L = c.R = pair; c.left = total - rank;
-    if (size <= tmax) { c.mode = 0; c.R = pair + hole->tab_off[nt][size] + rank; return c; }
+    c.mode = 2; c.op = 0; c.l0 = c.r0 = 0; c.cr = 1; c.inv = 0xffffffffu; c.L = c.R = pair; c.left = total - rank; c.rank = rank;
+    if (size <= tmax) {
+        const OperandSide s = operand_side(g, hole, nt, size, classes);
+        c.mode = 0; c.R = s.pair + rank; c.left = s.n - rank;
+        return c;
+    }
     if (tmax < 1 || size < 3) return c;
-    int p = g->bin_begin[nt];
+    int p = g->bin_begin[nt], a = 1;
     const int pe = g->bin_begin[nt + 1];
-    while (p + 1 < pe && g->bins[p + 1].off[size] <= rank) ++p;
-    u64 rem = rank - g->bins[p].off[size];
-    const int lnt = g->bins[p].lnt, rnt = g->bins[p].rnt;
-    u64 cl = 0, cr = 0;
-    int a = 1;
-    for (;; ++a) {
-        cl = g->cnt[lnt][a]; cr = g->cnt[rnt][size - 1 - a];
-        if (rem < cl * cr || a == size - 2) break;
-        rem -= cl * cr;
+    u64 rem = rank, cl = 0, cr = 0, base = 0;
+    if (!classes) {
+        while (p + 1 < pe && g->bins[p + 1].off[size] <= rank) ++p;
+        base = g->bins[p].off[size]; rem = rank - base;
+    }
+    for (;; ++p) {                                        // (without classes the production is known)
+        const int lnt = g->bins[p].lnt, rnt = g->bins[p].rnt;
+        if (classes) base = g->bins[p].off[size];
+        bool here = false;
+        for (a = 1; a <= size - 2; ++a) {
+            const u64 fl = g->cnt[lnt][a], fr = g->cnt[rnt][size - 1 - a];
+            cl = fl; cr = fr;
+            if (classes && a <= tmax && size - 1 - a <= tmax) {
+                cl = operand_side(g, hole, lnt, a, true).n; cr = operand_side(g, hole, rnt, size - 1 - a, true).n;
+            }
+            here = rem < cl * cr || (!classes && a == size - 2);
+            if (here) break;
+            rem -= cl * cr; base += fl * fr;
+        }
+        if (here || p + 1 >= pe) break;
     }
     c.left = cl * cr - rem;
+    c.rank = base + rem;
     if (a > tmax || size - 1 - a > tmax) return c;        // (an operand above the tables: the whole run goes one by one)
     u64 l, r;
     divmod_u64(rem, cr, l, r);
     c.mode = 1; c.op = g->bins[p].op;
-    c.L = pair + hole->tab_off[lnt][a]; c.R = pair + hole->tab_off[rnt][size - 1 - a];
+    c.L = operand_side(g, hole, g->bins[p].lnt, a, classes).pair; c.R = operand_side(g, hole, g->bins[p].rnt, size - 1 - a, classes).pair;
     c.l0 = (u32)l; c.r0 = (u32)r; c.cr = (u32)cr;
     c.inv = cr > 1 ? (u32)((1ull << 32) / cr) : 0xffffffffu;
     return c;
@@ -926,7 +994,7 @@ __device__ __forceinline__ void pair_op(const int2 (&x)[P], const int2 (&y)[P], 
 
 // Operands at + 32 p + lane of a run (those below n), their values at the two probes.
 template <int P>
-__device__ __forceinline__ void run_values(const JoinRun& c, const GrammarDev* g, const HoleDev* hole, int nt, int size, u64 rank, u32 at, u32 n,
+__device__ __forceinline__ void run_values(const JoinRun& c, const GrammarDev* g, const HoleDev* hole, int nt, int size, u32 at, u32 n,
                                            i32 (&a0)[P], i32 (&a1)[P], u32& alive, u32& wide) {
     const u32 lane = threadIdx.x & 31u;
     alive = wide = 0;
@@ -946,7 +1014,7 @@ __device__ __forceinline__ void run_values(const JoinRun& c, const GrammarDev* g
         for (int p = 0; p < P; ++p) {
             if (!((alive >> p) & 1u)) continue;
             i32 v0 = 0, v1 = 0;
-            const int st = join_value_slow(g, hole, nt, size, rank + at + 32u * p + lane, v0, v1);
+            const int st = join_value_slow(g, hole, nt, size, c.rank + at + 32u * p + lane, v0, v1);
 #pragma unroll
             for (int k = 0; k < P; ++k) if (k == p) { a0[k] = v0; a1[k] = v1; }
             if (st != 1) { alive &= ~(1u << p); wide |= (u32)(st == 2) << p; }
@@ -1093,13 +1161,19 @@ __device__ __noinline__ void join_fill(JoinWarp& w, const PlanDev& plan, const J
     __syncwarp();
 }
 
+// What `count` operands from number `first` on stand for in the count of candidates: themselves, or, where the segment counts by class, the
+// first ticket's for all there are.
+__device__ __forceinline__ u64 seg_operands(const JoinSeg& seg, const GrammarDev* g, u64 first, u64 count) {
+    return !seg.classes ? count : first == 0ull ? g->cnt[seg.nt][seg.esize] : 0ull;
+}
+
 // Operands [first, first + count) of a segment against the leaves (count <= the segment's chunk).
 template <int P>
 __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
                                          u64 first, u64 count, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
-    n.cands += count * w.hot.pairs;
+    n.cands += seg_operands(seg, g, first, count) * w.hot.pairs;
     const u32 lim = w.hot.lim;
     if (seg.exact == kExactFew) {
         for (u64 i = 0; i < count; ++i) join_exact(w, plan, seg, sk, hole, first + i, n);
@@ -1116,13 +1190,13 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     u32 nq = w.nq;
     u32 n_alive = 0;
     for (u64 done = 0; done < count;) {
-        const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done);
+        const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done, seg.classes != 0);
         const u32 n_run = (u32)(c.left < count - done ? c.left : count - done);
         const u32 off0 = (u32)(first + done - w.base) + lane;
         for (u32 at = 0; at < n_run; at += 32u * P) {
             i32 a0[P], a1[P];
             u32 alive, wide;
-            run_values<P>(c, g, hole, seg.nt, seg.esize, first + done, at, n_run, a0, a1, alive, wide);
+            run_values<P>(c, g, hole, seg.nt, seg.esize, at, n_run, a0, a1, alive, wide);
             bool any[P];
 #pragma unroll
             for (int p = 0; p < P; ++p) {
@@ -1319,7 +1393,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         pairs += g->cnt[grp.leaf_nt][1] * (u64)(__popc(grp.fmask) + __popc(grp.smask));
         sets_ok = sets_ok && hole->join_sets[grp.leaf_nt].ok != 0;
     }
-    n.cands += count * pairs;
+    n.cands += seg_operands(seg, g, first, count) * pairs;
     for (u64 at = 0; at < count; at += 32) {
         const u64 e = first + at + lane;
         const bool have = at + lane < count;
@@ -1330,7 +1404,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         i64 pl = -kMost, ph = kMost, ml = -kMost, mh = kMost;
         bool live = false, wide = false;
         if (have) {
-            ref = operand_ref(g, hole, seg.nt, seg.esize, e);
+            ref = operand_ref(g, hole, seg.nt, seg.esize, seg.classes ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e);
             live = true;
             for (int j0 = 0; j0 < np && live && !wide; j0 += kProbeStep) {
                 i64 val[kProbeStep];

@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
     probe_contexts(g, hole, s_n, ncand, s_pass0);
     if (t == 0)                                         // (thread 0 has written all of these itself)
         out[blockIdx.x] = LoadOut{hole->filter_ok, hole->tab_probes, hole->aff_ok, hole->join_on, hole->second, hole->n_probe, hole->tab_max_size,
-                                  hole->join_t0 == 0 || hole->join_t1 == 0 ? 1 : 0, hole->spec_bad, 0u};
+                                  hole->join_t0 == 0 || hole->join_t1 == 0 ? 1 : 0, hole->spec_bad, 0, {0}};
 }
 
 // The probes of a hole replaced by the host (xp_sketch_refine: points that ended whole-domain
@@ -2399,6 +2399,7 @@ __global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const __gri
 }
 
 }  // namespace xp
+#include "xp_classes.cuh"
 #include "xp_join.cuh"
 #include "xp_pairs.cuh"
 namespace xp {
@@ -3153,6 +3154,21 @@ cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last
     const int all = (most_probes + kSubProbes - 1) / kSubProbes;
     const int groups = (u64)n_jobs * most_entries >= 148ull * 2048 ? all : 1;
     chain(subvalue_kernel, dim3((unsigned)((most_entries + 255) / 256), (unsigned)((all + groups - 1) / groups), (unsigned)n_jobs), 256, 0, stream, jobs, size, last, groups);
+    return cudaGetLastError();
+}
+
+// The classes of one hole, `entries` subtrees of the size in question over n_nt nonterminals (most: of one of them).
+cudaError_t launch_classes(SketchDev* s, int hole, char* scratch, u64 entries, u64 most, int n_nt, LoadOut* out, cudaStream_t stream) {
+    ClassJob job;
+    const u32 slots = class_slots(entries);
+    job.s = s; job.hole = hole; job.pad = 0; job.out = out;
+    job.table = (u64*)scratch; job.mask = slots - 1u; job.at = (uint2*)(scratch + sizeof(u64) * (size_t)slots);
+    const cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(u64) * (size_t)slots, stream);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((most + kClassThreads - 1) / kClassThreads), (unsigned)n_nt);
+    chain(class_insert_kernel, grid, kClassThreads, 0, stream, job);
+    chain(class_number_kernel, grid, kClassThreads, 0, stream, job);
+    chain(class_member_kernel, grid, kClassThreads, 0, stream, job);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,97 @@
+"""Searches over operand classes (operands that no probe tells apart are met once, and taken apart where a candidate
+passes): against the oracle, and cut into rank windows small enough to be searched operand by operand."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.util import check_sketch
+from xp_instances import Hole, Sketch, Variable, constant_set, free_grammar, parse_expr, quasi_affine_grammar
+
+pytestmark = pytest.mark.gpu
+
+VS = [Variable("i", 0, 9), Variable("j", 0, 7)]
+
+
+@pytest.mark.parametrize("ops,consts", [
+    (["+", "-", "*", "/", "%"], constant_set(-13, 13)),                       # 4 205 operands of three nodes: just enough for classes
+    (["+", "-", "*", "min", "max", "%"], constant_set(-9, 12) + [1 << 20, 5]),
+    (["+", "*", "<<", ">>", "/"], constant_set(-4, 24)),                      # undefined shifts and divisions
+])
+@pytest.mark.parametrize("ctx,spec", [("i<HOLE", "i<((j*2)+1)"), ("HOLE<=j", "(i/3)<=j"), ("(j-HOLE)<(i-2)", "(i%4)<5")])
+def test_comparing_contexts(xp, ops, consts, ctx, spec):
+    g = free_grammar(VS, sorted(set(consts)), ops=ops)
+    check_sketch(xp, Sketch(g, [Hole(0, 5, ctx=parse_expr(ctx, VS), spec_expr=parse_expr(spec, VS))], name=f"{ctx}: {spec}"))
+
+
+def _large(spec, ops=("+", "-", "*", "/", "%"), consts=None, ctx=None):
+    """45 leaves, operators five at the root: the operands of five nodes of a search up to seven are above the tables."""
+    g = free_grammar(VS, consts or constant_set(-17, 25), ops=list(ops))
+    return Sketch(g, [Hole(0, 7, ctx=parse_expr(ctx, VS) if ctx else [], spec_expr=parse_expr(spec, VS))], name=spec)
+
+
+@pytest.mark.parametrize("sk", [
+    _large("((i*7)+j)*3"),
+    _large("(i/2)+(j%3)"),                                                    # small targets: most divisors are open
+    _large("min(i*3,j+4)", ops=("+", "-", "*", "min", "max")),
+    _large("(i*9)+j", consts=constant_set(-10, 30) + [1 << 20, 1 << 30]),     # operands beyond 31 bits
+    _large("(((i*3)+j)*8)+1", ctx="(HOLE*8)+1"),
+], ids=lambda s: s.name)
+def test_a_window_against_the_oracle(xp, sk):
+    """Windows wide enough to be searched by class, over both sides of a block's border, cut inside a class."""
+    gr = xp.xp_grammar_create(sk.grammar)
+    ls = xp.xp_sketch_load(gr, sk)
+    n = xp.xp_grammar_count(gr, 0, 7)[7]
+    width = min(n // 6, 60_000_000)
+    for begin in (n // 9, 3 * n // 5 + 12_345):
+        w = {7: (begin, begin + width)}
+        got = xp.xp_repair(ls, size_min=7, size_max=7, rank_ranges=[(0, 7, *w[7])])[0]
+        want = oracle.repair_hole(sk, 0, rank_ranges={**{k: (0, 0) for k in range(1, 7)}, **w})
+        assert got.match_count[7] == want.match_count[7], (sk.name, begin)
+        if want.match_count[7]:
+            assert (got.least_rank, got.least_text) == (want.least_rank, want.least_text)
+
+
+def _cut(xp, ls, size, n, parts):
+    """Matches and least rank at `size`, searched in rank windows."""
+    match, least = 0, None
+    for p in range(parts):
+        r = xp.xp_repair(ls, size_min=size, size_max=size, rank_ranges=[(0, size, n * p // parts, n * (p + 1) // parts)])[0]
+        match += r.match_count[size]
+        if r.match_count[size] and least is None:
+            least = r.least_rank
+    return match, least
+
+
+@pytest.mark.parametrize("spec", ["((i*7)+j)*3", "(i/2)+(j%3)", "((i+j)%5)*2"])
+def test_free_grammar_equals_its_windows(xp, spec):
+    sk = _large(spec)
+    gr = xp.xp_grammar_create(sk.grammar)
+    ls = xp.xp_sketch_load(gr, sk)
+    n = xp.xp_grammar_count(gr, 0, 7)[7]
+    r = xp.xp_repair(ls, size_min=7, size_max=7)[0]
+    match, least = _cut(xp, ls, 7, n, 61)
+    assert match > 0 and r.match_count[7] == match and r.least_rank == least
+    xp.xp_sketch_refine(ls)                              # other probes, other classes, the same answer
+    again = xp.xp_repair(ls)[0]
+    assert again.match_count[7] == match
+
+
+@pytest.mark.parametrize("table", [False, True])
+def test_quasi_affine_grammar_equals_its_windows(xp, table):
+    """Classes of five nodes under operands of seven (typed grammar, three nonterminals), over a box and a table of points."""
+    vs = [Variable("i", 0, 40), Variable("j", 0, 30)]
+    g = quasi_affine_grammar(vs, constant_set(-40, 40), list(range(1, 51)))
+    spec = "((i/3)*5)+(j%4)"
+    if table:
+        r = np.random.default_rng(3)
+        coords = np.stack([r.integers(0, 40, 333), r.integers(0, 30, 333)], axis=1).astype(np.int32)
+        want = (coords[:, 0].astype(np.int64) // 3) * 5 + coords[:, 1] % 4
+        sk = Sketch(g, [Hole(0, 9, spec_table=want)], coords)
+    else:
+        sk = Sketch(g, [Hole(0, 9, spec_expr=parse_expr(spec, vs))])
+    gr = xp.xp_grammar_create(g)
+    ls = xp.xp_sketch_load(gr, sk)
+    n = xp.xp_grammar_count(gr, 0, 9)[9]
+    r = xp.xp_repair(ls, size_min=9, size_max=9)[0]
+    match, least = _cut(xp, ls, 9, n, 64)
+    assert match > 0 and r.match_count[9] == match and r.least_rank == least
