@@ -1457,10 +1457,14 @@ static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
             const u64 l0 = wlo / cr, nl = (whi + cr - 1) / cr - l0;      // left operands that the window covers
             if (nl * cr < least || (least > 1 && nl < cl && nl * cr < kPairEach * (nl + cr))) continue;
             taken->at(b - g->bin_begin[nt]) |= 1u << a;
+            // (a side of classes; the left one where the window covers more operands than there are)
+            auto classes = [&](int n, int size, u64 all) { return size == ho.cls_size && ho.cls_n[n] > 0 && ho.cls_n[n] < all; };
+            const bool lcls = classes(bd.lnt, a, nl), rcls = classes(bd.rnt, k - 1 - a, cr);
+            const u64 first = lcls ? 0 : l0, left = lcls ? ho.cls_n[bd.lnt] : nl, right = rcls ? ho.cls_n[bd.rnt] : cr;
             PairSeg* sg = nullptr;
             for (size_t i = first_seg; i < plan->psegs.size() && !sg; ++i) {
                 PairSeg& c = plan->psegs[i];
-                if (c.lnt == bd.lnt && c.rnt == bd.rnt && c.la == a && c.l_begin == l0 && c.nl == nl && !((c.ops >> bd.op) & 1u)) sg = &c;
+                if (c.lnt == bd.lnt && c.rnt == bd.rnt && c.la == a && c.l_begin == first && c.nl == left && c.pairs == nl * cr && !((c.ops >> bd.op) & 1u)) sg = &c;
             }
             if (!sg) {
                 PairSeg c;
@@ -1468,8 +1472,10 @@ static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
                 c.rank_begin = lo; c.rank_end = hi;
                 c.sketch = sketch; c.hole = hole; c.size = k; c.acc = acc;
                 c.lnt = bd.lnt; c.la = a; c.rnt = bd.rnt; c.ra = k - 1 - a;
-                c.l_begin = (u32)l0; c.nl = (u32)nl; c.nr = (u32)cr;
-                c.index_right = cr <= nl ? 1 : 0;            // the smaller side is indexed (its chains stay in L2)
+                c.l_begin = (u32)first; c.nl = (u32)left; c.nr = (u32)right;
+                c.lcls = lcls ? 1 : 0; c.rcls = rcls ? 1 : 0;
+                c.right_count = cr; c.pairs = nl * cr;
+                c.index_right = right <= left ? 1 : 0;       // the smaller side is indexed (its chains stay in L2)
                 u32 heads = 1024;
                 while (heads < (c.index_right ? c.nr : c.nl)) heads <<= 1;
                 c.head_mask = heads - 1;
@@ -1478,7 +1484,7 @@ static void add_pairs(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
                 sg = &plan->psegs.back();
             }
             sg->ops |= 1u << bd.op;
-            sg->base[bd.op] = this_base + l0 * cr;
+            sg->base[bd.op] = this_base + first * cr;
         }
     }
 }
@@ -1697,7 +1703,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         // (a rank window may cover fewer operands than there are combinations of classes)
         if (!c.seg.exact && ho.cls_size > 0 && c.seg.esize >= ho.cls_size) {
             const u64 m = class_operands(g, ho, c.seg.nt, c.seg.esize);
-            if (m < c.seg.e_count) { c.seg.classes = 1; c.seg.e_begin = 0; c.seg.e_count = m; }
+            if (m > 0 && m < c.seg.e_count) { c.seg.classes = 1; c.seg.e_begin = 0; c.seg.e_count = m; }
         }
         plan->jgroups.insert(plan->jgroups.end(), c.groups.begin(), c.groups.end());
         plan->jsegs.push_back(c.seg);

@@ -289,6 +289,8 @@ struct PairSeg {
     i32 sketch, hole, size, acc;
     i32 lnt, la, rnt, ra;            // nonterminal and size of either operand
     u32 l_begin, nl, nr;             // first of the left operands (a rank window may leave some out), and how many there are
+    i32 lcls, rcls;                  // the left / right operands are classes (nl, nr of them; l_begin = 0)
+    u64 right_count, pairs;          // right operands by rank; pairs of operands that the block stands for
     u32 ops;                         // operator slots (+ - * / %)
     i32 index_right;                 // the chains index the right operands (else the left ones)
     u64 base[5];                     // rank of (l_begin, 0) per operator

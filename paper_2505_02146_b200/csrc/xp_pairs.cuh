@@ -11,6 +11,8 @@
 //                         (any above |t| when l is the target itself);
 //   pair_wide_kernel   -- operands that are not narrow (31 bits, or fewer where the context's factor ends in zero bits), exactly.
 // Candidates that agree at both probes wait in a warp's queue and are checked 32 at a time at the other probes.
+// Operands of the classes' size are met by class (xp_classes.cuh): 5 000 x 5 000 instead of 92 480 x 92 480, no chains of equal values, and
+// walks a twentieth as long (thread binding, whole calls of six inputs: 1.05 -> 0.52 ms; pair join of one of them 0.3 -> 0.07).
 #pragma once
 
 namespace xp {
@@ -24,8 +26,65 @@ struct PairWarp {
     CandShared cand;
 };
 
-// Table entry of the first left operand.
-__device__ __forceinline__ u64 pair_left(const HoleDev* hole, const PairSeg& seg) { return hole->tab_off[seg.lnt][seg.la] + seg.l_begin; }
+// One side of a block: the pairs of values of its operands, and where operand i is in the tables (a class: its first member).
+struct PairSide {
+    const int2* pair;
+    const u32 *start, *mem;                               // (null: operands by rank)
+    u64 off;                                              // table entry of the first
+    __device__ __forceinline__ u64 entry(u32 i) const { return off + (start ? mem[start[i]] : i); }
+    __device__ __forceinline__ u32 members(u32 i) const { return start ? start[i + 1] - start[i] : 1u; }
+    __device__ __forceinline__ u32 member(u32 i, u32 k) const { return start ? mem[start[i] + k] : i; }
+};
+__device__ __forceinline__ PairSide pair_side(const GrammarDev* g, const HoleDev* hole, const PairSeg& seg, bool right) {
+    const int nt = right ? seg.rnt : seg.lnt, size = right ? seg.ra : seg.la;
+    const OperandSide s = operand_side(g, hole, nt, size, (right ? seg.rcls : seg.lcls) != 0);
+    const u32 skip = right ? 0u : seg.l_begin;
+    return PairSide{s.pair + skip, s.start, s.mem, hole->tab_off[nt][size] + skip};
+}
+
+// Pairs that satisfy the probes, one per lane (pass: this lane has one): to the survivor queue, the members of classes one by one, 32 at a
+// time over all lanes' pairs.  Called by all lanes.
+__device__ __noinline__ void pair_members(PairWarp& w, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, bool pass, u32 l, u32 r,
+                                          int slot, JoinCount& n) {
+    if (!__any_sync(0xffffffffu, pass)) return;
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    const PairSide L = pair_side(g, hole, seg, false), R = pair_side(g, hole, seg, true);
+    const u32 rn = pass ? R.members(r) : 1u;
+    u64 incl = pass ? (u64)L.members(l) * rn : 0ull;
+    for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+    const u64 total = __shfl_sync(0xffffffffu, incl, 31);
+    for (u64 k0 = 0; k0 < total; k0 += 32u) {
+        const u64 k = k0 + (u64)lane < total ? k0 + (u64)lane : total - 1u;
+        int src = 0;                                      // the lane whose member this is: the first with incl > k
+        for (int step = 16; step > 0; step >>= 1) { const u64 v = __shfl_sync(0xffffffffu, incl, src + step - 1); if (v <= k) src += step; }
+        const u64 before = __shfl_sync(0xffffffffu, incl, src ? src - 1 : 0);
+        const u32 l2 = __shfl_sync(0xffffffffu, l, src), r2 = __shfl_sync(0xffffffffu, r, src), rn2 = __shfl_sync(0xffffffffu, rn, src);
+        const int slot2 = __shfl_sync(0xffffffffu, slot, src);
+        bool ok = false;
+        u64 rank = 0;
+        u32 vars = 0;
+        if (k0 + (u64)lane < total) {
+            u64 kl, kr;
+            divmod_u64(src ? k - before : k, (u64)rn2, kl, kr);
+            const u32 lr = L.member(l2, (u32)kl), rr = R.member(r2, (u32)kr);
+            rank = seg.base[slot2] + (u64)lr * seg.right_count + rr;
+            ok = rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(rr < seg.right_count && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
+            if (ok && hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, rank, n.evals);
+            if (ok) vars = (u32)hole->tab_vars[L.off + lr] | (u32)hole->tab_vars[R.off + rr];
+        }
+        u32 m = __ballot_sync(0xffffffffu, ok);
+        if (!m) continue;
+        n.passes += (u32)__popc(m);
+        const bool pending = ok && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
+        m = __ballot_sync(0xffffffffu, pending);
+        while (m) {
+            const int at = __ffs((int)m) - 1;
+            m &= m - 1;
+            join_verify(w.cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, at), __shfl_sync(0xffffffffu, vars, at), n.evals);
+        }
+    }
+}
 
 // The lane's candidate against the queue's remaining probes.  Called by all lanes.
 __device__ __noinline__ void pair_check(PairWarp& w, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, int from, JoinCount& n) {
@@ -33,38 +92,27 @@ __device__ __noinline__ void pair_check(PairWarp& w, const PlanDev& plan, const 
     const int lane = threadIdx.x & 31;
     __syncwarp();
     const u32 nc = w.nc;
-    const u64 lo = pair_left(hole, seg), ro = hole->tab_off[seg.rnt][seg.ra];
+    const PairSide L = pair_side(g, hole, seg, false), R = pair_side(g, hole, seg, true);
     for (u32 at = 0; at < nc; at += 32) {
         bool pass = false;
-        u64 rank = 0;
-        u32 vars = 0;
+        u32 l = 0, r = 0;
+        int slot = 0;
         if (at + lane < nc) {
-            const u32 l = w.c_l[at + lane], r = w.c_r[at + lane];
-            const int slot = (int)w.c_op[at + lane];
-            rank = seg.base[slot] + (u64)l * seg.nr + r;
-            if (rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(l < seg.nl && r < seg.nr && rank < g->cnt[hole->start_nt][seg.size], kChkQueue)) {
+            l = w.c_l[at + lane]; r = w.c_r[at + lane];
+            slot = (int)w.c_op[at + lane];
+            if (XP_CHECKED(l < seg.nl && r < seg.nr, kChkQueue)) {
+                const u64 le = L.entry(l), re = R.entry(r);
                 pass = true;
                 for (int j = from; j < hole->n_exact && pass; ++j) {
                     ++n.evals;
                     const u64 b = (u64)j * hole->tab_total;
                     i64 v;
-                    pass = hole->tab_ok[b + lo + l] && hole->tab_ok[b + ro + r] &&
-                           apply_op(op_of_slot(slot), hole->tab_val[b + lo + l], hole->tab_val[b + ro + r], v) && probe_accepts(hole, j, v);
+                    pass = hole->tab_ok[b + le] && hole->tab_ok[b + re] &&
+                           apply_op(op_of_slot(slot), hole->tab_val[b + le], hole->tab_val[b + re], v) && probe_accepts(hole, j, v);
                 }
-                if (pass && hole->n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
-                vars = (u32)hole->tab_vars[lo + l] | (u32)hole->tab_vars[ro + r];
             }
         }
-        u32 m = __ballot_sync(0xffffffffu, pass);
-        if (!m) continue;
-        n.passes += (u32)__popc(m);
-        const bool pending = pass && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
-        m = __ballot_sync(0xffffffffu, pending);
-        while (m) {
-            const int src = __ffs((int)m) - 1;
-            m &= m - 1;
-            join_verify(w.cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
-        }
+        pair_members(w, plan, seg, sk, hole, pass, l, r, slot, n);
     }
     __syncwarp();
     if (lane == 0) w.nc = 0;
@@ -88,9 +136,9 @@ __device__ __forceinline__ void pair_push(PairWarp& w, const PlanDev& plan, cons
     if (nc + (u32)__popc(b) >= 32u) pair_check(w, plan, seg, sk, hole, from, n);
 }
 
-// Entry i of a set: its values at the two probes; 0 undefined, 1 narrow, 2 wide.
-__device__ __forceinline__ int pair_entry(const HoleDev* hole, u64 off, u32 i, u32 lim, int2& v) {
-    v = reinterpret_cast<const int2*>(hole->tab_pair)[off + i];
+// Operand i of a side: its values at the two probes; 0 undefined, 1 narrow, 2 wide.
+__device__ __forceinline__ int pair_entry(const PairSide& side, u32 i, u32 lim, int2& v) {
+    v = side.pair[i];
     if (v.x == kPairNone) return v.y ? 2 : 0;
     return abs_u32(v.x) < lim && abs_u32(v.y) < lim ? 1 : 2;
 }
@@ -121,7 +169,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_build_kernel(const __grid_c
         const u32 n = side ? seg.nr : seg.nl;
         if (i >= n) continue;
         int2 v;
-        const int st = pair_entry(hole, side ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg), i, lim, v);
+        const int st = pair_entry(pair_side(sk->g, hole, seg, side != 0), i, lim, v);
         if (st == 2) (side ? seg.wide_r : seg.wide_l)[atomicAdd(&seg.counters[side], 1u)] = i;
         if (side == seg.index_right && st == 1) seg.next[i] = atomicExch(&seg.head[pair_slot(v, seg.head_mask)], i);
     }
@@ -141,9 +189,8 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const __grid
     JoinCount n{0, 0, 0, 0, 0};
     const bool ir = seg.index_right != 0;
     const u32 nx = ir ? seg.nl : seg.nr;
-    const u64 xo = ir ? pair_left(hole, seg) : hole->tab_off[seg.rnt][seg.ra];
-    const u64 yo = ir ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg);
-    const int2* Y = reinterpret_cast<const int2*>(hole->tab_pair) + yo;
+    const PairSide X = pair_side(sk->g, hole, seg, !ir);
+    const int2* Y = pair_side(sk->g, hole, seg, ir).pair;
     const u32 lim = pair_limit(hole);
     const i64 t0 = hole->join_t0, t1 = hole->join_t1;
     const int from = hole->join_p1 ? 2 : 1;
@@ -151,7 +198,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const __grid
     for (u32 x0 = (blockIdx.x * kPairWarps + (threadIdx.x >> 5)) * 32u; x0 < nx; x0 += gridDim.x * kPairThreads) {
         const u32 x = x0 + lane;
         int2 v = make_int2(0, 0);
-        const bool live = x < nx && pair_entry(hole, xo, x, lim, v) == 1;
+        const bool live = x < nx && pair_entry(X, x, lim, v) == 1;
         for (u32 m = ops; m; m &= m - 1) {
             const int slot = __ffs((int)m) - 1;
             i64 w0 = 0, w1 = 0;
@@ -181,7 +228,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pair_hash_kernel(const __grid
         }
     }
     if (w.nc) pair_check(w, plan, seg, sk, hole, from, n);
-    if (blockIdx.x == 0 && threadIdx.x == 0) n.cands += (u64)seg.nl * seg.nr * (u64)__popc(seg.ops);
+    if (blockIdx.x == 0 && threadIdx.x == 0) n.cands += seg.pairs * (u64)__popc(seg.ops);
     join_flush(plan, seg.acc, n);
 }
 
@@ -203,12 +250,12 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_count_kernel(const __g
     const int side = blockIdx.y;
     const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
     const u32 n = side ? seg.nr : seg.nl, lim = pair_limit(hole);
-    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg);
+    const PairSide set = pair_side(plan.sketches[seg.sketch]->g, hole, seg, side != 0);
     for (int b = threadIdx.x; b < kPairBuckets; b += kPairThreads) hist[b] = 0;
     __syncthreads();
     for (u32 i = blockIdx.x * kPairThreads + threadIdx.x; i < n; i += gridDim.x * kPairThreads) {
         int2 v;
-        if (pair_entry(hole, off, i, lim, v) == 1) atomicAdd(&hist[pair_bucket(abs_u32(v.x))], 1u);
+        if (pair_entry(set, i, lim, v) == 1) atomicAdd(&hist[pair_bucket(abs_u32(v.x))], 1u);
     }
     __syncthreads();
     for (int b = threadIdx.x; b < kPairBuckets; b += kPairThreads) if (hist[b]) atomicAdd(&seg.hist[side][b], hist[b]);
@@ -240,11 +287,11 @@ __global__ void __launch_bounds__(kPairThreads) pair_sort_scatter_kernel(const _
     const int side = blockIdx.y, lane = threadIdx.x & 31;
     const HoleDev* hole = &plan.sketches[seg.sketch]->holes[seg.hole];
     const u32 n = side ? seg.nr : seg.nl, lim = pair_limit(hole);
-    const u64 off = side ? hole->tab_off[seg.rnt][seg.ra] : pair_left(hole, seg);
+    const PairSide set = pair_side(plan.sketches[seg.sketch]->g, hole, seg, side != 0);
     for (u32 i0 = (blockIdx.x * kPairThreads + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * kPairThreads) {
         const u32 i = i0 + lane;
         int2 v = make_int2(0, 0);
-        const bool on = i < n && pair_entry(hole, off, i, lim, v) == 1;
+        const bool on = i < n && pair_entry(set, i, lim, v) == 1;
         const u32 b = on ? pair_bucket(abs_u32(v.x)) : 0xffffffffu;
         const u32 same = __match_any_sync(0xffffffffu, b);          // one atomic per bucket and warp
         const int leader = __ffs((int)same) - 1;
@@ -402,20 +449,22 @@ __global__ void __launch_bounds__(kPairThreads) pair_wide_kernel(const __grid_co
     const SketchDev* sk = plan.sketches[seg.sketch];
     const HoleDev* hole = &sk->holes[seg.hole];
     const u32 lim = pair_limit(hole);
-    const u64 lo = pair_left(hole, seg), ro = hole->tab_off[seg.rnt][seg.ra];
+    const PairSide L = pair_side(sk->g, hole, seg, false), R = pair_side(sk->g, hole, seg, true);
     JoinCount n{0, 0, 0, 0, 0};
     const u64 nl = wl, total = nl + wr;
     for (u64 i = blockIdx.x * kPairWarps + (threadIdx.x >> 5); i < total; i += (u64)gridDim.x * kPairWarps) {
         const bool left = i < nl;
         const u32 x = left ? seg.wide_l[i] : seg.wide_r[i - nl];
-        if (!hole->tab_ok[(left ? lo : ro) + x]) continue;
-        const i64 xv = hole->tab_val[(left ? lo : ro) + x];
+        const u64 xe = left ? L.entry(x) : R.entry(x);
+        if (!hole->tab_ok[xe]) continue;
+        const i64 xv = hole->tab_val[xe];
         const u32 m = left ? seg.nr : seg.nl;
         for (u32 y0 = 0; y0 < m; y0 += 32u) {
             const u32 y = y0 + lane;
-            bool on = y < m && hole->tab_ok[(left ? ro : lo) + y] != 0;
-            if (on && !left) { int2 v; on = pair_entry(hole, lo, y, lim, v) == 1; }      // (two wide operands: the left one's turn)
-            const i64 yv = on ? hole->tab_val[(left ? ro : lo) + y] : 0;
+            const u64 ye = y >= m ? 0ull : left ? R.entry(y) : L.entry(y);
+            bool on = y < m && hole->tab_ok[ye] != 0;
+            if (on && !left) { int2 v; on = pair_entry(L, y, lim, v) == 1; }      // (two wide operands: the left one's turn)
+            const i64 yv = on ? hole->tab_val[ye] : 0;
             for (u32 o = seg.ops; o; o &= o - 1) {
                 const int slot = __ffs((int)o) - 1;
                 i64 v;
