@@ -53,9 +53,8 @@ struct JointDev {
     // the search from one side: context coefficients per probe, part 1's chains, the listed pairs
     u64 A0[kJointProbes], A1[kJointProbes], B[kJointProbes];
     u32 undefined, head_mask;                             // undefined: bit j: a hole-free part of the context is undefined at probe j
-    u32* head;                                            // device, all ones at launch
-    u32* next;
-    u64* key;
+    u32* head;                                            // device, all ones at launch: (head_mask + 1) x lanes per candidate
+    uint4* node;                                          // per candidate of part 1: key (low, high word), next in its chain
     uint2* list;                                          // device, kJointList entries (candidate of part 0, of part 1)
     // results, read back together
     u64 match_count[kJointTotal + 1];
@@ -156,41 +155,59 @@ __device__ __forceinline__ int joint_locate(const JointDev* J, int part, u64 e, 
     return s;
 }
 
+// LANES threads per candidate, each with every LANES-th probe: sixteen evaluations one after the other were the kernel's whole time where
+// there are few candidates (5 000: 18 us for part 1, now 7), and unranking the candidate once per lane is what the others
+// pay for it where there are many.
+// The lanes of a candidate of part 0 also share the partners: a key has a chain for every LANES-th candidate of part 1, and each lane walks
+// one (five thousand candidates, a few hundred with the same key: 150 us in one chain, now 20).
+constexpr u64 kJointSpread = 1ull << 16;                  // candidates of either part up to which 16 lanes share one
+template <int LANES>
 __global__ void __launch_bounds__(128) joint_key_kernel(JointDev* J, int part) {
     chain_wait();
     const SketchDev* sk = J->sk;
     const GrammarDev* g = sk->g;
-    const u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x;
-    const int np = J->n_probe;
+    const u64 e = ((u64)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+    const int np = J->n_probe, sub = (int)(threadIdx.x % LANES);
     const u32 all = np >= 32 ? 0xffffffffu : (1u << np) - 1u;
     if ((J->spec_ok & all) != all || (J->undefined & all) != 0u) return;      // nothing can match
     u32 ran = 0;
-    u64 key = 0x243F6A8885A308D3ull;
+    u64 key = 0;
     bool ok = e < J->tab_total[part];
     if (ok) {
         u64 rank;
         const int s = joint_locate(J, part, e, rank);
         u32 code[kMaxSize];
         const int n = unrank(g, J->start_nt[part], s, rank, code);
-        for (int j = 0; j < np && ok; ++j) {
+#pragma unroll 1
+        for (int j = sub; j < np && ok; j += LANES) {
             i64 h;
             ++ran;
             ok = eval_cand(code, n, g->leaves, J->probe_pt[j], h);
-            const u64 v = part ? J->A1[j] * (u64)h : (u64)J->probe_spec[j] - J->B[j] - J->A0[j] * (u64)h;
-            key = (key ^ v) * 0x9E3779B97F4A7C15ull;
-            key ^= key >> 29;
+            u64 v = part ? J->A1[j] * (u64)h : (u64)J->probe_spec[j] - J->B[j] - J->A0[j] * (u64)h;
+            v = (v + (u64)(j + 1) * 0x9E3779B97F4A7C15ull) * 0xD1342543DE82EF95ull;      // (a sum over the probes, in any order)
+            v = (v ^ (v >> 32)) * 0xDA942042E4DD58B5ull;
+            key += v ^ (v >> 29);
         }
     }
+    if (LANES > 1) {
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) key += __shfl_xor_sync(0xffffffffu, key, o);
+        const u32 mine = ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) & ~(LANES - 1));
+        ok = (__ballot_sync(0xffffffffu, ok) & mine) == mine && (part == 0 || sub == 0);
+    }
     if (ok) {
-        u32* head = &J->head[(u32)(key >> 32) & J->head_mask];
-        if (part) { J->key[e] = key; J->next[e] = atomicExch(head, (u32)e); }
+        u32* head = &J->head[(((u32)(key >> 32) & J->head_mask) * LANES + (part ? (u32)(e % LANES) : (u32)sub))];
+        if (part) J->node[e] = make_uint4((u32)key, (u32)(key >> 32), atomicExch(head, (u32)e), 0u);
         else
-            for (u32 y = *head; y != 0xffffffffu; y = J->next[y])
-                if (J->key[y] == key) {                   // (an equal key that is no match fails on the domain, probes among it)
+            for (u32 y = *head; y != 0xffffffffu;) {
+                const uint4 q = J->node[y];
+                if (q.x == (u32)key && q.y == (u32)(key >> 32)) {      // (an equal key that is no match fails on the domain, probes among it)
                     const u64 at = atomicAdd((unsigned long long*)&J->listed, 1ull);
                     if (at >= kJointList) break;          // (the host takes the other form)
                     J->list[at] = make_uint2((u32)e, y);
                 }
+                y = q.z;
+            }
     }
     for (int o = 16; o > 0; o >>= 1) ran += __shfl_down_sync(0xffffffffu, ran, o);
     if ((threadIdx.x & 31) == 0 && ran) atomicAdd((unsigned long long*)&J->evals, (u64)ran);
@@ -214,17 +231,19 @@ __global__ void __launch_bounds__(256) joint_values_kernel(JointDev* J, int part
 }
 
 // The pair (tree r0 of size s0, tree r1 of size s1) on every domain point; called by all 32
-// lanes of a warp together.  Adds the points tried to evals.
+// lanes of a warp together, or by all threads of a CTA.  Adds the points tried to evals.
+template <bool CTA>
 __device__ __noinline__ bool joint_check_domain(const JointDev* J, int s0, u64 r0, int s1, u64 r1, u64& evals) {
     const SketchDev* sk = J->sk;
     const GrammarDev* g = sk->g;
-    const int lane = threadIdx.x & 31;
+    const int width = CTA ? (int)blockDim.x : 32;
     u32 c0[kMaxSize], c1[kMaxSize];
     const int n0 = unrank(g, J->start_nt[0], s0, r0, c0);
     const int n1 = unrank(g, J->start_nt[1], s1, r1, c1);
-    for (i64 base = 0; base < sk->n_points; base += 32) {
+#pragma unroll 1
+    for (i64 base = 0; base < sk->n_points; base += width) {
         bool bad = false;
-        const i64 pid = base + lane;
+        const i64 pid = base + (CTA ? (int)threadIdx.x : (int)(threadIdx.x & 31));
         if (pid < sk->n_points) {
             ++evals;
             i64 pt[kMaxVars];
@@ -237,7 +256,7 @@ __device__ __noinline__ bool joint_check_domain(const JointDev* J, int s0, u64 r
                  eval_joint(J->ctx, J->ctx_len, pt, h0, h1, v) && v == want;
             bad = !ok;
         }
-        if (__any_sync(0xffffffffu, bad)) return false;
+        if (CTA ? __syncthreads_or(bad) != 0 : __any_sync(0xffffffffu, bad)) return false;
     }
     return true;
 }
@@ -273,7 +292,7 @@ __global__ void __launch_bounds__(256) joint_pairs_kernel(JointDev* J, int s0, i
             const int src = __ffs((int)m) - 1;
             m &= m - 1;
             const u64 x0 = __shfl_sync(0xffffffffu, r0, src), x1 = __shfl_sync(0xffffffffu, r1, src);
-            if (joint_check_domain(J, s0, x0, s1, x1, evals) && lane == 0) {
+            if (joint_check_domain<false>(J, s0, x0, s1, x1, evals) && lane == 0) {
                 atomicAdd(&J->match_count[s0 + s1], 1ull);
                 atomicMin(&J->min_key[s0 + s1], ((u64)s0 << 48) | (x0 << 24) | x1);
             }
@@ -286,16 +305,19 @@ __global__ void __launch_bounds__(256) joint_pairs_kernel(JointDev* J, int s0, i
     }
 }
 
-// A warp per listed pair.
+// A CTA per listed pair while every CTA has few of them, a warp per pair where there are many: a pair's domain is a chain of steps that each
+// wait for the interpreter (480 points in 15 steps of a warp: 51 us, in 2 of a CTA: 14).
 __global__ void __launch_bounds__(256) joint_check_kernel(JointDev* J) {
     chain_wait();
     const u64 n = J->listed;
     if (n > kJointList) return;                           // (the list ran over: the host takes the other form)
+    const bool wide = n <= 4ull * gridDim.x;
     u64 evals = 0;
-    for (u64 i = (u64)blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += (u64)gridDim.x * 8) {
+    for (u64 i = wide ? (u64)blockIdx.x : (u64)blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += wide ? (u64)gridDim.x : (u64)gridDim.x * 8) {
         u64 r0, r1;
         const int s0 = joint_locate(J, 0, J->list[i].x, r0), s1 = joint_locate(J, 1, J->list[i].y, r1);
-        if (joint_check_domain(J, s0, r0, s1, r1, evals) && (threadIdx.x & 31) == 0) {
+        const bool ok = wide ? joint_check_domain<true>(J, s0, r0, s1, r1, evals) : joint_check_domain<false>(J, s0, r0, s1, r1, evals);
+        if (ok && (threadIdx.x & (wide ? 255 : 31)) == 0) {
             atomicAdd(&J->match_count[s0 + s1], 1ull);
             atomicMin(&J->min_key[s0 + s1], ((u64)s0 << 48) | (r0 << 24) | r1);
         }
@@ -437,13 +459,14 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
         size_t off = al(sizeof(JointDev));
         const size_t off_spec = off;
         if (copy_spec) off += al(sizeof(i64) * (size_t)si.n_points);
-        size_t off_val[2] = {0, 0}, off_ok[2] = {0, 0}, off_head = 0, off_next = 0, off_key = 0, off_list = 0;
+        size_t off_val[2] = {0, 0}, off_ok[2] = {0, 0}, off_head = 0, off_node = 0, off_list = 0;
+        const bool spread = entries[0] <= kJointSpread && entries[1] <= kJointSpread;
+        const u32 lanes = spread ? 16u : 1u;
         u32 heads = 1024;
-        while (heads < entries[1]) heads <<= 1;
+        while ((u64)heads * lanes < 2 * entries[1]) heads <<= 1;
         if (form == 0) {
-            off_head = off; off += al(sizeof(u32) * heads);
-            off_next = off; off += al(sizeof(u32) * entries[1]);
-            off_key = off; off += al(sizeof(u64) * entries[1]);
+            off_head = off; off += al(sizeof(u32) * heads * lanes);
+            off_node = off; off += al(sizeof(uint4) * entries[1]);
             off_list = off; off += al(sizeof(uint2) * kJointList);
         } else
             for (int k = 0; k < 2; ++k) {
@@ -463,7 +486,7 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
         if (d->spec_kind == XP_SPEC_EXPR) { h.spec_len = d->spec_len; memcpy(h.spec, d->spec_expr, sizeof(xp_instr) * d->spec_len); }
         else if (si.n_points > 0) h.spec_table = copy_spec ? (const i64*)(block + off_spec) : (const i64*)d->spec_table;
         for (int k = 0; k < 2; ++k) { h.tab_val[k] = (i64*)(block + off_val[k]); h.tab_ok[k] = (unsigned char*)(block + off_ok[k]); }
-        h.head = (u32*)(block + off_head); h.next = (u32*)(block + off_next); h.key = (u64*)(block + off_key); h.list = (uint2*)(block + off_list);
+        h.head = (u32*)(block + off_head); h.node = (uint4*)(block + off_node); h.list = (uint2*)(block + off_list);
         h.head_mask = heads - 1;
         for (int t = 0; t <= kJointTotal; ++t) h.min_key[t] = ~0ull;
         JointDev* dJ = (JointDev*)block;
@@ -471,7 +494,7 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
         cudaError_t e = ev.e0 ? cudaSuccess : ev.open();
         if (e == cudaSuccess) e = cudaMemcpyAsync(dJ, stage.p, sizeof(h), cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess && copy_spec) e = cudaMemcpyAsync(block + off_spec, d->spec_table, sizeof(i64) * (size_t)si.n_points, cudaMemcpyHostToDevice, stream);
-        if (e == cudaSuccess && form == 0) e = cudaMemsetAsync(block + off_head, 0xff, sizeof(u32) * heads, stream);
+        if (e == cudaSuccess && form == 0) e = cudaMemsetAsync(block + off_head, 0xff, sizeof(u32) * heads * lanes, stream);
         if (e == cudaSuccess) e = cudaEventRecord(ev.e0, stream);
         if (e == cudaSuccess) {
             chain(joint_probe_kernel, 1, 32, 0, stream, dJ, form == 0 ? 1 : 0);
@@ -481,7 +504,8 @@ extern "C" xp_status xp_repair_joint(const xp_sketch* sketch, const xp_joint_des
         if (form == 0) {
             for (int part = 1; part >= 0 && e == cudaSuccess; --part) {
                 if (entries[part] == 0) continue;
-                chain(joint_key_kernel, (unsigned)((entries[part] + 127) / 128), 128, 0, stream, dJ, part);
+                if (spread) chain(joint_key_kernel<16>, (unsigned)((entries[part] + 7) / 8), 128, 0, stream, dJ, part);
+                else chain(joint_key_kernel<1>, (unsigned)((entries[part] + 127) / 128), 128, 0, stream, dJ, part);
                 ++launches;
                 e = cudaGetLastError();
             }
