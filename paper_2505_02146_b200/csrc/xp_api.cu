@@ -1420,6 +1420,7 @@ constexpr size_t kPairFew = 2;               // sketches up to which kPairLeast 
 // A rank window cuts a block to some of its left operands, but the other side is indexed whole: a block with fewer rows than this,
 // or thereabouts, is done as tiles before the index is made (450 000 operands a side, remainders: 2 222 rows 0.26 ms, the index 1.9).
 constexpr u64 kPairEach = 1ull << 12;
+constexpr u64 kRangeSplit = 1ull << 15;      // ... up to which an operator is a segment of its own (with more there are warps enough at work)
 constexpr u64 kRangeMost = 1ull << 18;       // operands of a hole whose context compares from which the tiles take a leaf at the root too
 
 // Does the pair join know the block (production, left size a) of size k?  Both operands tabulated, an operator it has
@@ -1639,7 +1640,7 @@ static u64 class_operands(const xp_grammar* g, const HoleHost& ho, int nt, int s
 // Leaf-join segments of (start nonterminal, size k >= 3) restricted to ranks [lo, hi): one per operand nonterminal, with
 // a group per leaf nonterminal, for every operator with a leaf of it on either side of such an operand.  Copies of one
 // production open segments of their own; so do shifts, which only the exact form knows.
-static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi) {
+static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool few) {
     const int nt = ho.start_nt;
     const bool exact = ho.exact, compares = ho.compares;
     struct Open { JoinSeg seg; bool shifts; std::vector<JoinGroup> groups; };
@@ -1704,6 +1705,22 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         if (!c.seg.exact && ho.cls_size > 0 && c.seg.esize >= ho.cls_size) {
             const u64 m = class_operands(g, ho, c.seg.nt, c.seg.esize);
             if (m > 0 && m < c.seg.e_count) { c.seg.classes = 1; c.seg.e_begin = 0; c.seg.e_count = m; }
+        }
+        // An operand of a context that compares takes some hundred microseconds of a lane, and classes leave a few thousand of them: a
+        // segment per operator and side, so that as many warps share them (three conv holes: join 540 -> 430 us).
+        if (few && compares && !c.seg.exact && c.seg.e_count <= kRangeSplit) {
+            for (const JoinGroup& q : c.groups)
+                for (int b = 0; b < 2 * kOpSlots; ++b) {
+                    const int swap = b / kOpSlots, slot = b % kOpSlots;
+                    if (!(((swap ? q.smask : q.fmask) >> slot) & 1u)) continue;
+                    JoinGroup one = q;
+                    one.fmask = swap ? 0u : 1u << slot; one.smask = swap ? 1u << slot : 0u;
+                    c.seg.first_group = (i32)plan->jgroups.size();
+                    c.seg.n_groups = 1;
+                    plan->jgroups.push_back(one);
+                    plan->jsegs.push_back(c.seg);
+                }
+            continue;
         }
         plan->jgroups.insert(plan->jgroups.end(), c.groups.begin(), c.groups.end());
         plan->jsegs.push_back(c.seg);
@@ -1846,7 +1863,7 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 // (A range of hole values: the join's interval arithmetic per operand against a test per candidate.  27 leaves, size 7, 984 000
                 // operands, four specs: 13.4, 26.5, 10.2, 14.4 ms by the join, 14.9, 19.8, 10.7, 8.2 as tiles; 40 leaves, size 5: 0.4 against 1.4.)
                 const bool leaves = ho.compares && class_operands(s->g, ho, ho.start_nt, k - 2) > kRangeMost;
-                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi);
+                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, form != kFormMany);
                 const bool pairs = form >= kFormPairsSome;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
                 add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany, leaves);

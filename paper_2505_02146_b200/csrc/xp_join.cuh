@@ -196,7 +196,7 @@ __device__ __forceinline__ bool probes_accept(const HoleDev* hole, int j0, int n
 }
 
 // The candidate (operand, leaf) at the probes that have tables, in order; the first failure ends it.
-__device__ __forceinline__ bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
+__device__ __noinline__ bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
                                            bool swap, int op, int from, int n_exact, u64& evals) {
     for (int j = from; j < n_exact; ++j) {
         ++evals;
@@ -204,6 +204,31 @@ __device__ __forceinline__ bool exact_pair(const GrammarDev* g, const HoleDev* h
         if (!ref_value(g, hole, ref, nt, esize, j, a)) return false;
         const i64 c = var >= 0 ? hole->probe_pt[j][var] : cval;
         if (!apply_op(op, swap ? c : a, swap ? a : c, v) || !probe_accepts(hole, j, v)) return false;
+    }
+    return true;
+}
+
+// The same four probes at a time, for holes whose context compares: their candidates have passed the first four already, mostly pass all the
+// others, and one probe after the other waited 16 times for memory.
+__device__ __noinline__ bool exact_pair4(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
+                                         bool swap, int op, int from, int n_exact, u64& evals) {
+    for (int j0 = from; j0 < n_exact; j0 += kProbeStep) {
+        const int here = n_exact - j0 < kProbeStep ? n_exact - j0 : kProbeStep;
+        evals += (u64)here;
+        i64 v[kProbeStep];
+        if (ref_value4(g, hole, ref, nt, esize, j0, n_exact, v) != (1u << here) - 1u) return false;
+        bool ok = true;
+#pragma unroll 1
+        for (int k = 0; k < here; ++k) {
+            i64 a = v[0], r = 0;
+#pragma unroll
+            for (int q = 1; q < kProbeStep; ++q) if (q == k) a = v[q];
+            const i64 c = var >= 0 ? hole->probe_pt[j0 + k][var] : cval;
+            ok = apply_op(op, swap ? c : a, swap ? a : c, r) && ok;
+#pragma unroll
+            for (int q = 0; q < kProbeStep; ++q) if (q == k) v[q] = r;
+        }
+        if (!ok || !probes_accept(hole, j0, n_exact, v)) return false;
     }
     return true;
 }
@@ -301,8 +326,10 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
                 code = w.c_code[at + lane]; pos = w.c_pos[at + lane]; e = w.base + w.c_off[at + lane];
                 const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, class_operand(g, hole, seg.nt, seg.esize, e).rank(0));
                 const LeafDev lf = g->leaves[g->leaf_begin[plan.jgroups[seg.first_group + (int)(code >> 8)].leaf_nt] + (int)pos];
-                pass = exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, (code & 1u) != 0u, op_of_slot((int)((code >> 1) & 15u)), from,
-                                  hole->n_exact, n.evals);
+                const bool swap = (code & 1u) != 0u;
+                const int op = op_of_slot((int)((code >> 1) & 15u));
+                pass = hole->aff_ok ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals)
+                                    : exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals);
             }
             join_members(w, plan, seg, sk, hole, pass, e, pos, code, n);
             continue;
@@ -318,7 +345,8 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
                 XP_CHECKED(e < ne && (u64)pos < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue)) {
                 const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
                 const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
-                pass = exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals);
+                pass = hole->aff_ok ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals)
+                                    : exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals);
                 if (pass && hole->n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
                 vars = ref_vars(hole, ref) | (lf.var >= 0 ? 1u << lf.var : 0u);
             }
