@@ -206,14 +206,10 @@ __device__ void join_leaf_set(const GrammarDev* g, HoleDev* hole, int nt) {
     bad = bad || cabs >> 31 != 0;
     for (int o = 16; o > 0; o >>= 1) { const u64 q = __shfl_xor_sync(0xffffffffu, most, o); most = q > most ? q : most; }
     const bool ok = !__any_sync(0xffffffffu, bad);
-    bool member = false;                                  // lanes 0 and 1: is the target at probe 0 / 1 one of the constants?
-    if (lane < 2 && n_const > 0) {
-        const i64 v = lane ? t1 : t0;
-        int x = cb, y = vb;
-        while (x < y) { const int z = (x + y) >> 1; if (c[z].value < v) x = z + 1; else y = z; }
-        member = x < vb && c[x].value == v;
-    }
-    const u32 mm = __ballot_sync(0xffffffffu, member);
+    u32 mm = 0;                                           // is the target at probe 0 / 1 one of the constants?
+    if (n_const > 0)
+        for (int x = cb + lane; x < vb; x += 32) { const i64 v = c[x].value; mm |= (u32)(v == t0) | (u32)(v == t1) << 1; }
+    mm = __reduce_or_sync(0xffffffffu, mm);
     if (lane == 0) {
         S.n_entries = n > kJoinEntries ? 0 : n; S.n_const = n_const; S.const_begin = cb;
         S.cmin = ok ? (i32)lo : 0; S.cmax = ok ? (i32)hi : 0;
@@ -278,7 +274,7 @@ __device__ __forceinline__ void probe_contexts(const GrammarDev* g, HoleDev* hol
         }
     }
     __syncthreads();
-    if (t < 32) for (int nt = 0; nt < g->n_nt; ++nt) join_leaf_set(g, hole, nt);
+    for (int nt = t >> 5; nt < g->n_nt; nt += (int)(blockDim.x >> 5)) join_leaf_set(g, hole, nt);      // a warp each
 }
 
 // Choice of each hole's probe points, once per sketch.  A sample of small candidates (sizes 1, 3, 5, ranks spread evenly)
@@ -373,7 +369,7 @@ __global__ void __launch_bounds__(32 * kPrepWarps) prep_sample_kernel(const Load
     }
 }
 
-constexpr int kPrepThreads = 64;                        // one thread per sample
+constexpr int kPrepThreads = 128;                       // one thread per sample, a warp per nonterminal's leaf set
 __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jobs, const u32* masks, LoadOut* out) {
     chain_wait();
     SketchDev* s = jobs[blockIdx.x].s;
@@ -381,7 +377,7 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
     __shared__ i64 s_spec[kProbeSamples];
     __shared__ int s_ok[kProbeSamples];
     __shared__ u64 s_score[kProbeSamples];
-    __shared__ u32 s_mask[kProbeSamples][kPrepWords + 1];
+    __shared__ u32 s_mask[kProbeSamples][kPrepWords + 1];      // (rows past ns are never chosen)
     __shared__ int s_n, s_pass0;
     const int t = threadIdx.x, lane = t & 31;
     const int ns = s->n_samples, nv = s->n_vars;
@@ -401,39 +397,57 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
     const int ncand = prep_sizes(g, hole, sizes) > 0 ? kPrepCands : 0;
     __syncthreads();
     if (t < 32) {                                       // one warp picks: two samples per lane
-        u32 alive[kPrepWords];
+        constexpr int kEach = kProbeSamples / 32;
+        u32 mask[kEach][kPrepWords], alive[kPrepWords];
+#pragma unroll
+        for (int q = 0; q < kEach; ++q)
+#pragma unroll
+            for (int w = 0; w < kPrepWords; ++w) mask[q][w] = s_mask[lane + 32 * q][w];
+#pragma unroll
         for (int w = 0; w < kPrepWords; ++w) alive[w] = ncand ? 0xffffffffu : 0u;
         u64 chosen = 0;
         int n = 0, pass0 = 0, first = 0;
         u32 spec_ok = 0;
+#pragma unroll 1
         for (; n < kMaxProbe && n < ns; ++n) {
             u32 left = 0;
+#pragma unroll
             for (int w = 0; w < kPrepWords; ++w) left |= alive[w];
             if (n >= 2 && left == 0u) break;              // no sampled candidate is left: by score alone, all at once below
-            u64 best_key = ~0ull, best_score = 0;         // key: candidates that pass << 32 | 255 - difference from the first probe
-            int best = -1;
-            for (int i = lane; i < ns; i += 32) {
-                if ((chosen >> i) & 1ull) continue;
+            // The least (candidates that pass, 255 - difference from the first probe), then the largest score, then the least index: each of
+            // the four words by one reduction over the warp (a shuffled comparison of the whole key took 10 us for 16 probes).
+            u32 key[kEach], least = 0xffffffffu;
+#pragma unroll
+            for (int q = 0; q < kEach; ++q) {
+                const int i = lane + 32 * q;
                 u32 count = 0;
-                for (int w = 0; w < kPrepWords; ++w) count += (u32)__popc(alive[w] & s_mask[i][w]);
+#pragma unroll
+                for (int w = 0; w < kPrepWords; ++w) count += (u32)__popc(alive[w] & mask[q][w]);
                 u32 diff = 0;
-                if (n == 1) {
+                if (n == 1 && i < ns) {
+#pragma unroll 1
                     for (int d = 0; d < nv; ++d) diff += s_pt[i][d] != s_pt[first][d];
                     if (s_ok[i] && s_spec[i] != s_spec[first] && s_spec[i] != 0) diff += 16;
                 }
-                const u64 key = ((u64)count << 32) | (255u - diff);
-                if (best < 0 || key < best_key || (key == best_key && s_score[i] > best_score)) { best = i; best_key = key; best_score = s_score[i]; }
+                key[q] = i < ns && !((chosen >> i) & 1ull) ? (count << 8) | (255u - diff) : 0xffffffffu;
+                least = key[q] < least ? key[q] : least;
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                const u64 k2 = __shfl_xor_sync(0xffffffffu, best_key, o), sc2 = __shfl_xor_sync(0xffffffffu, best_score, o);
-                const int b2 = __shfl_xor_sync(0xffffffffu, best, o);
-                if (b2 >= 0 && (best < 0 || k2 < best_key || (k2 == best_key && (sc2 > best_score || (sc2 == best_score && b2 < best))))) {
-                    best = b2; best_key = k2; best_score = sc2;
-                }
-            }
+            least = __reduce_min_sync(0xffffffffu, least);
+            u64 score = 0;                                // of this lane's better one
+            int mine = kProbeSamples;
+#pragma unroll
+            for (int q = 0; q < kEach; ++q)
+                if (key[q] == least && (mine == kProbeSamples || s_score[lane + 32 * q] > score)) { mine = lane + 32 * q; score = s_score[mine]; }
+            bool in = mine < kProbeSamples;
+            const u32 hi = __reduce_max_sync(0xffffffffu, in ? (u32)(score >> 32) : 0u);
+            in = in && (u32)(score >> 32) == hi;
+            const u32 lo = __reduce_max_sync(0xffffffffu, in ? (u32)score : 0u);
+            in = in && (u32)score == lo;
+            const int best = (int)__reduce_min_sync(0xffffffffu, in ? (u32)mine : 0xffffffffu);
             chosen |= 1ull << best;
-            if (n == 0) { first = best; pass0 = (int)(best_key >> 32); }
+            if (n == 0) { first = best; pass0 = (int)(least >> 8); }
             if (s_ok[best]) spec_ok |= 1u << n;
+#pragma unroll
             for (int w = 0; w < kPrepWords; ++w) alive[w] &= s_mask[best][w];
             if (lane == 0) { hole->probe_id[n] = s->sample_id[best]; hole->probe_spec[n] = s_spec[best]; }
             if (lane < nv) hole->probe_pt[n][lane] = s_pt[best][lane];
