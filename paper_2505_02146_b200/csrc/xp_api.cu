@@ -1701,6 +1701,8 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         c.seg.first_group = (i32)plan->jgroups.size();
         c.seg.n_groups = (i32)c.groups.size();
         for (const JoinGroup& q : c.groups) if ((g->wide_leaf >> q.leaf_nt) & 1u) { c.seg.exact = kExactMany; c.seg.heavy = 1; }
+        for (const JoinGroup& q : c.groups) c.seg.leaves += (i32)g->cnt[q.leaf_nt][1];
+        if (c.seg.heavy) c.seg.leaves = 0;                // (these have forms of their own)
         // (a rank window may cover fewer operands than there are combinations of classes)
         if (!c.seg.exact && ho.cls_size > 0 && c.seg.esize >= ho.cls_size) {
             const u64 m = class_operands(g, ho, c.seg.nt, c.seg.esize);
@@ -1735,6 +1737,13 @@ static void add_direct(Plan* plan, int nt, int sketch, int hole, int acc, int k,
     plan->jsegs.push_back(sg);
 }
 
+// Small calls are bound by the chain of a ticket: conditions, suspects taken apart, probes one after the other.  Where all the
+// operands of a segment times its leaves are few, every one is tested at both probes instead (join_few), a ticket being 32 operands and a part
+// of the leaves, so that the call has a ticket for every warp.  (Two-variable nest, load and search:
+// 179 -> 168 us; tile bound 267 -> 213, expression pair 373 -> 313, means of five inputs, with the probes of a check four at a time.)
+constexpr u64 kFewPairs = 1ull << 20;        // (operand, leaf) pairs of a segment
+constexpr u64 kFewCall = 1ull << 23;         // ... and of all such segments of a call
+
 // Tickets of the leaf join.  A step is 32 operands (one per lane).  A ticket takes so
 // many steps that every warp of the device gets about four: fewer and the last wave is uneven, more and the
 // warps spend their time taking tickets.  64 steps at most.  In the exact form a ticket is one step, which costs as much as some
@@ -1747,6 +1756,10 @@ static void number_joins(Plan* plan) {
     u64 steps = 0, exact_steps = 0;
     for (const JoinSeg& c : plan->jsegs) (c.exact ? exact_steps : steps) += (c.e_count + 31) / 32;
     const u64 warps = (u64)search_warps();
+    u64 few_pairs = 0, few_steps = 0;
+    auto few = [](const JoinSeg& c) { return c.kind == kJoinLeaf && !c.exact && !c.heavy && !c.classes && c.leaves > 0 && c.e_count * (u64)c.leaves <= kFewPairs; };
+    for (const JoinSeg& c : plan->jsegs) if (few(c)) { few_pairs += c.e_count * (u64)c.leaves; few_steps += (c.e_count + 31) / 32; }
+    const u64 share = few_pairs <= kFewCall && few_steps > 0 ? (warps > few_steps ? warps / few_steps : 1) : 0;      // parts, if the leaves are enough
     const i32 form = exact_steps < 2 * warps ? kExactFew : kExactMany;
     u64 per = steps / (warps * 4);
     if (per < 1) per = 1;
@@ -1757,7 +1770,13 @@ static void number_joins(Plan* plan) {
         if (c.exact) c.exact = form;
         c.first_ticket = plan->n_join;
         c.chunk = (u32)(c.exact ? (form == kExactFew ? 1 : 32) : per * 32);
-        plan->n_join += (c.e_count + c.chunk - 1) / c.chunk;
+        c.parts = 0;
+        if (share && few(c)) {
+            const u64 most = ((u64)c.leaves + 3) / 4;
+            c.chunk = 32;
+            c.parts = (i32)(share < most ? share : most);
+        }
+        plan->n_join += (c.e_count + c.chunk - 1) / c.chunk * (u64)(c.parts > 0 ? c.parts : 1);
     }
 }
 

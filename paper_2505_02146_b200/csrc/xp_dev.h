@@ -258,6 +258,7 @@ struct JoinSeg {
     i32 exact;                       // kExactFew, kExactMany: there is no condition (shifts, a leaf of 2^31 or more), every candidate is evaluated on its own
     u32 chunk;                       // operands per ticket
     i32 heavy;                       // an operand costs many times the usual (exact form, contexts that compare): these go first
+    i32 leaves, parts;               // leaves of its groups; parts > 0: one ticket is 32 operands against one of so many parts of them (join_few)
     i32 classes, pad;                // operands are counted by class: e_begin = 0, e_count combinations of classes (class_operands)
     u64 e_begin, e_count;
 };

@@ -315,6 +315,8 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
     const int lane = threadIdx.x & 31;
     __syncwarp();
     const u32 nc = w.nc;
+    // (a call of one wave waits for this chain, and a candidate of a context that compares passes most probes: see exact_pair4)
+    const bool four = !hole->aff_ok || plan.n_join <= (u64)gridDim.x * kJoinWarps;
     for (u32 at = 0; at < nc; at += 32) {
         bool pass = false;
         u64 rank = 0;
@@ -328,7 +330,7 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
                 const LeafDev lf = g->leaves[g->leaf_begin[plan.jgroups[seg.first_group + (int)(code >> 8)].leaf_nt] + (int)pos];
                 const bool swap = (code & 1u) != 0u;
                 const int op = op_of_slot((int)((code >> 1) & 15u));
-                pass = hole->aff_ok ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals)
+                pass = !four ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals)
                                     : exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals);
             }
             join_members(w, plan, seg, sk, hole, pass, e, pos, code, n);
@@ -345,7 +347,7 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
                 XP_CHECKED(e < ne && (u64)pos < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue)) {
                 const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
                 const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
-                pass = hole->aff_ok ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals)
+                pass = !four ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals)
                                     : exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals);
                 if (pass && hole->n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
                 vars = ref_vars(hole, ref) | (lf.var >= 0 ? 1u << lf.var : 0u);
@@ -1299,6 +1301,71 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     __syncwarp();
 }
 
+// Operands [first, first + count), at most 32, against part `part` of the segment's leaves, for small calls: every operator at both probes, without
+// conditions and suspects in between (two-variable nest of 1 805 operands and 19 leaves, five operators: join 42 -> 28 us).
+__device__ __noinline__ void join_few(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, u64 first, u64 count,
+                                      int part, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int lane = threadIdx.x & 31;
+    i64 t0 = hole->join_t0, t1 = hole->join_t1;
+    const int p1 = hole->join_p1, from = p1 ? 2 : 1;
+    u32 lim = hole->join_on ? 0x7fffffffu : 0u, pairs = 0;
+    for (int gi = 0; gi < seg.n_groups; ++gi) {
+        const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+        const JoinSet* S = &hole->join_sets[grp.leaf_nt];
+        const u32 l = S->ok ? S->lim : 0u;
+        lim = l < lim ? l : lim;
+        pairs += (u32)g->cnt[grp.leaf_nt][1] * (u32)(__popc(grp.fmask) + __popc(grp.smask));
+    }
+    if (part == 0) n.cands += count * (u64)pairs;
+    for (u64 done = 0; done < count;) {
+        const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done, false);
+        const u32 n_run = (u32)(c.left < count - done ? c.left : count - done);
+        i32 a0[1], a1[1];
+        u32 alive, wide;
+        run_values<1>(c, g, hole, seg.nt, seg.esize, 0u, n_run, a0, a1, alive, wide);
+        if (alive && (abs_u32(a0[0]) >= lim || abs_u32(a1[0]) >= lim)) { alive = 0u; wide = 1u; }
+        const u64 e = first + done + lane;
+        // (wide operands meet all leaves at once, in the first part)
+        if (part == 0 && __any_sync(0xffffffffu, wide != 0u)) join_exact32(w, plan, seg, sk, hole, e, wide != 0u, from, n);
+        const u32 off = (u32)(e - w.base), n_alive = (u32)__popc(__ballot_sync(0xffffffffu, alive != 0u));
+        if (n_alive != 0u && !hole->join_none)
+            for (int gi = 0; gi < seg.n_groups; ++gi) {
+                const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
+                const u32 want = grp.fmask | (grp.smask << 16);
+                const bool divide = (want & (0x10001u << kSlotDiv | 0x10001u << kSlotMod)) != 0u;
+                const int nl = (int)g->cnt[grp.leaf_nt][1], lb = g->leaf_begin[grp.leaf_nt];
+                const int l0 = (int)((i64)nl * part / seg.parts), l1 = (int)((i64)nl * (part + 1) / seg.parts);
+                n.tests += (u64)((l1 - l0) * __popc(want)) * n_alive;
+                for (int at = l0; at < l1; at += 32) {
+                    i32 c0 = 0, c1 = 0;
+                    if (at + lane < l1) {
+                        const LeafDev lf = g->leaves[lb + at + lane];
+                        c0 = (i32)(lf.var >= 0 ? hole->probe_pt[0][lf.var] : lf.value);
+                        c1 = (i32)(lf.var >= 0 ? hole->probe_pt[p1][lf.var] : lf.value);
+                    }
+                    const int m = l1 - at < 32 ? l1 - at : 32;
+#pragma unroll 1
+                    for (int i = 0; i < m; ++i) {
+                        u32 hits = alive ? want : 0u;
+#pragma unroll 1
+                        for (int k = 0; k < 2; ++k) {
+                            hits &= narrow_bits(k ? a1[0] : a0[0], __shfl_sync(0xffffffffu, k ? c1 : c0, i), k ? t1 : t0, divide);
+                            if (!__any_sync(0xffffffffu, hits != 0u)) break;
+                        }
+                        n.suspects += (u32)__reduce_add_sync(0xffffffffu, (u32)__popc(hits));
+#pragma unroll 1
+                        for (u32 b = __reduce_or_sync(0xffffffffu, hits); b; b &= b - 1) {
+                            const int bit = __ffs((int)b) - 1;
+                            join_push(w, plan, seg, sk, hole, (hits >> bit) & 1u, off, (u32)(at + i), gi, bit & 15, bit >> 4, from, n);
+                        }
+                    }
+                }
+            }
+        done += n_run;
+    }
+}
+
 // What waits in the warp's queues when it leaves segment `index`.
 __device__ __noinline__ void join_leave(JoinWarp& w, const PlanDev& plan, int index, JoinCount& n) {
     const JoinSeg& seg = plan.jsegs[index];
@@ -1643,7 +1710,8 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
             lo = nlo;
         }
         const JoinSeg& seg = plan.jsegs[lo];
-        const u64 chunk = seg.chunk, from = (t - seg.first_ticket) * chunk, first = seg.e_begin + from;
+        const u64 chunk = seg.chunk, parts = seg.parts > 0 ? (u64)seg.parts : 1ull, part = (t - seg.first_ticket) % parts;
+        const u64 from = (t - seg.first_ticket) / parts * chunk, first = seg.e_begin + from;
         // (what waits in the queues is numbered in 32 bits, and a warp's tickets ascend)
         if (w.seg >= 0 && (w.seg != lo || (first + chunk - w.base) >> 32)) join_leave(w, plan, w.seg, n);
         if (seg.acc != acc) { join_flush(plan, acc, n); acc = seg.acc; }
@@ -1651,7 +1719,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
         const HoleDev* hole = &sk->holes[seg.hole];
         if (seg.kind == kJoinLeaf && w.seg != lo) {
             const bool fill = hole->aff_ok || seg.exact;
-            if (fill) join_fill(w, plan, seg, sk->g, hole);
+            if (fill && seg.parts == 0) join_fill(w, plan, seg, sk->g, hole);
             if (lane == 0) { w.base = first; if (fill) w.seg = lo; }
             __syncwarp();
         }
@@ -1659,6 +1727,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
         if ((hole->probe_spec_ok & all) == all && from < seg.e_count) {      // (a spec undefined at a probe: nothing can match)
             const u64 count = seg.e_count - from < chunk ? seg.e_count - from : chunk;
             if (seg.kind == kJoinDirect) direct_ticket(w, plan, seg, sk, hole, first, count, n);
+            else if (seg.parts > 0) join_few(w, plan, seg, sk, hole, first, count, (int)part, n);
             else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, first, count, n);
             else join_ticket<P>(w, plan, seg, sk, hole, first, count, n);
         }
