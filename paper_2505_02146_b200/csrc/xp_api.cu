@@ -1093,6 +1093,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         at += share;
     }
     const size_t staged = at;
+    const bool put = n == 1 && staged <= kPutMost;        // (a small sketch alone: straight to its places, without copy and scatter)
     const size_t at_out = al256(staged), at_scratch = at_out + al256(sizeof(LoadOut) * n_jobs);
     const size_t at_classes = at_scratch + al256(prepare_scratch_bytes((int)(n_jobs < kJobs ? n_jobs : kJobs)));
     size_t class_bytes = 0;
@@ -1130,6 +1131,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             std::atomic<size_t> next(0);
             std::atomic<int> bad(0);
             auto send = [&](size_t p) {
+                if (put) return;
                 const cudaError_t e = cudaMemcpyAsync(dev_block + piece_at[p], hold[p]->p, piece_end(p) - piece_at[p], cudaMemcpyHostToDevice, nullptr);
                 if (e != cudaSuccess) bad.store((int)e);
             };
@@ -1155,7 +1157,11 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
                 for (std::thread& th : pool) th.join();
             }
             err = (cudaError_t)bad.load();
-            if (err == cudaSuccess) err = launch_scatter((const LoadCopy*)(dev_block + at_copies), (int)copies.size(), dev_block, nullptr);
+            if (put) {
+                const u32 a = (u32)(at_shares / 16), b = a + (u32)(st[0].head / 16), c = b + (u32)(st[0].grammar_bytes / 16);
+                const PutPlaces to = {{dev_block, st[0].s->arena, (char*)st[0].s->g->d_g}, {a, b, c}};
+                err = launch_put(to, hold[0]->p, nullptr);
+            } else if (err == cudaSuccess) err = launch_scatter((const LoadCopy*)(dev_block + at_copies), (int)copies.size(), dev_block, nullptr);
             if (err == cudaSuccess) { sent = true; settle(); }
         }
         // (the staging blocks may go back once the copies have been made: they are waited for below, with everything else)
@@ -1203,13 +1209,13 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         const LoadJob* d_jobs = (const LoadJob*)(dev_block + at_jobs);
         for (size_t q = 0; q < n; q += kJobs) {
             const int m = (int)(n - q < kJobs ? n - q : kJobs);
-            XP_CUDA_B(launch_stage(d_list + q, m, most_staged, nullptr));
             XP_CUDA_B(launch_coord_bounds(d_list + q, m, most_points, nullptr));
         }
         for (size_t q = 0; q < n_jobs; q += kJobs) {
             const int m = (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs);
             // (what it decides per hole goes straight to page-locked memory: a few bytes, and no copy to queue behind the tables)
             LoadOut* out = (LoadOut*)(back.locked ? back.p : dev_block + at_out);
+            XP_CUDA_B(launch_stage_sample(d_list, q == 0 ? (int)n : 0, most_staged, d_jobs + q, m, dev_block + at_scratch, nullptr));
             XP_CUDA_B(launch_prepare(d_jobs + q, m, dev_block + at_scratch, out + q, nullptr));
         }
         for (size_t q = 0; q < n_jobs; q += kJobs)

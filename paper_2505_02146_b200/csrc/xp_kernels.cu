@@ -1,8 +1,8 @@
 // Device kernels of libxpiler_repair (sm_100a).
 //
-//   prep_sample_kernel, prepare_kernel -- per sketch, once at load: coordinates and spec values of the
+//   stage_sample_kernel, prepare_kernel -- per sketch, once at load: coordinates and spec values of the
 //                      sample points, choice and order of each hole's probe points.
-//   subvalue_kernel, stage_kernel, coord_bounds_kernel -- per sketch,
+//   subvalue_kernel, stage_sample_kernel, coord_bounds_kernel -- per sketch,
 //                      once at load: values (and variable sets) of all small subtrees at the probes;
 //                      points and spec values of a box; coordinate bounds of a table.
 //   join_kernel     -- (xp_join.cuh) the part of the search whose candidates have a leaf at the root.
@@ -22,6 +22,7 @@
 
 #include <atomic>
 #include <climits>
+#include <cstring>
 #include <mutex>
 
 #include "xp_device.cuh"
@@ -278,29 +279,42 @@ __device__ __forceinline__ void probe_contexts(const GrammarDev* g, HoleDev* hol
 }
 
 // Choice of each hole's probe points, once per sketch.  A sample of small candidates (sizes 1, 3, 5, ranks spread evenly)
-// is run on every sample point (prep_sample_kernel: a bit per sample and candidate); the probes are then picked greedily
+// is run on every sample point (sample_part: a bit per sample and candidate); the probes are then picked greedily
 // (prepare_kernel): each next probe is the sample that the fewest of the sampled candidates still alive (satisfying
 // all probes picked so far) also satisfy.  Ties: the second probe should differ from the first in spec value and
 // coordinates (the leaf join's conditions compare the two, and an operand that does not tell them apart passes), then
 // the larger |spec| + sum |coordinate| (large, distinct operand values make coincidences rare).
 // Only the amount of work downstream depends on this choice, never a result.
 //
-// The sampling is spread over 64 CTAs of 4 warps per hole (lane = candidate, warp = 2 samples): as one CTA per hole it
-// was bound by the instruction rate of a single SM (130 to 290 us of a load).  The context is brought to an affine map
+// The sampling is spread over 64 CTAs of 8 warps per hole (lane = candidate, warp = sample): as one CTA per hole it
+// was bound by the instruction rate of a single SM (130 to 290 us of a load).  A batch has CTAs enough with 8 per hole, and unranks each
+// candidate 8 times instead of 64 (1024 holes: 531 -> 464 us).  The context is brought to an affine map
 // or an interval once per sample instead of being interpreted for every candidate.
 constexpr int kPrepCands = 256;
 constexpr int kPrepWords = kPrepCands / 32;
-constexpr int kPrepWarps = 4, kPrepEach = 2;            // warps per CTA, samples per warp
-constexpr int kPrepSplit = kProbeSamples / (kPrepWarps * kPrepEach);
+constexpr int kPrepWarps = 8;                           // warps per CTA
+constexpr int kPrepMany = 8;                            // jobs of a load from which a warp takes eight samples instead of one
 
-// A sample point's coordinates and spec value, and what it scores in a tie (one thread per sample).
+// A sample point's coordinates and spec value, and what it scores in a tie (one thread per sample).  STAGED: the points of boxes and the values of
+// spec expressions are in their tables (otherwise they may be on their way there, and are derived).
+template <bool STAGED>
 __device__ __forceinline__ void prep_point(const SketchDev* s, const HoleDev* hole, int t, i64* pt, i64& spec, bool& ok, u64& score) {
     u64 mag = 0;
-    point_coords(s, s->sample_id[t], pt);
+    if (STAGED || s->domain_kind == XP_DOMAIN_TABLE) point_coords(s, s->sample_id[t], pt);
+    else {
+        u64 rem = (u64)s->sample_id[t];
+#pragma unroll 1
+        for (int d = s->n_vars - 1; d >= 0; --d) {
+            u64 q, r;
+            divmod_u64(rem, (u64)s->ext[d], q, r);
+            pt[d] = s->lo[d] + (i64)r;
+            rem = q;
+        }
+    }
     for (int d = 0; d < s->n_vars; ++d) mag += (u64)(pt[d] < 0 ? -pt[d] : pt[d]);
     spec = 0;
     ok = true;
-    if (hole->spec_table != nullptr) spec = hole->spec_table[s->sample_id[t]];
+    if (hole->spec_table != nullptr && (STAGED || hole->spec_len == 0)) spec = hole->spec_table[s->sample_id[t]];
     else ok = eval_code(hole->spec, hole->spec_len, pt, 0, spec);
     const u64 m = (u64)(spec < 0 ? -spec : spec);
     score = ok ? (m > (1ull << 62) ? (1ull << 62) : m) + mag : 0;
@@ -314,24 +328,23 @@ __device__ __forceinline__ int prep_sizes(const GrammarDev* g, const HoleDev* ho
     return n;
 }
 
-__global__ void __launch_bounds__(32 * kPrepWarps) prep_sample_kernel(const LoadJob* jobs, u32* masks) {
-    chain_wait();
-    constexpr int kHere = kPrepWarps * kPrepEach;        // samples of this CTA
-    const SketchDev* s = jobs[blockIdx.z].s;
-    const HoleDev* hole = &s->holes[jobs[blockIdx.z].hole];
+// 32 candidates (word) of a hole on the samples of one CTA, `each` per warp from `first` on.
+__device__ __forceinline__ void sample_part(const LoadJob& job, u32* out, int word, int first, int each) {
+    const SketchDev* s = job.s;
+    const HoleDev* hole = &s->holes[job.hole];
     const GrammarDev* g = s->g;
-    __shared__ i64 s_pt[kHere][kMaxVars], s_spec[kHere], s_lo[kHere], s_hi[kHere];
-    __shared__ u64 s_A[kHere], s_B[kHere];
-    __shared__ int s_form[kHere];                        // 0: no constraint can hold; 1: affine; 2: interval; 3: interpret
-    const int t = threadIdx.x, lane = t & 31, word = blockIdx.x, first = blockIdx.y * kHere;
+    __shared__ i64 s_pt[kProbeSamples][kMaxVars], s_spec[kProbeSamples], s_lo[kProbeSamples], s_hi[kProbeSamples];
+    __shared__ u64 s_A[kProbeSamples], s_B[kProbeSamples];
+    __shared__ int s_form[kProbeSamples];                // 0: no constraint can hold; 1: affine; 2: interval; 3: interpret
+    const int t = threadIdx.x, lane = t & 31;
     const int ns = s->n_samples;
-    if (t < kHere) {
+    if (t < kPrepWarps * each) {
         int form = 0;
         if (first + t < ns) {
             i64 pt[kMaxVars], v;
             bool ok;
             u64 score;
-            prep_point(s, hole, first + t, pt, v, ok, score);
+            prep_point<false>(s, hole, first + t, pt, v, ok, score);
             for (int d = 0; d < s->n_vars; ++d) s_pt[t][d] = pt[d];
             s_spec[t] = v;
             u64 A = 0, B = 0;
@@ -354,9 +367,9 @@ __global__ void __launch_bounds__(32 * kPrepWarps) prep_sample_kernel(const Load
             n = unrank(g, hole->start_nt, size, cnt >= per ? slot * (cnt / per) : slot, code);
     }
     __syncthreads();
-    u32* out = masks + (u64)blockIdx.z * kProbeSamples * kPrepWords;
-    for (int k = 0; k < kPrepEach; ++k) {
-        const int j = (t >> 5) * kPrepEach + k;
+#pragma unroll 1
+    for (int k = 0; k < each; ++k) {
+        const int j = (t >> 5) * each + k;
         if (first + j >= ns) break;
         const int form = s_form[j];
         i64 v = 0;
@@ -387,7 +400,7 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
         i64 pt[kMaxVars], v;
         bool ok;
         u64 score;
-        prep_point(s, hole, t, pt, v, ok, score);
+        prep_point<true>(s, hole, t, pt, v, ok, score);
         for (int d = 0; d < nv; ++d) s_pt[t][d] = pt[d];
         s_spec[t] = v; s_ok[t] = ok; s_score[t] = score;
         const u32* m = masks + ((u64)blockIdx.x * kProbeSamples + t) * kPrepWords;
@@ -1252,6 +1265,19 @@ __global__ void __launch_bounds__(256) scatter_kernel(const LoadCopy* copies, co
     for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < c.bytes / 16; i += (u64)gridDim.x * blockDim.x) to[i] = from[i];
 }
 
+// Up to kPutMost bytes from the host to up to three places, as the kernel's own parameters: they come with the launch, where a copy of a
+// few kilobytes from page-locked memory is handed from the compute queue to the copy engine and back (load and search of a two-variable nest: 168 -> 163 us; the head of a search's
+// plan gained nothing this way).
+template <int N> struct PutBlob { uint4 v[N]; };
+template <int N>
+__global__ void __launch_bounds__(32) put_kernel(const PutPlaces to, const __grid_constant__ PutBlob<N> blob) {
+    chain_wait();
+    const u32 i = blockIdx.x * 32u + threadIdx.x;
+    if (i >= to.end[2]) return;
+    const int k = i < to.end[0] ? 0 : i < to.end[1] ? 1 : 2;
+    reinterpret_cast<uint4*>(to.dst[k])[k ? i - to.end[k - 1] : i] = blob.v[i];
+}
+
 // Value of a spec expression at the kStageEach points of a thread; false where it is undefined.  The instructions are
 // decoded once for all of them, the top of the stack stays in registers, and a leaf goes straight into the operator that
 // follows it: the stack proper (local memory, whose stores all go through to L2) is touched where a subtree waits for another.
@@ -1313,12 +1339,10 @@ __device__ __forceinline__ bool eval_code_at(const xp_instr* __restrict__ code, 
 // Bound by the interpreter, and by launches where domains are small, hence one kernel for both (three holes of 1.8 million
 // points: 120 us as two kernels with local stacks, now 61; 80 MB are written, which takes 12).
 static_assert(kStageMaxPoints <= 1ull << 31, "point numbers and extents of a staged box are 32-bit");
-__global__ void __launch_bounds__(256) stage_kernel(SketchDev* const* list) {
-    chain_wait();
+__device__ __forceinline__ void stage_part(const SketchDev* sk, u32 block, u32 blocks) {
     __shared__ xp_instr s_code[kMaxCode];
     __shared__ u32 s_ext[kMaxVars], s_inv[kMaxVars];
     __shared__ StagePoints pts;
-    const SketchDev* sk = list[blockIdx.y];
     const i64 n = sk->n_points;
     const int nv = sk->n_vars, nh = sk->n_holes;
     const bool rows = sk->project;
@@ -1332,8 +1356,8 @@ __global__ void __launch_bounds__(256) stage_kernel(SketchDev* const* list) {
         pts.lo[threadIdx.x] = box ? sk->lo[threadIdx.x] : 0;
     }
     __syncthreads();
-    const i64 step = (i64)gridDim.x * 256 * kStageEach;
-    for (i64 first = (i64)blockIdx.x * 256 * kStageEach; first < n; first += step) {
+    const i64 step = (i64)blocks * 256 * kStageEach;
+    for (i64 first = (i64)block * 256 * kStageEach; first < n; first += step) {
         const i64 at = first + threadIdx.x;               // (the loop is uniform in a block: threads past the end take its first point)
         int n_pt = 0;
 #pragma unroll
@@ -1370,6 +1394,18 @@ __global__ void __launch_bounds__(256) stage_kernel(SketchDev* const* list) {
             for (int k = 0; k < kStageEach; ++k) if (k < n_pt) spec[at + 256 * k] = v[k];
         }
     }
+}
+
+// Staging and sampling of a load in one launch: neither needs the other.  Blocks [0, staged * n_sketches) stage, the others sample, 8 words of
+// candidates by 8 / each blocks of samples per job.  (One launch after the other: two-variable nest 163 us a
+// call, now 160; three conv holes 59 + 28 us, now 68.)
+__global__ void __launch_bounds__(256) stage_sample_kernel(SketchDev* const* list, u32 staged, u32 n_sketches, const LoadJob* jobs, u32* masks, int each) {
+    chain_wait();
+    static_assert(kPrepWarps * 32 == 256 && kProbeSamples / kPrepWarps == 8, "a CTA of either kind");
+    const u32 first = staged * n_sketches;
+    if (blockIdx.x < first) { stage_part(list[blockIdx.x / staged], blockIdx.x % staged, staged); return; }
+    const u32 b = blockIdx.x - first, per = (u32)(kPrepWords * (8 / each)), job = b / per, r = b % per;
+    sample_part(jobs[job], masks + (u64)job * kProbeSamples * kPrepWords, (int)(r % kPrepWords), (int)(r / kPrepWords) * kPrepWarps * each, each);
 }
 
 // Smallest and largest coordinate of every variable over the rows of a table domain, into the
@@ -3126,12 +3162,21 @@ __global__ void __launch_bounds__(256) int_div_reciprocal_kernel(u32* out, int i
 
 size_t prepare_scratch_bytes(int n_jobs) { return sizeof(u32) * (size_t)kProbeSamples * kPrepWords * (size_t)n_jobs; }
 
-cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadOut* out, cudaStream_t stream) {
+cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, const void* scratch, LoadOut* out, cudaStream_t stream) {
     if (n_jobs <= 0) return cudaSuccess;
-    chain(prep_sample_kernel, dim3(kPrepWords, kPrepSplit, (unsigned)n_jobs), 32 * kPrepWarps, 0, stream, jobs, (u32*)scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     chain(prepare_kernel, n_jobs, kPrepThreads, 0, stream, jobs, (const u32*)scratch, out);
+    return cudaGetLastError();
+}
+
+// Staging of n_sketches (0: none, or they have been staged) and sampling of n_jobs.
+cudaError_t launch_stage_sample(SketchDev* const* list, int n_sketches, i64 most_points, const LoadJob* jobs, int n_jobs, void* scratch, cudaStream_t stream) {
+    u64 staged = most_points > 0 && n_sketches > 0 ? (u64)((most_points + 256 * kStageEach - 1) / (256 * kStageEach)) : 0ull;
+    if (staged > 65536) staged = 65536;
+    while (staged * (u64)n_sketches > (1ull << 29)) staged = (staged + 1) / 2;      // (the blocks stride)
+    const int each = n_jobs >= kPrepMany ? 8 : 1;
+    const u64 blocks = staged * (u64)n_sketches + (u64)n_jobs * (u64)(kPrepWords * (8 / each));
+    if (blocks == 0) return cudaSuccess;
+    chain(stage_sample_kernel, (unsigned)blocks, 256, 0, stream, list, (u32)staged, staged ? (u32)n_sketches : 0u, jobs, (u32*)scratch, each);
     return cudaGetLastError();
 }
 
@@ -3156,10 +3201,16 @@ cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src
     return cudaGetLastError();
 }
 
-cudaError_t launch_stage(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream) {
-    if (most_points <= 0 || n_sketches <= 0) return cudaSuccess;
-    const i64 blocks = (most_points + 256 * kStageEach - 1) / (256 * kStageEach);
-    chain(stage_kernel, dim3((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)n_sketches), 256, 0, stream, list);
+template <int N>
+static void put_as(const PutPlaces& to, const char* src, cudaStream_t stream) {
+    PutBlob<N> blob;
+    memcpy(&blob, src, 16 * (size_t)to.end[2]);
+    chain(put_kernel<N>, (to.end[2] + 31u) / 32u, 32, 0, stream, to, blob);
+}
+cudaError_t launch_put(const PutPlaces& to, const char* src, cudaStream_t stream) {
+    if (to.end[2] == 0) return cudaSuccess;
+    if (to.end[2] <= 768u) put_as<768>(to, src, stream);
+    else put_as<(int)(kPutMost / 16)>(to, src, stream);
     return cudaGetLastError();
 }
 

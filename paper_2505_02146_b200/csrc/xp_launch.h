@@ -32,11 +32,14 @@ __device__ __forceinline__ void chain_wait() {
 #endif
 
 size_t prepare_scratch_bytes(int n_jobs);
-cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, void* scratch, LoadOut* out, cudaStream_t stream);
+cudaError_t launch_prepare(const LoadJob* jobs, int n_jobs, const void* scratch, LoadOut* out, cudaStream_t stream);
+cudaError_t launch_stage_sample(SketchDev* const* list, int n_sketches, i64 most_points, const LoadJob* jobs, int n_jobs, void* scratch, cudaStream_t stream);
 cudaError_t launch_scatter(const LoadCopy* copies, int n_copies, const char* src, cudaStream_t stream);
+constexpr size_t kPutMost = 31744;                   // (a launch takes 32 764 bytes of parameters)
+struct PutPlaces { char* dst[3]; u32 end[3]; };      // 16-byte words [end[k - 1], end[k]) go to dst[k]
+cudaError_t launch_put(const PutPlaces& to, const char* src, cudaStream_t stream);
 cudaError_t launch_reprobe(const LoadJob* jobs, int n_jobs, cudaStream_t stream);
 cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
-cudaError_t launch_stage(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last, int most_probes, u64 most_entries, cudaStream_t stream);
 // Operand classes of one hole (csrc/xp_classes.cuh); scratch: class_scratch_bytes(entries), 256-byte aligned.
 inline u32 class_slots(u64 entries) { u32 n = 1024; while (n < 2 * entries) n <<= 1; return n; }
