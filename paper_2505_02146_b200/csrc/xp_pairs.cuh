@@ -108,7 +108,7 @@ __device__ __noinline__ void pair_check(PairWarp& w, const PlanDev& plan, const 
                     const u64 b = (u64)j * hole->tab_total;
                     i64 v;
                     pass = hole->tab_ok[b + le] && hole->tab_ok[b + re] &&
-                           apply_op(op_of_slot(slot), hole->tab_val[b + le], hole->tab_val[b + re], v) && probe_accepts(hole, j, v);
+                           op_value(op_of_slot(slot), hole->tab_val[b + le], hole->tab_val[b + re], v) && probe_accepts(hole, j, v);
                 }
             }
         }
