@@ -271,8 +271,7 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
     u32 m = __ballot_sync(0xffffffffu, pass);
     if (!m) return;
     n.passes += (u32)__popc(m);
-    const bool pending = pass && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
-    m = __ballot_sync(0xffffffffu, pending);
+    m = __ballot_sync(0xffffffffu, push_survivors(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, pass, rank, vars));
     while (m) {
         const int src = __ffs((int)m) - 1;
         m &= m - 1;
@@ -280,11 +279,33 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
     }
 }
 
-// Probes without tables: the candidate is rebuilt in full.
-__device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev* hole, int size, u64 rank, u64& evals) {
+// The candidates of the lanes with `pass` at the probes without tables (from n_exact on), rebuilt in full: a few one after the other with the
+// probes over the lanes, many with a lane each.  (A lane by itself evaluated eight probes one after the other, and those without need
+// once more: 50 us at the end of a search over 800 000 operands of five nodes, now %FULL%.)  Called by all lanes.
+__device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev* hole, int size, bool pass, u64 rank, u64& evals) {
+    const int lane = threadIdx.x & 31, n_exact = hole->n_exact, n_probe = hole->n_probe;
+    u32 m = __ballot_sync(0xffffffffu, pass);
+    if (!m || n_exact >= n_probe) return pass;
     u32 code[kMaxSize];
-    const int n = unrank(g, hole->start_nt, size, rank, code);
-    return probe_check(g, hole, code, n, evals);
+    if (__popc(m) > 4) {
+        if (!pass) return false;
+        const int n = unrank(g, hole->start_nt, size, rank, code);
+        return probe_check(g, hole, code, n, evals, n_exact);
+    }
+    u32 good = 0;
+    for (; m; m &= m - 1) {
+        const int src = __ffs((int)m) - 1, j = n_exact + lane;
+        const int n = unrank(g, hole->start_nt, size, __shfl_sync(0xffffffffu, rank, src), code);
+        bool ok = true;
+        if (j < n_probe) {
+            i64 h = 0;
+            ++evals;
+            ok = ((hole->probe_spec_ok >> j) & 1u) && eval_cand(code, n, g->leaves, hole->probe_pt[j], h) &&
+                 ctx_matches(hole, hole->probe_pt[j], h, hole->probe_spec[j]);
+        }
+        if (__all_sync(0xffffffffu, ok)) good |= 1u << src;
+    }
+    return (good >> lane) & 1u;
 }
 
 // Candidates of a segment that counts by class, one per lane (pass: this lane has one, and it satisfies the probes with tables):
@@ -304,70 +325,92 @@ __device__ __noinline__ void join_members(JoinWarp& w, const PlanDev& plan, cons
         const u64 before = __shfl_sync(0xffffffffu, incl, src ? src - 1 : 0), e2 = __shfl_sync(0xffffffffu, e, src);
         const u32 pos2 = __shfl_sync(0xffffffffu, pos, src), code2 = __shfl_sync(0xffffffffu, code, src);
         bool ok = false;
-        u64 rank = 0;
+        u64 rank = 0, member = 0;
         u32 vars = 0;
+        const int swap = (int)(code2 & 1u), slot = (int)((code2 >> 1) & 15u);
+        const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code2 >> 8)];
         if (k0 + (u64)lane < total) {
-            const int swap = (int)(code2 & 1u), slot = (int)((code2 >> 1) & 15u);
-            const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code2 >> 8)];
-            const u64 member = class_operand(g, hole, seg.nt, seg.esize, e2).rank(src ? k - before : k);
             const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
+            member = class_operand(g, hole, seg.nt, seg.esize, e2).rank(src ? k - before : k);
             rank = grp.base[swap][slot] + (swap ? (u64)pos2 * ne + member : member * nl + (u64)pos2);
             ok = rank >= seg.rank_begin && rank < seg.rank_end &&
                  XP_CHECKED(member < ne && (u64)pos2 < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
-            if (ok && hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, rank, n.evals);
-            if (ok) {
-                const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos2];
-                vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, member)) | (lf.var >= 0 ? 1u << lf.var : 0u);
-            }
+        }
+        ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
+        if (ok) {
+            const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos2];
+            vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, member)) | (lf.var >= 0 ? 1u << lf.var : 0u);
         }
         join_survive(w, plan, sk, hole, seg, ok, rank, vars, n);
     }
 }
 
-// The candidates in the warp's second queue, one per lane: the probes from `from` on, exactly.  Called by all lanes.
+// The candidates in the warp's second queue: the probes from `from` on, exactly.  Up to four, what a warp leaves a segment or a small call with,
+// have their probes side by side in 16 lanes each; more take a lane each and, in a call of one wave, which waits for this chain, and for
+// contexts that compare, four probes a step (exact_pair4).  A member's values are its class's: one check serves for all of them.  Called by all lanes.
 __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, int from, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
     __syncwarp();
     const u32 nc = w.nc;
-    // (a call of one wave waits for this chain, and a candidate of a context that compares passes most probes: see exact_pair4)
-    const bool four = !hole->aff_ok || plan.n_join <= (u64)gridDim.x * kJoinWarps;
+    const int n_exact = hole->n_exact;
+    const bool classes = seg.classes != 0, four = !hole->aff_ok || plan.n_join <= (u64)gridDim.x * kJoinWarps;
     for (u32 at = 0; at < nc; at += 32) {
+        const bool spread = nc - at <= 4u;
+        u32 good = 0;                                     // spread: bit i: candidate i passes
         bool pass = false;
-        u64 rank = 0;
-        u32 vars = 0;
-        if (seg.classes) {                                // a member's values are its class's: one check for all of them
-            u64 e = 0;
-            u32 code = 0, pos = 0;
-            if (at + lane < nc) {
+        u64 rank = 0, e = 0;
+        u32 vars = 0, code = 0, pos = 0;
+#pragma unroll 1
+        for (u32 i0 = 0; i0 < (spread ? nc - at : 1u); i0 += 2u) {
+            const u32 i = spread ? i0 + (u32)(lane >> 4) : (u32)lane;
+            bool ok = at + i < nc;
+            if (ok) {
+                code = w.c_code[at + i]; pos = w.c_pos[at + i]; e = w.base + w.c_off[at + i];
+                const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u), op = op_of_slot(slot);
+                const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code >> 8)];
+                const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
+                const u64 first = classes ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e;
+                rank = grp.base[swap][slot] + (swap ? (u64)pos * ne + first : first * nl + (u64)pos);
+                ok = (classes || (rank >= seg.rank_begin && rank < seg.rank_end)) &&
+                     XP_CHECKED(first < ne && (u64)pos < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
+                if (ok) {
+                    const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, first);
+                    const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
+                    if (spread) {
+                        const int j = from + (lane & 15);
+                        if (j < n_exact) {
+                            i64 a = 0, v = 0;
+                            ++n.evals;
+                            ok = ref_value(g, hole, ref, seg.nt, seg.esize, j, a);
+                            const i64 c = lf.var >= 0 ? hole->probe_pt[j][lf.var] : lf.value;
+                            ok = ok && op_value(op, swap ? c : a, swap ? a : c, v) && probe_accepts(hole, j, v);
+                        }
+                    } else ok = four ? exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op, from, n_exact, n.evals)
+                                     : exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op, from, n_exact, n.evals);
+                    if (ok && !spread) vars = ref_vars(hole, ref) | (lf.var >= 0 ? 1u << lf.var : 0u);
+                }
+            }
+            if (spread) {
+                const u32 b = __ballot_sync(0xffffffffu, ok);
+                good |= (u32)((b & 0xffffu) == 0xffffu) << i0 | (u32)(b >> 16 == 0xffffu) << (i0 + 1u);
+            } else pass = ok;
+        }
+        if (spread) {                                     // candidate i to lane i
+            pass = lane < 4 && ((good >> lane) & 1u);
+            if (at + (u32)lane < nc && lane < 4) {
                 code = w.c_code[at + lane]; pos = w.c_pos[at + lane]; e = w.base + w.c_off[at + lane];
-                const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, class_operand(g, hole, seg.nt, seg.esize, e).rank(0));
-                const LeafDev lf = g->leaves[g->leaf_begin[plan.jgroups[seg.first_group + (int)(code >> 8)].leaf_nt] + (int)pos];
-                const bool swap = (code & 1u) != 0u;
-                const int op = op_of_slot((int)((code >> 1) & 15u));
-                pass = !four ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals)
-                                    : exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap, op, from, hole->n_exact, n.evals);
-            }
-            join_members(w, plan, seg, sk, hole, pass, e, pos, code, n);
-            continue;
-        }
-        if (at + lane < nc) {
-            const u32 code = w.c_code[at + lane], pos = w.c_pos[at + lane];
-            const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u);
-            const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code >> 8)];
-            const u64 e = w.base + w.c_off[at + lane];
-            const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
-            rank = grp.base[swap][slot] + (swap ? (u64)pos * ne + e : e * nl + (u64)pos);
-            if (rank >= seg.rank_begin && rank < seg.rank_end &&
-                XP_CHECKED(e < ne && (u64)pos < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue)) {
-                const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, e);
-                const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
-                pass = !four ? exact_pair(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals)
-                                    : exact_pair4(g, hole, ref, seg.nt, seg.esize, lf.var, lf.value, swap != 0, op_of_slot(slot), from, hole->n_exact, n.evals);
-                if (pass && hole->n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
-                vars = ref_vars(hole, ref) | (lf.var >= 0 ? 1u << lf.var : 0u);
+                if (pass && !classes) {
+                    const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u);
+                    const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code >> 8)];
+                    rank = grp.base[swap][slot] + (swap ? (u64)pos * g->cnt[seg.nt][seg.esize] + e : e * g->cnt[grp.leaf_nt][1] + (u64)pos);
+                    const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
+                    vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, e)) | (lf.var >= 0 ? 1u << lf.var : 0u);
+                }
             }
         }
+        if (classes) { join_members(w, plan, seg, sk, hole, pass, e, pos, code, n); continue; }
+        pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
         join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
     }
     __syncwarp();
@@ -1689,9 +1732,9 @@ __device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, con
                 i64 v[kProbeStep];
                 pass = ref_value4(g, hole, ref, seg.nt, seg.esize, j0, n_exact, v) == (1u << here) - 1u && probes_accept(hole, j0, n_exact, v);
             }
-            if (pass && n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, rank, n.evals);
             vars = ref_vars(hole, ref);
         }
+        pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
         const u32 b = __ballot_sync(0xffffffffu, pass);
         n.suspects += (u32)__popc(b);
         join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);

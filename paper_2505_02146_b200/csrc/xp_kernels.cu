@@ -664,9 +664,9 @@ __device__ __noinline__ void flush_acc(EvalShared& sh, const PlanDev& plan, u64&
 
 // Stage 2: exact check of one candidate on the hole's probe points, first failure ends it.
 __device__ __noinline__ bool probe_check(const GrammarDev* g, const HoleDev* hole, const u32* code, int n,
-                                            u64& my_evals) {
+                                            u64& my_evals, int from = 0) {
     const int np = hole->n_probe;
-    for (int j = 0; j < np; ++j) {
+    for (int j = from; j < np; ++j) {
         ++my_evals;
         if (!((hole->probe_spec_ok >> j) & 1)) return false;
         i64 h;
@@ -1064,6 +1064,41 @@ __device__ __forceinline__ bool push_survivor(const PlanDev& plan, const SketchD
     if (plan.surv_hist) atomicAdd(&plan.surv_hist[r.acc], 1u);       // (for the hole order the verification walks)
     if (plan.max_chunks > 1 && proj_points(sk, hole, vars, nullptr) > (i64)kVerifyChunk) plan.surv_long[atomicAdd(plan.surv_long_n, 1u)] = at;
     return true;
+}
+
+// The same for a warp: the candidates of the lanes with `pass`, all of one accumulator; returns whether this lane's has to be checked by the
+// warp.  One atomic per warp and counter: lane by lane the same three words took an update per survivor from every warp of the call, which
+// was most of a check (32 survivors of a guard: 25 -> %PUSH% us).  Called by all lanes.
+__device__ __forceinline__ bool push_survivors(const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, int sketch, int hole_index, int size,
+                                               int acc, bool pass, u64 rank, u32 vars) {
+    const u32 m = __ballot_sync(0xffffffffu, pass);
+    if (!m) return false;
+    const int lane = threadIdx.x & 31, leader = __ffs((int)m) - 1;
+    const u32 below = (1u << lane) - 1u;
+    u32 first = 0xffffffffu;                              // (saturates, as above)
+    if (lane == leader && *(volatile const u32*)plan.surv_n < plan.surv_cap) first = atomicAdd(plan.surv_n, (u32)__popc(m));
+    first = __shfl_sync(0xffffffffu, first, leader);
+    const u32 at = first + (u32)__popc(m & below);
+    const bool in = pass && first < plan.surv_cap && at < plan.surv_cap;
+    if (in) {
+        SurvDev r;
+        r.rank = rank; r.sketch = sketch; r.hole = hole_index; r.size = size; r.acc = acc;
+        r.state = 0; r.vars = vars;
+        plan.surv[at] = r;
+    }
+    const u32 mi = __ballot_sync(0xffffffffu, in);
+    if (plan.surv_hist && lane == leader && mi) atomicAdd(&plan.surv_hist[acc], (u32)__popc(mi));       // (for the hole order the verification walks)
+    if (plan.max_chunks > 1) {
+        const bool is_long = in && proj_points(sk, hole, vars, nullptr) > (i64)kVerifyChunk;
+        const u32 ml = __ballot_sync(0xffffffffu, is_long);
+        if (ml) {
+            u32 to = 0;
+            if (lane == leader) to = atomicAdd(plan.surv_long_n, (u32)__popc(ml));
+            to = __shfl_sync(0xffffffffu, to, leader);
+            if (is_long) plan.surv_long[to + (u32)__popc(ml & below)] = at;
+        }
+    }
+    return pass && !in;
 }
 
 // The warp checks one candidate on the whole domain itself and records a match in the CTA's

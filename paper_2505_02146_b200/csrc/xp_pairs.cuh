@@ -70,14 +70,13 @@ __device__ __noinline__ void pair_members(PairWarp& w, const PlanDev& plan, cons
             const u32 lr = L.member(l2, (u32)kl), rr = R.member(r2, (u32)kr);
             rank = seg.base[slot2] + (u64)lr * seg.right_count + rr;
             ok = rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(rr < seg.right_count && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
-            if (ok && hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, rank, n.evals);
             if (ok) vars = (u32)hole->tab_vars[L.off + lr] | (u32)hole->tab_vars[R.off + rr];
         }
+        ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
         u32 m = __ballot_sync(0xffffffffu, ok);
         if (!m) continue;
         n.passes += (u32)__popc(m);
-        const bool pending = ok && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
-        m = __ballot_sync(0xffffffffu, pending);
+        m = __ballot_sync(0xffffffffu, push_survivors(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, ok, rank, vars));
         while (m) {
             const int at = __ffs((int)m) - 1;
             m &= m - 1;
