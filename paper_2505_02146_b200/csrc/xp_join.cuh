@@ -281,7 +281,7 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
 
 // The candidates of the lanes with `pass` at the probes without tables (from n_exact on), rebuilt in full: a few one after the other with the
 // probes over the lanes, many with a lane each.  (A lane by itself evaluated eight probes one after the other, and those without need
-// once more: 50 us at the end of a search over 800 000 operands of five nodes, now %FULL%.)  Called by all lanes.
+// once more: 50 us at the end of a search over 800 000 operands of five nodes: whole call 384 -> 349 us.)  Called by all lanes.
 __device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev* hole, int size, bool pass, u64 rank, u64& evals) {
     const int lane = threadIdx.x & 31, n_exact = hole->n_exact, n_probe = hole->n_probe;
     u32 m = __ballot_sync(0xffffffffu, pass);
