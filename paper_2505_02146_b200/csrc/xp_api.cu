@@ -1426,7 +1426,8 @@ constexpr size_t kPairFew = 2;               // sketches up to which kPairLeast 
 // A rank window cuts a block to some of its left operands, but the other side is indexed whole: a block with fewer rows than this,
 // or thereabouts, is done as tiles before the index is made (450 000 operands a side, remainders: 2 222 rows 0.26 ms, the index 1.9).
 constexpr u64 kPairEach = 1ull << 12;
-constexpr u32 kRangeChunk = 8;               // operands of a ticket there: a warp checks its suspects by itself, some hundred of them from 32 operands
+constexpr i32 kRangeParts = 4;               // parts of the constants there: a warp checks its suspects by itself, some hundred of them from 32 operands and all
+                                             // constants (three conv holes: join 440 us in one part, 350 with 8 operands a ticket, 330 so)
 constexpr u64 kRangeSplit = 1ull << 15;      // ... up to which an operator is a segment of its own (with more there are warps enough at work)
 constexpr u64 kRangeMost = 1ull << 18;       // operands of a hole whose context compares from which the tiles take a leaf at the root too
 
@@ -1718,7 +1719,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         // An operand of a context that compares takes some hundred microseconds of a lane, and classes leave a few thousand of them: a
         // segment per operator and side, so that as many warps share them (three conv holes: join 540 -> 430 us).
         if (few && compares && !c.seg.exact && c.seg.e_count <= kRangeSplit) {
-            c.seg.chunk = kRangeChunk;
+            c.seg.parts = kRangeParts;
             for (const JoinGroup& q : c.groups)
                 for (int b = 0; b < 2 * kOpSlots; ++b) {
                     const int swap = b / kOpSlots, slot = b % kOpSlots;
@@ -1777,8 +1778,7 @@ static void number_joins(Plan* plan) {
     for (JoinSeg& c : plan->jsegs) {
         if (c.exact) c.exact = form;
         c.first_ticket = plan->n_join;
-        c.chunk = (u32)(c.exact ? (form == kExactFew ? 1 : 32) : c.chunk ? c.chunk : per * 32);      // (set: see add_joins)
-        c.parts = 0;
+        c.chunk = (u32)(c.exact ? (form == kExactFew ? 1 : 32) : c.parts > 0 ? 32 : per * 32);
         if (share && few(c)) {
             const u64 most = ((u64)c.leaves + 3) / 4;
             c.chunk = 32;

@@ -1525,8 +1525,9 @@ __device__ __forceinline__ bool range_accepts(int slot, const i32 (&x)[kRangePro
 
 // Operands [first, first + count) of a segment against the leaves, for a hole whose context compares: the value has to
 // lie in [rng_lo, rng_hi] at every probe.
+// Against part `part` of the constants where a segment has several (the variables and wide operands are in the first).
 __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole,
-                                          u64 first, u64 count, JoinCount& n) {
+                                          u64 first, u64 count, int part, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
     const int np = hole->n_exact, nr = np < kRangeProbes ? np : kRangeProbes;
@@ -1546,7 +1547,8 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         pairs += g->cnt[grp.leaf_nt][1] * (u64)(__popc(grp.fmask) + __popc(grp.smask));
         sets_ok = sets_ok && hole->join_sets[grp.leaf_nt].ok != 0;
     }
-    n.cands += seg_operands(seg, g, first, count) * pairs;
+    const int parts = seg.parts > 1 ? seg.parts : 1;
+    if (part == 0) n.cands += seg_operands(seg, g, first, count) * pairs;
     for (u64 at = 0; at < count; at += 32) {
         const u64 e = first + at + lane;
         const bool have = at + lane < count;
@@ -1581,7 +1583,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
             }
         }
         if (!sets_ok) wide = live;
-        if (__any_sync(0xffffffffu, live && wide)) join_exact32(w, plan, seg, sk, hole, e, live && wide, 0, n);
+        if (part == 0 && __any_sync(0xffffffffu, live && wide)) join_exact32(w, plan, seg, sk, hole, e, live && wide, 0, n);
         live = live && !wide;
         const u32 off = (u32)(e - w.base);
         const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
@@ -1618,10 +1620,12 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         }
         for (int gi = 0; gi < seg.n_groups; ++gi) {
             const JoinGroup& grp = plan.jgroups[seg.first_group + gi];
-            const i32 cb = g->const_begin[grp.leaf_nt], vb = g->var_begin[grp.leaf_nt], ve = g->const_begin[grp.leaf_nt + 1];
+            const i32 c_first = g->const_begin[grp.leaf_nt], vb_all = g->var_begin[grp.leaf_nt];
+            const i32 cb = c_first + (vb_all - c_first) * part / parts, vb = c_first + (vb_all - c_first) * (part + 1) / parts;      // this part's constants
+            const i32 v_first = part == 0 ? vb_all : g->const_begin[grp.leaf_nt + 1], ve = g->const_begin[grp.leaf_nt + 1];
             for (int swap = 0; swap < 2; ++swap) {
                 const u32 mask = swap ? grp.smask : grp.fmask;
-                n.tests += (u64)n_live * (u64)(__popc(mask) * (1 + ve - vb));
+                n.tests += (u64)n_live * (u64)(__popc(mask) * ((part == 0 ? 1 : 0) + ve - v_first));
                 for (u32 m = cb < vb ? mask & ~(1u << kSlotMod) : 0u; m; m &= m - 1) {
                     const int slot = __ffs((int)m) - 1;
                     i32 run[4] = {cb, cb, cb, cb};
@@ -1697,7 +1701,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
                             }
                         }
                 }
-                for (i32 ci = vb; ci < ve; ++ci) {        // variables one by one
+                for (i32 ci = v_first; ci < ve; ++ci) {   // variables one by one
                     const ConstDev c = g->consts[ci];
                     i32 cv[kRangeProbes];
 #pragma unroll
@@ -1788,8 +1792,8 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
         if ((hole->probe_spec_ok & all) == all && from < seg.e_count) {      // (a spec undefined at a probe: nothing can match)
             const u64 count = seg.e_count - from < chunk ? seg.e_count - from : chunk;
             if (seg.kind == kJoinDirect) direct_ticket(w, plan, seg, sk, hole, first, count, n);
+            else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, first, count, (int)part, n);
             else if (seg.parts > 0) join_few(w, plan, seg, sk, hole, first, count, (int)part, n);
-            else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, first, count, n);
             else join_ticket<P>(w, plan, seg, sk, hole, first, count, n);
         }
         u64 next = 0;
