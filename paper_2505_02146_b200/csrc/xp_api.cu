@@ -827,13 +827,22 @@ static xp_status load_begin(const xp_grammar* gc, const xp_sketch_desc* d, LoadS
             o.off_pair = off; off += al256(2 * sizeof(i32) * entries);
         }
         class_plan(g, hd, &s->holes[h]);
-        if (const size_t c = s->holes[h].cls_entries) { o.off_cls = off; off += al256(8 * c) + al256(4 * (c + kMaxNt + 1)) + al256(4 * c); }
         o.off_sets = off; off += al256(sizeof(JoinSet) * (size_t)g->n_nt);
         if (size_cap > s->tab_size_cap) s->tab_size_cap = size_cap;
         if (o.probes > s->tab_probes_cap) s->tab_probes_cap = o.probes;
     }
+    const size_t plain = off;                             // the classes come last: where memory is short the sketch does without
+    for (int h = 0; h < nh; ++h)
+        if (const size_t c = s->holes[h].cls_entries) { L->hole[h].off_cls = off; off += al256(8 * c) + al256(4 * (c + kMaxNt + 1)) + al256(4 * c); }
     size_t arena_granted = 0;
-    if (pool_alloc((void**)&s->arena, off, &s->arena_device, &arena_granted) != cudaSuccess) {
+    cudaError_t got = pool_alloc((void**)&s->arena, off, &s->arena_device, &arena_granted);
+    if (got != cudaSuccess && off > plain) {
+        (void)cudaGetLastError();
+        off = plain;
+        for (int h = 0; h < nh; ++h) { L->hole[h].off_cls = 0; s->holes[h].cls_entries = 0; }
+        got = pool_alloc((void**)&s->arena, off, &s->arena_device, &arena_granted);
+    }
+    if (got != cudaSuccess) {
         (void)cudaGetLastError();
         delete s;
         return fail(XP_ERR_NOMEM, "device memory for the sketch (" + std::to_string(off) + " bytes)");
@@ -1098,8 +1107,15 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     const size_t at_classes = at_scratch + al256(prepare_scratch_bytes((int)(n_jobs < kJobs ? n_jobs : kJobs)));
     size_t class_bytes = 0;
     for (size_t i = 0; i < n; ++i) { const size_t b = classes_scratch(st[i].s); class_bytes = b > class_bytes ? b : class_bytes; }
-    const size_t total = at_classes + class_bytes;
-    XP_CUDA_B(pool_alloc((void**)&dev_block, total, &dev_device, &dev_bytes));
+    size_t total = at_classes + class_bytes;
+    cudaError_t got = pool_alloc((void**)&dev_block, total, &dev_device, &dev_bytes);
+    if (got != cudaSuccess && class_bytes > 0) {          // (memory is short: without classes)
+        (void)cudaGetLastError();
+        class_bytes = 0;
+        total = at_classes;
+        got = pool_alloc((void**)&dev_block, total, &dev_device, &dev_bytes);
+    }
+    XP_CUDA_B(got);
     StageBlock back(sizeof(LoadOut) * n_jobs);
     if (!back.p) { undo(); return fail(XP_ERR_NOMEM, "out of host memory"); }
     {
@@ -1342,9 +1358,16 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         char* jobs_dev = nullptr;
         size_t jobs_bytes = 0;
         int jobs_device = 0;
-        const size_t at_classes = al256(sizeof(LoadJob) * jobs.size()), class_bytes = classes_scratch(s);
-        XP_CUDA(pool_alloc((void**)&jobs_dev, at_classes + class_bytes, &jobs_device, &jobs_bytes));
-        for (HoleDev& o : hh) memset(o.cls_count, 0, sizeof(o.cls_count));      // (holes without a promoted point are numbered again too)
+        const size_t at_classes = al256(sizeof(LoadJob) * jobs.size());
+        size_t class_bytes = classes_scratch(s);
+        cudaError_t got = pool_alloc((void**)&jobs_dev, at_classes + class_bytes, &jobs_device, &jobs_bytes);
+        if (got != cudaSuccess && class_bytes > 0) {      // (memory is short: without classes from here on)
+            (void)cudaGetLastError();
+            class_bytes = 0;
+            got = pool_alloc((void**)&jobs_dev, at_classes, &jobs_device, &jobs_bytes);
+        }
+        XP_CUDA(got);
+        for (HoleDev& o : hh) { memset(o.cls_count, 0, sizeof(o.cls_count)); o.cls_size = 0; }      // (holes without a promoted point are numbered again too)
         cudaError_t e = cudaMemcpyAsync(s->arena + s->off_holes, hh.data(), sizeof(HoleDev) * nh, cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(LoadJob) * jobs.size(), cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = launch_reprobe((const LoadJob*)jobs_dev, (int)jobs.size(), nullptr);
