@@ -1987,6 +1987,10 @@ static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size
     w.n_acc = (int)n_acc; w.n_segs = (int)plan.segs.size(); w.n_jsegs = (int)plan.jsegs.size(); w.n_sketches = (int)n_sketches;
     w.surv_cap = surv_cap;
     w.join_wide = plan.join_wide ? 1 : 0;
+    // (a call whose windows are all so small that candidates are checked one by one has nothing of the longer form to gain either)
+    w.join_batch = 1;
+    for (const JoinSeg& c : plan.jsegs)
+        if (c.classes || c.parts > 0 || (c.kind != kJoinDirect && n_sketches <= kPairMaxSketches)) { w.join_batch = 0; break; }
     i64 most = 0;
     w.dense = w.empty_domain = 0;
     for (size_t i = 0; i < n_sketches; ++i) {

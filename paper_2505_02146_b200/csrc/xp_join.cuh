@@ -23,9 +23,19 @@
 // Operands of JoinSet::lim or more, leaf sets with a wider leaf and shifts take the exact form, in 64 bits: 32 operands at a time, a
 // lane each (they too wait in a queue), or, where a segment has few operands, one at a time, lanes over the leaves.
 // Warps work on their own; nothing here waits for another warp.
-#pragma once
-
+//
+// This file is compiled twice.  XP_JOIN_BATCH: the form for batches without classes or tickets in parts.  Such a call has warps enough at
+// work to hide a check's chain, and waits for instructions instead: everything that only shortens the chain (probes side by side, several a step,
+// operators side by side) or serves classes is left out of it (search of 40 sketches 0.23 ms with it, 0.20 without; of 1024 3.97, 3.76).
 namespace xp {
+#undef XP_CLASSES
+#if XP_JOIN_BATCH
+#define XP_CLASSES(seg) 0
+namespace join_batch {
+#else
+#define XP_CLASSES(seg) (seg).classes
+namespace join_full {
+#endif
 
 constexpr int kJoinThreads = 256;
 constexpr int kJoinWarps = kJoinThreads / 32;
@@ -88,6 +98,9 @@ struct JoinCount { u64 evals; u64 tests, cands; u32 suspects, passes; };
 // turns, each with a 64-bit division of its own: where both values are below 2^31 in magnitude every operator but the shifts is computed
 // and one selected (1024 small snippets, load and search: 16.0 -> 15.0 ms).
 __device__ __forceinline__ bool op_value(int op, i64 x, i64 y, i64& v) {
+#if XP_JOIN_BATCH
+    return apply_op(op, x, y, v);
+#else
     constexpr i64 kEdge = 1ll << 31;
     if (x > -kEdge && x < kEdge && y > -kEdge && y < kEdge && (op <= XP_OP_MOD || op == XP_OP_MIN || op == XP_OP_MAX)) {
         const i32 a = (i32)x, b = (i32)y, d = b ? b : 1, q = a / d, r = a - q * d;      // (no overflow: a is not -2^31)
@@ -97,6 +110,7 @@ __device__ __forceinline__ bool op_value(int op, i64 x, i64 y, i64& v) {
         return b != 0 || (op != XP_OP_DIV && op != XP_OP_MOD);
     }
     return apply_op(op, x, y, v);
+#endif
 }
 
 // An operand subtree by reference: a table entry, an operation on two table entries, or (mode 2) its rank.
@@ -211,7 +225,12 @@ __device__ __forceinline__ bool probes_accept(const HoleDev* hole, int j0, int n
 }
 
 // The candidate (operand, leaf) at the probes that have tables, in order; the first failure ends it.
-__device__ __noinline__ bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
+#if XP_JOIN_BATCH
+__device__ __forceinline__
+#else
+__device__ __noinline__
+#endif
+bool exact_pair(const GrammarDev* g, const HoleDev* hole, const OperandRef& ref, int nt, int esize, i32 var, i64 cval,
                                            bool swap, int op, int from, int n_exact, u64& evals) {
     for (int j = from; j < n_exact; ++j) {
         ++evals;
@@ -271,7 +290,12 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
     u32 m = __ballot_sync(0xffffffffu, pass);
     if (!m) return;
     n.passes += (u32)__popc(m);
+#if XP_JOIN_BATCH
+    const bool pending = pass && !push_survivor(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, rank, vars);
+    m = __ballot_sync(0xffffffffu, pending);
+#else
     m = __ballot_sync(0xffffffffu, push_survivors(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, pass, rank, vars));
+#endif
     while (m) {
         const int src = __ffs((int)m) - 1;
         m &= m - 1;
@@ -284,6 +308,13 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
 // once more: 50 us at the end of a search over 800 000 operands of five nodes: whole call 384 -> 349 us.)  Called by all lanes.
 __device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev* hole, int size, bool pass, u64 rank, u64& evals) {
     const int lane = threadIdx.x & 31, n_exact = hole->n_exact, n_probe = hole->n_probe;
+#if XP_JOIN_BATCH
+    (void)lane; (void)n_exact; (void)n_probe;
+    if (!pass) return false;
+    u32 code[kMaxSize];
+    const int n = unrank(g, hole->start_nt, size, rank, code);
+    return probe_check(g, hole, code, n, evals, n_exact);
+#else
     u32 m = __ballot_sync(0xffffffffu, pass);
     if (!m || n_exact >= n_probe) return pass;
     u32 code[kMaxSize];
@@ -306,6 +337,7 @@ __device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev*
         if (__all_sync(0xffffffffu, ok)) good |= 1u << src;
     }
     return (good >> lane) & 1u;
+#endif
 }
 
 // Candidates of a segment that counts by class, one per lane (pass: this lane has one, and it satisfies the probes with tables):
@@ -336,7 +368,7 @@ __device__ __noinline__ void join_members(JoinWarp& w, const PlanDev& plan, cons
             ok = rank >= seg.rank_begin && rank < seg.rank_end &&
                  XP_CHECKED(member < ne && (u64)pos2 < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
         }
-        ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
+        if (hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
         if (ok) {
             const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos2];
             vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, member)) | (lf.var >= 0 ? 1u << lf.var : 0u);
@@ -354,9 +386,9 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
     __syncwarp();
     const u32 nc = w.nc;
     const int n_exact = hole->n_exact;
-    const bool classes = seg.classes != 0, four = !hole->aff_ok || plan.n_join <= (u64)gridDim.x * kJoinWarps;
+    const bool classes = XP_CLASSES(seg) != 0, four = !XP_JOIN_BATCH && (!hole->aff_ok || plan.n_join <= (u64)gridDim.x * kJoinWarps);
     for (u32 at = 0; at < nc; at += 32) {
-        const bool spread = nc - at <= 4u;
+        const bool spread = !XP_JOIN_BATCH && nc - at <= 4u;
         u32 good = 0;                                     // spread: bit i: candidate i passes
         bool pass = false;
         u64 rank = 0, e = 0;
@@ -410,7 +442,7 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
             }
         }
         if (classes) { join_members(w, plan, seg, sk, hole, pass, e, pos, code, n); continue; }
-        pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
+        if (n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
         join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
     }
     __syncwarp();
@@ -917,7 +949,7 @@ __device__ __noinline__ void join_exact32(JoinWarp& w, const PlanDev& plan, cons
     const bool two = hole->n_exact >= 2;
     i64 a0 = 0, a1 = 0;
     if (live) {
-        const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, seg.classes ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e);
+        const OperandRef ref = operand_ref(g, hole, seg.nt, seg.esize, XP_CLASSES(seg) ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e);
         live = ref_value(g, hole, ref, seg.nt, seg.esize, 0, a0) && (!two || ref_value(g, hole, ref, seg.nt, seg.esize, 1, a1));
     }
     const u32 n_live = (u32)__popc(__ballot_sync(0xffffffffu, live));
@@ -1252,7 +1284,7 @@ __device__ __noinline__ void join_fill(JoinWarp& w, const PlanDev& plan, const J
 // What `count` operands from number `first` on stand for in the count of candidates: themselves, or, where the segment counts by class, the
 // first ticket's for all there are.
 __device__ __forceinline__ u64 seg_operands(const JoinSeg& seg, const GrammarDev* g, u64 first, u64 count) {
-    return !seg.classes ? count : first == 0ull ? g->cnt[seg.nt][seg.esize] : 0ull;
+    return !XP_CLASSES(seg) ? count : first == 0ull ? g->cnt[seg.nt][seg.esize] : 0ull;
 }
 
 // Operands [first, first + count) of a segment against the leaves (count <= the segment's chunk).
@@ -1278,7 +1310,7 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
     u32 nq = w.nq;
     u32 n_alive = 0;
     for (u64 done = 0; done < count;) {
-        const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done, seg.classes != 0);
+        const JoinRun c = join_run(g, hole, seg.nt, seg.esize, first + done, XP_CLASSES(seg) != 0);
         const u32 n_run = (u32)(c.left < count - done ? c.left : count - done);
         const u32 off0 = (u32)(first + done - w.base) + lane;
         for (u32 at = 0; at < n_run; at += 32u * P) {
@@ -1559,7 +1591,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         i64 pl = -kMost, ph = kMost, ml = -kMost, mh = kMost;
         bool live = false, wide = false;
         if (have) {
-            ref = operand_ref(g, hole, seg.nt, seg.esize, seg.classes ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e);
+            ref = operand_ref(g, hole, seg.nt, seg.esize, XP_CLASSES(seg) ? class_operand(g, hole, seg.nt, seg.esize, e).rank(0) : e);
             live = true;
             for (int j0 = 0; j0 < np && live && !wide; j0 += kProbeStep) {
                 i64 val[kProbeStep];
@@ -1738,7 +1770,7 @@ __device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, con
             }
             vars = ref_vars(hole, ref);
         }
-        pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
+        if (n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
         const u32 b = __ballot_sync(0xffffffffu, pass);
         n.suspects += (u32)__popc(b);
         join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
@@ -1793,7 +1825,9 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
             const u64 count = seg.e_count - from < chunk ? seg.e_count - from : chunk;
             if (seg.kind == kJoinDirect) direct_ticket(w, plan, seg, sk, hole, first, count, n);
             else if (!hole->aff_ok && !seg.exact) range_ticket(w, plan, seg, sk, hole, first, count, (int)part, n);
+#if !XP_JOIN_BATCH
             else if (seg.parts > 0) join_few(w, plan, seg, sk, hole, first, count, (int)part, n);
+#endif
             else join_ticket<P>(w, plan, seg, sk, hole, first, count, n);
         }
         u64 next = 0;
@@ -1804,4 +1838,5 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
     join_flush(plan, acc, n);
 }
 
+}
 }  // namespace xp

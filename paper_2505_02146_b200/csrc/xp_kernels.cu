@@ -2485,7 +2485,12 @@ __global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const __gri
 
 }  // namespace xp
 #include "xp_classes.cuh"
+#define XP_JOIN_BATCH 1
 #include "xp_join.cuh"
+#undef XP_JOIN_BATCH
+#define XP_JOIN_BATCH 0
+#include "xp_join.cuh"
+namespace xp { using namespace join_full; }
 #include "xp_pairs.cuh"
 namespace xp {
 
@@ -3354,7 +3359,9 @@ cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64
         // a wave of persistent CTAs; a small search gets one warp per ticket on as many SMs as there are tickets
         u64 ctas = t_end - t_begin;
         if (ctas > (u64)R->join) ctas = R->join;
-        if (L.join_wide) chain(join_kernel<kJoinP>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
+        if (L.join_batch && L.join_wide) chain(join_batch::join_kernel<kJoinP>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
+        else if (L.join_batch) chain(join_batch::join_kernel<1>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
+        else if (L.join_wide) chain(join_kernel<kJoinP>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
         else chain(join_kernel<1>, (unsigned)ctas, kJoinThreads, 0, stream, pd);
     } else {
         pd.ticket_base = t_begin;

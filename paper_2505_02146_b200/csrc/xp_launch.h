@@ -59,6 +59,7 @@ struct SearchLayout {
     int n_segs, n_jsegs, n_psegs, n_sketches, n_acc;
     int dense;                       // some hole of the plan takes the second look: launch the search kernel's dense form
     int join_wide;                   // tickets of the leaf join are long enough for several operands per lane
+    int join_batch;                  // a batch without classes or tickets in parts: the leaf join's form for those
     int empty_domain;                // some sketch has no points at all
 };
 

@@ -72,7 +72,7 @@ __device__ __noinline__ void pair_members(PairWarp& w, const PlanDev& plan, cons
             ok = rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(rr < seg.right_count && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
             if (ok) vars = (u32)hole->tab_vars[L.off + lr] | (u32)hole->tab_vars[R.off + rr];
         }
-        ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
+        if (hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
         u32 m = __ballot_sync(0xffffffffu, ok);
         if (!m) continue;
         n.passes += (u32)__popc(m);
