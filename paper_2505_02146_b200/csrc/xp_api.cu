@@ -594,6 +594,7 @@ static u64 table_entries(const xp_grammar* g, int max_size, u64 (*off)[kMaxSize 
 // operand of the search is itself above the tables, each of them is met at least a hundred times; where the context compares, an
 // operand costs some ten thousand instructions against some hundred here.  Otherwise every operand is met once, and would be here too.
 constexpr u64 kClassLeast = 4096;            // subtrees from which it pays
+constexpr u64 kRangeMost = 1ull << 18;       // operands of a hole whose context compares from which the tiles take a leaf at the root too
 static void class_plan(const xp_grammar* g, const xp_hole_desc& hd, HoleHost* h) {
     int tmax = 0, top = 0, need = 0;
     (void)table_entries(g, hd.max_size, nullptr, &tmax);
@@ -606,7 +607,8 @@ static void class_plan(const xp_grammar* g, const xp_hole_desc& hd, HoleHost* h)
     if (all < kClassLeast) return;
     bool compares = false;
     for (int i = 0; i < hd.ctx_len; ++i) compares = compares || (hd.ctx[i].kind == XP_I_OP && (hd.ctx[i].arg == XP_OP_LT || hd.ctx[i].arg == XP_OP_LE));
-    h->cls_want = (need > top ? kClassAffine | kClassCompare : 0) | (compares ? kClassCompare : 0);
+    compares = compares && g->cnt[hd.start_nt][top] <= kRangeMost;       // (with more, such a context's operands go as tiles)
+    h->cls_want = (need > top ? kClassAffine : 0) | (compares ? kClassCompare : 0);
     if (h->cls_want) { h->cls_top = top; h->cls_entries = all; h->cls_most = most; }
 }
 
@@ -1452,7 +1454,6 @@ constexpr u64 kPairEach = 1ull << 12;
 constexpr i32 kRangeParts = 4;               // parts of the constants there: a warp checks its suspects by itself, some hundred of them from 32 operands and all
                                              // constants (three conv holes: join 440 us in one part, 350 with 8 operands a ticket, 330 so)
 constexpr u64 kRangeSplit = 1ull << 15;      // ... up to which an operator is a segment of its own (with more there are warps enough at work)
-constexpr u64 kRangeMost = 1ull << 18;       // operands of a hole whose context compares from which the tiles take a leaf at the root too
 
 // Does the pair join know the block (production, left size a) of size k?  Both operands tabulated, an operator it has
 // (products only where neither target is zero: a zero operand would leave its partner open).
@@ -1911,8 +1912,11 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 if (!ho.filter_ok || (o->flags & XP_FLAG_NO_FILTER)) { add_linear(plan, (int)i, h, acc, k, lo, hi); continue; }
                 if (k < 3 || (!forced && hi - lo < kTileMinRanks)) { add_direct(plan, ho.start_nt, (int)i, h, acc, k, lo, hi); continue; }
                 // (A range of hole values: the join's interval arithmetic per operand against a test per candidate.  27 leaves, size 7, 984 000
-                // operands, four specs: 13.4, 26.5, 10.2, 14.4 ms by the join, 14.9, 19.8, 10.7, 8.2 as tiles; 40 leaves, size 5: 0.4 against 1.4.)
-                const bool leaves = ho.compares && class_operands(s->g, ho, ho.start_nt, k - 2) > kRangeMost;
+                // operands, four specs: 13.4, 26.5, 10.2, 14.4 ms by the join, 14.9, 19.8, 10.7, 8.2 as tiles; 40 leaves, size 5: 0.4 against 1.4.
+                // What decides is the operands, not their classes: with so many the tables hold few probes, and a class is taken apart for each
+                // candidate that passes those.  40 leaves, size 7, 3.2 million operands, three specs: 210, 1290, 212 ms as tiles, 2270, 4220,
+                // 2400 by the join over classes; with a shift 144, 128 against 1500, 159, with a leaf of 2^33 119, 965 against 64, 807.)
+                const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
                 if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, form != kFormMany);
                 const bool pairs = form >= kFormPairsSome;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);

@@ -483,6 +483,8 @@ def test_many_operands_under_a_comparison(xp, ctx, spec):
     sk = Sketch(g, [Hole(0, 7, ctx=parse_expr(ctx, IJ), spec_expr=parse_expr(ctx.replace("HOLE", f"({spec})"), IJ))], name=ctx)
     n = oracle.counts(g, 0, 7)
     assert n[5] > 2**18
+    whole = xp.xp_repair(xp.xp_sketch_load(xp.xp_grammar_create(g), sk), size_min=7, size_max=7)[0]
+    assert whole.n_launches == 2                                        # tiles and the whole-domain check, no leaf join
     for p in range(5):
         at = p * (n[7] // 5)
         check_sketch(xp, sk, windows={1: (0, 0), 3: (0, 0), 5: (0, 0), 7: (at + 7, at + 100_000)})
