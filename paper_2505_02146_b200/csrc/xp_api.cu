@@ -1981,6 +1981,11 @@ static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size
     w.sorted = w.sort_off + align256(sizeof(u32) * (n_acc + 2));
     w.longs = w.sorted + align256(sizeof(u32) * (size_t)surv_cap);
     w.total = w.longs + align256(sizeof(u32) * (size_t)surv_cap);
+    // (the list of what candidates over classes stand for is where the hole order will be: that is made once the list has been worked off)
+    bool classes = false;
+    for (const JoinSeg& c : plan.jsegs) classes = classes || c.classes;
+    for (const PairSeg& c : plan.psegs) classes = classes || c.lcls || c.rcls;
+    w.member_cap = classes ? (u32)(sizeof(u32) * (size_t)surv_cap / sizeof(MemberRec)) : 0;
     w.n_psegs = (int)plan.psegs.size();
     w.pair_ones = w.total;
     for (const PairSeg& c : plan.psegs) w.total += align256(sizeof(u32) * ((size_t)c.head_mask + 1));
@@ -2109,6 +2114,11 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     XP_CUDA_R(cudaMemcpyAsync(ws, stage.p, w.head, cudaMemcpyHostToDevice, stream));
     XP_CUDA_R(cudaEventRecord(ev.e0, stream));
     xp_status stopped = XP_OK;
+    auto give_up = [&](bool more) {                       // after a bounded launch
+        if (o->cancel && *o->cancel) return XP_ERR_CANCELLED;
+        const double spent = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+        return o->timeout_ms > 0 && more && spent >= (double)o->timeout_ms ? XP_ERR_TIMEOUT : XP_OK;
+    };
     if (!o->cancel && o->timeout_ms <= 0) {
         XP_CUDA_R(launch_search_part(ws, w, true, 0, plan.n_join, false, stream, &launches));
         XP_CUDA_R(launch_search_part(ws, w, false, 0, plan.n_tickets, false, stream, &launches));
@@ -2121,16 +2131,28 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
                 const u64 t_end = t + (u64)XP_CANCEL_TICKETS < n_items ? t + (u64)XP_CANCEL_TICKETS : n_items;
                 XP_CUDA_R(launch_search_part(ws, w, kind == 0, t, t_end, t > 0, stream, &launches));
                 XP_CUDA_R(cudaStreamSynchronize(stream));
-                const bool more = t_end < n_items || (kind == 0 && plan.n_tickets > 0);
-                if (o->cancel && *o->cancel) stopped = XP_ERR_CANCELLED;
-                else if (o->timeout_ms > 0 && more &&
-                         std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count() >= (double)o->timeout_ms)
-                    stopped = XP_ERR_TIMEOUT;
+                stopped = give_up(t_end < n_items || (kind == 0 && plan.n_tickets > 0));
             }
         }
     }
     if (stopped == XP_OK) {
         XP_CUDA_R(launch_pairs(ws, w, plan.psegs.data(), stream, &launches));
+        if (!o->cancel && o->timeout_ms <= 0) XP_CUDA_R(launch_members(ws, w, 0, ~0ull, false, stream, &launches));
+    }
+    if (stopped == XP_OK && (o->cancel || o->timeout_ms > 0) && w.member_cap > 0) {
+        // (in bounded launches too; how many pieces there are is known by now)
+        u64* listed = (u64*)(check_word + 2);
+        XP_CUDA_R(cudaMemcpyAsync(listed, ws + 48, sizeof(*listed), cudaMemcpyDeviceToHost, stream));
+        XP_CUDA_R(cudaStreamSynchronize(stream));
+        const u64 pieces = *listed & ((1ull << 44) - 1);
+        for (u64 t = 0; (t == 0 || t < pieces) && stopped == XP_OK; t += (u64)XP_CANCEL_TICKETS) {
+            const u64 end = t + (u64)XP_CANCEL_TICKETS < pieces ? t + (u64)XP_CANCEL_TICKETS : pieces;
+            XP_CUDA_R(launch_members(ws, w, t, end, t > 0, stream, &launches));
+            XP_CUDA_R(cudaStreamSynchronize(stream));
+            stopped = give_up(end < pieces);
+        }
+    }
+    if (stopped == XP_OK) {
         bool told = false;
         XP_CUDA_R(launch_search_end(ws, w, plan.n_tickets + plan.n_join + plan.psegs.size() > 0, stage.locked ? (AccDev*)(stage.p + w.head) : nullptr, &told, stream, &launches));
         XP_CUDA_R(cudaEventRecord(ev.e1, stream));

@@ -195,4 +195,43 @@ __device__ __noinline__ ClassOperand class_operand(const GrammarDev* g, const Ho
     return c;                                             // (not reached: e is below the count that the host made the same way)
 }
 
+// ---- candidates that stand for many ----
+
+// A warp that has met candidates over classes takes them apart by itself while that is a few steps (member_own: fewer as the survivor queue fills;
+// once it is full each member that is left costs a whole-domain check).  Larger ones go to a list, whose
+// pieces all warps of the device share afterwards: subtrees that are 0 everywhere are one class of thousands, and where the target is one of
+// a few values (a term that collapses, a domain of few points, a guard that always holds) most matches belong to a few such classes, hence to a few
+// warps.  (16x12x8 points, 45 and 53 leaves, size 7, 6 and 10 million matches: operand by operand 1.19 and 1.45 s, by class
+// and the warps that met them 3.2 and 6.6.)
+constexpr u64 kMemberLeast = 16;             // members from which an entry pays; four times as many for each quarter of the list that is taken, so that the
+                                             // largest classes find a place (68 leaves, 2.2e7 matches: 7.8 s without, 2.1 with it)
+constexpr u64 kMemberMost = 1ull << 32;      // members of an entry; a larger one stays with its warp (entries, 2^17 and a warp's 32 more each, and
+                                             // pieces, 2^43 and 2^31 a warp, then stay in their parts of the counter)
+__device__ __forceinline__ u64 member_own(const PlanDev& plan) {
+    const u32 taken = __shfl_sync(0xffffffffu, *(volatile const u32*)plan.surv_n, 0);
+    return taken >= plan.surv_cap ? 32u : taken >= plan.surv_cap / 4u ? 256u : 1024u;
+}
+// The candidates of the lanes with `want` (count members each) to the list; returns whether this lane's is in it.  Called by all lanes.
+__device__ __noinline__ bool list_members(const PlanDev& plan, bool want, u64 count, u64 e, u32 pos, u32 code, i32 seg) {
+    const int lane = threadIdx.x & 31;
+    if (!plan.members) return false;
+    u64 now = 0;
+    if (lane == 31) now = *(volatile const u64*)plan.members_n;
+    now = __shfl_sync(0xffffffffu, now, 31);
+    if ((now >> 44) >= plan.member_cap || ((now >> 43) & 1u)) return false;
+    want = want && count >= kMemberLeast << (2u * ((u32)(now >> 44) * 4u / plan.member_cap)) && count <= kMemberMost;
+    const u32 m = __ballot_sync(0xffffffffu, want);
+    if (!m) return false;
+    const u64 pieces = want ? (count + kMemberPiece - 1) / kMemberPiece : 0ull;
+    u64 incl = pieces;
+    for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+    u64 old = 0;
+    if (lane == 31) old = atomicAdd((unsigned long long*)plan.members_n, ((u64)__popc(m) << 44) | incl);
+    old = __shfl_sync(0xffffffffu, old, 31);
+    const u64 at = (old >> 44) + (u64)__popc(m & ((1u << lane) - 1u));
+    const bool in = want && at < plan.member_cap;
+    if (in) plan.members[at] = MemberRec{e, (old & ((1ull << 44) - 1)) + incl - pieces, pos, code, seg, (u32)pieces};
+    return in;
+}
+
 }  // namespace xp

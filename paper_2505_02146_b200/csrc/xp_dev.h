@@ -310,6 +310,16 @@ struct PairSeg {
     int2* val[2];
 };
 
+// A candidate over operand classes that stands for many, left to members_kernel (csrc/xp_members.cuh) in pieces.
+struct MemberRec {
+    u64 e;                           // leaf join: number of the operand; pair join: left | right << 32
+    u64 first;                       // pieces of the entries before it
+    u32 pos, code;                   // leaf join: position of the leaf, group << 8 | slot << 1 | swapped; pair join: -, slot
+    i32 seg;                         // of the leaf join, or ~ of the pair join
+    u32 pieces;
+};
+constexpr u32 kMemberPiece = 64;     // members of a piece
+
 // One contiguous piece of work.  kind 0 (linear): ranks [rank_begin, rank_end) of `size`,
 // every candidate unranked on its own.  kind 1 (tile): the product of left subtrees
 // [a_begin, a_begin+a_count) x right subtrees of one (production group, left size).
@@ -383,6 +393,12 @@ struct PlanDev {
     // listed after the search so that the later chunks are walked for them alone.
     u32* surv_long;                  // device, surv_cap
     u32* surv_long_n;                // device counter, zero at launch
+    // The list of members_kernel (null: no operand of the call is a class): entries << 44 | their pieces (entries may run past
+    // member_cap), zero at launch; the counter of pieces taken; the pieces [member_base, member_end) belong to this launch.
+    MemberRec* members;
+    u64 *members_n, *member_ticket;
+    u64 member_base, member_end;
+    u32 member_cap, pad1;
     u32* verify_done;                // device counter of finished CTAs of the verification kernel, zero at launch
     AccDev* told;                    // page-locked: where the CTA that finishes last puts the accumulators (null: the host copies them)
 };

@@ -285,7 +285,7 @@ __device__ __noinline__ void join_verify(CandShared& cand, const PlanDev& plan, 
 
 // Candidates that passed the probes (one per lane at most) go to the survivor queue, or are checked
 // by the warp.  Called by all 32 lanes together.
-__device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, const JoinSeg& seg,
+__device__ __forceinline__ void join_survive(CandShared& cand, const PlanDev& plan, const SketchDev* sk, const HoleDev* hole, const JoinSeg& seg,
                                              bool pass, u64 rank, u32 vars, JoinCount& n) {
     u32 m = __ballot_sync(0xffffffffu, pass);
     if (!m) return;
@@ -299,7 +299,7 @@ __device__ __forceinline__ void join_survive(JoinWarp& w, const PlanDev& plan, c
     while (m) {
         const int src = __ffs((int)m) - 1;
         m &= m - 1;
-        join_verify(w.cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
+        join_verify(cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, src), __shfl_sync(0xffffffffu, vars, src), n.evals);
     }
 }
 
@@ -340,40 +340,52 @@ __device__ __noinline__ bool join_full_check(const GrammarDev* g, const HoleDev*
 #endif
 }
 
+// A member per lane (in: this lane has one): operand `member` of (nt, esize) under the leaf and operator of pos and code.  Called by all lanes.
+__device__ __forceinline__ void join_member(CandShared& cand, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, bool in, u64 member, u32 pos,
+                                         u32 code, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    const int swap = (int)(code & 1u), slot = (int)((code >> 1) & 15u);
+    const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code >> 8)];
+    bool ok = false;
+    u64 rank = 0;
+    u32 vars = 0;
+    if (in) {
+        const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
+        rank = grp.base[swap][slot] + (swap ? (u64)pos * ne + member : member * nl + (u64)pos);
+        ok = rank >= seg.rank_begin && rank < seg.rank_end &&
+             XP_CHECKED(member < ne && (u64)pos < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
+    }
+    if (hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
+    if (ok) {
+        const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos];
+        vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, member)) | (lf.var >= 0 ? 1u << lf.var : 0u);
+    }
+    join_survive(cand, plan, sk, hole, seg, ok, rank, vars, n);
+}
+
 // Candidates of a segment that counts by class, one per lane (pass: this lane has one, and it satisfies the probes with tables):
-// every member of the class is a candidate of its own, 32 at a time over all lanes' members.  Called by all lanes.
+// every member of the class is a candidate of its own, 32 at a time over all lanes' members, or left to members_kernel.  Called by all lanes.
 __device__ __noinline__ void join_members(JoinWarp& w, const PlanDev& plan, const JoinSeg& seg, const SketchDev* sk, const HoleDev* hole, bool pass, u64 e, u32 pos,
                                           u32 code, JoinCount& n) {
     if (!__any_sync(0xffffffffu, pass)) return;
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
-    u64 incl = pass ? class_operand(g, hole, seg.nt, seg.esize, e).members() : 0ull;
-    for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
-    const u64 total = __shfl_sync(0xffffffffu, incl, 31);
+    u64 mine = pass ? class_operand(g, hole, seg.nt, seg.esize, e).members() : 0ull, incl, total;
+    for (int listed = 0;; ++listed) {
+        incl = mine;
+        for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        total = __shfl_sync(0xffffffffu, incl, 31);
+        if (listed || total <= member_own(plan)) break;
+        if (list_members(plan, mine > 0u, mine, e, pos, code, (i32)(&seg - plan.jsegs))) mine = 0;
+    }
     for (u64 k0 = 0; k0 < total; k0 += 32u) {
         const u64 k = k0 + (u64)lane < total ? k0 + (u64)lane : total - 1u;
         int src = 0;                                      // the lane whose member this is: the first with incl > k
         for (int step = 16; step > 0; step >>= 1) { const u64 v = __shfl_sync(0xffffffffu, incl, src + step - 1); if (v <= k) src += step; }
         const u64 before = __shfl_sync(0xffffffffu, incl, src ? src - 1 : 0), e2 = __shfl_sync(0xffffffffu, e, src);
         const u32 pos2 = __shfl_sync(0xffffffffu, pos, src), code2 = __shfl_sync(0xffffffffu, code, src);
-        bool ok = false;
-        u64 rank = 0, member = 0;
-        u32 vars = 0;
-        const int swap = (int)(code2 & 1u), slot = (int)((code2 >> 1) & 15u);
-        const JoinGroup& grp = plan.jgroups[seg.first_group + (int)(code2 >> 8)];
-        if (k0 + (u64)lane < total) {
-            const u64 nl = g->cnt[grp.leaf_nt][1], ne = g->cnt[seg.nt][seg.esize];
-            member = class_operand(g, hole, seg.nt, seg.esize, e2).rank(src ? k - before : k);
-            rank = grp.base[swap][slot] + (swap ? (u64)pos2 * ne + member : member * nl + (u64)pos2);
-            ok = rank >= seg.rank_begin && rank < seg.rank_end &&
-                 XP_CHECKED(member < ne && (u64)pos2 < nl && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
-        }
-        if (hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
-        if (ok) {
-            const LeafDev lf = g->leaves[g->leaf_begin[grp.leaf_nt] + (int)pos2];
-            vars = ref_vars(hole, operand_ref(g, hole, seg.nt, seg.esize, member)) | (lf.var >= 0 ? 1u << lf.var : 0u);
-        }
-        join_survive(w, plan, sk, hole, seg, ok, rank, vars, n);
+        const bool in = k0 + (u64)lane < total;
+        join_member(w.cand, plan, seg, sk, hole, in, in ? class_operand(g, hole, seg.nt, seg.esize, e2).rank(src ? k - before : k) : 0ull, pos2, code2, n);
     }
 }
 
@@ -443,7 +455,7 @@ __device__ __noinline__ void join_check(JoinWarp& w, const PlanDev& plan, const 
         }
         if (classes) { join_members(w, plan, seg, sk, hole, pass, e, pos, code, n); continue; }
         if (n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
-        join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
+        join_survive(w.cand, plan, sk, hole, seg, pass, rank, vars, n);
     }
     __syncwarp();
     if (lane == 0) w.nc = 0;
@@ -1773,7 +1785,7 @@ __device__ __noinline__ void direct_ticket(JoinWarp& w, const PlanDev& plan, con
         if (n_exact < hole->n_probe) pass = join_full_check(g, hole, seg.size, pass, rank, n.evals);
         const u32 b = __ballot_sync(0xffffffffu, pass);
         n.suspects += (u32)__popc(b);
-        join_survive(w, plan, sk, hole, seg, pass, rank, vars, n);
+        join_survive(w.cand, plan, sk, hole, seg, pass, rank, vars, n);
     }
 }
 

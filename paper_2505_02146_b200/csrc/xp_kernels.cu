@@ -5,6 +5,7 @@
 //   subvalue_kernel, stage_sample_kernel, coord_bounds_kernel -- per sketch,
 //                      once at load: values (and variable sets) of all small subtrees at the probes;
 //                      points and spec values of a box; coordinate bounds of a table.
+//   members_kernel  -- (xp_members.cuh) candidates over operand classes that stand for many.
 //   join_kernel     -- (xp_join.cuh) the part of the search whose candidates have a leaf at the root.
 //   eval_kernel     -- the rest of the search.  Persistent CTAs take tickets (pieces of the rank space)
 //                      from an atomic counter; no CTA ever waits for another.
@@ -2492,6 +2493,7 @@ __global__ void __launch_bounds__(kThreads, XP_MIN_CTAS) eval_kernel(const __gri
 #include "xp_join.cuh"
 namespace xp { using namespace join_full; }
 #include "xp_pairs.cuh"
+#include "xp_members.cuh"
 namespace xp {
 
 // ------------------------------------------------------------------------------------------
@@ -3279,7 +3281,7 @@ cudaError_t launch_classes(SketchDev* s, int hole, char* scratch, u64 entries, u
 
 // CTAs of a kernel that fit the device at a time, and the SM count: asked once per device (the queries, and
 // the shared-memory attribute of the verification kernel, cost a microsecond or two each).
-struct Residency { int sms, eval_sparse, eval_dense, verify, join; };
+struct Residency { int sms, eval_sparse, eval_dense, verify, join, members; };
 static const Residency* residency() {
     static Residency table[64];
     static std::atomic<int> known[64];
@@ -3298,6 +3300,7 @@ static const Residency* residency() {
     r.eval_dense = r.sms * per_sm((const void*)eval_kernel<true>, kThreads, 0);
     r.verify = r.sms * per_sm((const void*)verify_kernel, kVerifyThreads, vsmem);
     r.join = r.sms * per_sm((const void*)join_kernel<kJoinP>, kJoinThreads, 0);
+    r.members = r.sms * per_sm((const void*)members_kernel, kMemberThreads, 0);
     static std::mutex mu;                                 // (two first calls at the same time compute the same values)
     std::lock_guard<std::mutex> lock(mu);
     table[dev] = r;
@@ -3337,6 +3340,11 @@ static PlanDev plan_on(char* base, const SearchLayout& L) {
     pd.surv_long = (u32*)(base + L.longs);
     pd.surv_long_n = (u32*)(base + 24);
     pd.verify_done = (u32*)(base + 40);
+    pd.members = L.member_cap ? (MemberRec*)(base + L.sorted) : nullptr;
+    pd.members_n = (u64*)(base + 48);
+    pd.member_ticket = (u64*)(base + 56);
+    pd.member_base = 0; pd.member_end = ~0ull;
+    pd.member_cap = L.member_cap; pd.pad1 = 0;
     pd.told = nullptr;
     return pd;
 }
@@ -3413,6 +3421,20 @@ cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_
     return cudaSuccess;
 }
 
+// The pieces [begin, end) of what the joins have listed over classes; `restart` as above.
+cudaError_t launch_members(char* base, const SearchLayout& L, u64 begin, u64 end, bool restart, cudaStream_t stream, int* n_launches) {
+    if (L.member_cap == 0) return cudaSuccess;
+    const Residency* R = residency();
+    if (!R) return cudaErrorInvalidDevice;
+    cudaError_t e;
+    if (restart && (e = cudaMemsetAsync(base + 56, 0, 8, stream)) != cudaSuccess) return e;
+    PlanDev pd = plan_on(base, L);
+    pd.member_base = begin; pd.member_end = end;
+    chain(members_kernel, (unsigned)R->members, kMemberThreads, 0, stream, pd);
+    *n_launches += 1;
+    return cudaGetLastError();
+}
+
 // Stage 3, after every part of the search has been queued.  acc_out: page-locked memory for the accumulators (or null).  Where
 // there are few of them the verification kernel writes them there itself (*told): a copy of some hundred bytes takes the
 // stream as long as one of 20 KB, 4 to 5 us of a small call.
@@ -3452,6 +3474,7 @@ static cudaError_t launch_search(char* base, const SearchLayout& L, u64 n_ticket
                                  int* n_launches) {
     cudaError_t e = launch_search_part(base, L, true, 0, n_join, false, stream, n_launches);
     if (e == cudaSuccess) e = launch_search_part(base, L, false, 0, n_tickets, false, stream, n_launches);
+    if (e == cudaSuccess) e = launch_members(base, L, 0, ~0ull, false, stream, n_launches);
     if (e != cudaSuccess) return e;
     return launch_search_end(base, L, n_tickets + n_join > 0, acc_out, told, stream, n_launches);
 }

@@ -47,14 +47,16 @@ inline size_t class_scratch_bytes(u64 entries) { return entries ? sizeof(u64) * 
 cudaError_t launch_classes(SketchDev* s, int hole, char* scratch, u64 entries, u64 most, int n_nt, LoadOut* out, cudaStream_t stream);
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
-//      build only), 24: long survivors (u32), 32: join ticket (u64), 40: finished verification CTAs (u32)   -- zero at launch
+//      build only), 24: long survivors (u32), 32: join ticket (u64), 40: finished verification CTAs (u32), 48: listed members
+//      (u64: MemberRec entries and pieces), 56: ticket of those pieces (u64)   -- zero at launch
 //   segs, jsegs, jgroups, psegs, sketches, acc: staged from the host;  [0, head) is what the host copies in
 //   hist: survivors per accumulator slot, zero at launch (staged);
-//   surv: the survivor queue (surv_cap entries); sort_off, sorted: its hole order -- written by the kernels only
+//   surv: the survivor queue (surv_cap entries); sort_off, sorted: its hole order (before that the list of members_kernel) -- written by the kernels only
 struct SearchLayout {
     size_t segs, jsegs, jgroups, psegs, sketches, acc, hist, head, surv, sort_off, sorted, longs, total;
     size_t pair_ones, pair_zeros, pair_rest;      // scratch of the pair join: [pair_ones, pair_zeros) all ones, [pair_zeros, pair_rest) zero at launch
     i32 first_points;                // points of the largest domain, at most kVerifyChunk
+    u32 member_cap;                  // entries of the list of members_kernel (0: no operand of the call is a class)
     u32 surv_cap, max_chunks;        // max_chunks: chunks of the whole-domain check that the largest domain needs
     int n_segs, n_jsegs, n_psegs, n_sketches, n_acc;
     int dense;                       // some hole of the plan takes the second look: launch the search kernel's dense form
@@ -67,6 +69,7 @@ struct SearchLayout {
 cudaError_t launch_search_part(char* base, const SearchLayout& L, bool join, u64 t_begin, u64 t_end, bool restart, cudaStream_t stream,
                                int* n_launches);
 cudaError_t launch_pairs(char* base, const SearchLayout& L, const PairSeg* host_segs, cudaStream_t stream, int* n_launches);
+cudaError_t launch_members(char* base, const SearchLayout& L, u64 begin, u64 end, bool restart, cudaStream_t stream, int* n_launches);
 cudaError_t launch_search_end(char* base, const SearchLayout& L, bool any_tickets, AccDev* acc_out, bool* told, cudaStream_t stream, int* n_launches);
 int search_warps();                                  // warps of the leaf join that run at a time
 constexpr size_t kStaticScratchBytes = 1u << 20;     // fixed scratch of the allocation-free entry point

@@ -42,18 +42,46 @@ __device__ __forceinline__ PairSide pair_side(const GrammarDev* g, const HoleDev
     return PairSide{s.pair + skip, s.start, s.mem, hole->tab_off[nt][size] + skip};
 }
 
+// A member per lane (in: this lane has one): left and right operand by rank.  Called by all lanes.
+__device__ __noinline__ void pair_member(CandShared& cand, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, const PairSide& L, const PairSide& R,
+                                         bool in, u32 lr, u32 rr, int slot, JoinCount& n) {
+    const GrammarDev* g = sk->g;
+    bool ok = false;
+    u64 rank = 0;
+    u32 vars = 0;
+    if (in) {
+        rank = seg.base[slot] + (u64)lr * seg.right_count + rr;
+        ok = rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(rr < seg.right_count && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
+        if (ok) vars = (u32)hole->tab_vars[L.off + lr] | (u32)hole->tab_vars[R.off + rr];
+    }
+    if (hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
+    u32 m = __ballot_sync(0xffffffffu, ok);
+    if (!m) return;
+    n.passes += (u32)__popc(m);
+    m = __ballot_sync(0xffffffffu, push_survivors(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, ok, rank, vars));
+    while (m) {
+        const int at = __ffs((int)m) - 1;
+        m &= m - 1;
+        join_verify(cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, at), __shfl_sync(0xffffffffu, vars, at), n.evals);
+    }
+}
+
 // Pairs that satisfy the probes, one per lane (pass: this lane has one): to the survivor queue, the members of classes one by one, 32 at a
-// time over all lanes' pairs.  Called by all lanes.
+// time over all lanes' pairs, or left to members_kernel.  Called by all lanes.
 __device__ __noinline__ void pair_members(PairWarp& w, const PlanDev& plan, const PairSeg& seg, const SketchDev* sk, const HoleDev* hole, bool pass, u32 l, u32 r,
                                           int slot, JoinCount& n) {
     if (!__any_sync(0xffffffffu, pass)) return;
-    const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
-    const PairSide L = pair_side(g, hole, seg, false), R = pair_side(g, hole, seg, true);
+    const PairSide L = pair_side(sk->g, hole, seg, false), R = pair_side(sk->g, hole, seg, true);
     const u32 rn = pass ? R.members(r) : 1u;
-    u64 incl = pass ? (u64)L.members(l) * rn : 0ull;
-    for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
-    const u64 total = __shfl_sync(0xffffffffu, incl, 31);
+    u64 mine = pass ? (u64)L.members(l) * rn : 0ull, incl, total;
+    for (int listed = 0;; ++listed) {
+        incl = mine;
+        for (int o = 1; o < 32; o <<= 1) { const u64 v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        total = __shfl_sync(0xffffffffu, incl, 31);
+        if (listed || total <= member_own(plan)) break;
+        if (list_members(plan, mine > 0u, mine, (u64)l | (u64)r << 32, 0u, (u32)slot, ~(i32)(&seg - plan.psegs))) mine = 0;
+    }
     for (u64 k0 = 0; k0 < total; k0 += 32u) {
         const u64 k = k0 + (u64)lane < total ? k0 + (u64)lane : total - 1u;
         int src = 0;                                      // the lane whose member this is: the first with incl > k
@@ -61,27 +89,10 @@ __device__ __noinline__ void pair_members(PairWarp& w, const PlanDev& plan, cons
         const u64 before = __shfl_sync(0xffffffffu, incl, src ? src - 1 : 0);
         const u32 l2 = __shfl_sync(0xffffffffu, l, src), r2 = __shfl_sync(0xffffffffu, r, src), rn2 = __shfl_sync(0xffffffffu, rn, src);
         const int slot2 = __shfl_sync(0xffffffffu, slot, src);
-        bool ok = false;
-        u64 rank = 0;
-        u32 vars = 0;
-        if (k0 + (u64)lane < total) {
-            u64 kl, kr;
-            divmod_u64(src ? k - before : k, (u64)rn2, kl, kr);
-            const u32 lr = L.member(l2, (u32)kl), rr = R.member(r2, (u32)kr);
-            rank = seg.base[slot2] + (u64)lr * seg.right_count + rr;
-            ok = rank >= seg.rank_begin && rank < seg.rank_end && XP_CHECKED(rr < seg.right_count && rank < g->cnt[hole->start_nt][seg.size], kChkQueue);
-            if (ok) vars = (u32)hole->tab_vars[L.off + lr] | (u32)hole->tab_vars[R.off + rr];
-        }
-        if (hole->n_exact < hole->n_probe) ok = join_full_check(g, hole, seg.size, ok, rank, n.evals);
-        u32 m = __ballot_sync(0xffffffffu, ok);
-        if (!m) continue;
-        n.passes += (u32)__popc(m);
-        m = __ballot_sync(0xffffffffu, push_survivors(plan, sk, hole, seg.sketch, seg.hole, seg.size, seg.acc, ok, rank, vars));
-        while (m) {
-            const int at = __ffs((int)m) - 1;
-            m &= m - 1;
-            join_verify(w.cand, plan, sk, hole, seg.size, seg.acc, __shfl_sync(0xffffffffu, rank, at), __shfl_sync(0xffffffffu, vars, at), n.evals);
-        }
+        const bool in = k0 + (u64)lane < total;
+        u64 kl = 0, kr = 0;
+        if (in) divmod_u64(src ? k - before : k, (u64)rn2, kl, kr);
+        pair_member(w.cand, plan, seg, sk, hole, L, R, in, in ? L.member(l2, (u32)kl) : 0u, in ? R.member(r2, (u32)kr) : 0u, slot2, n);
     }
 }
 

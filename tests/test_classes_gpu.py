@@ -95,3 +95,26 @@ def test_quasi_affine_grammar_equals_its_windows(xp, table):
     r = xp.xp_repair(ls, size_min=9, size_max=9)[0]
     match, least = _cut(xp, ls, 9, n, 64)
     assert match > 0 and r.match_count[9] == match and r.least_rank == least
+
+
+def test_matches_in_large_classes(xp):
+    """A target with a term that is 0 (j / 28): millions of matches, most of them in a few classes, which are listed and shared by all
+    warps; with a queue and a list that run over, and in bounded launches."""
+    import torch
+    sk = _large("((j/28)*13)+i")
+    gr = xp.xp_grammar_create(sk.grammar)
+    ls = xp.xp_sketch_load(gr, sk)
+    n = xp.xp_grammar_count(gr, 0, 7)[7]
+    only7 = dict(size_min=7, size_max=7)
+    r = xp.xp_repair(ls, **only7)[0]
+    match, least = _cut(xp, ls, 7, n, 61)
+    assert match > 2**20 and r.match_count[7] == match and r.least_rank == least
+    need = xp.xp_workspace_bytes([ls], **only7)
+    ws = torch.empty(need - 40 * (2**20 - 2**16), dtype=torch.uint8, device="cuda")
+    small = xp.xp_repair(ls, workspace=ws, **only7)[0]
+    assert small.match_count[7] == match and small.least_rank == least
+    bounded = xp.xp_repair(ls, timeout_ms=60_000, **only7)[0]
+    assert bounded.match_count[7] == match and bounded.least_rank == least
+    few = _large("((i*7)+j)*3")                          # (a launch takes 8192 pieces of 64 members; here there are none)
+    few = xp.xp_repair(xp.xp_sketch_load(gr, few), timeout_ms=60_000, **only7)[0]
+    assert bounded.n_launches >= few.n_launches + 3
