@@ -481,6 +481,7 @@ struct HoleHost {
     bool second = false;             // filter hits are looked at once more at probe 1 from the start (hits are frequent)
     int cls_size = 0;                // operands of this size are in classes, cls_n of each nonterminal (0: none)
     u32 cls_n[kMaxNt] = {0};
+    double pass_rate = 0;            // share of the load's sampled candidates that satisfied every probe with tables
     // What the load makes classes of: the size, and for which contexts (0: none); a grammar's subtrees of that size, and of one nonterminal at most.
     int cls_top = 0, cls_want = 0;
     u64 cls_entries = 0, cls_most = 0;
@@ -523,7 +524,7 @@ struct xp_sketch {
     // One per form (PlanForm): each is built once, under the lock, and only read from then on
     // (calls on several threads copy them at the same time); a refinement, during which no search may run, drops them.
     mutable std::mutex plan_mu;
-    mutable std::unique_ptr<const Plan> plan_kept[4];
+    mutable std::unique_ptr<const Plan> plan_kept[8];      // per form, with classes and without for comparing holes with many matches
 };
 
 // What the load's kernels settled for a hole.
@@ -538,6 +539,7 @@ static void hole_decided(HoleHost* h, const LoadOut& o) {
     h->second = o.second != 0;
     h->cls_size = o.cls_size;
     memcpy(h->cls_n, o.cls_n, sizeof(h->cls_n));
+    h->pass_rate = o.sample_n > 0 ? (double)o.sample_pass / (double)o.sample_n : 0.0;
     if (o.spec_bad) h->never = true;                      // the spec is undefined at some point
 }
 
@@ -1382,7 +1384,7 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
             return fail(XP_ERR_CUDA, std::string("xp_sketch_refine: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
         for (int h = 0; h < nh; ++h) {
             LoadOut o{hh[h].filter_ok, hh[h].tab_probes, hh[h].aff_ok, hh[h].join_on, hh[h].second, hh[h].n_probe, hh[h].tab_max_size,
-                      hh[h].join_t0 == 0 || hh[h].join_t1 == 0, 0u, hh[h].cls_size, {0}};
+                      hh[h].join_t0 == 0 || hh[h].join_t1 == 0, hh[h].sample_pass, hh[h].sample_n, 0u, hh[h].cls_size, {0}};
             memcpy(o.cls_n, hh[h].cls_n, sizeof(o.cls_n));
             hole_decided(&s->holes[h], o);
             s->n_probes[h] = hh[h].n_probe;
@@ -1814,10 +1816,17 @@ static void number_joins(Plan* plan) {
 
 constexpr u64 kTileMinRanks = 4096;          // smaller windows are searched rank by rank
 
+// Matches (candidates that satisfy the probes with tables, by the load's sample) that a call's comparing contexts may have for their operands to go by
+// class.  With more the list of members_kernel runs over, and where most candidates of an operand match, sharing the operands among the
+// warps shares the work best.  (100 guards of 29, 40 and 60 leaves, 1000 of 29, a quarter of them nearly always true: 1.7e6, 6e6, 2.6e7, 1.2e7 by the sample;
+// 95, 361, 1131, 715 ms operand by operand, 18, 870, 4500, 1190 by class.  An affine context has few matches per operand: the examples in
+// xp_classes.cuh are 2e7 by the sample.)
+constexpr double kClassMatches = 4.0;                     // ... for each entry of the survivor queue (a call on the fixed scratch has fewer: 20 guards, 28.7 / 59.8 ms)
+
 // What a plan may use: kFormMany, a batch: no pair join; the others, at most kPairMaxSketches sketches: narrow tiles where a block is small, and
 // without the pair join, with it from kPairLeastBatch pairs on, or from kPairLeast on.
 enum PlanForm { kFormMany = 0, kFormTiles = 1, kFormPairsSome = 2, kFormPairs = 3 };
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, Plan* plan);
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, bool dense, Plan* plan);
 
 // A sketch's tables, and the library's scratch, live on the device that was current when the sketch was
 // loaded: a call made with another device current would hand the kernels pointers of the wrong GPU.
@@ -1831,26 +1840,32 @@ static xp_status check_device(const xp_sketch* const* sk, size_t n) {
     return XP_OK;
 }
 
-// (may_pair: the call's scratch has room for the pair join's index)
-static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, bool may_pair, Plan* plan) {
+// (may_pair: the call's scratch has room for the pair join's index; queue: entries of its survivor queue)
+static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repair_opts* o, bool may_pair, u32 queue, Plan* plan) {
     // the pair join takes its blocks one after the other, several launches each: a batch keeps to the tiles, which
     // search all holes in one launch.  So does a call with a cancel word or a time limit: its launches are bounded, and the
     // host looks at both between them; a pair join's launch covers a whole block.
     const bool pairs = may_pair && !o->cancel && o->timeout_ms <= 0;
     const PlanForm form = n > kPairMaxSketches ? kFormMany : !pairs ? kFormTiles : n > kPairFew ? kFormPairsSome : kFormPairs;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
+    double matches = 0;                                   // of comparing holes with classes, by the sample
+    for (size_t i = 0; i < n; ++i)
+        if (sk[i])
+            for (const HoleHost& h : sk[i]->holes)
+                if (h.compares && h.cls_size > 0) for (int k = 1; k <= h.max_size; ++k) matches += h.pass_rate * (double)sk[i]->g->cnt[h.start_nt][k];
+    const bool dense = matches > kClassMatches * queue;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
         if (!s) return fail(XP_ERR_INVALID_ARG, "null sketch in batch");
-        if (!plain) { plan_sketch(s, i, o, form, plan); continue; }
+        if (!plain) { plan_sketch(s, i, o, form, dense, plan); continue; }
         const Plan* own;
         {
             std::lock_guard<std::mutex> lock(s->plan_mu);
-            std::unique_ptr<const Plan>& kept = s->plan_kept[form];
+            std::unique_ptr<const Plan>& kept = s->plan_kept[form + (dense ? 4 : 0)];
             if (!kept) {
                 std::unique_ptr<Plan> made(new Plan);
-                plan_sketch(s, 0, o, form, made.get());
+                plan_sketch(s, 0, o, form, dense, made.get());
                 made->acc.clear();                        // (made per call, below)
                 kept = std::move(made);
             }
@@ -1884,11 +1899,12 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
 }
 
 // One sketch's segments, accumulators and tickets, appended to the plan as sketch number i.
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, Plan* plan) {
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, bool dense, Plan* plan) {
     std::vector<u32> taken;
     {
         for (int h = 0; h < s->n_holes; ++h) {
-            const HoleHost& ho = s->holes[h];
+            HoleHost ho = s->holes[h];
+            if (dense && ho.compares && ho.pass_rate > 0) ho.cls_size = 0;
             AccDev a;
             memset(&a, 0, sizeof(a));
             for (int k = 0; k <= kMaxSize; ++k) a.min_rank[k] = ~0ull;
@@ -2040,7 +2056,7 @@ static void stage_plan(char* stage, char* ws, const SearchLayout& w, Plan& plan,
 extern "C" size_t xp_workspace_bytes(const xp_sketch* const* sketches, size_t n, const xp_repair_opts* opts) {
     if (!sketches || n == 0) return 0;
     Plan plan;
-    if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, true, &plan) != XP_OK) return 0;
+    if (build_plan(sketches, n, opts ? opts : &kDefaultOpts, true, kSurvMost, &plan) != XP_OK) return 0;
     return ws_layout(plan, sketches, n, kSurvMost).total;
 }
 
@@ -2053,7 +2069,7 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
     if (o->cancel && *o->cancel) return fail(XP_ERR_CANCELLED, "cancelled before launch");
     const auto t0 = std::chrono::steady_clock::now();
     Plan plan;
-    xp_status st = build_plan(sketches, n, o, true, &plan);
+    xp_status st = build_plan(sketches, n, o, true, kSurvMost, &plan);
     if (st == XP_OK) st = check_device(sketches, n);
     if (st != XP_OK) return st;
     cudaStream_t stream = (cudaStream_t)o->stream;
@@ -2071,7 +2087,7 @@ extern "C" xp_status xp_repair_batch(const xp_sketch* const* sketches, size_t n,
         // A refinement can change which blocks the pair join may take (a target that is no longer zero), and so what a call
         // needs: a caller's workspace made before it holds the plan without the pair join.
         plan = Plan();
-        st = build_plan(sketches, n, o, false, &plan);
+        st = build_plan(sketches, n, o, false, kSurvMost, &plan);
         if (st != XP_OK) return st;
         w = ws_layout(plan, sketches, n, kSurvMost);
         shrink();
@@ -2222,7 +2238,7 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
     if (o->n_rank_ranges < 0 || (o->n_rank_ranges > 0 && !o->rank_ranges)) return fail(XP_ERR_INVALID_ARG, "bad rank_ranges");
     if (o->cancel && *o->cancel) return fail(XP_ERR_CANCELLED, "cancelled before launch");
     Plan plan;
-    xp_status st = build_plan(&sketch, 1, o, false, &plan);
+    xp_status st = build_plan(&sketch, 1, o, false, kSurvCapStatic, &plan);
     if (st == XP_OK) st = check_device(&sketch, 1);
     if (st != XP_OK) return st;
     const SearchLayout w = ws_layout(plan, &sketch, 1, kSurvCapStatic);

@@ -147,7 +147,7 @@ struct HoleDev {
     // second: filter hits are also checked exactly at probe 1 before they are queued (needs tables, a
     // defined spec and an affine context at probe 1); sample_pass0: how many of the sample_n small
     // candidates sampled at load satisfied probe 0 (a high rate makes the second look worth its cost).
-    i32 second, sample_pass0, sample_n, pad4;
+    i32 second, sample_pass0, sample_n, sample_pass;      // sample_pass: how many of them satisfied every probe that has tables
     i32 second_ok;                                // the second look is possible (tables, spec and context at probe 1): a
                                                   // CTA that sees many filter hits for this hole turns it on for itself
     // Set by the host before the load's kernels run: the largest subtree size and the number of
@@ -221,7 +221,7 @@ struct LoadJob { SketchDev* s; i32 hole, pad; };
 struct LoadCopy { char* dst; u64 src, bytes; };
 
 // What the load's kernels settled for a hole, as the host reads it back.
-struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe, tab_max, target_zero; u32 spec_bad; i32 cls_size; u32 cls_n[kMaxNt]; };
+struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe, tab_max, target_zero, sample_pass, sample_n; u32 spec_bad; i32 cls_size; u32 cls_n[kMaxNt]; };
 
 // Per (sketch, hole) accumulators, zeroed (min_rank to all-ones) by the host before the launch.
 struct AccDev {

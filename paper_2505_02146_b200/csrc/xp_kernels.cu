@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
 #pragma unroll
         for (int w = 0; w < kPrepWords; ++w) alive[w] = ncand ? 0xffffffffu : 0u;
         u64 chosen = 0;
-        int n = 0, pass0 = 0, first = 0;
+        int n = 0, pass0 = 0, pass = 0, first = 0;
         u32 spec_ok = 0;
 #pragma unroll 1
         for (; n < kMaxProbe && n < ns; ++n) {
@@ -463,6 +463,11 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
             if (s_ok[best]) spec_ok |= 1u << n;
 #pragma unroll
             for (int w = 0; w < kPrepWords; ++w) alive[w] &= s_mask[best][w];
+            if (n < hole->tab_probes_cap) {
+                pass = 0;
+#pragma unroll
+                for (int w = 0; w < kPrepWords; ++w) pass += __popc(alive[w]);
+            }
             if (lane == 0) { hole->probe_id[n] = s->sample_id[best]; hole->probe_spec[n] = s_spec[best]; }
             if (lane < nv) hole->probe_pt[n][lane] = s_pt[best][lane];
         }
@@ -486,6 +491,7 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
         if (lane == 0) {
             hole->n_probe = n;
             hole->probe_spec_ok = spec_ok;
+            hole->sample_pass = pass;
             hole->sample_pass0 = pass0;                   // sampled candidates that satisfy the first probe chosen
             hole->sample_n = ncand;
             s_n = n; s_pass0 = pass0;
@@ -495,7 +501,7 @@ __global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const LoadJob* jo
     probe_contexts(g, hole, s_n, ncand, s_pass0);
     if (t == 0)                                         // (thread 0 has written all of these itself)
         out[blockIdx.x] = LoadOut{hole->filter_ok, hole->tab_probes, hole->aff_ok, hole->join_on, hole->second, hole->n_probe, hole->tab_max_size,
-                                  hole->join_t0 == 0 || hole->join_t1 == 0 ? 1 : 0, hole->spec_bad, 0, {0}};
+                                  hole->join_t0 == 0 || hole->join_t1 == 0 ? 1 : 0, hole->sample_pass, hole->sample_n, hole->spec_bad, 0, {0}};
 }
 
 // The probes of a hole replaced by the host (xp_sketch_refine: points that ended whole-domain

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
-from tests.util import check_sketch
+from tests.util import assert_same, check_sketch
 from xp_instances import Hole, Sketch, Variable, constant_set, free_grammar, parse_expr, quasi_affine_grammar
 
 pytestmark = pytest.mark.gpu
@@ -118,3 +118,24 @@ def test_matches_in_large_classes(xp):
     few = _large("((i*7)+j)*3")                          # (a launch takes 8192 pieces of 64 members; here there are none)
     few = xp.xp_repair(xp.xp_sketch_load(gr, few), timeout_ms=60_000, **only7)[0]
     assert bounded.n_launches >= few.n_launches + 3
+
+
+def test_guards_that_nearly_always_hold(xp):
+    """Where most candidates match, operands do not go by class: 1.7e7 matches, each operand met for itself."""
+    g = free_grammar(VS, constant_set(1, 68))
+    sk = Sketch(g, [Hole(0, 5, ctx=parse_expr("(0-HOLE)<1000000", VS), spec_expr=parse_expr("0<1", VS))])
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
+    r = xp.xp_repair(ls)[0]
+    n = r.cand_count
+    assert n[3] > 4096 and sum(n) > 2**24                # (enough for classes, and for 2^24 matches)
+    undefined = 0                                        # quotients and remainders with a divisor that is 0 somewhere
+    few = 200_000
+    for begin in (0, n[5] // 2, n[5] - few):
+        w = {1: (0, 0), 3: (0, 0), 5: (begin, begin + few)}
+        want = oracle.repair_hole(sk, 0, rank_ranges=w)
+        got = xp.xp_repair(ls, size_min=5, size_max=5, rank_ranges=[(0, 5, *w[5])])[0]
+        assert got.match_count[5] == want.match_count[5]
+        undefined += few - want.match_count[5]
+    match, least = _cut(xp, ls, 5, n[5], 7)
+    assert r.match_count[5] == match and match > 0.9 * n[5]
+    assert r.filter_tests > 0.8 * n[3] * 10 * 3          # every operand, five operators on either side, the constants and two variables
