@@ -482,9 +482,10 @@ struct HoleHost {
     int cls_size = 0;                // operands of this size are in classes, cls_n of each nonterminal (0: none)
     u32 cls_n[kMaxNt] = {0};
     double pass_rate = 0;            // share of the load's sampled candidates that satisfied every probe with tables
-    // What the load makes classes of: the size, and for which contexts (0: none); a grammar's subtrees of that size, and of one nonterminal at most.
+    // What the load makes classes of: the size, and for which contexts (0: none); a grammar's subtrees of that size.
     int cls_top = 0, cls_want = 0;
-    u64 cls_entries = 0, cls_most = 0;
+    u64 cls_entries = 0;
+    u32 cls_blocks = 0;              // blocks of the kernels that make them
 };
 
 struct Plan {
@@ -604,14 +605,14 @@ static void class_plan(const xp_grammar* g, const xp_hole_desc& hd, HoleHost* h)
         for (int k = 1; k <= hd.max_size - 2; ++k)
             if (g->cnt[nt][k] > 0) { need = k > need ? k : need; if (k <= tmax) top = k > top ? k : top; }
     if (top < 3) return;
-    u64 all = 0, most = 0;
-    for (int nt = 0; nt < g->n_nt; ++nt) { const u64 c = g->cnt[nt][top]; all += c; most = c > most ? c : most; }
+    u64 all = 0, blocks = 0;
+    for (int nt = 0; nt < g->n_nt; ++nt) { all += g->cnt[nt][top]; blocks += (g->cnt[nt][top] + kClassThreads - 1) / kClassThreads; }
     if (all < kClassLeast) return;
     bool compares = false;
     for (int i = 0; i < hd.ctx_len; ++i) compares = compares || (hd.ctx[i].kind == XP_I_OP && (hd.ctx[i].arg == XP_OP_LT || hd.ctx[i].arg == XP_OP_LE));
     compares = compares && g->cnt[hd.start_nt][top] <= kRangeMost;       // (with more, such a context's operands go as tiles)
     h->cls_want = (need > top ? kClassAffine : 0) | (compares ? kClassCompare : 0);
-    if (h->cls_want) { h->cls_top = top; h->cls_entries = all; h->cls_most = most; }
+    if (h->cls_want) { h->cls_top = top; h->cls_entries = all; h->cls_blocks = (u32)blocks; }
 }
 
 // One sketch on its way through a load: everything between its description and the moment the
@@ -991,18 +992,44 @@ static cudaError_t make_tables(const LoadJob* jobs, int n_jobs, int size_cap, in
     return e;
 }
 
-// The classes of the holes of a sketch that are to have them, one hole after the other in the same scratch.
-static size_t classes_scratch(const xp_sketch* s) {
-    size_t most = 0;
-    for (const HoleHost& h : s->holes) { const size_t b = class_scratch_bytes(h.cls_entries); most = b > most ? b : most; }
-    return most;
-}
-static cudaError_t make_classes(const xp_sketch* s, char* scratch, LoadOut* out) {
-    cudaError_t e = cudaSuccess;
-    for (int h = 0; h < s->n_holes && e == cudaSuccess; ++h)
-        if (s->holes[h].cls_entries > 0) e = launch_classes(s->d_s, h, scratch, s->holes[h].cls_entries, s->holes[h].cls_most, s->g->n_nt, out ? out + h : nullptr, nullptr);
-    return e;
-}
+// The classes of all holes of a load (or a refinement) that are to have them: groups of holes that share the scratch, a launch of each kernel for
+// a group.  A group's scratch: the tables of its holes, then where their subtrees belong.
+struct ClassGroup { size_t first, n, tables, bytes; u32 blocks; };
+constexpr size_t kClassScratch = 256ull << 20;            // scratch up to which holes share a group (1000 guards of 29 leaves: 165 MB)
+struct ClassPlan {
+    std::vector<ClassJob> jobs;                           // tables and places as offsets from the start of the scratch
+    std::vector<ClassGroup> groups;
+    size_t scratch = 0;                                   // of the largest group
+    void add(const xp_sketch* s, int hole, LoadOut* out) {
+        const HoleHost& h = s->holes[hole];
+        if (h.cls_entries == 0) return;
+        const size_t table = class_table_bytes(h.cls_entries), place = class_place_bytes(h.cls_entries);
+        if (groups.empty() || groups.back().bytes + table + place > kClassScratch || (u64)groups.back().blocks + h.cls_blocks >= 1ull << 30)
+            groups.push_back(ClassGroup{jobs.size(), 0, 0, 0, 0u});
+        ClassGroup& g = groups.back();
+        ClassJob j;
+        j.s = s->d_s; j.hole = hole; j.first_block = g.blocks; j.out = out; j.pad = 0;
+        j.table = (u64*)g.tables; j.at = (uint2*)(g.bytes - g.tables);
+        j.mask = class_slots(h.cls_entries) - 1u;
+        jobs.push_back(j);
+        ++g.n; g.tables += table; g.bytes += table + place; g.blocks += h.cls_blocks;
+        scratch = g.bytes > scratch ? g.bytes : scratch;
+    }
+    // The jobs as the kernels read them, and their launches (jobs_dev: where the host's copy of them goes).
+    void place(char* base) {
+        for (const ClassGroup& g : groups)
+            for (size_t i = g.first; i < g.first + g.n; ++i) {
+                jobs[i].table = (u64*)(base + (size_t)jobs[i].table);
+                jobs[i].at = (uint2*)(base + g.tables + (size_t)jobs[i].at);
+            }
+    }
+    cudaError_t launch(const ClassJob* jobs_dev, char* base) const {
+        cudaError_t e = cudaSuccess;
+        for (size_t i = 0; i < groups.size() && e == cudaSuccess; ++i)
+            e = launch_classes(jobs_dev + groups[i].first, (int)groups[i].n, jobs[groups[i].first], groups[i].blocks, base, groups[i].tables, nullptr);
+        return e;
+    }
+};
 
 // Loads of several threads run side by side (their kernels follow one another on the default stream).  A grammar's tables are sent by
 // the first load that needs them, and others may queue kernels that read them once that copy has been queued: a load takes the
@@ -1091,7 +1118,9 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     for (size_t i = 0; i < n; ++i) copies.push_back(LoadCopy{st[i].s->arena, 0, st[i].head});
     for (size_t i = 0; i < n; ++i) if (st[i].grammar_fresh) copies.push_back(LoadCopy{(char*)st[i].s->g->d_g, 0, st[i].grammar_bytes});
     const size_t at_list = 0, at_jobs = at_list + al256(sizeof(SketchDev*) * n), at_copies = at_jobs + al256(sizeof(LoadJob) * n_jobs);
-    const size_t at_shares = at_copies + al256(sizeof(LoadCopy) * copies.size());
+    ClassPlan cls;
+    for (size_t i = 0; i < n; ++i) for (int h = 0; h < st[i].s->n_holes; ++h) cls.add(st[i].s, h, nullptr);
+    const size_t at_cls = at_copies + al256(sizeof(LoadCopy) * copies.size()), at_shares = at_cls + al256(sizeof(ClassJob) * cls.jobs.size());
     std::vector<size_t> piece_at;                         // start of each piece; the lists are in the first
     size_t at = at_shares;
     piece_at.push_back(0);
@@ -1109,9 +1138,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
     const bool put = n == 1 && staged <= kPutMost;        // (a small sketch alone: straight to its places, without copy and scatter)
     const size_t at_out = al256(staged), at_scratch = at_out + al256(sizeof(LoadOut) * n_jobs);
     const size_t at_classes = at_scratch + al256(prepare_scratch_bytes((int)(n_jobs < kJobs ? n_jobs : kJobs)));
-    size_t class_bytes = 0;
-    for (size_t i = 0; i < n; ++i) { const size_t b = classes_scratch(st[i].s); class_bytes = b > class_bytes ? b : class_bytes; }
-    size_t total = at_classes + class_bytes;
+    size_t class_bytes = cls.scratch, total = at_classes + class_bytes;
     cudaError_t got = pool_alloc((void**)&dev_block, total, &dev_device, &dev_bytes);
     if (got != cudaSuccess && class_bytes > 0) {          // (memory is short: without classes)
         (void)cudaGetLastError();
@@ -1142,6 +1169,12 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
                 for (int h = 0; h < st[i].s->n_holes; ++h, ++j) ((LoadJob*)(lists + at_jobs))[j] = LoadJob{st[i].s->d_s, h, 0};
             }
             memcpy(lists + at_copies, copies.data(), sizeof(LoadCopy) * copies.size());
+            // (what the classes come to goes straight to page-locked memory like the rest of LoadOut)
+            LoadOut* out = (LoadOut*)(back.locked ? back.p : dev_block + at_out);
+            cls.place(dev_block + at_classes);
+            for (size_t i = 0, c = 0; i < n; out += st[i].s->n_holes, ++i)
+                for (int h = 0; h < st[i].s->n_holes; ++h) if (st[i].s->holes[h].cls_entries > 0) cls.jobs[c++].out = out + h;
+            memcpy(lists + at_cls, cls.jobs.data(), sizeof(ClassJob) * cls.jobs.size());
             // large batches fill their pieces with a few threads; whoever finishes a piece's last share sends the piece
             size_t n_threads = staged / (1u << 20) < n / 8 ? staged / (1u << 20) : n / 8;      // (starting a thread takes as long as filling some 300 KB)
             const unsigned hw = std::thread::hardware_concurrency();
@@ -1201,6 +1234,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
             const size_t np = (size_t)s->n_points, row = (size_t)(s->g->n_vars ? s->g->n_vars : 1);
             const size_t coords_bytes = sizeof(i32) * np * row, spec_bytes = sizeof(i64) * np;
             s->load_h2d = L.head + L.grammar_bytes + sizeof(SketchDev*) + sizeof(LoadJob) * (size_t)s->n_holes + sizeof(LoadCopy) * (L.grammar_fresh ? 2 : 1);
+            for (const HoleHost& hh : s->holes) if (hh.cls_entries > 0) s->load_h2d += sizeof(ClassJob);
             s->load_d2h = sizeof(LoadOut) * (size_t)s->n_holes;
             if (L.copy_coords && coords_bytes > kPackMax) {
                 XP_CUDA_B(cudaMemcpyAsync(s->arena + L.off_coords, L.d->coords, coords_bytes, cudaMemcpyHostToDevice, nullptr));
@@ -1223,7 +1257,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         // The load's kernels, in stream order, one launch of each for the whole batch: points of the boxes and values of
         // spec expressions (so that the whole-domain check, and the probe choice, read tables for every kind of domain);
         // bounds of the tables' coordinates; the probe choice; the subtree tables, bottom-up, for as many sizes and probes
-        // as there can be (blocks beyond what the probe choice settled on for their hole return at once).
+        // as there can be (blocks beyond what the probe choice settled on for their hole return at once); the operand classes.
         // Grids are cut into pieces of at most kJobs jobs (a grid dimension holds 65 535).
         SketchDev* const* d_list = (SketchDev* const*)(dev_block + at_list);
         const LoadJob* d_jobs = (const LoadJob*)(dev_block + at_jobs);
@@ -1240,10 +1274,7 @@ extern "C" xp_status xp_sketch_load_batch(const xp_grammar* const* grammars, con
         }
         for (size_t q = 0; q < n_jobs; q += kJobs)
             XP_CUDA_B(make_tables(d_jobs + q, (int)(n_jobs - q < kJobs ? n_jobs - q : kJobs), size_cap, probes_cap, most_entries));
-        if (class_bytes > 0) {
-            LoadOut* out = (LoadOut*)(back.locked ? back.p : dev_block + at_out);
-            for (size_t i = 0; i < n; out += st[i].s->n_holes, ++i) XP_CUDA_B(make_classes(st[i].s, dev_block + at_classes, out));
-        }
+        if (class_bytes > 0) XP_CUDA_B(cls.launch((const ClassJob*)(dev_block + at_cls), dev_block + at_classes));
         if (!back.locked) XP_CUDA_B(cudaMemcpyAsync(back.p, dev_block + at_out, sizeof(LoadOut) * n_jobs, cudaMemcpyDeviceToHost, nullptr));
         XP_CUDA_B(cudaStreamSynchronize(nullptr));
     }
@@ -1362,8 +1393,10 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         char* jobs_dev = nullptr;
         size_t jobs_bytes = 0;
         int jobs_device = 0;
-        const size_t at_classes = al256(sizeof(LoadJob) * jobs.size());
-        size_t class_bytes = classes_scratch(s);
+        ClassPlan cls;
+        for (int h = 0; h < nh; ++h) cls.add(s, h, nullptr);
+        const size_t at_cls = al256(sizeof(LoadJob) * jobs.size()), at_classes = at_cls + al256(sizeof(ClassJob) * cls.jobs.size());
+        size_t class_bytes = cls.scratch;
         cudaError_t got = pool_alloc((void**)&jobs_dev, at_classes + class_bytes, &jobs_device, &jobs_bytes);
         if (got != cudaSuccess && class_bytes > 0) {      // (memory is short: without classes from here on)
             (void)cudaGetLastError();
@@ -1374,9 +1407,11 @@ extern "C" xp_status xp_sketch_refine(xp_sketch* s, int32_t max_promote, int32_t
         for (HoleDev& o : hh) { memset(o.cls_count, 0, sizeof(o.cls_count)); o.cls_size = 0; }      // (holes without a promoted point are numbered again too)
         cudaError_t e = cudaMemcpyAsync(s->arena + s->off_holes, hh.data(), sizeof(HoleDev) * nh, cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(LoadJob) * jobs.size(), cudaMemcpyHostToDevice, nullptr);
+        cls.place(jobs_dev + at_classes);
+        if (e == cudaSuccess && class_bytes > 0) e = cudaMemcpyAsync(jobs_dev + at_cls, cls.jobs.data(), sizeof(ClassJob) * cls.jobs.size(), cudaMemcpyHostToDevice, nullptr);
         if (e == cudaSuccess) e = launch_reprobe((const LoadJob*)jobs_dev, (int)jobs.size(), nullptr);
         if (e == cudaSuccess) e = make_tables((const LoadJob*)jobs_dev, (int)jobs.size(), s->tab_size_cap, s->tab_probes_cap, s->entries_at);
-        if (e == cudaSuccess && class_bytes > 0) e = make_classes(s, jobs_dev + at_classes, nullptr);
+        if (e == cudaSuccess && class_bytes > 0) e = cls.launch((const ClassJob*)(jobs_dev + at_cls), jobs_dev + at_classes);
         if (e == cudaSuccess) e = cudaMemcpyAsync(hh.data(), s->arena + s->off_holes, sizeof(HoleDev) * nh, cudaMemcpyDeviceToHost, nullptr);
         const cudaError_t e2 = cudaStreamSynchronize(nullptr);
         pool_release(jobs_dev, jobs_bytes, jobs_device);

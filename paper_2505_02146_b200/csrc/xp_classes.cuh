@@ -10,6 +10,7 @@
 //   class_number_kernel  -- the member counted first numbers its class and takes the members' places, in the order of the subtrees
 //                           (a scan per block, one atomic per block);
 //   class_member_kernel  -- every member to its place.
+// One launch of each for all holes of a load (a block finds its job by its number: hole by hole, 1000 guards of 29 leaves took 35 ms of a load, now 2.8).
 // Bound by the latency of the table and of the values in L2: 45 us for either example, of a load.  The leaf join of the first search (2.1e11
 // candidates) went from 1.93 to 0.14 ms, whole calls of six inputs from 2.95 to 1.05 ms on average; the second (3.2e11) from 6.3 to 2.0 ms,
 // and from 14.4 to 6.8 on inputs with millions of suspects.  (Classes by the two join probes alone would be half as many in the second
@@ -18,15 +19,6 @@
 
 namespace xp {
 
-constexpr int kClassThreads = 256;
-struct ClassJob {
-    SketchDev* s;
-    i32 hole, pad;
-    u64* table;                      // mask + 1 words, zero at launch: members << 32 | first subtree + 1, then members << 32 | first place
-    u32 mask;
-    uint2* at;                       // per subtree: slot and number among the members (kClassNone: in no class)
-    LoadOut* out;                    // null: a refinement, the host reads the hole's record
-};
 constexpr u32 kClassNone = 0xffffffffu;
 
 __device__ __forceinline__ bool class_wanted(const HoleDev* hole) {
@@ -36,14 +28,35 @@ __device__ __forceinline__ bool class_wanted(const HoleDev* hole) {
     return hole->aff_ok ? (hole->cls_want & kClassAffine) && hole->join_on : (hole->cls_want & kClassCompare) != 0;
 }
 
-__global__ void __launch_bounds__(kClassThreads) class_insert_kernel(const __grid_constant__ ClassJob job) {
+// The job of this block, and of its nonterminals the one whose subtrees [first, first + kClassThreads) the block has.
+struct ClassPart { ClassJob job; u32 first; i32 nt; };
+__device__ __forceinline__ ClassPart class_part(const ClassJob* jobs, int n_jobs, const ClassJob& only) {
+    int lo = 0;
+    for (int hi = n_jobs; hi - lo > 1;) { const int mid = (lo + hi) >> 1; if (jobs[mid].first_block <= blockIdx.x) lo = mid; else hi = mid; }
+    ClassPart p;
+    p.job = n_jobs == 1 ? only : jobs[lo];             // (one hole: it comes with the launch)
+    const GrammarDev* g = p.job.s->g;
+    const int top = p.job.s->holes[p.job.hole].cls_top;
+    u32 block = blockIdx.x - p.job.first_block;
+    for (p.nt = 0; p.nt + 1 < g->n_nt; ++p.nt) {
+        const u32 here = ((u32)g->cnt[p.nt][top] + kClassThreads - 1) / kClassThreads;
+        if (block < here) break;
+        block -= here;
+    }
+    p.first = block * kClassThreads;
+    return p;
+}
+
+__global__ void __launch_bounds__(kClassThreads) class_insert_kernel(const ClassJob* jobs, int n_jobs, const __grid_constant__ ClassJob only) {
     chain_wait();
+    const ClassPart part = class_part(jobs, n_jobs, only);
+    const ClassJob& job = part.job;
     const HoleDev* hole = &job.s->holes[job.hole];
     if (!class_wanted(hole)) return;
-    const int nt = blockIdx.y, top = hole->cls_top, np = hole->n_exact;
+    const int nt = part.nt, top = hole->cls_top, np = hole->n_exact;
     const u64 first = hole->tab_off[0][top], base = hole->tab_off[nt][top], total = hole->tab_total;
-    const u32 count = (u32)job.s->g->cnt[nt][top], i = blockIdx.x * kClassThreads + threadIdx.x;
-    if (blockIdx.x * kClassThreads >= count) return;
+    const u32 count = (u32)job.s->g->cnt[nt][top], i = part.first + threadIdx.x;
+    if (part.first >= count) return;
     const i64* val = hole->tab_val + base;
     const unsigned char* def = hole->tab_ok + base;
     bool on = i < count;
@@ -77,17 +90,19 @@ __global__ void __launch_bounds__(kClassThreads) class_insert_kernel(const __gri
     if (i < count) job.at[(u32)(base - first) + i] = make_uint2(slot, (u32)(old >> 32) + (u32)__popc(same & ((1u << lane) - 1u)));
 }
 
-__global__ void __launch_bounds__(kClassThreads) class_number_kernel(const __grid_constant__ ClassJob job) {
+__global__ void __launch_bounds__(kClassThreads) class_number_kernel(const ClassJob* jobs, int n_jobs, const __grid_constant__ ClassJob only) {
     chain_wait();
     __shared__ u32 s_classes[kClassThreads / 32], s_members[kClassThreads / 32];
     __shared__ u64 s_base;
+    const ClassPart part = class_part(jobs, n_jobs, only);
+    const ClassJob& job = part.job;
     HoleDev* hole = &job.s->holes[job.hole];
     if (!class_wanted(hole)) return;
-    const int nt = blockIdx.y, top = hole->cls_top, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nt = part.nt, top = hole->cls_top, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const u64 base = hole->tab_off[nt][top];
     const u32 off = (u32)(base - hole->tab_off[0][top]);
-    const u32 count = (u32)job.s->g->cnt[nt][top], i = blockIdx.x * kClassThreads + threadIdx.x;
-    if (blockIdx.x * kClassThreads >= count) return;
+    const u32 count = (u32)job.s->g->cnt[nt][top], i = part.first + threadIdx.x;
+    if (part.first >= count) return;
     const uint2 at = i < count ? job.at[off + i] : make_uint2(kClassNone, 0u);
     const bool first = at.x != kClassNone && at.y == 0u;
     const u32 n = first ? (u32)(job.table[at.x] >> 32) : 0u, mine = __ballot_sync(0xffffffffu, first);
@@ -109,13 +124,16 @@ __global__ void __launch_bounds__(kClassThreads) class_number_kernel(const __gri
     job.table[at.x] = ((u64)n << 32) | place;
 }
 
-__global__ void __launch_bounds__(kClassThreads) class_member_kernel(const __grid_constant__ ClassJob job) {
+__global__ void __launch_bounds__(kClassThreads) class_member_kernel(const ClassJob* jobs, int n_jobs, const __grid_constant__ ClassJob only) {
     chain_wait();
+    const ClassPart part = class_part(jobs, n_jobs, only);
+    const ClassJob& job = part.job;
     HoleDev* hole = &job.s->holes[job.hole];
-    const int nt = blockIdx.y;
     const bool wanted = class_wanted(hole);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const int top = hole->cls_top;
+    const int top = hole->cls_top;
+    const GrammarDev* g = job.s->g;
+    if (blockIdx.x == job.first_block && (int)threadIdx.x < g->n_nt) {
+        const int nt = (int)threadIdx.x;
         const u32 n = wanted ? (u32)hole->cls_count[nt] : 0u;
         hole->cls_n[nt] = n;
         if (wanted) hole->cls_start[(u32)(hole->tab_off[nt][top] - hole->tab_off[0][top]) + (u32)nt + n] = (u32)(hole->cls_count[nt] >> 32);
@@ -123,8 +141,8 @@ __global__ void __launch_bounds__(kClassThreads) class_member_kernel(const __gri
         if (job.out) { job.out->cls_n[nt] = n; if (nt == 0) job.out->cls_size = wanted ? top : 0; }
     }
     if (!wanted) return;
-    const u32 off = (u32)(hole->tab_off[nt][hole->cls_top] - hole->tab_off[0][hole->cls_top]);
-    const u32 count = (u32)job.s->g->cnt[nt][hole->cls_top], i = blockIdx.x * kClassThreads + threadIdx.x;
+    const u32 off = (u32)(hole->tab_off[part.nt][top] - hole->tab_off[0][top]);
+    const u32 count = (u32)g->cnt[part.nt][top], i = part.first + threadIdx.x;
     if (i >= count) return;
     const uint2 at = job.at[off + i];
     if (at.x != kClassNone) hole->cls_mem[off + (u32)job.table[at.x] + at.y] = i;

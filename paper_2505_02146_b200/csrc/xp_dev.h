@@ -223,6 +223,17 @@ struct LoadCopy { char* dst; u64 src, bytes; };
 // What the load's kernels settled for a hole, as the host reads it back.
 struct LoadOut { i32 filter_ok, tab_probes, aff_ok, join_on, second, n_probe, tab_max, target_zero, sample_pass, sample_n; u32 spec_bad; i32 cls_size; u32 cls_n[kMaxNt]; };
 
+// One hole whose operands are put into classes (csrc/xp_classes.cuh).
+struct ClassJob {
+    SketchDev* s;
+    i32 hole;
+    u32 first_block;                 // blocks of the jobs before it
+    u64* table;                      // mask + 1 words, zero at launch: members << 32 | first subtree + 1, then members << 32 | first place
+    uint2* at;                       // per subtree: slot and number among the members (kClassNone: in no class)
+    LoadOut* out;                    // null: a refinement, the host reads the hole's record
+    u32 mask, pad;
+};
+
 // Per (sketch, hole) accumulators, zeroed (min_rank to all-ones) by the host before the launch.
 struct AccDev {
     u64 match_count[kMaxSize + 1];

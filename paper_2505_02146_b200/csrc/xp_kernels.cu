@@ -3270,18 +3270,13 @@ cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last
     return cudaGetLastError();
 }
 
-// The classes of one hole, `entries` subtrees of the size in question over n_nt nonterminals (most: of one of them).
-cudaError_t launch_classes(SketchDev* s, int hole, char* scratch, u64 entries, u64 most, int n_nt, LoadOut* out, cudaStream_t stream) {
-    ClassJob job;
-    const u32 slots = class_slots(entries);
-    job.s = s; job.hole = hole; job.pad = 0; job.out = out;
-    job.table = (u64*)scratch; job.mask = slots - 1u; job.at = (uint2*)(scratch + sizeof(u64) * (size_t)slots);
-    const cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(u64) * (size_t)slots, stream);
+cudaError_t launch_classes(const ClassJob* jobs, int n_jobs, const ClassJob& first, u32 blocks, char* scratch, size_t tables, cudaStream_t stream) {
+    if (n_jobs <= 0) return cudaSuccess;
+    const cudaError_t e = cudaMemsetAsync(scratch, 0, tables, stream);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((most + kClassThreads - 1) / kClassThreads), (unsigned)n_nt);
-    chain(class_insert_kernel, grid, kClassThreads, 0, stream, job);
-    chain(class_number_kernel, grid, kClassThreads, 0, stream, job);
-    chain(class_member_kernel, grid, kClassThreads, 0, stream, job);
+    chain(class_insert_kernel, blocks, kClassThreads, 0, stream, jobs, n_jobs, first);
+    chain(class_number_kernel, blocks, kClassThreads, 0, stream, jobs, n_jobs, first);
+    chain(class_member_kernel, blocks, kClassThreads, 0, stream, jobs, n_jobs, first);
     return cudaGetLastError();
 }
 

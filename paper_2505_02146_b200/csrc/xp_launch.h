@@ -41,10 +41,12 @@ cudaError_t launch_put(const PutPlaces& to, const char* src, cudaStream_t stream
 cudaError_t launch_reprobe(const LoadJob* jobs, int n_jobs, cudaStream_t stream);
 cudaError_t launch_coord_bounds(SketchDev* const* list, int n_sketches, i64 most_points, cudaStream_t stream);
 cudaError_t launch_subvalues(const LoadJob* jobs, int n_jobs, int size, int last, int most_probes, u64 most_entries, cudaStream_t stream);
-// Operand classes of one hole (csrc/xp_classes.cuh); scratch: class_scratch_bytes(entries), 256-byte aligned.
+// Operand classes (csrc/xp_classes.cuh) of `n_jobs` holes at once (first: the first of them), `blocks` blocks in all; tables: what lies at the start of `scratch` and is zeroed.
 inline u32 class_slots(u64 entries) { u32 n = 1024; while (n < 2 * entries) n <<= 1; return n; }
-inline size_t class_scratch_bytes(u64 entries) { return entries ? sizeof(u64) * ((size_t)class_slots(entries) + (size_t)entries) : 0; }
-cudaError_t launch_classes(SketchDev* s, int hole, char* scratch, u64 entries, u64 most, int n_nt, LoadOut* out, cudaStream_t stream);
+inline size_t class_table_bytes(u64 entries) { return sizeof(u64) * (size_t)class_slots(entries); }
+inline size_t class_place_bytes(u64 entries) { return sizeof(uint2) * (size_t)entries; }
+constexpr int kClassThreads = 256;
+cudaError_t launch_classes(const ClassJob* jobs, int n_jobs, const ClassJob& first, u32 blocks, char* scratch, size_t tables, cudaStream_t stream);
 // Layout of one call's device scratch (byte offsets from its 256-byte aligned base):
 //   0: eval ticket (u64), 8: verify ticket (u64), 16: survivor pushes (u32), 20: failed-check word (u32; checked
 //      build only), 24: long survivors (u32), 32: join ticket (u64), 40: finished verification CTAs (u32), 48: listed members

@@ -139,3 +139,49 @@ def test_guards_that_nearly_always_hold(xp):
     match, least = _cut(xp, ls, 5, n[5], 7)
     assert r.match_count[5] == match and match > 0.9 * n[5]
     assert r.filter_tests > 0.8 * n[3] * 10 * 3          # every operand, five operators on either side, the constants and two variables
+
+
+def test_classes_of_many_holes_in_one_load(xp):
+    """Sketches with one, two and no holes with classes, of several grammars, in one load: as if loaded one by one, and as the oracle has it."""
+    sks = []
+    for q in range(12):
+        consts = constant_set(-13, 13 + 2 * (q % 4)) if q % 3 else constant_set(-4, 4)
+        g = free_grammar(VS, consts, ops=["+", "-", "*", "/", "%"][:5 - q % 2 * (q % 3 == 0)])
+        holes = [Hole(0, 5, ctx=parse_expr("i<HOLE", VS), spec_expr=parse_expr(f"i<((j*2)+{q - 3})", VS))]
+        if q % 2:
+            holes.append(Hole(0, 5, ctx=parse_expr("(j-HOLE)<2", VS), spec_expr=parse_expr(f"(j-(i/{q}))<2", VS)))
+            holes.append(Hole(0, 3, spec_expr=parse_expr("i*2", VS)))
+        sks.append(Sketch(g, holes, name=f"sketch {q}"))
+    vs = [Variable("i", 0, 40), Variable("j", 0, 30)]
+    typed = quasi_affine_grammar(vs, constant_set(-20, 20), list(range(1, 31)))
+    sks.append(Sketch(typed, [Hole(0, 7, ctx=parse_expr("j<HOLE", vs), spec_expr=parse_expr("j<((i/2)+1)", vs))], name="typed"))
+    grs = [xp.xp_grammar_create(s.grammar) for s in sks]
+    many = xp.xp_sketch_load_batch(grs, sks)
+    together = xp.xp_repair_batch(many)
+    for q, sk in enumerate(sks):
+        alone = xp.xp_repair(xp.xp_sketch_load(grs[q], sk))
+        got = xp.xp_repair(many[q])
+        for h in range(len(sk.holes)):
+            if sk.name != "typed":
+                assert_same(alone[h], oracle.repair_hole(sk, h), f"{sk.name} hole {h}")
+            assert_same(got[h], alone[h], f"{sk.name} hole {h}")
+            assert_same(together[q][h], alone[h], f"{sk.name} hole {h} in the batch")
+            assert got[h].filter_tests == alone[h].filter_tests                  # (tests count classes where there are some)
+            if sk.name != "typed" and q % 3 and len(sk.holes[h].ctx):
+                assert got[h].filter_tests < 0.7 * got[h].cand_count[3] * 10 * 3
+
+
+def test_a_thousand_holes_share_a_load(xp):
+    """1100 guards whose classes are made in several groups of launches (their scratch has a bound)."""
+    g = [free_grammar(VS, constant_set(-k, 60 - k)) for k in range(4)]
+    sks = [Sketch(g[q % 4], [Hole(0, 5, ctx=parse_expr("i<HOLE", VS), spec_expr=parse_expr(f"i<((j*{q % 5})-{q % 7})", VS))]) for q in range(1100)]
+    grs = [xp.xp_grammar_create(m) for m in g]
+    ls = xp.xp_sketch_load_batch([grs[q % 4] for q in range(1100)], sks)
+    for q in (0, 1, 333, 700, 1098, 1099):
+        one = xp.xp_repair(xp.xp_sketch_load(grs[q % 4], sks[q]), size_max=3)
+        got = xp.xp_repair(ls[q], size_max=3)
+        assert_same(got[0], one[0])
+        w = [(0, 5, 3_000_000, 4_000_000)]
+        a, b = (xp.xp_repair(s, size_min=5, rank_ranges=w)[0] for s in (ls[q], xp.xp_sketch_load(grs[q % 4], sks[q])))
+        assert_same(a, b)
+        assert a.filter_tests == b.filter_tests
