@@ -496,7 +496,8 @@ struct Plan {
     std::vector<AccDev> acc;
     std::vector<u64> nominal_ops;    // per accumulator: cost-model operations of the filter stage
     u64 n_tickets = 0, n_join = 0;
-    bool join_wide = false;          // several operands per lane and step
+    bool join_wide = false;
+    bool whole = false;              // comparing contexts: every operator in one segment, whatever their number (the fewest bytes)          // several operands per lane and step
 };
 
 struct xp_sketch {
@@ -1488,7 +1489,7 @@ constexpr size_t kPairFew = 2;               // sketches up to which kPairLeast 
 // A rank window cuts a block to some of its left operands, but the other side is indexed whole: a block with fewer rows than this,
 // or thereabouts, is done as tiles before the index is made (450 000 operands a side, remainders: 2 222 rows 0.26 ms, the index 1.9).
 constexpr u64 kPairEach = 1ull << 12;
-constexpr i32 kRangeParts = 4;               // parts of the constants there: a warp checks its suspects by itself, some hundred of them from 32 operands and all
+constexpr int kRangeParts = 4;               // parts of the constants there: a warp checks its suspects by itself, some hundred of them from 32 operands and all
                                              // constants (three conv holes: join 440 us in one part, 350 with 8 operands a ticket, 330 so)
 constexpr u64 kRangeSplit = 1ull << 15;      // ... up to which an operator is a segment of its own (with more there are warps enough at work)
 
@@ -1731,7 +1732,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
             if (!swap) { e0 = wlo / cr; e1 = (whi + cr - 1) / cr; }
             else if (wlo / cr == (whi - 1) / cr) { e0 = wlo % cr; e1 = (whi - 1) % cr + 1; }
             const int slot = slot_of_op(bd.op);
-            const bool shifts = slot >= 7, ex = exact || shifts;      // (how many segments there are does not depend on `exact`)
+            const bool shifts = slot >= 7, ex = exact || shifts;      // (`exact` is the hole's; comparing contexts and classes make further segments below, for few sketches)
             Open* at = nullptr;
             JoinGroup* grp = nullptr;
             for (size_t i = 0; i < open.size() && !at; ++i) {
@@ -1770,8 +1771,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         c.seg.first_group = (i32)plan->jgroups.size();
         c.seg.n_groups = (i32)c.groups.size();
         for (const JoinGroup& q : c.groups) if ((g->wide_leaf >> q.leaf_nt) & 1u) { c.seg.exact = kExactMany; c.seg.heavy = 1; }
-        for (const JoinGroup& q : c.groups) c.seg.leaves += (i32)g->cnt[q.leaf_nt][1];
-        if (c.seg.heavy) c.seg.leaves = 0;                // (these have forms of their own)
+        for (const JoinGroup& q : c.groups) c.seg.chunk += (u32)g->cnt[q.leaf_nt][1];
         // (a rank window may cover fewer operands than there are combinations of classes)
         if (!c.seg.exact && ho.cls_size > 0 && c.seg.esize >= ho.cls_size) {
             const u64 m = class_operands(g, ho, c.seg.nt, c.seg.esize);
@@ -1827,8 +1827,8 @@ static void number_joins(Plan* plan) {
     for (const JoinSeg& c : plan->jsegs) (c.exact ? exact_steps : steps) += (c.e_count + 31) / 32;
     const u64 warps = (u64)search_warps();
     u64 few_pairs = 0, few_steps = 0;
-    auto few = [](const JoinSeg& c) { return c.kind == kJoinLeaf && !c.exact && !c.heavy && !c.classes && c.leaves > 0 && c.e_count * (u64)c.leaves <= kFewPairs; };
-    for (const JoinSeg& c : plan->jsegs) if (few(c)) { few_pairs += c.e_count * (u64)c.leaves; few_steps += (c.e_count + 31) / 32; }
+    auto few = [](const JoinSeg& c) { return c.kind == kJoinLeaf && !c.exact && !c.heavy && !c.classes && c.chunk > 0 && c.e_count * (u64)c.chunk <= kFewPairs; };
+    for (const JoinSeg& c : plan->jsegs) if (few(c)) { few_pairs += c.e_count * (u64)c.chunk; few_steps += (c.e_count + 31) / 32; }
     const u64 share = few_pairs <= kFewCall && few_steps > 0 ? (warps > few_steps ? warps / few_steps : 1) : 0;      // parts, if the leaves are enough
     const i32 form = exact_steps < 2 * warps ? kExactFew : kExactMany;
     u64 per = steps / (warps * 4);
@@ -1839,12 +1839,11 @@ static void number_joins(Plan* plan) {
     for (JoinSeg& c : plan->jsegs) {
         if (c.exact) c.exact = form;
         c.first_ticket = plan->n_join;
-        c.chunk = (u32)(c.exact ? (form == kExactFew ? 1 : 32) : c.parts > 0 ? 32 : per * 32);
         if (share && few(c)) {
-            const u64 most = ((u64)c.leaves + 3) / 4;
+            const u64 most = ((u64)c.chunk + 3) / 4, parts = share < most ? share : most;
             c.chunk = 32;
-            c.parts = (i32)(share < most ? share : most);
-        }
+            c.parts = (int16_t)(parts < 32767u ? parts : 32767u);
+        } else c.chunk = (u32)(c.exact ? (form == kExactFew ? 1 : 32) : c.parts > 0 ? 32 : per * 32);
         plan->n_join += (c.e_count + c.chunk - 1) / c.chunk * (u64)(c.parts > 0 ? c.parts : 1);
     }
 }
@@ -1893,7 +1892,7 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
         if (!s) return fail(XP_ERR_INVALID_ARG, "null sketch in batch");
-        if (!plain) { plan_sketch(s, i, o, form, dense, plan); continue; }
+        if (!plain || plan->whole) { plan_sketch(s, i, o, form, dense, plan); continue; }
         const Plan* own;
         {
             std::lock_guard<std::mutex> lock(s->plan_mu);
@@ -1968,7 +1967,7 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 // candidate that passes those.  40 leaves, size 7, 3.2 million operands, three specs: 210, 1290, 212 ms as tiles, 2270, 4220,
                 // 2400 by the join over classes; with a shift 144, 128 against 1500, 159, with a leaf of 2^33 119, 965 against 64, 807.)
                 const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
-                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, form != kFormMany);
+                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, form != kFormMany && !plan->whole);
                 const bool pairs = form >= kFormPairsSome;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
                 add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany, leaves);
@@ -2276,7 +2275,14 @@ extern "C" xp_status xp_repair_static(const xp_sketch* sketch, const xp_repair_o
     xp_status st = build_plan(&sketch, 1, o, false, kSurvCapStatic, &plan);
     if (st == XP_OK) st = check_device(&sketch, 1);
     if (st != XP_OK) return st;
-    const SearchLayout w = ws_layout(plan, &sketch, 1, kSurvCapStatic);
+    SearchLayout w = ws_layout(plan, &sketch, 1, kSurvCapStatic);
+    if (w.total > kStaticScratchBytes) {                  // (many holes: the plan with the fewest segments)
+        plan = Plan();
+        plan.whole = true;
+        st = build_plan(&sketch, 1, o, false, kSurvCapStatic, &plan);
+        if (st != XP_OK) return st;
+        w = ws_layout(plan, &sketch, 1, kSurvCapStatic);
+    }
     if (plan.acc.size() > 64)
         return fail(XP_ERR_TOO_LARGE, "xp_repair_static: the sketch has more than 64 holes; use xp_repair with a workspace");
     if (w.total > kStaticScratchBytes)

@@ -263,16 +263,17 @@ struct JoinGroup {
 struct JoinSeg {
     u64 first_ticket;
     u64 rank_begin, rank_end;        // window of ranks searched at this size
-    i32 sketch, hole, size, kind;
+    i32 sketch, hole, size;
+    int16_t kind, parts;             // parts > 0: a ticket is 32 operands against one of so many parts of the leaves (join_few, range_ticket)
     i32 acc, nt, esize, n_groups;
     i32 first_group;
     i32 exact;                       // kExactFew, kExactMany: there is no condition (shifts, a leaf of 2^31 or more), every candidate is evaluated on its own
-    u32 chunk;                       // operands per ticket
-    i32 heavy;                       // an operand costs many times the usual (exact form, contexts that compare): these go first
-    i32 leaves, parts;               // leaves of its groups; parts > 0: one ticket is 32 operands against one of so many parts of them (join_few)
-    i32 classes, pad;                // operands are counted by class: e_begin = 0, e_count combinations of classes (class_operands)
+    u32 chunk;                       // operands per ticket (until the tickets are numbered: leaves of its groups)
+    int16_t heavy;                   // an operand costs many times the usual (exact form, contexts that compare): these go first
+    int16_t classes;                 // operands are counted by class: e_begin = 0, e_count combinations of classes (class_operands)
     u64 e_begin, e_count;
 };
+static_assert(sizeof(JoinSeg) == 88, "sketches of many holes just fit the fixed scratch of a call that may not allocate");
 
 // One (left operands, right operands) block of the pair join (csrc/xp_pairs.cuh): every  L op R  of its operators.
 //

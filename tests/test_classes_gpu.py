@@ -185,3 +185,18 @@ def test_a_thousand_holes_share_a_load(xp):
         a, b = (xp.xp_repair(s, size_min=5, rank_ranges=w)[0] for s in (ls[q], xp.xp_sketch_load(grs[q % 4], sks[q])))
         assert_same(a, b)
         assert a.filter_tests == b.filter_tests
+
+
+def test_a_static_call_of_many_comparing_holes(xp):
+    """64 holes whose contexts compare, at three sizes with nine productions: the fixed scratch holds the plan that keeps an
+    operand set's operators together."""
+    g = free_grammar(VS, constant_set(1, 3), ops=["+", "-", "*", "/", "%", "min", "max", "+", "-"])
+    holes = [Hole(0, 7, ctx=parse_expr("i<HOLE", VS), spec_expr=parse_expr(f"i<(({1 + h % 5}+(j*{h % 4}))-{h % 3})", VS)) for h in range(64)]
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), Sketch(g, holes))
+    flag = dict(flags=xp.XP_FLAG_ALWAYS_FILTER)          # (size 3 too)
+    want = xp.xp_repair(ls, **flag)
+    got = xp.xp_repair_static(ls, **flag)
+    for h in range(64):
+        assert list(got[h].match_count)[:8] == want[h].match_count, h
+        assert got[h].solved == want[h].solved and (not want[h].solved or got[h].least_rank == want[h].least_rank)
+    assert any(w.solved for w in want)
