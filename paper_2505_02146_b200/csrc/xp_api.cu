@@ -1775,7 +1775,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         // (a rank window may cover fewer operands than there are combinations of classes)
         if (!c.seg.exact && ho.cls_size > 0 && c.seg.esize >= ho.cls_size) {
             const u64 m = class_operands(g, ho, c.seg.nt, c.seg.esize);
-            if (m > 0 && m < c.seg.e_count) { c.seg.classes = 1; c.seg.e_begin = 0; c.seg.e_count = m; }
+            if (m > 0 && m < c.seg.e_count) { c.seg.classes = 1; c.seg.e_begin = c.seg.e_count; c.seg.e_count = m; }
         }
         // An operand of a context that compares takes some hundred microseconds of a lane, and classes leave a few thousand of them: a
         // segment per operator and side, so that as many warps share them (three conv holes: join 540 -> 430 us).

@@ -270,7 +270,8 @@ struct JoinSeg {
     i32 exact;                       // kExactFew, kExactMany: there is no condition (shifts, a leaf of 2^31 or more), every candidate is evaluated on its own
     u32 chunk;                       // operands per ticket (until the tickets are numbered: leaves of its groups)
     int16_t heavy;                   // an operand costs many times the usual (exact form, contexts that compare): these go first
-    int16_t classes;                 // operands are counted by class: e_begin = 0, e_count combinations of classes (class_operands)
+    int16_t classes;                 // operands are counted by class: e_count combinations of classes (class_operands), from the first on;
+                                     // e_begin: operands of the rank window that they stand for
     u64 e_begin, e_count;
 };
 static_assert(sizeof(JoinSeg) == 88, "sketches of many holes just fit the fixed scratch of a call that may not allocate");

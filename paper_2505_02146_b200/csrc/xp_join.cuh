@@ -1294,9 +1294,9 @@ __device__ __noinline__ void join_fill(JoinWarp& w, const PlanDev& plan, const J
 }
 
 // What `count` operands from number `first` on stand for in the count of candidates: themselves, or, where the segment counts by class, the
-// first ticket's for all there are.
-__device__ __forceinline__ u64 seg_operands(const JoinSeg& seg, const GrammarDev* g, u64 first, u64 count) {
-    return !XP_CLASSES(seg) ? count : first == 0ull ? g->cnt[seg.nt][seg.esize] : 0ull;
+// first ticket's for all that the window covers.
+__device__ __forceinline__ u64 seg_operands(const JoinSeg& seg, u64 first, u64 count) {
+    return !XP_CLASSES(seg) ? count : first == 0ull ? seg.e_begin : 0ull;
 }
 
 // Operands [first, first + count) of a segment against the leaves (count <= the segment's chunk).
@@ -1305,7 +1305,7 @@ __device__ __noinline__ void join_ticket(JoinWarp& w, const PlanDev& plan, const
                                          u64 first, u64 count, JoinCount& n) {
     const GrammarDev* g = sk->g;
     const int lane = threadIdx.x & 31;
-    n.cands += seg_operands(seg, g, first, count) * w.hot.pairs;
+    n.cands += seg_operands(seg, first, count) * w.hot.pairs;
     const u32 lim = w.hot.lim;
     if (seg.exact == kExactFew) {
         for (u64 i = 0; i < count; ++i) join_exact(w, plan, seg, sk, hole, first + i, n);
@@ -1592,7 +1592,7 @@ __device__ __noinline__ void range_ticket(JoinWarp& w, const PlanDev& plan, cons
         sets_ok = sets_ok && hole->join_sets[grp.leaf_nt].ok != 0;
     }
     const int parts = seg.parts > 1 ? seg.parts : 1;
-    if (part == 0) n.cands += seg_operands(seg, g, first, count) * pairs;
+    if (part == 0) n.cands += seg_operands(seg, first, count) * pairs;
     for (u64 at = 0; at < count; at += 32) {
         const u64 e = first + at + lane;
         const bool have = at + lane < count;
@@ -1820,7 +1820,7 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_kernel(const __grid_cons
         u32 part = 0;
         u64 block = t - seg.first_ticket;
         if (seg.parts > 1) { part = (u32)block % (u32)seg.parts; block = (u32)block / (u32)seg.parts; }      // (few tickets: see number_joins)
-        const u64 from = block * chunk, first = seg.e_begin + from;
+        const u64 from = block * chunk, first = (XP_CLASSES(seg) ? 0ull : seg.e_begin) + from;
         // (what waits in the queues is numbered in 32 bits, and a warp's tickets ascend)
         if (w.seg >= 0 && (w.seg != lo || (first + chunk - w.base) >> 32)) join_leave(w, plan, w.seg, n);
         if (seg.acc != acc) { join_flush(plan, acc, n); acc = seg.acc; }

@@ -200,3 +200,16 @@ def test_a_static_call_of_many_comparing_holes(xp):
         assert list(got[h].match_count)[:8] == want[h].match_count, h
         assert got[h].solved == want[h].solved and (not want[h].solved or got[h].least_rank == want[h].least_rank)
     assert any(w.solved for w in want)
+
+
+def test_a_window_counts_its_own_candidates(xp):
+    """Candidates visited (tested or decided without a test) of a window that is searched by class: those of the window."""
+    sk = _large("((i*7)+j)*3")
+    gr = xp.xp_grammar_create(sk.grammar)
+    ls = xp.xp_sketch_load(gr, sk)
+    n = xp.xp_grammar_count(gr, 0, 7)
+    begin = n[1] * n[5] + n[3] * n[3]                     # the first production's sums of five nodes and a leaf
+    for width in (n[1] * 1_500_000, n[1] * 4_000_000):
+        r = xp.xp_repair(ls, size_min=7, size_max=7, rank_ranges=[(0, 7, begin, begin + width)])[0]
+        assert r.filter_tests < width // n[1] * 3        # (by class, or this test does not test what it says)
+        assert r.filter_tests + r.candidates_skipped == width
