@@ -1818,11 +1818,11 @@ constexpr u64 kFewCall = 1ull << 23;         // ... and of all such segments of 
 // many steps that every warp of the device gets about four: fewer and the last wave is uneven, more and the
 // warps spend their time taking tickets.  64 steps at most.  In the exact form a ticket is one step, which costs as much as some
 // hundred others; with fewer steps than two for every warp it is one operand, so that the warps share those.
-static void number_joins(Plan* plan) {
+static void number_joins(Plan* plan, size_t n_sketches) {
     if (plan->jsegs.empty()) return;
     // the heavy tickets of a few large sketches first, so that none of them is a call's last (batches are long enough to even out)
-    if (plan->jsegs.size() <= 64)
-        std::stable_sort(plan->jsegs.begin(), plan->jsegs.end(), [](const JoinSeg& a, const JoinSeg& b) { return a.heavy > b.heavy; });
+    if (plan->jsegs.size() <= 64 || n_sketches <= kPairMaxSketches)
+        std::stable_partition(plan->jsegs.begin(), plan->jsegs.end(), [](const JoinSeg& c) { return c.heavy != 0; });
     u64 steps = 0, exact_steps = 0;
     for (const JoinSeg& c : plan->jsegs) (c.exact ? exact_steps : steps) += (c.e_count + 31) / 32;
     const u64 warps = (u64)search_warps();
@@ -1928,7 +1928,7 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
             plan->jsegs[j].sketch = (i32)i; plan->jsegs[j].acc += acc_base; plan->jsegs[j].first_group += group_base;
         }
     }
-    number_joins(plan);
+    number_joins(plan, n);
     return XP_OK;
 }
 
