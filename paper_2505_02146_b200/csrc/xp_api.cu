@@ -526,7 +526,7 @@ struct xp_sketch {
     // One per form (PlanForm): each is built once, under the lock, and only read from then on
     // (calls on several threads copy them at the same time); a refinement, during which no search may run, drops them.
     mutable std::mutex plan_mu;
-    mutable std::unique_ptr<const Plan> plan_kept[8];      // per form, with classes and without for comparing holes with many matches
+    mutable std::unique_ptr<const Plan> plan_kept[15];     // per form and for which comparing holes classes are left out (ClassUse)
 };
 
 // What the load's kernels settled for a hole.
@@ -1707,10 +1707,12 @@ static u64 class_operands(const xp_grammar* g, const HoleHost& ho, int nt, int s
     return sum;
 }
 
+enum RangeSplit { kSplitNone, kSplitClasses, kSplitAll };     // which comparing contexts have a segment per operator and side
+
 // Leaf-join segments of (start nonterminal, size k >= 3) restricted to ranks [lo, hi): one per operand nonterminal, with
 // a group per leaf nonterminal, for every operator with a leaf of it on either side of such an operand.  Copies of one
 // production open segments of their own; so do shifts, which only the exact form knows.
-static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi, bool few) {
+static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int sketch, int hole, int acc, int k, u64 lo, u64 hi, RangeSplit split) {
     const int nt = ho.start_nt;
     const bool exact = ho.exact, compares = ho.compares;
     struct Open { JoinSeg seg; bool shifts; std::vector<JoinGroup> groups; };
@@ -1779,7 +1781,7 @@ static void add_joins(Plan* plan, const xp_grammar* g, const HoleHost& ho, int s
         }
         // An operand of a context that compares takes some hundred microseconds of a lane, and classes leave a few thousand of them: a
         // segment per operator and side, so that as many warps share them (three conv holes: join 540 -> 430 us).
-        if (few && compares && !c.seg.exact && c.seg.e_count <= kRangeSplit) {
+        if ((split == kSplitAll || (split == kSplitClasses && c.seg.classes)) && compares && !c.seg.exact && c.seg.e_count <= kRangeSplit) {
             c.seg.parts = kRangeParts;
             for (const JoinGroup& q : c.groups)
                 for (int b = 0; b < 2 * kOpSlots; ++b) {
@@ -1858,9 +1860,16 @@ constexpr u64 kTileMinRanks = 4096;          // smaller windows are searched ran
 constexpr double kClassMatches = 4.0;                     // ... for each entry of the survivor queue (a call on the fixed scratch has fewer: 20 guards, 28.7 / 59.8 ms)
 
 // What a plan may use: kFormMany, a batch: no pair join; the others, at most kPairMaxSketches sketches: narrow tiles where a block is small, and
-// without the pair join, with it from kPairLeastBatch pairs on, or from kPairLeast on.
-enum PlanForm { kFormMany = 0, kFormTiles = 1, kFormPairsSome = 2, kFormPairs = 3 };
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, bool dense, Plan* plan);
+// without the pair join, with it from kPairLeastBatch pairs on, or from kPairLeast on.  kFormDozens: a batch of up to kRangeSketches, in which comparing
+// contexts over classes are still cut into segments by operator: a tenth of the operands leaves too few tickets otherwise (10 guards of 29, 40 and 60
+// leaves: search 0.49, 0.74, 1.04 ms operand by operand, 0.56, 0.75, 1.01 by class in one segment, 0.37, 0.53, 0.80 so).
+constexpr size_t kRangeSketches = 64;
+// A larger batch goes by operand where fewer than one sketch in so many has a comparing hole with classes: these would take the whole call to the longer
+// form of the leaf join (500 sketches, 5 of them guards: search 2.19 ms, 2.39 so).
+constexpr size_t kClassShare = 16;
+enum PlanForm { kFormMany = 0, kFormTiles = 1, kFormPairsSome = 2, kFormPairs = 3, kFormDozens = 4, kForms = 5 };
+enum ClassUse { kUseAll = 0, kUseSparse = 1, kUseFew = 2 };     // classes of comparing holes: all, not where the sample has matches, none
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, ClassUse use, Plan* plan);
 
 // A sketch's tables, and the library's scratch, live on the device that was current when the sketch was
 // loaded: a call made with another device current would hand the kernels pointers of the wrong GPU.
@@ -1880,26 +1889,33 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
     // search all holes in one launch.  So does a call with a cancel word or a time limit: its launches are bounded, and the
     // host looks at both between them; a pair join's launch covers a whole block.
     const bool pairs = may_pair && !o->cancel && o->timeout_ms <= 0;
-    const PlanForm form = n > kPairMaxSketches ? kFormMany : !pairs ? kFormTiles : n > kPairFew ? kFormPairsSome : kFormPairs;
+    const PlanForm form = n > kRangeSketches ? kFormMany : n > kPairMaxSketches ? kFormDozens : !pairs ? kFormTiles : n > kPairFew ? kFormPairsSome : kFormPairs;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
     double matches = 0;                                   // of comparing holes with classes, by the sample
+    size_t with = 0;                                      // sketches that have some
     for (size_t i = 0; i < n; ++i)
-        if (sk[i])
-            for (const HoleHost& h : sk[i]->holes)
-                if (h.compares && h.cls_size > 0) for (int k = 1; k <= h.max_size; ++k) matches += h.pass_rate * (double)sk[i]->g->cnt[h.start_nt][k];
-    const bool dense = matches > kClassMatches * queue;
+        if (sk[i]) {
+            bool some = false;
+            for (const HoleHost& h : sk[i]->holes) {
+                if (!h.compares || h.cls_size == 0) continue;
+                some = true;
+                for (int k = 1; k <= h.max_size; ++k) matches += h.pass_rate * (double)sk[i]->g->cnt[h.start_nt][k];
+            }
+            with += some ? 1u : 0u;
+        }
+    const ClassUse use = form == kFormMany && with * kClassShare < n ? kUseFew : matches > kClassMatches * queue ? kUseSparse : kUseAll;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
         if (!s) return fail(XP_ERR_INVALID_ARG, "null sketch in batch");
-        if (!plain || plan->whole) { plan_sketch(s, i, o, form, dense, plan); continue; }
+        if (!plain || plan->whole) { plan_sketch(s, i, o, form, use, plan); continue; }
         const Plan* own;
         {
             std::lock_guard<std::mutex> lock(s->plan_mu);
-            std::unique_ptr<const Plan>& kept = s->plan_kept[form + (dense ? 4 : 0)];
+            std::unique_ptr<const Plan>& kept = s->plan_kept[form + kForms * use];
             if (!kept) {
                 std::unique_ptr<Plan> made(new Plan);
-                plan_sketch(s, 0, o, form, dense, made.get());
+                plan_sketch(s, 0, o, form, use, made.get());
                 made->acc.clear();                        // (made per call, below)
                 kept = std::move(made);
             }
@@ -1933,12 +1949,12 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
 }
 
 // One sketch's segments, accumulators and tickets, appended to the plan as sketch number i.
-static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, bool dense, Plan* plan) {
+static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, ClassUse use, Plan* plan) {
     std::vector<u32> taken;
     {
         for (int h = 0; h < s->n_holes; ++h) {
             HoleHost ho = s->holes[h];
-            if (dense && ho.compares && ho.pass_rate > 0) ho.cls_size = 0;
+            if (ho.compares && (use == kUseFew || (use == kUseSparse && ho.pass_rate > 0))) ho.cls_size = 0;
             AccDev a;
             memset(&a, 0, sizeof(a));
             for (int k = 0; k <= kMaxSize; ++k) a.min_rank[k] = ~0ull;
@@ -1967,10 +1983,10 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 // candidate that passes those.  40 leaves, size 7, 3.2 million operands, three specs: 210, 1290, 212 ms as tiles, 2270, 4220,
                 // 2400 by the join over classes; with a shift 144, 128 against 1500, 159, with a leaf of 2^33 119, 965 against 64, 807.)
                 const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
-                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, form != kFormMany && !plan->whole);
-                const bool pairs = form >= kFormPairsSome;
+                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, plan->whole || form == kFormMany ? kSplitNone : form == kFormDozens ? kSplitClasses : kSplitAll);
+                const bool pairs = form == kFormPairsSome || form == kFormPairs;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
-                add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany, leaves);
+                add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany && form != kFormDozens, leaves);
             }
         }
     }
