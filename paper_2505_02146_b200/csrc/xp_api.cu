@@ -77,6 +77,9 @@ cudaError_t pool_alloc(void** out, size_t bytes, int* device_out, size_t* grante
     if (e != cudaSuccess) return e;
     *device_out = dev;
     *granted = need;
+#ifdef XP_CHECKS
+    if (const char* most = getenv("XP_POOL_MOST")) if (need > strtoull(most, nullptr, 10)) return cudaErrorMemoryAllocation;      // (a test's full device)
+#endif
     std::lock_guard<std::mutex> lock(g_pool_mu);
     DevPool& p = g_pools[dev];
     // a kept block fits a request when it wastes at most an eighth of itself (sketches of varying

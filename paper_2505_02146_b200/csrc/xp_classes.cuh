@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(kClassThreads) class_insert_kernel(const Class
             if (same) { slot = s; break; }
         }
     }
+    (void)XP_CHECKED(!on || slot != kClassNone, kChkSlot);      // (the table has twice as many words as subtrees)
     // one atomic per class and warp (large classes are runs of neighbours)
     const int lane = threadIdx.x & 31;
     const u32 same = __match_any_sync(0xffffffffu, slot);
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(kClassThreads) class_number_kernel(const Class
     if (!first) return;
     const u32 id = (u32)s_base + s_classes[warp] + (u32)__popc(mine & ((1u << lane) - 1u));
     const u32 place = (u32)(s_base >> 32) + s_members[warp] + incl - n;
+    if (!XP_CHECKED(id < count && place + n <= count, kChkSlot)) return;
     hole->cls_pair[off + id] = reinterpret_cast<const int2*>(hole->tab_pair)[base + i];
     hole->cls_start[off + (u32)nt + id] = place;
     job.table[at.x] = ((u64)n << 32) | place;
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(kClassThreads) class_member_kernel(const Class
     const u32 count = (u32)g->cnt[part.nt][top], i = part.first + threadIdx.x;
     if (i >= count) return;
     const uint2 at = job.at[off + i];
-    if (at.x != kClassNone) hole->cls_mem[off + (u32)job.table[at.x] + at.y] = i;
+    if (at.x != kClassNone && XP_CHECKED(at.x <= job.mask && (u32)job.table[at.x] + at.y < count, kChkSlot)) hole->cls_mem[off + (u32)job.table[at.x] + at.y] = i;
 }
 
 // ---- what the joins read ----
@@ -212,6 +214,7 @@ __device__ __noinline__ ClassOperand class_operand(const GrammarDev* g, const Ho
             base += cl * cr;
         }
     }
+    (void)XP_CHECKED(false, kChkRank);
     return c;                                             // (not reached: e is below the count that the host made the same way)
 }
 

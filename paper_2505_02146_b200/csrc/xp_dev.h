@@ -382,7 +382,7 @@ struct PlanDev {
     const JoinSeg* jsegs;            // device
     const JoinGroup* jgroups;        // device
     const PairSeg* psegs;            // device
-    i32 n_jsegs, pad0;
+    i32 n_jsegs, n_psegs;
     u64 join_base, n_join;           // tickets of the leaf join that belong to this launch
     u64* join_ticket;                // device counter, zero at launch
     const SketchDev* const* sketches;  // device table of device pointers

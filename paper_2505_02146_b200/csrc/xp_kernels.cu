@@ -3324,7 +3324,7 @@ static PlanDev plan_on(char* base, const SearchLayout& L) {
     pd.jsegs = (const JoinSeg*)(base + L.jsegs);
     pd.jgroups = (const JoinGroup*)(base + L.jgroups);
     pd.psegs = (const PairSeg*)(base + L.psegs);
-    pd.n_jsegs = L.n_jsegs; pd.pad0 = 0;
+    pd.n_jsegs = L.n_jsegs; pd.n_psegs = L.n_psegs;
     pd.join_base = pd.n_join = 0;
     pd.join_ticket = (u64*)(base + 32);
     pd.sketches = (const SketchDev* const*)(base + L.sketches);

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(kMemberThreads, 2) members_kernel(const __grid
             }
         }
         const MemberRec rec = plan.members[at];
+        if (!XP_CHECKED(t - rec.first < rec.pieces && (rec.seg >= 0 ? rec.seg < plan.n_jsegs : ~rec.seg < plan.n_psegs), kChkSegment)) break;
         const u64 k_first = (t - rec.first) * kMemberPiece;
         const bool join = rec.seg >= 0;
         const int sketch = join ? plan.jsegs[rec.seg].sketch : plan.psegs[~rec.seg].sketch, hole_index = join ? plan.jsegs[rec.seg].hole : plan.psegs[~rec.seg].hole;

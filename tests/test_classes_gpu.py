@@ -1,5 +1,9 @@
 """Searches over operand classes (operands that no probe tells apart are met once, and taken apart where a candidate
 passes): against the oracle, and cut into rank windows small enough to be searched operand by operand."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -14,13 +18,16 @@ VS = [Variable("i", 0, 9), Variable("j", 0, 7)]
 
 @pytest.mark.parametrize("ops,consts", [
     (["+", "-", "*", "/", "%"], constant_set(-13, 13)),                       # 4 205 operands of three nodes: just enough for classes
-    (["+", "-", "*", "min", "max", "%"], constant_set(-9, 12) + [1 << 20, 5]),
+    (["+", "-", "*", "min", "max", "%"], constant_set(-9, 14) + [1 << 20, 5]),
     (["+", "*", "<<", ">>", "/"], constant_set(-4, 24)),                      # undefined shifts and divisions
 ])
 @pytest.mark.parametrize("ctx,spec", [("i<HOLE", "i<((j*2)+1)"), ("HOLE<=j", "(i/3)<=j"), ("(j-HOLE)<(i-2)", "(i%4)<5")])
 def test_comparing_contexts(xp, ops, consts, ctx, spec):
     g = free_grammar(VS, sorted(set(consts)), ops=ops)
-    check_sketch(xp, Sketch(g, [Hole(0, 5, ctx=parse_expr(ctx, VS), spec_expr=parse_expr(spec, VS))], name=f"{ctx}: {spec}"))
+    r = check_sketch(xp, Sketch(g, [Hole(0, 5, ctx=parse_expr(ctx, VS), spec_expr=parse_expr(spec, VS))], name=f"{ctx}: {spec}"))[0]
+    assert r.cand_count[3] >= 4096
+    if max(consts) < 100 and "<<" not in ops:            # (shifts and wide operands go the exact way: a test per leaf)
+        assert r.filter_tests < 0.7 * r.cand_count[3] * 10 * 3
 
 
 def _large(spec, ops=("+", "-", "*", "/", "%"), consts=None, ctx=None):
@@ -213,3 +220,71 @@ def test_a_window_counts_its_own_candidates(xp):
         r = xp.xp_repair(ls, size_min=7, size_max=7, rank_ranges=[(0, 7, begin, begin + width)])[0]
         assert r.filter_tests < width // n[1] * 3        # (by class, or this test does not test what it says)
         assert r.filter_tests + r.candidates_skipped == width
+
+
+def _odd_guard():
+    """j < HOLE holds everywhere but at one interior point, which no sample has: candidates survive the probes and fail there."""
+    vs = [Variable("i", 0, 40), Variable("j", 0, 40)]
+    ids = np.arange(1600, dtype=np.int64)
+    coords = np.stack([ids // 40, ids % 40], axis=1).astype(np.int32)
+    spec = np.ones(1600, dtype=np.int64)
+    spec[23 * 40 + 31] = 0
+    return Sketch(free_grammar(vs, constant_set(17, 47)), [Hole(0, 5, ctx=parse_expr("j<HOLE", vs), spec_table=spec)], coords, name="odd guard")
+
+
+def test_classes_after_a_refinement(xp):
+    """Promoted points are other probes and make other classes; a workspace made before still serves."""
+    import torch
+    sk = _odd_guard()
+    gr = xp.xp_grammar_create(sk.grammar)
+    ls = xp.xp_sketch_load(gr, sk)
+    ws = torch.empty(xp.xp_workspace_bytes([ls]), dtype=torch.uint8, device="cuda")
+    before = xp.xp_repair(ls, workspace=ws)[0]
+    assert before.cand_count[3] > 4096 and before.probe_survivors > sum(before.match_count)
+    assert xp.xp_sketch_refine(ls) >= 1
+    after = xp.xp_repair(ls, workspace=ws)[0]
+    assert_same(after, before)
+    assert after.probe_survivors < before.probe_survivors
+    w = {1: (0, 0), 3: (0, 0), 5: (300_000, 340_000)}
+    got = xp.xp_repair(ls, size_min=5, rank_ranges=[(0, 5, *w[5])])[0]
+    assert got.match_count[5] == oracle.repair_hole(sk, 0, rank_ranges=w).match_count[5]
+
+
+def test_a_load_without_memory_for_classes(xp, monkeypatch):
+    """The checked build can be told to refuse memory: a load (its own memory, or a batch's scratch) and a refinement without it."""
+    if os.environ.get("XP_CHECKED_BUILD") != "1":
+        pytest.skip("run through test_classes_under_the_checked_build")
+    sk = _odd_guard()
+    gr = xp.xp_grammar_create(sk.grammar)
+    plain = xp.xp_sketch_load(gr, sk)
+    want = xp.xp_repair(plain)[0]
+    size = xp.xp_sketch_info_get(plain).device_bytes
+
+    def by_operand(ls):
+        r = xp.xp_repair(ls)[0]
+        assert_same(r, want)
+        return r.filter_tests > 1.5 * want.filter_tests
+    monkeypatch.setenv("XP_POOL_MOST", str(size - 1))
+    assert by_operand(xp.xp_sketch_load(gr, sk))                                 # no room beside its tables
+    with pytest.raises(xp.XpError) as e:
+        monkeypatch.setenv("XP_POOL_MOST", "65536")
+        xp.xp_sketch_load(gr, sk)
+    assert e.value.status == 5
+    monkeypatch.setenv("XP_POOL_MOST", str(size + 4096))
+    many = xp.xp_sketch_load_batch([gr] * 8, [sk] * 8)                           # no room for the scratch of all
+    assert all(by_operand(ls) for ls in many[::3])
+    monkeypatch.delenv("XP_POOL_MOST")
+    assert xp.xp_sketch_refine(many[0]) >= 1 and not by_operand(many[0])         # (a refinement makes them)
+    monkeypatch.setenv("XP_POOL_MOST", "65536")
+    assert xp.xp_sketch_refine(many[0]) >= 0
+    assert_same(xp.xp_repair(many[0])[0], want)
+
+
+def test_classes_under_the_checked_build():
+    """Slots, places, members and entries of the list, with index checks compiled in (a failed one makes every search an error)."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    cases = "comparing_contexts or many_holes or large_classes or static_call or window_counts or refinement or without_memory or typed or quasi"
+    r = subprocess.run([sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", "-p", "no:cacheprovider", "tests/test_classes_gpu.py", "-k",
+                        f"({cases}) and not checked_build"], cwd=root, env=dict(os.environ, XP_CHECKED_BUILD="1"), capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-1000:]
+    assert " passed" in r.stdout and "skipped" not in r.stdout
