@@ -1834,7 +1834,10 @@ static void number_joins(Plan* plan, size_t n_sketches) {
     u64 few_pairs = 0, few_steps = 0;
     auto few = [](const JoinSeg& c) { return c.kind == kJoinLeaf && !c.exact && !c.heavy && !c.classes && c.chunk > 0 && c.e_count * (u64)c.chunk <= kFewPairs; };
     for (const JoinSeg& c : plan->jsegs) if (few(c)) { few_pairs += c.e_count * (u64)c.chunk; few_steps += (c.e_count + 31) / 32; }
-    const u64 share = few_pairs <= kFewCall && few_steps > 0 ? (warps > few_steps ? warps / few_steps : 1) : 0;      // parts, if the leaves are enough
+    // (not for the sake of a few holes of a batch whose others compare: an expression pair in a guard, search 0.65 / 0.67 ms)
+    bool plain = n_sketches <= kPairMaxSketches;
+    if (!plain) { plain = true; for (const JoinSeg& c : plan->jsegs) plain = plain && !c.heavy; }
+    const u64 share = plain && few_pairs <= kFewCall && few_steps > 0 ? (warps > few_steps ? warps / few_steps : 1) : 0;      // parts, if the leaves are enough
     const i32 form = exact_steps < 2 * warps ? kExactFew : kExactMany;
     u64 per = steps / (warps * 4);
     if (per < 1) per = 1;
@@ -2065,10 +2068,13 @@ static SearchLayout ws_layout(const Plan& plan, const xp_sketch* const* sk, size
     w.n_acc = (int)n_acc; w.n_segs = (int)plan.segs.size(); w.n_jsegs = (int)plan.jsegs.size(); w.n_sketches = (int)n_sketches;
     w.surv_cap = surv_cap;
     w.join_wide = plan.join_wide ? 1 : 0;
-    // (a call whose windows are all so small that candidates are checked one by one has nothing of the longer form to gain either)
+    // (the longer form is for classes, tickets in parts, and few sketches whose tickets are one wave: with more the warps hide the chain
+    // of a check, and it is the shorter code that counts.  A quasi-affine
+    // grammar with 4.1 million operands, size 9, two targets: 511, 193 ms, in the longer form 577, 224.)
+    const bool wave = n_sketches <= kPairMaxSketches && plan.n_join <= (u64)search_warps();
     w.join_batch = 1;
     for (const JoinSeg& c : plan.jsegs)
-        if (c.classes || c.parts > 0 || (c.kind != kJoinDirect && n_sketches <= kPairMaxSketches)) { w.join_batch = 0; break; }
+        if (c.classes || c.parts > 0 || (c.kind != kJoinDirect && wave)) { w.join_batch = 0; break; }
     i64 most = 0;
     w.dense = w.empty_domain = 0;
     for (size_t i = 0; i < n_sketches; ++i) {
