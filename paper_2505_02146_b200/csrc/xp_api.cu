@@ -1834,10 +1834,7 @@ static void number_joins(Plan* plan, size_t n_sketches) {
     u64 few_pairs = 0, few_steps = 0;
     auto few = [](const JoinSeg& c) { return c.kind == kJoinLeaf && !c.exact && !c.heavy && !c.classes && c.chunk > 0 && c.e_count * (u64)c.chunk <= kFewPairs; };
     for (const JoinSeg& c : plan->jsegs) if (few(c)) { few_pairs += c.e_count * (u64)c.chunk; few_steps += (c.e_count + 31) / 32; }
-    // (not for the sake of a few holes of a batch whose others compare: an expression pair in a guard, search 0.65 / 0.67 ms)
-    bool plain = n_sketches <= kPairMaxSketches;
-    if (!plain) { plain = true; for (const JoinSeg& c : plan->jsegs) plain = plain && !c.heavy; }
-    const u64 share = plain && few_pairs <= kFewCall && few_steps > 0 ? (warps > few_steps ? warps / few_steps : 1) : 0;      // parts, if the leaves are enough
+    const u64 share = few_pairs <= kFewCall && few_steps > 0 ? (warps > few_steps ? warps / few_steps : 1) : 0;      // parts, if the leaves are enough
     const i32 form = exact_steps < 2 * warps ? kExactFew : kExactMany;
     u64 per = steps / (warps * 4);
     if (per < 1) per = 1;
