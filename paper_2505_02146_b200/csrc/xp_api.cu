@@ -1860,7 +1860,10 @@ constexpr u64 kTileMinRanks = 4096;          // smaller windows are searched ran
 // warps shares the work best.  (100 guards of 29, 40 and 60 leaves, 1000 of 29, a quarter of them nearly always true: 1.7e6, 6e6, 2.6e7, 1.2e7 by the sample;
 // 95, 361, 1131, 715 ms operand by operand, 18, 870, 4500, 1190 by class.  An affine context has few matches per operand: the examples in
 // xp_classes.cuh are 2e7 by the sample.)
-constexpr double kClassMatches = 4.0;                     // ... for each entry of the survivor queue (a call on the fixed scratch has fewer: 20 guards, 28.7 / 59.8 ms)
+constexpr double kClassMatches = 4.0;                     // ... for each entry of the survivor queue
+// Candidates of such contexts, likewise: the sample does not see what is rarer than one in 256.  (On the fixed scratch, with its 8192 entries: guards of 29 and 60
+// leaves, 1.2e6 and 1.1e7 candidates, 0.18, 0.36 ms operand by operand, 0.10, 0.15 by class; 20 of 12 leaves, size 7, 3.5e7 each, 28.7 against 41 to 60.)
+constexpr double kClassCandidates = 2048.0;
 
 // What a plan may use: kFormMany, a batch: no pair join; the others, at most kPairMaxSketches sketches: narrow tiles where a block is small, and
 // without the pair join, with it from kPairLeastBatch pairs on, or from kPairLeast on.  kFormDozens: a batch of up to kRangeSketches, in which comparing
@@ -1894,7 +1897,7 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
     const bool pairs = may_pair && !o->cancel && o->timeout_ms <= 0;
     const PlanForm form = n > kRangeSketches ? kFormMany : n > kPairMaxSketches ? kFormDozens : !pairs ? kFormTiles : n > kPairFew ? kFormPairsSome : kFormPairs;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
-    double matches = 0;                                   // of comparing holes with classes, by the sample
+    double candidates = 0, matches = 0;                   // of comparing holes with classes; matches by the sample
     size_t with = 0;                                      // sketches that have some
     for (size_t i = 0; i < n; ++i)
         if (sk[i]) {
@@ -1902,11 +1905,14 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
             for (const HoleHost& h : sk[i]->holes) {
                 if (!h.compares || h.cls_size == 0) continue;
                 some = true;
-                for (int k = 1; k <= h.max_size; ++k) matches += h.pass_rate * (double)sk[i]->g->cnt[h.start_nt][k];
+                for (int k = 1; k <= h.max_size; ++k) {
+                    const double c = (double)sk[i]->g->cnt[h.start_nt][k];
+                    candidates += c; matches += h.pass_rate * c;
+                }
             }
             with += some ? 1u : 0u;
         }
-    const ClassUse use = form == kFormMany && with * kClassShare < n ? kUseFew : matches > kClassMatches * queue ? kUseSparse : kUseAll;
+    const ClassUse use = (form == kFormMany && with * kClassShare < n) || candidates > kClassCandidates * queue ? kUseFew : matches > kClassMatches * queue ? kUseSparse : kUseAll;
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
@@ -1986,7 +1992,7 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 // candidate that passes those.  40 leaves, size 7, 3.2 million operands, three specs: 210, 1290, 212 ms as tiles, 2270, 4220,
                 // 2400 by the join over classes; with a shift 144, 128 against 1500, 159, with a leaf of 2^33 119, 965 against 64, 807.)
                 const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
-                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, plan->whole || form == kFormMany ? kSplitNone : form == kFormDozens ? kSplitClasses : kSplitAll);
+                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, plan->whole || form == kFormMany || use == kUseFew ? kSplitNone : form == kFormDozens ? kSplitClasses : kSplitAll);
                 const bool pairs = form == kFormPairsSome || form == kFormPairs;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
                 add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany && form != kFormDozens, leaves);

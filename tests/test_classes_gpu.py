@@ -222,6 +222,24 @@ def test_a_window_counts_its_own_candidates(xp):
         assert r.filter_tests + r.candidates_skipped == width
 
 
+def test_calls_that_leave_classes_out(xp):
+    """Comparing contexts go by operand where the scratch is small for their candidates, and where few sketches of a large batch have one."""
+    g = free_grammar(VS, constant_set(-4, 6), ops=["+", "-", "*", "/", "%", "min", "max"])
+    sk = Sketch(g, [Hole(0, 7, ctx=parse_expr("i<HOLE", VS), spec_expr=parse_expr(f"i<((i/{h + 2})+(j%{h + 3}))", VS)) for h in range(3)])
+    ls = xp.xp_sketch_load(xp.xp_grammar_create(g), sk)
+    for got, want in zip(xp.xp_repair_static(ls), xp.xp_repair(ls)):
+        assert list(got.match_count)[:8] == want.match_count and got.least_rank == want.least_rank
+        assert got.evals_executed > want.evals_executed  # (every operand is met for itself)
+    g5 = free_grammar(VS, constant_set(-13, 17))
+    sks = [Sketch(g5, [Hole(0, 5, ctx=parse_expr("i<HOLE", VS), spec_expr=parse_expr("i<((j*2)+1)", VS))])] + \
+          [Sketch(g5, [Hole(0, 3, spec_expr=parse_expr(f"(i*{q % 5})+j", VS))]) for q in range(69)]
+    gr = xp.xp_grammar_create(g5)
+    batch = xp.xp_sketch_load_batch([gr] * len(sks), sks)
+    together, alone = xp.xp_repair_batch(batch)[0][0], xp.xp_repair(batch[0])[0]
+    assert_same(together, alone)
+    assert together.filter_tests > 1.5 * alone.filter_tests
+
+
 def _odd_guard():
     """j < HOLE holds everywhere but at one interior point, which no sample has: candidates survive the probes and fail there."""
     vs = [Variable("i", 0, 40), Variable("j", 0, 40)]
