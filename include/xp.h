@@ -202,11 +202,12 @@ typedef struct {
     uint64_t filter_tests;          /* filter-stage tests that ran: pairs of operand subtrees both defined at the first probe
                                        point, times the operators whose test loop was entered; where one operand is a leaf,
                                        operands defined at the probes times (leaves tested one by one, plus one condition that
-                                       decides all constants together) times the operators */
+                                       decides all constants together) times the operators.  Operands that no probe tells apart
+                                       are met once, and counted once here */
     uint64_t candidates_skipped;    /* candidates of the operand tiles and joins visited that were decided without a test of
                                        their own: a constant leaf decided together with the others, an operand undefined at the probe (a zero divisor inside it), a remainder whose
                                        divisor cannot exceed the target's magnitude, a quotient or remainder of 32-bit
-                                       operands against a target outside 32 bits.  With a rank window the tiles also
+                                       operands against a target outside 32 bits, a twin of an operand that was met.  With a rank window the tiles also
                                        cover some ranks outside it; those count here or in filter_tests as well. */
     uint64_t h2d_bytes, d2h_bytes;  /* bytes the call copied to and from the device (the whole call, every hole) */
 } xp_result_view;
