@@ -529,7 +529,7 @@ struct xp_sketch {
     // One per form (PlanForm): each is built once, under the lock, and only read from then on
     // (calls on several threads copy them at the same time); a refinement, during which no search may run, drops them.
     mutable std::mutex plan_mu;
-    mutable std::unique_ptr<const Plan> plan_kept[15];     // per form and for which comparing holes classes are left out (ClassUse)
+    mutable std::unique_ptr<const Plan> plan_kept[35];     // per form and for which holes classes are left out (ClassUse)
 };
 
 // What the load's kernels settled for a hole.
@@ -1864,6 +1864,8 @@ constexpr double kClassMatches = 4.0;                     // ... for each entry 
 // Candidates of such contexts, likewise: the sample does not see what is rarer than one in 256.  (On the fixed scratch, with its 8192 entries: guards of 29 and 60
 // leaves, 1.2e6 and 1.1e7 candidates, 0.18, 0.36 ms operand by operand, 0.10, 0.15 by class; 20 of 12 leaves, size 7, 3.5e7 each, 28.7 against 41 to 60.)
 constexpr double kClassCandidates = 2048.0;
+// Matches of affine contexts: 136 leaves, size 7, 131 072 points, a target that is a variable (8.3e8 by the sample, 9.4e7 in fact): 48 s operand by operand, 101 by class.
+constexpr double kClassMatchesAffine = 256.0;
 
 // What a plan may use: kFormMany, a batch: no pair join; the others, at most kPairMaxSketches sketches: narrow tiles where a block is small, and
 // without the pair join, with it from kPairLeastBatch pairs on, or from kPairLeast on.  kFormDozens: a batch of up to kRangeSketches, in which comparing
@@ -1874,7 +1876,8 @@ constexpr size_t kRangeSketches = 64;
 // form of the leaf join (500 sketches, 5 of them guards: search 2.19 ms, 2.39 so).
 constexpr size_t kClassShare = 16;
 enum PlanForm { kFormMany = 0, kFormTiles = 1, kFormPairsSome = 2, kFormPairs = 3, kFormDozens = 4, kForms = 5 };
-enum ClassUse { kUseAll = 0, kUseSparse = 1, kUseFew = 2 };     // classes of comparing holes: all, not where the sample has matches, none
+// Classes of comparing holes: all, not where the sample has matches, none; kUseSparseAffine (beside these): of the others not where it has some.
+enum ClassUse { kUseAll = 0, kUseSparse = 1, kUseFew = 2, kUseSparseAffine = 4 };
 static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, PlanForm form, ClassUse use, Plan* plan);
 
 // A sketch's tables, and the library's scratch, live on the device that was current when the sketch was
@@ -1897,13 +1900,17 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
     const bool pairs = may_pair && !o->cancel && o->timeout_ms <= 0;
     const PlanForm form = n > kRangeSketches ? kFormMany : n > kPairMaxSketches ? kFormDozens : !pairs ? kFormTiles : n > kPairFew ? kFormPairsSome : kFormPairs;
     const bool plain = o->size_min <= 0 && o->size_max <= 0 && o->n_rank_ranges == 0 && o->flags == 0;
-    double candidates = 0, matches = 0;                   // of comparing holes with classes; matches by the sample
+    double candidates = 0, matches = 0, affine = 0;       // of comparing holes with classes; matches by the sample, and those of the other holes with some
     size_t with = 0;                                      // sketches that have some
     for (size_t i = 0; i < n; ++i)
         if (sk[i]) {
             bool some = false;
             for (const HoleHost& h : sk[i]->holes) {
-                if (!h.compares || h.cls_size == 0) continue;
+                if (h.cls_size == 0) continue;
+                if (!h.compares) {
+                    for (int k = 1; k <= h.max_size; ++k) affine += h.pass_rate * (double)sk[i]->g->cnt[h.start_nt][k];
+                    continue;
+                }
                 some = true;
                 for (int k = 1; k <= h.max_size; ++k) {
                     const double c = (double)sk[i]->g->cnt[h.start_nt][k];
@@ -1912,7 +1919,8 @@ static xp_status build_plan(const xp_sketch* const* sk, size_t n, const xp_repai
             }
             with += some ? 1u : 0u;
         }
-    const ClassUse use = (form == kFormMany && with * kClassShare < n) || candidates > kClassCandidates * queue ? kUseFew : matches > kClassMatches * queue ? kUseSparse : kUseAll;
+    const int left_out = (form == kFormMany && with * kClassShare < n) || candidates > kClassCandidates * queue ? kUseFew : matches > kClassMatches * queue ? kUseSparse : kUseAll;
+    const ClassUse use = (ClassUse)(left_out | (affine > kClassMatchesAffine * queue ? kUseSparseAffine : 0));
     if (n > 16) { plan->segs.reserve(n * 8); plan->acc.reserve(n * 2); plan->nominal_ops.reserve(n * 2); }
     for (size_t i = 0; i < n; ++i) {
         const xp_sketch* s = sk[i];
@@ -1963,7 +1971,8 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
     {
         for (int h = 0; h < s->n_holes; ++h) {
             HoleHost ho = s->holes[h];
-            if (ho.compares && (use == kUseFew || (use == kUseSparse && ho.pass_rate > 0))) ho.cls_size = 0;
+            const int left_out = use & 3;
+            if (ho.compares ? left_out == kUseFew || (left_out == kUseSparse && ho.pass_rate > 0) : (use & kUseSparseAffine) && ho.pass_rate > 0) ho.cls_size = 0;
             AccDev a;
             memset(&a, 0, sizeof(a));
             for (int k = 0; k <= kMaxSize; ++k) a.min_rank[k] = ~0ull;
@@ -1992,7 +2001,7 @@ static void plan_sketch(const xp_sketch* s, size_t i, const xp_repair_opts* o, P
                 // candidate that passes those.  40 leaves, size 7, 3.2 million operands, three specs: 210, 1290, 212 ms as tiles, 2270, 4220,
                 // 2400 by the join over classes; with a shift 144, 128 against 1500, 159, with a leaf of 2^33 119, 965 against 64, 807.)
                 const bool leaves = ho.compares && s->g->cnt[ho.start_nt][k - 2] > kRangeMost;
-                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, plan->whole || form == kFormMany || use == kUseFew ? kSplitNone : form == kFormDozens ? kSplitClasses : kSplitAll);
+                if (!leaves) add_joins(plan, s->g, ho, (int)i, h, acc, k, lo, hi, plan->whole || form == kFormMany || (use & 3) == kUseFew ? kSplitNone : form == kFormDozens ? kSplitClasses : kSplitAll);
                 const bool pairs = form == kFormPairsSome || form == kFormPairs;
                 if (pairs) add_pairs(plan, s->g, ho, (int)i, h, acc, k, lo, hi, o->flags & XP_FLAG_ALWAYS_PAIR ? 1 : form == kFormPairs ? kPairLeast : kPairLeastBatch, &taken);
                 add_tiles(plan, s->g, pairs ? &taken : nullptr, ho.start_nt, (int)i, h, acc, k, lo, hi, ho.compares ? kBcTileSlow : kBcTile, form != kFormMany && form != kFormDozens, leaves);

@@ -240,6 +240,24 @@ def test_calls_that_leave_classes_out(xp):
     assert together.filter_tests > 1.5 * alone.filter_tests
 
 
+def test_a_target_that_collapses_to_a_variable(xp):
+    """A variable is the target (k / 28 is 0): more matches than the list of classes is for, so a window wide enough for classes goes by operand."""
+    vs = [Variable("i", 0, 4), Variable("j", 0, 7), Variable("k", 0, 8)]
+    g = free_grammar(vs, constant_set(-64, 64, [2**e for e in range(11)]))
+    gr = xp.xp_grammar_create(g)
+    ls, other = (xp.xp_sketch_load(gr, Sketch(g, [Hole(0, 7, spec_expr=parse_expr(spec, vs))])) for spec in ("((k/28)*13)+j", "((i*13)+j)*5"))
+    n = xp.xp_grammar_count(gr, 0, 7)
+    begin, width = n[1] * n[5] + n[3] * n[3], n[1] * 8_000_000            # sums of five nodes and a leaf
+
+    def window(s, lo, hi):
+        return xp.xp_repair(s, size_min=7, size_max=7, rank_ranges=[(0, 7, begin + lo, begin + hi)])[0]
+    r = window(ls, 0, width)
+    parts = [window(ls, width * p // 16, width * (p + 1) // 16) for p in range(16)]
+    assert r.match_count[7] == sum(x.match_count[7] for x in parts) > 0
+    assert r.least_rank == next(x.least_rank for x in parts if x.match_count[7])
+    assert window(other, 0, width).n_launches == r.n_launches + 1           # (members_kernel: by class)
+
+
 def _odd_guard():
     """j < HOLE holds everywhere but at one interior point, which no sample has: candidates survive the probes and fail there."""
     vs = [Variable("i", 0, 40), Variable("j", 0, 40)]
