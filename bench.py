@@ -40,16 +40,16 @@ DIVISION_COST = None
 # Counters of the search kernels per step and workload, from the ncu captures in profiles/search_kernels.md (dram = dram__bytes_read.sum +
 # dram__bytes_write.sum, thread_inst = smsp__thread_inst_executed.sum).  They describe the kernel sources whose hash is
 # given; bench.py reports them (roofline.traffic, roofline.frac_executed) only while the sources still have that hash.
-NCU_CAPTURE = {"kernel_hash": "5f5200d70ae6f484", "date": "2026-12-03",
-               "config2": {"thread_inst": 2.365e9, "dram_bytes": 3.63e6},
-               "config3": {"thread_inst": 1.713e9, "dram_bytes": 2.80e7},
-               "config4": {"thread_inst": 3.402e10, "dram_bytes": 6.03e7}}
+NCU_CAPTURE = {"kernel_hash": "9bc316f57788a847", "date": "2026-12-03",
+               "config2": {"thread_inst": 2.369e9, "dram_bytes": 4.03e6},
+               "config3": {"thread_inst": 1.714e9, "dram_bytes": 2.84e7},
+               "config4": {"thread_inst": 3.404e10, "dram_bytes": 6.10e7}}
 
 
 def kernel_hash() -> str:
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2505_02146_b200", "csrc")
-    for name in ("xp_dev.h", "xp_device.cuh", "xp_kernels.cu", "xp_classes.cuh", "xp_join.cuh", "xp_pairs.cuh"):
+    for name in ("xp_dev.h", "xp_device.cuh", "xp_kernels.cu", "xp_classes.cuh", "xp_join.cuh", "xp_pairs.cuh", "xp_members.cuh"):
         h.update(open(os.path.join(csrc, name), "rb").read())
     return h.hexdigest()[:16]
 
